@@ -1,9 +1,9 @@
-// st_sym_moment2, fp32 path for few features (d % 8 == 0, d <= 64) and many samples -- the regime
+// st_sym_moment2, fp32 path for few features (see moment2_use_small in moment2.cu) -- the regime
 // of the paper's covariance workloads (Section 7.2; its real datasets have 6 and 13 features).
 //
 // out[p(i,j)] = sum_n X[n,i] X[n,j], 0 <= i <= j < d  (Section 3, M1; Section 5.5, y_U = i <= j).
 //
-// The d columns are dealt to d/8 "column blocks"; block b owns columns 4b..4b+3 of the first half
+// The d columns, padded to a multiple of 8, are dealt to "column blocks" of 8; block b owns columns 4b..4b+3 of the first half
 // of a row and the same four of the second half (two 16-byte chunks, so that the threads of a warp
 // read one contiguous 128-byte segment per load and a row can stay in its natural layout).  Every
 // unordered pair of columns lies in exactly one unordered pair of blocks, so the 8x8 tiles {x,y}
@@ -26,7 +26,7 @@
 namespace st {
 
 constexpr int M2S_MAX_THREADS = 256;
-constexpr int M2S_MAX_ITEMS = 32;
+constexpr int M2S_MAX_BLOCKS = 31;         // column blocks: one item per thread at most (d <= 248; dense control: 22 blocks)
 constexpr int M2S_BUFFERS = 3;
 constexpr int M2S_STAGE_BYTES = 57344;     // upper bound of one stage (3 stages + slack fit in 227 KB)
 
@@ -40,37 +40,74 @@ __device__ __forceinline__ void m2s_bulk_load(void *dst, const void *src, uint32
                  : "memory");
 }
 
-// work items: tiles {s,p} and {s,q} of column blocks; q == 255 marks an item with one tile only
-struct M2SmallItems {
-    int n;
-    unsigned char s[M2S_MAX_ITEMS], p[M2S_MAX_ITEMS], q[M2S_MAX_ITEMS];
-};
+// Number of work items, and item t: tiles {s,p} and {s,q} of column blocks (q = -1: one tile only).  Structured:
+// for every block y the tiles {x,y}, x <= y, are paired along x with y as the common block (floor(y^2/4) items come
+// before those of y); when their number is odd, tile {0,y} is held back, and the held-back tiles (y even) are paired
+// with block 0 in common.  Dense control: all ordered tiles (x,y), paired along y with x in common.
+__host__ __device__ inline int m2s_nitems(int nbk, bool dense)
+{
+    return dense ? nbk * ((nbk + 1) / 2) : (nbk * (nbk + 1) / 2 + 1) / 2;
+}
+__device__ __forceinline__ void m2s_item(int t, int nbk, bool dense, int &s, int &p, int &q)
+{
+    if (dense) {
+        const int per = (nbk + 1) / 2;
+        s = t / per;
+        p = 2 * (t - s * per);
+        q = p + 1 < nbk ? p + 1 : -1;
+        return;
+    }
+    const int paired = nbk * nbk / 4;
+    if (t < paired) {
+        int y = (int)(2.f * sqrtf((float)t));
+        while (y * y / 4 > t) --y;
+        while ((y + 1) * (y + 1) / 4 <= t) ++y;
+        s = y;
+        p = ((y + 1) & 1) + 2 * (t - y * y / 4);
+        q = p + 1;
+    } else {
+        s = 0;
+        p = 4 * (t - paired);
+        q = p + 2 < nbk ? p + 2 : -1;
+    }
+}
+
+// Pitch, in words, of the block-level sum's buffer: at least rg * nitems, and nitems modulo 32.
+__host__ __device__ inline int m2s_red_pitch(int rg, int nitems)
+{
+    const int cells = rg * nitems;
+    return cells + ((nitems - cells) & 31);
+}
 
 struct M2SmallArgs {
     const float *X;
     float *partials;      // [slices][128][nitems]
     unsigned *status;     // workspace header (status and detail words)
     int64_t N, ldx, rows_per_slice;
-    int d, nbk, rg, rpg, dense, bar_floats;
-    M2SmallItems items;
+    int d, pitch, nbk, nitems, rg, rpg, dense, bar_floats;
 };
 
 // column of element e (0..7) of column block b
 __device__ __forceinline__ int m2s_column(int b, int e, int half) { return (e < 4) ? 4 * b + e : half + 4 * b + (e - 4); }
 
+// BULK: rows start on 16-byte boundaries and arrive by bulk copies, in shared memory at their own pitch; otherwise
+// they are copied word by word to a pitch rounded up to 16 bytes (one copy instruction per 32 words, against more
+// than 64 FMA instructions).  Either way a tile that reaches past column d reads whatever follows the row: only
+// sums that are dropped contain it.  [50021,75]: 23 us the call, 71 with the plain 64 x 64 tiles that served it before.
+template <bool BULK>
 __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const M2SmallArgs a)
 {
     extern __shared__ __align__(16) float smem[];
     const int stage_rows = a.rg * a.rpg;
-    const int stage_floats = stage_rows * a.d;
+    const int stage_floats = stage_rows * a.pitch;
     const int tid = threadIdx.x, nthreads = blockDim.x;
-    const int nitems = a.items.n;
+    const int nitems = a.nitems;
     const int item_rg = tid / nitems, item = tid - item_rg * nitems;
     const bool active = item_rg < a.rg;
     const int half = 4 * a.nbk;
-    const int bs = a.items.s[item], bp = a.items.p[item];
-    const int bq = a.items.q[item] == 255 ? bp : a.items.q[item];
-    const int os = 4 * bs, op = 4 * bp, oq = 4 * bq;
+    int bs, bp, bq;
+    m2s_item(item, a.nbk, a.dense != 0, bs, bp, bq);
+    const int os = 4 * bs, op = 4 * bp, oq = bq < 0 ? op : 4 * bq;
 
     float accp[8][8], accq[8][8];                      // tiles {s,p} and {s,q}
 #pragma unroll
@@ -97,14 +134,27 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
 
     const int nstages = (n_end > n_begin) ? (int)((n_end - n_begin + stage_rows - 1) / stage_rows) : 0;
     const bool contiguous = (a.ldx == a.d);
+    const int copy_r = tid / a.d, copy_c = tid - copy_r * a.d;                   // word copies: first element of this thread,
+    const int copy_dr = nthreads / a.d, copy_dc = nthreads - copy_dr * a.d;      // and the way to its next one
     // the rows of a stage arrive by bulk copies issued from warp 0: one copy when the rows are
     // contiguous in memory, one per row otherwise; rows past the end of the slice are not copied
     // and not read
     auto issue_stage = [&](int buf, int s) {
-        if (tid >= 32) return;
+        if (BULK && tid >= 32) return;
         const int64_t n0 = n_begin + (int64_t)s * stage_rows;
         const int rows = (n_end - n0 < stage_rows) ? (int)(n_end - n0) : stage_rows;
         float *dst = smem + buf * stage_floats;
+        if (!BULK) {
+            const float *src = a.X + n0 * a.ldx;
+            int r = copy_r, c = copy_c;
+            while (r < rows) {
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(tc::smem_u32(dst + r * a.pitch + c)), "l"(src + r * a.ldx + c));
+                r += copy_dr;
+                c += copy_dc;
+                if (c >= a.d) { c -= a.d; ++r; }
+            }
+            return;
+        }
         const uint32_t row_bytes = (uint32_t)a.d * 4u;
         if (tid == 0) tc::mbar_expect_tx(&full[buf], (uint32_t)rows * row_bytes);
         __syncwarp();
@@ -115,16 +165,21 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
         }
     };
 
-    for (int s = 0; s < M2S_BUFFERS - 1 && s < nstages; ++s) issue_stage(s, s);
-    const int step = a.rg * a.d;
+    for (int s = 0; s < M2S_BUFFERS - 1; ++s) {
+        if (s < nstages) issue_stage(s, s);
+        if (!BULK) asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    const int step = a.rg * a.pitch;
     int buf = 0;
     uint32_t parity = 0;
     for (int s = 0; s < nstages; ++s) {
         // a wait that gives up raises the abort flag; every thread still walks all stages so that
         // the block-wide barriers stay matched, and the host reads the status word afterwards
-        (void)tc::mbar_wait(&full[buf], parity, abort_flag, a.status, 1);
+        if (BULK) (void)tc::mbar_wait(&full[buf], parity, abort_flag, a.status, 1);
+        else asm volatile("cp.async.wait_group %0;" ::"n"(M2S_BUFFERS - 2) : "memory");
         __syncthreads();                                // stage s-1 is consumed: its buffer may be refilled
         if (s + M2S_BUFFERS - 1 < nstages) issue_stage(buf == 0 ? M2S_BUFFERS - 1 : buf - 1, s + M2S_BUFFERS - 1);
+        if (!BULK) asm volatile("cp.async.commit_group;" ::: "memory");
         int qn = a.rpg;
         if (s == nstages - 1) {                         // last stage of the slice: only the rows that exist
             const int rows = (int)(n_end - n_begin - (int64_t)s * stage_rows);
@@ -132,7 +187,7 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
             if (qn > a.rpg) qn = a.rpg;
         }
         if (active) {
-            const float *row = smem + buf * stage_floats + item_rg * a.d;
+            const float *row = smem + buf * stage_floats + item_rg * a.pitch;
 #pragma unroll 2
             for (int q = 0; q < qn; ++q, row += step) {
                 const float4 s0 = *reinterpret_cast<const float4 *>(row + os);
@@ -159,7 +214,7 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
         }
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the sum over the slices may be launched; it waits for this grid to end
-    if (*abort_flag && tid == 0) {
+    if (BULK && *abort_flag && tid == 0) {
         // after a time-out: give the copies still in flight a bounded time to land before the
         // shared memory is reused or released
         for (int s = (nstages > M2S_BUFFERS ? nstages - M2S_BUFFERS : 0); s < nstages; ++s)
@@ -169,11 +224,13 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
     __syncthreads();                                   // every thread is done with the stage buffers
 
     // block-level sum over the row groups, in group order (reproducible): the sums go to shared
-    // memory as red[k][group][item] (consecutive threads, consecutive words; k < 64 is tile {s,p},
-    // k >= 64 tile {s,q}), output (k, item) is then summed over the groups by `parts` threads, each
-    // over a fixed range, and by one thread over the parts.
+    // memory as red[k][group][item] (k < 64 is tile {s,p}, k >= 64 tile {s,q}), output (k, item) is then
+    // summed over the groups by `parts` threads, each over a fixed range, and by one thread over the parts.
+    // The pitch of k is nitems modulo 32 words: consecutive threads, which own consecutive (k, item), then read
+    // consecutive words (with one item and an unpadded pitch all 32 lanes of a warp met in one bank:
+    // [10000,8] 21 us the call, now 6.6).
     float *red = smem;
-    const int cells = a.rg * nitems;
+    const int cells = m2s_red_pitch(a.rg, nitems);
     if (active) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -194,6 +251,7 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
             const int k = o / nitems, t = o - k * nitems;
             const float *p = red + k * cells + t;
             float sum = 0.f;
+#pragma unroll 8
             for (int g = 0; g < a.rg; ++g) sum += p[g * nitems];
             mine[o] = sum;
         }
@@ -207,6 +265,7 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
             int g_end = (part + 1) * per;
             if (g_end > a.rg) g_end = a.rg;
             float sum = 0.f;
+#pragma unroll 8
             for (int g = part * per; g < g_end; ++g) sum += p[g * nitems];
             scratch[part * nout + o] = sum;
         }
@@ -219,105 +278,85 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
     }
 }
 
-// out[p(ci,cj)] = sum over the slices, in slice order, of element (k, item) of the partials.
+// out[p(ci,cj)] = sum over the slices of element (k, item) of the partials: a block owns 32 elements, warp w adds the
+// slices w, w + 8, ... with all its loads in flight, then the eight sums are added in order (a fixed order).
 __global__ void __launch_bounds__(256)
 moment2_small_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int nbk, int slices,
-                            int dense, const M2SmallItems items)
+                            int dense, int nitems)
 {
+    __shared__ float part[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int o = blockIdx.x * 32 + lane;              // < nitems * 128, a multiple of 32
+    const int k = o / nitems, item = o - k * nitems;
+    const int i8 = (k >> 3) & 7, j8 = k & 7;
+    int x, p, q;
+    m2s_item(item, nbk, dense != 0, x, p, q);
+    const int y = (k < 64) ? p : q;
+    const int ci = m2s_column(x, i8, 4 * nbk), cj = m2s_column(y, j8, 4 * nbk);
+    // not an output: the second tile of the odd item out; the lower half of a diagonal tile (the dense control also
+    // computes the tiles below the diagonal and discards them here); the padding of the last column blocks
+    const bool use = y >= 0 && !((x == y && i8 > j8) || (dense && x > y)) && ci < d && cj < d;
+    const int64_t at = tri_encode(d, ci < cj ? ci : cj, ci < cj ? cj : ci);
     // launched as a programmatic dependent of the kernel that writes the partial sums: the launch overlaps
     // that kernel's tail, and nothing is read before it has completed
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int o = blockIdx.x * 256 + threadIdx.x;
-    const int nitems = items.n;
-    if (o >= nitems * 128) return;
-    const int k = o / nitems, item = o - k * nitems;
-    const int i8 = (k >> 3) & 7, j8 = k & 7;
-    const int x = items.s[item];
-    const int y = (k < 64) ? items.p[item] : items.q[item];
-    if (y == 255) return;                              // odd item out: no second tile
-    // a diagonal tile keeps its upper half; the dense control also computes the tiles below the
-    // diagonal and discards them here
-    if ((x == y && i8 > j8) || (dense && x > y)) return;
-    const int ci = m2s_column(x, i8, 4 * nbk), cj = m2s_column(y, j8, 4 * nbk);
-    float s = 0.f;
     const size_t stride = (size_t)nitems * 128;
-    for (int k0 = 0; k0 < slices; k0 += 32) {
-        float v[32];
+    float s = 0.f;
+    for (int k0 = warp; k0 < slices; k0 += 8 * 20) {   // 148 slices: one batch
+        float v[20];
 #pragma unroll
-        for (int u = 0; u < 32; ++u) v[u] = (k0 + u < slices) ? __ldcg(partials + (size_t)(k0 + u) * stride + o) : 0.f;
+        for (int u = 0; u < 20; ++u) v[u] = (use && k0 + 8 * u < slices) ? __ldcg(partials + (size_t)(k0 + 8 * u) * stride + o) : 0.f;
 #pragma unroll
-        for (int u = 0; u < 32; ++u) s += v[u];
+        for (int u = 0; u < 20; ++u) s += v[u];
     }
-    const int64_t at = tri_encode(d, ci < cj ? ci : cj, ci < cj ? cj : ci);
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || !use) return;
+    s = part[0][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += part[w][lane];
     if (ST_BOUNDS_OK(at, tri_rows(d), 2)) out[at] = s;
 }
 
 struct M2SmallPlan {
-    int nbk, rg, rpg, threads, slices;
+    int nbk, pitch, nitems, rg, rpg, threads, slices;
     int64_t rows_per_slice;
     size_t smem, data_bytes, partial_bytes;
-    M2SmallItems items;
 };
 
-bool moment2_small_applies(int64_t N, int64_t d)
+// FMA slots that the kernel occupies per sample row (idle threads included); 0 when it does not cover d.
+int64_t moment2_small_slots(int64_t d, unsigned flags)
 {
-    return d % 8 == 0 && d >= 8 && d <= 64 && N >= 1;
-}
-
-// Pairs the tiles up into items with a common block.  Structured: for every block y the tiles
-// {x,y}, x <= y, are paired along x with y as the common block; when their number is odd, tile
-// {0,y} is held back, and the held-back tiles are paired with block 0 in common.  Dense control:
-// all ordered tiles (x,y), paired along y with x in common.
-static M2SmallItems moment2_small_items(int nbk, bool dense)
-{
-    M2SmallItems t;
-    t.n = 0;
-    auto add = [&](int s, int p, int q) {
-        t.s[t.n] = (unsigned char)s;
-        t.p[t.n] = (unsigned char)p;
-        t.q[t.n] = (unsigned char)q;
-        ++t.n;
-    };
-    if (dense) {
-        for (int x = 0; x < nbk; ++x)
-            for (int y = 0; y < nbk; y += 2) add(x, y, y + 1 < nbk ? y + 1 : 255);
-    } else {
-        int held[8], nheld = 0;
-        for (int y = 0; y < nbk; ++y) {
-            int x = 0;
-            if ((y + 1) % 2 == 1) {
-                held[nheld++] = y;
-                x = 1;
-            }
-            for (; x + 1 <= y; x += 2) add(y, x, x + 1);
-        }
-        for (int h = 0; h < nheld; h += 2) add(0, held[h], h + 1 < nheld ? held[h + 1] : 255);
-    }
-    for (int i = t.n; i < M2S_MAX_ITEMS; ++i) t.s[i] = t.p[i] = t.q[i] = 0;
-    return t;
+    const int64_t nbk = (d + 7) / 8;
+    if (nbk > M2S_MAX_BLOCKS) return 0;
+    const int n = m2s_nitems((int)nbk, (flags & ST_FLAG_DENSE_CONTROL) != 0);
+    if (n > M2S_MAX_THREADS) return 0;
+    return 128 * M2S_MAX_THREADS / (M2S_MAX_THREADS / n);
 }
 
 static M2SmallPlan moment2_small_plan(int64_t N, int64_t d, unsigned flags)
 {
     M2SmallPlan p;
-    p.nbk = (int)d / 8;
-    p.items = moment2_small_items(p.nbk, (flags & ST_FLAG_DENSE_CONTROL) != 0);
-    const int nitems = p.items.n;
-    const int max_stage_rows = M2S_STAGE_BYTES / (4 * (int)d);
+    p.nbk = (int)(d + 7) / 8;
+    const int nitems = p.nitems = m2s_nitems(p.nbk, (flags & ST_FLAG_DENSE_CONTROL) != 0);
+    p.pitch = (int)(d + 3) / 4 * 4;
+    const int max_stage_rows = M2S_STAGE_BYTES / (4 * p.pitch);
     p.rg = M2S_MAX_THREADS / nitems;
     if (p.rg > max_stage_rows / 8) p.rg = max_stage_rows / 8;
     if (p.rg < 1) p.rg = 1;
     p.threads = (nitems * p.rg + 31) / 32 * 32;
     p.rpg = 8;
     int64_t slices = sm_count_or_default();
-    const int64_t max_slices = (N + p.rg * 8 - 1) / (p.rg * 8);
+    // few samples: shorter slices fill more SMs (four rows per thread and stage: [4096,64] 9.4 us, eight 10.2, two 14.1)
+    while (p.rpg > 4 && N <= slices * p.rg * p.rpg / 2) p.rpg /= 2;
+    const int64_t max_slices = (N + p.rg * p.rpg - 1) / (p.rg * p.rpg);
     if (slices > max_slices) slices = max_slices;
     p.rows_per_slice = (N + slices - 1) / slices;
     p.slices = (int)((N + p.rows_per_slice - 1) / p.rows_per_slice);
     // long slices: 16 rows per thread and stage halve the number of block-wide barriers
     if (p.rg * 16 <= max_stage_rows && p.rows_per_slice >= 4 * p.rg * 16) p.rpg = 16;
-    const size_t cells = (size_t)p.rg * nitems;
-    const size_t main_bytes = (size_t)M2S_BUFFERS * p.rg * p.rpg * d * sizeof(float);
+    const size_t cells = (size_t)m2s_red_pitch(p.rg, nitems);
+    const size_t main_bytes = (size_t)M2S_BUFFERS * p.rg * p.rpg * p.pitch * sizeof(float) + 32;   // the last row is read past its end
     const size_t sum_bytes = (128 * cells + (size_t)M2S_MAX_THREADS) * sizeof(float);
     p.data_bytes = round_up(main_bytes > sum_bytes ? main_bytes : sum_bytes, 16);
     p.smem = p.data_bytes + 64;                        // barriers and the abort flag behind the data
@@ -340,17 +379,22 @@ st_status moment2_small(const float *X, int64_t N, int64_t d, int64_t ldx, float
     a.X = X;
     a.partials = (float *)((unsigned char *)ws + kWsHeaderBytes);
     a.N = N; a.ldx = ldx; a.rows_per_slice = p.rows_per_slice;
-    a.d = (int)d; a.nbk = p.nbk; a.rg = p.rg; a.rpg = p.rpg;
-    a.items = p.items;
+    a.d = (int)d; a.pitch = p.pitch; a.nbk = p.nbk; a.rg = p.rg; a.rpg = p.rpg;
+    a.nitems = p.nitems;
     a.status = (unsigned *)ws;
     a.bar_floats = (int)(p.data_bytes / sizeof(float));
     a.dense = (flags & ST_FLAG_DENSE_CONTROL) ? 1 : 0;
-    if (!ensure_dynamic_smem(moment2_small_kernel, p.smem)) return ST_ERR_CUDA;
-    moment2_small_kernel<<<p.slices, p.threads, p.smem, stream>>>(a);
+    if (d % 4 == 0 && ldx % 4 == 0) {
+        if (!ensure_dynamic_smem(moment2_small_kernel<true>, p.smem)) return ST_ERR_CUDA;
+        moment2_small_kernel<true><<<p.slices, p.threads, p.smem, stream>>>(a);
+    } else {
+        if (!ensure_dynamic_smem(moment2_small_kernel<false>, p.smem)) return ST_ERR_CUDA;
+        moment2_small_kernel<false><<<p.slices, p.threads, p.smem, stream>>>(a);
+    }
     if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
-    const int n = p.items.n * 128;
+    const int n = p.nitems * 128;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((n + 255) / 256));
+    cfg.gridDim = dim3((unsigned)(n / 32));
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = stream;
@@ -361,7 +405,7 @@ st_status moment2_small(const float *X, int64_t N, int64_t d, int64_t ldx, float
     cfg.numAttrs = 1;
     const float *partials = a.partials;
     const int di = (int)d, dense = a.dense;
-    if (cudaLaunchKernelEx(&cfg, moment2_small_reduce_kernel, partials, out, di, p.nbk, p.slices, dense, p.items) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, moment2_small_reduce_kernel, partials, out, di, p.nbk, p.slices, dense, p.nitems) != cudaSuccess) {
         (void)cudaGetLastError();
         return ST_ERR_CUDA;
     }

@@ -239,6 +239,19 @@ def test_moment2_f32_many_features(st, N, d):
         assert oracle.rel_err(expand2(st, out, d), Tw, Sw) <= TOL_F32
 
 
+# register-tile kernel (up to 248 features, rows copied whole or word by word) and 128 x 128 tiles with a last tile
+# column that is one column, half or all but one column wide; slices from one row up, splits with a ragged tail
+@pytest.mark.parametrize("N,d", [(1, 7), (147, 9), (3001, 15), (20011, 33), (4097, 65), (1185, 75), (500, 121), (257, 176),
+                                 (301, 191), (700, 192), (129, 193), (65, 247), (999, 248), (64, 249), (513, 257), (511, 320),
+                                 (80, 321), (2500, 383)])
+def test_moment2_f32_edges_of_both_kernels(st, N, d):
+    X = workloads.draw((N, d), "normal", 170 + N + d)
+    T, S = oracle.moment2(X)
+    for flags in (0, st.ST_FLAG_DENSE_CONTROL):
+        got = expand2(st, st.st_sym_moment2(dev(X), flags=flags), d)
+        assert oracle.rel_err(got, T, S) <= TOL_F32, (N, d, flags)
+
+
 def test_moment2_f32_strided_rows_and_all_ones(st):
     N, d, ldx = 300, 20, 28
     buf = workloads.draw((N, ldx), "normal", 5)
