@@ -1,21 +1,30 @@
 // st_pack / st_unpack: gather the unique set T_U of a dense tensor into the packed layout
 // (T_C = T * T_U, Section 4) and reconstruct the dense tensor from it
-// (T = T_C + T_R * T_C, Section 6, Property 5).  HBM-bound index-decode copies.
+// (T = T_C + T_R * T_C, Section 6, Property 5).  HBM-bound copies.
 //
-// Two kernels.
-//   slice_copy_kernel (st_pack, st_unpack with zero fill): the dense array is cut into slices
-//   along its last structured index (matrix row i; pair (i,j) of an order-3 tensor).  In every
-//   supported structure the unique positions of a slice are ONE contiguous run of columns
-//   [lo,hi) that is also contiguous in the packed array, so a slice is "zeros, one flat copy,
-//   zeros" and needs no per-element index arithmetic at all: the run and its packed offset come
-//   from the closed forms of st_index.cuh once per slice.  Copies run in units of U bytes (16
-//   where the row width allows); long slices are split into parts over several thread groups.
-//   structured_copy_kernel (st_unpack with symmetric fill): one lane group per dense row
-//   decodes its index tuple, maps it through the redundancy map and copies the row.
+// The dense array is cut into slices along its last structured index (matrix row i; pair (i,j) of an
+// order-3 tensor, triple of an order-4 one).
+//   slice_copy_kernel (st_pack, st_thp, st_unpack with zero fill): in every supported structure the unique
+//   positions of a slice are ONE contiguous run of columns [lo,hi) that is also contiguous in the packed
+//   array, so a slice is "zeros, one flat copy, zeros" and needs no per-element index arithmetic at all: the
+//   run and its packed offset come from the closed forms of st_index.cuh once per slice.  Long slices are
+//   split into parts over several thread groups.
+//   sym_slice_kernel (st_unpack with symmetric fill): the positions of a slice from its largest fixed index on
+//   are such a run too; in front of it every position is mapped through the redundancy map by itself.
+//   sym_tile_kernel: the same for a matrix of single elements, through 32 x 32 tiles.
+//
+// A run starts wherever the closed form says, so source and destination usually differ in their offset from a
+// 16-byte boundary.  copy_flat stores whole 16-byte units all the same and takes each from the two aligned units
+// that hold it (the second one is an L1 hit), shifted in registers.  Measured against copies in the widest unit that
+// divides a row, each position of a symmetric fill by itself (pack + unpack): tet d = 60, rows of 33 floats, 72 -> 24 us;
+// tri d = 900, rows of 17 bf16, 125 -> 27 us; simplex4 d = 50 floats, 87 -> 22 us; tet d = 175 bf16, 55 -> 17 us.
 #include "st_common.cuh"
 #include "st_index.cuh"
 
 namespace st {
+
+constexpr int COPY_UNITS = 4;              // 16-byte units that a thread of the slice copies has in flight
+constexpr int64_t PART_BYTES = 32768;      // most of a slice that one thread group copies ([384,384,75]: 128 KiB starve the chip)
 
 struct LayoutArgs {
     int kind;
@@ -24,175 +33,95 @@ struct LayoutArgs {
     int64_t width;       // band: kl+ku+1
     int64_t packed_rows;
     int64_t dense_rows;
-    int64_t chunks;      // units of U bytes per row
+    int64_t row_bytes;   // of one position (`inner` elements)
 };
 
-// Dense row index of packed row p, or -1 for a band slot outside the matrix.
-template <int KIND>
-__device__ __forceinline__ int64_t dense_row_of_packed(const LayoutArgs &a, int64_t p)
+template <int ES> struct Elem;
+template <> struct Elem<2> { typedef uint16_t T; };
+template <> struct Elem<4> { typedef uint32_t T; };
+template <> struct Elem<8> { typedef uint2 T; };
+
+// 16 bytes at byte `off` (a multiple of ES) of the two aligned units at p.
+template <int ES>
+__device__ __forceinline__ uint4 load_unit(const uint4 *p, unsigned off)
 {
-    if (KIND == ST_TRI_UPPER) {
-        int64_t i, j;
-        tri_decode(a.d, p, i, j);
-        return i * a.d + j;
-    } else if (KIND == ST_TET) {
-        int64_t i, j, k;
-        tet_decode(a.d, p, i, j, k);
-        return (i * a.d + j) * a.d + k;
-    } else if (KIND == ST_BAND) {
-        const int64_t i = p / a.width;
-        const int64_t j = i + (p - i * a.width) - a.kl;
-        return (j >= 0 && j < a.d) ? i * a.d + j : -1;
-    } else if (KIND == ST_FIXED_ROW) {
-        return a.kl * a.d + p;
-    } else if (KIND == ST_FIXED_COL) {
-        return p * a.d + a.kl;
-    } else if (KIND == ST_SIMPLEX4) {
-        int64_t i = 0;                                   // slab i: the largest i with simp4_slab_start(d, i) <= p
-        while (i + 1 < a.d && simp4_slab_start(a.d, i + 1) <= p) ++i;
-        int64_t j, k, l;
-        tet_decode(a.d - i, p - simp4_slab_start(a.d, i), j, k, l);
-        return (((i * a.d) + (i + j)) * a.d + (i + k)) * a.d + (i + l);
-    } else {
-        const int64_t bb = a.bs * a.bs;
-        const int64_t b = p / bb;
-        const int64_t rem = p - b * bb;
-        const int64_t ii = rem / a.bs;
-        const int64_t jj = rem - ii * a.bs;
-        return (b * a.bs + ii) * a.d + b * a.bs + jj;
+    const uint4 a = __ldg(p);
+    if (off == 0) return a;
+    const uint4 b = __ldg(p + 1);
+    uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x;
+    if (off & 8) { w0 = a.z; w1 = a.w; w2 = b.x; w3 = b.y; w4 = b.z; }
+    if (ES < 8) {
+        const uint32_t w5 = (off & 8) ? b.w : b.y;
+        if (off & 4) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
     }
-}
-
-// Packed row that dense row r is read from, or -1 when the position is a structural zero.
-template <int KIND>
-__device__ __forceinline__ int64_t packed_row_of_dense(const LayoutArgs &a, int64_t r)
-{
-    if (KIND == ST_TRI_UPPER) {
-        int64_t i = r / a.d, j = r - i * a.d;
-        if (i > j) {
-            if (a.fill != ST_FILL_SYMMETRIC) return -1;
-            int64_t t = i; i = j; j = t;     // T_R(i,j,i',j') = (j<i)*(i'=j)*(j'=i)
-        }
-        return tri_encode(a.d, i, j);
-    } else if (KIND == ST_TET) {
-        const int64_t ij = r / a.d;
-        int64_t k = r - ij * a.d;
-        int64_t i = ij / a.d, j = ij - i * a.d;
-        if (!(i <= j && j <= k)) {
-            if (a.fill != ST_FILL_SYMMETRIC) return -1;
-            int64_t t;                        // representative = sorted index triple
-            if (i > j) { t = i; i = j; j = t; }
-            if (j > k) { t = j; j = k; k = t; }
-            if (i > j) { t = i; i = j; j = t; }
-        }
-        return tet_encode(a.d, i, j, k);
-    } else if (KIND == ST_BAND) {
-        const int64_t i = r / a.d, j = r - i * a.d;
-        const int64_t s = j - i + a.kl;
-        return (s >= 0 && s < a.width) ? i * a.width + s : -1;
-    } else if (KIND == ST_FIXED_ROW) {
-        const int64_t i = r / a.d;
-        return i == a.kl ? r - i * a.d : -1;
-    } else if (KIND == ST_FIXED_COL) {
-        const int64_t i = r / a.d;
-        return r - i * a.d == a.kl ? i : -1;
-    } else if (KIND == ST_SIMPLEX4) {
-        int64_t v[4];
-        int64_t q = r;
-        v[3] = q % a.d; q /= a.d;
-        v[2] = q % a.d; q /= a.d;
-        v[1] = q % a.d; v[0] = q / a.d;
-        if (!(v[0] <= v[1] && v[1] <= v[2] && v[2] <= v[3])) {
-            if (a.fill != ST_FILL_SYMMETRIC) return -1;
-            // representative = sorted index tuple (sorting network for four keys)
-#define ST_CSWAP(x, y) { if (v[x] > v[y]) { const int64_t t = v[x]; v[x] = v[y]; v[y] = t; } }
-            ST_CSWAP(0, 1) ST_CSWAP(2, 3) ST_CSWAP(0, 2) ST_CSWAP(1, 3) ST_CSWAP(1, 2)
-#undef ST_CSWAP
-        }
-        return simp4_encode(a.d, v[0], v[1], v[2], v[3]);
-    } else {
-        const int64_t i = r / a.d, j = r - i * a.d;
-        const int64_t b = i / a.bs;
-        if (j / a.bs != b) return -1;
-        return (i * a.bs) + (j - b * a.bs);   // ((b*bs + i')*bs + j') with b*bs+i' = i
+    if (ES < 4 && (off & 2)) {
+        w0 = __funnelshift_r(w0, w1, 16);
+        w1 = __funnelshift_r(w1, w2, 16);
+        w2 = __funnelshift_r(w2, w3, 16);
+        w3 = __funnelshift_r(w3, w4, 16);
     }
+    return make_uint4(w0, w1, w2, w3);
 }
 
-template <typename U>
-__device__ __forceinline__ U zero_unit();
-template <> __device__ __forceinline__ uint4 zero_unit<uint4>() { return make_uint4(0, 0, 0, 0); }
-template <> __device__ __forceinline__ uint2 zero_unit<uint2>() { return make_uint2(0, 0); }
-template <> __device__ __forceinline__ uint32_t zero_unit<uint32_t>() { return 0u; }
-template <> __device__ __forceinline__ uint16_t zero_unit<uint16_t>() { return 0; }
+__device__ __forceinline__ uint32_t mul_word(uint32_t a, uint32_t b) { return __float_as_uint(__uint_as_float(a) * __uint_as_float(b)); }
 
-// Element-wise product of two units of fp32 values (the Hadamard variant of st_pack).
-__device__ __forceinline__ uint4 mul_unit(uint4 a, uint4 b)
+// dst[0..n) = src[0..n) (bytes, multiples of ES) by the `g` threads of a group, U units of a thread in flight; MUL:
+// times mul[0..n), fp32, which is offset from a 16-byte boundary as dst is.  The elements in front of the first whole
+// unit of dst and behind the last one are loaded ahead of the units, so that they cost no round trip of their own.
+template <int ES, bool MUL, int U>
+__device__ __forceinline__ void copy_flat(unsigned char *dst, const unsigned char *src, const unsigned char *mul, int n, int lane, int g)
 {
-    return make_uint4(__float_as_uint(__uint_as_float(a.x) * __uint_as_float(b.x)),
-                      __float_as_uint(__uint_as_float(a.y) * __uint_as_float(b.y)),
-                      __float_as_uint(__uint_as_float(a.z) * __uint_as_float(b.z)),
-                      __float_as_uint(__uint_as_float(a.w) * __uint_as_float(b.w)));
-}
-__device__ __forceinline__ uint2 mul_unit(uint2 a, uint2 b)
-{
-    return make_uint2(__float_as_uint(__uint_as_float(a.x) * __uint_as_float(b.x)),
-                      __float_as_uint(__uint_as_float(a.y) * __uint_as_float(b.y)));
-}
-__device__ __forceinline__ uint32_t mul_unit(uint32_t a, uint32_t b)
-{
-    return __float_as_uint(__uint_as_float(a) * __uint_as_float(b));
-}
-__device__ __forceinline__ uint16_t mul_unit(uint16_t a, uint16_t) { return a; }   // not reached: fp32 rows are whole words
-
-// PACK = true : rows of `dst` are packed rows, source rows are dense rows.
-// PACK = false: rows of `dst` are dense rows, source rows are packed rows.
-template <int KIND, typename U, bool PACK>
-__global__ void __launch_bounds__(256)
-structured_copy_kernel(const U *__restrict__ src, U *__restrict__ dst, LayoutArgs a, int group_shift)
-{
-    const int64_t rows = PACK ? a.packed_rows : a.dense_rows;
-    const int g = 1 << group_shift;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t groups = ((int64_t)gridDim.x * blockDim.x) >> group_shift;
-    const int lane = (int)(tid & (g - 1));
-    for (int64_t row = tid >> group_shift; row < rows; row += groups) {
-        const int64_t srow = PACK ? dense_row_of_packed<KIND>(a, row) : packed_row_of_dense<KIND>(a, row);
-        U *out = dst + row * a.chunks;
-        if (srow >= 0 && !ST_BOUNDS_OK(srow, PACK ? a.dense_rows : a.packed_rows, 1)) continue;
-        if (srow >= 0) {
-            const U *in = src + srow * a.chunks;
-            for (int64_t c = lane; c < a.chunks; c += g) out[c] = in[c];
-        } else {
-            for (int64_t c = lane; c < a.chunks; c += g) out[c] = zero_unit<U>();
-        }
+    typedef typename Elem<ES>::T E;
+    int head = (int)((0u - (unsigned)(uintptr_t)dst) & 15u);
+    if (head > n) head = n;
+    const int units = (n - head) >> 4;
+    const int ends = n - (units << 4);
+    auto end_at = [&](int e) { return e < head ? e : e + (units << 4); };
+    auto end_load = [&](int e) {
+        E v = __ldg(reinterpret_cast<const E *>(src + end_at(e)));
+        if constexpr (MUL) v = mul_word(v, __ldg(reinterpret_cast<const uint32_t *>(mul + end_at(e))));
+        return v;
+    };
+    const int e0 = lane * ES;
+    E ev = E{};
+    if (e0 < ends) ev = end_load(e0);
+    const unsigned off = (unsigned)(uintptr_t)(src + head) & 15u;
+    const uint4 *in = reinterpret_cast<const uint4 *>(src + head - off);
+    uint4 *out = reinterpret_cast<uint4 *>(dst + head);
+    const uint4 *m = MUL ? reinterpret_cast<const uint4 *>(mul + head) : nullptr;
+    for (int u0 = lane; u0 < units; u0 += U * g) {
+        uint4 v[U], w[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (u0 + k * g < units) {
+                v[k] = load_unit<ES>(in + u0 + k * g, off);
+                if (MUL) w[k] = __ldg(m + u0 + k * g);
+            }
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (u0 + k * g < units) {
+                if (MUL) v[k] = make_uint4(mul_word(v[k].x, w[k].x), mul_word(v[k].y, w[k].y), mul_word(v[k].z, w[k].z), mul_word(v[k].w, w[k].w));
+                out[u0 + k * g] = v[k];
+            }
     }
+    if (e0 < ends) *reinterpret_cast<E *>(dst + end_at(e0)) = ev;
+    for (int e = e0 + g * ES; e < ends; e += g * ES) *reinterpret_cast<E *>(dst + end_at(e)) = end_load(e);   // small groups only
 }
 
-// Symmetric fill of a plain matrix / order-3 tensor of 4-byte elements (the reconstruction of a moment
-// output): one thread per dense element, indices from the thread coordinates, 32-bit arithmetic only.
-template <int KIND>
-__global__ void __launch_bounds__(256)
-sym_unpack32_kernel(const uint32_t *__restrict__ packed, uint32_t *__restrict__ dense, unsigned d)
+template <int ES>
+__device__ __forceinline__ void zero_flat(unsigned char *dst, int n, int lane, int g)
 {
-    const unsigned x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= d || y >= d) return;
-    if (KIND == ST_TRI_UPPER) {
-        const unsigned i = y < x ? y : x, j = y < x ? x : y;             // representative (min, max): T_R of the symmetric structure
-        dense[y * d + x] = packed[i * (2 * d - i + 1) / 2 + (j - i)];
-    } else {
-        unsigned a = blockIdx.z, b = y, c = x, t;                        // dense (i, j, k) = (z, y, x); sort to a <= b <= c
-        if (a > b) { t = a; a = b; b = t; }
-        if (b > c) { t = b; b = c; c = t; }
-        if (a > b) { t = a; a = b; b = t; }
-        const unsigned m = d - a, jj = b - a, kk = c - a;
-        const unsigned slab = d * (d + 1) / 2 * (d + 2) / 3 - m * (m + 1) / 2 * (m + 2) / 3;
-        dense[(blockIdx.z * d + y) * d + x] = packed[slab + jj * (2 * m - jj + 1) / 2 + (kk - jj)];
-    }
+    typedef typename Elem<ES>::T E;
+    int head = (int)((0u - (unsigned)(uintptr_t)dst) & 15u);
+    if (head > n) head = n;
+    const int units = (n - head) >> 4;
+    const int ends = n - (units << 4);
+    for (int e = lane * ES; e < ends; e += g * ES) *reinterpret_cast<E *>(dst + (e < head ? e : e + (units << 4))) = E{};
+    uint4 *out = reinterpret_cast<uint4 *>(dst + head);
+    for (int u = lane; u < units; u += g) out[u] = make_uint4(0, 0, 0, 0);
 }
 
-// Run of unique columns of slice s, in rows of `chunks` units: dense columns [lo,hi) of the
-// slice map to packed rows prow.. (contiguous).  For ST_BAND also the extent of the fixed-width
-// packed row [band0, band1) whose slots outside the run are zero-filled by pack.
+// Run of unique columns of slice s: dense columns [lo,hi) of the slice map to packed rows prow.. (contiguous).
 template <int KIND>
 __device__ __forceinline__ void slice_run(const LayoutArgs &a, int64_t s, int64_t &lo, int64_t &hi, int64_t &prow)
 {
@@ -224,20 +153,20 @@ __device__ __forceinline__ void slice_run(const LayoutArgs &a, int64_t s, int64_
     }
 }
 
-template <int KIND, typename U, bool PACK>
+template <int KIND, int ES, bool PACK, bool MUL>
 __global__ void __launch_bounds__(256)
-slice_copy_kernel(const U *__restrict__ src, U *__restrict__ dst, LayoutArgs a, int group_shift, int parts,
-                  int64_t part_units, const U *__restrict__ mul)
+slice_copy_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst, LayoutArgs a, int group_shift, int parts,
+                  int part_bytes, const unsigned char *__restrict__ mul)
 {
-    // mul (pack only, fp32 elements): a second packed operand; the gathered values are multiplied by it
+    // MUL (pack only, fp32 elements): a second packed operand; the gathered values are multiplied by it
     const int g = 1 << group_shift;
     const int lane = (int)(threadIdx.x & (g - 1));
     const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> group_shift;
     const int64_t ngroups = ((int64_t)gridDim.x * blockDim.x) >> group_shift;
     const int64_t nslices = (KIND == ST_TET) ? a.d * a.d : (KIND == ST_SIMPLEX4) ? a.d * a.d * a.d : a.d;
-    const int64_t su = a.d * a.chunks;                        // units per dense slice
+    const int64_t sb = a.d * a.row_bytes;                     // bytes per dense slice
     for (int64_t item = gid; item < nslices * parts; item += ngroups) {
-        const int64_t s = item / parts;
+        const int64_t s = parts == 1 ? item : item / parts;
         const int64_t part = item - s * parts;
         int64_t lo, hi, prow;
         slice_run<KIND>(a, s, lo, hi, prow);
@@ -245,39 +174,158 @@ slice_copy_kernel(const U *__restrict__ src, U *__restrict__ dst, LayoutArgs a, 
         if (hi > lo && !(ST_BOUNDS_OK(lo, a.d, 1) && ST_BOUNDS_OK(hi - 1, a.d, 1) && ST_BOUNDS_OK(prow, a.packed_rows, 1) &&
                          ST_BOUNDS_OK(prow + (hi - lo) - 1, a.packed_rows, 1)))
             continue;
-        const int64_t c0 = lo * a.chunks, c1 = hi * a.chunks;  // units of the run inside the slice
+        const int64_t c0 = lo * a.row_bytes, c1 = hi * a.row_bytes;   // the run inside the slice
         // pack splits the run itself into parts, unpack the whole dense slice (it writes all of it)
-        const int64_t r0 = PACK ? c0 : 0, r1 = PACK ? c1 : su;
-        int64_t u0 = r0 + part * part_units;                  // this part covers dense units [u0, u1) of the slice
-        int64_t u1 = u0 + part_units;
+        const int64_t r0 = PACK ? c0 : 0, r1 = PACK ? c1 : sb;
+        int64_t u0 = r0 + part * part_bytes;                  // this part covers dense bytes [u0, u1) of the slice
+        int64_t u1 = u0 + part_bytes;
         if (u0 > r1) u0 = r1;
         if (u1 > r1) u1 = r1;
         const int64_t x0 = u0 > c0 ? u0 : c0, x1 = u1 < c1 ? u1 : c1;   // run clipped to this part
+        const int64_t p0 = prow * a.row_bytes - c0;           // packed byte of dense byte 0 of the slice, were it in the run
         if (PACK) {
-            const U *in = src + s * su;
-            U *out = dst + prow * a.chunks - c0;                // out[u] for dense unit u of the run
-            if (mul) {
-                const U *m = mul + prow * a.chunks - c0;
-                for (int64_t u = x0 + lane; u < x1; u += g) out[u] = mul_unit(in[u], m[u]);
-            } else {
-                for (int64_t u = x0 + lane; u < x1; u += g) out[u] = in[u];
-            }
+            if (x1 > x0) copy_flat<ES, MUL, COPY_UNITS>(dst + p0 + x0, src + s * sb + x0, mul + p0 + x0, (int)(x1 - x0), lane, g);
             if (KIND == ST_BAND && part == 0) {
                 // slots of the fixed-width packed row that fall outside the matrix
-                U *row = dst + s * a.width * a.chunks;
-                const int64_t first = (prow - s * a.width) * a.chunks, last = first + (c1 - c0);
-                const int64_t wu = a.width * a.chunks;
-                for (int64_t u = lane; u < first; u += g) row[u] = zero_unit<U>();
-                for (int64_t u = last + lane; u < wu; u += g) row[u] = zero_unit<U>();
+                unsigned char *row = dst + s * a.width * a.row_bytes;
+                const int64_t first = (prow - s * a.width) * a.row_bytes, last = first + (c1 - c0), wb = a.width * a.row_bytes;
+                for (int64_t z = 0; z < first; z += part_bytes) zero_flat<ES>(row + z, (int)(first - z < part_bytes ? first - z : part_bytes), lane, g);
+                for (int64_t z = last; z < wb; z += part_bytes) zero_flat<ES>(row + z, (int)(wb - z < part_bytes ? wb - z : part_bytes), lane, g);
             }
         } else {
-            U *out = dst + s * su;
-            const U *in = src + prow * a.chunks - c0;
+            unsigned char *out = dst + s * sb;
             const int64_t z1 = u1 < c0 ? u1 : c0;               // zeros before the run
-            for (int64_t u = u0 + lane; u < z1; u += g) out[u] = zero_unit<U>();
-            for (int64_t u = x0 + lane; u < x1; u += g) out[u] = in[u];
+            if (z1 > u0) zero_flat<ES>(out + u0, (int)(z1 - u0), lane, g);
+            if (x1 > x0) copy_flat<ES, false, COPY_UNITS>(out + x0, src + p0 + x0, nullptr, (int)(x1 - x0), lane, g);
             const int64_t z2 = u0 > c1 ? u0 : c1;               // zeros after the run
-            for (int64_t u = z2 + lane; u < u1; u += g) out[u] = zero_unit<U>();
+            if (u1 > z2) zero_flat<ES>(out + z2, (int)(u1 - z2), lane, g);
+        }
+    }
+}
+
+// Closed forms of st_index.cuh in the index type I: unsigned where every index fits in 31 bits.
+template <typename I> __device__ __forceinline__ I tri_n(I d) { return d * (d + 1) / 2; }
+template <typename I> __device__ __forceinline__ I tet_n(I d) { return d * (d + 1) / 2 * (d + 2) / 3; }
+template <typename I> __device__ __forceinline__ I simp4_n(I d) { return tet_n<I>(d) * (d + 3) / 4; }
+template <typename I> __device__ __forceinline__ I tri_at(I d, I i, I j) { return i * (2 * d - i + 1) / 2 + (j - i); }
+template <typename I> __device__ __forceinline__ I tet_at(I d, I i, I j, I k) { return tet_n<I>(d) - tet_n<I>(d - i) + tri_at<I>(d - i, j - i, k - i); }
+template <typename I> __device__ __forceinline__ I simp4_at(I d, I i, I j, I k, I l) { return simp4_n<I>(d) - simp4_n<I>(d - i) + tet_at<I>(d - i, j - i, k - i, l - i); }
+
+// Packed row of position x of the slice whose fixed indices are a <= b <= c (as many as KIND has); x < the largest.
+template <int KIND, typename I>
+__device__ __forceinline__ I sym_row(I d, I a, I b, I c, I x)
+{
+    if (KIND == ST_TRI_UPPER) return tri_at<I>(d, x, a);
+    if (KIND == ST_TET) return x < a ? tet_at<I>(d, x, a, b) : tet_at<I>(d, a, x, b);
+    return x < a ? simp4_at<I>(d, x, a, b, c) : x < b ? simp4_at<I>(d, a, x, b, c) : simp4_at<I>(d, a, b, x, c);
+}
+
+// One warp per part of a slice.  Positions from the largest fixed index on: one flat copy.  In front of it a lane
+// group per position (`inner` elements), or a lane per position when it is a single element.
+template <int KIND, int ES, typename I>
+__global__ void __launch_bounds__(256)
+sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst, I d, I nslices, int parts, int part_rows,
+                 int row_bytes, int group_shift, int64_t packed_rows)
+{
+    typedef typename Elem<ES>::T E;
+    const int lane = (int)(threadIdx.x & 31);
+    const I nitems = nslices * (I)parts, nwarps = (I)gridDim.x * (I)(blockDim.x / 32);
+    for (I item = (I)blockIdx.x * (I)(blockDim.x / 32) + (I)(threadIdx.x / 32); item < nitems; item += nwarps) {
+        const I s = parts == 1 ? item : item / (I)parts;
+        const I x0 = (item - s * (I)parts) * (I)part_rows;
+        const I x1 = x0 + (I)part_rows < d ? x0 + (I)part_rows : d;
+        I a, b = 0, c = 0, top, t;                                       // fixed indices in increasing order
+        if (KIND == ST_TRI_UPPER) {
+            a = top = s;
+        } else if (KIND == ST_TET) {
+            a = s / d; b = s - a * d;
+            if (a > b) { t = a; a = b; b = t; }
+            top = b;
+        } else {
+            const I ij = s / d;
+            c = s - ij * d; a = ij / d; b = ij - a * d;
+            if (a > b) { t = a; a = b; b = t; }
+            if (b > c) { t = b; b = c; c = t; }
+            if (a > b) { t = a; a = b; b = t; }
+            top = c;
+        }
+        unsigned char *out = dst + (int64_t)s * d * row_bytes;
+        const I xr = x0 > top ? x0 : top;                                // first position of the run in this part
+        if (xr < x1) {
+            const I p = KIND == ST_TRI_UPPER ? tri_at<I>(d, a, xr) : KIND == ST_TET ? tet_at<I>(d, a, b, xr) : simp4_at<I>(d, a, b, c, xr);
+            if (ST_BOUNDS_OK(p, packed_rows, 1) && ST_BOUNDS_OK((int64_t)p + (x1 - xr) - 1, packed_rows, 1))
+                copy_flat<ES, false, 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32);
+        }
+        const I xe = x1 < top ? x1 : top;
+        if (row_bytes == ES) {
+            for (I x = x0 + (I)lane; x < xe; x += 32) {
+                const I p = sym_row<KIND, I>(d, a, b, c, x);
+                if (ST_BOUNDS_OK(p, packed_rows, 1)) reinterpret_cast<E *>(out)[x] = __ldg(reinterpret_cast<const E *>(src) + p);
+            }
+        } else {
+            const int g = 1 << group_shift;
+            for (I x = x0 + (I)(lane >> group_shift); x < xe; x += (I)(32 >> group_shift)) {
+                const I p = sym_row<KIND, I>(d, a, b, c, x);
+                if (ST_BOUNDS_OK(p, packed_rows, 1))
+                    copy_flat<ES, false, 1>(out + (int64_t)x * row_bytes, src + (int64_t)p * row_bytes, nullptr, row_bytes, lane & (g - 1), g);
+            }
+        }
+    }
+}
+
+// Symmetric fill of single elements (the reconstruction of a moment).  With the leading indices fixed (none, i, or
+// i1 <= i2) the last two indices span a symmetric matrix; a block reads one 32 x 32 tile (j <= k) of its upper triangle,
+// lanes along k, and writes it twice, the second time transposed through shared memory -- and, for i1 < i2, both again
+// into the slab (i2, i1).  Lanes read consecutive packed words wherever k is the largest index.
+template <int KIND, int ES>
+__global__ void __launch_bounds__(256)
+sym_tile_kernel(const typename Elem<ES>::T *__restrict__ packed, typename Elem<ES>::T *__restrict__ dense, unsigned d, unsigned nt, int64_t packed_rows)
+{
+    typedef typename Elem<ES>::T E;
+    __shared__ E tile[32][33];
+    const unsigned i1 = blockIdx.y, i2 = blockIdx.z;       // leading indices
+    if (KIND == ST_SIMPLEX4 && i1 > i2) return;
+    int64_t bi64, bj64;
+    tri_decode((int64_t)nt, (int64_t)blockIdx.x, bi64, bj64);
+    const unsigned bi = (unsigned)bi64, bj = (unsigned)bj64;
+    const unsigned tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    E *const out = KIND == ST_TRI_UPPER ? dense : KIND == ST_TET ? dense + (size_t)i1 * d * d : dense + ((size_t)i1 * d + i2) * d * d;
+    E *const out2 = KIND == ST_SIMPLEX4 ? dense + ((size_t)i2 * d + i1) * d * d : out;
+    auto at = [&](unsigned j, unsigned k) -> unsigned {     // j <= k
+        if (KIND == ST_TRI_UPPER) return tri_at<unsigned>(d, j, k);
+        if (KIND == ST_TET) return i1 <= j ? tet_at<unsigned>(d, i1, j, k) : i1 <= k ? tet_at<unsigned>(d, j, i1, k) : tet_at<unsigned>(d, j, k, i1);
+        unsigned a = i1, b = i2, c = j, e = k, t;           // two sorted pairs, merged
+        if (a > c) { t = a; a = c; c = t; }
+        if (b > e) { t = b; b = e; e = t; }
+        if (b > c) { t = b; b = c; c = t; }
+        return simp4_at<unsigned>(d, a, b, c, e);
+    };
+    E v[4];
+#pragma unroll
+    for (unsigned q = 0; q < 4; ++q) {
+        const unsigned j = bi * 32 + ty + 8 * q, k = bj * 32 + tx;
+        if (j <= k && k < d) {
+            const unsigned p = at(j, k);
+            v[q] = ST_BOUNDS_OK(p, packed_rows, 1) ? __ldg(packed + p) : E{};
+        }
+    }
+#pragma unroll
+    for (unsigned q = 0; q < 4; ++q) {
+        const unsigned j = bi * 32 + ty + 8 * q, k = bj * 32 + tx;
+        if (j <= k && k < d) {
+            tile[ty + 8 * q][tx] = v[q];
+            out[(size_t)j * d + k] = v[q];
+            if (KIND == ST_SIMPLEX4 && i1 < i2) out2[(size_t)j * d + k] = v[q];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (unsigned q = 0; q < 4; ++q) {
+        const unsigned k = bj * 32 + ty + 8 * q, j = bi * 32 + tx;       // dense row k, column j < k
+        if (j < k && k < d) {
+            const E w = tile[tx][ty + 8 * q];
+            out[(size_t)k * d + j] = w;
+            if (KIND == ST_SIMPLEX4 && i1 < i2) out2[(size_t)k * d + j] = w;
         }
     }
 }
@@ -350,57 +398,87 @@ static int dtype_bytes(st_dtype t)
     }
 }
 
-template <int KIND, typename U, bool PACK>
+template <int KIND, int ES>
+static st_status launch_sym(const void *src, void *dst, const LayoutArgs &a, cudaStream_t s)
+{
+    typedef typename Elem<ES>::T E;
+    // packed indices and d^2 in 32 bits
+    const bool small = a.d <= (KIND == ST_TRI_UPPER ? 32768 : KIND == ST_TET ? 1024 : 200);
+    if (a.row_bytes == ES && small) {
+        const unsigned nt = (unsigned)((a.d + 31) / 32);
+        const dim3 grid(nt * (nt + 1) / 2, KIND == ST_TRI_UPPER ? 1u : (unsigned)a.d, KIND == ST_SIMPLEX4 ? (unsigned)a.d : 1u);
+        sym_tile_kernel<KIND, ES><<<grid, 256, 0, s>>>((const E *)src, (E *)dst, (unsigned)a.d, nt, a.packed_rows);
+        return launch_status();
+    }
+    if (a.row_bytes > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
+    // parts of about 2 KiB, a multiple of 32 positions where a lane takes one each
+    const int64_t part_rows = a.row_bytes == ES ? 128 : (2048 + a.row_bytes - 1) / a.row_bytes;
+    const int64_t parts = (a.d + part_rows - 1) / part_rows;
+    int shift = 0;
+    while (shift < 5 && (int64_t(16) << shift) < a.row_bytes) ++shift;
+    const int64_t nslices = a.dense_rows / a.d, items = nslices * parts;
+    const int64_t want = (items + 7) / 8, cap = (int64_t)sm_count_or_default() * 16;
+    const unsigned grid = (unsigned)(want < cap ? want : cap);
+    const unsigned char *in = (const unsigned char *)src;
+    unsigned char *out = (unsigned char *)dst;
+    if (small && items < (int64_t(1) << 31))
+        sym_slice_kernel<KIND, ES, unsigned><<<grid, 256, 0, s>>>(in, out, (unsigned)a.d, (unsigned)nslices, (int)parts, (int)part_rows,
+                                                                   (int)a.row_bytes, shift, a.packed_rows);
+    else
+        sym_slice_kernel<KIND, ES, int64_t><<<grid, 256, 0, s>>>(in, out, a.d, nslices, (int)parts, (int)part_rows, (int)a.row_bytes,
+                                                                  shift, a.packed_rows);
+    return launch_status();
+}
+
+template <int KIND, int ES, bool PACK>
 static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cudaStream_t s, const void *mul)
 {
     const int64_t cap = (int64_t)sm_count_or_default() * 16;
-    if (!PACK && a.fill == ST_FILL_SYMMETRIC && sizeof(U) == 4 && a.chunks == 1 &&
-        ((KIND == ST_TRI_UPPER && a.d <= 32768) || (KIND == ST_TET && a.d <= 1024))) {
-        const dim3 block(32, 8), grid((unsigned)((a.d + 31) / 32), (unsigned)((a.d + 7) / 8), KIND == ST_TET ? (unsigned)a.d : 1u);
-        sym_unpack32_kernel<(KIND == ST_TET ? ST_TET : ST_TRI_UPPER)><<<grid, block, 0, s>>>((const uint32_t *)src, (uint32_t *)dst, (unsigned)a.d);
-        return launch_status();
-    }
-    if (!PACK && a.fill == ST_FILL_SYMMETRIC) {
-        // redundancy map: one lane group per dense row
-        int shift = 0;
-        while ((1 << shift) < 32 && (int64_t(1) << shift) < a.chunks) ++shift;
-        const int64_t threads = a.dense_rows << shift;
-        const int64_t want = (threads + 255) / 256;
-        const int grid = (int)(want < cap ? (want < 1 ? 1 : want) : cap);
-        structured_copy_kernel<KIND, U, PACK><<<grid, 256, 0, s>>>((const U *)src, (U *)dst, a, shift);
-        return launch_status();
-    }
-    // slices: about 8 units per thread, at most 8192 units per (slice, part).  Pack splits the
+    // slices: about four 16-byte units per thread, at most PART_BYTES per (slice, part).  Pack splits the
     // longest run of unique columns, unpack the whole dense slice.
     int64_t run_rows = a.d;
     if (KIND == ST_BAND) run_rows = a.width < a.d ? a.width : a.d;
     if (KIND == ST_BLOCKDIAG) run_rows = a.bs;
     if (KIND == ST_FIXED_COL) run_rows = 1;
-    const int64_t su = (PACK ? run_rows : a.d) * a.chunks;
-    int parts = (int)((su + 8191) / 8192);
-    if (parts < 1) parts = 1;
-    const int64_t pu = (su + parts - 1) / parts;
+    const int64_t sb = (PACK ? run_rows : a.d) * a.row_bytes;
+    int64_t parts = (sb + PART_BYTES - 1) / PART_BYTES;
+    const int64_t pb = ((sb + parts - 1) / parts + 15) / 16 * 16;
+    parts = (sb + pb - 1) / pb;
+    if (parts > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
     int shift = 0;
-    while ((1 << shift) < 256 && (int64_t(8) << shift) < pu) ++shift;
+    while ((1 << shift) < 256 && (int64_t(16 * COPY_UNITS) << shift) < pb) ++shift;
     const int64_t nslices = (KIND == ST_TET) ? a.d * a.d : (KIND == ST_SIMPLEX4) ? a.d * a.d * a.d : a.d;
     const int64_t threads = (nslices * parts) << shift;
     const int64_t want = (threads + 255) / 256;
     const int grid = (int)(want < cap ? (want < 1 ? 1 : want) : cap);
-    slice_copy_kernel<KIND, U, PACK><<<grid, 256, 0, s>>>((const U *)src, (U *)dst, a, shift, parts, pu, (const U *)mul);
+    const unsigned char *in = (const unsigned char *)src, *m = (const unsigned char *)mul;
+    unsigned char *out = (unsigned char *)dst;
+    if constexpr (PACK && ES == 4) {
+        if (mul) {
+            slice_copy_kernel<KIND, ES, PACK, true><<<grid, 256, 0, s>>>(in, out, a, shift, (int)parts, (int)pb, m);
+            return launch_status();
+        }
+    }
+    slice_copy_kernel<KIND, ES, PACK, false><<<grid, 256, 0, s>>>(in, out, a, shift, (int)parts, (int)pb, m);
     return launch_status();
 }
 
-template <typename U, bool PACK>
+template <int ES, bool PACK>
 static st_status dispatch_kind(const void *src, void *dst, const LayoutArgs &a, cudaStream_t s, const void *mul)
 {
+    if constexpr (!PACK) {
+        if (a.fill == ST_FILL_SYMMETRIC)
+            return a.kind == ST_TRI_UPPER ? launch_sym<ST_TRI_UPPER, ES>(src, dst, a, s)
+                 : a.kind == ST_TET ? launch_sym<ST_TET, ES>(src, dst, a, s) : launch_sym<ST_SIMPLEX4, ES>(src, dst, a, s);
+    }
     switch (a.kind) {
-    case ST_TRI_UPPER: return launch_copy<ST_TRI_UPPER, U, PACK>(src, dst, a, s, mul);
-    case ST_TET: return launch_copy<ST_TET, U, PACK>(src, dst, a, s, mul);
-    case ST_BAND: return launch_copy<ST_BAND, U, PACK>(src, dst, a, s, mul);
-    case ST_FIXED_ROW: return launch_copy<ST_FIXED_ROW, U, PACK>(src, dst, a, s, mul);
-    case ST_FIXED_COL: return launch_copy<ST_FIXED_COL, U, PACK>(src, dst, a, s, mul);
-    case ST_SIMPLEX4: return launch_copy<ST_SIMPLEX4, U, PACK>(src, dst, a, s, mul);
-    default: return launch_copy<ST_BLOCKDIAG, U, PACK>(src, dst, a, s, mul);
+    case ST_TRI_UPPER: return launch_copy<ST_TRI_UPPER, ES, PACK>(src, dst, a, s, mul);
+    case ST_TET: return launch_copy<ST_TET, ES, PACK>(src, dst, a, s, mul);
+    case ST_BAND: return launch_copy<ST_BAND, ES, PACK>(src, dst, a, s, mul);
+    case ST_FIXED_ROW: return launch_copy<ST_FIXED_ROW, ES, PACK>(src, dst, a, s, mul);
+    case ST_FIXED_COL: return launch_copy<ST_FIXED_COL, ES, PACK>(src, dst, a, s, mul);
+    case ST_SIMPLEX4: return launch_copy<ST_SIMPLEX4, ES, PACK>(src, dst, a, s, mul);
+    default: return launch_copy<ST_BLOCKDIAG, ES, PACK>(src, dst, a, s, mul);
     }
 }
 
@@ -423,13 +501,12 @@ static st_status copy_entry(const st_layout *L, st_dtype dtype, const void *src,
     a.width = L->kl + L->ku + 1;
     a.packed_rows = packed_rows_of(L);
     a.dense_rows = dense_rows_of(L);
-    const int64_t w = L->inner * es;   // bytes per row
+    a.row_bytes = L->inner * es;
     cudaStream_t s = (cudaStream_t)stream;
-    if (w % 16 == 0) { a.chunks = w / 16; return dispatch_kind<uint4, PACK>(src, dst, a, s, mul); }
-    if (w % 8 == 0)  { a.chunks = w / 8;  return dispatch_kind<uint2, PACK>(src, dst, a, s, mul); }
-    if (w % 4 == 0)  { a.chunks = w / 4;  return dispatch_kind<uint32_t, PACK>(src, dst, a, s, mul); }
-    a.chunks = w / 2;
-    return dispatch_kind<uint16_t, PACK>(src, dst, a, s, mul);
+    // the widest word that divides a position's bytes (the product of st_thp is made word by word)
+    if (a.row_bytes % 8 == 0 && !mul) return dispatch_kind<8, PACK>(src, dst, a, s, mul);
+    if (a.row_bytes % 4 == 0) return dispatch_kind<4, PACK>(src, dst, a, s, mul);
+    return dispatch_kind<2, PACK>(src, dst, a, s, mul);
 }
 
 }  // namespace st

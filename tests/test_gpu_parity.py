@@ -129,6 +129,26 @@ def test_pack_unpack_bit_exact(st, inner, dtype):
             assert torch.equal(again, got_p), (lay, "round trip")
 
 
+# symmetric fill: edges of its 32 x 32 tiles, every order; copies: runs that start at any offset from a 16-byte
+# boundary, single elements of every size, slices longer than one part
+@pytest.mark.parametrize("kind,d,inner,dtype", [
+    ("ST_TRI_UPPER", 31, 1, np.uint16), ("ST_TRI_UPPER", 33, 1, np.uint64), ("ST_TRI_UPPER", 65, 2, np.uint32), ("ST_TRI_UPPER", 96, 1, np.uint32),
+    ("ST_TRI_UPPER", 260, 75, np.uint32), ("ST_TRI_UPPER", 300, 61, np.uint16), ("ST_TET", 32, 1, np.uint16), ("ST_TET", 33, 1, np.uint32),
+    ("ST_TET", 65, 1, np.uint64), ("ST_TET", 23, 33, np.uint32), ("ST_SIMPLEX4", 8, 1, np.uint16), ("ST_SIMPLEX4", 33, 1, np.uint32),
+    ("ST_SIMPLEX4", 11, 7, np.uint16), ("ST_FIXED_COL", 90, 301, np.uint32), ("ST_FIXED_ROW", 70, 301, np.uint16)])
+def test_copies_at_odd_offsets_and_tile_edges(st, kind, d, inner, dtype):
+    lay = st.Layout(getattr(st, kind), d, inner, kl=d // 2 if kind.startswith("ST_FIXED") else 0)
+    nd = st.st_dense_elems(lay)
+    dense = np.random.default_rng(nd).integers(1, np.iinfo(dtype).max, size=nd, dtype=dtype)
+    signed = {2: np.int16, 4: np.int32, 8: np.int64}[dense.itemsize]
+    packed = oracle.pack(dense, lay.kind, d, inner=inner, **okw(lay))
+    got = st.st_pack(torch.from_numpy(dense.view(signed)).cuda(), lay)
+    assert np.array_equal(got.cpu().numpy().view(dtype), packed)
+    for fill in [st.ST_FILL_ZERO] + ([] if kind.startswith("ST_FIXED") else [st.ST_FILL_SYMMETRIC]):
+        want = oracle.unpack(packed, lay.kind, d, inner=inner, fill=fill, **okw(lay)).reshape(-1)
+        assert np.array_equal(st.st_unpack(got, lay, fill=fill).cpu().numpy().view(dtype), want), fill
+
+
 def test_unpack_of_symmetric_tensor_restores_it(st):
     """Property 5: T = T_C + T_R * T_C for a tensor that has the structure."""
     d = 37
