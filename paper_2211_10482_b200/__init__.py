@@ -9,6 +9,8 @@ been built the first call raises.
 from __future__ import annotations
 
 import ctypes
+import functools
+import math
 import os
 from dataclasses import dataclass
 
@@ -144,8 +146,15 @@ def _dev(t: torch.Tensor, name: str) -> int:
     return t.data_ptr()
 
 
-def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+# The launch path of a small call is host-bound (its kernels run a few microseconds), so what a call asks of
+# torch per launch is kept to the bare queries: the current stream's handle costs 3 us through
+# torch.cuda.current_stream() and 0.3 us this way.
+if hasattr(torch._C, "_cuda_getCurrentRawStream"):
+    def _stream() -> int:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+else:
+    def _stream() -> int:
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _check(status: int, where: str) -> None:
@@ -153,12 +162,26 @@ def _check(status: int, where: str) -> None:
         raise StError(status, where)
 
 
+@functools.lru_cache(maxsize=256)
+def _layout_info(layout: Layout):
+    """(pointer to the C descriptor, packed elements, dense elements) of a layout, by its value."""
+    c = layout.c()
+    L = lib()
+    return ctypes.pointer(c), int(L.st_packed_elems(ctypes.byref(c))), int(L.st_dense_elems(ctypes.byref(c)))
+
+
+@functools.lru_cache(maxsize=1024)
+def _ws_bytes(device: int, op: int, a: int, b: int, c: int, e: int, flags: int) -> int:
+    """Workspace of a request on a device (its SM count decides), at least the 256-byte header."""
+    return max(st_workspace_bytes(op, a, b, c, e, flags), 256)
+
+
 def st_packed_elems(layout: Layout) -> int:
-    return int(lib().st_packed_elems(ctypes.byref(layout.c())))
+    return _layout_info(layout)[1]
 
 
 def st_dense_elems(layout: Layout) -> int:
-    return int(lib().st_dense_elems(ctypes.byref(layout.c())))
+    return _layout_info(layout)[2]
 
 
 def st_workspace_bytes(op: int, a: int, b: int, c: int = 0, e: int = 0, flags: int = 0) -> int:
@@ -178,45 +201,48 @@ def set_allocator(fn) -> None:
     _allocator = fn
 
 
-def _alloc(numel: int, dtype, device) -> torch.Tensor:
-    if _allocator is not None:
-        return _allocator(int(numel), dtype, device)
-    return torch.empty(int(numel), dtype=dtype, device=device)
+def _alloc(shape, dtype, device) -> torch.Tensor:
+    """A tensor of `shape` (an element count or a tuple)."""
+    if _allocator is None:
+        return torch.empty(shape, dtype=dtype, device=device)
+    if isinstance(shape, int):
+        return _allocator(shape, dtype, device)
+    return _allocator(math.prod(shape), dtype, device).view(shape)
 
 
-def _workspace(query, device, ws: torch.Tensor | None) -> torch.Tensor:
-    """The caller's workspace, or a fresh one of the size that `query()` reports.  Either way it is
+def _workspace(ws: torch.Tensor | None, device, op: int, a: int, b: int, c: int, e: int, flags: int) -> torch.Tensor:
+    """The caller's workspace, or a fresh one of the size of the request.  Either way it is
     remembered as the device's last workspace, so that st_check_status() can read the status word
     that the call's kernels may have written."""
     if ws is None:
-        ws = _alloc(max(int(query()), 256), torch.uint8, device)
+        ws = _alloc(_ws_bytes(torch.cuda.current_device(), op, a, b, c, e, flags), torch.uint8, device)
     _last_ws[ws.device.index] = ws
     return ws
 
 
 def st_pack(dense: torch.Tensor, layout: Layout, out: torch.Tensor | None = None) -> torch.Tensor:
-    n = st_packed_elems(layout)
+    desc, n, n_dense = _layout_info(layout)
     if n < 0:
         raise StError(ST_ERR_SHAPE, "st_packed_elems")
-    if dense.numel() != st_dense_elems(layout):
-        raise ValueError("dense has %d elements, layout needs %d" % (dense.numel(), st_dense_elems(layout)))
+    if dense.numel() != n_dense:
+        raise ValueError("dense has %d elements, layout needs %d" % (dense.numel(), n_dense))
     if out is None:
         out = _alloc(n, dense.dtype, dense.device)
-    _check(lib().st_pack(ctypes.byref(layout.c()), _dtype(dense), _dev(dense, "dense"), _dev(out, "out"),
+    _check(lib().st_pack(desc, _dtype(dense), _dev(dense, "dense"), _dev(out, "out"),
                          _stream()), "st_pack")
     return out
 
 
 def st_unpack(packed: torch.Tensor, layout: Layout, fill: int = ST_FILL_ZERO,
               out: torch.Tensor | None = None) -> torch.Tensor:
-    n = st_dense_elems(layout)
+    desc, n_packed, n = _layout_info(layout)
     if n < 0:
         raise StError(ST_ERR_SHAPE, "st_dense_elems")
-    if packed.numel() != st_packed_elems(layout):
-        raise ValueError("packed has %d elements, layout needs %d" % (packed.numel(), st_packed_elems(layout)))
+    if packed.numel() != n_packed:
+        raise ValueError("packed has %d elements, layout needs %d" % (packed.numel(), n_packed))
     if out is None:
         out = _alloc(n, packed.dtype, packed.device)
-    _check(lib().st_unpack(ctypes.byref(layout.c()), _dtype(packed), _dev(packed, "packed"), _dev(out, "out"),
+    _check(lib().st_unpack(desc, _dtype(packed), _dev(packed, "packed"), _dev(out, "out"),
                            int(fill), _stream()), "st_unpack")
     return out
 
@@ -230,7 +256,7 @@ def st_sym_moment2(X: torch.Tensor, out: torch.Tensor | None = None, ws: torch.T
     xdt = _DTYPES[X.dtype]
     if out is None:
         out = _alloc(d * (d + 1) // 2, torch.float32, X.device)
-    ws = _workspace(lambda: st_workspace_bytes(ST_OP_SYM_MOMENT2, N, d, xdt, 0, flags), X.device, ws)
+    ws = _workspace(ws, X.device, ST_OP_SYM_MOMENT2, N, d, xdt, 0, flags)
     _check(lib().st_sym_moment2(_dev(X, "X"), xdt, N, d, X.stride(0), _dev(out, "out"), ws.data_ptr(),
                                 ws.numel() * ws.element_size(), flags, _stream()), "st_sym_moment2")
     return out
@@ -244,7 +270,7 @@ def st_sym_moment3(X: torch.Tensor, out: torch.Tensor | None = None, ws: torch.T
         raise TypeError("X must be float32")
     if out is None:
         out = _alloc(d * (d + 1) * (d + 2) // 6, torch.float32, X.device)
-    ws = _workspace(lambda: st_workspace_bytes(ST_OP_SYM_MOMENT3, N, d, 0, 0, flags), X.device, ws)
+    ws = _workspace(ws, X.device, ST_OP_SYM_MOMENT3, N, d, 0, 0, flags)
     _check(lib().st_sym_moment3(_dev(X, "X"), N, d, X.stride(0), _dev(out, "out"), ws.data_ptr(),
                                 ws.numel() * ws.element_size(), flags, _stream()), "st_sym_moment3")
     return out
@@ -258,7 +284,7 @@ def st_sym_moment4(X: torch.Tensor, out: torch.Tensor | None = None, ws: torch.T
         raise TypeError("X must be float32")
     if out is None:
         out = _alloc(d * (d + 1) * (d + 2) * (d + 3) // 24, torch.float32, X.device)
-    ws = _workspace(lambda: st_workspace_bytes(ST_OP_SYM_MOMENT4, N, d, 0, 0, flags), X.device, ws)
+    ws = _workspace(ws, X.device, ST_OP_SYM_MOMENT4, N, d, 0, 0, flags)
     _check(lib().st_sym_moment4(_dev(X, "X"), N, d, X.stride(0), _dev(out, "out"), ws.data_ptr(),
                                 ws.numel() * ws.element_size(), flags, _stream()), "st_sym_moment4")
     return out
@@ -291,8 +317,8 @@ def st_mttkrp_tri(Bp: torch.Tensor, C: torch.Tensor, D: torch.Tensor, out: torch
     if Bp.numel() != want or D.shape[1] != R:
         raise ValueError("shape mismatch")
     if out is None:
-        out = _alloc(I * R, torch.float32, Bp.device).view(I, R)
-    ws = _workspace(lambda: st_workspace_bytes(ST_OP_MTTKRP_TRI, I, K, R, 0, flags), Bp.device, ws)
+        out = _alloc((I, R), torch.float32, Bp.device)
+    ws = _workspace(ws, Bp.device, ST_OP_MTTKRP_TRI, I, K, R, 0, flags)
     _check(lib().st_mttkrp_tri(_dev(Bp, "Bp"), I, K, _dev(C, "C"), _dev(D, "D"), R, _dev(out, "out"),
                                ws.data_ptr(), ws.numel() * ws.element_size(), flags, _stream()),
            "st_mttkrp_tri")
@@ -311,8 +337,8 @@ def st_mttkrp_slice(Bp: torch.Tensor, C: torch.Tensor, D: torch.Tensor, I: int, 
     if Bp.numel() != rows * K or D.shape[1] != R:
         raise ValueError("shape mismatch")
     if out is None:
-        out = _alloc(I * R, torch.float32, Bp.device).view(I, R)
-    ws = _workspace(lambda: st_workspace_bytes(ST_OP_MTTKRP_SLICE, I, J, K, R, flags), Bp.device, ws)
+        out = _alloc((I, R), torch.float32, Bp.device)
+    ws = _workspace(ws, Bp.device, ST_OP_MTTKRP_SLICE, I, J, K, R, flags)
     _check(lib().st_mttkrp_slice(_dev(Bp, "Bp"), I, J, K, fixed_i, fixed_j, _dev(C, "C"), _dev(D, "D"), R,
                                  _dev(out, "out"), ws.data_ptr(), ws.numel() * ws.element_size(), flags, _stream()),
            "st_mttkrp_slice")
@@ -331,8 +357,8 @@ def st_ttm_blockdiag(Bp: torch.Tensor, U: torch.Tensor, nblocks: int, bs: int,
     if Bp.numel() != rows * K:
         raise ValueError("shape mismatch")
     if out is None:
-        out = _alloc(rows * R, torch.float32, Bp.device).view(rows, R)
-    ws = _workspace(lambda: st_workspace_bytes(ST_OP_TTM_BLOCKDIAG, nblocks, bs, K, R, flags), Bp.device, ws)
+        out = _alloc((rows, R), torch.float32, Bp.device)
+    ws = _workspace(ws, Bp.device, ST_OP_TTM_BLOCKDIAG, nblocks, bs, K, R, flags)
     _check(lib().st_ttm_blockdiag(_dev(Bp, "Bp"), nblocks, bs, K, _dev(U, "U"), R, _dev(out, "out"),
                                   ws.data_ptr(), ws.numel() * ws.element_size(), flags, _stream()),
            "st_ttm_blockdiag")
@@ -345,13 +371,14 @@ def st_ttm_packed(Bp: torch.Tensor, U: torch.Tensor, layout: Layout, out: torch.
     K, R = U.shape
     if Bp.dtype != torch.float32 or U.dtype != torch.float32:
         raise TypeError("inputs must be float32")
-    if layout.inner != K or Bp.numel() != st_packed_elems(layout):
+    desc, n_packed, _ = _layout_info(layout)
+    if layout.inner != K or Bp.numel() != n_packed:
         raise ValueError("shape mismatch")
     rows = Bp.numel() // K
     if out is None:
-        out = _alloc(rows * R, torch.float32, Bp.device).view(rows, R)
-    ws = _workspace(lambda: st_workspace_bytes(ST_OP_TTM_BLOCKDIAG, rows, 1, K, R, flags), Bp.device, ws)
-    _check(lib().st_ttm_packed(ctypes.byref(layout.c()), _dev(Bp, "Bp"), _dev(U, "U"), R, _dev(out, "out"),
+        out = _alloc((rows, R), torch.float32, Bp.device)
+    ws = _workspace(ws, Bp.device, ST_OP_TTM_BLOCKDIAG, rows, 1, K, R, flags)
+    _check(lib().st_ttm_packed(desc, _dev(Bp, "Bp"), _dev(U, "U"), R, _dev(out, "out"),
                                ws.data_ptr(), ws.numel() * ws.element_size(), flags, _stream()), "st_ttm_packed")
     return out
 
@@ -360,11 +387,12 @@ def st_thp(Bp: torch.Tensor, C: torch.Tensor, layout: Layout, out: torch.Tensor 
     """Ap = Bp * (C at the unique positions of `layout`): packed B, dense C, packed result."""
     if Bp.dtype != torch.float32 or C.dtype != torch.float32:
         raise TypeError("inputs must be float32")
-    if Bp.numel() != st_packed_elems(layout) or C.numel() != st_dense_elems(layout):
+    desc, n_packed, n_dense = _layout_info(layout)
+    if Bp.numel() != n_packed or C.numel() != n_dense:
         raise ValueError("shape mismatch")
     if out is None:
-        out = _alloc(Bp.numel(), torch.float32, Bp.device).view(Bp.shape)
-    _check(lib().st_thp(ctypes.byref(layout.c()), _dev(Bp, "Bp"), _dev(C, "C"), _dev(out, "out"), _stream()), "st_thp")
+        out = _alloc(tuple(Bp.shape), torch.float32, Bp.device)
+    _check(lib().st_thp(desc, _dev(Bp, "Bp"), _dev(C, "C"), _dev(out, "out"), _stream()), "st_thp")
     return out
 
 
@@ -374,7 +402,7 @@ def st_packed_axpby(alpha: float, a: torch.Tensor, beta: float, b: torch.Tensor,
     if a.dtype != torch.float32 or b.dtype != torch.float32 or a.numel() != b.numel():
         raise ValueError("two float32 arrays of the same size are needed")
     if out is None:
-        out = _alloc(a.numel(), torch.float32, a.device).view(a.shape)
+        out = _alloc(tuple(a.shape), torch.float32, a.device)
     _check(lib().st_packed_axpby(a.numel(), alpha, _dev(a, "a"), beta, _dev(b, "b"), _dev(out, "out"), _stream()),
            "st_packed_axpby")
     return out
@@ -385,7 +413,7 @@ def st_packed_mul(a: torch.Tensor, b: torch.Tensor, out: torch.Tensor | None = N
     if a.dtype != torch.float32 or b.dtype != torch.float32 or a.numel() != b.numel():
         raise ValueError("two float32 arrays of the same size are needed")
     if out is None:
-        out = _alloc(a.numel(), torch.float32, a.device).view(a.shape)
+        out = _alloc(tuple(a.shape), torch.float32, a.device)
     _check(lib().st_packed_mul(a.numel(), _dev(a, "a"), _dev(b, "b"), _dev(out, "out"), _stream()), "st_packed_mul")
     return out
 
