@@ -5,7 +5,7 @@
 // motion, Section 5.5) the sum is a contraction over the samples,
 //     out[(i,j), k] = sum_n P[n,(i,j)] X[n,k],      P[n,(i,j)] = X[n,i] X[n,j]   (i <= j),
 // that is a GEMM [pairs x samples] x [samples x d] whose left operand exists nowhere in memory.
-// This kernel makes P on the fly.  A loader warp writes slices of 32 (TF32) or 64 (bf16) samples of X^T,
+// This kernel makes P on the fly.  Loader warps fetch slices of 32 (TF32) or 64 (bf16) samples and write X^T,
 // rounded, into shared memory in the K-major 128-byte-swizzled form the tensor core reads (lane =
 // sample).  Producer warps read their lane's x_i and x_j back from that slice, multiply the
 // pairs of one tile (8 values of i x 16 values of j) and store the products, rounded to TF32, in
@@ -26,8 +26,6 @@
 
 namespace st {
 
-st_status sum_slices_launch(const float *partials, float *out, int64_t elems, int slices, cudaStream_t stream);
-
 namespace m3tc {
 constexpr int DP = 64;                       // largest d
 constexpr int TI = 8, TJ = 16;               // a tile holds the pairs (8 IB + a, 16 JB + b)
@@ -37,24 +35,27 @@ constexpr int A_STAGE_BYTES = BM * ROW_BYTES; // 16 KiB
 constexpr int B_STAGE_BYTES = DP * ROW_BYTES; // 8 KiB
 constexpr int NA_MAX = 10;                   // A stages in flight (TF32: 10, bf16: 8; even: see the issuers)
 constexpr int NB = 4;                        // X^T slices in flight
-constexpr int X32_STAGE_BYTES = DP * 64 * 4; // bf16 path: fp32 copy of a slice of X^T for the producers (16 KiB)
+constexpr int X_PITCH = DP + 1;              // floats per row of a slice of X as it arrives: lanes that read one column of
+                                             // consecutive samples touch every bank once
 constexpr int PRODUCERS = 8;                 // producer warps (also the epilogue warps)
 constexpr int MMA_WARPS = 2;                 // issuer w takes the stages q = w (mod 2): while one polls, the other's MMAs run
 constexpr int MMA_WARP = PRODUCERS, LOAD_WARP = PRODUCERS + MMA_WARPS;
-constexpr int LOAD_WARPS = 1;                // one loader: slices are filled in order
+constexpr int LOAD_WARPS = 4;                // fetch slices of X and turn them into the right operand
+constexpr int FETCH_AHEAD = 2;               // slices in flight
 constexpr int THREADS = 32 * (PRODUCERS + MMA_WARPS + LOAD_WARPS);
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int MAX_GROUP_TILES = 12;
-constexpr int EPI_PITCH = DP + 1;             // floats per row of the epilogue's transposing buffer
+constexpr int x_stage_bytes(bool bf16) { return (bf16 ? 64 : 32) * X_PITCH * 4; }
 constexpr size_t smem_bytes(bool bf16)
 {
-    return 1024 + (size_t)(bf16 ? 8 : 10) * A_STAGE_BYTES + (size_t)NB * B_STAGE_BYTES +
-           (bf16 ? (size_t)NB * X32_STAGE_BYTES : 0) + 512;
+    return 1024 + (size_t)(bf16 ? 8 : 10) * A_STAGE_BYTES + (size_t)NB * B_STAGE_BYTES + (size_t)NB * x_stage_bytes(bf16) + 512;
 }
+static_assert(smem_bytes(true) <= 227 * 1024 && smem_bytes(false) <= 227 * 1024, "shared memory of a block");
 
 struct Tile {
     unsigned char ib, jb;
     unsigned short col;                      // first tensor-memory column of the tile's accumulator
+    int part;                                // first of its partial sums in a slice
 };
 
 struct Args {
@@ -62,7 +63,7 @@ struct Args {
     float *partials;
     unsigned *status;
     int64_t N, ldx, rows_per_slice;
-    int d, dcols, out_elems, vec;            // dcols = d rounded up to a multiple of 16
+    int d, dcols, part_elems;                // part_elems: partial sums per slice; dcols = d rounded up to a multiple of 16
     int ntiles[2];
     Tile tiles[2][MAX_GROUP_TILES];
 };
@@ -70,6 +71,13 @@ struct Args {
 // byte offset of the 4-byte word `lane` (one TF32 sample, or two bf16 samples) inside a 128-byte row whose
 // index has (row & 7) == m
 __device__ __forceinline__ uint32_t swz(int lane, int m) { return (uint32_t)((((lane >> 2) ^ m) << 4) + ((lane & 3) << 2)); }
+
+__device__ __forceinline__ uint64_t m3tc_pack2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
 
 template <bool BF16>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -82,8 +90,9 @@ moment3_tc_kernel(const __grid_constant__ Args a)
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *a_stage0 = smem;
     unsigned char *b_stage0 = smem + (size_t)NA * A_STAGE_BYTES;
-    unsigned char *x32_stage0 = b_stage0 + (size_t)NB * B_STAGE_BYTES;   // bf16 path only
-    uint64_t *bars = (uint64_t *)(x32_stage0 + (BF16 ? (size_t)NB * X32_STAGE_BYTES : 0));
+    constexpr int X_STAGE_FLOATS = KS * X_PITCH;
+    float *x_stage0 = (float *)(b_stage0 + (size_t)NB * B_STAGE_BYTES);   // slices of X as they are in memory, [sample][X_PITCH]
+    uint64_t *bars = (uint64_t *)(x_stage0 + (size_t)NB * X_STAGE_FLOATS);
     uint64_t *a_full = bars, *a_empty = bars + NA_MAX, *b_full = bars + 2 * NA_MAX, *b_empty = bars + 2 * NA_MAX + NB,
              *acc_full = bars + 2 * NA_MAX + 2 * NB;
     uint64_t *iss_sync = acc_full + 1;
@@ -101,7 +110,7 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             mbar_init(&a_empty[s], 1);
         }
         for (int s = 0; s < NB; ++s) {
-            mbar_init(&b_full[s], 1);
+            mbar_init(&b_full[s], LOAD_WARPS);
             mbar_init(&b_empty[s], MMA_WARPS);
         }
         mbar_init(acc_full, MMA_WARPS);
@@ -139,38 +148,29 @@ moment3_tc_kernel(const __grid_constant__ Args a)
         // the A ring) and nprod <= NB * tg (stages covered by the slices of the X^T ring).
         const int nprod = min(min(PRODUCERS, NA), NB * tg);
         bool ok = true;
+        int slice = warp / tg, ti = warp - slice * tg, as = warp, use = 0;     // of stage q
+        const int dslice = nprod / tg, dti = nprod - dslice * tg;
         for (int64_t q = warp; q < nstages && ok && warp < nprod; q += nprod) {
-            const int slice = (int)(q / tg), ti = (int)(q - (int64_t)slice * tg);
             const int bs = slice % NB;
             if (!mbar_wait(&b_full[bs], (uint32_t)((slice / NB) & 1), abort_flag, a.status, 11)) break;
             // this lane's sample: x_i for the tile's 8 values of i, x_j for its 16 values of j
             const unsigned char *bst = b_stage0 + (size_t)bs * B_STAGE_BYTES;
             const Tile t = tiles[ti];
-            // TF32: the rounded values of the MMA's own slice; bf16: the fp32 copy, two samples per lane,
-            // so that every product is rounded once
-            float xi[TI][BF16 ? 2 : 1], xj[TJ][BF16 ? 2 : 1];
+            // TF32: the rounded values of the MMA's own slice; bf16: the slice of X itself, samples `lane` and
+            // `lane` + 32, so that every product is rounded once
+            uint64_t xi[TI], xj[TJ];                       // TF32: the low word only
             if (BF16) {
-                const unsigned char *xst = x32_stage0 + (size_t)bs * X32_STAGE_BYTES + 8 * lane;
+                const float *xst = x_stage0 + (size_t)bs * X_STAGE_FLOATS + lane * X_PITCH;
 #pragma unroll
-                for (int e = 0; e < TI; ++e) {
-                    const float2 v = *reinterpret_cast<const float2 *>(xst + (TI * t.ib + e) * 256);
-                    xi[e][0] = v.x; xi[e][BF16 ? 1 : 0] = v.y;
-                }
+                for (int e = 0; e < TI; ++e) xi[e] = m3tc_pack2(xst[TI * t.ib + e], xst[(BF16 ? 32 : 0) * X_PITCH + TI * t.ib + e]);
 #pragma unroll
-                for (int e = 0; e < TJ; ++e) {
-                    const float2 v = *reinterpret_cast<const float2 *>(xst + (TJ * t.jb + e) * 256);
-                    xj[e][0] = v.x; xj[e][BF16 ? 1 : 0] = v.y;
-                }
+                for (int e = 0; e < TJ; ++e) xj[e] = m3tc_pack2(xst[TJ * t.jb + e], xst[(BF16 ? 32 : 0) * X_PITCH + TJ * t.jb + e]);
             } else {
 #pragma unroll
-                for (int e = 0; e < TI; ++e)
-                    xi[e][0] = *reinterpret_cast<const float *>(bst + (TI * t.ib + e) * 128 + sw[e & 7]);
+                for (int e = 0; e < TI; ++e) xi[e] = *reinterpret_cast<const uint32_t *>(bst + (TI * t.ib + e) * 128 + sw[e & 7]);
 #pragma unroll
-                for (int e = 0; e < TJ; ++e)
-                    xj[e][0] = *reinterpret_cast<const float *>(bst + (TJ * t.jb + e) * 128 + sw[e & 7]);
+                for (int e = 0; e < TJ; ++e) xj[e] = *reinterpret_cast<const uint32_t *>(bst + (TJ * t.jb + e) * 128 + sw[e & 7]);
             }
-            const int as = (int)(q % NA);
-            const int64_t use = q / NA;
             if (use > 0 && !mbar_wait(&a_empty[as], (uint32_t)((use - 1) & 1), abort_flag, a.status, 12)) {
                 ok = false;
                 break;
@@ -184,76 +184,54 @@ moment3_tc_kernel(const __grid_constant__ Args a)
                     uint32_t v;
                     if (BF16) {
                         // two samples per word, each product rounded once to bf16 (first sample in the low half)
-                        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(v) : "f"(xi[e][BF16 ? 1 : 0] * xj[f][BF16 ? 1 : 0]), "f"(xi[e][0] * xj[f][0]));
+                        uint64_t p;
+                        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(p) : "l"(xi[e]), "l"(xj[f]));
+                        asm("{\n\t.reg .f32 a, b;\n\tmov.b64 {a, b}, %1;\n\tcvt.rn.bf16x2.f32 %0, b, a;\n\t}" : "=r"(v) : "l"(p));
                     } else {
                         // round to nearest TF32 (ties away from zero): the tensor core ignores the low 13 bits
-                        v = __float_as_uint(xi[e][0] * xj[f][0]) + 0x1000u;
+                        v = __float_as_uint(__uint_as_float((uint32_t)xi[e]) * __uint_as_float((uint32_t)xj[f])) + 0x1000u;
                     }
                     *reinterpret_cast<uint32_t *>(ast + (e * TJ + f) * 128 + sw[f & 7]) = v;
                 }
             fence_proxy_async();      // generic-proxy stores must be visible to the tensor core
             __syncwarp();
             if (lane == 0) mbar_arrive(&a_full[as]);
+            slice += dslice;
+            ti += dti;
+            if (ti >= tg) { ti -= tg; ++slice; }
+            as += nprod;
+            if (as >= NA) { as -= NA; ++use; }
         }
 
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the slice sums may be launched; they wait for this grid to end
         // ---- epilogue: tensor memory -> this slice's partial sums ---------------------------------
         if (nstages > 0 && mbar_wait(acc_full, 0u, abort_flag, a.status, 13)) {
             tc_fence_after();
-            float *__restrict__ mine = a.partials + (size_t)blockIdx.y * a.out_elems;
-            // All MMAs are complete, so the A ring is free: every warp takes EPI_PITCH x 32 floats of it
-            // to turn "one thread = one pair, registers = k" into rows of consecutive k.  In the packed
-            // order the rows (i, j, k >= j) of one i and consecutive j follow each other, so the 16 rows of
-            // one i of a tile form one contiguous run in memory.
-            float *tr = reinterpret_cast<float *>(a_stage0) + (size_t)warp * (32 * EPI_PITCH);
+            // partial sums of a tile: [column][row], so that a warp stores 32 consecutive rows (pairs) of one column k
+            // straight from tensor memory; rows with i > j are not outputs and are skipped
+            float *__restrict__ mine = a.partials + (size_t)blockIdx.y * a.part_elems;
             const int q4 = warp & 3;                                // lanes 32*q4 .. 32*q4+31 of tensor memory
             for (int ti = warp >> 2; ti < tg; ti += PRODUCERS / 4) {
                 const Tile t = tiles[ti];
-                const int kstart = TJ * t.jb, ncols = a.dcols - kstart;
+                const int ncols = a.dcols - TJ * t.jb;
                 uint32_t v[DP];
 #pragma unroll
                 for (int c0 = 0; c0 < DP; c0 += 16)                 // all loads of the tile in flight, one wait
                     if (c0 < ncols)
                         tmem_ld_32x16(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(t.col + c0), v + c0);
                 tmem_ld_wait();
+                const int r = q4 * 32 + lane;
+                const int i = TI * t.ib + r / TJ, j = TJ * t.jb + r % TJ;
+                float *dst = mine + t.part + r;
+                if (i <= j && j < a.d) {
 #pragma unroll
-                for (int c0 = 0; c0 < DP; c0 += 16)
-                    if (c0 < ncols) {
+                    for (int c0 = 0; c0 < DP; c0 += 16)
+                        if (c0 < ncols) {
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) tr[lane * EPI_PITCH + c0 + e] = __uint_as_float(v[c0 + e]);
-                    }
-                __syncwarp();
-                // lane rr describes row rr: first output element and (shift, length) of its run of k
-                int my_base = 0, my_run = 0;
-                {
-                    const int r = q4 * 32 + lane;
-                    const int i = TI * t.ib + r / TJ, j = TJ * t.jb + r % TJ;
-                    if (i <= j && j < a.d) {
-                        // first element of row (i, j, k = j ..) of the packed tetrahedron, in 32-bit arithmetic
-                        const int m = a.d - i, jj = j - i;
-                        my_base = a.out_elems - m * (m + 1) * (m + 2) / 6 + jj * (2 * m - jj + 1) / 2;
-                        my_run = ((j - kstart) << 8) | (a.d - j);
-                    }
+                            for (int e = 0; e < 16; ++e)
+                                if (ST_BOUNDS_OK(t.part + r + (c0 + e) * BM, a.part_elems, 4)) dst[(c0 + e) * BM] = __uint_as_float(v[c0 + e]);
+                        }
                 }
-                for (int rr0 = 0; rr0 < 32; rr0 += 8) {             // eight rows: all loads, then all stores
-                    float v0[8], v1[8];
-                    int base[8], len[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        base[u] = __shfl_sync(0xffffffffu, my_base, rr0 + u);
-                        const int run = __shfl_sync(0xffffffffu, my_run, rr0 + u);
-                        len[u] = run & 255;
-                        const float *src = tr + (rr0 + u) * EPI_PITCH + (run >> 8);
-                        v0[u] = lane < len[u] ? src[lane] : 0.f;
-                        v1[u] = lane + 32 < len[u] ? src[lane + 32] : 0.f;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        if (lane < len[u] && ST_BOUNDS_OK(base[u] + lane, a.out_elems, 4)) mine[base[u] + lane] = v0[u];
-                        if (lane + 32 < len[u] && ST_BOUNDS_OK(base[u] + lane + 32, a.out_elems, 4)) mine[base[u] + lane + 32] = v1[u];
-                    }
-                }
-                __syncwarp();
             }
         }
     } else if (warp < LOAD_WARP) {
@@ -265,17 +243,21 @@ moment3_tc_kernel(const __grid_constant__ Args a)
         const int iw = warp - MMA_WARP;
         if (elect_one()) {
             bool ok = true;
+            int q_slot = 0;                                         // ring slot and phase of stage q = slice * tg + ti
+            uint32_t q_parity = 0;
             for (int slice = 0; slice < nslices && ok; ++slice) {
                 const int bs = slice % NB;
                 if (!mbar_wait(&b_full[bs], (uint32_t)((slice / NB) & 1), abort_flag, a.status, 14)) break;
                 const uint32_t sb = smem_u32(b_stage0 + (size_t)bs * B_STAGE_BYTES);
                 for (int ti = 0; ti < tg; ++ti) {
-                    const int64_t q = (int64_t)slice * tg + ti;
-                    if ((int)(q & 1) != iw) continue;
+                    const int as = q_slot;
+                    const uint32_t a_parity = q_parity;
+                    const bool mine = (q_slot & 1) == iw;          // NA is even
+                    if (++q_slot == NA) { q_slot = 0; q_parity ^= 1u; }
+                    if (!mine) continue;
                     const Tile t = tiles[ti];
                     const int kstart = TJ * t.jb, ncols = a.dcols - kstart;
-                    const int as = (int)(q % NA);
-                    if (!mbar_wait(&a_full[as], (uint32_t)((q / NA) & 1), abort_flag, a.status, 15)) {
+                    if (!mbar_wait(&a_full[as], a_parity, abort_flag, a.status, 15)) {
                         ok = false;
                         break;
                     }
@@ -302,66 +284,83 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             }
         }
     } else {
-        // ---- loader: slices of X^T (row = column c of X), rounded to TF32 or bf16.  A lane owns one
-        // 4-byte word of every row: sample `lane` (TF32) or samples 2*lane, 2*lane+1 (bf16).
-        constexpr int SPL = BF16 ? 2 : 1;                            // samples per lane
-        constexpr int CH = 32;                                       // columns per pass
-        constexpr int PF_AHEAD = 4;                                  // slices of L2 prefetch distance
+        // ---- loaders: slices of X by asynchronous copies, consecutive lanes along a row (one warp that read a
+        // sample per lane, two round trips to memory per slice, was what the whole kernel waited for), then X^T
+        // (row = column c of X) rounded to TF32 or bf16.  A lane owns one 4-byte word of every row of X^T: sample
+        // `lane` (TF32) or samples `lane` and `lane` + 32 (bf16; the order of the samples is the one of the products).
+        const int lt = (int)threadIdx.x - 32 * LOAD_WARP, lw = warp - LOAD_WARP;
+        // the block's rows are asked for in L2 far ahead: PREFETCH slices now, one more with every slice fetched
+        constexpr int PREFETCH = 16;
+        auto prefetch = [&](int64_t first, int64_t last) {                // rows
+            if (last > n_end) last = n_end;
+            if (first >= last) return;
+            const char *lo = reinterpret_cast<const char *>(a.X + first * a.ldx);
+            const int64_t bytes = ((last - 1 - first) * a.ldx + a.d) * 4;
+            for (int64_t o = 128 * (int64_t)lt; o < bytes; o += 128 * 32 * LOAD_WARPS) asm volatile("prefetch.global.L2 [%0];" ::"l"(lo + o));
+        };
+        prefetch(n_begin, n_begin + PREFETCH * KS);
+        // columns d .. dcols-1 are never written again
+        for (int e = lt; e < NB * X_STAGE_FLOATS; e += 32 * LOAD_WARPS) x_stage0[e] = 0.f;
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * LOAD_WARPS) : "memory");
+        // a warp copies 32 / width rows at a time, width lanes along each (and a second time for columns 32 and up)
+        const int width = a.d <= 8 ? 8 : a.d <= 16 ? 16 : 32;
+        const int fr0 = (lw * 32 + lane) / width, fc = lane & (width - 1), fstep = 32 * LOAD_WARPS / width;
+        auto fetch = [&](int slice) {
+            const int64_t n0 = n_begin + (int64_t)slice * KS;
+            const int rows = n_end - n0 < KS ? (int)(n_end - n0) : KS;
+            uint32_t dst = smem_u32(x_stage0 + (size_t)(slice % NB) * X_STAGE_FLOATS + fr0 * X_PITCH + fc);
+            const float *src = a.X + (n0 + fr0) * a.ldx + fc;
+            const int64_t src_step = fstep * a.ldx;
+            const bool c0 = fc < a.d, c1 = fc + 32 < a.d;
+#pragma unroll 4
+            for (int r = fr0; r < KS; r += fstep, dst += (uint32_t)(fstep * X_PITCH * 4), src += src_step) {
+                const bool in = r < rows;                                  // samples past the end: zeros
+                const int sz = in ? 4 : 0;
+                if (c0) asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(in ? src : a.X), "r"(sz));
+                if (c1) asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 128u), "l"(in ? src + 32 : a.X), "r"(sz));
+            }
+            prefetch(n0 + PREFETCH * KS, n0 + (PREFETCH + 1) * KS);
+        };
+        for (int s = 0; s < FETCH_AHEAD; ++s) {
+            if (s < nslices) fetch(s);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
         for (int slice = 0; slice < nslices; ++slice) {
-            const int bs = slice % NB, use = slice / NB;
+            const int bs = slice % NB;
+            // a slice's buffers are free once the MMAs of the slice NB before it are complete
+            uint32_t failed = 0;
+            const int next = slice + FETCH_AHEAD, use = next / NB;
+            if (next < nslices) {
+                if (use > 0 && !mbar_wait(&b_empty[next % NB], (uint32_t)((use - 1) & 1), abort_flag, a.status, 16)) failed = 1;
+                else fetch(next);
+            }
+            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group %0;" ::"n"(FETCH_AHEAD) : "memory");
+            // every loader's copies of the slice have landed; all loaders leave together if one gave up
+            asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %0, 0;\n\tbar.red.or.pred q, 1, %1, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                         : "+r"(failed) : "n"(32 * LOAD_WARPS) : "memory");
+            if (failed) break;
             unsigned char *bst = b_stage0 + (size_t)bs * B_STAGE_BYTES;
-            bool waited = false;
-            // pull the rows of later slices into L2 while this one is worked on
-            for (int ahead = (slice == 0 ? 1 : PF_AHEAD); ahead <= PF_AHEAD; ++ahead)
+            const float *xst = x_stage0 + (size_t)bs * X_STAGE_FLOATS + lane * X_PITCH;
+            for (int c8 = 8 * lw; c8 < a.dcols; c8 += 8 * LOAD_WARPS) {
+                float x[8], y[8];
 #pragma unroll
-                for (int u = 0; u < SPL; ++u) {
-                    const int64_t n = n_begin + (int64_t)(slice + ahead) * KS + SPL * lane + u;
-                    if (n < n_end) {
-                        const char *pf = reinterpret_cast<const char *>(a.X + n * a.ldx);
-                        for (int o = 0; o < a.d * 4; o += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + o));
-                    }
-                }
-            for (int c0 = 0; c0 < DP; c0 += CH) {
-                float x[SPL][CH];
-#pragma unroll
-                for (int u = 0; u < SPL; ++u) {
-                    const int64_t n = n_begin + (int64_t)slice * KS + SPL * lane + u;
-                    const bool row_ok = n < n_end;
-                    if (a.vec) {
-                        const float4 *src = reinterpret_cast<const float4 *>(a.X + (row_ok ? n : n_begin) * a.ldx + c0);
-#pragma unroll
-                        for (int c = 0; c < CH / 4; ++c) {
-                            const float4 v = (row_ok && c0 + 4 * c < a.d) ? __ldg(src + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-                            x[u][4 * c] = v.x; x[u][4 * c + 1] = v.y; x[u][4 * c + 2] = v.z; x[u][4 * c + 3] = v.w;
-                        }
-                    } else {
-                        const float *src = a.X + (row_ok ? n : n_begin) * a.ldx + c0;
-#pragma unroll
-                        for (int c = 0; c < CH; ++c) x[u][c] = (row_ok && c0 + c < a.d) ? __ldg(src + c) : 0.f;
-                    }
-                }
-                if (!waited) {
-                    if (use > 0 && !mbar_wait(&b_empty[bs], (uint32_t)((use - 1) & 1), abort_flag, a.status, 16)) break;
-                    waited = true;
+                for (int c = 0; c < 8; ++c) {
+                    x[c] = xst[c8 + c];
+                    y[c] = BF16 ? xst[(BF16 ? 32 * X_PITCH : 0) + c8 + c] : 0.f;
                 }
 #pragma unroll
-                for (int c = 0; c < CH; ++c) {
+                for (int c = 0; c < 8; ++c) {
                     uint32_t t;
-                    if (BF16) {
-                        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(t) : "f"(x[SPL - 1][c]), "f"(x[0][c]));
-                        *reinterpret_cast<float2 *>(x32_stage0 + (size_t)bs * X32_STAGE_BYTES + (c0 + c) * 256 + 8 * lane) =
-                            make_float2(x[0][c], x[SPL - 1][c]);
-                    } else {
-                        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(t) : "f"(x[0][c]));
-                    }
-                    *reinterpret_cast<uint32_t *>(bst + (c0 + c) * 128 + sw[c & 7]) = t;
+                    if (BF16) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(t) : "f"(y[c]), "f"(x[c]));
+                    else asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(t) : "f"(x[c]));
+                    *reinterpret_cast<uint32_t *>(bst + (c8 + c) * 128 + sw[c]) = t;
                 }
             }
-            if (!waited) break;
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(&b_full[bs]);
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
@@ -371,11 +370,55 @@ moment3_tc_kernel(const __grid_constant__ Args a)
     }
 }
 
+struct SumArgs {
+    const float *partials;
+    float *out;
+    int slices, part_elems, d, ntiles;
+    Tile tiles[2 * MAX_GROUP_TILES];
+};
+
+// out[q(i,j,k)] = sum over the slices of the partial sum of row (i, j), column k of a tile: a block owns 32 rows of one
+// column, warp w adds the slices w, w + 8, ... with its loads in flight, then the eight sums are added in order.
+constexpr int SUM_WARPS = 8;
+__global__ void __launch_bounds__(32 * SUM_WARPS)
+moment3_tc_sum_kernel(const __grid_constant__ SumArgs a)
+{
+    __shared__ float part[SUM_WARPS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;
+    int ti = 0;
+    while (ti + 1 < a.ntiles && a.tiles[ti + 1].part <= e) ++ti;
+    const Tile t = a.tiles[ti];
+    const int r = (e - t.part) % BM, k = TJ * t.jb + (e - t.part) / BM;
+    const int i = TI * t.ib + r / TJ, j = TJ * t.jb + r % TJ;
+    const bool use = i <= j && j <= k && k < a.d;
+    asm volatile("griddepcontrol.wait;" ::: "memory");     // launched as a programmatic dependent of the main kernel
+    float s = 0.f;
+    if (use) {
+        constexpr int BATCH = 10;
+        for (int k0 = warp; k0 < a.slices; k0 += BATCH * SUM_WARPS) {
+            float v[BATCH];
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) v[u] = k0 + u * SUM_WARPS < a.slices ? __ldcg(a.partials + (size_t)(k0 + u * SUM_WARPS) * a.part_elems + e) : 0.f;
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) s += v[u];
+        }
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || !use) return;
+#pragma unroll
+    for (int w = 1; w < SUM_WARPS; ++w) s += part[w][lane];
+    const int64_t at = tet_encode(a.d, i, j, k);
+    if (ST_BOUNDS_OK(at, tet_rows(a.d), 4)) a.out[at] = s;
+}
+
 struct Plan {
     int groups, slices, dcols;
     int ntiles[2];
     Tile tiles[2][MAX_GROUP_TILES];
-    int64_t rows_per_slice, out_elems;
+    int64_t rows_per_slice;
+    int part_elems;
     bool ok;
 };
 
@@ -385,7 +428,6 @@ static Plan plan(int64_t N, int64_t d, bool bf16)
     Plan p{};
     p.ok = false;
     if (N <= 0 || d < 1 || d > DP) return p;
-    p.out_elems = tet_rows(d);
     p.dcols = (int)((d + 15) / 16 * 16);
     // tiles in the order (JB, IB); a tile exists when it holds some i <= j < d
     Tile all[2 * MAX_GROUP_TILES];
@@ -396,6 +438,8 @@ static Plan plan(int64_t N, int64_t d, bool bf16)
             all[n].ib = (unsigned char)ib;
             all[n].jb = (unsigned char)jb;
             cols[n] = p.dcols - jb * TJ;
+            all[n].part = p.part_elems;
+            p.part_elems += cols[n] * BM;
             total_cols += cols[n];
             ++n;
         }
@@ -430,7 +474,7 @@ size_t moment3_tc_workspace(int64_t N, int64_t d, bool bf16)
 {
     const m3tc::Plan p = m3tc::plan(N, d, bf16);
     if (!p.ok) return 0;
-    return kWsHeaderBytes + (size_t)p.slices * p.out_elems * sizeof(float);
+    return kWsHeaderBytes + (size_t)p.slices * p.part_elems * sizeof(float);
 }
 
 st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
@@ -439,7 +483,7 @@ st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *o
     using namespace m3tc;
     const Plan p = plan(N, d, bf16);
     if (!p.ok) return ST_ERR_UNSUPPORTED;
-    const size_t need = kWsHeaderBytes + (size_t)p.slices * p.out_elems * sizeof(float);
+    const size_t need = kWsHeaderBytes + (size_t)p.slices * p.part_elems * sizeof(float);
     if (!ws || ws_bytes < need) return ST_ERR_WORKSPACE;
     if (!aligned256(ws)) return ST_ERR_ALIGN;
     const DeviceInfo di = device_info();
@@ -450,8 +494,7 @@ st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *o
     a.partials = (float *)((unsigned char *)ws + kWsHeaderBytes);
     a.status = (unsigned *)ws;
     a.N = N; a.ldx = ldx; a.rows_per_slice = p.rows_per_slice;
-    a.d = (int)d; a.dcols = p.dcols; a.out_elems = (int)p.out_elems;
-    a.vec = (ldx % 4 == 0 && d % 4 == 0) ? 1 : 0;
+    a.d = (int)d; a.dcols = p.dcols; a.part_elems = p.part_elems;
     for (int g = 0; g < 2; ++g) {
         a.ntiles[g] = p.ntiles[g];
         for (int t = 0; t < MAX_GROUP_TILES; ++t) a.tiles[g][t] = p.tiles[g][t];
@@ -464,7 +507,29 @@ st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *o
         moment3_tc_kernel<false><<<dim3(p.groups, p.slices), THREADS, smem_bytes(false), stream>>>(a);
     }
     if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
-    return sum_slices_launch(a.partials, out, p.out_elems, p.slices, stream);
+    SumArgs m;
+    m.partials = a.partials;
+    m.out = out;
+    m.slices = p.slices;
+    m.part_elems = p.part_elems;
+    m.d = (int)d;
+    m.ntiles = p.ntiles[0] + p.ntiles[1];
+    for (int t = 0; t < m.ntiles; ++t) m.tiles[t] = t < p.ntiles[0] ? p.tiles[0][t] : p.tiles[1][t - p.ntiles[0]];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.part_elems / 32));
+    cfg.blockDim = dim3(32 * SUM_WARPS);
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, moment3_tc_sum_kernel, m) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ST_ERR_CUDA;
+    }
+    return ST_OK;
 }
 
 }  // namespace st
