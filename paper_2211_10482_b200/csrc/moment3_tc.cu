@@ -15,14 +15,14 @@
 // Accumulators of all tiles of a block stay in tensor memory for the block's whole sample
 // range; at d = 64 they need 640 columns, so two blocks ("groups") share one sample range.
 //
-// What bounds it: an MMA of M = 128 takes about 49 ns whatever N <= 128 is, and N <= d <= 64 here, so the
-// time goes with the number of MMAs (4 per tile and slice) and with what the issuing threads do between them
-// (a barrier poll behind tcgen05.mma instructions of the same thread returns only as they drain: two issuer
-// warps take alternate stages), not with the tensor arithmetic.  bf16 halves the number of MMAs
-// (64 samples per slice instead of 32).  Products and x_k rounded to TF32 / bf16, fp32 accumulation: 5e-3
-// tolerance (bf16: for N >= 1000).
+// What bounds it: shared memory.  Per tile and slice the producers store 16 KB of products and the tensor core reads
+// them back with the columns of X^T (an MMA of M = 128, N <= 64 takes 39 to 48 cycles, bound by its operand reads); the
+// stages of eight producer warps come every 320 cycles.  Two issuer warps take alternate stages: polls and commits
+// between the MMAs cost one alone about 100 cycles per stage.  bf16 halves the number of stages (64 samples per slice
+// instead of 32).  Products and x_k rounded to TF32 / bf16, fp32 accumulation: 5e-3 tolerance (bf16: for N >= 1000).
 #include "tc_common.cuh"
 #include "st_index.cuh"
+#include <type_traits>
 
 namespace st {
 
@@ -32,25 +32,33 @@ constexpr int TI = 8, TJ = 16;               // a tile holds the pairs (8 IB + a
 constexpr int BM = TI * TJ;                  // 128 pairs = rows of the MMA
 constexpr int ROW_BYTES = 128;               // one swizzled row: 32 TF32 or 64 bf16 samples
 constexpr int A_STAGE_BYTES = BM * ROW_BYTES; // 16 KiB
-constexpr int B_STAGE_BYTES = DP * ROW_BYTES; // 8 KiB
 constexpr int NA_MAX = 10;                   // A stages in flight (TF32: 10, bf16: 8; even: see the issuers)
-constexpr int NB = 4;                        // X^T slices in flight
-constexpr int X_PITCH = DP + 1;              // floats per row of a slice of X as it arrives: lanes that read one column of
-                                             // consecutive samples touch every bank once
+constexpr int NB_MAX = 16;                   // slices in flight: as many as fit beside the A stages (4 at d = 64), see ring()
 constexpr int PRODUCERS = 8;                 // producer warps (also the epilogue warps)
 constexpr int MMA_WARPS = 2;                 // issuer w takes the stages q = w (mod 2): while one polls, the other's MMAs run
 constexpr int MMA_WARP = PRODUCERS, LOAD_WARP = PRODUCERS + MMA_WARPS;
 constexpr int LOAD_WARPS = 4;                // fetch slices of X and turn them into the right operand
-constexpr int FETCH_AHEAD = 2;               // slices in flight
 constexpr int THREADS = 32 * (PRODUCERS + MMA_WARPS + LOAD_WARPS);
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int MAX_GROUP_TILES = 12;
-constexpr int x_stage_bytes(bool bf16) { return (bf16 ? 64 : 32) * X_PITCH * 4; }
-constexpr size_t smem_bytes(bool bf16)
+// A slice in flight: dcols rows of X^T as the right operand, and the samples as they are in memory, rows of dcols + 1
+// floats (an odd pitch: lanes that read one column of consecutive samples touch every bank once).
+constexpr size_t FIXED_SMEM = 1024 + 1024;    // alignment of the first stage; barriers
+constexpr size_t b_stage_bytes(int dcols) { return (size_t)dcols * ROW_BYTES; }
+constexpr size_t x_stage_bytes(int dcols, bool bf16) { return (size_t)(bf16 ? 64 : 32) * (dcols + 1) * 4; }
+constexpr size_t a_ring_bytes(bool bf16) { return (size_t)(bf16 ? 8 : 10) * A_STAGE_BYTES; }
+constexpr int ring(int dcols, bool bf16)
 {
-    return 1024 + (size_t)(bf16 ? 8 : 10) * A_STAGE_BYTES + (size_t)NB * B_STAGE_BYTES + (size_t)NB * x_stage_bytes(bf16) + 512;
+    const size_t n = (227 * 1024 - FIXED_SMEM - a_ring_bytes(bf16)) / (b_stage_bytes(dcols) + x_stage_bytes(dcols, bf16));
+    return n > NB_MAX ? NB_MAX : (int)n;
 }
-static_assert(smem_bytes(true) <= 227 * 1024 && smem_bytes(false) <= 227 * 1024, "shared memory of a block");
+static_assert(ring(DP, true) >= 4 && ring(DP, false) >= 4, "four slices in flight at least");
+constexpr size_t smem_bytes(int dcols, bool bf16)
+{
+    return FIXED_SMEM + a_ring_bytes(bf16) + ring(dcols, bf16) * (b_stage_bytes(dcols) + x_stage_bytes(dcols, bf16));
+}
+// slices whose copies are under way while one is turned into the right operand
+__host__ __device__ constexpr int fetch_ahead(int nb) { return nb >= 12 ? 8 : nb >= 8 ? 5 : 2; }
 
 struct Tile {
     unsigned char ib, jb;
@@ -63,6 +71,7 @@ struct Args {
     float *partials;
     unsigned *status;
     int64_t N, ldx, rows_per_slice;
+    int nb;                                  // slices in flight
     int d, dcols, part_elems;                // part_elems: partial sums per slice; dcols = d rounded up to a multiple of 16
     int ntiles[2];
     Tile tiles[2][MAX_GROUP_TILES];
@@ -89,12 +98,13 @@ moment3_tc_kernel(const __grid_constant__ Args a)
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *a_stage0 = smem;
+    const int NB = a.nb, x_pitch = a.dcols + 1;
+    const uint32_t B_STAGE_BYTES = (uint32_t)a.dcols * ROW_BYTES, X_STAGE_FLOATS = (uint32_t)(KS * x_pitch);
     unsigned char *b_stage0 = smem + (size_t)NA * A_STAGE_BYTES;
-    constexpr int X_STAGE_FLOATS = KS * X_PITCH;
-    float *x_stage0 = (float *)(b_stage0 + (size_t)NB * B_STAGE_BYTES);   // slices of X as they are in memory, [sample][X_PITCH]
-    uint64_t *bars = (uint64_t *)(x_stage0 + (size_t)NB * X_STAGE_FLOATS);
-    uint64_t *a_full = bars, *a_empty = bars + NA_MAX, *b_full = bars + 2 * NA_MAX, *b_empty = bars + 2 * NA_MAX + NB,
-             *acc_full = bars + 2 * NA_MAX + 2 * NB;
+    uint64_t *bars = (uint64_t *)(b_stage0 + (size_t)NB * (B_STAGE_BYTES + 4 * X_STAGE_FLOATS));
+    float *x_stage0 = (float *)(b_stage0 + (size_t)NB * B_STAGE_BYTES);   // slices of X as they are in memory
+    uint64_t *a_full = bars, *a_empty = bars + NA_MAX, *b_full = bars + 2 * NA_MAX, *b_empty = bars + 2 * NA_MAX + NB_MAX,
+             *acc_full = bars + 2 * NA_MAX + 2 * NB_MAX;
     uint64_t *iss_sync = acc_full + 1;
     uint32_t *tmem_slot = (uint32_t *)(acc_full + 2);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
@@ -148,11 +158,12 @@ moment3_tc_kernel(const __grid_constant__ Args a)
         // the A ring) and nprod <= NB * tg (stages covered by the slices of the X^T ring).
         const int nprod = min(min(PRODUCERS, NA), NB * tg);
         bool ok = true;
-        int slice = warp / tg, ti = warp - slice * tg, as = warp, use = 0;     // of stage q
+        int bs = warp / tg, ti = warp - bs * tg, as = warp, use = 0;           // of stage q; bs: ring position of its slice
+        uint32_t b_parity = 0;
+        while (bs >= NB) { bs -= NB; b_parity ^= 1u; }
         const int dslice = nprod / tg, dti = nprod - dslice * tg;
         for (int64_t q = warp; q < nstages && ok && warp < nprod; q += nprod) {
-            const int bs = slice % NB;
-            if (!mbar_wait(&b_full[bs], (uint32_t)((slice / NB) & 1), abort_flag, a.status, 11)) break;
+            if (!mbar_wait(&b_full[bs], b_parity, abort_flag, a.status, 11)) break;
             // this lane's sample: x_i for the tile's 8 values of i, x_j for its 16 values of j
             const unsigned char *bst = b_stage0 + (size_t)bs * B_STAGE_BYTES;
             const Tile t = tiles[ti];
@@ -160,11 +171,11 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             // `lane` + 32, so that every product is rounded once
             uint64_t xi[TI], xj[TJ];                       // TF32: the low word only
             if (BF16) {
-                const float *xst = x_stage0 + (size_t)bs * X_STAGE_FLOATS + lane * X_PITCH;
+                const float *xst = x_stage0 + (size_t)bs * X_STAGE_FLOATS + lane * x_pitch;
 #pragma unroll
-                for (int e = 0; e < TI; ++e) xi[e] = m3tc_pack2(xst[TI * t.ib + e], xst[(BF16 ? 32 : 0) * X_PITCH + TI * t.ib + e]);
+                for (int e = 0; e < TI; ++e) xi[e] = m3tc_pack2(xst[TI * t.ib + e], xst[(BF16 ? 32 : 0) * x_pitch + TI * t.ib + e]);
 #pragma unroll
-                for (int e = 0; e < TJ; ++e) xj[e] = m3tc_pack2(xst[TJ * t.jb + e], xst[(BF16 ? 32 : 0) * X_PITCH + TJ * t.jb + e]);
+                for (int e = 0; e < TJ; ++e) xj[e] = m3tc_pack2(xst[TJ * t.jb + e], xst[(BF16 ? 32 : 0) * x_pitch + TJ * t.jb + e]);
             } else {
 #pragma unroll
                 for (int e = 0; e < TI; ++e) xi[e] = *reinterpret_cast<const uint32_t *>(bst + (TI * t.ib + e) * 128 + sw[e & 7]);
@@ -196,9 +207,10 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             fence_proxy_async();      // generic-proxy stores must be visible to the tensor core
             __syncwarp();
             if (lane == 0) mbar_arrive(&a_full[as]);
-            slice += dslice;
+            bs += dslice;
             ti += dti;
-            if (ti >= tg) { ti -= tg; ++slice; }
+            if (ti >= tg) { ti -= tg; ++bs; }
+            while (bs >= NB) { bs -= NB; b_parity ^= 1u; }
             as += nprod;
             if (as >= NA) { as -= NA; ++use; }
         }
@@ -244,10 +256,12 @@ moment3_tc_kernel(const __grid_constant__ Args a)
         if (elect_one()) {
             bool ok = true;
             int q_slot = 0;                                         // ring slot and phase of stage q = slice * tg + ti
-            uint32_t q_parity = 0;
+            uint32_t q_parity = 0, b_parity = 0;
+            int b_slot = 0;
             for (int slice = 0; slice < nslices && ok; ++slice) {
-                const int bs = slice % NB;
-                if (!mbar_wait(&b_full[bs], (uint32_t)((slice / NB) & 1), abort_flag, a.status, 14)) break;
+                const int bs = b_slot;
+                if (!mbar_wait(&b_full[bs], b_parity, abort_flag, a.status, 14)) break;
+                if (++b_slot == NB) { b_slot = 0; b_parity ^= 1u; }
                 const uint32_t sb = smem_u32(b_stage0 + (size_t)bs * B_STAGE_BYTES);
                 for (int ti = 0; ti < tg; ++ti) {
                     const int as = q_slot;
@@ -299,54 +313,67 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             for (int64_t o = 128 * (int64_t)lt; o < bytes; o += 128 * 32 * LOAD_WARPS) asm volatile("prefetch.global.L2 [%0];" ::"l"(lo + o));
         };
         prefetch(n_begin, n_begin + PREFETCH * KS);
-        // columns d .. dcols-1 are never written again
-        for (int e = lt; e < NB * X_STAGE_FLOATS; e += 32 * LOAD_WARPS) x_stage0[e] = 0.f;
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * LOAD_WARPS) : "memory");
-        // a warp copies 32 / width rows at a time, width lanes along each (and a second time for columns 32 and up)
-        const int width = a.d <= 8 ? 8 : a.d <= 16 ? 16 : 32;
-        const int fr0 = (lw * 32 + lane) / width, fc = lane & (width - 1), fstep = 32 * LOAD_WARPS / width;
-        auto fetch = [&](int slice) {
+        // a warp copies 32 / W rows at a time, W lanes along each (and a second time for columns 32 and up); lanes past
+        // column d and samples past the end write zeros
+        auto copy_rows = [&](auto width, int64_t n0, int rows, uint32_t dst) {
+            constexpr int W = decltype(width)::value, STEP = 32 * LOAD_WARPS / W;
+            const int r0 = lt / W, c = lt % W;
+            const float *src = a.X + (n0 + r0) * a.ldx + c;
+            const int64_t src_step = STEP * a.ldx;
+            const bool c0 = c < a.d, c1 = W == 32 && c + 32 < a.d, wide = W == 32 && a.dcols > 32;
+            dst += (uint32_t)(r0 * x_pitch + c) * 4u;
+#pragma unroll 8
+            for (int r = r0; r < KS; r += STEP, dst += (uint32_t)(STEP * x_pitch) * 4u, src += src_step) {
+                const bool p0 = c0 && r < rows, p1 = c1 && r < rows;
+                const float *s0 = p0 ? src : a.X, *s1 = p1 ? src + 32 : a.X;
+                if (W == 32 || c < a.dcols)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(s0), "r"(p0 ? 4 : 0));
+                if (wide && c + 32 < a.dcols)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 128u), "l"(s1), "r"(p1 ? 4 : 0));
+            }
+        };
+        int fetch_slot = 0;
+        auto fetch = [&](int slice) {                                     // called with slice = 0, 1, 2, ...
             const int64_t n0 = n_begin + (int64_t)slice * KS;
             const int rows = n_end - n0 < KS ? (int)(n_end - n0) : KS;
-            uint32_t dst = smem_u32(x_stage0 + (size_t)(slice % NB) * X_STAGE_FLOATS + fr0 * X_PITCH + fc);
-            const float *src = a.X + (n0 + fr0) * a.ldx + fc;
-            const int64_t src_step = fstep * a.ldx;
-            const bool c0 = fc < a.d, c1 = fc + 32 < a.d;
-#pragma unroll 4
-            for (int r = fr0; r < KS; r += fstep, dst += (uint32_t)(fstep * X_PITCH * 4), src += src_step) {
-                const bool in = r < rows;                                  // samples past the end: zeros
-                const int sz = in ? 4 : 0;
-                if (c0) asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(in ? src : a.X), "r"(sz));
-                if (c1) asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 128u), "l"(in ? src + 32 : a.X), "r"(sz));
-            }
+            const uint32_t dst = smem_u32(x_stage0 + (size_t)fetch_slot * X_STAGE_FLOATS);
+            if (++fetch_slot == NB) fetch_slot = 0;
+            if (a.dcols == 16) copy_rows(std::integral_constant<int, 16>{}, n0, rows, dst);
+            else copy_rows(std::integral_constant<int, 32>{}, n0, rows, dst);
             prefetch(n0 + PREFETCH * KS, n0 + (PREFETCH + 1) * KS);
         };
-        for (int s = 0; s < FETCH_AHEAD; ++s) {
+        const int ahead = fetch_ahead(NB);
+        for (int s = 0; s < ahead; ++s) {
             if (s < nslices) fetch(s);
             asm volatile("cp.async.commit_group;" ::: "memory");
         }
+        int bs = 0;
+        uint32_t free_parity = 1;                                         // of the buffers that the next fetch fills
         for (int slice = 0; slice < nslices; ++slice) {
-            const int bs = slice % NB;
             // a slice's buffers are free once the MMAs of the slice NB before it are complete
             uint32_t failed = 0;
-            const int next = slice + FETCH_AHEAD, use = next / NB;
+            const int next = slice + ahead;
             if (next < nslices) {
-                if (use > 0 && !mbar_wait(&b_empty[next % NB], (uint32_t)((use - 1) & 1), abort_flag, a.status, 16)) failed = 1;
+                if (next >= NB && fetch_slot == 0) free_parity ^= 1u;
+                if (next >= NB && !mbar_wait(&b_empty[fetch_slot], free_parity, abort_flag, a.status, 16)) failed = 1;
                 else fetch(next);
             }
-            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group %0;" ::"n"(FETCH_AHEAD) : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (ahead == 8) asm volatile("cp.async.wait_group 8;" ::: "memory");
+            else if (ahead == 5) asm volatile("cp.async.wait_group 5;" ::: "memory");
+            else asm volatile("cp.async.wait_group 2;" ::: "memory");
             // every loader's copies of the slice have landed; all loaders leave together if one gave up
             asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %0, 0;\n\tbar.red.or.pred q, 1, %1, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
                          : "+r"(failed) : "n"(32 * LOAD_WARPS) : "memory");
             if (failed) break;
             unsigned char *bst = b_stage0 + (size_t)bs * B_STAGE_BYTES;
-            const float *xst = x_stage0 + (size_t)bs * X_STAGE_FLOATS + lane * X_PITCH;
+            const float *xst = x_stage0 + (size_t)bs * X_STAGE_FLOATS + lane * x_pitch;
             for (int c8 = 8 * lw; c8 < a.dcols; c8 += 8 * LOAD_WARPS) {
                 float x[8], y[8];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     x[c] = xst[c8 + c];
-                    y[c] = BF16 ? xst[(BF16 ? 32 * X_PITCH : 0) + c8 + c] : 0.f;
+                    y[c] = BF16 ? xst[(BF16 ? 32 * x_pitch : 0) + c8 + c] : 0.f;
                 }
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
@@ -359,6 +386,7 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(&b_full[bs]);
+            if (++bs == NB) bs = 0;
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     }
@@ -488,23 +516,24 @@ st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *o
     if (!aligned256(ws)) return ST_ERR_ALIGN;
     const DeviceInfo di = device_info();
     if (!di.ok) return ST_ERR_CUDA;
-    if (smem_bytes(bf16) > (size_t)di.max_smem_optin) return ST_ERR_UNSUPPORTED;
+    if (smem_bytes(p.dcols, bf16) > (size_t)di.max_smem_optin) return ST_ERR_UNSUPPORTED;
     Args a;
     a.X = X;
     a.partials = (float *)((unsigned char *)ws + kWsHeaderBytes);
     a.status = (unsigned *)ws;
     a.N = N; a.ldx = ldx; a.rows_per_slice = p.rows_per_slice;
+    a.nb = ring(p.dcols, bf16);
     a.d = (int)d; a.dcols = p.dcols; a.part_elems = p.part_elems;
     for (int g = 0; g < 2; ++g) {
         a.ntiles[g] = p.ntiles[g];
         for (int t = 0; t < MAX_GROUP_TILES; ++t) a.tiles[g][t] = p.tiles[g][t];
     }
     if (bf16) {
-        if (!ensure_dynamic_smem(moment3_tc_kernel<true>, smem_bytes(true))) return ST_ERR_CUDA;
-        moment3_tc_kernel<true><<<dim3(p.groups, p.slices), THREADS, smem_bytes(true), stream>>>(a);
+        if (!ensure_dynamic_smem(moment3_tc_kernel<true>, smem_bytes(p.dcols, true))) return ST_ERR_CUDA;
+        moment3_tc_kernel<true><<<dim3(p.groups, p.slices), THREADS, smem_bytes(p.dcols, true), stream>>>(a);
     } else {
-        if (!ensure_dynamic_smem(moment3_tc_kernel<false>, smem_bytes(false))) return ST_ERR_CUDA;
-        moment3_tc_kernel<false><<<dim3(p.groups, p.slices), THREADS, smem_bytes(false), stream>>>(a);
+        if (!ensure_dynamic_smem(moment3_tc_kernel<false>, smem_bytes(p.dcols, false))) return ST_ERR_CUDA;
+        moment3_tc_kernel<false><<<dim3(p.groups, p.slices), THREADS, smem_bytes(p.dcols, false), stream>>>(a);
     }
     if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
     SumArgs m;
