@@ -1,14 +1,16 @@
-// st_sym_moment2, tensor-core path: out[p(i,j)] = sum_n X[n,i] X[n,j], X in bfloat16, fp32
-// accumulation (Section 3, M1; the outer product summed over samples is a symmetric
-// rank-N update, i.e. a triangular tile GEMM X^T X).
+// st_sym_moment2, tensor-core paths: out[p(i,j)] = sum_n X[n,i] X[n,j], fp32 accumulation (Section 3, M1; the outer
+// product summed over samples is a symmetric rank-N update, i.e. a triangular tile GEMM X^T X).  Three forms of X:
+//   M2_BF16   bfloat16
+//   M2_TF32   fp32, of which the tensor core reads the upper 19 bits
+//   M2_SPLIT  fp32 written by a pass of its own as x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi
 //
-// Output tiles are 128 rows (i) x 256 columns (j).  Only tiles that contain an entry with
-// i <= j are launched; tiles wholly below the diagonal are never issued, and of a tile whose
-// left 128 columns lie below the diagonal only the right 128 x 128 half is issued (N = 128).
-// The sample range of every tile is split over the same number of blocks, so that the blocks of
-// one sample range run in step and share X through L2; every block accumulates its tile
-// over its samples in tensor memory and keeps an fp32 partial tile; a second kernel adds
-// the partials of a tile in fixed order and writes the packed upper triangle.
+// A cluster of two blocks owns an output tile of 256 rows (i) x up to 256 columns (j) for a range of the samples.
+// Only tiles that contain an entry with i <= j are launched, and a tile of the last column is as wide as the columns
+// left, rounded up to 32.  Block r of the pair stages columns 256*TM+128r.. (its 128 rows of the A operand) and its
+// half of the columns of the B operand; on full diagonal tiles the two coincide and are loaded once.  The leader block
+// issues one MMA of M = 256 for the pair; each block keeps the accumulator of its 128 rows in its own tensor memory
+// and adds it into an fp32 partial tile; a second kernel adds the partial tiles of all sample ranges in a fixed order
+// and writes the packed upper triangle.
 //
 // The tensor core adds into its fp32 accumulator without round-to-nearest, so a chain of
 // many thousands of accumulating MMAs drifts low (measured: -7.7e-4 relative on all-positive
@@ -18,10 +20,16 @@
 //
 // Both operands of X^T X are "MN-major" for the tensor core: X is [N, d] row-major, so the
 // output index (i or j) is contiguous and the reduction index n strides by a row.  TMA
-// loads boxes of 64 columns x 64 rows with the 128-byte swizzle, which is exactly the
-// canonical MN-major layout of tcgen05 (8 rows x 128 bytes per swizzle atom).  When the
-// 128 columns of the A panel lie inside the columns of the B panel (tiles on the diagonal)
-// only the B panel is loaded and A aliases it.
+// loads boxes of 128 bytes x KROWS rows with the 128-byte swizzle, which is exactly the
+// canonical MN-major layout of tcgen05 (8 rows x 128 bytes per swizzle atom).  An MN-major operand of 32-bit elements
+// (TF32) has one legal shared-memory form, the 128-byte swizzle of 32-byte units, which the copies write (tensor-map
+// swizzle "128B, atom 32B") and the descriptors name.
+//
+// What bounds it: wide tiles the tensor pipe and the L2 that feeds it; every column panel is read by all tiles of its
+// row and column, so clusters that work on the same samples must run in step to share X in L2.  Four stages of 32 KB
+// are the measured optimum there: with six or seven the clusters of a sample range drift apart and the kernel gets
+// 5-12% slower, with three it starves.  M2_SPLIT makes its three products from one load of both parts (64 instead of
+// 96 bytes per sample and column pair).  Few features: the latency of a stage, hence more and smaller stages.
 //
 // Warp roles (192 threads): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner,
 // warps 2..5 = epilogue (TMEM -> registers -> global), one per 32-lane quarter of TMEM.
@@ -31,291 +39,93 @@
 
 namespace st {
 
+enum { M2_BF16 = 0, M2_TF32 = 1, M2_SPLIT = 2 };
+
 namespace m2tc {
-constexpr int BM = 128, BN = 256;
-constexpr int KROWS = 64;                       // sample rows per pipeline stage
-constexpr int BOXC = 64;                        // columns per TMA box (128 bytes of bf16)
-constexpr int BOX_BYTES = BOXC * KROWS * 2;     // 8 KiB
-constexpr int NBOX_A = BM / BOXC, NBOX_B = BN / BOXC;
-constexpr int STAGE_BYTES = (NBOX_A + NBOX_B) * BOX_BYTES;   // 48 KiB
-constexpr int STAGES = 4;
-constexpr int THREADS = 192;
-constexpr int MAX_TILES = 288;
-constexpr int MAX_BLOCKS = 448;
-constexpr uint32_t TMEM_COLS = 512;              // two 128 x 256 fp32 accumulators
-constexpr int FLUSH_CHUNKS = 64;                 // stages (of 64 samples) per accumulator phase
-constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
-
-struct TileTable {
-    int ntiles, nblocks;
-    unsigned short tm[MAX_TILES];          // tile row (units of 128)
-    unsigned short tn[MAX_TILES];          // tile column (units of 256)
-    unsigned char half[MAX_TILES];         // 1: only columns 128..255 of the tile are issued
-    unsigned short nsplit[MAX_TILES];      // blocks that share the samples of this tile
-    unsigned short first_block[MAX_TILES];
-    unsigned short blk_tile[MAX_BLOCKS];   // block -> tile
-};
-}  // namespace m2tc
-
-__global__ void __launch_bounds__(m2tc::THREADS, 1)
-moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict__ partials, unsigned *status,
-                  int chunks_total, const __grid_constant__ m2tc::TileTable tab)
-{
-    using namespace m2tc;
-    using namespace tc;
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t *bars = (uint64_t *)(smem + (size_t)STAGES * STAGE_BYTES);
-    uint64_t *full = bars, *empty = bars + STAGES, *acc_full = bars + 2 * STAGES, *acc_empty = bars + 2 * STAGES + 2;
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * STAGES + 4);
-    volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tile = tab.blk_tile[blockIdx.x];
-    const int split = (int)blockIdx.x - tab.first_block[tile];
-    const int nsplit = tab.nsplit[tile];
-    const int tm = tab.tm[tile], tn = tab.tn[tile];
-    const bool half = tab.half[tile] != 0;
-    const bool a_in_b = (tm >> 1) == tn;
-    const int chunks_per_split = (chunks_total + nsplit - 1) / nsplit;
-    const int c_begin = split * chunks_per_split;
-    int c_end = c_begin + chunks_per_split;
-    if (c_end > chunks_total) c_end = chunks_total;
-    const int nchunks = c_end > c_begin ? c_end - c_begin : 0;
-    const int nphases = (nchunks + FLUSH_CHUNKS - 1) / FLUSH_CHUNKS;
-    const int ncols = half ? BN / 2 : BN;                 // issued columns of the tile
-    const int b_box0 = half ? NBOX_B / 2 : 0;             // first B box that is loaded
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 4);     // one arrival per epilogue warp
-        }
-        *abort_flag = 0;
-        if (blockIdx.x == 0) {
-            // the status words are cleared here instead of by a separate memset; a time-out
-            // report can only be written 2^24 failed polls later
-            status[kWsStatusWord] = 0;
-            status[kWsDetailWord] = 0;
-        }
-        fence_barrier_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(tmem_slot, TMEM_COLS);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-
-    if (warp == 0) {
-        // ---------------- TMA producer
-        if (elect_one()) {
-            prefetch_tmap(&tmap);
-            const int nb_boxes = NBOX_B - b_box0;
-            const uint32_t tx = (uint32_t)((a_in_b ? nb_boxes : NBOX_A + nb_boxes) * BOX_BYTES);
-            for (int c = 0; c < nchunks; ++c) {
-                const int s = c % STAGES;
-                if (c >= STAGES && !mbar_wait(&empty[s], ((c / STAGES) - 1) & 1, abort_flag, status, 1)) break;
-                unsigned char *st_base = smem + (size_t)s * STAGE_BYTES;
-                mbar_expect_tx(&full[s], tx);
-                const int row = (c_begin + c) * KROWS;
-                for (int b = b_box0; b < NBOX_B; ++b)
-                    tma_load_2d(st_base + b * BOX_BYTES, &tmap, &full[s], tn * BN + b * BOXC, row);
-                if (!a_in_b)
-                    for (int b = 0; b < NBOX_A; ++b)
-                        tma_load_2d(st_base + (NBOX_B + b) * BOX_BYTES, &tmap, &full[s], tm * BM + b * BOXC, row);
-            }
-        }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer
-        if (elect_one()) {
-            const uint32_t idesc = half ? make_idesc(1, 1, 1, BM, BN / 2) : make_idesc(1, 1, 1, BM, BN);
-            const uint32_t a_off = a_in_b ? (uint32_t)((tm & 1) * NBOX_A * BOX_BYTES) : (uint32_t)(NBOX_B * BOX_BYTES);
-            const uint32_t b_off = (uint32_t)(b_box0 * BOX_BYTES);
-            // descriptors of k-step 0 of every stage; a k-step of 16 rows advances the start
-            // address by two swizzle atoms (2048 bytes = 128 in descriptor units)
-            const uint32_t sb0 = smem_u32(smem);
-            const uint64_t adesc_base = make_smem_desc(sb0 + a_off, BOX_BYTES, 1024);
-            const uint64_t bdesc_base = make_smem_desc(sb0 + b_off, BOX_BYTES, 1024);
-            bool ok = true;
-            int c = 0;
-            for (int ph = 0; ph < nphases && ok; ++ph) {
-                const int buf = ph & 1;
-                if (ph >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((ph >> 1) - 1) & 1), abort_flag, status, 4)) break;
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
-                const int ce = (c + FLUSH_CHUNKS < nchunks) ? c + FLUSH_CHUNKS : nchunks;
-                uint32_t accumulate = 0;
-                for (; c < ce; ++c) {
-                    const int s = c % STAGES;
-                    if (!mbar_wait(&full[s], (c / STAGES) & 1, abort_flag, status, 2)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint64_t ad = adesc_base + (uint64_t)(s * (STAGE_BYTES >> 4));
-                    const uint64_t bd = bdesc_base + (uint64_t)(s * (STAGE_BYTES >> 4));
-#pragma unroll
-                    for (int k = 0; k < KROWS / 16; ++k) {
-                        mma_bf16(d_tmem, ad + (uint64_t)(k * 128), bd + (uint64_t)(k * 128), idesc, accumulate);
-                        accumulate = 1;
-                    }
-                    tc_commit(&empty[s]);          // frees the stage when these MMAs have read it
-                }
-                tc_commit(&acc_full[buf]);         // this accumulator phase is complete
-            }
-        }
-    } else {
-        // ---------------- epilogue: TMEM lanes 32q..32q+31 belong to warp q = warp % 4
-        const int q = warp & 3;
-        float *dst = partials + ((size_t)blockIdx.x * BM + (q * 32 + lane)) * BN;
-        if (nphases == 0) {
-            for (int c0 = 0; c0 < ncols; c0 += 4) *reinterpret_cast<float4 *>(dst + c0) = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        for (int ph = 0; ph < nphases; ++ph) {
-            const int buf = ph & 1;
-            if (!mbar_wait(&acc_full[buf], (uint32_t)((ph >> 1) & 1), abort_flag, status, 3)) break;
-            tc_fence_after();
-#pragma unroll 1
-            for (int c0 = 0; c0 < ncols; c0 += 32) {
-                uint32_t r[32];
-                tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c0), r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int e = 0; e < 32; e += 4) {
-                    float4 v = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
-                                           __uint_as_float(r[e + 3]));
-                    float4 *p = reinterpret_cast<float4 *>(dst + c0 + e);
-                    if (ph > 0) {
-                        const float4 o = *p;        // written by this same thread in the previous phase
-                        v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
-                    }
-                    *p = v;
-                }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem_base, TMEM_COLS);
-    }
-}
-
-// out[p(i,j)] = sum over splits of the partial tiles, i <= j only.
-__global__ void __launch_bounds__(256)
-moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d,
-                         const __grid_constant__ m2tc::TileTable tab)
-{
-    using namespace m2tc;
-    const int tile = blockIdx.x;
-    const int tm = tab.tm[tile], tn = tab.tn[tile], nsplit = tab.nsplit[tile];
-    const int ncols = tab.half[tile] ? BN / 2 : BN;
-    const int col0 = tn * BN + (tab.half[tile] ? BN / 2 : 0);
-    const float *base = partials + (size_t)tab.first_block[tile] * (BM * BN);
-    for (int e = blockIdx.y * 256 + threadIdx.x; e < BM * BN; e += gridDim.y * 256) {
-        const int r = e / BN, c = e - r * BN;
-        const int gi = tm * BM + r, gj = col0 + c;
-        if (c < ncols && gi < d && gj < d && gi <= gj) {
-            float s = 0.f;
-            for (int k0 = 0; k0 < nsplit; k0 += 8) {
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = (k0 + u < nsplit) ? __ldcg(&base[(size_t)(k0 + u) * (BM * BN) + e]) : 0.f;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) s += v[u];
-            }
-            if (ST_BOUNDS_OK(tri_encode(d, gi, gj), tri_rows(d), 2)) out[tri_encode(d, gi, gj)] = s;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
-// Two-block variant (d >= 512): a cluster of two blocks owns a 256 x 256 tile.  Block r stages
-// columns 256*TM+128r.. (its 128 rows of the A operand) and columns 256*TN+128r.. (its half of
-// the B operand); on diagonal tiles the two coincide and are loaded once.  The leader block
-// issues one MMA of M = 256, N = 256 for the pair; each block keeps the accumulator of its 128
-// rows in its own tensor memory.  Per MMA cycle a block now fetches a third less from L2 than in
-// the one-block kernel (whose tensor pipe idled ~30% of the time waiting for operands).  Four
-// stages of 64 samples are the measured optimum: with 6 or 7 stages the blocks of a sample range
-// drift apart, share less of X in L2 and the kernel gets 5-12% slower; with 3 it starves.
-//
-// The same kernel reads an fp32 X as TF32 (template argument): the tensor core takes the upper 19 bits of every
-// fp32 word, so the boxes are 32 columns (128 bytes) wide, a stage holds 32 samples and an MMA spans 8 of them;
-// the bytes per stage, the MMAs per stage and everything after the accumulator are the same.  An MN-major
-// operand of 32-bit elements has one legal shared-memory form, the 128-byte swizzle of 32-byte units, which
-// the copies write (tensor-map swizzle "128B, atom 32B") and the descriptors name.
-namespace m2tc2 {
 constexpr int BM = 256, BN = 256;               // tile of the pair
-constexpr int HALF = 128;                       // rows / B columns staged per block
-constexpr int STAGE_BYTES = 32768;              // HALF columns of A and of B over the sample rows of one stage
-constexpr int STAGES = 4;
+constexpr int HALF = 128;                       // rows staged per block, and most B columns
+constexpr int MAX_STAGES = 24;
+constexpr size_t STAGES_BYTES = 131072;         // all stages together
+constexpr size_t STAGES_BYTES_1 = 196608;       // a single tile: nobody to keep in step with
 constexpr int THREADS = 192;
 constexpr int MAX_TILES = 160;
 constexpr uint32_t TMEM_COLS = 512;
-constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
-template <bool TF32> struct Shape {
-    static constexpr int ELEM = TF32 ? 4 : 2;
-    static constexpr int KROWS = TF32 ? 32 : 64;            // sample rows per stage
-    static constexpr int KMMA = TF32 ? 8 : 16;              // sample rows per MMA
+template <int MODE> struct Shape {
+    static constexpr int ELEM = MODE == M2_TF32 ? 4 : 2;
+    static constexpr int PARTS = MODE == M2_SPLIT ? 2 : 1;  // hi and lo
+    static constexpr int KROWS = MODE == M2_BF16 ? 64 : 32; // sample rows per stage
+    static constexpr int KMMA = MODE == M2_TF32 ? 8 : 16;   // sample rows per MMA
     static constexpr int BOXC = 128 / ELEM;                 // columns per TMA box (128 bytes)
     static constexpr int BOX_BYTES = 128 * KROWS;
-    static constexpr int NBOX = HALF / BOXC;                // boxes per operand per block
-    static constexpr int FLUSH_CHUNKS = 4096 / KROWS;       // 4096 samples (256 or 512 MMAs) per accumulator phase
-    static_assert(2 * NBOX * BOX_BYTES == STAGE_BYTES, "stage size");
+    static constexpr int NBOX = HALF / BOXC;                // most boxes per operand and part in a block
+    // accumulating MMAs per phase: 256 (bf16), 512 (TF32, half the samples each), 252 (split)
+    static constexpr int FLUSH_CHUNKS = MODE == M2_BF16 ? 64 : MODE == M2_TF32 ? 128 : 42;
 };
 
 struct TileTable {
-    int ntiles, nsplit;
-    unsigned char tm[MAX_TILES];   // units of 256
-    unsigned char tn[MAX_TILES];
+    int ntiles;
+    unsigned char tm[MAX_TILES], tn[MAX_TILES];        // tile row and column (units of 256)
+    unsigned char width[MAX_TILES];                    // columns, units of 32
+    unsigned short first[MAX_TILES + 1];               // first cluster: the clusters of a tile share its samples
 };
-}  // namespace m2tc2
+struct Args {
+    float *partials;                                   // [2 * cluster + block][HALF][BN]
+    unsigned *status;
+    int d, chunks_total, stages, nb, na;               // nb, na: boxes of B and A per part in a stage
+    int lo_row0;                                       // M2_SPLIT: first row of the lo part
+    TileTable tab;
+};
+}  // namespace m2tc
 
-template <bool TF32>
-__global__ void __launch_bounds__(m2tc2::THREADS, 1)
-moment2_tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict__ partials, unsigned *status,
-                       int chunks_total, const __grid_constant__ m2tc2::TileTable tab, int seg_chunks, int lo_row0)
+// Tile of a cluster.
+__device__ __forceinline__ int m2tc_tile_of(const m2tc::TileTable &t, int cluster)
 {
-    // seg_chunks > 0: the rows of the tensor are [hi part of X; lo part of X] (lo_row0 = first row of the lo part)
-    // and the sample loop runs over three segments of seg_chunks stages: A and B from hi, A from hi and B from lo,
-    // A from lo and B from hi -- the sum is hi^T hi + hi^T lo + lo^T hi, symmetric, so the tiles stay the upper ones.
-    using namespace m2tc2;
+    int lo = 0, hi = t.ntiles - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((int)t.first[mid] <= cluster) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(m2tc::THREADS, 1)
+moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ m2tc::Args a)
+{
+    using namespace m2tc;
     using namespace tc;
-    using S = Shape<TF32>;
-    constexpr int KROWS = S::KROWS, BOXC = S::BOXC, BOX_BYTES = S::BOX_BYTES, NBOX = S::NBOX, FLUSH_CHUNKS = S::FLUSH_CHUNKS;
+    using S = Shape<MODE>;
+    constexpr int KROWS = S::KROWS, BOXC = S::BOXC, BOX_BYTES = S::BOX_BYTES, NBOX = S::NBOX;
+    constexpr int PARTS = S::PARTS;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t *bars = (uint64_t *)(smem + (size_t)STAGES * STAGE_BYTES);
-    uint64_t *full = bars, *empty = bars + STAGES, *acc_full = bars + 2 * STAGES, *acc_empty = bars + 2 * STAGES + 2;
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * STAGES + 4);
+    const uint32_t part_bytes = (uint32_t)((a.nb + a.na) * BOX_BYTES), stage_bytes = PARTS * part_bytes;
+    const int stages = a.stages;
+    // an MMA reads 128 columns of A per block, na boxes of which were loaded: behind the last stage there is room for the others
+    uint64_t *bars = (uint64_t *)(smem + (size_t)stages * stage_bytes + (size_t)(NBOX - a.na) * BOX_BYTES);
+    uint64_t *full = bars, *empty = bars + MAX_STAGES, *acc_full = bars + 2 * MAX_STAGES, *acc_empty = bars + 2 * MAX_STAGES + 2;
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * MAX_STAGES + 4);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();            // 0 = leader
     const int cluster = blockIdx.x >> 1;
-    const int tile = cluster / tab.nsplit, split = cluster - tile * tab.nsplit;
-    const int tm = tab.tm[tile], tn = tab.tn[tile];
-    const bool diag = (tm == tn) && seg_chunks == 0;    // A columns == B columns (and rows) in every block: one load serves both
-    const int chunks_per_split = (chunks_total + tab.nsplit - 1) / tab.nsplit;
+    const int tile = m2tc_tile_of(a.tab, cluster), split = cluster - a.tab.first[tile];
+    const int nsplit = a.tab.first[tile + 1] - a.tab.first[tile];
+    const int tm = a.tab.tm[tile], tn = a.tab.tn[tile], width = 32 * a.tab.width[tile];
+    // narrow tiles are cheap to flush: chains half as long, as short as those of twice as many sample ranges
+    const int FLUSH_CHUNKS = MODE == M2_BF16 && width <= HALF ? S::FLUSH_CHUNKS / 2 : S::FLUSH_CHUNKS;
+    const bool alias = tm == tn && width == BN;         // A columns == B columns in both blocks: one load serves both
+    const int chunks_per_split = (a.chunks_total + nsplit - 1) / nsplit;
     const int c_begin = split * chunks_per_split;
     int c_end = c_begin + chunks_per_split;
-    if (c_end > chunks_total) c_end = chunks_total;
+    if (c_end > a.chunks_total) c_end = a.chunks_total;
     const int nchunks = c_end > c_begin ? c_end - c_begin : 0;
     const int nphases = (nchunks + FLUSH_CHUNKS - 1) / FLUSH_CHUNKS;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < stages; ++s) {
             mbar_init(&full[s], 1);          // leader's producer arrives once and announces the bytes of both blocks
             mbar_init(&empty[s], 1);         // one commit per use, delivered to both blocks
         }
@@ -327,8 +137,8 @@ moment2_tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, float *__restri
         if (blockIdx.x == 0) {
             // the status words are cleared here instead of by a separate memset; a time-out
             // report can only be written 2^24 failed polls later
-            status[kWsStatusWord] = 0;
-            status[kWsDetailWord] = 0;
+            a.status[kWsStatusWord] = 0;
+            a.status[kWsDetailWord] = 0;
         }
         fence_barrier_init();
     }
@@ -341,99 +151,121 @@ moment2_tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, float *__restri
     cluster_sync_all();                      // both blocks' barriers exist before anything is signalled across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the kernel that writes the operand may still be running
 
     if (warp == 0) {
         // ---------------- TMA producer (both blocks): own boxes, completion counted on the leader's barrier
         if (elect_one()) {
             prefetch_tmap(&tmap);
-            const uint32_t own_tx = (uint32_t)((diag ? NBOX : 2 * NBOX) * BOX_BYTES);
+            // boxes of A that hold columns of X (the others would only make rows that are never read)
+            auto boxes_a = [&](int r) {
+                const int left = a.d - tm * BM - r * HALF;
+                return alias || left <= 0 ? 0 : left >= HALF ? NBOX : (left + BOXC - 1) / BOXC;
+            };
+            const int nb = (width / 2 + BOXC - 1) / BOXC, na = boxes_a((int)rank);
+            const uint32_t tx = (uint32_t)((2 * nb + boxes_a(0) + boxes_a(1)) * PARTS * BOX_BYTES);
+            const int col_a = tm * BM + (int)rank * HALF, col_b = tn * BN + (int)rank * (width / 2);
+            const uint32_t bar0 = map_to_cta(smem_u32(full), 0);
+            int s = 0;
+            uint32_t parity = 1;
             for (int c = 0; c < nchunks; ++c) {
-                const int s = c % STAGES;
-                if (c >= STAGES && !mbar_wait(&empty[s], ((c / STAGES) - 1) & 1, abort_flag, status, 1)) break;
-                unsigned char *st_base = smem + (size_t)s * STAGE_BYTES;
-                if (rank == 0) mbar_expect_tx(&full[s], 2 * own_tx);
-                const uint32_t bar = map_to_cta(smem_u32(&full[s]), 0);
-                int row_a = (c_begin + c) * KROWS, row_b = row_a;
-                if (seg_chunks > 0) {
-                    const int gc = c_begin + c, seg = gc / seg_chunks;
-                    row_a = row_b = (gc - seg * seg_chunks) * KROWS;
-                    if (seg == 1) row_b += lo_row0;
-                    if (seg == 2) row_a += lo_row0;
+                if (c >= stages && !mbar_wait(&empty[s], parity, abort_flag, a.status, 1)) break;
+                if (rank == 0) mbar_expect_tx(&full[s], tx);
+                const uint32_t bar = bar0 + (uint32_t)(s * sizeof(uint64_t));
+                const int row = (c_begin + c) * KROWS;
+#pragma unroll
+                for (int p = 0; p < PARTS; ++p) {
+                    unsigned char *base = smem + (size_t)s * stage_bytes + (size_t)p * part_bytes;
+                    const int y = row + (p ? a.lo_row0 : 0);
+                    for (int b = 0; b < nb; ++b)            // B half (and A on full diagonal tiles)
+                        tma_load_2d_pair(base + b * BOX_BYTES, &tmap, bar, col_b + b * BOXC, y);
+                    for (int b = 0; b < na; ++b)            // A rows of this block
+                        tma_load_2d_pair(base + (a.nb + b) * BOX_BYTES, &tmap, bar, col_a + b * BOXC, y);
                 }
-                for (int b = 0; b < NBOX; ++b)          // B half (and A on diagonal tiles)
-                    tma_load_2d_pair(st_base + b * BOX_BYTES, &tmap, bar, tn * BN + (int)rank * HALF + b * BOXC, row_b);
-                if (!diag)
-                    for (int b = 0; b < NBOX; ++b)      // A rows of this block
-                        tma_load_2d_pair(st_base + (NBOX + b) * BOX_BYTES, &tmap, bar, tm * BM + (int)rank * HALF + b * BOXC, row_a);
+                if (++s == stages) { s = 0; parity ^= 1u; }
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader only)
         if (rank == 0 && elect_one()) {
-            constexpr uint32_t idesc = make_idesc(TF32 ? 2 : 1, 1, 1, BM, BN);
-            const uint32_t a_off = diag ? 0u : (uint32_t)(NBOX * BOX_BYTES);
+            const uint32_t idesc = make_idesc(MODE == M2_TF32 ? 2 : 1, 1, 1, BM, (uint32_t)width);
+            const uint32_t a_off = alias ? 0u : (uint32_t)(a.nb * BOX_BYTES);
             const uint32_t sb0 = smem_u32(smem);
             // bf16: groups of 8 sample rows, 16-byte swizzle units; fp32 read as TF32: groups of 4, 32-byte units
-            const uint64_t adesc_base = make_smem_desc(sb0 + a_off, BOX_BYTES, TF32 ? 512 : 1024, TF32 ? 1 : 2);
-            const uint64_t bdesc_base = make_smem_desc(sb0, BOX_BYTES, TF32 ? 512 : 1024, TF32 ? 1 : 2);
+            const uint64_t adesc_base = make_smem_desc(sb0 + a_off, BOX_BYTES, MODE == M2_TF32 ? 512 : 1024, MODE == M2_TF32 ? 1 : 2);
+            const uint64_t bdesc_base = make_smem_desc(sb0, BOX_BYTES, MODE == M2_TF32 ? 512 : 1024, MODE == M2_TF32 ? 1 : 2);
+            const uint64_t lo = (uint64_t)(part_bytes >> 4);
             bool ok = true;
-            int c = 0;
+            int c = 0, s = 0;
+            uint32_t parity = 0;
             for (int ph = 0; ph < nphases && ok; ++ph) {
                 const int buf = ph & 1;
-                if (ph >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((ph >> 1) - 1) & 1), abort_flag, status, 4)) break;
+                if (ph >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((ph >> 1) - 1) & 1), abort_flag, a.status, 4)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
                 const int ce = (c + FLUSH_CHUNKS < nchunks) ? c + FLUSH_CHUNKS : nchunks;
                 uint32_t accumulate = 0;
                 for (; c < ce; ++c) {
-                    const int s = c % STAGES;
-                    if (!mbar_wait(&full[s], (c / STAGES) & 1, abort_flag, status, 2)) {
+                    if (!mbar_wait(&full[s], parity, abort_flag, a.status, 2)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint64_t ad = adesc_base + (uint64_t)(s * (STAGE_BYTES >> 4));
-                    const uint64_t bd = bdesc_base + (uint64_t)(s * (STAGE_BYTES >> 4));
+                    const uint64_t ad = adesc_base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
+                    const uint64_t bd = bdesc_base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
 #pragma unroll
                     for (int k = 0; k < KROWS / S::KMMA; ++k) {
                         // one MMA spans KMMA sample rows of 128 bytes: 2048 bytes (bf16) or 1024 bytes (TF32) further on
                         constexpr int STEP = S::KMMA * 128 / 16;
-                        if (TF32) mma_tf32_pair(d_tmem, ad + (uint64_t)(k * STEP), bd + (uint64_t)(k * STEP), idesc, accumulate);
-                        else mma_bf16_pair(d_tmem, ad + (uint64_t)(k * STEP), bd + (uint64_t)(k * STEP), idesc, accumulate);
+                        const uint64_t ak = ad + (uint64_t)(k * STEP), bk = bd + (uint64_t)(k * STEP);
+                        if (MODE == M2_TF32) mma_tf32_pair(d_tmem, ak, bk, idesc, accumulate);
+                        else mma_bf16_pair(d_tmem, ak, bk, idesc, accumulate);
                         accumulate = 1;
+                        if (MODE == M2_SPLIT) {
+                            mma_bf16_pair(d_tmem, ak, bk + lo, idesc, 1u);
+                            mma_bf16_pair(d_tmem, ak + lo, bk, idesc, 1u);
+                        }
                     }
                     tc_commit_pair(&empty[s]);
+                    if (++s == stages) { s = 0; parity ^= 1u; }
                 }
                 tc_commit_pair(&acc_full[buf]);
             }
         }
     } else {
-        // ---------------- epilogue (both blocks): own 128 rows of the tile
+        // ---------------- epilogue (both blocks): own 128 rows of the tile; what lies past column d or wholly below the
+        // diagonal is not stored (the reduction reads i <= j < d only)
         const int q = warp & 3;
-        float *dst = partials + ((size_t)blockIdx.x * HALF + (q * 32 + lane)) * BN;
+        const int row0 = (int)rank * HALF + q * 32;
+        const bool rows = tm * BM + row0 < a.d;
+        const int c_first = tm == tn ? row0 : 0;         // row0 is a multiple of 32
+        float *dst = a.partials + ((size_t)blockIdx.x * HALF + (q * 32 + lane)) * BN;
         const uint32_t leader_acc_empty0 = map_to_cta(smem_u32(&acc_empty[0]), 0);
-        if (nphases == 0) {
-            for (int c0 = 0; c0 < BN; c0 += 4) *reinterpret_cast<float4 *>(dst + c0) = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (nphases == 0 && rows) {
+            for (int c0 = c_first; c0 < width; c0 += 4) *reinterpret_cast<float4 *>(dst + c0) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         for (int ph = 0; ph < nphases; ++ph) {
             const int buf = ph & 1;
-            if (!mbar_wait(&acc_full[buf], (uint32_t)((ph >> 1) & 1), abort_flag, status, 3)) break;
+            if (!mbar_wait(&acc_full[buf], (uint32_t)((ph >> 1) & 1), abort_flag, a.status, 3)) break;
             tc_fence_after();
+            if (ph == nphases - 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            if (rows) {
 #pragma unroll 1
-            for (int c0 = 0; c0 < BN; c0 += 32) {
-                uint32_t r[32];
-                tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c0), r);
-                tmem_ld_wait();
+                for (int c0 = c_first; c0 < width; c0 += 32) {
+                    uint32_t r[32];
+                    tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c0), r);
+                    tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; e += 4) {
-                    float4 v = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
-                                           __uint_as_float(r[e + 3]));
-                    float4 *p = reinterpret_cast<float4 *>(dst + c0 + e);
-                    if (ph > 0) {
-                        const float4 o = *p;
-                        v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+                    for (int e = 0; e < 32; e += 4) {
+                        float4 v = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
+                                               __uint_as_float(r[e + 3]));
+                        float4 *p = reinterpret_cast<float4 *>(dst + c0 + e);
+                        if (ph > 0) {
+                            const float4 o = *p;
+                            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+                        }
+                        *p = v;
                     }
-                    *p = v;
                 }
             }
             tc_fence_before();
@@ -450,189 +282,274 @@ moment2_tc_pair_kernel(const __grid_constant__ CUtensorMap tmap, float *__restri
     }
 }
 
+// Sums of the partial tiles over the sample ranges, i <= j < d only.  `wps` warps share 32 V columns of a row: the first
+// adds ranges 0, wps, 2 wps, ... with its loads in flight, and so on, then their sums are added in order.  V = 4 where
+// there are few ranges, so that a thread still has enough loads in flight.
+// PAIRS: X holds pair features (see moment4.cu) and row (i,j) of the result goes straight to the packed 4-simplex: its
+// unique entries are the columns from pair (j,j) = rowmap[row].x on, one run on both sides; rowmap[row].y + column is
+// the place of a column's entry.
+template <bool PAIRS, int V>
 __global__ void __launch_bounds__(256)
-moment2_tc_pair_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d,
-                              const __grid_constant__ m2tc2::TileTable tab)
+moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int npairs, int64_t out_elems,
+                         const int2 *__restrict__ rowmap, const __grid_constant__ m2tc::TileTable tab)
 {
-    using namespace m2tc2;
-    const int tile = blockIdx.x;
-    const int tm = tab.tm[tile], tn = tab.tn[tile], nsplit = tab.nsplit;
-    // partial of (tile, split, block r) lives in slot 2*(tile*nsplit+split)+r, a [128][256] array
-    for (int e = blockIdx.y * 256 + threadIdx.x; e < BM * BN; e += gridDim.y * 256) {
-        const int r = e / BN, c = e - r * BN;
+    using namespace m2tc;
+    __shared__ float part[2][8][32 * V];
+    const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tm = tab.tm[tile], tn = tab.tn[tile], width = 32 * tab.width[tile], uw = (width + 32 * V - 1) / (32 * V);
+    const int first = tab.first[tile], nsplit = tab.first[tile + 1] - first;
+    const int rows = d - tm * BM < BM ? d - tm * BM : BM;
+    const int wps = nsplit <= 8 ? 1 : nsplit <= 16 ? 2 : nsplit <= 32 ? 4 : 8;  // about eight loads per thread
+    const int per = 8 / wps, w0 = warp % wps;
+    const size_t stride = (size_t)2 * HALF * BN;
+    constexpr int BATCH = V == 1 ? 10 : 4;
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as a programmatic dependent of the main kernel
+    int buf = 0;
+    for (int u0 = blockIdx.y * per; u0 < rows * uw; u0 += gridDim.y * per) {
+        const int u = u0 + warp / wps, r = u / uw, c = (u - r * uw) * (32 * V) + V * lane;   // this thread's columns c .. c+V-1
         const int gi = tm * BM + r, gj = tn * BN + c;
-        if (gi < d && gj < d && gi <= gj) {
-            const float *base = partials + ((size_t)(2 * tile * nsplit + (r >> 7)) * HALF + (r & 127)) * BN + c;
-            const size_t stride = (size_t)2 * HALF * BN;
-            float s = 0.f;
-            for (int k0 = 0; k0 < nsplit; k0 += 8) {
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = (k0 + u < nsplit) ? __ldcg(base + (size_t)(k0 + u) * stride) : 0.f;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) s += v[u];
-            }
-            if (ST_BOUNDS_OK(tri_encode(d, gi, gj), tri_rows(d), 2)) out[tri_encode(d, gi, gj)] = s;
+        int lo = gi, hi = d;                               // columns of this row that are outputs
+        int64_t at;                                        // of column gj
+        if (PAIRS) {
+            const int2 m = gi < npairs ? rowmap[gi] : make_int2(1 << 30, 0);
+            lo = m.x;
+            hi = npairs;                                   // not the padding
+            at = m.y + gj;
+        } else {
+            at = tri_encode(d, gi, gj);
         }
+        const bool use = r < rows && c < width && gj + V > lo && gj < hi;
+        float s[V];
+#pragma unroll
+        for (int x = 0; x < V; ++x) s[x] = 0.f;
+        const float *base = partials + ((size_t)(2 * first + (r >> 7)) * HALF + (r & 127)) * BN + c;
+        for (int k0 = w0; k0 < nsplit; k0 += BATCH * wps) {
+            float v[BATCH][V];
+#pragma unroll
+            for (int e = 0; e < BATCH; ++e) {
+                const bool in = use && k0 + wps * e < nsplit;
+                const float *p = base + (size_t)(k0 + wps * e) * stride;
+                if (V == 4) {
+                    const float4 q = in ? __ldcg(reinterpret_cast<const float4 *>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[e][0] = q.x; v[e][V > 1 ? 1 : 0] = q.y; v[e][V > 2 ? 2 : 0] = q.z; v[e][V > 3 ? 3 : 0] = q.w;
+                } else {
+                    v[e][0] = in ? __ldcg(p) : 0.f;
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < BATCH; ++e)
+#pragma unroll
+                for (int x = 0; x < V; ++x) s[x] += v[e][x];
+        }
+        if (wps > 1) {
+#pragma unroll
+            for (int x = 0; x < V; ++x) part[buf][warp][32 * x + lane] = s[x];
+            __syncthreads();
+        }
+        if (w0 == 0 && use) {
+#pragma unroll
+            for (int x = 0; x < V; ++x) {
+                for (int w = 1; w < wps; ++w) s[x] += part[buf][warp + w][32 * x + lane];
+                if (gj + x >= lo && gj + x < hi && ST_BOUNDS_OK(at + x, out_elems, PAIRS ? 7 : 2)) out[at + x] = s[x];
+            }
+        }
+        buf ^= 1;
     }
 }
 
-struct M2Tc2Plan {
-    m2tc2::TileTable tab;
-    int chunks_total;
-    size_t partial_bytes;
+struct M2TcPlan {
+    m2tc::TileTable tab;
+    int chunks_total, stages, nb, na;
+    size_t partial_bytes, smem;
     bool ok;
 };
 
-static M2Tc2Plan m2tc2_plan(int64_t N, int64_t d, unsigned flags, bool tf32 = false, int segments = 1)
+template <int MODE>
+static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
 {
-    using namespace m2tc2;
-    const int KROWS = tf32 ? Shape<true>::KROWS : Shape<false>::KROWS;
-    M2Tc2Plan p;
+    using namespace m2tc;
+    using S = Shape<MODE>;
+    M2TcPlan p;
     p.ok = false;
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
     const int nt = (int)((d + BM - 1) / BM);
     int n = 0;
+    double cost[MAX_TILES];
+    p.nb = p.na = 0;
     for (int tn = 0; tn < nt; ++tn)
         for (int tm = 0; tm < nt; ++tm) {
             if (tm > tn && !dense) continue;
             if (n >= MAX_TILES) return p;
+            const int left = (int)d - tn * BN, width = left >= BN ? BN : (left + 31) / 32 * 32;
             p.tab.tm[n] = (unsigned char)tm;
             p.tab.tn[n] = (unsigned char)tn;
+            p.tab.width[n] = (unsigned char)(width / 32);
+            // time per stage, a full tile = 1: the 256 columns of A are loaded whatever the width (the MMA alone would be
+            // 43 cycles at 64 columns against 128; with 0.35 in place of 0.7 [400000,304] bf16 ran 127 us instead of 111)
+            cost[n] = 0.7 + 0.3 * width / BN;
+            const int nb = (width / 2 + S::BOXC - 1) / S::BOXC;
+            if (nb > p.nb) p.nb = nb;
+            if (!(tm == tn && width == BN)) {
+                const int la = (int)d - tm * BM, na = la >= HALF ? S::NBOX : (la + S::BOXC - 1) / S::BOXC;
+                if (na > p.na) p.na = na;
+            }
             ++n;
         }
-    for (int i = n; i < MAX_TILES; ++i) p.tab.tm[i] = p.tab.tn[i] = 0;
+    for (int i = n; i < MAX_TILES; ++i) p.tab.tm[i] = p.tab.tn[i] = p.tab.width[i] = 0;
     p.tab.ntiles = n;
-    const int64_t chunks = segments * ((N + KROWS - 1) / KROWS);
+    const int64_t chunks = (N + S::KROWS - 1) / S::KROWS;
     if (chunks > (int64_t(1) << 30)) return p;
     p.chunks_total = (int)chunks;
-    int64_t per = (sm_count_or_default() / 2) / n;   // clusters per tile: equal, so that sample ranges run in step
-    if (per < 1) per = 1;
-    if (per > chunks) per = chunks;
-    p.tab.nsplit = (int)per;
-    p.partial_bytes = (size_t)2 * n * per * HALF * BN * sizeof(float);
-    p.ok = true;
-    return p;
-}
-
-static bool m2_use_pair(int64_t d) { return d >= 512; }
-
-struct M2TcPlan {
-    m2tc::TileTable tab;
-    int chunks_total;
-    size_t partial_bytes;
-    bool ok;
-};
-
-static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
-{
-    using namespace m2tc;
-    M2TcPlan p;
-    p.ok = false;
-    const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
-    const int ntm = (int)((d + BM - 1) / BM), ntn = (int)((d + BN - 1) / BN);
-    int n = 0;
-    for (int tn = 0; tn < ntn; ++tn)
-        for (int tm = 0; tm < ntm; ++tm) {
-            const bool touches_upper = (int64_t)tm * BM <= (int64_t)tn * BN + BN - 1;
-            if (!touches_upper && !dense) continue;
-            if (n >= MAX_TILES) return p;
-            p.tab.tm[n] = (unsigned short)tm;
-            p.tab.tn[n] = (unsigned short)tn;
-            // rows 128*tm.. against columns 256*tn..256*tn+127: all below the diagonal when tm == 2*tn+1
-            const bool half = !dense && tm == 2 * tn + 1;
-            p.tab.half[n] = half ? 1 : 0;
-            ++n;
-        }
-    p.tab.ntiles = n;
-    for (int i = n; i < MAX_TILES; ++i) {
-        p.tab.tm[i] = p.tab.tn[i] = p.tab.nsplit[i] = p.tab.first_block[i] = 0;
-        p.tab.half[i] = 0;
+    const size_t stage = (size_t)S::PARTS * (p.nb + p.na) * S::BOX_BYTES;
+    p.stages = (int)((n == 1 ? STAGES_BYTES_1 : STAGES_BYTES) / stage);
+    if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
+    p.smem = (size_t)p.stages * stage + (size_t)(S::NBOX - p.na) * S::BOX_BYTES + 1024 + 512;
+    // Clusters (one per pair of SMs) are dealt one by one to the tile whose share of the samples takes longest; then every
+    // tile gives back what it does not need to keep up with the slowest.  Tiles of equal width so get equal shares: their
+    // clusters run in step and share X in L2 (with unequal shares the wide case was 12-20% slower on more SMs).
+    int split[MAX_TILES];
+    int64_t left = sm_count_or_default() / 2 - n;
+    for (int i = 0; i < n; ++i) split[i] = 1;
+    double longest = 0;
+    for (;;) {
+        int worst = 0;
+        for (int i = 1; i < n; ++i)
+            if (cost[i] / split[i] > cost[worst] / split[worst]) worst = i;
+        longest = cost[worst] / split[worst];
+        if (left <= 0 || split[worst] >= chunks) break;
+        ++split[worst];
+        --left;
     }
-    const int64_t chunks = (N + KROWS - 1) / KROWS;
-    if (chunks > (int64_t(1) << 30)) return p;
-    p.chunks_total = (int)chunks;
-    // splits: the same number for every tile.  Blocks that work on the same sample range then run
-    // in step and share the rows of X through L2 (X is read from HBM once); unequal splits were
-    // measured 12-20% slower although they use more SMs.
-    const int sms = sm_count_or_default();
-    int64_t per = sms / n;
-    if (per < 1) per = 1;
-    if (per > chunks) per = chunks;
-    for (int i = 0; i < n; ++i) p.tab.nsplit[i] = (unsigned short)per;
-    const int blocks = (int)per * n;
-    if (blocks > MAX_BLOCKS) return p;
-    int b = 0;
+    int first = 0;
     for (int i = 0; i < n; ++i) {
-        p.tab.first_block[i] = (unsigned short)b;
-        for (int s = 0; s < p.tab.nsplit[i]; ++s) p.tab.blk_tile[b++] = (unsigned short)i;
+        while (split[i] > 1 && cost[i] / (split[i] - 1) <= longest * (1 + 1e-9)) --split[i];
+        p.tab.first[i] = (unsigned short)first;
+        first += split[i];
     }
-    for (int i = b; i < MAX_BLOCKS; ++i) p.tab.blk_tile[i] = 0;
-    p.tab.nblocks = b;
-    p.partial_bytes = (size_t)b * BM * BN * sizeof(float);
+    for (int i = n; i <= MAX_TILES; ++i) p.tab.first[i] = (unsigned short)first;
+    p.partial_bytes = (size_t)2 * first * HALF * BN * sizeof(float);
     p.ok = true;
     return p;
 }
 
-// Launches the pair kernel and the sum of its partial tiles.
-template <bool TF32>
-static st_status m2_pair_launch(const M2Tc2Plan &q, const void *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws,
-                                cudaStream_t stream, size_t part_off = kWsHeaderBytes, int seg_chunks = 0, int lo_row0 = 0)
+// Launches the tile kernel and the sum of its partial tiles.  rows: rows of X in memory; npairs > 0: X holds pair
+// features and the result goes to the packed 4-simplex of `simplex` entries.
+template <int MODE>
+static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int64_t d, int64_t ldx, float *out, float *partials,
+                             unsigned *status, cudaStream_t stream, int lo_row0 = 0, int npairs = 0,
+                             const int2 *rowmap = nullptr, int64_t simplex = 0)
 {
-    using S = m2tc2::Shape<TF32>;
-    CUtensorMap tm2;
-    if (!tc::make_tmap_2d(&tm2, TF32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, X, (uint64_t)N,
+    using S = m2tc::Shape<MODE>;
+    CUtensorMap tmap;
+    if (!tc::make_tmap_2d(&tmap, MODE == M2_TF32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, X, (uint64_t)rows,
                           (uint64_t)d, (uint64_t)ldx * S::ELEM, S::BOXC, S::KROWS,
-                          TF32 ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B))
+                          MODE == M2_TF32 ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B))
         return ST_ERR_CUDA;
-    float *part2 = (float *)((unsigned char *)ws + part_off);
-    if (!ensure_dynamic_smem(moment2_tc_pair_kernel<TF32>, m2tc2::SMEM_BYTES)) return ST_ERR_CUDA;
+    m2tc::Args a;
+    a.partials = partials; a.status = status; a.d = (int)d;
+    a.chunks_total = q.chunks_total; a.stages = q.stages; a.nb = q.nb; a.na = q.na; a.lo_row0 = lo_row0;
+    a.tab = q.tab;
+    if (!ensure_dynamic_smem(moment2_tc_kernel<MODE>, q.smem)) return ST_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * q.tab.ntiles * q.tab.nsplit);
-    cfg.blockDim = dim3(m2tc2::THREADS);
-    cfg.dynamicSmemBytes = m2tc2::SMEM_BYTES;
+    cfg.gridDim = dim3(2 * (unsigned)q.tab.first[q.tab.ntiles]);
+    cfg.blockDim = dim3(m2tc::THREADS);
+    cfg.dynamicSmemBytes = q.smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // behind the pass that writes a split operand or pair features
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, moment2_tc_pair_kernel<TF32>, tm2, part2, (unsigned *)ws, q.chunks_total, q.tab, seg_chunks,
-                           lo_row0) != cudaSuccess) {
+    cfg.numAttrs = (MODE == M2_SPLIT || npairs > 0) ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, moment2_tc_kernel<MODE>, tmap, a) != cudaSuccess) {
         (void)cudaGetLastError();
         return ST_ERR_CUDA;
     }
-    moment2_tc_pair_reduce_kernel<<<dim3(q.tab.ntiles, 64), 256, 0, stream>>>(part2, out, (int)d, q.tab);
-    return launch_status();
+    int most = 0;                                                         // sample ranges of a tile
+    for (int t = 0; t < q.tab.ntiles; ++t) most = q.tab.first[t + 1] - q.tab.first[t] > most ? q.tab.first[t + 1] - q.tab.first[t] : most;
+    const unsigned blocks = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
+    cudaLaunchConfig_t rcfg = {};
+    rcfg.gridDim = dim3((unsigned)q.tab.ntiles, blocks < 64 ? 64 : blocks > 1024 ? 1024 : blocks);
+    rcfg.blockDim = dim3(256);
+    rcfg.stream = stream;
+    rcfg.attrs = attr + 1;
+    rcfg.numAttrs = 1;
+    auto reduce = [&](auto kernel) {
+        const float *cpart = partials;
+        if (cudaLaunchKernelEx(&rcfg, kernel, cpart, out, (int)d, npairs, npairs > 0 ? simplex : tri_rows(d), rowmap, q.tab) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return ST_ERR_CUDA;
+        }
+        return ST_OK;
+    };
+    if (most <= 4) return npairs > 0 ? reduce(moment2_tc_reduce_kernel<true, 4>) : reduce(moment2_tc_reduce_kernel<false, 4>);
+    return npairs > 0 ? reduce(moment2_tc_reduce_kernel<true, 1>) : reduce(moment2_tc_reduce_kernel<false, 1>);
 }
 
-// fp32 input read as TF32 by the pair kernel (any d that is a multiple of 4: tiles beyond d are zero-filled by the copies)
+// Room for the partial tiles of the structured call and of its dense control: one workspace serves both.
+template <int MODE>
+static size_t m2tc_partial_room(int64_t N, int64_t d, size_t bytes)
+{
+    for (unsigned f : {0u, ST_FLAG_DENSE_CONTROL}) {
+        const M2TcPlan q = m2tc_plan<MODE>(N, d, f);
+        if (q.ok && q.partial_bytes > bytes) bytes = q.partial_bytes;
+    }
+    return bytes;
+}
+
+template <int MODE>
+static size_t m2tc_workspace(int64_t N, int64_t d, unsigned flags)
+{
+    if (N <= 0 || d <= 0 || d > 4096 || N > (int64_t(1) << 31) - 64) return 0;
+    const M2TcPlan q = m2tc_plan<MODE>(N, d, flags);
+    return q.ok ? kWsHeaderBytes + m2tc_partial_room<MODE>(N, d, q.partial_bytes) : 0;
+}
+
+template <int MODE>
+static st_status m2tc_run(const void *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes, unsigned flags,
+                          cudaStream_t stream)
+{
+    if (d > 4096 || N > (int64_t(1) << 31) - 64) return ST_ERR_UNSUPPORTED;
+    const M2TcPlan q = m2tc_plan<MODE>(N, d, flags);
+    if (!q.ok) return ST_ERR_UNSUPPORTED;
+    if (!ws || ws_bytes < kWsHeaderBytes + q.partial_bytes) return ST_ERR_WORKSPACE;
+    if (!aligned256(ws)) return ST_ERR_ALIGN;
+    return m2tc_launch<MODE>(q, X, N, d, ldx, out, (float *)((unsigned char *)ws + kWsHeaderBytes), (unsigned *)ws, stream);
+}
+
+// fp32 input read as TF32 (any d that is a multiple of 4: tiles beyond d are zero-filled by the copies)
 size_t moment2_tf32_tc_workspace(int64_t N, int64_t d, unsigned flags)
 {
-    if (N <= 0 || d <= 0 || d % 4 != 0 || d > 4096 || N > (int64_t(1) << 31) - 64) return 0;
-    const M2Tc2Plan q = m2tc2_plan(N, d, flags, true);
-    return q.ok ? kWsHeaderBytes + q.partial_bytes : 0;
+    return d % 4 != 0 ? 0 : m2tc_workspace<M2_TF32>(N, d, flags);
 }
 
 st_status moment2_tf32_tc(const void *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
                           unsigned flags, cudaStream_t stream)
 {
     if (d % 4 != 0 || ldx % 4 != 0) return ST_ERR_ALIGN;
-    if (d > 4096 || N > (int64_t(1) << 31) - 64) return ST_ERR_UNSUPPORTED;
-    const M2Tc2Plan q = m2tc2_plan(N, d, flags, true);
-    if (!q.ok) return ST_ERR_UNSUPPORTED;
-    if (!ws || ws_bytes < kWsHeaderBytes + q.partial_bytes) return ST_ERR_WORKSPACE;
-    if (!aligned256(ws)) return ST_ERR_ALIGN;
-    return m2_pair_launch<true>(q, X, N, d, ldx, out, ws, stream);
+    return m2tc_run<M2_TF32>(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
+}
+
+size_t moment2_bf16_tc_workspace(int64_t N, int64_t d, unsigned flags)
+{
+    return d % 8 != 0 ? 0 : m2tc_workspace<M2_BF16>(N, d, flags);
+}
+
+st_status moment2_bf16_tc(const void *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
+                          unsigned flags, cudaStream_t stream)
+{
+    if (d % 8 != 0 || ldx % 8 != 0) return ST_ERR_ALIGN;
+    return m2tc_run<M2_BF16>(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
 }
 
 // ---------------------------------------------------------------------------------------------
 // fp32 input at the fp32 tolerance on the tensor cores (ST_FLAG_TC_SPLIT): every x is written once as
 // hi = bf16(x) and lo = bf16(x - hi) (x - hi - lo is below 2^-16 |x|), and the pair kernel adds
-// hi^T hi + hi^T lo + lo^T hi over three passes of the samples (lo^T lo is below 2^-16 of the result).
-// The split pass reads X once and writes the same number of bytes; the three passes then run at the bf16 rate.
+// hi^T hi + hi^T lo + lo^T hi from one stage of both parts (lo^T lo is below 2^-16 of the result).
+// The split pass reads X once and writes the same number of bytes: HBM bound.
 __global__ void __launch_bounds__(256)
 moment2_split_rows_kernel(const float *__restrict__ X, int64_t N, int64_t Np, int d, int64_t ldx, __nv_bfloat16 *__restrict__ Z)
 {
@@ -651,10 +568,11 @@ moment2_split_rows_kernel(const float *__restrict__ X, int64_t N, int64_t Np, in
         *reinterpret_cast<uint2 *>(Z + (Np + n) * d + c) =
             make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
     }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tile kernel may be launched; it waits for this grid to end
 }
 
 struct M2SplitPlan {
-    M2Tc2Plan q;
+    M2TcPlan q;
     int64_t Np;
     size_t z_off, part_off, total;
     bool ok;
@@ -665,9 +583,8 @@ static M2SplitPlan m2_split_plan(int64_t N, int64_t d, unsigned flags)
     M2SplitPlan p{};
     p.ok = false;
     if (N <= 0 || d <= 0 || d % 8 != 0 || d > 4096 || N > (int64_t(1) << 29)) return p;
-    const int KROWS = m2tc2::Shape<false>::KROWS;
-    p.Np = (N + KROWS - 1) / KROWS * KROWS;
-    p.q = m2tc2_plan(N, d, flags, false, 3);
+    p.Np = (N + 63) / 64 * 64;
+    p.q = m2tc_plan<M2_SPLIT>(N, d, flags);
     if (!p.q.ok) return p;
     p.z_off = kWsHeaderBytes;
     p.part_off = round_up(p.z_off + (size_t)2 * p.Np * d * sizeof(__nv_bfloat16), 256);
@@ -676,30 +593,10 @@ static M2SplitPlan m2_split_plan(int64_t N, int64_t d, unsigned flags)
     return p;
 }
 
-// The three-segment product for a caller that has written the parts itself (the fourth moment makes its pair
-// features straight into this form): Z = [hi rows; lo rows], each part N rounded up to 64 rows with zero rows
-// at the end, d columns, bf16.
-int64_t moment2_split_part_rows(int64_t N) { return (N + 63) / 64 * 64; }
-
-size_t moment2_split_parts_workspace(int64_t N, int64_t d)
-{
-    const M2SplitPlan p = m2_split_plan(N, d, 0);
-    return p.ok ? kWsHeaderBytes + p.q.partial_bytes : 0;
-}
-
-st_status moment2_split_tc_parts(const void *Z, int64_t N, int64_t d, float *out, void *ws, size_t ws_bytes, cudaStream_t stream)
-{
-    const M2SplitPlan p = m2_split_plan(N, d, 0);
-    if (!p.ok) return ST_ERR_UNSUPPORTED;
-    if (!ws || ws_bytes < kWsHeaderBytes + p.q.partial_bytes) return ST_ERR_WORKSPACE;
-    if (!aligned256(ws) || !aligned16(Z)) return ST_ERR_ALIGN;
-    return m2_pair_launch<false>(p.q, Z, 2 * p.Np, d, d, out, ws, stream, kWsHeaderBytes, p.q.chunks_total / 3, (int)p.Np);
-}
-
 size_t moment2_split_tc_workspace(int64_t N, int64_t d, unsigned flags)
 {
     const M2SplitPlan p = m2_split_plan(N, d, flags);
-    return p.ok ? p.total : 0;
+    return p.ok ? p.part_off + m2tc_partial_room<M2_SPLIT>(N, d, p.q.partial_bytes) : 0;
 }
 
 st_status moment2_split_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
@@ -716,49 +613,29 @@ st_status moment2_split_tc(const float *X, int64_t N, int64_t d, int64_t ldx, fl
     const int64_t cap = (int64_t)sm_count_or_default() * 16;
     moment2_split_rows_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, stream>>>(X, N, p.Np, (int)d, ldx, Z);
     if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
-    return m2_pair_launch<false>(p.q, Z, 2 * p.Np, d, d, out, ws, stream, p.part_off, p.q.chunks_total / 3, (int)p.Np);
+    return m2tc_launch<M2_SPLIT>(p.q, Z, 2 * p.Np, d, d, out, (float *)((unsigned char *)ws + p.part_off), (unsigned *)ws, stream, (int)p.Np);
 }
 
-size_t moment2_bf16_tc_workspace(int64_t N, int64_t d, unsigned flags)
+// The second moment of pair features that the caller has written, its unique 4-tuples straight into the packed
+// 4-simplex (see moment4.cu).  split: P = [hi rows; lo rows], each part N rounded up to 64 rows with zero rows at the
+// end; else N rows of bf16.  dP columns; rowmap as in moment2_tc_reduce_kernel.
+int64_t moment2_split_part_rows(int64_t N) { return (N + 63) / 64 * 64; }
+
+size_t moment2_pairs_partial_bytes(int64_t N, int64_t dP, bool split)
 {
-    if (N <= 0 || d <= 0 || d % 8 != 0 || d > 4096 || N > (int64_t(1) << 31) - 64) return 0;
-    if (m2_use_pair(d)) {
-        const M2Tc2Plan q = m2tc2_plan(N, d, flags);
-        return q.ok ? kWsHeaderBytes + q.partial_bytes : 0;
-    }
-    const M2TcPlan p = m2tc_plan(N, d, flags);
-    return p.ok ? kWsHeaderBytes + p.partial_bytes : 0;
+    if (N <= 0 || dP <= 0 || dP > 4096 || N > (int64_t(1) << 29)) return 0;
+    const M2TcPlan q = split ? m2tc_plan<M2_SPLIT>(N, dP, 0) : m2tc_plan<M2_BF16>(N, dP, 0);
+    return q.ok ? q.partial_bytes : 0;
 }
 
-st_status moment2_bf16_tc(const void *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
-                          unsigned flags, cudaStream_t stream)
+st_status moment2_pairs_tc(const void *P, int64_t N, int64_t dP, int npairs, bool split, const int2 *rowmap, int64_t simplex, float *out,
+                           float *partials, unsigned *status, cudaStream_t stream)
 {
-    using namespace m2tc;
-    if (d % 8 != 0 || ldx % 8 != 0) return ST_ERR_ALIGN;
-    if (d > 4096 || N > (int64_t(1) << 31) - 64) return ST_ERR_UNSUPPORTED;
-    if (m2_use_pair(d)) {
-        const M2Tc2Plan q = m2tc2_plan(N, d, flags);
-        if (!q.ok) return ST_ERR_UNSUPPORTED;
-        if (!ws || ws_bytes < kWsHeaderBytes + q.partial_bytes) return ST_ERR_WORKSPACE;
-        if (!aligned256(ws)) return ST_ERR_ALIGN;
-        return m2_pair_launch<false>(q, X, N, d, ldx, out, ws, stream);
+    if (split) {
+        const int64_t Np = moment2_split_part_rows(N);
+        return m2tc_launch<M2_SPLIT>(m2tc_plan<M2_SPLIT>(N, dP, 0), P, 2 * Np, dP, dP, out, partials, status, stream, (int)Np, npairs, rowmap, simplex);
     }
-    const M2TcPlan p = m2tc_plan(N, d, flags);
-    if (!p.ok) return ST_ERR_UNSUPPORTED;
-    const size_t need = kWsHeaderBytes + p.partial_bytes;
-    if (!ws || ws_bytes < need) return ST_ERR_WORKSPACE;
-    if (!aligned256(ws)) return ST_ERR_ALIGN;
-    CUtensorMap tmap;
-    if (!tc::make_tmap_2d(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, X, (uint64_t)N, (uint64_t)d, (uint64_t)ldx * 2,
-                          BOXC, KROWS))
-        return ST_ERR_CUDA;
-    float *partials = (float *)((unsigned char *)ws + kWsHeaderBytes);
-    if (!ensure_dynamic_smem(moment2_tc_kernel, SMEM_BYTES)) return ST_ERR_CUDA;
-    moment2_tc_kernel<<<p.tab.nblocks, THREADS, SMEM_BYTES, stream>>>(tmap, partials, (unsigned *)ws, p.chunks_total,
-                                                                      p.tab);
-    if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
-    moment2_tc_reduce_kernel<<<dim3(p.tab.ntiles, 32), 256, 0, stream>>>(partials, out, (int)d, p.tab);
-    return launch_status();
+    return m2tc_launch<M2_BF16>(m2tc_plan<M2_BF16>(N, dP, 0), P, N, dP, dP, out, partials, status, stream, 0, npairs, rowmap, simplex);
 }
 
 }  // namespace st

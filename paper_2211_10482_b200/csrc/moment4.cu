@@ -11,8 +11,9 @@
 //                            to bf16 (ST_FLAG_TC_BF16, 5e-3) or, for the fp32 tolerance, on P written as hi + lo
 //                            bf16 parts and multiplied in three partial products (d <= 89: the pair features
 //                            fit the kernel's 4096 columns); beyond that the fp32 FMA kernel on an fp32 P
-//   3. simplex_gather_kernel all entries (i,j,*,*) of the 4-simplex are one run of row (i,j) of that triangle,
-//                            from column (j,j) on: contiguous on both sides
+//   3. all entries (i,j,*,*) of the 4-simplex are one run of row (i,j) of that triangle, from column (j,j) on,
+//      contiguous on both sides: the sum over the partial tiles of step 2 writes them there (tensor-core paths);
+//      simplex_gather_kernel copies them from the packed triangle (fp32 FMA path)
 // Step 2 works on the symmetric pair-by-pair matrix, whose unique set (pairs p <= q) is about
 // three times larger than the set of unique 4-tuples: the entries with j > k are computed and
 // not gathered.
@@ -25,8 +26,9 @@ namespace st {
 
 size_t moment2_workspace(int64_t N, int64_t d, int xdt, unsigned flags);
 int64_t moment2_split_part_rows(int64_t N);
-size_t moment2_split_parts_workspace(int64_t N, int64_t d);
-st_status moment2_split_tc_parts(const void *Z, int64_t N, int64_t d, float *out, void *ws, size_t ws_bytes, cudaStream_t stream);
+size_t moment2_pairs_partial_bytes(int64_t N, int64_t dP, bool split);
+st_status moment2_pairs_tc(const void *P, int64_t N, int64_t dP, int npairs, bool split, const int2 *rowmap, int64_t simplex, float *out,
+                           float *partials, unsigned *status, cudaStream_t stream);
 
 namespace m4 {
 
@@ -35,8 +37,8 @@ constexpr int EXP_ROWS = 32;        // sample rows per pass of a block
 constexpr int EXP_THREADS = 192;
 
 struct Plan {
-    int64_t dP, p_bytes, m2_elems, m2_ws, Np;
-    size_t off_p, off_m2, off_ws, total;
+    int64_t dP, p_bytes, Np;
+    size_t off_p, off_m2, off_ws, m2_ws, total;     // off_m2: packed triangle (fp32 path) or row map; off_ws: workspace or partial tiles of step 2
     bool bf16, split, ok;
 };
 
@@ -47,23 +49,19 @@ static Plan plan(int64_t N, int64_t d, unsigned flags)
     if (N <= 0 || d < 1 || d > MAX_D) return p;
     p.bf16 = (flags & ST_FLAG_TC_BF16) != 0;
     p.dP = (tri_rows(d) + 63) / 64 * 64;
-    p.m2_elems = tri_rows(p.dP);
     // fp32 result: the pair features are written as hi + lo bf16 parts and multiplied on the tensor cores in three
     // partial products (the fp32 tolerance) wherever that kernel reaches; else fp32 features and the fp32 FMA kernel
     p.Np = moment2_split_part_rows(N);
-    p.m2_ws = p.bf16 ? 0 : (int64_t)moment2_split_parts_workspace(N, p.dP);
+    p.m2_ws = moment2_pairs_partial_bytes(N, p.dP, !p.bf16);
     p.split = !p.bf16 && p.m2_ws != 0;
-    if (p.split) {
-        p.p_bytes = 2 * p.Np * p.dP * 2;
-    } else {
-        p.p_bytes = N * p.dP * (p.bf16 ? 2 : 4);
-        p.m2_ws = (int64_t)moment2_workspace(N, p.dP, p.bf16 ? ST_BF16 : ST_F32, 0);
-    }
+    const bool fma = !p.bf16 && !p.split;
+    if (fma) p.m2_ws = moment2_workspace(N, p.dP, ST_F32, 0);
     if (p.m2_ws == 0) return p;
+    p.p_bytes = p.split ? 2 * p.Np * p.dP * 2 : N * p.dP * (p.bf16 ? 2 : 4);
     p.off_p = kWsHeaderBytes;
     p.off_m2 = round_up(p.off_p + (size_t)p.p_bytes, 256);
-    p.off_ws = round_up(p.off_m2 + (size_t)p.m2_elems * 4, 256);
-    p.total = p.off_ws + (size_t)p.m2_ws;
+    p.off_ws = round_up(p.off_m2 + (fma ? (size_t)tri_rows(p.dP) * sizeof(float) : (size_t)tri_rows(d) * sizeof(int2)), 256);
+    p.total = p.off_ws + p.m2_ws;
     p.ok = true;
     return p;
 }
@@ -84,11 +82,12 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *dst, float a, float b, flo
 // row with one 8- or 16-byte store.  HBM bound: the write of P.
 // SPLIT: every product p is written twice, hi = bf16(p) in row n and lo = bf16(p - hi) in row Np + n; the rows
 // N .. Np-1 of either part are zero.
+// rowmap (tensor-core paths): where the unique entries of row p of P^T P start and go to, see moment2_tc_reduce_kernel.
 // COLS: columns of a staged row per lane, (d + 1 + 31) / 32 rounded up to an instance (2, 3 or 5).
 template <typename OutT, bool SPLIT, int COLS>
 __global__ void __launch_bounds__(EXP_THREADS)
 pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, OutT *__restrict__ P, int dP, int npairs,
-                   int64_t Np)
+                   int64_t Np, int2 *__restrict__ rowmap)
 {
     extern __shared__ __align__(16) float xs[];                       // 2 x [EXP_ROWS][d + 1], column d is zero
     const int pitch = d + 1;
@@ -103,6 +102,10 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
             tri_decode(d, p + u, a, b);
             ci[u] = (int)a;
             cj[u] = (int)b;
+            if (rowmap && blockIdx.y == 0) {
+                const int64_t q0 = tri_encode(d, b, b);
+                rowmap[p + u] = make_int2((int)q0, (int)(simp4_encode(d, a, b, b, b) - q0));
+            }
         }
     }
     const bool inside = p < dP;
@@ -160,6 +163,7 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
             }
         }
     }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tile kernel may be launched; it waits for this grid to end
 }
 
 // One block per unique pair (i,j): the entries (i,j,k,l), j <= k <= l, follow each other in the 4-simplex in the
@@ -213,31 +217,33 @@ extern "C" st_status st_sym_moment4(const float *X, int64_t N, int64_t d, int64_
     if (!aligned256(ws)) return ST_ERR_ALIGN;
     cudaStream_t stream = (cudaStream_t)stream_;
     unsigned char *w = (unsigned char *)ws;
-    float *M2 = (float *)(w + p.off_m2);
     const int npairs = (int)tri_rows(d);
     const size_t smem = (size_t)2 * EXP_ROWS * (d + 1) * sizeof(float);
     const unsigned col_groups = (unsigned)((p.dP + 4 * EXP_THREADS - 1) / (4 * EXP_THREADS));
     const int64_t passes = ((p.split ? p.Np : N) + EXP_ROWS - 1) / EXP_ROWS;
     const int64_t cap = ((int64_t)sm_count_or_default() * 8 + col_groups - 1) / col_groups;
     const dim3 grid(col_groups, (unsigned)(passes < cap ? passes : cap));
+    int2 *rowmap = (p.split || p.bf16) ? (int2 *)(w + p.off_m2) : nullptr;
     auto expand = [&](auto tag, auto split_tag) {
         using T = decltype(tag);
         constexpr bool SP = decltype(split_tag)::value;
         T *dst = (T *)(w + p.off_p);
         if (d + 1 <= 64)
-            pair_expand_kernel<T, SP, 2><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np);
+            pair_expand_kernel<T, SP, 2><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
         else if (d + 1 <= 96)
-            pair_expand_kernel<T, SP, 3><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np);
+            pair_expand_kernel<T, SP, 3><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
         else
-            pair_expand_kernel<T, SP, 5><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np);
+            pair_expand_kernel<T, SP, 5><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
     };
     if (p.split) expand(__nv_bfloat16(), std::true_type());
     else if (p.bf16) expand(__nv_bfloat16(), std::false_type());
     else expand(float(), std::false_type());
     if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
-    const st_status rc = p.split ? moment2_split_tc_parts(w + p.off_p, N, p.dP, M2, w + p.off_ws, (size_t)p.m2_ws, stream)
-                                 : st_sym_moment2(w + p.off_p, p.bf16 ? ST_BF16 : ST_F32, N, p.dP, p.dP, M2, w + p.off_ws,
-                                                  (size_t)p.m2_ws, 0, stream_);
+    if (p.split || p.bf16)
+        return moment2_pairs_tc(w + p.off_p, N, p.dP, npairs, p.split, rowmap, simp4_rows(d), out_packed, (float *)(w + p.off_ws), (unsigned *)w,
+                                stream);
+    float *M2 = (float *)(w + p.off_m2);
+    const st_status rc = st_sym_moment2(w + p.off_p, ST_F32, N, p.dP, p.dP, M2, w + p.off_ws, p.m2_ws, 0, stream_);
     if (rc != ST_OK) return rc;
     simplex_gather_kernel<<<(unsigned)npairs, 128, 0, stream>>>(M2, out_packed, (int)d, p.dP, (unsigned *)w,
                                                                 (const unsigned *)(w + p.off_ws));

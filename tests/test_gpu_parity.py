@@ -784,6 +784,21 @@ def test_moment2_split_tensor_core_on_fp32_input(st, N, d):
     assert np.array_equal(expand2(st, out2, d), got)
 
 
+# tiles as wide as the columns left (32 .. 256 in steps of 32), operands of one to all boxes, more stages than chunks and
+# rings that wrap many times, chains cut several times in narrow tiles
+@pytest.mark.parametrize("N,d", [(1, 8), (70, 40), (9000, 24), (65537, 8), (40000, 72), (3000, 136), (20000, 160), (1500, 264),
+                                 (12000, 288), (700, 392), (5000, 488), (2100, 544)])
+def test_moment2_tensor_core_tile_widths(st, N, d):
+    X = workloads.draw((N, d), "normal", 40 + N + d)
+    bits = workloads.f32_to_bf16_bits(X)
+    Tb, Sb = oracle.moment2(workloads.bf16_bits_to_f32(bits))
+    assert oracle.rel_err(expand2(st, st.st_sym_moment2(bf16_dev(bits)), d), Tb, Sb) <= TOL_F32
+    T, S = oracle.moment2(X)
+    assert oracle.rel_err(expand2(st, st.st_sym_moment2(dev(X), flags=st.ST_FLAG_TC_SPLIT), d), T, S) <= TOL_F32
+    Tt, St = oracle.moment2((X.view(np.uint32) & np.uint32(0xFFFFE000)).view(np.float32))
+    assert oracle.rel_err(expand2(st, st.st_sym_moment2(dev(X), flags=st.ST_FLAG_TC_TF32), d), Tt, St) <= TOL_F32
+
+
 def test_moment2_split_sums_of_squares_do_not_drift(st):
     """All-positive sums over many samples: the accumulation chain is cut often enough that the diagonal stays
     inside the fp32 tolerance (a tensor-core accumulator rounds towards zero)."""
