@@ -20,7 +20,10 @@ constexpr int BM = 128;                    // fibres per tile
 constexpr int KC = 32;                     // floats per k-slice (128 bytes)
 constexpr int STAGE_BYTES = BM * KC * 4;   // 16 KiB
 constexpr int THREADS = 192;
-constexpr int MAX_STAGES = 10;
+// 96 KB of fibres in flight per SM: a copy loop without arithmetic reads 269 MB at 6.5 TB/s with six stages, 5.9 with ten and
+// 5.8 with thirteen (the memory system queues); this kernel 56.4 us with five or six ([64,64,64,256] x [256,64], 269 MB
+// read, 67 written), 57.2 with eight, 58.9 with ten, 58.8 with four.
+constexpr int MAX_STAGES = 6;
 }  // namespace ttmtc
 
 enum { TC_TTM = 0, TC_MTTKRP_PACKED = 1, TC_MTTKRP_DENSE = 2 };
