@@ -2,14 +2,15 @@
 
 Argument marshalling only: every function takes torch CUDA tensors, passes their raw device
 pointers, extents and the current CUDA stream to the C entry point of the same name, and
-raises ``StError`` when the call returns a non-zero status.  torch is used for device
-memory and streams only; there is no CPU or torch fallback -- if the shared library has not
+raises ``StError`` when the call returns a non-zero status.  The marshalling is native code
+(``csrc/binding.cpp``); ``lib()`` is the ctypes view of the same library.  torch is used for device
+memory and streams only; there is no CPU or torch fallback -- if the shared libraries have not
 been built the first call raises.
 """
 from __future__ import annotations
 
 import ctypes
-import functools
+import importlib
 import math
 import os
 from dataclasses import dataclass
@@ -123,19 +124,22 @@ def status_string(status: int) -> str:
     return lib().st_status_string(int(status)).decode()
 
 
-_DTYPES = {torch.float32: ST_F32, torch.bfloat16: ST_BF16, torch.float64: ST_F64}
+_native = None
 
 
-def _dtype(t: torch.Tensor) -> int:
-    if t.dtype in _DTYPES:
-        return _DTYPES[t.dtype]
-    if t.dtype in (torch.int32, torch.uint32):
-        return ST_F32    # pack/unpack are bit copies: any 4-byte type travels as ST_F32
-    if t.dtype in (torch.int16, torch.uint16, torch.float16):
-        return ST_BF16
-    if t.dtype == torch.int64:
-        return ST_F64
-    raise TypeError("unsupported dtype %s" % t.dtype)
+def _bind():
+    """The native binding, told the addresses of the library's entry points (raises if either has not been built)."""
+    global _native
+    L = lib()
+    try:
+        b = importlib.import_module("._binding", __name__)
+    except ModuleNotFoundError:
+        raise RuntimeError("_binding.so is missing: build it with `python -m paper_2211_10482_b200._build`") from None
+    b.bind({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in EXPORTS}, StError,
+           torch.float32, torch.uint8, _last_ws)
+    b.set_allocator(_allocator)
+    _native = b
+    return b
 
 
 def _dev(t: torch.Tensor, name: str) -> int:
@@ -146,15 +150,8 @@ def _dev(t: torch.Tensor, name: str) -> int:
     return t.data_ptr()
 
 
-# The launch path of a small call is host-bound (its kernels run a few microseconds), so what a call asks of
-# torch per launch is kept to the bare queries: the current stream's handle costs 3 us through
-# torch.cuda.current_stream() and 0.3 us this way.
-if hasattr(torch._C, "_cuda_getCurrentRawStream"):
-    def _stream() -> int:
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
-else:
-    def _stream() -> int:
-        return torch.cuda.current_stream().cuda_stream
+def _stream() -> int:
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _check(status: int, where: str) -> None:
@@ -162,26 +159,12 @@ def _check(status: int, where: str) -> None:
         raise StError(status, where)
 
 
-@functools.lru_cache(maxsize=256)
-def _layout_info(layout: Layout):
-    """(pointer to the C descriptor, packed elements, dense elements) of a layout, by its value."""
-    c = layout.c()
-    L = lib()
-    return ctypes.pointer(c), int(L.st_packed_elems(ctypes.byref(c))), int(L.st_dense_elems(ctypes.byref(c)))
-
-
-@functools.lru_cache(maxsize=1024)
-def _ws_bytes(device: int, op: int, a: int, b: int, c: int, e: int, flags: int) -> int:
-    """Workspace of a request on a device (its SM count decides), at least the 256-byte header."""
-    return max(st_workspace_bytes(op, a, b, c, e, flags), 256)
-
-
 def st_packed_elems(layout: Layout) -> int:
-    return _layout_info(layout)[1]
+    return int(lib().st_packed_elems(ctypes.byref(layout.c())))
 
 
 def st_dense_elems(layout: Layout) -> int:
-    return _layout_info(layout)[2]
+    return int(lib().st_dense_elems(ctypes.byref(layout.c())))
 
 
 def st_workspace_bytes(op: int, a: int, b: int, c: int = 0, e: int = 0, flags: int = 0) -> int:
@@ -199,6 +182,8 @@ def set_allocator(fn) -> None:
     surround every buffer with guard bands."""
     global _allocator
     _allocator = fn
+    if _native is not None:
+        _native.set_allocator(fn)
 
 
 def _alloc(shape, dtype, device) -> torch.Tensor:
@@ -210,84 +195,31 @@ def _alloc(shape, dtype, device) -> torch.Tensor:
     return _allocator(math.prod(shape), dtype, device).view(shape)
 
 
-def _workspace(ws: torch.Tensor | None, device, op: int, a: int, b: int, c: int, e: int, flags: int) -> torch.Tensor:
-    """The caller's workspace, or a fresh one of the size of the request.  Either way it is
-    remembered as the device's last workspace, so that st_check_status() can read the status word
-    that the call's kernels may have written."""
-    if ws is None:
-        ws = _alloc(_ws_bytes(torch.cuda.current_device(), op, a, b, c, e, flags), torch.uint8, device)
-    _last_ws[ws.device.index] = ws
-    return ws
-
-
 def st_pack(dense: torch.Tensor, layout: Layout, out: torch.Tensor | None = None) -> torch.Tensor:
-    desc, n, n_dense = _layout_info(layout)
-    if n < 0:
-        raise StError(ST_ERR_SHAPE, "st_packed_elems")
-    if dense.numel() != n_dense:
-        raise ValueError("dense has %d elements, layout needs %d" % (dense.numel(), n_dense))
-    if out is None:
-        out = _alloc(n, dense.dtype, dense.device)
-    _check(lib().st_pack(desc, _dtype(dense), _dev(dense, "dense"), _dev(out, "out"),
-                         _stream()), "st_pack")
-    return out
+    return (_native or _bind()).pack(dense, layout, out)
 
 
 def st_unpack(packed: torch.Tensor, layout: Layout, fill: int = ST_FILL_ZERO,
               out: torch.Tensor | None = None) -> torch.Tensor:
-    desc, n_packed, n = _layout_info(layout)
-    if n < 0:
-        raise StError(ST_ERR_SHAPE, "st_dense_elems")
-    if packed.numel() != n_packed:
-        raise ValueError("packed has %d elements, layout needs %d" % (packed.numel(), n_packed))
-    if out is None:
-        out = _alloc(n, packed.dtype, packed.device)
-    _check(lib().st_unpack(desc, _dtype(packed), _dev(packed, "packed"), _dev(out, "out"),
-                           int(fill), _stream()), "st_unpack")
-    return out
+    return (_native or _bind()).unpack(packed, layout, fill, out)
 
 
 def st_sym_moment2(X: torch.Tensor, out: torch.Tensor | None = None, ws: torch.Tensor | None = None,
                    flags: int = 0) -> torch.Tensor:
     """Packed upper triangle of X^T X; X is [N, d] float32 or bfloat16."""
-    N, d = X.shape
-    if X.dtype not in (torch.float32, torch.bfloat16):
-        raise TypeError("X must be float32 or bfloat16")
-    xdt = _DTYPES[X.dtype]
-    if out is None:
-        out = _alloc(d * (d + 1) // 2, torch.float32, X.device)
-    ws = _workspace(ws, X.device, ST_OP_SYM_MOMENT2, N, d, xdt, 0, flags)
-    _check(lib().st_sym_moment2(_dev(X, "X"), xdt, N, d, X.stride(0), _dev(out, "out"), ws.data_ptr(),
-                                ws.numel() * ws.element_size(), flags, _stream()), "st_sym_moment2")
-    return out
+    return (_native or _bind()).moment2(X, out, ws, flags)
 
 
 def st_sym_moment3(X: torch.Tensor, out: torch.Tensor | None = None, ws: torch.Tensor | None = None,
                    flags: int = 0) -> torch.Tensor:
     """Packed tetrahedron sum_n X[n,i] X[n,j] X[n,k], i<=j<=k; X is [N, d] float32."""
-    N, d = X.shape
-    if X.dtype != torch.float32:
-        raise TypeError("X must be float32")
-    if out is None:
-        out = _alloc(d * (d + 1) * (d + 2) // 6, torch.float32, X.device)
-    ws = _workspace(ws, X.device, ST_OP_SYM_MOMENT3, N, d, 0, 0, flags)
-    _check(lib().st_sym_moment3(_dev(X, "X"), N, d, X.stride(0), _dev(out, "out"), ws.data_ptr(),
-                                ws.numel() * ws.element_size(), flags, _stream()), "st_sym_moment3")
-    return out
+    return (_native or _bind()).moment3(X, out, ws, flags)
 
 
 def st_sym_moment4(X: torch.Tensor, out: torch.Tensor | None = None, ws: torch.Tensor | None = None,
                    flags: int = 0) -> torch.Tensor:
     """Packed 4-simplex sum_n X[n,i] X[n,j] X[n,k] X[n,l], i<=j<=k<=l; X is [N, d] float32."""
-    N, d = X.shape
-    if X.dtype != torch.float32:
-        raise TypeError("X must be float32")
-    if out is None:
-        out = _alloc(d * (d + 1) * (d + 2) * (d + 3) // 24, torch.float32, X.device)
-    ws = _workspace(ws, X.device, ST_OP_SYM_MOMENT4, N, d, 0, 0, flags)
-    _check(lib().st_sym_moment4(_dev(X, "X"), N, d, X.stride(0), _dev(out, "out"), ws.data_ptr(),
-                                ws.numel() * ws.element_size(), flags, _stream()), "st_sym_moment4")
-    return out
+    return (_native or _bind()).moment4(X, out, ws, flags)
 
 
 def st_sym_moment3_static(X: torch.Tensor, out: torch.Tensor, flags: int = 0) -> torch.Tensor:
@@ -308,114 +240,42 @@ def st_mttkrp_tri(Bp: torch.Tensor, C: torch.Tensor, D: torch.Tensor, out: torch
                   ws: torch.Tensor | None = None, flags: int = 0) -> torch.Tensor:
     """A[i,r] = sum_{j>=i,k} Bp[p(i,j),k] C[j,r] D[k,r]; Bp is [I(I+1)/2, K] (dense [I,I,K] with the
     dense-control flag)."""
-    I, R = C.shape
-    K = D.shape[0]
-    for t in (Bp, C, D):
-        if t.dtype != torch.float32:
-            raise TypeError("inputs must be float32")
-    want = I * I * K if (flags & ST_FLAG_DENSE_CONTROL) else I * (I + 1) // 2 * K
-    if Bp.numel() != want or D.shape[1] != R:
-        raise ValueError("shape mismatch")
-    if out is None:
-        out = _alloc((I, R), torch.float32, Bp.device)
-    ws = _workspace(ws, Bp.device, ST_OP_MTTKRP_TRI, I, K, R, 0, flags)
-    _check(lib().st_mttkrp_tri(_dev(Bp, "Bp"), I, K, _dev(C, "C"), _dev(D, "D"), R, _dev(out, "out"),
-                               ws.data_ptr(), ws.numel() * ws.element_size(), flags, _stream()),
-           "st_mttkrp_tri")
-    return out
+    return (_native or _bind()).mttkrp_tri(Bp, C, D, out, ws, flags)
 
 
 def st_mttkrp_slice(Bp: torch.Tensor, C: torch.Tensor, D: torch.Tensor, I: int, fixed_i: int = -1, fixed_j: int = -1,
                     out: torch.Tensor | None = None, ws: torch.Tensor | None = None, flags: int = 0) -> torch.Tensor:
     """MTTKRP on a tensor that is non-zero only where i == fixed_i and / or j == fixed_j; Bp is that slice."""
-    J, R = C.shape
-    K = D.shape[0]
-    for t in (Bp, C, D):
-        if t.dtype != torch.float32:
-            raise TypeError("inputs must be float32")
-    rows = (1 if fixed_j >= 0 else J) if fixed_i >= 0 else I
-    if Bp.numel() != rows * K or D.shape[1] != R:
-        raise ValueError("shape mismatch")
-    if out is None:
-        out = _alloc((I, R), torch.float32, Bp.device)
-    ws = _workspace(ws, Bp.device, ST_OP_MTTKRP_SLICE, I, J, K, R, flags)
-    _check(lib().st_mttkrp_slice(_dev(Bp, "Bp"), I, J, K, fixed_i, fixed_j, _dev(C, "C"), _dev(D, "D"), R,
-                                 _dev(out, "out"), ws.data_ptr(), ws.numel() * ws.element_size(), flags, _stream()),
-           "st_mttkrp_slice")
-    return out
+    return (_native or _bind()).mttkrp_slice(Bp, C, D, I, fixed_i, fixed_j, out, ws, flags)
 
 
 def st_ttm_blockdiag(Bp: torch.Tensor, U: torch.Tensor, nblocks: int, bs: int,
                      out: torch.Tensor | None = None, ws: torch.Tensor | None = None,
                      flags: int = 0) -> torch.Tensor:
     """Ap[b,i',j',r] = sum_k Bp[b,i',j',k] U[k,r] on the diagonal blocks only."""
-    K, R = U.shape
-    if Bp.dtype != torch.float32 or U.dtype != torch.float32:
-        raise TypeError("inputs must be float32")
-    d = nblocks * bs
-    rows = d * d if (flags & ST_FLAG_DENSE_CONTROL) else nblocks * bs * bs
-    if Bp.numel() != rows * K:
-        raise ValueError("shape mismatch")
-    if out is None:
-        out = _alloc((rows, R), torch.float32, Bp.device)
-    ws = _workspace(ws, Bp.device, ST_OP_TTM_BLOCKDIAG, nblocks, bs, K, R, flags)
-    _check(lib().st_ttm_blockdiag(_dev(Bp, "Bp"), nblocks, bs, K, _dev(U, "U"), R, _dev(out, "out"),
-                                  ws.data_ptr(), ws.numel() * ws.element_size(), flags, _stream()),
-           "st_ttm_blockdiag")
-    return out
+    return (_native or _bind()).ttm_blockdiag(Bp, U, nblocks, bs, out, ws, flags)
 
 
 def st_ttm_packed(Bp: torch.Tensor, U: torch.Tensor, layout: Layout, out: torch.Tensor | None = None,
                   ws: torch.Tensor | None = None, flags: int = 0) -> torch.Tensor:
     """Ap[p,r] = sum_k Bp[p,k] U[k,r] for every packed position p of `layout` (inner = K)."""
-    K, R = U.shape
-    if Bp.dtype != torch.float32 or U.dtype != torch.float32:
-        raise TypeError("inputs must be float32")
-    desc, n_packed, _ = _layout_info(layout)
-    if layout.inner != K or Bp.numel() != n_packed:
-        raise ValueError("shape mismatch")
-    rows = Bp.numel() // K
-    if out is None:
-        out = _alloc((rows, R), torch.float32, Bp.device)
-    ws = _workspace(ws, Bp.device, ST_OP_TTM_BLOCKDIAG, rows, 1, K, R, flags)
-    _check(lib().st_ttm_packed(desc, _dev(Bp, "Bp"), _dev(U, "U"), R, _dev(out, "out"),
-                               ws.data_ptr(), ws.numel() * ws.element_size(), flags, _stream()), "st_ttm_packed")
-    return out
+    return (_native or _bind()).ttm_packed(Bp, U, layout, out, ws, flags)
 
 
 def st_thp(Bp: torch.Tensor, C: torch.Tensor, layout: Layout, out: torch.Tensor | None = None) -> torch.Tensor:
     """Ap = Bp * (C at the unique positions of `layout`): packed B, dense C, packed result."""
-    if Bp.dtype != torch.float32 or C.dtype != torch.float32:
-        raise TypeError("inputs must be float32")
-    desc, n_packed, n_dense = _layout_info(layout)
-    if Bp.numel() != n_packed or C.numel() != n_dense:
-        raise ValueError("shape mismatch")
-    if out is None:
-        out = _alloc(tuple(Bp.shape), torch.float32, Bp.device)
-    _check(lib().st_thp(desc, _dev(Bp, "Bp"), _dev(C, "C"), _dev(out, "out"), _stream()), "st_thp")
-    return out
+    return (_native or _bind()).thp(Bp, C, layout, out)
 
 
 def st_packed_axpby(alpha: float, a: torch.Tensor, beta: float, b: torch.Tensor,
                     out: torch.Tensor | None = None) -> torch.Tensor:
     """out = alpha * a + beta * b for two packed float32 arrays of the same layout (out may be a or b)."""
-    if a.dtype != torch.float32 or b.dtype != torch.float32 or a.numel() != b.numel():
-        raise ValueError("two float32 arrays of the same size are needed")
-    if out is None:
-        out = _alloc(tuple(a.shape), torch.float32, a.device)
-    _check(lib().st_packed_axpby(a.numel(), alpha, _dev(a, "a"), beta, _dev(b, "b"), _dev(out, "out"), _stream()),
-           "st_packed_axpby")
-    return out
+    return (_native or _bind()).axpby(alpha, a, beta, b, out)
 
 
 def st_packed_mul(a: torch.Tensor, b: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
     """out = a * b for two packed float32 arrays of the same layout (out may be a or b)."""
-    if a.dtype != torch.float32 or b.dtype != torch.float32 or a.numel() != b.numel():
-        raise ValueError("two float32 arrays of the same size are needed")
-    if out is None:
-        out = _alloc(tuple(a.shape), torch.float32, a.device)
-    _check(lib().st_packed_mul(a.numel(), _dev(a, "a"), _dev(b, "b"), _dev(out, "out"), _stream()), "st_packed_mul")
-    return out
+    return (_native or _bind()).mul(a, b, out)
 
 
 def st_check_status(ws: torch.Tensor | None = None) -> int:

@@ -1,8 +1,10 @@
-"""Builds libstructtensor.so (sm_100a) in-tree with nvcc.  Run as a module or call build()."""
+"""Builds libstructtensor.so (sm_100a, nvcc) and the Python binding _binding.so (g++) in-tree.  Run as a module or call
+build()."""
 from __future__ import annotations
 
 import concurrent.futures
 import os
+import shutil
 import subprocess
 import sys
 
@@ -12,6 +14,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libstructtensor.so")
+BINDING_SRC = os.path.join(CSRC, "binding.cpp")
+BINDING = os.path.join(HERE, "_binding.so")
 # debug build with device-side range checks (-DST_BOUNDS_CHECK; relocatable device code for its one device-wide word)
 OBJDIR_CHECK = os.path.join(HERE, "_build_check")
 LIB_CHECK = os.path.join(HERE, "libstructtensor_check.so")
@@ -52,6 +56,28 @@ def _compile(src: str, verbose: bool, check: bool = False) -> str:
     return obj
 
 
+def _build_binding(force: bool) -> None:
+    deps = (BINDING_SRC, os.path.join(INCLUDE, "structtensor.h"))
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(map(os.path.getmtime, deps)):
+        return
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")))
+    tmp = BINDING + ".%d.tmp" % os.getpid()
+    # the torch libraries are in the process before the module is imported, so no search path is recorded for them
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+           "-I", INCLUDE, "-isystem", os.path.join(root, "include"),
+           "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-isystem", os.path.join(cuda, "include"), "-isystem", sysconfig.get_paths()["include"], BINDING_SRC, "-o", tmp,
+           "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed for binding.cpp:\n%s\n%s" % (res.stdout, res.stderr))
+    os.replace(tmp, BINDING)
+
+
 def build(force: bool = False, verbose: bool = False, check: bool = False) -> str:
     """Compiles every .cu under csrc/ and links the shared library (check=True: the range-checking debug build)."""
     objdir, lib = (OBJDIR_CHECK, LIB_CHECK) if check else (OBJDIR, LIB)
@@ -61,8 +87,11 @@ def build(force: bool = False, verbose: bool = False, check: bool = False) -> st
             if f.endswith(".o"):
                 os.remove(os.path.join(objdir, f))
     srcs = _sources()
-    with concurrent.futures.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    with concurrent.futures.ThreadPoolExecutor(max_workers=min(8, len(srcs) + 1)) as ex:
+        binding = None if check else ex.submit(_build_binding, force)
         objs = list(ex.map(lambda s: _compile(s, verbose, check), srcs))
+    if binding is not None:
+        binding.result()
     if force or not os.path.exists(lib) or any(os.path.getmtime(o) > os.path.getmtime(lib) for o in objs):
         tmp = lib + ".%d.tmp" % os.getpid()
         cmd = ["nvcc", "-shared", "-gencode", "arch=compute_100a,code=sm_100a", *(["-rdc=true"] if check else []), "-o", tmp, *objs]
