@@ -65,6 +65,12 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem, bool va
     const int sz = valid ? 16 : 0;         // src-size 0: the 16 bytes are zero-filled
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(sz));
 }
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem, bool valid)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    const int sz = valid ? 4 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(s), "l"(gmem), "r"(sz));
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
@@ -97,14 +103,12 @@ __device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c)
 // the loop is "row base + immediate" (integer multiply-adds share the FMA pipe: with run-time strides
 // the kernel was 9 % slower at d = 64).
 template <int J0, bool DIAG, int DC>
-__device__ __forceinline__ void m3_stage(const float *__restrict__ xs, int rows_, int d_, int pi, int oj, int ok, int half_,
+__device__ __forceinline__ void m3_stage(const float *__restrict__ row, int rows, int step_, int pi, int oj, int ok, int half_,
                                          uint64_t (&acc)[8][4])
 {
-    const int d = DC > 0 ? DC : d_, half = DC > 0 ? DC / 2 : half_;
-    const int rows = DC > 0 ? M3_STAGE_ROWS : rows_;      // the instance with compile-time strides has full stages
+    const int step = DC > 0 ? DC : step_, half = DC > 0 ? DC / 2 : half_;
 #pragma unroll 2
-    for (int r = 0; r < rows; ++r) {
-        const float *row = xs + r * d;
+    for (int r = 0; r < rows; ++r, row += step) {
         const float xi = row[pi];
         const float4 ja = *reinterpret_cast<const float4 *>(row + oj);
         const float4 jb = *reinterpret_cast<const float4 *>(row + oj + half);
@@ -138,10 +142,15 @@ struct M3Args {
     const unsigned *gtile;
     int64_t N, ldx, rows_per_slice;
     int d, dp, rows, out_elems;
+    int nw, rg;                            // rg > 1: the table has nw warps, and rg copies of them share the rows of a stage
 };
 
-// ALIGNED: rows are staged by asynchronous 16-byte copies; otherwise by plain 4-byte loads (an instance of
+// ALIGNED: rows are staged by asynchronous 16-byte copies; otherwise by 4-byte ones (an instance of
 // its own: with both loaders in one kernel the common one ran 7 % slower).
+//
+// Few features make few tiles: one warp's worth at d = 16.  Row group g of rg then takes rows g, g + rg, ... of every
+// stage, and the groups' sums are added in shared memory, in group order, before they go to memory.  [23208,16]: 32 us with
+// one warp per variant walking all rows, 12.5 now; [4096,24] 18.9 and 12.6.
 template <int WARPS, int DC, bool ALIGNED>
 __global__ void __launch_bounds__(M3_THREADS, 1)
 moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
@@ -156,8 +165,11 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
     extern __shared__ __align__(16) float smem[];   // M3_BUFFERS stages of a.rows x dp floats
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int group = blockIdx.x;
-    const int slot = group * M3_WPB + warp;
-    const int variant = a.gtile ? a.gvariant[slot] : tab.variant[slot];
+    const int rg = DC > 0 ? 1 : a.rg;
+    const int row_group = rg > 1 ? warp / a.nw : 0;
+    const int slot = rg > 1 ? warp - row_group * a.nw : group * M3_WPB + warp;
+    const bool working = rg == 1 || row_group < rg;
+    const int variant = !working ? 255 : a.gtile ? a.gvariant[slot] : tab.variant[slot];
     const unsigned t = a.gtile ? a.gtile[slot * 32 + lane] : m3_unpack16(tab.tile[slot * 32 + lane]);
     const bool valid = (t >> 31) != 0u;
     const int ti = t & 511, tjb = (t >> 9) & 63, tkb = (t >> 15) & 63;
@@ -176,7 +188,7 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
     const int64_t n_begin = (int64_t)blockIdx.y * rows_per_slice;
     int64_t n_end = n_begin + rows_per_slice;
     if (n_end > N) n_end = N;
-    const int stage_rows = DC > 0 ? M3_STAGE_ROWS : a.rows;
+    const int stage_rows = a.rows;
     const int stage_floats = stage_rows * dp;
     const int chunks_per_row = dp / 4;
     const int stage_chunks = stage_rows * chunks_per_row;
@@ -192,12 +204,13 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
                 cp_async16(dst + r * dp + 4 * sc, X + (in ? n * ldx + 4 * g : 0), in);
             }
         } else {
-            // rows that are not 16-byte aligned: one float at a time (the barrier of the stage orders the stores)
+            // rows that are not 16-byte aligned: one float at a time
             for (int e = tid; e < stage_rows * dp; e += M3_THREADS) {
                 const int r = e / dp, c = e - r * dp;
                 const int64_t n = n0 + r;
                 const int g = c >> 2, sc = (g & 1) ? nbk + (g >> 1) : (g >> 1);
-                dst[r * dp + 4 * sc + (c & 3)] = (n < n_end && c < d) ? X[n * ldx + c] : 0.f;
+                const bool in = n < n_end && c < d;
+                cp_async4(dst + r * dp + 4 * sc + (c & 3), X + (in ? n * ldx + c : 0), in);
             }
         }
         cp_async_commit();
@@ -217,23 +230,59 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
             load_stage((int)((s + M3_BUFFERS - 1) % M3_BUFFERS), n_begin + (s + M3_BUFFERS - 1) * stage_rows);
         else
             cp_async_commit();
-        const float *xs = smem + (int)(s % M3_BUFFERS) * stage_floats;
+        // this row group's rows of the stage; rows past the end of the slice are not visited
+        const int64_t left = n_end - (n_begin + s * stage_rows);
+        const int in_stage = left < stage_rows ? (int)left : stage_rows;
+        const int rows = rg > 1 ? (in_stage - row_group + rg - 1) / rg : in_stage;
+        const int step = DC > 0 ? DC : rg * dp;
+        const float *xs = smem + (int)(s % M3_BUFFERS) * stage_floats + row_group * dp;
         switch (variant) {
-        case 0: m3_stage<0, false, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
-        case 1: m3_stage<0, true, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
-        case 2: m3_stage<1, false, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
-        case 3: m3_stage<2, false, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
-        case 4: m3_stage<3, false, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
-        case 5: m3_stage<4, false, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
-        case 6: m3_stage<5, false, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
-        case 7: m3_stage<6, false, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
-        case 8: m3_stage<7, false, DC>(xs, stage_rows, dp, pi, oj, ok, half, acc); break;
+        case 0: m3_stage<0, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 1: m3_stage<0, true, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 2: m3_stage<1, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 3: m3_stage<2, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 4: m3_stage<3, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 5: m3_stage<4, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 6: m3_stage<5, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 7: m3_stage<6, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 8: m3_stage<7, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
         default: break;
         }
     }
     cp_async_wait<0>();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the slice sums may be launched; they wait for this grid to end
 
+    if (rg > 1) {
+        // red[sum][row group][table thread]; row group g adds and stores sums g, g + rg, ...
+        const int nt = a.nw * 32, all = rg * nt;
+        float *red = smem;
+        __syncthreads();
+        if (working) {
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    float lo, hi;
+                    unpack2(acc[r][c], lo, hi);
+                    red[(8 * r + 2 * c) * all + tid] = lo;
+                    red[(8 * r + 2 * c + 1) * all + tid] = hi;
+                }
+        }
+        __syncthreads();
+        if (!valid || !working) return;
+        float *mine = a.partials + (size_t)blockIdx.y * out_elems;
+        const int td = tid - row_group * nt;
+        for (int v = row_group; v < 64; v += rg) {
+            const int j = 8 * tjb + (v >> 3), k = 8 * tkb + (v & 7);
+            if (j < ti || k < j || k >= d) continue;
+            const float *p = red + v * all + td;
+            float sum = 0.f;
+            for (int g = 0; g < rg; ++g) sum += p[g * nt];
+            const int at = (int)tet_encode(d, ti, j, k);
+            if (ST_BOUNDS_OK(at, out_elems, 3)) mine[at] = sum;
+        }
+        return;
+    }
     if (!valid || variant == 255) return;
     float *mine = a.partials + (size_t)blockIdx.y * out_elems;
 #pragma unroll
@@ -329,6 +378,7 @@ static int variant_cost(int v)
 // and tile word per thread slot, group-major.
 struct M3HostTable {
     int groups = 0;
+    int nw = 0, rg = 1;                    // rg > 1: one group of nw warps, repeated rg times over the rows
     std::vector<unsigned char> variant;    // groups * M3_WPB
     std::vector<unsigned> tile;            // groups * M3_WPB * 32
 };
@@ -350,15 +400,42 @@ static void build_table(int d, bool dense, M3HostTable &tab)
             }
     }
     std::vector<WarpDesc> warps;
-    for (int v = 0; v < 9; ++v)
-        for (size_t o = 0; o < lists[v].size(); o += 32) {
-            WarpDesc w;
-            w.variant = v;
-            w.cost = variant_cost(v);
-            w.tiles.assign(lists[v].begin() + o, lists[v].begin() + std::min(lists[v].size(), o + 32));
-            warps.push_back(w);
+    auto add = [&](int v, std::vector<unsigned> tiles) {
+        WarpDesc w;
+        w.variant = v;
+        w.cost = variant_cost(v);
+        w.tiles = std::move(tiles);
+        warps.push_back(w);
+    };
+    // whole warps of one variant; what is left over shares warps of a variant that covers its members (what such a tile
+    // computes beyond its own entries is not stored): the full tile, or among the row-limited ones the longest
+    std::vector<std::pair<int, unsigned>> rest;
+    for (int v = 0; v < 9; ++v) {
+        const size_t whole = lists[v].size() / 32 * 32;
+        for (size_t o = 0; o < whole; o += 32) add(v, std::vector<unsigned>(lists[v].begin() + o, lists[v].begin() + o + 32));
+        for (size_t o = whole; o < lists[v].size(); ++o) rest.push_back({v, lists[v][o]});
+    }
+    for (size_t o = 0; o < rest.size(); o += 32) {
+        std::vector<unsigned> tiles;
+        int v = rest[o].first;
+        for (size_t e = o; e < rest.size() && e < o + 32; ++e) {
+            const int w = rest[e].first;
+            if (w != v) v = (v < 2 || w < 2) ? 0 : std::min(v, w);
+            tiles.push_back(rest[e].second);
         }
+        add(v, tiles);
+    }
     const int nw = (int)warps.size();
+    if (2 * nw <= M3_WPB) {
+        tab.groups = 1;
+        tab.nw = nw;
+        tab.rg = M3_WPB / nw;
+        for (const WarpDesc &w : warps) {
+            tab.variant.push_back((unsigned char)w.variant);
+            for (int l = 0; l < 32; ++l) tab.tile.push_back(l < (int)w.tiles.size() ? w.tiles[l] : 0u);
+        }
+        return;
+    }
     const int groups = (nw + M3_WPB - 1) / M3_WPB;
     // deal warps, most expensive first, to the scheduler bin (group, warp%4) with the least load,
     // then swap warps between the fullest bin and the others while that lowers the maximum
@@ -413,6 +490,7 @@ static void build_table(int d, bool dense, M3HostTable &tab)
         if (!improved) break;
     }
     tab.groups = groups;
+    tab.nw = nw;
     tab.variant.assign((size_t)groups * M3_WPB, 255);
     tab.tile.assign((size_t)groups * M3_WPB * 32, 0u);
     for (int b = 0; b < bins; ++b) {
@@ -450,24 +528,32 @@ struct M3Plan {
     size_t smem;
 };
 
-// Block groups per sample slice; slices fill the SMs once.
-static M3Plan moment3_plan(int64_t N, int64_t d, int groups)
+// Block groups per sample slice; slices fill the SMs once.  A slice has at least 32 rows, or four per row group: shorter
+// ones cost more in partial sums than they save.
+static M3Plan moment3_plan(int64_t N, int64_t d, const M3HostTable &tab)
 {
     M3Plan p;
-    p.groups = groups;
+    p.groups = tab.groups;
     p.dp = (int)((d + 7) / 8 * 8);
     p.out_elems = tet_rows(d);
-    int rows = (int)(M3_SMEM_BUDGET / ((size_t)M3_BUFFERS * p.dp * sizeof(float))) / 8 * 8;
-    p.rows = rows > M3_STAGE_ROWS ? M3_STAGE_ROWS : rows;
-    p.smem = (size_t)M3_BUFFERS * p.rows * p.dp * sizeof(float);
+    int64_t cap = (int64_t)(M3_SMEM_BUDGET / ((size_t)M3_BUFFERS * p.dp * sizeof(float))) / 8 * 8;
+    if (cap > M3_STAGE_ROWS) cap = M3_STAGE_ROWS;
     const int sms = sm_count_or_default();
-    int64_t slices = sms / groups;
+    int64_t slices = sms / p.groups;
     if (slices < 1) slices = 1;
-    const int64_t max_slices = (N + p.rows - 1) / p.rows;
+    const int64_t least = tab.rg > 1 ? 4 * tab.rg : 32;
+    const int64_t max_slices = (N + least - 1) / least;
     if (slices > max_slices) slices = max_slices;
     p.rows_per_slice = (N + slices - 1) / slices;
     p.slices = (int)((N + p.rows_per_slice - 1) / p.rows_per_slice);
-    p.table_bytes = d > M3_PARAM_D ? round_up((size_t)groups * M3_WPB * (1 + 32 * sizeof(unsigned)), 256) : 0;
+    const int64_t stages = (p.rows_per_slice + cap - 1) / cap;      // of equal length
+    p.rows = (int)((p.rows_per_slice + stages - 1) / stages);
+    p.smem = (size_t)M3_BUFFERS * p.rows * p.dp * sizeof(float);
+    if (tab.rg > 1) {                                               // the sums of all row groups
+        const size_t red = (size_t)64 * tab.nw * tab.rg * 32 * sizeof(float);
+        if (red > p.smem) p.smem = red;
+    }
+    p.table_bytes = d > M3_PARAM_D ? round_up((size_t)p.groups * M3_WPB * (1 + 32 * sizeof(unsigned)), 256) : 0;
     return p;
 }
 
@@ -477,7 +563,7 @@ static st_status moment3_launch(const float *X, int64_t N, int64_t d, int64_t ld
 {
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
     const M3HostTable &tab = cached_table((int)d, dense);
-    const M3Plan p = moment3_plan(N, d, tab.groups);
+    const M3Plan p = moment3_plan(N, d, tab);
     const size_t need = kWsHeaderBytes + p.table_bytes + (size_t)p.slices * p.out_elems * sizeof(float);
     if (!ws || ws_bytes < need) return ST_ERR_WORKSPACE;
     if (!aligned256(ws)) return ST_ERR_ALIGN;
@@ -490,12 +576,13 @@ static st_status moment3_launch(const float *X, int64_t N, int64_t d, int64_t ld
     a.gvariant = nullptr; a.gtile = nullptr;
     a.N = N; a.ldx = ldx; a.rows_per_slice = p.rows_per_slice;
     a.d = (int)d; a.dp = p.dp; a.rows = p.rows; a.out_elems = (int)p.out_elems;
+    a.nw = tab.nw; a.rg = tab.rg;
     const bool aligned = d % 4 == 0 && ldx % 4 == 0;
     static M3Table<WARPS> empty_table;      // the parameter slot of launches that read the table from memory
     M3Table<WARPS> local;
     const M3Table<WARPS> *param = &empty_table;
     if (p.table_bytes == 0) {
-        if ((size_t)tab.groups * M3_WPB > (size_t)WARPS) return ST_ERR_UNSUPPORTED;
+        if (tab.variant.size() > (size_t)WARPS) return ST_ERR_UNSUPPORTED;
         for (int i = 0; i < WARPS; ++i) local.variant[i] = i < (int)tab.variant.size() ? tab.variant[i] : 255;
         for (int i = 0; i < WARPS * 32; ++i) local.tile[i] = i < (int)tab.tile.size() ? m3_pack16(tab.tile[i]) : (unsigned short)0;
         param = &local;
@@ -513,7 +600,7 @@ static st_status moment3_launch(const float *X, int64_t N, int64_t d, int64_t ld
     if (!aligned) {
         if (!ensure_dynamic_smem(moment3_kernel<WARPS, 0, false>, p.smem)) return ST_ERR_CUDA;
         moment3_kernel<WARPS, 0, false><<<grid, M3_THREADS, p.smem, stream>>>(a, *param);
-    } else if (p.dp == M3_PARAM_D && p.rows == M3_STAGE_ROWS) {   // d = 60, 64 has its own instance with compile-time strides
+    } else if (p.dp == M3_PARAM_D) {   // d = 60, 64 has its own instance with compile-time strides
         if (!ensure_dynamic_smem(moment3_kernel<WARPS, M3_PARAM_D, true>, p.smem)) return ST_ERR_CUDA;
         moment3_kernel<WARPS, M3_PARAM_D, true><<<grid, M3_THREADS, p.smem, stream>>>(a, *param);
     } else {
@@ -534,7 +621,7 @@ size_t moment3_workspace(int64_t N, int64_t d, unsigned flags)
         return (flags & ST_FLAG_DENSE_CONTROL) ? 0 : moment3_tc_workspace(N, d, (flags & ST_FLAG_TC_BF16) != 0);
     if (N <= 0 || d < 1 || d > M3_MAX_D) return 0;
     const M3HostTable &tab = cached_table((int)d, (flags & ST_FLAG_DENSE_CONTROL) != 0);
-    const M3Plan p = moment3_plan(N, d, tab.groups);
+    const M3Plan p = moment3_plan(N, d, tab);
     return kWsHeaderBytes + p.table_bytes + (size_t)p.slices * p.out_elems * sizeof(float);
 }
 

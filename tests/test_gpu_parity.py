@@ -337,6 +337,17 @@ def test_fixed_order_calls_give_the_same_bits_twenty_times(st):
         st._allocator.check()
 
 
+
+# row groups (few features: copies of the same warps share the rows of a stage), tiles of several variants in one warp, slices
+# from one row up, stages of any length, rows that start at any 4-byte offset
+@pytest.mark.parametrize("N,d", [(1, 3), (63, 9), (65, 16), (4097, 17), (1000, 24), (3333, 31), (257, 33), (31, 48), (9500, 57),
+                                 (2000, 60), (129, 63), (77, 72)])
+def test_moment3_f32_row_groups_and_short_slices(st, N, d):
+    X = workloads.draw((N, d), "normal", 310 + N + d)
+    T, S = oracle.moment3(X)
+    assert oracle.rel_err(expand3(st, st.st_sym_moment3(dev(X)), d), T, S) <= TOL_F32
+
+
 @pytest.mark.parametrize("d", [1, 2, 3, 5, 8, 16, 17, 24, 40, 57, 63, 64])
 @pytest.mark.parametrize("N", [1, 63, 64, 65, 1000])
 def test_moment3_small(st, N, d):
