@@ -175,6 +175,15 @@ __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t *r)
         : "r"(taddr)
         : "memory");
 }
+// 16 lanes x 16 consecutive columns in the fragment form of a matrix product: thread t receives, for g = 0, 1 and h = 0, 1,
+// lane (base lane + t / 4 + 8 h), columns 8 g + 2 (t % 4) and the next one in r[4 g + 2 h], r[4 g + 2 h + 1].
+__device__ __forceinline__ void tmem_ld_16x16(uint32_t taddr, uint32_t *r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ bool elect_one()

@@ -25,7 +25,7 @@
 // convert -> store -> proxy fence -> barrier, so there are four of them per scheduler).
 #include "tc_common.cuh"
 #include "st_index.cuh"
-#include "mttkrp_common.cuh"
+#include "fibre_epilogue.cuh"
 #include <cuda_bf16.h>
 
 namespace st {
@@ -216,75 +216,21 @@ __global__ void __launch_bounds__(split::THREADS, 1) ttm_split_kernel(const Spli
         for (int t = 0; t < my_tiles; ++t) {
             const int buf = t & 1;
             const int64_t tile = blockIdx.x + (int64_t)t * gridDim.x;
-            const int64_t row = tile * BM + q * 32 + lane;
-            const bool valid = row < a.rows;
-            // MTTKRP: the fibre's (i, j) and, for R = 32, its row of C are fetched before the accumulator is
+            const int64_t unit = tile * (BM / 32) + q;
+            // MTTKRP: the fibres' (i, j) and the first columns of their rows of C are fetched before the accumulator is
             // waited for -- with the memory system saturated by the fibre stream a dependent load costs
             // microseconds, which would otherwise stall the tile after next
-            int64_t gi = -1, gj = 0;
-            WarpRuns runs{0u, 0u};
-            float4 cpre[8];
-            const bool pre = a.mode != SP_TTM && R == 32;
+            UnitFibres f;
+            float2 cpre[2][4];
             if (a.mode != SP_TTM) {
-                if (valid) {
-                    if (a.mode == SP_MTTKRP_PACKED) tri_decode(a.I, row, gi, gj);
-                    else { gi = row / a.div; gj = row - gi * a.div; }
-                }
-                runs = warp_runs(valid, (int)gi, lane);
-                if (pre) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        cpre[e] = valid ? __ldg(reinterpret_cast<const float4 *>(a.C + gj * R) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+                f = unit_fibres(unit * 32, a.rows, a.mode == SP_MTTKRP_DENSE, a.I, a.div, lane);
+                unit_load_c(f, a.C, R, 0, lane, cpre);
             }
             if (!mbar_wait(&acc_full[buf], (uint32_t)((t >> 1) & 1), abort_flag, a.status, 4)) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * R);
-            // 16 columns at a time keeps the register count low; cv = the fibre's four float4 of C for them
-            auto chunk = [&](int c0, const float4 &cv0, const float4 &cv1, const float4 &cv2, const float4 &cv3) {
-                float v[16];
-                {
-                    uint32_t r1[16], r2[16];
-                    tmem_ld_32x16(taddr + (uint32_t)c0, r1);
-                    tmem_ld_32x16(taddr + (uint32_t)(R + c0), r2);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(r1[e]) + __uint_as_float(r2[e]);
-                }
-                if (a.mode == SP_TTM) {
-                    if (valid) {
-                        float4 *dst = reinterpret_cast<float4 *>(a.out + row * R + c0);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) dst[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-                    }
-                } else {
-                    const float4 cv[4] = {cv0, cv1, cv2, cv3};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {            // lanes without a fibre hold zeros in cv
-                        v[4 * e + 0] *= cv[e].x;
-                        v[4 * e + 1] *= cv[e].y;
-                        v[4 * e + 2] *= cv[e].z;
-                        v[4 * e + 3] *= cv[e].w;
-                    }
-                    warp_store_runs16(v, runs, valid, (int)gi, tile * (BM / 32) + q, lane, a.out, R, c0,
-                                      mttkrp_slots(a.rows, 32, a.I, 1));
-                }
-            };
-            if (pre) {
-                chunk(0, cpre[0], cpre[1], cpre[2], cpre[3]);
-                chunk(16, cpre[4], cpre[5], cpre[6], cpre[7]);
-            } else {
-                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int c0 = 0; c0 < R; c0 += 16) {
-                    float4 cv[4] = {z, z, z, z};
-                    if (a.mode != SP_TTM && valid) {
-                        const float4 *crow = reinterpret_cast<const float4 *>(a.C + gj * R + c0);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) cv[e] = __ldg(crow + e);
-                    }
-                    chunk(c0, cv[0], cv[1], cv[2], cv[3]);
-                }
-            }
+            if (a.mode == SP_TTM) ttm_epilogue<true>(taddr, R, unit * 32, a.rows, a.out, lane);
+            else mttkrp_epilogue<true>(taddr, R, f, a.C, unit, a.out, mttkrp_slots(a.rows, 32, a.I, 1), lane, cpre);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);

@@ -11,7 +11,7 @@
 // next.  Warp roles: warp 0 TMA producer, warp 1 MMA issuer / TMEM owner, warps 2..5 epilogue.
 #include "tc_common.cuh"
 #include "st_index.cuh"
-#include "mttkrp_common.cuh"
+#include "fibre_epilogue.cuh"
 
 namespace st {
 
@@ -194,71 +194,21 @@ ttm_tc_kernel(const __grid_constant__ CUtensorMap tmap, const TtmTcArgs a)
             const int buf = t & 1;
             int64_t tile = blockIdx.x + (int64_t)t * gridDim.x;
             if (a.reverse) tile = a.ntiles - 1 - tile;
-            const int64_t row = tile * BM + q * 32 + lane;
-            // MTTKRP: the fibre's (i, j) and, for R = 32, its row of C are fetched before the accumulator is
+            const int64_t unit = tile * (BM / 32) + q;
+            // MTTKRP: the fibres' (i, j) and the first columns of their rows of C are fetched before the accumulator is
             // waited for -- with the memory system saturated by the fibre stream a dependent load costs
             // microseconds
-            const bool valid = row < a.rows;
-            int64_t gi = -1, gj = 0;
-            WarpRuns runs{0u, 0u};
-            float4 cpre[8];
-            const bool pre = a.mode != TC_TTM && a.R == 32;
+            UnitFibres f;
+            float2 cpre[2][4];
             if (a.mode != TC_TTM) {
-                if (valid) {
-                    if (a.mode == TC_MTTKRP_PACKED) tri_decode(a.I, row, gi, gj);
-                    else { gi = row / a.div; gj = row - gi * a.div; }
-                }
-                runs = warp_runs(valid, (int)gi, lane);
-                if (pre) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        cpre[e] = valid ? __ldg(reinterpret_cast<const float4 *>(a.C + gj * a.R) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+                f = unit_fibres(unit * 32, a.rows, a.mode == TC_MTTKRP_DENSE, a.I, a.div, lane);
+                unit_load_c(f, a.C, a.R, 0, lane, cpre);
             }
             if (!mbar_wait(&acc_full[buf], (uint32_t)((t >> 1) & 1), abort_flag, a.status, 4)) break;
             tc_fence_after();
-            if (a.mode == TC_TTM) {
-                float *dst = a.out + row * a.R;
-                for (int c0 = 0; c0 < a.R; c0 += 32) {
-                    uint32_t r[32];
-                    tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * a.R + c0), r);
-                    tmem_ld_wait();
-                    if (row < a.rows) {
-#pragma unroll
-                        for (int e = 0; e < 32; e += 4)
-                            if (c0 + e < a.R)
-                                *reinterpret_cast<uint4 *>(dst + c0 + e) = make_uint4(r[e], r[e + 1], r[e + 2], r[e + 3]);
-                    }
-                }
-            } else {
-                // MTTKRP: this lane's fibre is row (i,j); scale by C[j,:], then sum every run of fibres of
-                // the warp that share i and write it to partial slot (unit + i), unit = row / 32 (see
-                // mttkrp_common.cuh).  The 32 fibres of a warp are consecutive, so they usually share i:
-                // one transposing shuffle reduction and one coalesced store per 32 columns.
-                const int gi32 = (int)gi;
-                const int64_t unit = tile * (BM / 32) + q;
-                for (int c0 = 0; c0 < a.R && runs.heads != 0u; c0 += 32) {
-                    uint32_t r[32];
-                    tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * a.R + c0), r);
-                    tmem_ld_wait();
-                    float v[32];
-                    if (valid) {
-                        const float4 *crow = reinterpret_cast<const float4 *>(a.C + gj * a.R + c0);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float4 c = pre ? cpre[e] : __ldg(crow + e);
-                            v[4 * e + 0] = c.x * __uint_as_float(r[4 * e + 0]);
-                            v[4 * e + 1] = c.y * __uint_as_float(r[4 * e + 1]);
-                            v[4 * e + 2] = c.z * __uint_as_float(r[4 * e + 2]);
-                            v[4 * e + 3] = c.w * __uint_as_float(r[4 * e + 3]);
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = 0.f;
-                    }
-                    warp_store_runs(v, runs, valid, gi32, unit, lane, a.out, a.R, c0, mttkrp_slots(a.rows, 32, a.I, 1));
-                }
-            }
+            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * a.R);
+            if (a.mode == TC_TTM) ttm_epilogue<false>(taddr, a.R, unit * 32, a.rows, a.out, lane);
+            else mttkrp_epilogue<false>(taddr, a.R, f, a.C, unit, a.out, mttkrp_slots(a.rows, 32, a.I, 1), lane, cpre);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);
