@@ -19,7 +19,10 @@ namespace ttmtc {
 constexpr int BM = 128;                    // fibres per tile
 constexpr int KC = 32;                     // floats per k-slice (128 bytes)
 constexpr int STAGE_BYTES = BM * KC * 4;   // 16 KiB
-constexpr int THREADS = 192;
+// Groups of four epilogue warps, on alternate tiles.  Short fibres leave an MTTKRP tile's epilogue (two dependent trips to L2)
+// as the chain: I = 900, K = 48, R = 64 runs 59 us with one group, 42 with two.
+constexpr int EPI_GROUPS = 2;
+constexpr int THREADS = 64 + 128 * EPI_GROUPS;
 // 96 KB of fibres in flight per SM: a copy loop without arithmetic reads 269 MB at 6.5 TB/s with six stages, 5.9 with ten and
 // 5.8 with thirteen (the memory system queues); this kernel 56.4 us with five or six ([64,64,64,256] x [256,64], 269 MB
 // read, 67 written), 57.2 with eight, 58.9 with ten, 58.8 with four.
@@ -190,7 +193,7 @@ ttm_tc_kernel(const __grid_constant__ CUtensorMap tmap, const TtmTcArgs a)
         }
     } else {
         const int q = warp & 3;
-        for (int t = 0; t < my_tiles; ++t) {
+        for (int t = (warp - 2) >> 2; t < my_tiles; t += EPI_GROUPS) {
             const int buf = t & 1;
             int64_t tile = blockIdx.x + (int64_t)t * gridDim.x;
             if (a.reverse) tile = a.ntiles - 1 - tile;
