@@ -87,6 +87,8 @@ __global__ void __launch_bounds__(RG_THREADS, 1) rowgemm_kernel(const RgArgs a)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tc = lane % CT, fib = lane / CT;
 
+    pdl_wait();
+    pdl_trigger();
     if (a.status && blockIdx.x == 0 && tid == 0) {      // no bounded waits in this kernel: the status is "ok"
         a.status[kWsStatusWord] = 0;
         a.status[kWsDetailWord] = 0;
@@ -243,7 +245,6 @@ __global__ void __launch_bounds__(RG_THREADS, 1) rowgemm_kernel(const RgArgs a)
             for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
     }
     asm volatile("cp.async.wait_group 0;\n" ::);
-    if (MODE != RG_TTM) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the row sums may be launched
 }
 
 // Second pass of MTTKRP: one warp per row of A adds the partial slots of that row in increasing
@@ -252,7 +253,8 @@ __global__ void __launch_bounds__(256)
 mttkrp_rowsum_kernel(const float *__restrict__ part, float *__restrict__ A, int64_t I_full, int64_t i_off, MttkrpRows m,
                      int R, int unit_rows, int ksplit)
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched early: wait for the kernel that wrote the partials
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t ii = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (ii >= I_full) return;
@@ -290,21 +292,7 @@ mttkrp_rowsum_kernel(const float *__restrict__ part, float *__restrict__ A, int6
 st_status mttkrp_rowsum_launch(const float *part, float *A_full, int64_t I_full, int64_t i_off, const MttkrpRows &m,
                                int R, int unit_rows, int ksplit, cudaStream_t stream)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((I_full + 7) / 8));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, mttkrp_rowsum_kernel, part, A_full, I_full, i_off, m, R, unit_rows, ksplit) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ST_ERR_CUDA;
-    }
-    return ST_OK;
+    return launch(mttkrp_rowsum_kernel, dim3((unsigned)((I_full + 7) / 8)), 256, 0, stream, part, A_full, I_full, i_off, m, R, unit_rows, ksplit);
 }
 
 // tile shape by R: {TM, stages}; a warp owns TM * 32 / (R/8) consecutive fibres, a tile is the block's 16 warps
@@ -366,8 +354,7 @@ static st_status rowgemm_launch(const RgArgs &a0, cudaStream_t stream)
     const int grid = p.grid;
     auto run = [&](auto kernel) -> st_status {
         if (!ensure_dynamic_smem(kernel, smem)) return ST_ERR_CUDA;
-        kernel<<<grid, RG_THREADS, smem, stream>>>(a);
-        return launch_status();
+        return launch(kernel, grid, RG_THREADS, smem, stream, a);
     };
     switch (a.R) {
     case 8: return run(rowgemm_kernel<2, 1, 3, MODE>);

@@ -146,7 +146,8 @@ moment2_gemm_reduce_kernel(const float *__restrict__ partials, float *__restrict
     const float *base = partials + (size_t)(g.first[kind] + t) * (T * T);
     const size_t stride = (size_t)g.n[kind] * (T * T);
     const int wps = nsplit <= 8 ? 1 : nsplit <= 16 ? 2 : nsplit <= 32 ? 4 : 8;      // about eight loads per thread
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as a programmatic dependent of the main kernel
+    pdl_wait();
+    pdl_trigger();
     if (bi > bj) return;                                 // dense control: lower tiles are discarded
     int buf = 0;
     const int per = 8 / wps, first = warp % wps;
@@ -202,6 +203,8 @@ moment2_gemm_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, 
                     unsigned *status)
 {
     extern __shared__ __align__(16) float smem[];     // MG_STAGES x { As[MG_KC][MG_T], Bs[MG_KC][MG_T] }
+    pdl_wait();
+    pdl_trigger();
     if (blockIdx.x == 0 && threadIdx.x == 0) {        // no bounded waits here: the status is "ok"
         status[kWsStatusWord] = 0;
         status[kWsDetailWord] = 0;
@@ -283,7 +286,6 @@ moment2_gemm_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, 
             }
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         // what was not computed is not stored: the reduction reads i <= j < d only
         float *mine = partials + (size_t)blockIdx.x * (MG_T * MG_T);
 #pragma unroll
@@ -311,30 +313,12 @@ static st_status moment2_gemm(const float *X, int64_t N, int64_t d, int64_t ldx,
     if (!aligned256(ws)) return ST_ERR_ALIGN;
     float *partials = (float *)((unsigned char *)ws + kWsHeaderBytes);
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0, vec = d % 4 == 0 && ldx % 4 == 0;
-    auto run = [&](auto kernel) {
-        kernel<<<g.first[4], MG_THREADS, MG_SMEM, stream>>>(X, N, (int)d, ldx, partials, g, (unsigned *)ws);
-    };
-    if (dense) { if (vec) run(moment2_gemm_kernel<true, true>); else run(moment2_gemm_kernel<true, false>); }
-    else       { if (vec) run(moment2_gemm_kernel<false, true>); else run(moment2_gemm_kernel<false, false>); }
-    if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g.n[0] + g.n[1] + g.n[2] + g.n[3], 128);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const float *cpart = partials;
-    const int di = (int)d;
-    if (cudaLaunchKernelEx(&cfg, dense ? moment2_gemm_reduce_kernel<true> : moment2_gemm_reduce_kernel<false>, cpart, out, di, g) !=
-        cudaSuccess) {
-        (void)cudaGetLastError();
-        return ST_ERR_CUDA;
-    }
-    return ST_OK;
+    auto run = [&](auto kernel) { return launch(kernel, g.first[4], MG_THREADS, MG_SMEM, stream, X, N, (int)d, ldx, partials, g, (unsigned *)ws); };
+    const st_status rc = dense ? (vec ? run(moment2_gemm_kernel<true, true>) : run(moment2_gemm_kernel<true, false>))
+                               : (vec ? run(moment2_gemm_kernel<false, true>) : run(moment2_gemm_kernel<false, false>));
+    if (rc != ST_OK) return rc;
+    return launch(dense ? moment2_gemm_reduce_kernel<true> : moment2_gemm_reduce_kernel<false>, dim3(g.n[0] + g.n[1] + g.n[2] + g.n[3], 128), 256, 0,
+                  stream, partials, out, (int)d, g);
 }
 
 // Which of the two kernels: the one with fewer FMA slots per sample row, each divided by the fraction of the FMA

@@ -124,11 +124,15 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
     if (tid == 0) {
         for (int b = 0; b < M2S_BUFFERS; ++b) tc::mbar_init(&full[b], 1);
         *abort_flag = 0;
+        tc::fence_barrier_init();
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (tid == 0) {
         if (blockIdx.x == 0) {      // a time-out report can only be written 2^24 failed polls later
             a.status[kWsStatusWord] = 0;
             a.status[kWsDetailWord] = 0;
         }
-        tc::fence_barrier_init();
     }
     __syncthreads();
 
@@ -213,7 +217,6 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
             parity ^= 1u;
         }
     }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the sum over the slices may be launched; it waits for this grid to end
     if (BULK && *abort_flag && tid == 0) {
         // after a time-out: give the copies still in flight a bounded time to land before the
         // shared memory is reused or released
@@ -297,9 +300,8 @@ moment2_small_reduce_kernel(const float *__restrict__ partials, float *__restric
     // computes the tiles below the diagonal and discards them here); the padding of the last column blocks
     const bool use = y >= 0 && !((x == y && i8 > j8) || (dense && x > y)) && ci < d && cj < d;
     const int64_t at = tri_encode(d, ci < cj ? ci : cj, ci < cj ? cj : ci);
-    // launched as a programmatic dependent of the kernel that writes the partial sums: the launch overlaps
-    // that kernel's tail, and nothing is read before it has completed
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
+    pdl_trigger();
     const size_t stride = (size_t)nitems * 128;
     float s = 0.f;
     for (int k0 = warp; k0 < slices; k0 += 8 * 20) {   // 148 slices: one batch
@@ -384,32 +386,13 @@ st_status moment2_small(const float *X, int64_t N, int64_t d, int64_t ldx, float
     a.status = (unsigned *)ws;
     a.bar_floats = (int)(p.data_bytes / sizeof(float));
     a.dense = (flags & ST_FLAG_DENSE_CONTROL) ? 1 : 0;
-    if (d % 4 == 0 && ldx % 4 == 0) {
-        if (!ensure_dynamic_smem(moment2_small_kernel<true>, p.smem)) return ST_ERR_CUDA;
-        moment2_small_kernel<true><<<p.slices, p.threads, p.smem, stream>>>(a);
-    } else {
-        if (!ensure_dynamic_smem(moment2_small_kernel<false>, p.smem)) return ST_ERR_CUDA;
-        moment2_small_kernel<false><<<p.slices, p.threads, p.smem, stream>>>(a);
-    }
-    if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
-    const int n = p.nitems * 128;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n / 32));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const float *partials = a.partials;
-    const int di = (int)d, dense = a.dense;
-    if (cudaLaunchKernelEx(&cfg, moment2_small_reduce_kernel, partials, out, di, p.nbk, p.slices, dense, p.nitems) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ST_ERR_CUDA;
-    }
-    return ST_OK;
+    auto run = [&](auto kernel) {
+        if (!ensure_dynamic_smem(kernel, p.smem)) return ST_ERR_CUDA;
+        return launch(kernel, p.slices, p.threads, p.smem, stream, a);
+    };
+    const st_status rc = (d % 4 == 0 && ldx % 4 == 0) ? run(moment2_small_kernel<true>) : run(moment2_small_kernel<false>);
+    if (rc != ST_OK) return rc;
+    return launch(moment2_small_reduce_kernel, (unsigned)(p.nitems * 128 / 32), 256, 0, stream, a.partials, out, (int)d, p.nbk, p.slices, a.dense, p.nitems);
 }
 
 }  // namespace st

@@ -134,12 +134,6 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             mbar_init(&acc_empty[b], 8);     // four epilogue warps in each of the two blocks (leader's copy is used)
         }
         *abort_flag = 0;
-        if (blockIdx.x == 0) {
-            // the status words are cleared here instead of by a separate memset; a time-out
-            // report can only be written 2^24 failed polls later
-            a.status[kWsStatusWord] = 0;
-            a.status[kWsDetailWord] = 0;
-        }
         fence_barrier_init();
     }
     if (warp == 1) {
@@ -151,7 +145,14 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     cluster_sync_all();                      // both blocks' barriers exist before anything is signalled across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // the kernel that writes the operand may still be running
+    pdl_wait();
+    pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // the status words are cleared here instead of by a separate memset; a time-out
+        // report can only be written 2^24 failed polls later
+        a.status[kWsStatusWord] = 0;
+        a.status[kWsDetailWord] = 0;
+    }
 
     if (warp == 0) {
         // ---------------- TMA producer (both blocks): own boxes, completion counted on the leader's barrier
@@ -248,7 +249,6 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             const int buf = ph & 1;
             if (!mbar_wait(&acc_full[buf], (uint32_t)((ph >> 1) & 1), abort_flag, a.status, 3)) break;
             tc_fence_after();
-            if (ph == nphases - 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             if (rows) {
 #pragma unroll 1
                 for (int c0 = c_first; c0 < width; c0 += 32) {
@@ -303,7 +303,8 @@ moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__
     const int per = 8 / wps, w0 = warp % wps;
     const size_t stride = (size_t)2 * HALF * BN;
     constexpr int BATCH = V == 1 ? 10 : 4;
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as a programmatic dependent of the main kernel
+    pdl_wait();
+    pdl_trigger();
     int buf = 0;
     for (int u0 = blockIdx.y * per; u0 < rows * uw; u0 += gridDim.y * per) {
         const int u = u0 + warp / wps, r = u / uw, c = (u - r * uw) * (32 * V) + V * lane;   // this thread's columns c .. c+V-1
@@ -460,10 +461,10 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // behind the pass that writes a split operand or pair features
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = (MODE == M2_SPLIT || npairs > 0) ? 2 : 1;
+    cfg.numAttrs = 2;
     if (cudaLaunchKernelEx(&cfg, moment2_tc_kernel<MODE>, tmap, a) != cudaSuccess) {
         (void)cudaGetLastError();
         return ST_ERR_CUDA;
@@ -471,19 +472,9 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     int most = 0;                                                         // sample ranges of a tile
     for (int t = 0; t < q.tab.ntiles; ++t) most = q.tab.first[t + 1] - q.tab.first[t] > most ? q.tab.first[t + 1] - q.tab.first[t] : most;
     const unsigned blocks = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
-    cudaLaunchConfig_t rcfg = {};
-    rcfg.gridDim = dim3((unsigned)q.tab.ntiles, blocks < 64 ? 64 : blocks > 1024 ? 1024 : blocks);
-    rcfg.blockDim = dim3(256);
-    rcfg.stream = stream;
-    rcfg.attrs = attr + 1;
-    rcfg.numAttrs = 1;
+    const dim3 rgrid((unsigned)q.tab.ntiles, blocks < 64 ? 64 : blocks > 1024 ? 1024 : blocks);
     auto reduce = [&](auto kernel) {
-        const float *cpart = partials;
-        if (cudaLaunchKernelEx(&rcfg, kernel, cpart, out, (int)d, npairs, npairs > 0 ? simplex : tri_rows(d), rowmap, q.tab) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return ST_ERR_CUDA;
-        }
-        return ST_OK;
+        return launch(kernel, rgrid, 256, 0, stream, partials, out, (int)d, npairs, npairs > 0 ? simplex : tri_rows(d), rowmap, q.tab);
     };
     if (most <= 4) return npairs > 0 ? reduce(moment2_tc_reduce_kernel<true, 4>) : reduce(moment2_tc_reduce_kernel<false, 4>);
     return npairs > 0 ? reduce(moment2_tc_reduce_kernel<true, 1>) : reduce(moment2_tc_reduce_kernel<false, 1>);
@@ -554,6 +545,8 @@ __global__ void __launch_bounds__(256)
 moment2_split_rows_kernel(const float *__restrict__ X, int64_t N, int64_t Np, int d, int64_t ldx, __nv_bfloat16 *__restrict__ Z)
 {
     // Z: [2 Np, d]; rows 0 .. Np-1 hi, rows Np .. 2Np-1 lo; rows N .. Np-1 of either part are zero
+    pdl_wait();
+    pdl_trigger();
     const int64_t quads = (int64_t)Np * (d / 4);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < quads; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t n = e / (d / 4);
@@ -568,7 +561,6 @@ moment2_split_rows_kernel(const float *__restrict__ X, int64_t N, int64_t Np, in
         *reinterpret_cast<uint2 *>(Z + (Np + n) * d + c) =
             make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
     }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tile kernel may be launched; it waits for this grid to end
 }
 
 struct M2SplitPlan {
@@ -611,8 +603,8 @@ st_status moment2_split_tc(const float *X, int64_t N, int64_t d, int64_t ldx, fl
     const int64_t quads = p.Np * (d / 4);
     const int64_t want = (quads + 255) / 256;
     const int64_t cap = (int64_t)sm_count_or_default() * 16;
-    moment2_split_rows_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, stream>>>(X, N, p.Np, (int)d, ldx, Z);
-    if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
+    const st_status rc = launch(moment2_split_rows_kernel, (unsigned)(want < cap ? want : cap), 256, 0, stream, X, N, p.Np, (int)d, ldx, Z);
+    if (rc != ST_OK) return rc;
     return m2tc_launch<M2_SPLIT>(p.q, Z, 2 * p.Np, d, d, out, (float *)((unsigned char *)ws + p.part_off), (unsigned *)ws, stream, (int)p.Np);
 }
 

@@ -158,6 +158,8 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
     const float *__restrict__ X = a.X;
     const int64_t N = a.N, ldx = a.ldx, rows_per_slice = a.rows_per_slice;
     const int d = a.d, dp = DC > 0 ? DC : a.dp, out_elems = a.out_elems;
+    pdl_wait();
+    pdl_trigger();
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {   // this kernel has no bounded waits: the status is "ok"
         a.status[kWsStatusWord] = 0;
         a.status[kWsDetailWord] = 0;
@@ -250,7 +252,6 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
         }
     }
     cp_async_wait<0>();
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the slice sums may be launched; they wait for this grid to end
 
     if (rg > 1) {
         // red[sum][row group][table thread]; row group g adds and stores sums g, g + rg, ...
@@ -309,9 +310,8 @@ __global__ void __launch_bounds__(32 * SUM_GROUPS)
 sum_slices_kernel(const float *__restrict__ partials, float *__restrict__ out, int64_t elems, int slices)
 {
     __shared__ float part[SUM_GROUPS][32];
-    // launched as a programmatic dependent of the kernel that writes the partial sums: the launch itself
-    // overlaps that kernel's tail, and nothing is read before that kernel has completed
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int64_t e = (int64_t)blockIdx.x * 32 + lane;
     float s = 0.f;
@@ -336,25 +336,6 @@ sum_slices_kernel(const float *__restrict__ partials, float *__restrict__ out, i
         for (int w = 1; w < SUM_GROUPS; ++w) t += part[w][lane];
         out[e] = t;
     }
-}
-
-st_status sum_slices_launch(const float *partials, float *out, int64_t elems, int slices, cudaStream_t stream)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((elems + 31) / 32));
-    cfg.blockDim = dim3(32 * SUM_GROUPS);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, sum_slices_kernel, partials, out, elems, slices) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ST_ERR_CUDA;
-    }
-    return ST_OK;
 }
 
 // ---- host side: tile table ------------------------------------------------------------
@@ -596,19 +577,15 @@ static st_status moment3_launch(const float *X, int64_t N, int64_t d, int64_t ld
         a.gtile = gt;
         a.gvariant = gv;
     }
-    dim3 grid(p.groups, p.slices);
-    if (!aligned) {
-        if (!ensure_dynamic_smem(moment3_kernel<WARPS, 0, false>, p.smem)) return ST_ERR_CUDA;
-        moment3_kernel<WARPS, 0, false><<<grid, M3_THREADS, p.smem, stream>>>(a, *param);
-    } else if (p.dp == M3_PARAM_D) {   // d = 60, 64 has its own instance with compile-time strides
-        if (!ensure_dynamic_smem(moment3_kernel<WARPS, M3_PARAM_D, true>, p.smem)) return ST_ERR_CUDA;
-        moment3_kernel<WARPS, M3_PARAM_D, true><<<grid, M3_THREADS, p.smem, stream>>>(a, *param);
-    } else {
-        if (!ensure_dynamic_smem(moment3_kernel<WARPS, 0, true>, p.smem)) return ST_ERR_CUDA;
-        moment3_kernel<WARPS, 0, true><<<grid, M3_THREADS, p.smem, stream>>>(a, *param);
-    }
-    if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
-    return sum_slices_launch(a.partials, out, p.out_elems, p.slices, stream);
+    auto run = [&](auto kernel) {
+        if (!ensure_dynamic_smem(kernel, p.smem)) return ST_ERR_CUDA;
+        return launch(kernel, dim3(p.groups, p.slices), M3_THREADS, p.smem, stream, a, *param);
+    };
+    // d = 60, 64 has its own instance with compile-time strides
+    const st_status rc = !aligned ? run(moment3_kernel<WARPS, 0, false>)
+                       : p.dp == M3_PARAM_D ? run(moment3_kernel<WARPS, M3_PARAM_D, true>) : run(moment3_kernel<WARPS, 0, true>);
+    if (rc != ST_OK) return rc;
+    return launch(sum_slices_kernel, dim3((unsigned)((p.out_elems + 31) / 32)), 32 * SUM_GROUPS, 0, stream, a.partials, out, p.out_elems, p.slices);
 }
 
 size_t moment3_tc_workspace(int64_t N, int64_t d, bool bf16);

@@ -126,10 +126,6 @@ moment3_tc_kernel(const __grid_constant__ Args a)
         mbar_init(acc_full, MMA_WARPS);
         mbar_init(iss_sync, MMA_WARPS);
         *abort_flag = 0;
-        if (blockIdx.x == 0 && blockIdx.y == 0) {
-            a.status[kWsStatusWord] = 0;
-            a.status[kWsDetailWord] = 0;
-        }
         fence_barrier_init();
     }
     if (warp == MMA_WARP) {
@@ -140,6 +136,12 @@ moment3_tc_kernel(const __grid_constant__ Args a)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
+    pdl_trigger();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        a.status[kWsStatusWord] = 0;
+        a.status[kWsDetailWord] = 0;
+    }
 
     const int64_t n_begin = (int64_t)blockIdx.y * a.rows_per_slice;
     int64_t n_end = n_begin + a.rows_per_slice;
@@ -215,7 +217,6 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             if (as >= NA) { as -= NA; ++use; }
         }
 
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the slice sums may be launched; they wait for this grid to end
         // ---- epilogue: tensor memory -> this slice's partial sums ---------------------------------
         if (nstages > 0 && mbar_wait(acc_full, 0u, abort_flag, a.status, 13)) {
             tc_fence_after();
@@ -420,7 +421,8 @@ moment3_tc_sum_kernel(const __grid_constant__ SumArgs a)
     const int r = (e - t.part) % BM, k = TJ * t.jb + (e - t.part) / BM;
     const int i = TI * t.ib + r / TJ, j = TJ * t.jb + r % TJ;
     const bool use = i <= j && j <= k && k < a.d;
-    asm volatile("griddepcontrol.wait;" ::: "memory");     // launched as a programmatic dependent of the main kernel
+    pdl_wait();
+    pdl_trigger();
     float s = 0.f;
     if (use) {
         constexpr int BATCH = 10;
@@ -528,14 +530,12 @@ st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *o
         a.ntiles[g] = p.ntiles[g];
         for (int t = 0; t < MAX_GROUP_TILES; ++t) a.tiles[g][t] = p.tiles[g][t];
     }
-    if (bf16) {
-        if (!ensure_dynamic_smem(moment3_tc_kernel<true>, smem_bytes(p.dcols, true))) return ST_ERR_CUDA;
-        moment3_tc_kernel<true><<<dim3(p.groups, p.slices), THREADS, smem_bytes(p.dcols, true), stream>>>(a);
-    } else {
-        if (!ensure_dynamic_smem(moment3_tc_kernel<false>, smem_bytes(p.dcols, false))) return ST_ERR_CUDA;
-        moment3_tc_kernel<false><<<dim3(p.groups, p.slices), THREADS, smem_bytes(p.dcols, false), stream>>>(a);
-    }
-    if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
+    auto run = [&](auto kernel) {
+        if (!ensure_dynamic_smem(kernel, smem_bytes(p.dcols, bf16))) return ST_ERR_CUDA;
+        return launch(kernel, dim3(p.groups, p.slices), THREADS, smem_bytes(p.dcols, bf16), stream, a);
+    };
+    const st_status rc = bf16 ? run(moment3_tc_kernel<true>) : run(moment3_tc_kernel<false>);
+    if (rc != ST_OK) return rc;
     SumArgs m;
     m.partials = a.partials;
     m.out = out;
@@ -544,21 +544,7 @@ st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *o
     m.d = (int)d;
     m.ntiles = p.ntiles[0] + p.ntiles[1];
     for (int t = 0; t < m.ntiles; ++t) m.tiles[t] = t < p.ntiles[0] ? p.tiles[0][t] : p.tiles[1][t - p.ntiles[0]];
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.part_elems / 32));
-    cfg.blockDim = dim3(32 * SUM_WARPS);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, moment3_tc_sum_kernel, m) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ST_ERR_CUDA;
-    }
-    return ST_OK;
+    return launch(moment3_tc_sum_kernel, (unsigned)(p.part_elems / 32), 32 * SUM_WARPS, 0, stream, m);
 }
 
 }  // namespace st

@@ -91,6 +91,8 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
 {
     extern __shared__ __align__(16) float xs[];                       // 2 x [EXP_ROWS][d + 1], column d is zero
     const int pitch = d + 1;
+    pdl_wait();
+    pdl_trigger();
     // gridDim.x = column groups, gridDim.y = row groups
     const int p = (blockIdx.x * EXP_THREADS + threadIdx.x) * 4;       // this thread's columns p .. p+3
     int ci[4], cj[4];
@@ -163,7 +165,6 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
             }
         }
     }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tile kernel may be launched; it waits for this grid to end
 }
 
 // One block per unique pair (i,j): the entries (i,j,k,l), j <= k <= l, follow each other in the 4-simplex in the
@@ -173,6 +174,8 @@ __global__ void __launch_bounds__(128)
 simplex_gather_kernel(const float *__restrict__ M2, float *__restrict__ out, int d, int64_t dP, unsigned *status,
                       const unsigned *inner_status)
 {
+    pdl_wait();
+    pdl_trigger();
     // the second-moment step ran on its own part of the workspace: its status becomes the call's
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         status[kWsStatusWord] = inner_status[kWsStatusWord];
@@ -229,23 +232,19 @@ extern "C" st_status st_sym_moment4(const float *X, int64_t N, int64_t d, int64_
         constexpr bool SP = decltype(split_tag)::value;
         T *dst = (T *)(w + p.off_p);
         if (d + 1 <= 64)
-            pair_expand_kernel<T, SP, 2><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
-        else if (d + 1 <= 96)
-            pair_expand_kernel<T, SP, 3><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
-        else
-            pair_expand_kernel<T, SP, 5><<<grid, EXP_THREADS, smem, stream>>>(X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
+            return launch(pair_expand_kernel<T, SP, 2>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
+        if (d + 1 <= 96)
+            return launch(pair_expand_kernel<T, SP, 3>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
+        return launch(pair_expand_kernel<T, SP, 5>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
     };
-    if (p.split) expand(__nv_bfloat16(), std::true_type());
-    else if (p.bf16) expand(__nv_bfloat16(), std::false_type());
-    else expand(float(), std::false_type());
-    if (cudaGetLastError() != cudaSuccess) return ST_ERR_CUDA;
+    st_status rc = p.split ? expand(__nv_bfloat16(), std::true_type())
+                 : p.bf16 ? expand(__nv_bfloat16(), std::false_type()) : expand(float(), std::false_type());
+    if (rc != ST_OK) return rc;
     if (p.split || p.bf16)
         return moment2_pairs_tc(w + p.off_p, N, p.dP, npairs, p.split, rowmap, simp4_rows(d), out_packed, (float *)(w + p.off_ws), (unsigned *)w,
                                 stream);
     float *M2 = (float *)(w + p.off_m2);
-    const st_status rc = st_sym_moment2(w + p.off_p, ST_F32, N, p.dP, p.dP, M2, w + p.off_ws, p.m2_ws, 0, stream_);
+    rc = st_sym_moment2(w + p.off_p, ST_F32, N, p.dP, p.dP, M2, w + p.off_ws, p.m2_ws, 0, stream_);
     if (rc != ST_OK) return rc;
-    simplex_gather_kernel<<<(unsigned)npairs, 128, 0, stream>>>(M2, out_packed, (int)d, p.dP, (unsigned *)w,
-                                                                (const unsigned *)(w + p.off_ws));
-    return launch_status();
+    return launch(simplex_gather_kernel, (unsigned)npairs, 128, 0, stream, M2, out_packed, (int)d, p.dP, (unsigned *)w, (const unsigned *)(w + p.off_ws));
 }

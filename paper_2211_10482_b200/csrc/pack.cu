@@ -159,6 +159,8 @@ slice_copy_kernel(const unsigned char *__restrict__ src, unsigned char *__restri
                   int part_bytes, const unsigned char *__restrict__ mul)
 {
     // MUL (pack only, fp32 elements): a second packed operand; the gathered values are multiplied by it
+    pdl_wait();
+    pdl_trigger();
     const int g = 1 << group_shift;
     const int lane = (int)(threadIdx.x & (g - 1));
     const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> group_shift;
@@ -228,6 +230,8 @@ sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restric
                  int row_bytes, int group_shift, int64_t packed_rows)
 {
     typedef typename Elem<ES>::T E;
+    pdl_wait();
+    pdl_trigger();
     const int lane = (int)(threadIdx.x & 31);
     const I nitems = nslices * (I)parts, nwarps = (I)gridDim.x * (I)(blockDim.x / 32);
     for (I item = (I)blockIdx.x * (I)(blockDim.x / 32) + (I)(threadIdx.x / 32); item < nitems; item += nwarps) {
@@ -283,6 +287,8 @@ sym_tile_kernel(const typename Elem<ES>::T *__restrict__ packed, typename Elem<E
 {
     typedef typename Elem<ES>::T E;
     __shared__ E tile[32][33];
+    pdl_wait();
+    pdl_trigger();
     const unsigned i1 = blockIdx.y, i2 = blockIdx.z;       // leading indices
     if (KIND == ST_SIMPLEX4 && i1 > i2) return;
     int64_t bi64, bj64;
@@ -337,6 +343,8 @@ template <int OP>
 __global__ void __launch_bounds__(256)
 packed_binary_kernel(const float *a, const float *b, float *out, int64_t n, float alpha, float beta)
 {
+    pdl_wait();
+    pdl_trigger();
     const int64_t n4 = n >> 2;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n4; e += stride) {
@@ -407,8 +415,7 @@ static st_status launch_sym(const void *src, void *dst, const LayoutArgs &a, cud
     if (a.row_bytes == ES && small) {
         const unsigned nt = (unsigned)((a.d + 31) / 32);
         const dim3 grid(nt * (nt + 1) / 2, KIND == ST_TRI_UPPER ? 1u : (unsigned)a.d, KIND == ST_SIMPLEX4 ? (unsigned)a.d : 1u);
-        sym_tile_kernel<KIND, ES><<<grid, 256, 0, s>>>((const E *)src, (E *)dst, (unsigned)a.d, nt, a.packed_rows);
-        return launch_status();
+        return launch(sym_tile_kernel<KIND, ES>, grid, 256, 0, s, (const E *)src, (E *)dst, (unsigned)a.d, nt, a.packed_rows);
     }
     if (a.row_bytes > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
     // parts of about 2 KiB, a multiple of 32 positions where a lane takes one each
@@ -422,12 +429,10 @@ static st_status launch_sym(const void *src, void *dst, const LayoutArgs &a, cud
     const unsigned char *in = (const unsigned char *)src;
     unsigned char *out = (unsigned char *)dst;
     if (small && items < (int64_t(1) << 31))
-        sym_slice_kernel<KIND, ES, unsigned><<<grid, 256, 0, s>>>(in, out, (unsigned)a.d, (unsigned)nslices, (int)parts, (int)part_rows,
-                                                                   (int)a.row_bytes, shift, a.packed_rows);
-    else
-        sym_slice_kernel<KIND, ES, int64_t><<<grid, 256, 0, s>>>(in, out, a.d, nslices, (int)parts, (int)part_rows, (int)a.row_bytes,
-                                                                  shift, a.packed_rows);
-    return launch_status();
+        return launch(sym_slice_kernel<KIND, ES, unsigned>, grid, 256, 0, s, in, out, (unsigned)a.d, (unsigned)nslices, (int)parts, (int)part_rows,
+                      (int)a.row_bytes, shift, a.packed_rows);
+    return launch(sym_slice_kernel<KIND, ES, int64_t>, grid, 256, 0, s, in, out, a.d, nslices, (int)parts, (int)part_rows, (int)a.row_bytes, shift,
+                  a.packed_rows);
 }
 
 template <int KIND, int ES, bool PACK>
@@ -450,17 +455,12 @@ static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cu
     const int64_t nslices = (KIND == ST_TET) ? a.d * a.d : (KIND == ST_SIMPLEX4) ? a.d * a.d * a.d : a.d;
     const int64_t threads = (nslices * parts) << shift;
     const int64_t want = (threads + 255) / 256;
-    const int grid = (int)(want < cap ? (want < 1 ? 1 : want) : cap);
+    const unsigned grid = (unsigned)(want < cap ? (want < 1 ? 1 : want) : cap);
     const unsigned char *in = (const unsigned char *)src, *m = (const unsigned char *)mul;
     unsigned char *out = (unsigned char *)dst;
-    if constexpr (PACK && ES == 4) {
-        if (mul) {
-            slice_copy_kernel<KIND, ES, PACK, true><<<grid, 256, 0, s>>>(in, out, a, shift, (int)parts, (int)pb, m);
-            return launch_status();
-        }
-    }
-    slice_copy_kernel<KIND, ES, PACK, false><<<grid, 256, 0, s>>>(in, out, a, shift, (int)parts, (int)pb, m);
-    return launch_status();
+    if constexpr (PACK && ES == 4)
+        if (mul) return launch(slice_copy_kernel<KIND, ES, PACK, true>, grid, 256, 0, s, in, out, a, shift, (int)parts, (int)pb, m);
+    return launch(slice_copy_kernel<KIND, ES, PACK, false>, grid, 256, 0, s, in, out, a, shift, (int)parts, (int)pb, m);
 }
 
 template <int ES, bool PACK>
@@ -538,9 +538,7 @@ static st_status packed_binary(int op, int64_t n, const float *a, const float *b
     if (!st::aligned16(a) || !st::aligned16(b) || !st::aligned16(out)) return ST_ERR_ALIGN;
     const int64_t want = (n / 4 + 255) / 256, cap = (int64_t)st::sm_count_or_default() * 16;
     const unsigned grid = (unsigned)(want < 1 ? 1 : (want < cap ? want : cap));
-    if (op == 0) st::packed_binary_kernel<0><<<grid, 256, 0, (cudaStream_t)stream>>>(a, b, out, n, alpha, beta);
-    else st::packed_binary_kernel<1><<<grid, 256, 0, (cudaStream_t)stream>>>(a, b, out, n, alpha, beta);
-    return st::launch_status();
+    return st::launch(op == 0 ? st::packed_binary_kernel<0> : st::packed_binary_kernel<1>, grid, 256, 0, (cudaStream_t)stream, a, b, out, n, alpha, beta);
 }
 
 st_status st_packed_axpby(int64_t n, float alpha, const float *a, float beta, const float *b, float *out, void *stream)

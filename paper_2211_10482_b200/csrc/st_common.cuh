@@ -94,9 +94,34 @@ inline bool ensure_dynamic_smem(Kernel kernel, size_t bytes)
     return true;
 }
 
-inline st_status launch_status()
+// Every kernel is launched as a programmatic dependent of whatever precedes it in the stream: its blocks may be placed and
+// set up while the kernel before it finishes, which hides one to two microseconds per launch in a chain of short calls.
+// For that every block of every kernel calls pdl_wait() before its first access to global memory (it returns when all
+// kernels before this one have completed and their writes are visible), and pdl_trigger() once the next kernel's blocks
+// may be placed: after its own TMEM allocation, where it has one.
+#if defined(__CUDACC__)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+inline st_status launch(void (*kernel)(Params...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, Args... args)
 {
-    return cudaGetLastError() == cudaSuccess ? ST_OK : ST_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, (Params)args...) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ST_ERR_CUDA;
+    }
+    return ST_OK;
 }
+#endif
 
 }  // namespace st

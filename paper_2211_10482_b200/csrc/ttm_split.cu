@@ -110,10 +110,6 @@ __global__ void __launch_bounds__(split::THREADS, 1) ttm_split_kernel(const Spli
             mbar_init(&acc_empty[b], EPI_WARPS);
         }
         *abort_flag = 0;
-        if (blockIdx.x == 0) {      // a time-out report can only be written 2^24 failed polls later
-            a.status[kWsStatusWord] = 0;
-            a.status[kWsDetailWord] = 0;
-        }
         fence_barrier_init();
     }
     if (warp == MMA_WARP) {
@@ -124,6 +120,14 @@ __global__ void __launch_bounds__(split::THREADS, 1) ttm_split_kernel(const Spli
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
+    pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // the status words are cleared here instead of by a separate memset; a time-out
+        // report can only be written 2^24 failed polls later
+        a.status[kWsStatusWord] = 0;
+        a.status[kWsDetailWord] = 0;
+    }
 
     const int my_tiles = (a.ntiles > (int)blockIdx.x) ? (a.ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int R = a.R;
@@ -320,8 +324,6 @@ __global__ void __launch_bounds__(split::THREADS, 1) ttm_split_kernel(const Spli
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    // MTTKRP: the kernel that adds the partial sums may be launched now (it waits for this grid to end)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     if (warp == MMA_WARP) {
@@ -376,12 +378,10 @@ static st_status split_rows_launch(const float *Bp, int64_t rows, int64_t K, con
     const int grid = a.ntiles < di.sm_count ? a.ntiles : di.sm_count;
     if (p.land == 3) {
         if (!ensure_dynamic_smem(ttm_split_kernel<3>, p.smem)) return ST_ERR_CUDA;
-        ttm_split_kernel<3><<<grid, THREADS, p.smem, stream>>>(a);
-    } else {
-        if (!ensure_dynamic_smem(ttm_split_kernel<2>, p.smem)) return ST_ERR_CUDA;
-        ttm_split_kernel<2><<<grid, THREADS, p.smem, stream>>>(a);
+        return launch(ttm_split_kernel<3>, grid, THREADS, p.smem, stream, a);
     }
-    return launch_status();
+    if (!ensure_dynamic_smem(ttm_split_kernel<2>, p.smem)) return ST_ERR_CUDA;
+    return launch(ttm_split_kernel<2>, grid, THREADS, p.smem, stream, a);
 }
 
 size_t ttm_split_workspace(int64_t rows, int64_t K, int64_t R)

@@ -72,12 +72,6 @@ ttm_tc_kernel(const __grid_constant__ CUtensorMap tmap, const TtmTcArgs a)
             mbar_init(&acc_empty[b], 4);     // one arrival per epilogue warp
         }
         *abort_flag = 0;
-        if (blockIdx.x == 0) {
-            // the status words are cleared here instead of by a separate memset; a time-out
-            // report can only be written 2^24 failed polls later
-            a.status[kWsStatusWord] = 0;
-            a.status[kWsDetailWord] = 0;
-        }
         fence_barrier_init();
     }
     if (warp == 1) {
@@ -88,6 +82,14 @@ ttm_tc_kernel(const __grid_constant__ CUtensorMap tmap, const TtmTcArgs a)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
+    pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // the status words are cleared here instead of by a separate memset; a time-out
+        // report can only be written 2^24 failed polls later
+        a.status[kWsStatusWord] = 0;
+        a.status[kWsDetailWord] = 0;
+    }
 
     if (warp != 0) {
         // Warps 1..5 build U^T while warp 0 already streams fibres: U rounded to TF32, K-major with
@@ -217,8 +219,6 @@ ttm_tc_kernel(const __grid_constant__ CUtensorMap tmap, const TtmTcArgs a)
             if (lane == 0) mbar_arrive(&acc_empty[buf]);
         }
     }
-    // MTTKRP: the kernel that adds the partial sums may be launched now (it waits for this grid to end)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -325,8 +325,7 @@ static st_status tc_rows_launch(const float *Bp, int64_t rows, int64_t K, const 
     a.reverse = mode != TC_TTM ? 1 : 0;
     if (!ensure_dynamic_smem(ttm_tc_kernel, p.smem)) return ST_ERR_CUDA;
     const int grid = a.ntiles < di.sm_count ? a.ntiles : di.sm_count;
-    ttm_tc_kernel<<<grid, THREADS, p.smem, stream>>>(tmap, a);
-    return launch_status();
+    return launch(ttm_tc_kernel, grid, THREADS, p.smem, stream, tmap, a);
 }
 
 }  // namespace st

@@ -1152,3 +1152,43 @@ def test_thp_and_ttm_packed_at_the_benchmark_size(st):
     rows = np.unique(np.concatenate([[0, 511, 512, Bp.shape[0] - 1], rng.integers(0, Bp.shape[0], 300)]))
     T, S = oracle.ttm(Bp[rows], U)
     assert oracle.rel_err(A[rows], T, S) <= 5e-3
+
+
+@pytest.mark.parametrize("N,d", [(5000, 40), (300, 80)])
+def test_dependent_launches_keep_the_order_of_two_streams_and_a_graph(st, N, d):
+    """Every kernel may be placed before the one in front of it has finished: inputs written just before by other work, by
+    another stream or by the library itself must be complete when they are read, eagerly and in a captured graph."""
+    X = dev(workloads.draw((N, d), "normal", 5))
+    lay = st.Layout(st.ST_TRI_UPPER, d)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    want = [st.st_unpack(st.st_sym_moment2(2 * X), lay, st.ST_FILL_SYMMETRIC), st.st_sym_moment3(X)]
+    torch.cuda.synchronize()
+
+    def work():
+        Y = torch.zeros_like(X)
+        Y.copy_(X)
+        there, back = torch.cuda.Event(), torch.cuda.Event()
+        there.record(s1)
+        s2.wait_event(there)
+        with torch.cuda.stream(s2):
+            Z = Y * 2
+            third = st.st_sym_moment3(Y)
+            back.record(s2)
+        s1.wait_event(back)
+        return st.st_unpack(st.st_sym_moment2(Z), lay, st.ST_FILL_SYMMETRIC), third
+
+    st.set_allocator(None)          # a captured graph has its own pool
+    try:
+        with torch.cuda.stream(s1):
+            eager = [work() for _ in range(3)]
+            s1.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=s1):
+                captured = work()
+            for _ in range(3):
+                graph.replay()
+            s1.synchronize()
+    finally:
+        st.set_allocator(GuardAllocator())
+    for got in eager + [captured]:
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
