@@ -405,17 +405,26 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
     p.stages = (int)((n == 1 ? STAGES_BYTES_1 : STAGES_BYTES) / stage);
     if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
     p.smem = (size_t)p.stages * stage + (size_t)(S::NBOX - p.na) * S::BOX_BYTES + 1024 + 512;
-    // Clusters (one per pair of SMs) are dealt one by one to the tile whose share of the samples takes longest; then every
-    // tile gives back what it does not need to keep up with the slowest.  Tiles of equal width so get equal shares: their
-    // clusters run in step and share X in L2 (with unequal shares the wide case was 12-20% slower on more SMs).
+    // Clusters (one per pair of SMs) go to the tiles in proportion to their cost, the remaining ones each to the tile whose
+    // share of the samples takes longest; then every tile gives back what it does not need to keep up with the slowest.
+    // Tiles of equal width so get equal shares: their clusters run in step and share X in L2 (with unequal shares the wide
+    // case was 12-20% slower on more SMs).
     int split[MAX_TILES];
-    int64_t left = sm_count_or_default() / 2 - n;
-    for (int i = 0; i < n; ++i) split[i] = 1;
+    const int clusters = sm_count_or_default() / 2;
+    double sum = 0;
+    for (int i = 0; i < n; ++i) sum += cost[i];
+    int64_t left = clusters;
+    for (int i = 0; i < n; ++i) {
+        int64_t k = (int64_t)(cost[i] * clusters / sum);
+        k = k < 1 ? 1 : k > chunks ? chunks : k;
+        split[i] = (int)k;
+        left -= k;
+    }
     double longest = 0;
     for (;;) {
         int worst = 0;
         for (int i = 1; i < n; ++i)
-            if (cost[i] / split[i] > cost[worst] / split[worst]) worst = i;
+            if (cost[i] * split[worst] > cost[worst] * split[i]) worst = i;
         longest = cost[worst] / split[worst];
         if (left <= 0 || split[worst] >= chunks) break;
         ++split[worst];

@@ -17,13 +17,15 @@
 // 16-byte boundary.  copy_flat stores whole 16-byte units all the same and takes each from the two aligned units
 // that hold it (the second one is an L1 hit), shifted in registers.  Measured against copies in the widest unit that
 // divides a row, each position of a symmetric fill by itself (pack + unpack): tet d = 60, rows of 33 floats, 72 -> 24 us;
-// tri d = 900, rows of 17 bf16, 125 -> 27 us; simplex4 d = 50 floats, 87 -> 22 us; tet d = 175 bf16, 55 -> 17 us.
+// tri d = 900, rows of 17 bf16, 125 -> 21 us; simplex4 d = 64 floats, 220 -> 32 us; tet d = 200 bf16, 27 -> 9 us.
 #include "st_common.cuh"
 #include "st_index.cuh"
+#include <type_traits>
 
 namespace st {
 
 constexpr int COPY_UNITS = 4;              // 16-byte units that a thread of the slice copies has in flight
+constexpr int SYM_WORDS = 4;               // words that a lane of the symmetric fill has in flight
 constexpr int64_t PART_BYTES = 32768;      // most of a slice that one thread group copies ([384,384,75]: 128 KiB starve the chip)
 
 struct LayoutArgs {
@@ -40,6 +42,7 @@ template <int ES> struct Elem;
 template <> struct Elem<2> { typedef uint16_t T; };
 template <> struct Elem<4> { typedef uint32_t T; };
 template <> struct Elem<8> { typedef uint2 T; };
+template <> struct Elem<16> { typedef uint4 T; };
 
 // 16 bytes at byte `off` (a multiple of ES) of the two aligned units at p.
 template <int ES>
@@ -121,41 +124,84 @@ __device__ __forceinline__ void zero_flat(unsigned char *dst, int n, int lane, i
     for (int u = lane; u < units; u += g) out[u] = make_uint4(0, 0, 0, 0);
 }
 
-// Run of unique columns of slice s: dense columns [lo,hi) of the slice map to packed rows prow.. (contiguous).
-template <int KIND>
-__device__ __forceinline__ void slice_run(const LayoutArgs &a, int64_t s, int64_t &lo, int64_t &hi, int64_t &prow)
+// Closed forms of st_index.cuh in the index type I: unsigned where every index fits in 31 bits.
+template <typename I> __device__ __forceinline__ I tri_n(I d) { return d * (d + 1) / 2; }
+template <typename I> __device__ __forceinline__ I tet_n(I d) { return d * (d + 1) / 2 * (d + 2) / 3; }
+template <typename I> __device__ __forceinline__ I simp4_n(I d) { return tet_n<I>(d) * (d + 3) / 4; }
+template <typename I> __device__ __forceinline__ I tri_at(I d, I i, I j) { return i * (2 * d - i + 1) / 2 + (j - i); }
+template <typename I> __device__ __forceinline__ I tet_at(I d, I i, I j, I k) { return tet_n<I>(d) - tet_n<I>(d - i) + tri_at<I>(d - i, j - i, k - i); }
+template <typename I> __device__ __forceinline__ I simp4_at(I d, I i, I j, I k, I l) { return simp4_n<I>(d) - simp4_n<I>(d - i) + tet_at<I>(d - i, j - i, k - i, l - i); }
+template <typename I> __device__ __forceinline__ void tri_dec(I d, I p, I &i, I &j)
 {
+    const I b = 2 * d + 1;
+    const I root = (I)sqrtf((float)(b * b - 8 * p));
+    I ii = root < b ? (b - root) >> 1 : 0;
+    if (ii > d - 1) ii = d - 1;
+    while (ii > 0 && tri_at<I>(d, ii, ii) > p) --ii;
+    while (ii + 1 < d && tri_at<I>(d, ii + 1, ii + 1) <= p) ++ii;
+    i = ii;
+    j = ii + (p - tri_at<I>(d, ii, ii));
+}
+template <typename I> __device__ __forceinline__ void tet_dec(I d, I q, I &i, I &j, I &k)
+{
+    const I r = tet_n<I>(d) - q;                              // positions left; the slab of side m holds tet(m-1) < r <= tet(m)
+    I m = (I)cbrtf(6.0f * (float)r);
+    if (m < 1) m = 1;
+    if (m > d) m = d;
+    while (m > 1 && tet_n<I>(m - 1) >= r) --m;
+    while (m < d && tet_n<I>(m) < r) ++m;
+    i = d - m;
+    tri_dec<I>(m, tet_n<I>(m) - r, j, k);
+    j += i;
+    k += i;
+}
+
+// Run of unique columns of slice s: dense columns [lo,hi) of the slice map to packed rows prow.. (contiguous).
+// PACK of an order-3 or order-4 tensor visits the slices with a run only: item s is then the s-th of those, and s becomes
+// the number of its slice.
+template <int KIND, bool PACK, typename I>
+__device__ __forceinline__ void slice_run(const LayoutArgs &a, I &s, I &lo, I &hi, I &prow)
+{
+    const I d = (I)a.d, kl = (I)a.kl;
     if (KIND == ST_TRI_UPPER) {
-        lo = s; hi = a.d; prow = tri_row_start(a.d, s);
+        lo = s; hi = d; prow = tri_at<I>(d, s, s);
     } else if (KIND == ST_TET) {
-        const int64_t i = s / a.d, j = s - i * a.d;
+        I i, j;
+        if (PACK) { tri_dec<I>(d, s, i, j); s = i * d + j; }
+        else { i = s / d; j = s - i * d; }
         if (j < i) { lo = hi = 0; prow = 0; }
-        else { lo = j; hi = a.d; prow = tet_encode(a.d, i, j, j); }
+        else { lo = j; hi = d; prow = tet_at<I>(d, i, j, j); }
     } else if (KIND == ST_BAND) {
-        lo = s - a.kl; if (lo < 0) lo = 0;
-        hi = s + a.ku + 1; if (hi > a.d) hi = a.d;
+        lo = s > kl ? s - kl : 0;
+        hi = s + (I)a.ku + 1 < d ? s + (I)a.ku + 1 : d;
         if (hi < lo) hi = lo;
-        prow = s * a.width + (lo - (s - a.kl));
+        prow = s * (I)a.width + (lo + kl - s);
     } else if (KIND == ST_FIXED_ROW) {
-        if (s == a.kl) { lo = 0; hi = a.d; } else { lo = hi = 0; }
+        if (s == kl) { lo = 0; hi = d; } else { lo = hi = 0; }
         prow = 0;
     } else if (KIND == ST_FIXED_COL) {
-        lo = a.kl; hi = a.kl + 1; prow = s;
+        lo = kl; hi = kl + 1; prow = s;
     } else if (KIND == ST_SIMPLEX4) {
         // slice s = (i, j, k): its unique entries are l = k .. d-1 when i <= j <= k
-        const int64_t ij = s / a.d, k = s - ij * a.d;
-        const int64_t i = ij / a.d, j = ij - i * a.d;
-        if (i <= j && j <= k) { lo = k; hi = a.d; prow = simp4_encode(a.d, i, j, k, k); }
+        I i, j, k;
+        if (PACK) {
+            tet_dec<I>(d, s, i, j, k);
+            s = (i * d + j) * d + k;
+        } else {
+            const I ij = s / d;
+            k = s - ij * d; i = ij / d; j = ij - i * d;
+        }
+        if (i <= j && j <= k) { lo = k; hi = d; prow = simp4_at<I>(d, i, j, k, k); }
         else { lo = hi = 0; prow = 0; }
     } else {
-        const int64_t b = s / a.bs;
-        lo = b * a.bs; hi = lo + a.bs; prow = s * a.bs;
+        const I bs = (I)a.bs, b = s / bs;
+        lo = b * bs; hi = lo + bs; prow = s * bs;
     }
 }
 
-template <int KIND, int ES, bool PACK, bool MUL>
+template <int KIND, int ES, bool PACK, bool MUL, typename I>
 __global__ void __launch_bounds__(256)
-slice_copy_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst, LayoutArgs a, int group_shift, int parts,
+slice_copy_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst, LayoutArgs a, I nitems, int group_shift, int parts,
                   int part_bytes, const unsigned char *__restrict__ mul)
 {
     // MUL (pack only, fp32 elements): a second packed operand; the gathered values are multiplied by it
@@ -163,20 +209,18 @@ slice_copy_kernel(const unsigned char *__restrict__ src, unsigned char *__restri
     pdl_trigger();
     const int g = 1 << group_shift;
     const int lane = (int)(threadIdx.x & (g - 1));
-    const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> group_shift;
-    const int64_t ngroups = ((int64_t)gridDim.x * blockDim.x) >> group_shift;
-    const int64_t nslices = (KIND == ST_TET) ? a.d * a.d : (KIND == ST_SIMPLEX4) ? a.d * a.d * a.d : a.d;
+    const I gid = (I)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> group_shift);
+    const I ngroups = (I)(((int64_t)gridDim.x * blockDim.x) >> group_shift);
     const int64_t sb = a.d * a.row_bytes;                     // bytes per dense slice
-    for (int64_t item = gid; item < nslices * parts; item += ngroups) {
-        const int64_t s = parts == 1 ? item : item / parts;
-        const int64_t part = item - s * parts;
-        int64_t lo, hi, prow;
-        slice_run<KIND>(a, s, lo, hi, prow);
+    for (I item = gid; item < nitems; item += ngroups) {
+        I s = parts == 1 ? item : item / (I)parts, lo, hi, prow;
+        const int64_t part = item - s * (I)parts;
+        slice_run<KIND, PACK, I>(a, s, lo, hi, prow);
         // a non-empty run lies inside the slice and inside the packed array
         if (hi > lo && !(ST_BOUNDS_OK(lo, a.d, 1) && ST_BOUNDS_OK(hi - 1, a.d, 1) && ST_BOUNDS_OK(prow, a.packed_rows, 1) &&
-                         ST_BOUNDS_OK(prow + (hi - lo) - 1, a.packed_rows, 1)))
+                         ST_BOUNDS_OK((int64_t)prow + (hi - lo) - 1, a.packed_rows, 1)))
             continue;
-        const int64_t c0 = lo * a.row_bytes, c1 = hi * a.row_bytes;   // the run inside the slice
+        const int64_t c0 = (int64_t)lo * a.row_bytes, c1 = (int64_t)hi * a.row_bytes;   // the run inside the slice
         // pack splits the run itself into parts, unpack the whole dense slice (it writes all of it)
         const int64_t r0 = PACK ? c0 : 0, r1 = PACK ? c1 : sb;
         int64_t u0 = r0 + part * part_bytes;                  // this part covers dense bytes [u0, u1) of the slice
@@ -184,18 +228,18 @@ slice_copy_kernel(const unsigned char *__restrict__ src, unsigned char *__restri
         if (u0 > r1) u0 = r1;
         if (u1 > r1) u1 = r1;
         const int64_t x0 = u0 > c0 ? u0 : c0, x1 = u1 < c1 ? u1 : c1;   // run clipped to this part
-        const int64_t p0 = prow * a.row_bytes - c0;           // packed byte of dense byte 0 of the slice, were it in the run
+        const int64_t p0 = (int64_t)prow * a.row_bytes - c0;           // packed byte of dense byte 0 of the slice, were it in the run
         if (PACK) {
-            if (x1 > x0) copy_flat<ES, MUL, COPY_UNITS>(dst + p0 + x0, src + s * sb + x0, mul + p0 + x0, (int)(x1 - x0), lane, g);
+            if (x1 > x0) copy_flat<ES, MUL, COPY_UNITS>(dst + p0 + x0, src + (int64_t)s * sb + x0, mul + p0 + x0, (int)(x1 - x0), lane, g);
             if (KIND == ST_BAND && part == 0) {
                 // slots of the fixed-width packed row that fall outside the matrix
-                unsigned char *row = dst + s * a.width * a.row_bytes;
-                const int64_t first = (prow - s * a.width) * a.row_bytes, last = first + (c1 - c0), wb = a.width * a.row_bytes;
+                unsigned char *row = dst + (int64_t)s * a.width * a.row_bytes;
+                const int64_t first = ((int64_t)prow - (int64_t)s * a.width) * a.row_bytes, last = first + (c1 - c0), wb = a.width * a.row_bytes;
                 for (int64_t z = 0; z < first; z += part_bytes) zero_flat<ES>(row + z, (int)(first - z < part_bytes ? first - z : part_bytes), lane, g);
                 for (int64_t z = last; z < wb; z += part_bytes) zero_flat<ES>(row + z, (int)(wb - z < part_bytes ? wb - z : part_bytes), lane, g);
             }
         } else {
-            unsigned char *out = dst + s * sb;
+            unsigned char *out = dst + (int64_t)s * sb;
             const int64_t z1 = u1 < c0 ? u1 : c0;               // zeros before the run
             if (z1 > u0) zero_flat<ES>(out + u0, (int)(z1 - u0), lane, g);
             if (x1 > x0) copy_flat<ES, false, COPY_UNITS>(out + x0, src + p0 + x0, nullptr, (int)(x1 - x0), lane, g);
@@ -204,14 +248,6 @@ slice_copy_kernel(const unsigned char *__restrict__ src, unsigned char *__restri
         }
     }
 }
-
-// Closed forms of st_index.cuh in the index type I: unsigned where every index fits in 31 bits.
-template <typename I> __device__ __forceinline__ I tri_n(I d) { return d * (d + 1) / 2; }
-template <typename I> __device__ __forceinline__ I tet_n(I d) { return d * (d + 1) / 2 * (d + 2) / 3; }
-template <typename I> __device__ __forceinline__ I simp4_n(I d) { return tet_n<I>(d) * (d + 3) / 4; }
-template <typename I> __device__ __forceinline__ I tri_at(I d, I i, I j) { return i * (2 * d - i + 1) / 2 + (j - i); }
-template <typename I> __device__ __forceinline__ I tet_at(I d, I i, I j, I k) { return tet_n<I>(d) - tet_n<I>(d - i) + tri_at<I>(d - i, j - i, k - i); }
-template <typename I> __device__ __forceinline__ I simp4_at(I d, I i, I j, I k, I l) { return simp4_n<I>(d) - simp4_n<I>(d - i) + tet_at<I>(d - i, j - i, k - i, l - i); }
 
 // Packed row of position x of the slice whose fixed indices are a <= b <= c (as many as KIND has); x < the largest.
 template <int KIND, typename I>
@@ -222,12 +258,12 @@ __device__ __forceinline__ I sym_row(I d, I a, I b, I c, I x)
     return x < a ? simp4_at<I>(d, x, a, b, c) : x < b ? simp4_at<I>(d, a, x, b, c) : simp4_at<I>(d, a, b, x, c);
 }
 
-// One warp per part of a slice.  Positions from the largest fixed index on: one flat copy.  In front of it a lane
-// group per position (`inner` elements), or a lane per position when it is a single element.
+// One warp per part of a slice.  Positions from the largest fixed index on: one flat copy.  In front of it lanes run along
+// the words of the positions (up to 32 words each), or a lane group copies a position (`inner` elements) at a time.
 template <int KIND, int ES, typename I>
 __global__ void __launch_bounds__(256)
 sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst, I d, I nslices, int parts, int part_rows,
-                 int row_bytes, int group_shift, int64_t packed_rows)
+                 int row_bytes, unsigned inv, int group_shift, int64_t packed_rows)
 {
     typedef typename Elem<ES>::T E;
     pdl_wait();
@@ -261,10 +297,25 @@ sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restric
                 copy_flat<ES, false, 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32);
         }
         const I xe = x1 < top ? x1 : top;
-        if (row_bytes == ES) {
-            for (I x = x0 + (I)lane; x < xe; x += 32) {
-                const I p = sym_row<KIND, I>(d, a, b, c, x);
-                if (ST_BOUNDS_OK(p, packed_rows, 1)) reinterpret_cast<E *>(out)[x] = __ldg(reinterpret_cast<const E *>(src) + p);
+        const int words = row_bytes / ES;
+        if (words <= 32) {
+            // lanes along the words of consecutive positions: word e belongs to position e / words (inv: 2^16 / words rounded
+            // up; e < 2^12)
+            const unsigned n = xe > x0 ? (unsigned)(xe - x0) * (unsigned)words : 0u;
+            E *o = reinterpret_cast<E *>(out + (int64_t)x0 * row_bytes);
+            for (unsigned e0 = (unsigned)lane; e0 < n; e0 += 32 * SYM_WORDS) {
+                E v[SYM_WORDS];
+#pragma unroll
+                for (int u = 0; u < SYM_WORDS; ++u) {
+                    const unsigned e = e0 + 32 * u;
+                    if (e >= n) continue;
+                    const unsigned dx = (e * inv) >> 16;
+                    const I p = sym_row<KIND, I>(d, a, b, c, x0 + (I)dx);
+                    v[u] = ST_BOUNDS_OK(p, packed_rows, 1) ? __ldg(reinterpret_cast<const E *>(src) + (int64_t)p * words + (e - dx * (unsigned)words)) : E{};
+                }
+#pragma unroll
+                for (int u = 0; u < SYM_WORDS; ++u)
+                    if (e0 + 32 * u < n) o[e0 + 32 * u] = v[u];
             }
         } else {
             const int g = 1 << group_shift;
@@ -418,8 +469,10 @@ static st_status launch_sym(const void *src, void *dst, const LayoutArgs &a, cud
         return launch(sym_tile_kernel<KIND, ES>, grid, 256, 0, s, (const E *)src, (E *)dst, (unsigned)a.d, nt, a.packed_rows);
     }
     if (a.row_bytes > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
-    // parts of about 2 KiB, a multiple of 32 positions where a lane takes one each
-    const int64_t part_rows = a.row_bytes == ES ? 128 : (2048 + a.row_bytes - 1) / a.row_bytes;
+    // parts of about 2 KiB (4 KiB of 16-byte words)
+    const int64_t words = a.row_bytes / ES;
+    const int64_t part_rows = words <= 32 ? 256 / words < 8 ? 8 : 256 / words : (2048 + a.row_bytes - 1) / a.row_bytes;
+    const unsigned inv = words <= 32 ? (unsigned)((65536 + words - 1) / words) : 0u;
     const int64_t parts = (a.d + part_rows - 1) / part_rows;
     int shift = 0;
     while (shift < 5 && (int64_t(16) << shift) < a.row_bytes) ++shift;
@@ -430,8 +483,8 @@ static st_status launch_sym(const void *src, void *dst, const LayoutArgs &a, cud
     unsigned char *out = (unsigned char *)dst;
     if (small && items < (int64_t(1) << 31))
         return launch(sym_slice_kernel<KIND, ES, unsigned>, grid, 256, 0, s, in, out, (unsigned)a.d, (unsigned)nslices, (int)parts, (int)part_rows,
-                      (int)a.row_bytes, shift, a.packed_rows);
-    return launch(sym_slice_kernel<KIND, ES, int64_t>, grid, 256, 0, s, in, out, a.d, nslices, (int)parts, (int)part_rows, (int)a.row_bytes, shift,
+                      (int)a.row_bytes, inv, shift, a.packed_rows);
+    return launch(sym_slice_kernel<KIND, ES, int64_t>, grid, 256, 0, s, in, out, a.d, nslices, (int)parts, (int)part_rows, (int)a.row_bytes, inv, shift,
                   a.packed_rows);
 }
 
@@ -452,21 +505,34 @@ static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cu
     if (parts > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
     int shift = 0;
     while ((1 << shift) < 256 && (int64_t(16 * COPY_UNITS) << shift) < pb) ++shift;
-    const int64_t nslices = (KIND == ST_TET) ? a.d * a.d : (KIND == ST_SIMPLEX4) ? a.d * a.d * a.d : a.d;
-    const int64_t threads = (nslices * parts) << shift;
+    // pack of a tensor of order 3 or 4: only the slices that have a run
+    const int64_t nslices = KIND == ST_TET ? (PACK ? tri_rows(a.d) : a.d * a.d) : KIND == ST_SIMPLEX4 ? (PACK ? tet_rows(a.d) : a.d * a.d * a.d) : a.d;
+    const int64_t nitems = nslices * parts, threads = nitems << shift;
     const int64_t want = (threads + 255) / 256;
     const unsigned grid = (unsigned)(want < cap ? (want < 1 ? 1 : want) : cap);
     const unsigned char *in = (const unsigned char *)src, *m = (const unsigned char *)mul;
     unsigned char *out = (unsigned char *)dst;
+    // 32-bit index arithmetic: every index and the intermediate products of the closed forms stay below 2^31
+    const bool small = nitems < (int64_t(1) << 30) && a.packed_rows < (int64_t(1) << 31) && a.width < (int64_t(1) << 30) &&
+                       a.d <= (KIND == ST_TET ? 1024 : KIND == ST_SIMPLEX4 ? 200 : 20000);
+    auto run = [&](auto mul_tag, auto index) {
+        typedef decltype(index) I;
+        return launch(slice_copy_kernel<KIND, ES, PACK, decltype(mul_tag)::value, I>, grid, 256, 0, s, in, out, a, (I)nitems, shift, (int)parts,
+                      (int)pb, m);
+    };
     if constexpr (PACK && ES == 4)
-        if (mul) return launch(slice_copy_kernel<KIND, ES, PACK, true>, grid, 256, 0, s, in, out, a, shift, (int)parts, (int)pb, m);
-    return launch(slice_copy_kernel<KIND, ES, PACK, false>, grid, 256, 0, s, in, out, a, shift, (int)parts, (int)pb, m);
+        if (mul) return small ? run(std::true_type{}, 0u) : run(std::true_type{}, int64_t(0));
+    return small ? run(std::false_type{}, 0u) : run(std::false_type{}, int64_t(0));
 }
 
 template <int ES, bool PACK>
 static st_status dispatch_kind(const void *src, void *dst, const LayoutArgs &a, cudaStream_t s, const void *mul)
 {
     if constexpr (!PACK) {
+        if constexpr (ES == 8)
+            if (a.fill == ST_FILL_SYMMETRIC && a.row_bytes % 16 == 0)
+                return a.kind == ST_TRI_UPPER ? launch_sym<ST_TRI_UPPER, 16>(src, dst, a, s)
+                     : a.kind == ST_TET ? launch_sym<ST_TET, 16>(src, dst, a, s) : launch_sym<ST_SIMPLEX4, 16>(src, dst, a, s);
         if (a.fill == ST_FILL_SYMMETRIC)
             return a.kind == ST_TRI_UPPER ? launch_sym<ST_TRI_UPPER, ES>(src, dst, a, s)
                  : a.kind == ST_TET ? launch_sym<ST_TET, ES>(src, dst, a, s) : launch_sym<ST_SIMPLEX4, ES>(src, dst, a, s);
