@@ -35,6 +35,7 @@
 // warps 2..5 = epilogue (TMEM -> registers -> global), one per 32-lane quarter of TMEM.
 #include "tc_common.cuh"
 #include "st_index.cuh"
+#include "pair_layout.cuh"
 #include <cuda_bf16.h>
 
 namespace st {
@@ -64,14 +65,16 @@ template <int MODE> struct Shape {
 
 struct TileTable {
     int ntiles;
-    unsigned char tm[MAX_TILES], tn[MAX_TILES];        // tile row and column (units of 256)
+    unsigned char diag[MAX_TILES];                     // on the diagonal: the columns start where the rows do
     unsigned char width[MAX_TILES];                    // columns, units of 32
+    unsigned short row[MAX_TILES], col[MAX_TILES];     // first row and column of the result, units of 8
+    unsigned short rows[MAX_TILES];                    // at most 256
     unsigned short first[MAX_TILES + 1];               // first cluster: the clusters of a tile share its samples
 };
 struct Args {
     float *partials;                                   // [2 * cluster + block][HALF][BN]
     unsigned *status;
-    int d, chunks_total, stages, nb, na;               // nb, na: boxes of B and A per part in a stage
+    int chunks_total, stages, nb, na;                  // nb, na: boxes of B and A per part in a stage
     int lo_row0;                                       // M2_SPLIT: first row of the lo part
     TileTable tab;
 };
@@ -113,10 +116,11 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     const int cluster = blockIdx.x >> 1;
     const int tile = m2tc_tile_of(a.tab, cluster), split = cluster - a.tab.first[tile];
     const int nsplit = a.tab.first[tile + 1] - a.tab.first[tile];
-    const int tm = a.tab.tm[tile], tn = a.tab.tn[tile], width = 32 * a.tab.width[tile];
+    const int row = 8 * a.tab.row[tile], rows = a.tab.rows[tile], col = 8 * a.tab.col[tile], width = 32 * a.tab.width[tile];
+    const bool diag = a.tab.diag[tile] != 0;
     // narrow tiles are cheap to flush: chains half as long, as short as those of twice as many sample ranges
     const int FLUSH_CHUNKS = MODE == M2_BF16 && width <= HALF ? S::FLUSH_CHUNKS / 2 : S::FLUSH_CHUNKS;
-    const bool alias = tm == tn && width == BN;         // A columns == B columns in both blocks: one load serves both
+    const bool alias = diag && width == BN;             // A columns == B columns in both blocks: one load serves both
     const int chunks_per_split = (a.chunks_total + nsplit - 1) / nsplit;
     const int c_begin = split * chunks_per_split;
     int c_end = c_begin + chunks_per_split;
@@ -160,12 +164,12 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             prefetch_tmap(&tmap);
             // boxes of A that hold columns of X (the others would only make rows that are never read)
             auto boxes_a = [&](int r) {
-                const int left = a.d - tm * BM - r * HALF;
+                const int left = rows - r * HALF;
                 return alias || left <= 0 ? 0 : left >= HALF ? NBOX : (left + BOXC - 1) / BOXC;
             };
             const int nb = (width / 2 + BOXC - 1) / BOXC, na = boxes_a((int)rank);
             const uint32_t tx = (uint32_t)((2 * nb + boxes_a(0) + boxes_a(1)) * PARTS * BOX_BYTES);
-            const int col_a = tm * BM + (int)rank * HALF, col_b = tn * BN + (int)rank * (width / 2);
+            const int col_a = row + (int)rank * HALF, col_b = col + (int)rank * (width / 2);
             const uint32_t bar0 = map_to_cta(smem_u32(full), 0);
             int s = 0;
             uint32_t parity = 1;
@@ -173,11 +177,11 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                 if (c >= stages && !mbar_wait(&empty[s], parity, abort_flag, a.status, 1)) break;
                 if (rank == 0) mbar_expect_tx(&full[s], tx);
                 const uint32_t bar = bar0 + (uint32_t)(s * sizeof(uint64_t));
-                const int row = (c_begin + c) * KROWS;
+                const int sample = (c_begin + c) * KROWS;
 #pragma unroll
                 for (int p = 0; p < PARTS; ++p) {
                     unsigned char *base = smem + (size_t)s * stage_bytes + (size_t)p * part_bytes;
-                    const int y = row + (p ? a.lo_row0 : 0);
+                    const int y = sample + (p ? a.lo_row0 : 0);
                     for (int b = 0; b < nb; ++b)            // B half (and A on full diagonal tiles)
                         tma_load_2d_pair(base + b * BOX_BYTES, &tmap, bar, col_b + b * BOXC, y);
                     for (int b = 0; b < na; ++b)            // A rows of this block
@@ -234,22 +238,22 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             }
         }
     } else {
-        // ---------------- epilogue (both blocks): own 128 rows of the tile; what lies past column d or wholly below the
-        // diagonal is not stored (the reduction reads i <= j < d only)
+        // ---------------- epilogue (both blocks): own 128 rows of the tile; what is past the tile's rows or
+        // wholly below the diagonal is not stored (the reduction does not read it)
         const int q = warp & 3;
         const int row0 = (int)rank * HALF + q * 32;
-        const bool rows = tm * BM + row0 < a.d;
-        const int c_first = tm == tn ? row0 : 0;         // row0 is a multiple of 32
+        const bool used = row0 < rows;
+        const int c_first = diag ? row0 : 0;         // row0 is a multiple of 32
         float *dst = a.partials + ((size_t)blockIdx.x * HALF + (q * 32 + lane)) * BN;
         const uint32_t leader_acc_empty0 = map_to_cta(smem_u32(&acc_empty[0]), 0);
-        if (nphases == 0 && rows) {
+        if (nphases == 0 && used) {
             for (int c0 = c_first; c0 < width; c0 += 4) *reinterpret_cast<float4 *>(dst + c0) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         for (int ph = 0; ph < nphases; ++ph) {
             const int buf = ph & 1;
             if (!mbar_wait(&acc_full[buf], (uint32_t)((ph >> 1) & 1), abort_flag, a.status, 3)) break;
             tc_fence_after();
-            if (rows) {
+            if (used) {
 #pragma unroll 1
                 for (int c0 = c_first; c0 < width; c0 += 32) {
                     uint32_t r[32];
@@ -285,20 +289,19 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 // Sums of the partial tiles over the sample ranges, i <= j < d only.  `wps` warps share 32 V columns of a row: the first
 // adds ranges 0, wps, 2 wps, ... with its loads in flight, and so on, then their sums are added in order.  V = 4 where
 // there are few ranges, so that a thread still has enough loads in flight.
-// PAIRS: X holds pair features (see moment4.cu) and row (i,j) of the result goes straight to the packed 4-simplex: its
-// unique entries are the columns from pair (j,j) = rowmap[row].x on, one run on both sides; rowmap[row].y + column is
-// the place of a column's entry.
+// PAIRS: X holds pair features in the order of pair_layout.cuh; pairs[column] is the pair of a column, and an entry goes
+// to the place of its 4-tuple in the packed 4-simplex, if this is the product that was chosen for that tuple.
 template <bool PAIRS, int V>
 __global__ void __launch_bounds__(256)
-moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int npairs, int64_t out_elems,
-                         const int2 *__restrict__ rowmap, const __grid_constant__ m2tc::TileTable tab)
+moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int features, int64_t out_elems,
+                         const unsigned *__restrict__ pairs, const __grid_constant__ m2tc::TileTable tab)
 {
     using namespace m2tc;
     __shared__ float part[2][8][32 * V];
     const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tm = tab.tm[tile], tn = tab.tn[tile], width = 32 * tab.width[tile], uw = (width + 32 * V - 1) / (32 * V);
+    const int row = 8 * tab.row[tile], col = 8 * tab.col[tile], width = 32 * tab.width[tile], uw = (width + 32 * V - 1) / (32 * V);
     const int first = tab.first[tile], nsplit = tab.first[tile + 1] - first;
-    const int rows = d - tm * BM < BM ? d - tm * BM : BM;
+    const int rows = tab.rows[tile];
     const int wps = nsplit <= 8 ? 1 : nsplit <= 16 ? 2 : nsplit <= 32 ? 4 : 8;  // about eight loads per thread
     const int per = 8 / wps, w0 = warp % wps;
     const size_t stride = (size_t)2 * HALF * BN;
@@ -308,18 +311,23 @@ moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__
     int buf = 0;
     for (int u0 = blockIdx.y * per; u0 < rows * uw; u0 += gridDim.y * per) {
         const int u = u0 + warp / wps, r = u / uw, c = (u - r * uw) * (32 * V) + V * lane;   // this thread's columns c .. c+V-1
-        const int gi = tm * BM + r, gj = tn * BN + c;
-        int lo = gi, hi = d;                               // columns of this row that are outputs
-        int64_t at;                                        // of column gj
-        if (PAIRS) {
-            const int2 m = gi < npairs ? rowmap[gi] : make_int2(1 << 30, 0);
-            lo = m.x;
-            hi = npairs;                                   // not the padding
-            at = m.y + gj;
-        } else {
-            at = tri_encode(d, gi, gj);
+        const int gi = row + r, gj = col + c;
+        const bool in_tile = r < rows && c < width;
+        const int at0 = PAIRS ? 0 : (int)tri_encode(d, gi, gj);
+        int at[V];                                         // where the columns go to, -1: not an output
+        bool use = false;
+#pragma unroll
+        for (int x = 0; x < V; ++x) {
+            at[x] = -1;
+            if (PAIRS) {
+                int i, j, k, l;
+                if (in_tile && gj + x < d && pair_product(pairs[gi], pairs[gj + x], i, j, k, l))
+                    at[x] = (int)simp4_encode(features, i, j, k, l);
+            } else if (in_tile && gi <= gj + x && gj + x < d) {
+                at[x] = at0 + x;
+            }
+            use |= at[x] >= 0;
         }
-        const bool use = r < rows && c < width && gj + V > lo && gj < hi;
         float s[V];
 #pragma unroll
         for (int x = 0; x < V; ++x) s[x] = 0.f;
@@ -351,7 +359,7 @@ moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__
 #pragma unroll
             for (int x = 0; x < V; ++x) {
                 for (int w = 1; w < wps; ++w) s[x] += part[buf][warp + w][32 * x + lane];
-                if (gj + x >= lo && gj + x < hi && ST_BOUNDS_OK(at + x, out_elems, PAIRS ? 7 : 2)) out[at + x] = s[x];
+                if (at[x] >= 0 && ST_BOUNDS_OK(at[x], out_elems, PAIRS ? 7 : 2)) out[at[x]] = s[x];
             }
         }
         buf ^= 1;
@@ -365,41 +373,50 @@ struct M2TcPlan {
     bool ok;
 };
 
+// Time per stage, a full tile = 1: the 256 columns of A are loaded whatever the width (the MMA alone would be 43 cycles
+// at 64 columns against 128; with 0.35 in place of 0.7 [400000,304] bf16 ran 127 us instead of 111).
+static double m2tc_cost(int width) { return 0.7 + 0.3 * width / m2tc::BN; }
+
+// Tiles of a plan while it is made.
+struct M2TcTiles {
+    M2TcPlan *p;
+    int n;
+    double cost[m2tc::MAX_TILES];
+    template <int MODE>
+    bool add(int row, int rows, int col, int width, bool diag)
+    {
+        using namespace m2tc;
+        using S = Shape<MODE>;
+        if (n >= MAX_TILES) return false;
+        p->tab.row[n] = (unsigned short)(row / 8);
+        p->tab.rows[n] = (unsigned short)rows;
+        p->tab.col[n] = (unsigned short)(col / 8);
+        p->tab.width[n] = (unsigned char)(width / 32);
+        p->tab.diag[n] = diag ? 1 : 0;
+        cost[n] = m2tc_cost(width);
+        const int nb = (width / 2 + S::BOXC - 1) / S::BOXC;
+        if (nb > p->nb) p->nb = nb;
+        if (!(diag && width == BN)) {
+            const int na = rows >= HALF ? S::NBOX : (rows + S::BOXC - 1) / S::BOXC;
+            if (na > p->na) p->na = na;
+        }
+        ++n;
+        return true;
+    }
+};
+
+// Sample ranges, stages and sizes of a plan whose tiles are known.
 template <int MODE>
-static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
+static void m2tc_finish(M2TcPlan &p, const M2TcTiles &t, int64_t N)
 {
     using namespace m2tc;
     using S = Shape<MODE>;
-    M2TcPlan p;
-    p.ok = false;
-    const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
-    const int nt = (int)((d + BM - 1) / BM);
-    int n = 0;
-    double cost[MAX_TILES];
-    p.nb = p.na = 0;
-    for (int tn = 0; tn < nt; ++tn)
-        for (int tm = 0; tm < nt; ++tm) {
-            if (tm > tn && !dense) continue;
-            if (n >= MAX_TILES) return p;
-            const int left = (int)d - tn * BN, width = left >= BN ? BN : (left + 31) / 32 * 32;
-            p.tab.tm[n] = (unsigned char)tm;
-            p.tab.tn[n] = (unsigned char)tn;
-            p.tab.width[n] = (unsigned char)(width / 32);
-            // time per stage, a full tile = 1: the 256 columns of A are loaded whatever the width (the MMA alone would be
-            // 43 cycles at 64 columns against 128; with 0.35 in place of 0.7 [400000,304] bf16 ran 127 us instead of 111)
-            cost[n] = 0.7 + 0.3 * width / BN;
-            const int nb = (width / 2 + S::BOXC - 1) / S::BOXC;
-            if (nb > p.nb) p.nb = nb;
-            if (!(tm == tn && width == BN)) {
-                const int la = (int)d - tm * BM, na = la >= HALF ? S::NBOX : (la + S::BOXC - 1) / S::BOXC;
-                if (na > p.na) p.na = na;
-            }
-            ++n;
-        }
-    for (int i = n; i < MAX_TILES; ++i) p.tab.tm[i] = p.tab.tn[i] = p.tab.width[i] = 0;
+    const int n = t.n;
+    const double *cost = t.cost;
+    for (int i = n; i < MAX_TILES; ++i) p.tab.diag[i] = p.tab.width[i] = p.tab.row[i] = p.tab.rows[i] = p.tab.col[i] = 0;
     p.tab.ntiles = n;
     const int64_t chunks = (N + S::KROWS - 1) / S::KROWS;
-    if (chunks > (int64_t(1) << 30)) return p;
+    if (chunks > (int64_t(1) << 30)) return;
     p.chunks_total = (int)chunks;
     const size_t stage = (size_t)S::PARTS * (p.nb + p.na) * S::BOX_BYTES;
     p.stages = (int)((n == 1 ? STAGES_BYTES_1 : STAGES_BYTES) / stage);
@@ -439,15 +456,87 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
     for (int i = n; i <= MAX_TILES; ++i) p.tab.first[i] = (unsigned short)first;
     p.partial_bytes = (size_t)2 * first * HALF * BN * sizeof(float);
     p.ok = true;
+}
+
+template <int MODE>
+static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
+{
+    using namespace m2tc;
+    M2TcPlan p{};
+    M2TcTiles t{&p, 0, {}};
+    const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
+    const int nt = (int)((d + BM - 1) / BM);
+    for (int tn = 0; tn < nt; ++tn)
+        for (int tm = 0; tm < nt; ++tm) {
+            if (tm > tn && !dense) continue;
+            const int left = (int)d - tn * BN, width = left >= BN ? BN : (left + 31) / 32 * 32, below = (int)d - tm * BM;
+            if (!t.add<MODE>(tm * BM, below < BM ? below : BM, tn * BN, width, tm == tn)) return p;
+        }
+    m2tc_finish<MODE>(p, t, N);
     return p;
 }
 
-// Launches the tile kernel and the sum of its partial tiles.  rows: rows of X in memory; npairs > 0: X holds pair
-// features and the result goes to the packed 4-simplex of `simplex` entries.
+// Tiles of the products of pair features that pair_layout.cuh names, in turn to f(row, rows, col, width, on the diagonal).
+template <class F>
+static void pair_tiles(const PairLayout &L, F f)
+{
+    using namespace m2tc;
+    auto strip = [&](int row, int rows, int col, int end) {
+        for (int c = col; c < end; c += BN) f(row, rows, c, end - c >= BN ? BN : (end - c + 31) / 32 * 32, c == row);
+    };
+    for (int r = 0; r < L.within; r += BM) strip(r, L.within - r < BM ? L.within - r : BM, r, L.cols);
+    for (int r = 0; r < L.rows_n && L.prod_n > 0; r += BM)
+        strip(L.rows + r, L.rows_n - r < BM ? L.rows_n - r : BM, L.prod, L.prod + L.prod_n);
+}
+
+// Ranges of the features: one, two or three of about equal size, or four and a smaller one, whichever gives the cheapest
+// tiles.  (Four and a smaller one: 45 features take 256 rows as 11, 11, 11, 10 and 2, but 261 as five nines.)
+PairLayout pair_layout(int features)
+{
+    PairLayout best{};
+    double least = 0;
+    for (int option = 0; option < 4 + features / 4; ++option) {
+        const int last = option < 3 ? 0 : option - 3, m = option < 3 ? option + 1 : 4;   // m equal ranges and the last one
+        PairLayout L{};
+        int n[5] = {0, 0, 0, 0, last}, within = 0;
+        for (int g = 0; g < m; ++g) n[g] = (features - last) / m + (g < (features - last) % m ? 1 : 0);
+        for (int g = 0; g < 5; ++g) {
+            L.lo[g + 1] = L.lo[g] + n[g];
+            within += n[g] * (n[g] + 1) / 2;
+        }
+        L.features = features;
+        L.within = within;
+        L.rows_n = n[0] * n[1] + (n[0] + n[1]) * n[4];
+        L.prod_n = n[2] * n[3] + (n[2] + n[3]) * n[4];
+        L.rows = (within + 7) / 8 * 8;
+        L.prod = (L.rows + L.rows_n + 7) / 8 * 8;
+        L.cols = L.prod + (int)tri_rows(features) - within - L.rows_n;
+        double cost = 0;
+        pair_tiles(L, [&](int, int, int, int width, bool) { cost += m2tc_cost(width); });
+        if (option == 0 || cost < least) {
+            best = L;
+            least = cost;
+        }
+    }
+    return best;
+}
+
+template <int MODE>
+static M2TcPlan m2tc_plan_pairs(int64_t N, const PairLayout &L)
+{
+    M2TcPlan p{};
+    M2TcTiles t{&p, 0, {}};
+    bool ok = true;
+    pair_tiles(L, [&](int row, int rows, int col, int width, bool diag) { ok = ok && t.add<MODE>(row, rows, col, width, diag); });
+    if (ok) m2tc_finish<MODE>(p, t, N);
+    return p;
+}
+
+// Launches the tile kernel and the sum of its partial tiles.  rows: rows of X in memory; pairs: X holds the pair features
+// of `features` features and the result goes to their packed 4-simplex.
 template <int MODE>
 static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int64_t d, int64_t ldx, float *out, float *partials,
-                             unsigned *status, cudaStream_t stream, int lo_row0 = 0, int npairs = 0,
-                             const int2 *rowmap = nullptr, int64_t simplex = 0)
+                             unsigned *status, cudaStream_t stream, int lo_row0 = 0, const unsigned *pairs = nullptr, int features = 0)
 {
     using S = m2tc::Shape<MODE>;
     CUtensorMap tmap;
@@ -456,7 +545,7 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
                           MODE == M2_TF32 ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B))
         return ST_ERR_CUDA;
     m2tc::Args a;
-    a.partials = partials; a.status = status; a.d = (int)d;
+    a.partials = partials; a.status = status;
     a.chunks_total = q.chunks_total; a.stages = q.stages; a.nb = q.nb; a.na = q.na; a.lo_row0 = lo_row0;
     a.tab = q.tab;
     if (!ensure_dynamic_smem(moment2_tc_kernel<MODE>, q.smem)) return ST_ERR_CUDA;
@@ -483,10 +572,10 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     const unsigned blocks = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
     const dim3 rgrid((unsigned)q.tab.ntiles, blocks < 64 ? 64 : blocks > 1024 ? 1024 : blocks);
     auto reduce = [&](auto kernel) {
-        return launch(kernel, rgrid, 256, 0, stream, partials, out, (int)d, npairs, npairs > 0 ? simplex : tri_rows(d), rowmap, q.tab);
+        return launch(kernel, rgrid, 256, 0, stream, partials, out, (int)d, features, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.tab);
     };
-    if (most <= 4) return npairs > 0 ? reduce(moment2_tc_reduce_kernel<true, 4>) : reduce(moment2_tc_reduce_kernel<false, 4>);
-    return npairs > 0 ? reduce(moment2_tc_reduce_kernel<true, 1>) : reduce(moment2_tc_reduce_kernel<false, 1>);
+    if (most <= 4) return pairs ? reduce(moment2_tc_reduce_kernel<true, 4>) : reduce(moment2_tc_reduce_kernel<false, 4>);
+    return pairs ? reduce(moment2_tc_reduce_kernel<true, 1>) : reduce(moment2_tc_reduce_kernel<false, 1>);
 }
 
 // Room for the partial tiles of the structured call and of its dense control: one workspace serves both.
@@ -617,26 +706,26 @@ st_status moment2_split_tc(const float *X, int64_t N, int64_t d, int64_t ldx, fl
     return m2tc_launch<M2_SPLIT>(p.q, Z, 2 * p.Np, d, d, out, (float *)((unsigned char *)ws + p.part_off), (unsigned *)ws, stream, (int)p.Np);
 }
 
-// The second moment of pair features that the caller has written, its unique 4-tuples straight into the packed
-// 4-simplex (see moment4.cu).  split: P = [hi rows; lo rows], each part N rounded up to 64 rows with zero rows at the
-// end; else N rows of bf16.  dP columns; rowmap as in moment2_tc_reduce_kernel.
+// The products of pair features that the caller has written (moment4.cu), straight into the packed 4-simplex.  split:
+// P = [hi rows; lo rows], each part N rounded up to 64 rows with zero rows at the end; else N rows of bf16.  ldp: columns
+// of P, those of the layout and zeros after them.
 int64_t moment2_split_part_rows(int64_t N) { return (N + 63) / 64 * 64; }
 
-size_t moment2_pairs_partial_bytes(int64_t N, int64_t dP, bool split)
+size_t moment2_pairs_partial_bytes(int64_t N, const PairLayout &L, bool split)
 {
-    if (N <= 0 || dP <= 0 || dP > 4096 || N > (int64_t(1) << 29)) return 0;
-    const M2TcPlan q = split ? m2tc_plan<M2_SPLIT>(N, dP, 0) : m2tc_plan<M2_BF16>(N, dP, 0);
+    if (N <= 0 || N > (int64_t(1) << 29)) return 0;
+    const M2TcPlan q = split ? m2tc_plan_pairs<M2_SPLIT>(N, L) : m2tc_plan_pairs<M2_BF16>(N, L);
     return q.ok ? q.partial_bytes : 0;
 }
 
-st_status moment2_pairs_tc(const void *P, int64_t N, int64_t dP, int npairs, bool split, const int2 *rowmap, int64_t simplex, float *out,
+st_status moment2_pairs_tc(const void *P, int64_t N, const PairLayout &L, int64_t ldp, bool split, const unsigned *pairs, float *out,
                            float *partials, unsigned *status, cudaStream_t stream)
 {
-    if (split) {
-        const int64_t Np = moment2_split_part_rows(N);
-        return m2tc_launch<M2_SPLIT>(m2tc_plan<M2_SPLIT>(N, dP, 0), P, 2 * Np, dP, dP, out, partials, status, stream, (int)Np, npairs, rowmap, simplex);
-    }
-    return m2tc_launch<M2_BF16>(m2tc_plan<M2_BF16>(N, dP, 0), P, N, dP, dP, out, partials, status, stream, 0, npairs, rowmap, simplex);
+    const int64_t Np = moment2_split_part_rows(N);
+    if (split)
+        return m2tc_launch<M2_SPLIT>(m2tc_plan_pairs<M2_SPLIT>(N, L), P, 2 * Np, ldp, ldp, out, partials, status, stream, (int)Np, pairs,
+                                     L.features);
+    return m2tc_launch<M2_BF16>(m2tc_plan_pairs<M2_BF16>(N, L), P, N, ldp, ldp, out, partials, status, stream, 0, pairs, L.features);
 }
 
 }  // namespace st

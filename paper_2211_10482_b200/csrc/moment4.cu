@@ -5,20 +5,21 @@
 // M3 is the second moment of the pair features: with P[n,(i,j)] = X[n,i] X[n,j] over the unique
 // pairs i<=j (the rows of vec(f (x) f) that are not redundant),
 //     out[s(i,j,k,l)] = sum_n P[n,(i,j)] P[n,(k,l)],
-// and (i,j,k,l) is a unique 4-tuple exactly when j <= k.  Three steps, all on the GPU:
-//   1. pair_expand_kernel    P [N, dP], dP = d(d+1)/2 rounded up to 64 (zero columns), fp32 or bf16
-//   2. st_sym_moment2 on P   the packed upper triangle of P^T P: the tensor-core triangular tile GEMM, on P rounded
-//                            to bf16 (ST_FLAG_TC_BF16, 5e-3) or, for the fp32 tolerance, on P written as hi + lo
-//                            bf16 parts and multiplied in three partial products (d <= 89: the pair features
-//                            fit the kernel's 4096 columns); beyond that the fp32 FMA kernel on an fp32 P
-//   3. all entries (i,j,*,*) of the 4-simplex are one run of row (i,j) of that triangle, from column (j,j) on,
-//      contiguous on both sides: the sum over the partial tiles of step 2 writes them there (tensor-core paths);
-//      simplex_gather_kernel copies them from the packed triangle (fp32 FMA path)
-// Step 2 works on the symmetric pair-by-pair matrix, whose unique set (pairs p <= q) is about
-// three times larger than the set of unique 4-tuples: the entries with j > k are computed and
-// not gathered.
+// and every unique 4-tuple is such a product.  All on the GPU:
+//   1. pair_expand_kernel   P [N, dP], the pairs rounded up to 64 columns (zeros)
+//   2. tensor cores (up to 4096 pair features, d <= 90): the triangular tile GEMM of moment2_tc.cu on P rounded to bf16
+//      (ST_FLAG_TC_BF16, 5e-3) or, for the fp32 tolerance, on P written as hi + lo bf16 parts and multiplied in three
+//      partial products.  The columns of P are in the order of pair_layout.cuh, in which a few tiles hold a product for
+//      every 4-tuple, and the sum over their partial tiles goes straight to the packed 4-simplex.  With the pairs in
+//      packed order (a tuple where j <= k, so all tiles of the triangle) [30011,45] ran 136 us, now 90; with the rows'
+//      pairs ordered by j and a copy of them by k for the columns (a staircase, P twice as large) 135; [14831,64] 253,
+//      now 136, the staircase 150; [114839,23] 107, now 97.
+//   3. more features, or more samples than those kernels take: the fp32 FMA kernel on an fp32 P in packed order.  The
+//      entries (i,j,*,*) are one run of row (i,j) of its packed triangle, from column (j,j) on (i <= j <= k <= l), which
+//      simplex_gather_kernel copies.
 #include "st_common.cuh"
 #include "st_index.cuh"
+#include "pair_layout.cuh"
 #include <cuda_bf16.h>
 #include <type_traits>
 
@@ -26,19 +27,22 @@ namespace st {
 
 size_t moment2_workspace(int64_t N, int64_t d, int xdt, unsigned flags);
 int64_t moment2_split_part_rows(int64_t N);
-size_t moment2_pairs_partial_bytes(int64_t N, int64_t dP, bool split);
-st_status moment2_pairs_tc(const void *P, int64_t N, int64_t dP, int npairs, bool split, const int2 *rowmap, int64_t simplex, float *out,
+PairLayout pair_layout(int features);
+size_t moment2_pairs_partial_bytes(int64_t N, const PairLayout &L, bool split);
+st_status moment2_pairs_tc(const void *P, int64_t N, const PairLayout &L, int64_t ldp, bool split, const unsigned *pairs, float *out,
                            float *partials, unsigned *status, cudaStream_t stream);
 
 namespace m4 {
 
-constexpr int MAX_D = 128;          // fp32 path; the bf16 path ends where the pair features exceed the tensor-core kernel's 4096 columns (d <= 89)
+constexpr int MAX_D = 128;          // fp32 path; the bf16 path ends where the pair features exceed 4096 columns (d <= 90)
 constexpr int EXP_ROWS = 32;        // sample rows per pass of a block
 constexpr int EXP_THREADS = 192;
+constexpr int64_t TC_COLS = 4096;   // most pair features on the tensor cores
 
 struct Plan {
-    int64_t dP, p_bytes, Np;
-    size_t off_p, off_m2, off_ws, m2_ws, total;     // off_m2: packed triangle (fp32 path) or row map; off_ws: workspace or partial tiles of step 2
+    int64_t dP, p_bytes, Np;                        // dP: columns of P, a multiple of 64
+    PairLayout layout;                              // of the columns on the tensor-core paths
+    size_t off_p, off_m2, off_ws, m2_ws, total;     // off_m2: packed triangle (fp32 FMA path) or pair of each column; off_ws: workspace or partial tiles of step 2
     bool bf16, split, ok;
 };
 
@@ -52,15 +56,22 @@ static Plan plan(int64_t N, int64_t d, unsigned flags)
     // fp32 result: the pair features are written as hi + lo bf16 parts and multiplied on the tensor cores in three
     // partial products (the fp32 tolerance) wherever that kernel reaches; else fp32 features and the fp32 FMA kernel
     p.Np = moment2_split_part_rows(N);
-    p.m2_ws = moment2_pairs_partial_bytes(N, p.dP, !p.bf16);
-    p.split = !p.bf16 && p.m2_ws != 0;
-    const bool fma = !p.bf16 && !p.split;
-    if (fma) p.m2_ws = moment2_workspace(N, p.dP, ST_F32, 0);
+    if (p.dP <= TC_COLS) {
+        p.layout = pair_layout((int)d);
+        p.m2_ws = moment2_pairs_partial_bytes(N, p.layout, !p.bf16);
+    }
+    if (p.m2_ws != 0) {
+        p.split = !p.bf16;
+        p.dP = (p.layout.cols + 63) / 64 * 64;
+    } else if (!p.bf16) {
+        p.m2_ws = moment2_workspace(N, p.dP, ST_F32, 0);
+    }
     if (p.m2_ws == 0) return p;
+    const bool fma = !p.bf16 && !p.split;
     p.p_bytes = p.split ? 2 * p.Np * p.dP * 2 : N * p.dP * (p.bf16 ? 2 : 4);
     p.off_p = kWsHeaderBytes;
     p.off_m2 = round_up(p.off_p + (size_t)p.p_bytes, 256);
-    p.off_ws = round_up(p.off_m2 + (fma ? (size_t)tri_rows(p.dP) * sizeof(float) : (size_t)tri_rows(d) * sizeof(int2)), 256);
+    p.off_ws = round_up(p.off_m2 + (fma ? (size_t)tri_rows(p.dP) * sizeof(float) : (size_t)p.dP * sizeof(unsigned)), 256);
     p.total = p.off_ws + p.m2_ws;
     p.ok = true;
     return p;
@@ -76,19 +87,20 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *dst, float a, float b, flo
     *reinterpret_cast<uint2 *>(dst) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
 }
 
-// P[n, p(i,j)] = X[n,i] X[n,j] for the unique pairs in packed order, zeros in the padding
+// P[n, p] = X[n,i] X[n,j] for the pair (i,j) of column p (in packed order, or LAYOUT), zeros in the padding
 // columns.  A block stages EXP_ROWS rows of X per pass (one extra column holds zero); a thread owns
 // four adjacent columns of P, decodes their index pairs once and writes them for every staged
 // row with one 8- or 16-byte store.  HBM bound: the write of P.
 // SPLIT: every product p is written twice, hi = bf16(p) in row n and lo = bf16(p - hi) in row Np + n; the rows
 // N .. Np-1 of either part are zero.
-// rowmap (tensor-core paths): where the unique entries of row p of P^T P start and go to, see moment2_tc_reduce_kernel.
+// LAYOUT (tensor-core paths): the order of pair_layout.cuh; pairs[p] becomes the pair of column p.
 // COLS: columns of a staged row per lane, (d + 1 + 31) / 32 rounded up to an instance (2, 3 or 5).
 template <typename OutT, bool SPLIT, int COLS>
 __global__ void __launch_bounds__(EXP_THREADS)
-pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, OutT *__restrict__ P, int dP, int npairs,
-                   int64_t Np, int2 *__restrict__ rowmap)
+pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, OutT *__restrict__ P, int dP, int npairs, int64_t Np,
+                   const __grid_constant__ PairLayout layout, unsigned *__restrict__ pairs)
 {
+    constexpr bool LAYOUT = sizeof(OutT) == 2;
     extern __shared__ __align__(16) float xs[];                       // 2 x [EXP_ROWS][d + 1], column d is zero
     const int pitch = d + 1;
     pdl_wait();
@@ -99,15 +111,18 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         ci[u] = cj[u] = d;                                            // padding column: 0 * 0
-        if (p + u < npairs) {
+        if (LAYOUT) {
+            const unsigned e = p + u < dP ? pair_of_column(layout, p + u) : kPairNone;
+            if (e != kPairNone) {
+                ci[u] = (int)(e & 255);
+                cj[u] = (int)((e >> 8) & 255);
+            }
+            if (blockIdx.y == 0 && p + u < dP) pairs[p + u] = e;
+        } else if (p + u < npairs) {
             int64_t a, b;
             tri_decode(d, p + u, a, b);
             ci[u] = (int)a;
             cj[u] = (int)b;
-            if (rowmap && blockIdx.y == 0) {
-                const int64_t q0 = tri_encode(d, b, b);
-                rowmap[p + u] = make_int2((int)q0, (int)(simp4_encode(d, a, b, b, b) - q0));
-            }
         }
     }
     const bool inside = p < dP;
@@ -226,23 +241,22 @@ extern "C" st_status st_sym_moment4(const float *X, int64_t N, int64_t d, int64_
     const int64_t passes = ((p.split ? p.Np : N) + EXP_ROWS - 1) / EXP_ROWS;
     const int64_t cap = ((int64_t)sm_count_or_default() * 8 + col_groups - 1) / col_groups;
     const dim3 grid(col_groups, (unsigned)(passes < cap ? passes : cap));
-    int2 *rowmap = (p.split || p.bf16) ? (int2 *)(w + p.off_m2) : nullptr;
+    unsigned *pairs = (unsigned *)(w + p.off_m2);
     auto expand = [&](auto tag, auto split_tag) {
         using T = decltype(tag);
         constexpr bool SP = decltype(split_tag)::value;
         T *dst = (T *)(w + p.off_p);
         if (d + 1 <= 64)
-            return launch(pair_expand_kernel<T, SP, 2>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
+            return launch(pair_expand_kernel<T, SP, 2>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, p.layout, pairs);
         if (d + 1 <= 96)
-            return launch(pair_expand_kernel<T, SP, 3>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
-        return launch(pair_expand_kernel<T, SP, 5>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, rowmap);
+            return launch(pair_expand_kernel<T, SP, 3>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, p.layout, pairs);
+        return launch(pair_expand_kernel<T, SP, 5>, grid, EXP_THREADS, smem, stream, X, N, (int)d, ldx, dst, (int)p.dP, npairs, p.Np, p.layout, pairs);
     };
     st_status rc = p.split ? expand(__nv_bfloat16(), std::true_type())
                  : p.bf16 ? expand(__nv_bfloat16(), std::false_type()) : expand(float(), std::false_type());
     if (rc != ST_OK) return rc;
     if (p.split || p.bf16)
-        return moment2_pairs_tc(w + p.off_p, N, p.dP, npairs, p.split, rowmap, simp4_rows(d), out_packed, (float *)(w + p.off_ws), (unsigned *)w,
-                                stream);
+        return moment2_pairs_tc(w + p.off_p, N, p.layout, p.dP, p.split, pairs, out_packed, (float *)(w + p.off_ws), (unsigned *)w, stream);
     float *M2 = (float *)(w + p.off_m2);
     rc = st_sym_moment2(w + p.off_p, ST_F32, N, p.dP, p.dP, M2, w + p.off_ws, p.m2_ws, 0, stream_);
     if (rc != ST_OK) return rc;

@@ -595,6 +595,21 @@ def test_moment4_more_than_64_features(st, flag_name, N, d):
         assert abs(lhs - rhs) <= (5e-3 if flags else TOL_F32) * float(np.sum(np.abs(Xd).sum(axis=1) ** 4))
 
 
+@pytest.mark.parametrize("flag_name", [None, "ST_FLAG_TC_BF16"])
+@pytest.mark.parametrize("d", [22, 23, 31, 32, 37, 38, 44, 45, 46, 48, 64, 71, 90])
+def test_moment4_every_entry_whatever_ranges_the_features_are_cut_into(st, d, flag_name):
+    # one, two, three, four and five ranges, one and several tiles in either block.  Small integers: the pair features are
+    # exact in bf16 and all sums exact in fp32, so an entry that is missing, doubled or misplaced cannot hide.
+    N = 37
+    X = np.random.default_rng(d).integers(-3, 4, size=(N, d)).astype(np.float32)
+    got = st.st_sym_moment4(dev(X), flags=getattr(st, flag_name) if flag_name else 0).cpu().numpy()
+    ii, jj, kk, ll = np.array(list(itertools.combinations_with_replacement(range(d), 4)), dtype=np.int64).T
+    want = np.zeros(ii.size)
+    for x in X.astype(np.float64):
+        want += x[ii] * x[jj] * x[kk] * x[ll]
+    assert np.array_equal(got, want)
+
+
 def test_moment4_is_reconstructed_once_at_the_end_of_a_chain(st):
     # fourth moments of two batches are added in packed space (one structure: the sum keeps it) and the dense
     # d^4 tensor is rebuilt once through the redundancy map of the 4-simplex (Section 5.5; Section 6, Property 5)
