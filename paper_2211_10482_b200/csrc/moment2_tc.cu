@@ -1,13 +1,15 @@
 // st_sym_moment2, tensor-core paths: out[p(i,j)] = sum_n X[n,i] X[n,j], fp32 accumulation (Section 3, M1; the outer
-// product summed over samples is a symmetric rank-N update, i.e. a triangular tile GEMM X^T X).  Three forms of X:
+// product summed over samples is a symmetric rank-N update, i.e. a triangular tile GEMM X^T X).  Four forms of X:
 //   M2_BF16   bfloat16
 //   M2_TF32   fp32, of which the tensor core reads the upper 19 bits
-//   M2_SPLIT  fp32 written by a pass of its own as x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi
+//   M2_CONV   fp32, in the kernel x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi
+//   M2_SPLIT  the same products of hi and lo that lie in memory (the pair features of moment4.cu)
 //
 // A cluster of two blocks owns an output tile of 256 rows (i) x up to 256 columns (j) for a range of the samples.
 // Only tiles that contain an entry with i <= j are launched, and a tile of the last column is as wide as the columns
 // left, rounded up to 32.  Block r of the pair stages columns 256*TM+128r.. (its 128 rows of the A operand) and its
-// half of the columns of the B operand; on full diagonal tiles the two coincide and are loaded once.  The leader block
+// half of the columns of the B operand; on full diagonal tiles the two coincide and are loaded once, and where all rows are
+// in the first block its A holds its B ([1048576,64] bf16 57 us with both loaded, now 50; [271319,8] 22, now 16).  The leader block
 // issues one MMA of M = 256 for the pair; each block keeps the accumulator of its 128 rows in its own tensor memory
 // and adds it into an fp32 partial tile; a second kernel adds the partial tiles of all sample ranges in a fixed order
 // and writes the packed upper triangle.
@@ -31,8 +33,16 @@
 // 5-12% slower, with three it starves.  M2_SPLIT makes its three products from one load of both parts (64 instead of
 // 96 bytes per sample and column pair).  Few features: the latency of a stage, hence more and smaller stages.
 //
-// Warp roles (192 threads): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner,
-// warps 2..5 = epilogue (TMEM -> registers -> global), one per 32-lane quarter of TMEM.
+// M2_CONV: a pass that wrote hi and lo before moved 8 bytes a value through HBM on top of the 4 read here, and took
+// 176 of the 590 us of [262144,520], now 490; [1048576,256] 700, now 340; [1048576,64] 245, now 143.  Copies bring the
+// fp32 boxes, converting warps rewrite them in place and arrive at the leader's barrier.  Bound by shared memory: per
+// 32 samples of a full tile off the diagonal 256 cycles each for the copy, the reads and the writes and 384 for the
+// operands of 768 cycles of MMA.  Loads through registers instead of the copies avoid two of these, but every arrival
+// then waits for the loads in flight (760 us).
+//
+// Warp roles (192 threads, M2_CONV 384 more): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner,
+// warps 2..5 = epilogue (TMEM -> registers -> global), one per 32-lane quarter of TMEM,
+// warps 6.. convert.
 #include "tc_common.cuh"
 #include "st_index.cuh"
 #include "pair_layout.cuh"
@@ -40,7 +50,7 @@
 
 namespace st {
 
-enum { M2_BF16 = 0, M2_TF32 = 1, M2_SPLIT = 2 };
+enum { M2_BF16 = 0, M2_TF32 = 1, M2_SPLIT = 2, M2_CONV = 3 };
 
 namespace m2tc {
 constexpr int BM = 256, BN = 256;               // tile of the pair
@@ -49,11 +59,14 @@ constexpr int MAX_STAGES = 24;
 constexpr size_t STAGES_BYTES = 131072;         // all stages together
 constexpr size_t STAGES_BYTES_1 = 196608;       // a single tile: nobody to keep in step with
 constexpr int THREADS = 192;
+constexpr int CONV_GROUPS = 3;                  // M2_CONV: groups of four converting warps on successive stages
+constexpr int CONV_THREADS = 128 * CONV_GROUPS;
+constexpr size_t STAGES_BYTES_CONV = 196608;    // with 131072 [262144,520] ran 552 us instead of 510, [30000,520] 78 instead of 68
 constexpr int MAX_TILES = 160;
 constexpr uint32_t TMEM_COLS = 512;
 template <int MODE> struct Shape {
     static constexpr int ELEM = MODE == M2_TF32 ? 4 : 2;
-    static constexpr int PARTS = MODE == M2_SPLIT ? 2 : 1;  // hi and lo
+    static constexpr int PARTS = MODE >= M2_SPLIT ? 2 : 1;  // hi and lo
     static constexpr int KROWS = MODE == M2_BF16 ? 64 : 32; // sample rows per stage
     static constexpr int KMMA = MODE == M2_TF32 ? 8 : 16;   // sample rows per MMA
     static constexpr int BOXC = 128 / ELEM;                 // columns per TMA box (128 bytes)
@@ -74,6 +87,7 @@ struct TileTable {
 struct Args {
     float *partials;                                   // [2 * cluster + block][HALF][BN]
     unsigned *status;
+    int d;                                             // columns of X
     int chunks_total, stages, nb, na;                  // nb, na: boxes of B and A per part in a stage
     int lo_row0;                                       // M2_SPLIT: first row of the lo part
     TileTable tab;
@@ -93,7 +107,7 @@ __device__ __forceinline__ int m2tc_tile_of(const m2tc::TileTable &t, int cluste
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(m2tc::THREADS, 1)
+__global__ void __launch_bounds__(MODE == M2_CONV ? m2tc::THREADS + m2tc::CONV_THREADS : m2tc::THREADS, 1)
 moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ m2tc::Args a)
 {
     using namespace m2tc;
@@ -104,11 +118,15 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t part_bytes = (uint32_t)((a.nb + a.na) * BOX_BYTES), stage_bytes = PARTS * part_bytes;
+    // M2_CONV: a box of fp32 becomes its hi and its lo box in place; else all hi boxes, then all lo boxes
+    constexpr int BOX_PITCH = MODE == M2_CONV ? 2 * BOX_BYTES : BOX_BYTES;
+    const uint32_t lo_off = MODE == M2_CONV ? BOX_BYTES : part_bytes;
     const int stages = a.stages;
     // an MMA reads 128 columns of A per block, na boxes of which were loaded: behind the last stage there is room for the others
-    uint64_t *bars = (uint64_t *)(smem + (size_t)stages * stage_bytes + (size_t)(NBOX - a.na) * BOX_BYTES);
+    uint64_t *bars = (uint64_t *)(smem + (size_t)stages * stage_bytes + (size_t)(NBOX - a.na) * BOX_PITCH);
     uint64_t *full = bars, *empty = bars + MAX_STAGES, *acc_full = bars + 2 * MAX_STAGES, *acc_empty = bars + 2 * MAX_STAGES + 2;
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * MAX_STAGES + 4);
+    uint64_t *raw = bars + 2 * MAX_STAGES + 4;          // M2_CONV: fp32 boxes have landed
+    uint32_t *tmem_slot = (uint32_t *)(raw + MAX_STAGES);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -121,6 +139,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     // narrow tiles are cheap to flush: chains half as long, as short as those of twice as many sample ranges
     const int FLUSH_CHUNKS = MODE == M2_BF16 && width <= HALF ? S::FLUSH_CHUNKS / 2 : S::FLUSH_CHUNKS;
     const bool alias = diag && width == BN;             // A columns == B columns in both blocks: one load serves both
+    const bool lead = diag && rows <= HALF;             // all rows in the first block, whose A holds its half of B as well
     const int chunks_per_split = (a.chunks_total + nsplit - 1) / nsplit;
     const int c_begin = split * chunks_per_split;
     int c_end = c_begin + chunks_per_split;
@@ -130,7 +149,9 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
-            mbar_init(&full[s], 1);          // leader's producer arrives once and announces the bytes of both blocks
+            // leader's producer arrives once and announces the bytes of both blocks; converting warps arrive each
+            mbar_init(&full[s], MODE == M2_CONV ? 8 : 1);
+            if (MODE == M2_CONV) mbar_init(&raw[s], 1);
             mbar_init(&empty[s], 1);         // one commit per use, delivered to both blocks
         }
         for (int b = 0; b < 2; ++b) {
@@ -158,18 +179,42 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         a.status[kWsDetailWord] = 0;
     }
 
-    if (warp == 0) {
+    // boxes of BU columns that block r loads: of B, and of A the ones that hold rows of the result (and nothing past the
+    // last column; what is not loaded makes entries that are never read)
+    constexpr int BU = MODE == M2_CONV ? 32 : BOXC;
+    auto boxes_b = [&](int r) {
+        int n = lead && r == 0 && rows > width / 2 ? rows : width / 2;
+        if (n > a.d - col - r * (width / 2)) n = a.d - col - r * (width / 2);
+        return n <= 0 ? 0 : (n + BU - 1) / BU;
+    };
+    auto boxes_a = [&](int r) {
+        const int n = rows - r * HALF;
+        return alias || lead || n <= 0 ? 0 : n >= HALF ? HALF / BU : (n + BU - 1) / BU;
+    };
+    const int col_a = row + (int)rank * HALF, col_b = col + (int)rank * (width / 2);
+    if (MODE == M2_CONV && warp == 0) {
+        // ---------------- TMA producer (both blocks): own boxes, fp32
+        if (elect_one()) {
+            prefetch_tmap(&tmap);
+            const int nb = boxes_b((int)rank), na = boxes_a((int)rank);
+            int s = 0;
+            uint32_t parity = 1;
+            for (int c = 0; c < nchunks; ++c) {
+                if (c >= stages && !mbar_wait(&empty[s], parity, abort_flag, a.status, 1)) break;
+                mbar_expect_tx(&raw[s], (uint32_t)((nb + na) * BOX_BYTES));
+                unsigned char *base = smem + (size_t)s * stage_bytes;
+                const int y = (c_begin + c) * KROWS;
+                for (int b = 0; b < nb; ++b) tma_load_2d(base + b * BOX_BYTES, &tmap, &raw[s], col_b + b * BU, y);
+                for (int b = 0; b < na; ++b) tma_load_2d(base + (2 * a.nb + b) * BOX_BYTES, &tmap, &raw[s], col_a + b * BU, y);
+                if (++s == stages) { s = 0; parity ^= 1u; }
+            }
+        }
+    } else if (warp == 0) {
         // ---------------- TMA producer (both blocks): own boxes, completion counted on the leader's barrier
         if (elect_one()) {
             prefetch_tmap(&tmap);
-            // boxes of A that hold columns of X (the others would only make rows that are never read)
-            auto boxes_a = [&](int r) {
-                const int left = rows - r * HALF;
-                return alias || left <= 0 ? 0 : left >= HALF ? NBOX : (left + BOXC - 1) / BOXC;
-            };
-            const int nb = (width / 2 + BOXC - 1) / BOXC, na = boxes_a((int)rank);
-            const uint32_t tx = (uint32_t)((2 * nb + boxes_a(0) + boxes_a(1)) * PARTS * BOX_BYTES);
-            const int col_a = row + (int)rank * HALF, col_b = col + (int)rank * (width / 2);
+            const int nb = boxes_b((int)rank), na = boxes_a((int)rank);
+            const uint32_t tx = (uint32_t)((boxes_b(0) + boxes_b(1) + boxes_a(0) + boxes_a(1)) * PARTS * BOX_BYTES);
             const uint32_t bar0 = map_to_cta(smem_u32(full), 0);
             int s = 0;
             uint32_t parity = 1;
@@ -194,12 +239,12 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         // ---------------- MMA issuer (leader only)
         if (rank == 0 && elect_one()) {
             const uint32_t idesc = make_idesc(MODE == M2_TF32 ? 2 : 1, 1, 1, BM, (uint32_t)width);
-            const uint32_t a_off = alias ? 0u : (uint32_t)(a.nb * BOX_BYTES);
+            const uint32_t a_off = alias || lead ? 0u : (uint32_t)(a.nb * BOX_PITCH);
             const uint32_t sb0 = smem_u32(smem);
             // bf16: groups of 8 sample rows, 16-byte swizzle units; fp32 read as TF32: groups of 4, 32-byte units
-            const uint64_t adesc_base = make_smem_desc(sb0 + a_off, BOX_BYTES, MODE == M2_TF32 ? 512 : 1024, MODE == M2_TF32 ? 1 : 2);
-            const uint64_t bdesc_base = make_smem_desc(sb0, BOX_BYTES, MODE == M2_TF32 ? 512 : 1024, MODE == M2_TF32 ? 1 : 2);
-            const uint64_t lo = (uint64_t)(part_bytes >> 4);
+            const uint64_t adesc_base = make_smem_desc(sb0 + a_off, BOX_PITCH, MODE == M2_TF32 ? 512 : 1024, MODE == M2_TF32 ? 1 : 2);
+            const uint64_t bdesc_base = make_smem_desc(sb0, BOX_PITCH, MODE == M2_TF32 ? 512 : 1024, MODE == M2_TF32 ? 1 : 2);
+            const uint64_t lo = (uint64_t)(lo_off >> 4);
             bool ok = true;
             int c = 0, s = 0;
             uint32_t parity = 0;
@@ -211,7 +256,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                 const int ce = (c + FLUSH_CHUNKS < nchunks) ? c + FLUSH_CHUNKS : nchunks;
                 uint32_t accumulate = 0;
                 for (; c < ce; ++c) {
-                    if (!mbar_wait(&full[s], parity, abort_flag, a.status, 2)) {
+                    if (!mbar_wait<MODE == M2_CONV>(&full[s], parity, abort_flag, a.status, 2)) {
                         ok = false;
                         break;
                     }
@@ -226,7 +271,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                         if (MODE == M2_TF32) mma_tf32_pair(d_tmem, ak, bk, idesc, accumulate);
                         else mma_bf16_pair(d_tmem, ak, bk, idesc, accumulate);
                         accumulate = 1;
-                        if (MODE == M2_SPLIT) {
+                        if (PARTS == 2) {
                             mma_bf16_pair(d_tmem, ak, bk + lo, idesc, 1u);
                             mma_bf16_pair(d_tmem, ak + lo, bk, idesc, 1u);
                         }
@@ -236,6 +281,63 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                 }
                 tc_commit_pair(&acc_full[buf]);
             }
+        }
+    } else if (MODE == M2_CONV && warp >= THREADS / 32) {
+        // ---------------- converting warps (both blocks): x = hi + lo, each in the form that a copy of boxes of 64 columns x
+        // 32 rows with the 128-byte swizzle leaves.  A warp takes eight rows of all boxes of a stage.  They are two runs of
+        // 1024 bytes of every pair of boxes of 32 columns, the first of which becomes hi and the second lo: in place.
+        constexpr int H = 4, PAIRS_B = 2;
+        const int cw = warp - THREADS / 32, group = cw >> 2;
+        const int r0 = lane >> 4, c4 = (lane & 15) * 4;           // rows r0 + 2h of the eight, columns c4 .. c4+3
+        const int nb = boxes_b((int)rank), na = boxes_a((int)rank);
+        const uint32_t bar0 = map_to_cta(smem_u32(full), 0);
+        uint32_t from[H], to[H];
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const int r = r0 + 2 * h;
+            from[h] = (uint32_t)((cw & 3) * 1024 + (c4 >> 5) * BOX_BYTES + r * 128 + ((((c4 >> 2) & 7) ^ r) << 4));
+            to[h] = (uint32_t)((cw & 3) * 1024 + r * 128 + (((c4 >> 3) ^ r) << 4) + (c4 & 4) * 2);
+        }
+        int s = group % stages;
+        uint32_t parity = (uint32_t)(group / stages) & 1u;
+        bool ok = true;
+        for (int c = group; c < nchunks; c += CONV_GROUPS) {
+            ok = ok && mbar_wait(&raw[s], parity, abort_flag, a.status, 1);
+            unsigned char *stage = smem + (size_t)s * stage_bytes;
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const int n = side ? na : nb;
+                unsigned char *p = stage + (side ? a.nb * BOX_PITCH : 0);
+                float4 v[PAIRS_B][H];
+#pragma unroll
+                for (int q = 0; q < PAIRS_B; ++q)
+                    if (2 * q + (c4 >> 5) < n) {
+#pragma unroll
+                        for (int h = 0; h < H; ++h) v[q][h] = *reinterpret_cast<const float4 *>(p + q * BOX_PITCH + from[h]);
+                    }
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < PAIRS_B; ++q)
+                    if (2 * q + (c4 >> 5) < n) {
+#pragma unroll
+                        for (int h = 0; h < H; ++h) {
+                            const float4 x = v[q][h];
+                            const __nv_bfloat162 h0 = __floats2bfloat162_rn(x.x, x.y), h1 = __floats2bfloat162_rn(x.z, x.w);
+                            const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
+                            const __nv_bfloat162 l0 = __floats2bfloat162_rn(x.x - f0.x, x.y - f0.y), l1 = __floats2bfloat162_rn(x.z - f1.x, x.w - f1.y);
+                            unsigned char *w = p + q * BOX_PITCH + to[h];
+                            *reinterpret_cast<uint2 *>(w) =
+                                make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
+                            *reinterpret_cast<uint2 *>(w + BOX_BYTES) =
+                                make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
+                        }
+                    }
+            }
+            fence_proxy_async();          // generic writes, read by the tensor core
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(bar0 + (uint32_t)(s * sizeof(uint64_t)));
+            s += CONV_GROUPS;
+            while (s >= stages) { s -= stages; parity ^= 1u; }
         }
     } else {
         // ---------------- epilogue (both blocks): own 128 rows of the tile; what is past the tile's rows or
@@ -394,9 +496,10 @@ struct M2TcTiles {
         p->tab.width[n] = (unsigned char)(width / 32);
         p->tab.diag[n] = diag ? 1 : 0;
         cost[n] = m2tc_cost(width);
-        const int nb = (width / 2 + S::BOXC - 1) / S::BOXC;
+        const bool lead = diag && rows <= HALF;
+        const int cols_b = lead && rows > width / 2 ? rows : width / 2, nb = (cols_b + S::BOXC - 1) / S::BOXC;
         if (nb > p->nb) p->nb = nb;
-        if (!(diag && width == BN)) {
+        if (!(diag && width == BN) && !lead) {
             const int na = rows >= HALF ? S::NBOX : (rows + S::BOXC - 1) / S::BOXC;
             if (na > p->na) p->na = na;
         }
@@ -419,9 +522,12 @@ static void m2tc_finish(M2TcPlan &p, const M2TcTiles &t, int64_t N)
     if (chunks > (int64_t(1) << 30)) return;
     p.chunks_total = (int)chunks;
     const size_t stage = (size_t)S::PARTS * (p.nb + p.na) * S::BOX_BYTES;
-    p.stages = (int)((n == 1 ? STAGES_BYTES_1 : STAGES_BYTES) / stage);
+    p.stages = (int)((MODE == M2_CONV ? STAGES_BYTES_CONV : n == 1 ? STAGES_BYTES_1 : STAGES_BYTES) / stage);
     if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
-    p.smem = (size_t)p.stages * stage + (size_t)(S::NBOX - p.na) * S::BOX_BYTES + 1024 + 512;
+    // a stage always belongs to the same group of converting warps: a group that came by only every other time could not
+    // tell the two apart by the parity of the barrier
+    if (MODE == M2_CONV) p.stages -= p.stages % CONV_GROUPS;
+    p.smem = (size_t)p.stages * stage + (size_t)(S::NBOX - p.na) * S::BOX_BYTES * (MODE == M2_CONV ? 2 : 1) + 1024 + 1024;
     // Clusters (one per pair of SMs) go to the tiles in proportion to their cost, the remaining ones each to the tile whose
     // share of the samples takes longest; then every tile gives back what it does not need to keep up with the slowest.
     // Tiles of equal width so get equal shares: their clusters run in step and share X in L2 (with unequal shares the wide
@@ -536,22 +642,23 @@ static M2TcPlan m2tc_plan_pairs(int64_t N, const PairLayout &L)
 // of `features` features and the result goes to their packed 4-simplex.
 template <int MODE>
 static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int64_t d, int64_t ldx, float *out, float *partials,
-                             unsigned *status, cudaStream_t stream, int lo_row0 = 0, const unsigned *pairs = nullptr, int features = 0)
+                             unsigned *status, cudaStream_t stream, int64_t lo_row0 = 0, const unsigned *pairs = nullptr, int features = 0)
 {
     using S = m2tc::Shape<MODE>;
     CUtensorMap tmap;
-    if (!tc::make_tmap_2d(&tmap, MODE == M2_TF32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, X, (uint64_t)rows,
-                          (uint64_t)d, (uint64_t)ldx * S::ELEM, S::BOXC, S::KROWS,
+    if (!tc::make_tmap_2d(&tmap, MODE == M2_TF32 || MODE == M2_CONV ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, X, (uint64_t)rows,
+                          (uint64_t)d, (uint64_t)ldx * (MODE == M2_CONV ? 4 : S::ELEM), MODE == M2_CONV ? 32 : S::BOXC, S::KROWS,
                           MODE == M2_TF32 ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B))
         return ST_ERR_CUDA;
     m2tc::Args a;
     a.partials = partials; a.status = status;
-    a.chunks_total = q.chunks_total; a.stages = q.stages; a.nb = q.nb; a.na = q.na; a.lo_row0 = lo_row0;
+    a.chunks_total = q.chunks_total; a.stages = q.stages; a.nb = q.nb; a.na = q.na; a.lo_row0 = (int)lo_row0; a.d = (int)d;
+   
     a.tab = q.tab;
     if (!ensure_dynamic_smem(moment2_tc_kernel<MODE>, q.smem)) return ST_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)q.tab.first[q.tab.ntiles]);
-    cfg.blockDim = dim3(m2tc::THREADS);
+    cfg.blockDim = dim3(MODE == M2_CONV ? m2tc::THREADS + m2tc::CONV_THREADS : m2tc::THREADS);
     cfg.dynamicSmemBytes = q.smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -635,75 +742,20 @@ st_status moment2_bf16_tc(const void *X, int64_t N, int64_t d, int64_t ldx, floa
 }
 
 // ---------------------------------------------------------------------------------------------
-// fp32 input at the fp32 tolerance on the tensor cores (ST_FLAG_TC_SPLIT): every x is written once as
-// hi = bf16(x) and lo = bf16(x - hi) (x - hi - lo is below 2^-16 |x|), and the pair kernel adds
-// hi^T hi + hi^T lo + lo^T hi from one stage of both parts (lo^T lo is below 2^-16 of the result).
-// The split pass reads X once and writes the same number of bytes: HBM bound.
-__global__ void __launch_bounds__(256)
-moment2_split_rows_kernel(const float *__restrict__ X, int64_t N, int64_t Np, int d, int64_t ldx, __nv_bfloat16 *__restrict__ Z)
-{
-    // Z: [2 Np, d]; rows 0 .. Np-1 hi, rows Np .. 2Np-1 lo; rows N .. Np-1 of either part are zero
-    pdl_wait();
-    pdl_trigger();
-    const int64_t quads = (int64_t)Np * (d / 4);
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < quads; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t n = e / (d / 4);
-        const int c = (int)(e - n * (d / 4)) * 4;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (n < N) x = __ldcs(reinterpret_cast<const float4 *>(X + n * ldx + c));
-        const __nv_bfloat162 h0 = __floats2bfloat162_rn(x.x, x.y), h1 = __floats2bfloat162_rn(x.z, x.w);
-        const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
-        const __nv_bfloat162 l0 = __floats2bfloat162_rn(x.x - f0.x, x.y - f0.y), l1 = __floats2bfloat162_rn(x.z - f1.x, x.w - f1.y);
-        *reinterpret_cast<uint2 *>(Z + n * d + c) =
-            make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
-        *reinterpret_cast<uint2 *>(Z + (Np + n) * d + c) =
-            make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
-    }
-}
-
-struct M2SplitPlan {
-    M2TcPlan q;
-    int64_t Np;
-    size_t z_off, part_off, total;
-    bool ok;
-};
-
-static M2SplitPlan m2_split_plan(int64_t N, int64_t d, unsigned flags)
-{
-    M2SplitPlan p{};
-    p.ok = false;
-    if (N <= 0 || d <= 0 || d % 8 != 0 || d > 4096 || N > (int64_t(1) << 29)) return p;
-    p.Np = (N + 63) / 64 * 64;
-    p.q = m2tc_plan<M2_SPLIT>(N, d, flags);
-    if (!p.q.ok) return p;
-    p.z_off = kWsHeaderBytes;
-    p.part_off = round_up(p.z_off + (size_t)2 * p.Np * d * sizeof(__nv_bfloat16), 256);
-    p.total = p.part_off + p.q.partial_bytes;
-    p.ok = true;
-    return p;
-}
-
+// fp32 input at the fp32 tolerance on the tensor cores (ST_FLAG_TC_SPLIT): x = hi + lo with hi = bf16(x) and
+// lo = bf16(x - hi) (what is left is below 2^-16 |x|), and the pair kernel adds hi^T hi + hi^T lo + lo^T hi (lo^T lo is
+// below 2^-16 of the result).
 size_t moment2_split_tc_workspace(int64_t N, int64_t d, unsigned flags)
 {
-    const M2SplitPlan p = m2_split_plan(N, d, flags);
-    return p.ok ? p.part_off + m2tc_partial_room<M2_SPLIT>(N, d, p.q.partial_bytes) : 0;
+    return d % 8 != 0 || N > (int64_t(1) << 29) ? 0 : m2tc_workspace<M2_CONV>(N, d, flags);
 }
 
 st_status moment2_split_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
                            unsigned flags, cudaStream_t stream)
 {
     if (d % 8 != 0 || ldx % 4 != 0) return ST_ERR_ALIGN;
-    const M2SplitPlan p = m2_split_plan(N, d, flags);
-    if (!p.ok) return ST_ERR_UNSUPPORTED;
-    if (!ws || ws_bytes < p.total) return ST_ERR_WORKSPACE;
-    if (!aligned256(ws)) return ST_ERR_ALIGN;
-    __nv_bfloat16 *Z = (__nv_bfloat16 *)((unsigned char *)ws + p.z_off);
-    const int64_t quads = p.Np * (d / 4);
-    const int64_t want = (quads + 255) / 256;
-    const int64_t cap = (int64_t)sm_count_or_default() * 16;
-    const st_status rc = launch(moment2_split_rows_kernel, (unsigned)(want < cap ? want : cap), 256, 0, stream, X, N, p.Np, (int)d, ldx, Z);
-    if (rc != ST_OK) return rc;
-    return m2tc_launch<M2_SPLIT>(p.q, Z, 2 * p.Np, d, d, out, (float *)((unsigned char *)ws + p.part_off), (unsigned *)ws, stream, (int)p.Np);
+    if (N > (int64_t(1) << 29)) return ST_ERR_UNSUPPORTED;
+    return m2tc_run<M2_CONV>(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
 }
 
 // The products of pair features that the caller has written (moment4.cu), straight into the packed 4-simplex.  split:

@@ -595,6 +595,22 @@ def test_moment4_more_than_64_features(st, flag_name, N, d):
         assert abs(lhs - rhs) <= (5e-3 if flags else TOL_F32) * float(np.sum(np.abs(Xd).sum(axis=1) ** 4))
 
 
+@pytest.mark.parametrize("N,d,ldx", [(1, 8, 8), (31, 40, 44), (33, 128, 128), (5000, 136, 136), (9001, 200, 200),
+                                     (4097, 264, 300), (70001, 8, 8), (70001, 264, 264)])
+def test_moment2_split_converted_in_the_kernel(st, N, d, ldx):
+    # one and two row blocks, ragged boxes, samples and pitches, rings that wrap many times.  x - hi - lo and lo times lo
+    # are each below 2^-16 relative, so what is dropped stays below 4 * 2^-16 of the sum of magnitudes, inside TOL_F32.
+    X = workloads.draw((N, ldx), "normal", 900 + N + d)
+    Xd, out = dev(X), guarded(st, d * (d + 1) // 2)
+    nbytes = st.st_workspace_bytes(st.ST_OP_SYM_MOMENT2, N, d, st.ST_F32, 0, st.ST_FLAG_TC_SPLIT)
+    ws = guarded(st, nbytes, torch.uint8)
+    rc = st.lib().st_sym_moment2(Xd.data_ptr(), st.ST_F32, N, d, ldx, out.data_ptr(), ws.data_ptr(), nbytes, st.ST_FLAG_TC_SPLIT,
+                                 torch.cuda.current_stream().cuda_stream)
+    assert rc == st.ST_OK
+    T, S = oracle.moment2(np.ascontiguousarray(X[:, :d]))
+    assert oracle.rel_err(expand2(st, out, d), T, S) <= TOL_F32, (N, d)
+
+
 @pytest.mark.parametrize("flag_name", [None, "ST_FLAG_TC_BF16"])
 @pytest.mark.parametrize("d", [22, 23, 31, 32, 37, 38, 44, 45, 46, 48, 64, 71, 90])
 def test_moment4_every_entry_whatever_ranges_the_features_are_cut_into(st, d, flag_name):
