@@ -28,6 +28,9 @@ namespace st {
 constexpr int M2S_MAX_THREADS = 256;
 constexpr int M2S_MAX_BLOCKS = 31;         // column blocks: one item per thread at most (d <= 248; dense control: 22 blocks)
 constexpr int M2S_BUFFERS = 3;
+constexpr int M2S_CLUSTER = 16;            // one-launch form: blocks of a cluster
+constexpr int M2S_CLUSTER_THREADS = 128;   // half the threads: half the sums to add ([4096,64] 7.1 us, with 256 threads 7.9)
+constexpr int M2S_CLUSTER_ITEMS = 5;       // at most, per cluster ([4096,100]: five 9.3 us, three 15.2; [4096,64]: 7.1, nine 8.1)
 constexpr int M2S_STAGE_BYTES = 57344;     // upper bound of one stage (3 stages + slack fit in 227 KB)
 
 // bulk copy global -> shared of `bytes` (a multiple of 16, both addresses 16-byte aligned),
@@ -85,16 +88,35 @@ struct M2SmallArgs {
     unsigned *status;     // workspace header (status and detail words)
     int64_t N, ldx, rows_per_slice;
     int d, pitch, nbk, nitems, rg, rpg, dense, bar_floats;
+    float *out;           // CLUSTER: the result
+    int items_all;        // CLUSTER: nitems counts those of a cluster
 };
 
 // column of element e (0..7) of column block b
 __device__ __forceinline__ int m2s_column(int b, int e, int half) { return (e < 4) ? 4 * b + e : half + 4 * b + (e - 4); }
 
+// Whether element k of an item is an output, and which: not the second tile of the odd item out; not the lower half of a
+// diagonal tile (the dense control also computes the tiles below the diagonal and discards them here); not the padding of
+// the last column blocks.
+__device__ __forceinline__ bool m2s_output(int k, int item, int nbk, bool dense, int d, int64_t &at)
+{
+    const int i8 = (k >> 3) & 7, j8 = k & 7;
+    int x, p, q;
+    m2s_item(item, nbk, dense, x, p, q);
+    const int y = (k < 64) ? p : q;
+    const int ci = m2s_column(x, i8, 4 * nbk), cj = m2s_column(y, j8, 4 * nbk);
+    at = tri_encode(d, ci < cj ? ci : cj, ci < cj ? cj : ci);
+    return y >= 0 && !((x == y && i8 > j8) || (dense && x > y)) && ci < d && cj < d;
+}
+
 // BULK: rows start on 16-byte boundaries and arrive by bulk copies, in shared memory at their own pitch; otherwise
 // they are copied word by word to a pitch rounded up to 16 bytes (one copy instruction per 32 words, against more
 // than 64 FMA instructions).  Either way a tile that reaches past column d reads whatever follows the row: only
 // sums that are dropped contain it.  [50021,75]: 23 us the call, 71 with the plain 64 x 64 tiles that served it before.
-template <bool BULK>
+// CLUSTER: few samples, one launch.  A cluster of M2S_CLUSTER blocks (gridDim.x) owns nitems work items (gridDim.y clusters),
+// its blocks own slices of the samples, and the sums of the blocks are added through distributed shared memory instead of
+// partials and a second launch.
+template <bool BULK, bool CLUSTER>
 __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const M2SmallArgs a)
 {
     extern __shared__ __align__(16) float smem[];
@@ -106,7 +128,8 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
     const bool active = item_rg < a.rg;
     const int half = 4 * a.nbk;
     int bs, bp, bq;
-    m2s_item(item, a.nbk, a.dense != 0, bs, bp, bq);
+    const int item0 = CLUSTER ? (int)blockIdx.y * nitems : 0;
+    m2s_item(CLUSTER ? (item0 + item < a.items_all ? item0 + item : 0) : item, a.nbk, a.dense != 0, bs, bp, bq);
     const int os = 4 * bs, op = 4 * bp, oq = bq < 0 ? op : 4 * bq;
 
     float accp[8][8], accq[8][8];                      // tiles {s,p} and {s,q}
@@ -129,7 +152,7 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
     pdl_wait();
     pdl_trigger();
     if (tid == 0) {
-        if (blockIdx.x == 0) {      // a time-out report can only be written 2^24 failed polls later
+        if (blockIdx.x == 0 && blockIdx.y == 0) {      // a time-out report can only be written 2^24 failed polls later
             a.status[kWsStatusWord] = 0;
             a.status[kWsDetailWord] = 0;
         }
@@ -248,7 +271,7 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
     int parts = nthreads / nout;
     if (parts < 1) parts = 1;
     if (parts > a.rg) parts = a.rg;
-    float *mine = a.partials + (size_t)blockIdx.x * nout;
+    float *mine = CLUSTER ? red + 128 * cells + M2S_MAX_THREADS : a.partials + (size_t)blockIdx.x * nout;
     if (parts == 1) {
         for (int o = tid; o < nout; o += nthreads) {
             const int k = o / nitems, t = o - k * nitems;
@@ -279,6 +302,23 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
             mine[tid] = sum;
         }
     }
+    if (CLUSTER) {
+        tc::cluster_sync_all();                        // all blocks' sums are written
+        const int per = (nout + M2S_CLUSTER - 1) / M2S_CLUSTER, o_end = nout < ((int)blockIdx.x + 1) * per ? nout : ((int)blockIdx.x + 1) * per;
+        for (int o = (int)blockIdx.x * per + tid; o < o_end; o += nthreads) {
+            const int k = o / nitems, t = item0 + o - k * nitems;
+            int64_t at;
+            if (t >= a.items_all || !m2s_output(k, t, a.nbk, a.dense != 0, a.d, at)) continue;
+            float v[M2S_CLUSTER], sum = 0.f;
+#pragma unroll
+            for (int r = 0; r < M2S_CLUSTER; ++r)
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v[r]) : "r"(tc::map_to_cta(tc::smem_u32(mine + o), (uint32_t)r)));
+#pragma unroll
+            for (int r = 0; r < M2S_CLUSTER; ++r) sum += v[r];
+            if (ST_BOUNDS_OK(at, tri_rows(a.d), 2)) a.out[at] = sum;
+        }
+        tc::cluster_sync_all();                        // no block leaves while its sums are read
+    }
 }
 
 // out[p(ci,cj)] = sum over the slices of element (k, item) of the partials: a block owns 32 elements, warp w adds the
@@ -291,15 +331,8 @@ moment2_small_reduce_kernel(const float *__restrict__ partials, float *__restric
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int o = blockIdx.x * 32 + lane;              // < nitems * 128, a multiple of 32
     const int k = o / nitems, item = o - k * nitems;
-    const int i8 = (k >> 3) & 7, j8 = k & 7;
-    int x, p, q;
-    m2s_item(item, nbk, dense != 0, x, p, q);
-    const int y = (k < 64) ? p : q;
-    const int ci = m2s_column(x, i8, 4 * nbk), cj = m2s_column(y, j8, 4 * nbk);
-    // not an output: the second tile of the odd item out; the lower half of a diagonal tile (the dense control also
-    // computes the tiles below the diagonal and discards them here); the padding of the last column blocks
-    const bool use = y >= 0 && !((x == y && i8 > j8) || (dense && x > y)) && ci < d && cj < d;
-    const int64_t at = tri_encode(d, ci < cj ? ci : cj, ci < cj ? cj : ci);
+    int64_t at;
+    const bool use = m2s_output(k, item, nbk, dense != 0, d, at);
     pdl_wait();
     pdl_trigger();
     const size_t stride = (size_t)nitems * 128;
@@ -366,15 +399,74 @@ static M2SmallPlan moment2_small_plan(int64_t N, int64_t d, unsigned flags)
     return p;
 }
 
+// Plan of the one-launch form: clusters of blocks over the items, blocks over the samples.
+static M2SmallPlan moment2_cluster_plan(int64_t N, int64_t d, unsigned flags, int &clusters)
+{
+    M2SmallPlan p;
+    p.nbk = (int)(d + 7) / 8;
+    const int all = m2s_nitems(p.nbk, (flags & ST_FLAG_DENSE_CONTROL) != 0);
+    clusters = (all + M2S_CLUSTER_ITEMS - 1) / M2S_CLUSTER_ITEMS;
+    p.nitems = (all + clusters - 1) / clusters;
+    clusters = (all + p.nitems - 1) / p.nitems;
+    p.pitch = (int)(d + 3) / 4 * 4;
+    const int max_stage_rows = M2S_STAGE_BYTES / (4 * p.pitch);
+    p.rg = M2S_CLUSTER_THREADS / p.nitems;
+    if (p.rg > max_stage_rows / 8) p.rg = max_stage_rows / 8;
+    p.threads = (p.nitems * p.rg + 31) / 32 * 32;
+    p.slices = M2S_CLUSTER;
+    p.rows_per_slice = (N + M2S_CLUSTER - 1) / M2S_CLUSTER;
+    p.rpg = p.rows_per_slice >= 16 * p.rg ? 8 : 4;
+    const size_t cells = (size_t)m2s_red_pitch(p.rg, p.nitems);
+    const size_t main_bytes = (size_t)M2S_BUFFERS * p.rg * p.rpg * p.pitch * sizeof(float) + 32;
+    const size_t sum_bytes = (128 * cells + (size_t)M2S_MAX_THREADS + 128 * (size_t)p.nitems) * sizeof(float);
+    p.data_bytes = round_up(main_bytes > sum_bytes ? main_bytes : sum_bytes, 16);
+    p.smem = p.data_bytes + 64;
+    p.partial_bytes = 0;
+    return p;
+}
+
+// Few samples: one launch instead of two, about 2 us of the host's time per call.  On the GPU (us, one launch / two):
+// [256,64] 5.0 / 7.5, [4096,8] 4.0 / 5.8, [4096,64] 7.1 / 7.7, [4096,100] 9.3 / 12.3, but [16384,24] 8.3 / 6.3 and
+// [16384,64] 12.0 / 10.1: its blocks are fewer, and every cluster reads all of X.  Copies word by word: [256,75] 5.6 / 8.4,
+// [4096,75] 12.2 / 9.9.
+static bool m2s_use_cluster(int64_t N, int64_t d, bool bulk) { return N * d <= (bulk ? 300000 : 100000); }
+
 size_t moment2_small_workspace(int64_t N, int64_t d, unsigned flags)
 {
     return kWsHeaderBytes + moment2_small_plan(N, d, flags).partial_bytes;
 }
 
+template <class Kernel>
+static st_status m2s_launch_cluster(Kernel kernel, int clusters, const M2SmallPlan &p, const M2SmallArgs &a, cudaStream_t stream)
+{
+    if (!ensure_dynamic_smem(kernel, p.smem) || (M2S_CLUSTER > 8 && !allow_large_clusters(kernel))) return ST_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(M2S_CLUSTER, (unsigned)clusters);
+    cfg.blockDim = dim3((unsigned)p.threads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = M2S_CLUSTER;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    if (cudaLaunchKernelEx(&cfg, kernel, a) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ST_ERR_CUDA;
+    }
+    return ST_OK;
+}
+
 st_status moment2_small(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
                         unsigned flags, cudaStream_t stream)
 {
-    const M2SmallPlan p = moment2_small_plan(N, d, flags);
+    const bool bulk = d % 4 == 0 && ldx % 4 == 0;
+    int clusters = 0;
+    const M2SmallPlan p = m2s_use_cluster(N, d, bulk) ? moment2_cluster_plan(N, d, flags, clusters) : moment2_small_plan(N, d, flags);
     if (!ws || ws_bytes < kWsHeaderBytes + p.partial_bytes) return ST_ERR_WORKSPACE;
     if (!aligned256(ws)) return ST_ERR_ALIGN;
     M2SmallArgs a;
@@ -386,11 +478,17 @@ st_status moment2_small(const float *X, int64_t N, int64_t d, int64_t ldx, float
     a.status = (unsigned *)ws;
     a.bar_floats = (int)(p.data_bytes / sizeof(float));
     a.dense = (flags & ST_FLAG_DENSE_CONTROL) ? 1 : 0;
+    if (clusters > 0) {
+        a.out = out;
+        a.items_all = m2s_nitems(p.nbk, a.dense != 0);
+        return bulk ? m2s_launch_cluster(moment2_small_kernel<true, true>, clusters, p, a, stream)
+                    : m2s_launch_cluster(moment2_small_kernel<false, true>, clusters, p, a, stream);
+    }
     auto run = [&](auto kernel) {
         if (!ensure_dynamic_smem(kernel, p.smem)) return ST_ERR_CUDA;
         return launch(kernel, p.slices, p.threads, p.smem, stream, a);
     };
-    const st_status rc = (d % 4 == 0 && ldx % 4 == 0) ? run(moment2_small_kernel<true>) : run(moment2_small_kernel<false>);
+    const st_status rc = bulk ? run(moment2_small_kernel<true, false>) : run(moment2_small_kernel<false, false>);
     if (rc != ST_OK) return rc;
     return launch(moment2_small_reduce_kernel, (unsigned)(p.nitems * 128 / 32), 256, 0, stream, a.partials, out, (int)d, p.nbk, p.slices, a.dense, p.nitems);
 }

@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cstddef>
 #include <map>
+#include <set>
 #include <mutex>
 #include <utility>
 #include "structtensor.h"
@@ -91,6 +92,24 @@ inline bool ensure_dynamic_smem(Kernel kernel, size_t bytes)
         return false;
     }
     have = bytes;
+    return true;
+}
+
+// Clusters of more than eight blocks have to be allowed per kernel and device.
+template <typename Kernel>
+inline bool allow_large_clusters(Kernel kernel)
+{
+    static std::mutex lock;
+    static std::set<std::pair<const void *, int>> done;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> guard(lock);
+    if (done.count(std::make_pair((const void *)kernel, dev))) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    done.insert(std::make_pair((const void *)kernel, dev));
     return true;
 }
 

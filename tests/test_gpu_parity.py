@@ -259,6 +259,18 @@ def test_moment2_f32_many_features(st, N, d):
         assert oracle.rel_err(expand2(st, out, d), Tw, Sw) <= TOL_F32
 
 
+@pytest.mark.parametrize("N,d", [(1, 1), (15, 4), (17, 8), (600, 13), (4096, 24), (4096, 64), (3001, 100), (200, 248), (1600, 61)])
+def test_moment2_f32_one_launch(st, N, d):
+    # few samples: clusters of blocks, also with fewer samples than blocks, an item short in the last cluster, word copies;
+    # fp32 sums of N terms in a fixed order
+    X = workloads.draw((N, d), "normal", 170 + N + d)
+    T, S = oracle.moment2(X)
+    for flags in (0, st.ST_FLAG_DENSE_CONTROL):
+        got = st.st_sym_moment2(dev(X), flags=flags)
+        assert oracle.rel_err(expand2(st, got, d), T, S) <= TOL_F32, (N, d, flags)
+        assert torch.equal(got, st.st_sym_moment2(dev(X), flags=flags))
+
+
 # register-tile kernel (up to 248 features, rows copied whole or word by word) and 128 x 128 tiles with a last tile
 # column that is one column, half or all but one column wide; slices from one row up, splits with a ragged tail
 @pytest.mark.parametrize("N,d", [(1, 7), (147, 9), (3001, 15), (20011, 33), (4097, 65), (1185, 75), (500, 121), (257, 176),
