@@ -395,7 +395,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 // to the place of its 4-tuple in the packed 4-simplex, if this is the product that was chosen for that tuple.
 template <bool PAIRS, int V>
 __global__ void __launch_bounds__(256)
-moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int features, int64_t out_elems,
+moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int features, int within, int64_t out_elems,
                          const unsigned *__restrict__ pairs, const __grid_constant__ m2tc::TileTable tab)
 {
     using namespace m2tc;
@@ -415,21 +415,8 @@ moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__
         const int u = u0 + warp / wps, r = u / uw, c = (u - r * uw) * (32 * V) + V * lane;   // this thread's columns c .. c+V-1
         const int gi = row + r, gj = col + c;
         const bool in_tile = r < rows && c < width;
-        const int at0 = PAIRS ? 0 : (int)tri_encode(d, gi, gj);
-        int at[V];                                         // where the columns go to, -1: not an output
-        bool use = false;
-#pragma unroll
-        for (int x = 0; x < V; ++x) {
-            at[x] = -1;
-            if (PAIRS) {
-                int i, j, k, l;
-                if (in_tile && gj + x < d && pair_product(pairs[gi], pairs[gj + x], i, j, k, l))
-                    at[x] = (int)simp4_encode(features, i, j, k, l);
-            } else if (in_tile && gi <= gj + x && gj + x < d) {
-                at[x] = at0 + x;
-            }
-            use |= at[x] >= 0;
-        }
+        // what is loaded does not wait for what has to be looked up
+        const bool use = in_tile && gj + V > (PAIRS && gi >= within ? 0 : gi) && gj < d;
         float s[V];
 #pragma unroll
         for (int x = 0; x < V; ++x) s[x] = 0.f;
@@ -451,6 +438,18 @@ moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__
             for (int e = 0; e < BATCH; ++e)
 #pragma unroll
                 for (int x = 0; x < V; ++x) s[x] += v[e][x];
+        }
+        int at[V];                                         // where the columns go to, -1: not an output
+        const int at0 = PAIRS ? 0 : (int)tri_encode(d, gi, gj);
+#pragma unroll
+        for (int x = 0; x < V; ++x) {
+            at[x] = -1;
+            if (PAIRS) {
+                int i, j, k, l;
+                if (use && gj + x < d && pair_product(pairs[gi], pairs[gj + x], i, j, k, l)) at[x] = pair_place(features, i, j, k, l);
+            } else if (use && gi <= gj + x && gj + x < d) {
+                at[x] = at0 + x;
+            }
         }
         if (wps > 1) {
 #pragma unroll
@@ -599,7 +598,8 @@ static void pair_tiles(const PairLayout &L, F f)
 // tiles.  (Four and a smaller one: 45 features take 256 rows as 11, 11, 11, 10 and 2, but 261 as five nines.)
 PairLayout pair_layout(int features)
 {
-    PairLayout best{};
+    thread_local PairLayout best{};                        // of the last call: the size query and the call itself need it
+    if (best.features == features) return best;
     double least = 0;
     for (int option = 0; option < 4 + features / 4; ++option) {
         const int last = option < 3 ? 0 : option - 3, m = option < 3 ? option + 1 : 4;   // m equal ranges and the last one
@@ -628,9 +628,14 @@ PairLayout pair_layout(int features)
 }
 
 template <int MODE>
-static M2TcPlan m2tc_plan_pairs(int64_t N, const PairLayout &L)
+static const M2TcPlan &m2tc_plan_pairs(int64_t N, const PairLayout &L)
 {
-    M2TcPlan p{};
+    thread_local M2TcPlan p{};                             // of the last call, as above
+    thread_local int64_t of[3] = {0, 0, 0};
+    const int64_t now[3] = {N, L.features, sm_count_or_default()};
+    if (of[0] == now[0] && of[1] == now[1] && of[2] == now[2]) return p;
+    for (int i = 0; i < 3; ++i) of[i] = now[i];
+    p = M2TcPlan{};
     M2TcTiles t{&p, 0, {}};
     bool ok = true;
     pair_tiles(L, [&](int row, int rows, int col, int width, bool diag) { ok = ok && t.add<MODE>(row, rows, col, width, diag); });
@@ -642,7 +647,7 @@ static M2TcPlan m2tc_plan_pairs(int64_t N, const PairLayout &L)
 // of `features` features and the result goes to their packed 4-simplex.
 template <int MODE>
 static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int64_t d, int64_t ldx, float *out, float *partials,
-                             unsigned *status, cudaStream_t stream, int64_t lo_row0 = 0, const unsigned *pairs = nullptr, int features = 0)
+                             unsigned *status, cudaStream_t stream, int64_t lo_row0 = 0, const unsigned *pairs = nullptr, int features = 0, int within = 0)
 {
     using S = m2tc::Shape<MODE>;
     CUtensorMap tmap;
@@ -679,7 +684,7 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     const unsigned blocks = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
     const dim3 rgrid((unsigned)q.tab.ntiles, blocks < 64 ? 64 : blocks > 1024 ? 1024 : blocks);
     auto reduce = [&](auto kernel) {
-        return launch(kernel, rgrid, 256, 0, stream, partials, out, (int)d, features, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.tab);
+        return launch(kernel, rgrid, 256, 0, stream, partials, out, (int)d, features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.tab);
     };
     if (most <= 4) return pairs ? reduce(moment2_tc_reduce_kernel<true, 4>) : reduce(moment2_tc_reduce_kernel<false, 4>);
     return pairs ? reduce(moment2_tc_reduce_kernel<true, 1>) : reduce(moment2_tc_reduce_kernel<false, 1>);
@@ -766,7 +771,7 @@ int64_t moment2_split_part_rows(int64_t N) { return (N + 63) / 64 * 64; }
 size_t moment2_pairs_partial_bytes(int64_t N, const PairLayout &L, bool split)
 {
     if (N <= 0 || N > (int64_t(1) << 29)) return 0;
-    const M2TcPlan q = split ? m2tc_plan_pairs<M2_SPLIT>(N, L) : m2tc_plan_pairs<M2_BF16>(N, L);
+    const M2TcPlan &q = split ? m2tc_plan_pairs<M2_SPLIT>(N, L) : m2tc_plan_pairs<M2_BF16>(N, L);
     return q.ok ? q.partial_bytes : 0;
 }
 
@@ -776,8 +781,8 @@ st_status moment2_pairs_tc(const void *P, int64_t N, const PairLayout &L, int64_
     const int64_t Np = moment2_split_part_rows(N);
     if (split)
         return m2tc_launch<M2_SPLIT>(m2tc_plan_pairs<M2_SPLIT>(N, L), P, 2 * Np, ldp, ldp, out, partials, status, stream, (int)Np, pairs,
-                                     L.features);
-    return m2tc_launch<M2_BF16>(m2tc_plan_pairs<M2_BF16>(N, L), P, N, ldp, ldp, out, partials, status, stream, 0, pairs, L.features);
+                                     L.features, L.within);
+    return m2tc_launch<M2_BF16>(m2tc_plan_pairs<M2_BF16>(N, L), P, N, ldp, ldp, out, partials, status, stream, 0, pairs, L.features, L.within);
 }
 
 }  // namespace st

@@ -103,11 +103,10 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
     constexpr bool LAYOUT = sizeof(OutT) == 2;
     extern __shared__ __align__(16) float xs[];                       // 2 x [EXP_ROWS][d + 1], column d is zero
     const int pitch = d + 1;
-    pdl_wait();
-    pdl_trigger();
     // gridDim.x = column groups, gridDim.y = row groups
     const int p = (blockIdx.x * EXP_THREADS + threadIdx.x) * 4;       // this thread's columns p .. p+3
     int ci[4], cj[4];
+    unsigned pair[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         ci[u] = cj[u] = d;                                            // padding column: 0 * 0
@@ -117,7 +116,7 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
                 ci[u] = (int)(e & 255);
                 cj[u] = (int)((e >> 8) & 255);
             }
-            if (blockIdx.y == 0 && p + u < dP) pairs[p + u] = e;
+            pair[u] = e;
         } else if (p + u < npairs) {
             int64_t a, b;
             tri_decode(d, p + u, a, b);
@@ -126,6 +125,9 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
         }
     }
     const bool inside = p < dP;
+    pdl_wait();
+    pdl_trigger();
+    if (LAYOUT && blockIdx.y == 0 && inside) *reinterpret_cast<uint4 *>(pairs + p) = make_uint4(pair[0], pair[1], pair[2], pair[3]);
     const int64_t rows_total = SPLIT ? Np : N;
     // Two stage buffers: the rows of the next pass travel from global memory into registers while the current ones are
     // multiplied, and one block barrier per pass is enough (a buffer is rewritten two passes later, after every

@@ -74,4 +74,12 @@ ST_HD bool pair_product(unsigned a, unsigned b, int &i, int &j, int &k, int &l)
     return gr == 2 && gs == 3;
 }
 
+// simp4_encode in 32 bits: 4096 pairs, 90 features.
+ST_HD int pair_place(int d, int i, int j, int k, int l)
+{
+    const unsigned a = (unsigned)(d - i), b = (unsigned)(d - j), c = (unsigned)(d - k), n = (unsigned)d;
+    return (int)((n * (n + 1) * (n + 2) * (n + 3) - a * (a + 1) * (a + 2) * (a + 3)) / 24 + (a * (a + 1) * (a + 2) - b * (b + 1) * (b + 2)) / 6 +
+                 (b * (b + 1) - c * (c + 1)) / 2) + l - k;
+}
+
 }  // namespace st
