@@ -85,7 +85,7 @@ struct TileTable {
     unsigned short first[MAX_TILES + 1];               // first cluster: the clusters of a tile share its samples
 };
 struct Args {
-    float *partials;                                   // [2 * cluster + block][HALF][BN]
+    float *partials;                                   // [2 * cluster + block][BN / 4][HALF][4]: four columns of a row side by side
     unsigned *status;
     int d;                                             // columns of X
     int chunks_total, stages, nb, na;                  // nb, na: boxes of B and A per part in a stage
@@ -346,10 +346,10 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         const int row0 = (int)rank * HALF + q * 32;
         const bool used = row0 < rows;
         const int c_first = diag ? row0 : 0;         // row0 is a multiple of 32
-        float *dst = a.partials + ((size_t)blockIdx.x * HALF + (q * 32 + lane)) * BN;
+        float *dst = a.partials + (size_t)blockIdx.x * HALF * BN + (q * 32 + lane) * 4;       // columns c .. c+3: + c HALF
         const uint32_t leader_acc_empty0 = map_to_cta(smem_u32(&acc_empty[0]), 0);
         if (nphases == 0 && used) {
-            for (int c0 = c_first; c0 < width; c0 += 4) *reinterpret_cast<float4 *>(dst + c0) = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int c0 = c_first; c0 < width; c0 += 4) *reinterpret_cast<float4 *>(dst + c0 * HALF) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         for (int ph = 0; ph < nphases; ++ph) {
             const int buf = ph & 1;
@@ -365,7 +365,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                     for (int e = 0; e < 32; e += 4) {
                         float4 v = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
                                                __uint_as_float(r[e + 3]));
-                        float4 *p = reinterpret_cast<float4 *>(dst + c0 + e);
+                        float4 *p = reinterpret_cast<float4 *>(dst + (c0 + e) * HALF);
                         if (ph > 0) {
                             const float4 o = *p;
                             v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
@@ -388,61 +388,50 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     }
 }
 
-// Sums of the partial tiles over the sample ranges, i <= j < d only.  `wps` warps share 32 V columns of a row: the first
-// adds ranges 0, wps, 2 wps, ... with its loads in flight, and so on, then their sums are added in order.  V = 4 where
-// there are few ranges, so that a thread still has enough loads in flight.
+// Sums of the partial tiles over the sample ranges, i <= j < d only.  A warp owns 32 rows and four columns, which lie side
+// by side in a partial tile as the epilogue's warps wrote them: with whole rows there, a warp's store met 32 lines, and
+// the last flush of a 256-wide tile took 4 us.  `wps` warps share a unit: the first adds ranges 0, wps, 2 wps, ... with its
+// loads in flight, and so on, then their sums are added in order.
 // PAIRS: X holds pair features in the order of pair_layout.cuh; pairs[column] is the pair of a column, and an entry goes
 // to the place of its 4-tuple in the packed 4-simplex, if this is the product that was chosen for that tuple.
-template <bool PAIRS, int V>
+template <bool PAIRS>
 __global__ void __launch_bounds__(256)
 moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int features, int within, int64_t out_elems,
                          const unsigned *__restrict__ pairs, const __grid_constant__ m2tc::TileTable tab)
 {
     using namespace m2tc;
-    __shared__ float part[2][8][32 * V];
+    __shared__ float4 part[2][8][32];
     const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int row = 8 * tab.row[tile], col = 8 * tab.col[tile], width = 32 * tab.width[tile], uw = (width + 32 * V - 1) / (32 * V);
+    const int row = 8 * tab.row[tile], col = 8 * tab.col[tile], rows = tab.rows[tile];
+    const int quads = (min(32 * (int)tab.width[tile], d - col) + 3) / 4, units = (rows + 31) / 32 * quads;
     const int first = tab.first[tile], nsplit = tab.first[tile + 1] - first;
-    const int rows = tab.rows[tile];
     const int wps = nsplit <= 8 ? 1 : nsplit <= 16 ? 2 : nsplit <= 32 ? 4 : 8;  // about eight loads per thread
     const int per = 8 / wps, w0 = warp % wps;
     const size_t stride = (size_t)2 * HALF * BN;
-    constexpr int BATCH = V == 1 ? 10 : 4;
+    constexpr int BATCH = 10;
     pdl_wait();
     pdl_trigger();
     int buf = 0;
-    for (int u0 = blockIdx.y * per; u0 < rows * uw; u0 += gridDim.y * per) {
-        const int u = u0 + warp / wps, r = u / uw, c = (u - r * uw) * (32 * V) + V * lane;   // this thread's columns c .. c+V-1
+    for (int u0 = blockIdx.y * per; u0 < units; u0 += gridDim.y * per) {
+        const int u = u0 + warp / wps, r = u / quads * 32 + lane, c = u % quads * 4;      // this thread's row, columns c .. c+3
         const int gi = row + r, gj = col + c;
-        const bool in_tile = r < rows && c < width;
         // what is loaded does not wait for what has to be looked up
-        const bool use = in_tile && gj + V > (PAIRS && gi >= within ? 0 : gi) && gj < d;
-        float s[V];
-#pragma unroll
-        for (int x = 0; x < V; ++x) s[x] = 0.f;
-        const float *base = partials + ((size_t)(2 * first + (r >> 7)) * HALF + (r & 127)) * BN + c;
+        const bool use = u < units && r < rows && gj + 4 > (PAIRS && gi >= within ? 0 : gi);
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float *base = partials + (size_t)(2 * first + (r >> 7)) * HALF * BN + c * HALF + (r & 127) * 4;
         for (int k0 = w0; k0 < nsplit; k0 += BATCH * wps) {
-            float v[BATCH][V];
-#pragma unroll
-            for (int e = 0; e < BATCH; ++e) {
-                const bool in = use && k0 + wps * e < nsplit;
-                const float *p = base + (size_t)(k0 + wps * e) * stride;
-                if (V == 4) {
-                    const float4 q = in ? __ldcg(reinterpret_cast<const float4 *>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    v[e][0] = q.x; v[e][V > 1 ? 1 : 0] = q.y; v[e][V > 2 ? 2 : 0] = q.z; v[e][V > 3 ? 3 : 0] = q.w;
-                } else {
-                    v[e][0] = in ? __ldcg(p) : 0.f;
-                }
-            }
+            float4 v[BATCH];
 #pragma unroll
             for (int e = 0; e < BATCH; ++e)
+                v[e] = use && k0 + wps * e < nsplit ? __ldcg(reinterpret_cast<const float4 *>(base + (size_t)(k0 + wps * e) * stride))
+                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int x = 0; x < V; ++x) s[x] += v[e][x];
+            for (int e = 0; e < BATCH; ++e) { s.x += v[e].x; s.y += v[e].y; s.z += v[e].z; s.w += v[e].w; }
         }
-        int at[V];                                         // where the columns go to, -1: not an output
+        int at[4];                                         // where the columns go to, -1: not an output
         const int at0 = PAIRS ? 0 : (int)tri_encode(d, gi, gj);
 #pragma unroll
-        for (int x = 0; x < V; ++x) {
+        for (int x = 0; x < 4; ++x) {
             at[x] = -1;
             if (PAIRS) {
                 int i, j, k, l;
@@ -452,16 +441,18 @@ moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__
             }
         }
         if (wps > 1) {
-#pragma unroll
-            for (int x = 0; x < V; ++x) part[buf][warp][32 * x + lane] = s[x];
+            part[buf][warp][lane] = s;
             __syncthreads();
         }
         if (w0 == 0 && use) {
-#pragma unroll
-            for (int x = 0; x < V; ++x) {
-                for (int w = 1; w < wps; ++w) s[x] += part[buf][warp + w][32 * x + lane];
-                if (at[x] >= 0 && ST_BOUNDS_OK(at[x], out_elems, PAIRS ? 7 : 2)) out[at[x]] = s[x];
+            for (int w = 1; w < wps; ++w) {
+                const float4 v = part[buf][warp + w][lane];
+                s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
             }
+            const float f[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (at[x] >= 0 && ST_BOUNDS_OK(at[x], out_elems, PAIRS ? 7 : 2)) out[at[x]] = f[x];
         }
         buf ^= 1;
     }
@@ -679,15 +670,10 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
         (void)cudaGetLastError();
         return ST_ERR_CUDA;
     }
-    int most = 0;                                                         // sample ranges of a tile
-    for (int t = 0; t < q.tab.ntiles; ++t) most = q.tab.first[t + 1] - q.tab.first[t] > most ? q.tab.first[t + 1] - q.tab.first[t] : most;
     const unsigned blocks = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
     const dim3 rgrid((unsigned)q.tab.ntiles, blocks < 64 ? 64 : blocks > 1024 ? 1024 : blocks);
-    auto reduce = [&](auto kernel) {
-        return launch(kernel, rgrid, 256, 0, stream, partials, out, (int)d, features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.tab);
-    };
-    if (most <= 4) return pairs ? reduce(moment2_tc_reduce_kernel<true, 4>) : reduce(moment2_tc_reduce_kernel<false, 4>);
-    return pairs ? reduce(moment2_tc_reduce_kernel<true, 1>) : reduce(moment2_tc_reduce_kernel<false, 1>);
+    return launch(pairs ? moment2_tc_reduce_kernel<true> : moment2_tc_reduce_kernel<false>, rgrid, 256, 0, stream, partials, out, (int)d,
+                  features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.tab);
 }
 
 // Room for the partial tiles of the structured call and of its dense control: one workspace serves both.
