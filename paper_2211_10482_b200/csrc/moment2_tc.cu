@@ -390,10 +390,13 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 
 // Sums of the partial tiles over the sample ranges, i <= j < d only.  A warp owns 32 rows and four columns, which lie side
 // by side in a partial tile as the epilogue's warps wrote them: with whole rows there, a warp's store met 32 lines, and
-// the last flush of a 256-wide tile took 4 us.  `wps` warps share a unit: the first adds ranges 0, wps, 2 wps, ... with its
-// loads in flight, and so on, then their sums are added in order.
+// the last flush of a 256-wide tile took 4 us.  `wps` warps share a unit: the first adds ranges 0, wps, 2 wps, ..., four
+// loads at a time, and so on, then their sums are added in order.  (Ten loads at a time and eight ranges per warp take so
+// many registers that the blocks do not all fit beside the next kernel's: [4096,1024] 17.4 us, now 14.2; fourth moment of
+// [4096,24] 18.8, now 16.0.)
 // PAIRS: X holds pair features in the order of pair_layout.cuh; pairs[column] is the pair of a column, and an entry goes
 // to the place of its 4-tuple in the packed 4-simplex, if this is the product that was chosen for that tuple.
+__host__ __device__ inline int m2tc_sum_warps(int nsplit) { return nsplit <= 4 ? 1 : nsplit <= 8 ? 2 : nsplit <= 16 ? 4 : 8; }
 template <bool PAIRS>
 __global__ void __launch_bounds__(256)
 moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int features, int within, int64_t out_elems,
@@ -405,10 +408,10 @@ moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__
     const int row = 8 * tab.row[tile], col = 8 * tab.col[tile], rows = tab.rows[tile];
     const int quads = (min(32 * (int)tab.width[tile], d - col) + 3) / 4, units = (rows + 31) / 32 * quads;
     const int first = tab.first[tile], nsplit = tab.first[tile + 1] - first;
-    const int wps = nsplit <= 8 ? 1 : nsplit <= 16 ? 2 : nsplit <= 32 ? 4 : 8;  // about eight loads per thread
+    const int wps = m2tc_sum_warps(nsplit);
     const int per = 8 / wps, w0 = warp % wps;
     const size_t stride = (size_t)2 * HALF * BN;
-    constexpr int BATCH = 10;
+    constexpr int BATCH = 4;
     pdl_wait();
     pdl_trigger();
     int buf = 0;
@@ -670,8 +673,16 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
         (void)cudaGetLastError();
         return ST_ERR_CUDA;
     }
-    const unsigned blocks = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
-    const dim3 rgrid((unsigned)q.tab.ntiles, blocks < 64 ? 64 : blocks > 1024 ? 1024 : blocks);
+    // blocks for all units of a tile, up to 16 per SM together: more of them would only be in the way of the next kernel's
+    unsigned blocks = 1;
+    for (int t = 0; t < q.tab.ntiles; ++t) {
+        const unsigned per = 8u / (unsigned)m2tc_sum_warps(q.tab.first[t + 1] - q.tab.first[t]);
+        const unsigned n = ((unsigned)((q.tab.rows[t] + 31) / 32 * 8 * q.tab.width[t]) + per - 1) / per;
+        if (n > blocks) blocks = n;
+    }
+    const unsigned most = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
+    if (blocks > most) blocks = most < 64 ? 64 : most;
+    const dim3 rgrid((unsigned)q.tab.ntiles, blocks);
     return launch(pairs ? moment2_tc_reduce_kernel<true> : moment2_tc_reduce_kernel<false>, rgrid, 256, 0, stream, partials, out, (int)d,
                   features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.tab);
 }
