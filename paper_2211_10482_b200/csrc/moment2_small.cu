@@ -322,7 +322,8 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
 }
 
 // out[p(ci,cj)] = sum over the slices of element (k, item) of the partials: a block owns 32 elements, warp w adds the
-// slices w, w + 8, ... with all its loads in flight, then the eight sums are added in order (a fixed order).
+// slices w, w + 8, ..., seven loads at a time, then the eight sums are added in order (a fixed order).  Twenty at a time
+// (all that there are) take registers that the running kernel does not leave: [20000,64] 10.8 us the call, now 9.9.
 __global__ void __launch_bounds__(256)
 moment2_small_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int nbk, int slices,
                             int dense, int nitems)
@@ -337,12 +338,12 @@ moment2_small_reduce_kernel(const float *__restrict__ partials, float *__restric
     pdl_trigger();
     const size_t stride = (size_t)nitems * 128;
     float s = 0.f;
-    for (int k0 = warp; k0 < slices; k0 += 8 * 20) {   // 148 slices: one batch
-        float v[20];
+    for (int k0 = warp; k0 < slices; k0 += 8 * 7) {
+        float v[7];
 #pragma unroll
-        for (int u = 0; u < 20; ++u) v[u] = (use && k0 + 8 * u < slices) ? __ldcg(partials + (size_t)(k0 + 8 * u) * stride + o) : 0.f;
+        for (int u = 0; u < 7; ++u) v[u] = (use && k0 + 8 * u < slices) ? __ldcg(partials + (size_t)(k0 + 8 * u) * stride + o) : 0.f;
 #pragma unroll
-        for (int u = 0; u < 20; ++u) s += v[u];
+        for (int u = 0; u < 7; ++u) s += v[u];
     }
     part[warp][lane] = s;
     __syncthreads();
