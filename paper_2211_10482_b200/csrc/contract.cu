@@ -253,37 +253,36 @@ __global__ void __launch_bounds__(256)
 mttkrp_rowsum_kernel(const float *__restrict__ part, float *__restrict__ A, int64_t I_full, int64_t i_off, MttkrpRows m,
                      int R, int unit_rows, int ksplit)
 {
-    pdl_wait();
-    pdl_trigger();
+    // where this warp's slots are takes two 64-bit divisions and does not have to wait
     const int lane = threadIdx.x & 31;
     const int64_t ii = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (ii >= I_full) return;
     const int64_t i = ii - i_off;
     float *dst = A + ii * R;
-    if (i < 0 || i >= m.I) {
-        for (int r = lane; r < R; r += 32) dst[r] = 0.f;
-        return;
+    int64_t first = 0, n = 0;
+    if (ii < I_full && i >= 0 && i < m.I) {
+        int64_t s, e;
+        if (m.mode == MK_PACKED) { s = tri_row_start(m.I, i); e = s + (m.I - i); }
+        else { s = i * m.div; e = s + m.div; }
+        if (e > m.rows) e = m.rows;
+        if (e > s) {
+            const int64_t u0 = s / unit_rows, u1 = (e - 1) / unit_rows;
+            first = (u0 + i) * ksplit;
+            n = (u1 - u0 + 1) * ksplit;
+            if (!ST_BOUNDS_OK(first + n - 1, mttkrp_slots(m.rows, unit_rows, m.I, ksplit), 6)) n = -1;
+        }
     }
-    int64_t s, e;
-    if (m.mode == MK_PACKED) { s = tri_row_start(m.I, i); e = s + (m.I - i); }
-    else { s = i * m.div; e = s + m.div; }
-    if (e > m.rows) e = m.rows;
-    const int64_t u0 = s / unit_rows, u1 = (e - 1) / unit_rows;
+    pdl_wait();
+    pdl_trigger();
+    if (ii >= I_full || n < 0) return;
     for (int r = lane; r < R; r += 32) {
         float sum = 0.f;
-        if (e > s) {
-            const float *p = part + ((u0 + i) * ksplit) * R + r;
-            const int64_t n = (u1 - u0 + 1) * ksplit;
-            if (!ST_BOUNDS_OK((u0 + i) * ksplit + n - 1, mttkrp_slots(m.rows, unit_rows, m.I, ksplit), 6)) continue;
-            int64_t k = 0;
-            for (; k + 8 <= n; k += 8) {               // eight independent loads in flight
-                float t[8];
+        const float *p = part + first * R + r;
+        for (int64_t k = 0; k < n; k += 8) {               // eight independent loads in flight
+            float t[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) t[u] = __ldcg(p + (k + u) * R);
+            for (int u = 0; u < 8; ++u) t[u] = k + u < n ? __ldcg(p + (k + u) * R) : 0.f;
 #pragma unroll
-                for (int u = 0; u < 8; ++u) sum += t[u];
-            }
-            for (; k < n; ++k) sum += __ldcg(p + k * R);
+            for (int u = 0; u < 8; ++u) sum += t[u];
         }
         dst[r] = sum;
     }
