@@ -25,6 +25,10 @@
 namespace st {
 
 constexpr int COPY_UNITS = 4;              // 16-byte units that a thread of the slice copies has in flight
+// Slice copies have grids as large as the work: blocks then start in the order of memory.  With 16 blocks per SM that walk the array in
+// strides, of which only some fit at a time, it was written in several sweeps with holes ([4096,4096,64] zero fill 755 us,
+// now 624; [2000,2000,64] 253, now 229).
+constexpr int64_t MAX_GRID = int64_t(1) << 30;
 constexpr int SYM_WORDS = 4;               // words that a lane of the symmetric fill has in flight
 constexpr int64_t PART_BYTES = 32768;      // most of a slice that one thread group copies ([384,384,75]: 128 KiB starve the chip)
 
@@ -266,6 +270,9 @@ sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restric
                  int row_bytes, unsigned inv, int group_shift, int64_t packed_rows)
 {
     typedef typename Elem<ES>::T E;
+    // rows of whole 16-byte units of a matrix: two units of a lane in flight ([1000,1000,40] 56 us, now 49; the shorter runs
+    // of a tet got slower)
+    constexpr bool WIDE = ES == 16 && KIND == ST_TRI_UPPER;
     pdl_wait();
     pdl_trigger();
     const int lane = (int)(threadIdx.x & 31);
@@ -294,7 +301,7 @@ sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restric
         if (xr < x1) {
             const I p = KIND == ST_TRI_UPPER ? tri_at<I>(d, a, xr) : KIND == ST_TET ? tet_at<I>(d, a, b, xr) : simp4_at<I>(d, a, b, c, xr);
             if (ST_BOUNDS_OK(p, packed_rows, 1) && ST_BOUNDS_OK((int64_t)p + (x1 - xr) - 1, packed_rows, 1))
-                copy_flat<ES, false, 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32);
+                copy_flat<ES, false, WIDE ? 2 : 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32);
         }
         const I xe = x1 < top ? x1 : top;
         const int words = row_bytes / ES;
@@ -321,8 +328,12 @@ sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restric
             const int g = 1 << group_shift;
             for (I x = x0 + (I)(lane >> group_shift); x < xe; x += (I)(32 >> group_shift)) {
                 const I p = sym_row<KIND, I>(d, a, b, c, x);
-                if (ST_BOUNDS_OK(p, packed_rows, 1))
-                    copy_flat<ES, false, 1>(out + (int64_t)x * row_bytes, src + (int64_t)p * row_bytes, nullptr, row_bytes, lane & (g - 1), g);
+                if (!ST_BOUNDS_OK(p, packed_rows, 1)) continue;
+                unsigned char *o = out + (int64_t)x * row_bytes;
+                const unsigned char *from = src + (int64_t)p * row_bytes;
+                // more than one unit per lane: two in flight (aligned rows: rows of 800 bytes 172 us at d = 700, now 141)
+                if (WIDE && row_bytes > 512) copy_flat<ES, false, 2>(o, from, nullptr, row_bytes, lane & (g - 1), g);
+                else copy_flat<ES, false, 1>(o, from, nullptr, row_bytes, lane & (g - 1), g);
             }
         }
     }
@@ -491,7 +502,7 @@ static st_status launch_sym(const void *src, void *dst, const LayoutArgs &a, cud
 template <int KIND, int ES, bool PACK>
 static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cudaStream_t s, const void *mul)
 {
-    const int64_t cap = (int64_t)sm_count_or_default() * 16;
+    const int64_t cap = MAX_GRID;
     // slices: about four 16-byte units per thread, at most PART_BYTES per (slice, part).  Pack splits the
     // longest run of unique columns, unpack the whole dense slice.
     int64_t run_rows = a.d;
@@ -602,7 +613,9 @@ static st_status packed_binary(int op, int64_t n, const float *a, const float *b
     if (!a || !b || !out) return ST_ERR_NULL;
     if (n <= 0) return ST_ERR_SHAPE;
     if (!st::aligned16(a) || !st::aligned16(b) || !st::aligned16(out)) return ST_ERR_ALIGN;
-    const int64_t want = (n / 4 + 255) / 256, cap = (int64_t)st::sm_count_or_default() * 16;
+    // operands that stay in L2: one wave of blocks that walk ([5544000] 6.3 us, a block per 1024 elements 7.4); larger ones in
+    // the order of memory ([10^8] 168 us, one wave 183)
+    const int64_t want = (n / 4 + 255) / 256, cap = n < (int64_t(1) << 24) ? (int64_t)st::sm_count_or_default() * 16 : st::MAX_GRID;
     const unsigned grid = (unsigned)(want < 1 ? 1 : (want < cap ? want : cap));
     return st::launch(op == 0 ? st::packed_binary_kernel<0> : st::packed_binary_kernel<1>, grid, 256, 0, (cudaStream_t)stream, a, b, out, n, alpha, beta);
 }
