@@ -10,7 +10,8 @@
 //   2. tensor cores (up to 4096 pair features, d <= 90): the triangular tile GEMM of moment2_tc.cu on P rounded to bf16
 //      (ST_FLAG_TC_BF16, 5e-3) or, for the fp32 tolerance, on P written as hi + lo bf16 parts and multiplied in three
 //      partial products.  The columns of P are in the order of pair_layout.cuh, in which a few tiles hold a product for
-//      every 4-tuple, and the sum over their partial tiles goes straight to the packed 4-simplex.  With the pairs in
+//      every 4-tuple (bf16: one range, which is the packed order, since there the results depend on which pairs are
+//      multiplied), and the sum over their partial tiles goes straight to the packed 4-simplex.  With the pairs in
 //      packed order (a tuple where j <= k, so all tiles of the triangle) [30011,45] ran 136 us, now 90; with the rows'
 //      pairs ordered by j and a copy of them by k for the columns (a staircase, P twice as large) 135; [14831,64] 253,
 //      now 136, the staircase 150; [114839,23] 107, now 97.
@@ -27,7 +28,7 @@ namespace st {
 
 size_t moment2_workspace(int64_t N, int64_t d, int xdt, unsigned flags);
 int64_t moment2_split_part_rows(int64_t N);
-PairLayout pair_layout(int features);
+PairLayout pair_layout(int features, bool one);
 size_t moment2_pairs_partial_bytes(int64_t N, const PairLayout &L, bool split);
 st_status moment2_pairs_tc(const void *P, int64_t N, const PairLayout &L, int64_t ldp, bool split, const unsigned *pairs, float *out,
                            float *partials, unsigned *status, cudaStream_t stream);
@@ -57,7 +58,7 @@ static Plan plan(int64_t N, int64_t d, unsigned flags)
     // partial products (the fp32 tolerance) wherever that kernel reaches; else fp32 features and the fp32 FMA kernel
     p.Np = moment2_split_part_rows(N);
     if (p.dP <= TC_COLS) {
-        p.layout = pair_layout((int)d);
+        p.layout = pair_layout((int)d, p.bf16);
         p.m2_ws = moment2_pairs_partial_bytes(N, p.layout, !p.bf16);
     }
     if (p.m2_ws != 0) {
