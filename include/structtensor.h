@@ -175,12 +175,12 @@ st_status st_sym_moment3(const float *X, int64_t N, int64_t d, int64_t ldx,
  * samples: the last block of the degree-2 polynomial-regression covariance; its unique elements
  * are the 4-tuples with repetition i<=j<=k<=l, "about 23x" fewer than d^4):
  *     out[s(i,j,k,l)] = sum_n X[n,i] X[n,j] X[n,k] X[n,l]   for 0 <= i <= j <= k <= l < d
- * X: fp32 [N, ldx], ldx >= d, 1 <= d <= 128 (ST_FLAG_TC_BF16: d <= 89).  out_packed: d(d+1)(d+2)(d+3)/24 floats in the
+ * X: fp32 [N, ldx], ldx >= d, 1 <= d <= 128 (ST_FLAG_TC_BF16: d <= 90).  out_packed: d(d+1)(d+2)(d+3)/24 floats in the
  * lexicographic order of the unique set (slab i holds the tetrahedron (j,k,l) of side d-i).
  * Computed as the second moment of the pair features P[n,(i,j)] = X[n,i] X[n,j], i<=j, which
- * the call materialises in the workspace (N * roundup(d(d+1)/2, 64) elements; query the size
- * with ST_OP_SYM_MOMENT4), followed by a gather of the entries with j <= k.  Default: the 1e-4 tolerance of
- * the fp32 paths -- for d <= 89 every fp32 pair product is stored as hi + lo bf16 parts and the tensor-core
+ * the call materialises in the workspace (about N * d(d+1)/2 elements; query the size
+ * with ST_OP_SYM_MOMENT4), of which the products that stand for a 4-tuple are kept.  Default: the 1e-4 tolerance of
+ * the fp32 paths -- for d <= 90 every fp32 pair product is stored as hi + lo bf16 parts and the tensor-core
  * triangular tile GEMM adds three partial products (hi hi + hi lo + lo hi) with fp32 accumulation; for larger d
  * an fp32 P and fp32 FMA arithmetic.  ST_FLAG_TC_BF16 stores P rounded to bf16 and runs one pass of the same
  * GEMM (5e-3 tolerance for N >= 1000). */

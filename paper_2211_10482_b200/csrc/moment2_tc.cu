@@ -34,7 +34,7 @@
 // 96 bytes per sample and column pair).  Few features: the latency of a stage, hence more and smaller stages.
 //
 // M2_CONV: a pass that wrote hi and lo before moved 8 bytes a value through HBM on top of the 4 read here, and took
-// 176 of the 590 us of [262144,520], now 490; [1048576,256] 700, now 340; [1048576,64] 245, now 143.  Copies bring the
+// 176 of the 590 us of [262144,520], now 410; [1048576,256] 700, now 285; [1048576,64] 245, now 143.  Copies bring the
 // fp32 boxes, converting warps rewrite them in place and arrive at the leader's barrier.  Bound by shared memory: per
 // 32 samples of a full tile off the diagonal 256 cycles each for the copy, the reads and the writes and 384 for the
 // operands of 768 cycles of MMA.  Loads through registers instead of the copies avoid two of these, but every arrival

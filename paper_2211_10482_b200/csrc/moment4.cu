@@ -12,7 +12,7 @@
 //      partial products.  The columns of P are in the order of pair_layout.cuh, in which a few tiles hold a product for
 //      every 4-tuple (bf16: one range, which is the packed order, since there the results depend on which pairs are
 //      multiplied), and the sum over their partial tiles goes straight to the packed 4-simplex.  With the pairs in
-//      packed order (a tuple where j <= k, so all tiles of the triangle) [30011,45] ran 136 us, now 90; with the rows'
+//      packed order (a tuple where j <= k, so all tiles of the triangle) [30011,45] ran 136 us, then 90, and with the sums of today 80; with the rows'
 //      pairs ordered by j and a copy of them by k for the columns (a staircase, P twice as large) 135; [14831,64] 253,
 //      now 136, the staircase 150; [114839,23] 107, now 97.
 //   3. more features, or more samples than those kernels take: the fp32 FMA kernel on an fp32 P in packed order.  The
