@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(RG_THREADS, 1) rowgemm_kernel(const RgArgs a)
 // Second pass of MTTKRP: one warp per row of A adds the partial slots of that row in increasing
 // order (units, then k-splits) and writes the row; rows the fibres do not reach are zero.
 __global__ void __launch_bounds__(256)
-mttkrp_rowsum_kernel(const float *__restrict__ part, float *__restrict__ A, int64_t I_full, int64_t i_off, MttkrpRows m,
+mttkrp_rowsum_kernel(const float *part, float *A, int64_t I_full, int64_t i_off, MttkrpRows m,
                      int R, int unit_rows, int ksplit)
 {
     // where this warp's slots are takes two 64-bit divisions and does not have to wait

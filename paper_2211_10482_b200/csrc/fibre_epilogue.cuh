@@ -38,7 +38,7 @@ __device__ __forceinline__ void fibre_load16(uint32_t taddr, int R, float (&v)[2
 }
 
 template <bool SUM>
-__device__ __forceinline__ void ttm_epilogue(uint32_t taddr, int R, int64_t row0, int64_t rows, float *__restrict__ out, int lane)
+__device__ __forceinline__ void ttm_epilogue(uint32_t taddr, int R, int64_t row0, int64_t rows, float *out, int lane)
 {
     float *dst = out + (row0 + (lane >> 2)) * R + 2 * (lane & 3);
     const int64_t left = rows - row0 - (lane >> 2);
@@ -95,19 +95,19 @@ __device__ __forceinline__ UnitFibres unit_fibres(int64_t row0, int64_t rows, bo
 }
 
 // Columns c .. c + 15 of the rows of C that this thread's fibres take.
-__device__ __forceinline__ void unit_load_c(const UnitFibres &f, const float *__restrict__ C, int R, int c, int lane, float2 (&x)[2][4])
+__device__ __forceinline__ void unit_load_c(const UnitFibres &f, const float *C, int R, int c, int lane, float2 (&x)[2][4])
 {
 #pragma unroll
     for (int h = 0; h < 4; ++h)
 #pragma unroll
-        for (int g = 0; g < 2; ++g) x[g][h] = __ldg(reinterpret_cast<const float2 *>(C + (int64_t)f.j[h] * R + c + 8 * g + 2 * (lane & 3)));
+        for (int g = 0; g < 2; ++g) x[g][h] = *reinterpret_cast<const float2 *>(C + (int64_t)f.j[h] * R + c + 8 * g + 2 * (lane & 3));
 }
 
 // Sums over the runs of fibres with the same i, times C, to the partial slots (unit + i).  cpre: unit_load_c of column 0,
 // asked for before the accumulator was waited for; the next columns' are asked for one step ahead.
 template <bool SUM>
-__device__ __forceinline__ void mttkrp_epilogue(uint32_t taddr, int R, const UnitFibres &f, const float *__restrict__ C, int64_t unit,
-                                                float *__restrict__ part, int64_t nslots, int lane, float2 (&cpre)[2][4])
+__device__ __forceinline__ void mttkrp_epilogue(uint32_t taddr, int R, const UnitFibres &f, const float *C, int64_t unit,
+                                                float *part, int64_t nslots, int lane, float2 (&cpre)[2][4])
 {
     if (f.n == 0) return;
     for (int c = 0; c < R; c += 16) {

@@ -134,7 +134,7 @@ static MgGrid moment2_gemm_plan(int64_t N, int64_t d, unsigned flags)
 // trip to memory costs microseconds.
 template <bool DENSE>
 __global__ void __launch_bounds__(256)
-moment2_gemm_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, const MgGrid g)
+moment2_gemm_reduce_kernel(const float *partials, float *out, int d, const MgGrid g)
 {
     constexpr int T = MG_T;
     constexpr int BATCH = 4;                             // eight take registers that the running kernel does not leave: [20000,256] 54 us, now 47
@@ -200,7 +200,7 @@ __device__ __forceinline__ uint64_t mg_ffma2(uint64_t a, uint64_t b, uint64_t c)
 // per stage and thread beside 512 packed FMAs).
 template <bool DENSE, bool VEC>
 __global__ void __launch_bounds__(MG_THREADS, 2)
-moment2_gemm_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, float *__restrict__ partials, const MgGrid g,
+moment2_gemm_kernel(const float *X, int64_t N, int d, int64_t ldx, float *partials, const MgGrid g,
                     unsigned *status)
 {
     extern __shared__ __align__(16) float smem[];     // MG_STAGES x { As[MG_KC][MG_T], Bs[MG_KC][MG_T] }

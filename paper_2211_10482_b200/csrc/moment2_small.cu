@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
 // slices w, w + 8, ..., seven loads at a time, then the eight sums are added in order (a fixed order).  Twenty at a time
 // (all that there are) take registers that the running kernel does not leave: [20000,64] 10.8 us the call, now 9.9.
 __global__ void __launch_bounds__(256)
-moment2_small_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int nbk, int slices,
+moment2_small_reduce_kernel(const float *partials, float *out, int d, int nbk, int slices,
                             int dense, int nitems)
 {
     __shared__ float part[8][32];

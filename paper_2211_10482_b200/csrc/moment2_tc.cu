@@ -399,8 +399,8 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 __host__ __device__ inline int m2tc_sum_warps(int nsplit) { return nsplit <= 4 ? 1 : nsplit <= 8 ? 2 : nsplit <= 16 ? 4 : 8; }
 template <bool PAIRS>
 __global__ void __launch_bounds__(256)
-moment2_tc_reduce_kernel(const float *__restrict__ partials, float *__restrict__ out, int d, int features, int within, int64_t out_elems,
-                         const unsigned *__restrict__ pairs, const __grid_constant__ m2tc::TileTable tab)
+moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features, int within, int64_t out_elems,
+                         const unsigned *pairs, const __grid_constant__ m2tc::TileTable tab)
 {
     using namespace m2tc;
     __shared__ float4 part[2][8][32];

@@ -155,7 +155,7 @@ template <int WARPS, int DC, bool ALIGNED>
 __global__ void __launch_bounds__(M3_THREADS, 1)
 moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
 {
-    const float *__restrict__ X = a.X;
+    const float *X = a.X;
     const int64_t N = a.N, ldx = a.ldx, rows_per_slice = a.rows_per_slice;
     const int d = a.d, dp = DC > 0 ? DC : a.dp, out_elems = a.out_elems;
     pdl_wait();
@@ -308,7 +308,7 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
 // than the running kernel leaves, and start later ([4096,24] 12.2 us the call, now 11.2; twenty 14.7).
 constexpr int SUM_GROUPS = 8;
 __global__ void __launch_bounds__(32 * SUM_GROUPS)
-sum_slices_kernel(const float *__restrict__ partials, float *__restrict__ out, int64_t elems, int slices)
+sum_slices_kernel(const float *partials, float *out, int64_t elems, int slices)
 {
     __shared__ float part[SUM_GROUPS][32];
     pdl_wait();

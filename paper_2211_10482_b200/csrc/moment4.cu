@@ -98,8 +98,8 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *dst, float a, float b, flo
 // COLS: columns of a staged row per lane, (d + 1 + 31) / 32 rounded up to an instance (2, 3 or 5).
 template <typename OutT, bool SPLIT, int COLS>
 __global__ void __launch_bounds__(EXP_THREADS)
-pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, OutT *__restrict__ P, int dP, int npairs, int64_t Np,
-                   const __grid_constant__ PairLayout layout, unsigned *__restrict__ pairs)
+pair_expand_kernel(const float *X, int64_t N, int d, int64_t ldx, OutT *P, int dP, int npairs, int64_t Np,
+                   const __grid_constant__ PairLayout layout, unsigned *pairs)
 {
     constexpr bool LAYOUT = sizeof(OutT) == 2;
     extern __shared__ __align__(16) float xs[];                       // 2 x [EXP_ROWS][d + 1], column d is zero
@@ -189,7 +189,7 @@ pair_expand_kernel(const float *__restrict__ X, int64_t N, int d, int64_t ldx, O
 // order of the pairs (k,l), and in row (i,j) of the packed pair-by-pair triangle they are the columns from pair
 // (j,j) to the last one: one contiguous run on both sides, of d-j + ... + 1 elements.
 __global__ void __launch_bounds__(128)
-simplex_gather_kernel(const float *__restrict__ M2, float *__restrict__ out, int d, int64_t dP, unsigned *status,
+simplex_gather_kernel(const float *M2, float *out, int d, int64_t dP, unsigned *status,
                       const unsigned *inner_status)
 {
     pdl_wait();

@@ -52,9 +52,9 @@ template <> struct Elem<16> { typedef uint4 T; };
 template <int ES>
 __device__ __forceinline__ uint4 load_unit(const uint4 *p, unsigned off)
 {
-    const uint4 a = __ldg(p);
+    const uint4 a = p[0];
     if (off == 0) return a;
-    const uint4 b = __ldg(p + 1);
+    const uint4 b = p[1];
     uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x;
     if (off & 8) { w0 = a.z; w1 = a.w; w2 = b.x; w3 = b.y; w4 = b.z; }
     if (ES < 8) {
@@ -85,8 +85,8 @@ __device__ __forceinline__ void copy_flat(unsigned char *dst, const unsigned cha
     const int ends = n - (units << 4);
     auto end_at = [&](int e) { return e < head ? e : e + (units << 4); };
     auto end_load = [&](int e) {
-        E v = __ldg(reinterpret_cast<const E *>(src + end_at(e)));
-        if constexpr (MUL) v = mul_word(v, __ldg(reinterpret_cast<const uint32_t *>(mul + end_at(e))));
+        E v = *reinterpret_cast<const E *>(src + end_at(e));
+        if constexpr (MUL) v = mul_word(v, *reinterpret_cast<const uint32_t *>(mul + end_at(e)));
         return v;
     };
     const int e0 = lane * ES;
@@ -102,7 +102,7 @@ __device__ __forceinline__ void copy_flat(unsigned char *dst, const unsigned cha
         for (int k = 0; k < U; ++k)
             if (u0 + k * g < units) {
                 v[k] = load_unit<ES>(in + u0 + k * g, off);
-                if (MUL) w[k] = __ldg(m + u0 + k * g);
+                if (MUL) w[k] = m[u0 + k * g];
             }
 #pragma unroll
         for (int k = 0; k < U; ++k)
@@ -205,8 +205,8 @@ __device__ __forceinline__ void slice_run(const LayoutArgs &a, I &s, I &lo, I &h
 
 template <int KIND, int ES, bool PACK, bool MUL, typename I>
 __global__ void __launch_bounds__(256)
-slice_copy_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst, LayoutArgs a, I nitems, int group_shift, int parts,
-                  int part_bytes, const unsigned char *__restrict__ mul)
+slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I nitems, int group_shift, int parts,
+                  int part_bytes, const unsigned char *mul)
 {
     // MUL (pack only, fp32 elements): a second packed operand; the gathered values are multiplied by it
     pdl_wait();
@@ -266,7 +266,7 @@ __device__ __forceinline__ I sym_row(I d, I a, I b, I c, I x)
 // the words of the positions (up to 32 words each), or a lane group copies a position (`inner` elements) at a time.
 template <int KIND, int ES, typename I>
 __global__ void __launch_bounds__(256)
-sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst, I d, I nslices, int parts, int part_rows,
+sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, int parts, int part_rows,
                  int row_bytes, unsigned inv, int group_shift, int64_t packed_rows)
 {
     typedef typename Elem<ES>::T E;
@@ -318,7 +318,7 @@ sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restric
                     if (e >= n) continue;
                     const unsigned dx = (e * inv) >> 16;
                     const I p = sym_row<KIND, I>(d, a, b, c, x0 + (I)dx);
-                    v[u] = ST_BOUNDS_OK(p, packed_rows, 1) ? __ldg(reinterpret_cast<const E *>(src) + (int64_t)p * words + (e - dx * (unsigned)words)) : E{};
+                    v[u] = ST_BOUNDS_OK(p, packed_rows, 1) ? reinterpret_cast<const E *>(src)[(int64_t)p * words + (e - dx * (unsigned)words)] : E{};
                 }
 #pragma unroll
                 for (int u = 0; u < SYM_WORDS; ++u)
@@ -345,7 +345,7 @@ sym_slice_kernel(const unsigned char *__restrict__ src, unsigned char *__restric
 // into the slab (i2, i1).  Lanes read consecutive packed words wherever k is the largest index.
 template <int KIND, int ES>
 __global__ void __launch_bounds__(256)
-sym_tile_kernel(const typename Elem<ES>::T *__restrict__ packed, typename Elem<ES>::T *__restrict__ dense, unsigned d, unsigned nt, int64_t packed_rows)
+sym_tile_kernel(const typename Elem<ES>::T *packed, typename Elem<ES>::T *dense, unsigned d, unsigned nt, int64_t packed_rows)
 {
     typedef typename Elem<ES>::T E;
     __shared__ E tile[32][33];
@@ -374,7 +374,7 @@ sym_tile_kernel(const typename Elem<ES>::T *__restrict__ packed, typename Elem<E
         const unsigned j = bi * 32 + ty + 8 * q, k = bj * 32 + tx;
         if (j <= k && k < d) {
             const unsigned p = at(j, k);
-            v[q] = ST_BOUNDS_OK(p, packed_rows, 1) ? __ldg(packed + p) : E{};
+            v[q] = ST_BOUNDS_OK(p, packed_rows, 1) ? packed[p] : E{};
         }
     }
 #pragma unroll

@@ -118,6 +118,9 @@ inline bool allow_large_clusters(Kernel kernel)
 // For that every block of every kernel calls pdl_wait() before its first access to global memory (it returns when all
 // kernels before this one have completed and their writes are visible), and pdl_trigger() once the next kernel's blocks
 // may be placed: after its own TMEM allocation, where it has one.
+// What a kernel reads from global memory may so have been written while its blocks were already there.  It is read by coherent
+// loads, asynchronous copies or TMA, never by the read-only path (`__ldg`, or a const pointer declared __restrict__, for which
+// the compiler may choose that path and move the load ahead of the wait): that is for data no one writes during the kernel.
 #if defined(__CUDACC__)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(split::THREADS, 1) ttm_split_kernel(const Spli
             float4 v[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                v[e] = (k0 + e < a.K) ? __ldg(reinterpret_cast<const float4 *>(a.W + (size_t)(k0 + e) * R + r0))
+                v[e] = (k0 + e < a.K) ? *reinterpret_cast<const float4 *>(a.W + (size_t)(k0 + e) * R + r0)
                                       : make_float4(0.f, 0.f, 0.f, 0.f);
             unsigned char *reg = w_smem + (size_t)kc * w_region;
 #pragma unroll

@@ -108,7 +108,7 @@ ttm_tc_kernel(const __grid_constant__ CUtensorMap tmap, const TtmTcArgs a)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int k = kc * KC + 4 * q + e;
-                    v[u][e] = it < items && k < a.K ? __ldg(reinterpret_cast<const float4 *>(a.U + (size_t)k * a.R + r0))
+                    v[u][e] = it < items && k < a.K ? *reinterpret_cast<const float4 *>(a.U + (size_t)k * a.R + r0)
                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }

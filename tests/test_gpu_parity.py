@@ -1235,3 +1235,39 @@ def test_dependent_launches_keep_the_order_of_two_streams_and_a_graph(st, N, d):
         st.set_allocator(GuardAllocator())
     for got in eager + [captured]:
         assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+def test_inputs_written_by_the_kernel_just_before_are_read_as_written(st):
+    """Back to back in the same buffers, with other values every time: what axpby, pack and the second moment write is
+    read at once by the fill, the MTTKRP forms and the fourth moment's own kernels.  The calls of one input give the same
+    bits whenever they are made."""
+    d, inner, I, K, R = 200, 5, 60, 64, 32
+    lay, cube = st.Layout(st.ST_TRI_UPPER, d, inner), st.Layout(st.ST_TRI_UPPER, I, K)
+    new = lambda n: guarded(st, n)
+    base = dev(workloads.draw((st.st_packed_elems(lay),), "normal", 1))
+    cubes = dev(workloads.draw((st.st_dense_elems(cube),), "normal", 2))
+    C, D, X = (dev(workloads.draw(s, "normal", 3)) for s in ((I, R), (K, R), (700, 24)))
+    total, dense, packed, scaled = new(base.numel()), new(st.st_dense_elems(lay)), new(st.st_packed_elems(cube)), torch.empty_like(cubes)
+    A = [new(I * R) for _ in range(3)]
+    flags = (0, st.ST_FLAG_TC_TF32, st.ST_FLAG_TC_SPLIT)
+
+    def pass_of(f, wait):
+        sync = torch.cuda.synchronize if wait else lambda: None
+        st.st_packed_axpby(f, base, 0.0, base, out=total)
+        sync()
+        st.st_unpack(total, lay, st.ST_FILL_SYMMETRIC, out=dense)
+        torch.mul(cubes, f, out=scaled)
+        sync()
+        st.st_pack(scaled, cube, out=packed)
+        sync()
+        for fl, a in zip(flags, A):
+            st.st_mttkrp_tri(packed, C, D, out=a, flags=fl)
+        return [dense.clone()] + [a.clone() for a in A] + [st.st_sym_moment4(X * f)]
+
+    want = {f: pass_of(f, True) for f in (1.0, -0.5, 3.0)}
+    bad = torch.zeros((), dtype=torch.int64, device="cuda")
+    for it in range(60):
+        f = (1.0, -0.5, 3.0)[it % 3]
+        for a, b in zip(pass_of(f, False), want[f]):
+            bad += (a != b).sum()
+    assert int(bad) == 0

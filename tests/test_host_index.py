@@ -160,3 +160,17 @@ def test_layout_sizes_and_host_side_validation():
     # beyond 64 features the tile table of the call lives in the workspace too
     assert st.st_workspace_bytes(st.ST_OP_SYM_MOMENT3, 100, 128) > 128 * 129 * 130 // 6 * 4 + 6528 * 4
     assert st.st_workspace_bytes(st.ST_OP_SYM_MOMENT2, 4096, 64, st.ST_F32) >= 256
+
+
+def test_kernels_do_not_read_through_the_read_only_path():
+    # Every kernel is launched as a programmatic dependent: its blocks may be there while its input is still being written.
+    # ld.global.nc, __ldg and what a compiler makes of `const T *__restrict__` kernel parameters are for data that is
+    # read-only for as long as the kernel lives.
+    found = []
+    for name in sorted(os.listdir(CSRC)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        found += [(name, w) for w in re.findall(r"__ldg\s*\(|ld\.global(?:\.\w+)*\.nc", text)]
+        for head in re.findall(r"__global__[^{;]*\{", text):
+            found += [(name, w) for w in re.findall(r"const\s+[\w:<> ]+\*\s*__restrict__", head)]
+        found += [(name, w) for w in re.findall(r"const\s+[\w:]+\s*\*\s*__restrict__\s*\w+\s*=\s*a\.", text)]
+    assert not found, found
