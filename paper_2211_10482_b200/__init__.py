@@ -231,6 +231,8 @@ def st_sym_moment3_static(X: torch.Tensor, out: torch.Tensor, flags: int = 0) ->
         raise TypeError("X and out must be float32")
     if out.numel() != d * (d + 1) * (d + 2) // 6:
         raise ValueError("out must hold d(d+1)(d+2)/6 elements")
+    if X.device != out.device:
+        raise ValueError("out must be on the device of X")
     _check(lib().st_sym_moment3_static(_dev(X, "X"), N, d, X.stride(0), _dev(out, "out"), flags, _stream()),
            "st_sym_moment3_static")
     return out

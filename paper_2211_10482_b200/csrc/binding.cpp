@@ -85,6 +85,28 @@ void *device_ptr(const at::Tensor &t, const char *name)
 
 const float *f32_ptr(const at::Tensor &t, const char *name) { return (const float *)device_ptr(t, name); }
 
+// The kernels run on one device and take every pointer as its memory.
+void want_device_of(const at::Tensor &x, const at::Tensor &t, const char *name)
+{
+    if (t.device() != x.device()) {
+        PyErr_Format(PyExc_ValueError, "%s must be on the device of the first operand", name);
+        throw Failed();
+    }
+}
+
+// The address that `bytes` bytes of results go to.
+void *result_ptr(const at::Tensor &x, PyObject *out, size_t bytes)
+{
+    const at::Tensor &t = tensor(out, "out");
+    void *p = device_ptr(t, "out");
+    want_device_of(x, t, "out");
+    if (t.nbytes() < bytes) {
+        PyErr_Format(PyExc_ValueError, "out has %zu bytes, the result %zu", (size_t)t.nbytes(), bytes);
+        throw Failed();
+    }
+    return p;
+}
+
 int64_t integer(PyObject *o)
 {
     const long long v = PyLong_AsLongLong(o);
@@ -212,9 +234,10 @@ Workspace workspace(PyObject *given, PyObject *like, const at::Tensor &t, int op
     }
     Ref hold(o);
     const at::Tensor &ws = tensor(o, "ws");
-    Ref index(PyLong_FromLong(ws.is_cuda() ? ws.get_device() : 0));
+    void *ptr = device_ptr(ws, "ws");
+    want_device_of(t, ws, "ws");
+    Ref index(PyLong_FromLong(ws.get_device()));
     if (PyDict_SetItem(last_ws, index.o, o) != 0) throw Failed();
-    void *ptr = ws.data_ptr();
     const size_t bytes = ws.nbytes();
     return Workspace{std::move(hold), ptr, bytes};
 }
@@ -262,7 +285,7 @@ PyObject *py_pack(PyObject *const *v)                    // dense, layout, out
     void *src = device_ptr(dense, "dense");
     Ref out(Py_None == v[2] ? [&] { Ref ty(PyObject_GetAttr(v[0], s_dtype)); return allocate(v[0], dense, {n}, dense.scalar_type(), ty.o); }()
                             : (Py_INCREF(v[2]), v[2]));
-    void *dst = device_ptr(tensor(out.o, "out"), "out");
+    void *dst = result_ptr(dense, out.o, (size_t)n * dense.element_size());
     call("st_pack", [&](void *s) { return api.pack(&l, type, src, dst, s); });
     return out.release();
 }
@@ -282,7 +305,7 @@ PyObject *py_unpack(PyObject *const *v)                  // packed, layout, fill
     void *src = device_ptr(packed, "packed");
     Ref out(Py_None == v[3] ? [&] { Ref ty(PyObject_GetAttr(v[0], s_dtype)); return allocate(v[0], packed, {n}, packed.scalar_type(), ty.o); }()
                             : (Py_INCREF(v[3]), v[3]));
-    void *dst = device_ptr(tensor(out.o, "out"), "out");
+    void *dst = result_ptr(packed, out.o, (size_t)n * packed.element_size());
     call("st_unpack", [&](void *s) { return api.unpack(&l, type, src, dst, fill, s); });
     return out.release();
 }
@@ -295,8 +318,9 @@ PyObject *py_thp(PyObject *const *v)                     // Bp, C, layout, out
     const st_layout l = layout_of(v[2]);
     if (B.numel() != api.packed_elems(&l) || C.numel() != api.dense_elems(&l)) fail(PyExc_ValueError, "shape mismatch");
     const float *b = f32_ptr(B, "Bp"), *c = f32_ptr(C, "C");
+    want_device_of(B, C, "C");
     Ref out(output(v[3], v[0], B, B.sizes()));
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(B, out.o, sizeof(float) * (size_t)B.numel());
     call("st_thp", [&](void *s) { return api.thp(&l, b, c, o, s); });
     return out.release();
 }
@@ -313,8 +337,9 @@ PyObject *py_axpby(PyObject *const *v)                   // alpha, a, beta, b, o
     const at::Tensor &a = tensor(v[1], "a"), &b = tensor(v[3], "b");
     want_pair(a, b);
     const float *pa = f32_ptr(a, "a"), *pb = f32_ptr(b, "b");
+    want_device_of(a, b, "b");
     Ref out(output(v[4], v[1], a, a.sizes()));
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(a, out.o, sizeof(float) * (size_t)a.numel());
     const int64_t n = a.numel();
     call("st_packed_axpby", [&](void *s) { return api.packed_axpby(n, alpha, pa, beta, pb, o, s); });
     return out.release();
@@ -325,8 +350,9 @@ PyObject *py_mul(PyObject *const *v)                     // a, b, out
     const at::Tensor &a = tensor(v[0], "a"), &b = tensor(v[1], "b");
     want_pair(a, b);
     const float *pa = f32_ptr(a, "a"), *pb = f32_ptr(b, "b");
+    want_device_of(a, b, "b");
     Ref out(output(v[2], v[0], a, a.sizes()));
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(a, out.o, sizeof(float) * (size_t)a.numel());
     const int64_t n = a.numel();
     call("st_packed_mul", [&](void *s) { return api.packed_mul(n, pa, pb, o, s); });
     return out.release();
@@ -344,7 +370,7 @@ PyObject *py_moment2(PyObject *const *v)                 // X, out, ws, flags
     const void *x = device_ptr(X, "X");
     Ref out(output(v[1], v[0], X, {d * (d + 1) / 2}));
     const Workspace w = workspace(v[2], v[0], X, ST_OP_SYM_MOMENT2, N, d, type, 0, flags);
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(X, out.o, sizeof(float) * (size_t)(d * (d + 1) / 2));
     call("st_sym_moment2", [&](void *s) { return api.sym_moment2(x, type, N, d, ldx, o, w.ptr, w.bytes, flags, s); });
     return out.release();
 }
@@ -360,7 +386,7 @@ PyObject *moment34(PyObject *const *v, int order)        // X, out, ws, flags
     const float *x = f32_ptr(X, "X");
     Ref out(output(v[1], v[0], X, {order == 3 ? tet : tet * (d + 3) / 4}));
     const Workspace w = workspace(v[2], v[0], X, order == 3 ? ST_OP_SYM_MOMENT3 : ST_OP_SYM_MOMENT4, N, d, 0, 0, flags);
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(X, out.o, sizeof(float) * (size_t)(order == 3 ? tet : tet * (d + 3) / 4));
     const auto f = order == 3 ? api.sym_moment3 : api.sym_moment4;
     call(order == 3 ? "st_sym_moment3" : "st_sym_moment4", [&](void *s) { return f(x, N, d, ldx, o, w.ptr, w.bytes, flags, s); });
     return out.release();
@@ -379,9 +405,11 @@ PyObject *py_mttkrp_tri(PyObject *const *v)              // Bp, C, D, out, ws, f
     const int64_t want = (flags & ST_FLAG_DENSE_CONTROL) ? I * I * K : I * (I + 1) / 2 * K;
     if (B.numel() != want || D.size(1) != R) fail(PyExc_ValueError, "shape mismatch");
     const float *b = f32_ptr(B, "Bp"), *c = f32_ptr(C, "C"), *d = f32_ptr(D, "D");
+    want_device_of(B, C, "C");
+    want_device_of(B, D, "D");
     Ref out(output(v[3], v[0], B, {I, R}));
     const Workspace w = workspace(v[4], v[0], B, ST_OP_MTTKRP_TRI, I, K, R, 0, flags);
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(B, out.o, sizeof(float) * (size_t)(I * R));
     call("st_mttkrp_tri", [&](void *s) { return api.mttkrp_tri(b, I, K, c, d, R, o, w.ptr, w.bytes, flags, s); });
     return out.release();
 }
@@ -397,9 +425,11 @@ PyObject *py_mttkrp_slice(PyObject *const *v)            // Bp, C, D, I, fixed_i
     const int64_t rows = fi >= 0 ? (fj >= 0 ? 1 : J) : I;
     if (B.numel() != rows * K || D.size(1) != R) fail(PyExc_ValueError, "shape mismatch");
     const float *b = f32_ptr(B, "Bp"), *c = f32_ptr(C, "C"), *d = f32_ptr(D, "D");
+    want_device_of(B, C, "C");
+    want_device_of(B, D, "D");
     Ref out(output(v[6], v[0], B, {I, R}));
     const Workspace w = workspace(v[7], v[0], B, ST_OP_MTTKRP_SLICE, I, J, K, R, flags);
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(B, out.o, sizeof(float) * (size_t)(I * R));
     call("st_mttkrp_slice", [&](void *s) { return api.mttkrp_slice(b, I, J, K, fi, fj, c, d, R, o, w.ptr, w.bytes, flags, s); });
     return out.release();
 }
@@ -415,9 +445,10 @@ PyObject *py_ttm_blockdiag(PyObject *const *v)           // Bp, U, nblocks, bs, 
     const int64_t rows = (flags & ST_FLAG_DENSE_CONTROL) ? d * d : nb * bs * bs;
     if (B.numel() != rows * K) fail(PyExc_ValueError, "shape mismatch");
     const float *b = f32_ptr(B, "Bp"), *u = f32_ptr(U, "U");
+    want_device_of(B, U, "U");
     Ref out(output(v[4], v[0], B, {rows, R}));
     const Workspace w = workspace(v[5], v[0], B, ST_OP_TTM_BLOCKDIAG, nb, bs, K, R, flags);
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(B, out.o, sizeof(float) * (size_t)(rows * R));
     call("st_ttm_blockdiag", [&](void *s) { return api.ttm_blockdiag(b, nb, bs, K, u, R, o, w.ptr, w.bytes, flags, s); });
     return out.release();
 }
@@ -434,9 +465,10 @@ PyObject *py_ttm_packed(PyObject *const *v)              // Bp, U, layout, out, 
     const int64_t rows = B.numel() / K;
     const unsigned flags = flag_bits(v[5]);
     const float *b = f32_ptr(B, "Bp"), *u = f32_ptr(U, "U");
+    want_device_of(B, U, "U");
     Ref out(output(v[3], v[0], B, {rows, R}));
     const Workspace w = workspace(v[4], v[0], B, ST_OP_TTM_BLOCKDIAG, rows, 1, K, R, flags);
-    float *o = (float *)device_ptr(tensor(out.o, "out"), "out");
+    float *o = (float *)result_ptr(B, out.o, sizeof(float) * (size_t)(rows * R));
     call("st_ttm_packed", [&](void *s) { return api.ttm_packed(&l, b, u, R, o, w.ptr, w.bytes, flags, s); });
     return out.release();
 }

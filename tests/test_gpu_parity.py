@@ -1271,3 +1271,33 @@ def test_inputs_written_by_the_kernel_just_before_are_read_as_written(st):
         for a, b in zip(pass_of(f, False), want[f]):
             bad += (a != b).sum()
     assert int(bad) == 0
+
+
+def test_a_buffer_that_a_call_would_write_past_is_refused_before_anything_runs(st):
+    lay, cube = st.Layout(st.ST_TRI_UPPER, 9, 2), st.Layout(st.ST_TRI_UPPER, 4, 8)
+    X, P, E, B = (torch.zeros(*s, device="cuda") for s in ((40, 9), (90,), (162,), (10, 8)))
+    C, U, blocks = (torch.zeros(*s, device="cuda") for s in ((4, 8), (8, 8), (12, 8)))
+    calls = {"pack": (90, lambda **k: st.st_pack(E, lay, **k)), "unpack": (162, lambda **k: st.st_unpack(P, lay, **k)),
+             "thp": (90, lambda **k: st.st_thp(P, E, lay, **k)), "axpby": (90, lambda **k: st.st_packed_axpby(1.0, P, 1.0, P, **k)),
+             "mul": (90, lambda **k: st.st_packed_mul(P, P, **k)), "moment2": (45, lambda **k: st.st_sym_moment2(X, **k)),
+             "moment3": (165, lambda **k: st.st_sym_moment3(X, **k)), "moment4": (495, lambda **k: st.st_sym_moment4(X, **k)),
+             "mttkrp": (32, lambda **k: st.st_mttkrp_tri(B, C, U, **k)),
+             "slice": (56, lambda **k: st.st_mttkrp_slice(B[:4], C, U, 7, fixed_i=2, **k)),
+             "blockdiag": (96, lambda **k: st.st_ttm_blockdiag(blocks, U, 3, 2, **k)),
+             "ttm": (80, lambda **k: st.st_ttm_packed(B, U, cube, **k))}
+    for name, (n, call) in calls.items():
+        room = torch.zeros(n + 8, device="cuda")
+        want = call().reshape(-1)
+        got = call(out=room)                                       # longer than needed is no harm, and the tail stays
+        assert got is room and torch.equal(room[:n], want) and int(torch.count_nonzero(room[n:])) == 0, name
+        for bad in (room[:n - 1], room[:n].to(torch.bfloat16), torch.zeros(n)):
+            with pytest.raises(ValueError):
+                call(out=bad)
+        with pytest.raises(TypeError):
+            call(out=room.data_ptr())
+        if name in ("pack", "unpack", "thp", "axpby", "mul"):
+            continue
+        for bad in (torch.zeros(1 << 20, dtype=torch.uint8), torch.zeros(1 << 20, dtype=torch.uint8, device="cuda")[::2],
+                    torch.zeros(1, dtype=torch.uint8, device="cuda").expand(1 << 20)):
+            with pytest.raises(ValueError):
+                call(ws=bad)
