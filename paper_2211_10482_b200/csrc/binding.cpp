@@ -11,6 +11,7 @@
 #include <cstdint>
 #include <cstring>
 #include <exception>
+#include <initializer_list>
 #include <map>
 #include <string>
 #include <tuple>
@@ -124,6 +125,15 @@ float real(PyObject *o)
     const double v = PyFloat_AsDouble(o);
     if (v == -1.0 && PyErr_Occurred()) throw Failed();
     return (float)v;
+}
+
+// The product, or -1, which no element count equals, where it leaves 64 bits.
+int64_t times(std::initializer_list<int64_t> factors)
+{
+    int64_t n = 1;
+    for (const int64_t f : factors)
+        if (f < 0 || __builtin_mul_overflow(n, f, &n)) return -1;
+    return n;
 }
 
 int64_t field(PyObject *layout, PyObject *name)
@@ -402,7 +412,7 @@ PyObject *py_mttkrp_tri(PyObject *const *v)              // Bp, C, D, out, ws, f
     for (const at::Tensor *t : {&B, &C, &D}) want_f32(*t, "inputs");
     const int64_t I = C.size(0), R = C.size(1), K = D.size(0);
     const unsigned flags = flag_bits(v[5]);
-    const int64_t want = (flags & ST_FLAG_DENSE_CONTROL) ? I * I * K : I * (I + 1) / 2 * K;
+    const int64_t want = (flags & ST_FLAG_DENSE_CONTROL) ? times({I, I, K}) : times({I % 2 ? I : I / 2, I % 2 ? (I + 1) / 2 : I + 1, K});
     if (B.numel() != want || D.size(1) != R) fail(PyExc_ValueError, "shape mismatch");
     const float *b = f32_ptr(B, "Bp"), *c = f32_ptr(C, "C"), *d = f32_ptr(D, "D");
     want_device_of(B, C, "C");
@@ -423,7 +433,7 @@ PyObject *py_mttkrp_slice(PyObject *const *v)            // Bp, C, D, I, fixed_i
     const int64_t J = C.size(0), R = C.size(1), K = D.size(0), I = integer(v[3]), fi = integer(v[4]), fj = integer(v[5]);
     const unsigned flags = flag_bits(v[8]);
     const int64_t rows = fi >= 0 ? (fj >= 0 ? 1 : J) : I;
-    if (B.numel() != rows * K || D.size(1) != R) fail(PyExc_ValueError, "shape mismatch");
+    if (B.numel() != times({rows, K}) || D.size(1) != R) fail(PyExc_ValueError, "shape mismatch");
     const float *b = f32_ptr(B, "Bp"), *c = f32_ptr(C, "C"), *d = f32_ptr(D, "D");
     want_device_of(B, C, "C");
     want_device_of(B, D, "D");
@@ -440,10 +450,10 @@ PyObject *py_ttm_blockdiag(PyObject *const *v)           // Bp, U, nblocks, bs, 
     want_2d(U, "U");
     want_f32(B, "inputs");
     want_f32(U, "inputs");
-    const int64_t K = U.size(0), R = U.size(1), nb = integer(v[2]), bs = integer(v[3]), d = nb * bs;
+    const int64_t K = U.size(0), R = U.size(1), nb = integer(v[2]), bs = integer(v[3]), d = times({nb, bs});
     const unsigned flags = flag_bits(v[6]);
-    const int64_t rows = (flags & ST_FLAG_DENSE_CONTROL) ? d * d : nb * bs * bs;
-    if (B.numel() != rows * K) fail(PyExc_ValueError, "shape mismatch");
+    const int64_t rows = (flags & ST_FLAG_DENSE_CONTROL) ? times({d, d}) : times({d, bs});
+    if (B.numel() != times({rows, K})) fail(PyExc_ValueError, "shape mismatch");
     const float *b = f32_ptr(B, "Bp"), *u = f32_ptr(U, "U");
     want_device_of(B, U, "U");
     Ref out(output(v[4], v[0], B, {rows, R}));

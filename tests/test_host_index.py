@@ -174,3 +174,16 @@ def test_kernels_do_not_read_through_the_read_only_path():
             found += [(name, w) for w in re.findall(r"const\s+[\w:<> ]+\*\s*__restrict__", head)]
         found += [(name, w) for w in re.findall(r"const\s+[\w:]+\s*\*\s*__restrict__\s*\w+\s*=\s*a\.", text)]
     assert not found, found
+
+
+def test_sizes_that_leave_64_bits_do_not_match_by_wrapping_around():
+    import torch
+    import paper_2211_10482_b200 as st
+    B, U = torch.zeros(4), torch.zeros(4, 8)
+    for nb, bs in ((2 ** 62 + 1, 1), (-(2 ** 62) + 1, 1), (-1, -1)):        # nb bs bs 4 = 4 modulo 2^64; two signs that cancel
+        with pytest.raises(ValueError, match="shape mismatch"):
+            st.st_ttm_blockdiag(B, U, nb, bs)
+    with pytest.raises(ValueError, match="shape mismatch"):                 # (2^32)^2 = 0 modulo 2^64
+        st.st_ttm_blockdiag(torch.zeros(0), U, 2 ** 32, 1, flags=st.ST_FLAG_DENSE_CONTROL)
+    with pytest.raises(ValueError, match="shape mismatch"):
+        st.st_mttkrp_tri(torch.zeros(0), torch.zeros(2 ** 33, 0), torch.zeros(4, 0))
