@@ -114,6 +114,16 @@ int64_t integer(PyObject *o)
     if (v == -1 && PyErr_Occurred()) throw Failed();
     return v;
 }
+// What int() makes of it.
+int64_t whole(PyObject *o)
+{
+    PyObject *v = PyNumber_Long(o);
+    if (!v) throw Failed();
+    const long long x = PyLong_AsLongLong(v);
+    Py_DECREF(v);
+    if (x == -1 && PyErr_Occurred()) throw Failed();
+    return x;
+}
 unsigned flag_bits(PyObject *o)
 {
     const unsigned long v = PyLong_AsUnsignedLongMask(o);
@@ -311,7 +321,7 @@ PyObject *py_unpack(PyObject *const *v)                  // packed, layout, fill
         throw Failed();
     }
     const st_dtype type = copy_dtype(packed);
-    const st_fill fill = (st_fill)integer(v[2]);
+    const st_fill fill = (st_fill)whole(v[2]);
     void *src = device_ptr(packed, "packed");
     Ref out(Py_None == v[3] ? [&] { Ref ty(PyObject_GetAttr(v[0], s_dtype)); return allocate(v[0], packed, {n}, packed.scalar_type(), ty.o); }()
                             : (Py_INCREF(v[3]), v[3]));

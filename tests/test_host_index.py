@@ -187,3 +187,15 @@ def test_sizes_that_leave_64_bits_do_not_match_by_wrapping_around():
         st.st_ttm_blockdiag(torch.zeros(0), U, 2 ** 32, 1, flags=st.ST_FLAG_DENSE_CONTROL)
     with pytest.raises(ValueError, match="shape mismatch"):
         st.st_mttkrp_tri(torch.zeros(0), torch.zeros(2 ** 33, 0), torch.zeros(4, 0))
+
+
+def test_a_fill_is_whatever_int_makes_of_it():
+    import torch
+    import paper_2211_10482_b200 as st
+    packed, lay = torch.zeros(6), st.Layout(st.ST_TRI_UPPER, 3)
+    for fill in (1, 1.0, "1", True, np.int64(1)):
+        with pytest.raises(ValueError, match="CUDA"):                       # accepted: the host tensor is what is refused
+            st.st_unpack(packed, lay, fill)
+    for fill in (None, "x", 1j):
+        with pytest.raises((TypeError, ValueError), match="int"):
+            st.st_unpack(packed, lay, fill)
