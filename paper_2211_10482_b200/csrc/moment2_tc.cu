@@ -335,7 +335,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             }
             fence_proxy_async();          // generic writes, read by the tensor core
             __syncwarp();
-            if (lane == 0) mbar_arrive_remote(bar0 + (uint32_t)(s * sizeof(uint64_t)));
+            if (lane == 0) mbar_arrive_cluster_smem(bar0 + (uint32_t)(s * sizeof(uint64_t)));
             s += CONV_GROUPS;
             while (s >= stages) { s -= stages; parity ^= 1u; }
         }

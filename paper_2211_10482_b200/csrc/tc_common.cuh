@@ -284,11 +284,12 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// The same without a cluster-wide release, for shared memory that this block's tensor core will read (after
-// fence_proxy_async): nothing has to travel.  With the release an arrival took 1100 to 1700 cycles.
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr)
+// The same where what has to be seen is in this block's shared memory: the release at cluster scope is a fence that orders
+// writes there only.  The full release also waits for the block's traffic with global memory: 1100 to 1700 cycles an arrival.
+__device__ __forceinline__ void mbar_arrive_cluster_smem(uint32_t cluster_addr)
 {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // TMA load whose completion is counted on a barrier that may live in the peer block of the pair
 // (no multicast: every block fetches its own tile).

@@ -199,3 +199,17 @@ def test_a_fill_is_whatever_int_makes_of_it():
     for fill in (None, "x", 1j):
         with pytest.raises((TypeError, ValueError), match="int"):
             st.st_unpack(packed, lay, fill)
+
+
+def test_arrivals_at_another_block_name_the_scope_of_the_cluster():
+    # An arrival orders nothing for another block's threads unless its scope, or that of a fence before a relaxed one, is the
+    # cluster's; without one it is that of the block.
+    found = []
+    for name in sorted(os.listdir(CSRC)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        for m in re.finditer(r"mbarrier\.arrive[\w.:]*shared::cluster", text):
+            if ".release.cluster" in m.group():
+                continue
+            if ".relaxed.cluster" not in m.group() or "fence.release.sync_restrict::shared::cta.cluster" not in text[max(0, m.start() - 200):m.start()]:
+                found.append((name, m.group()))
+    assert not found, found
