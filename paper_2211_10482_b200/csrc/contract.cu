@@ -247,51 +247,83 @@ __global__ void __launch_bounds__(RG_THREADS, 1) rowgemm_kernel(const RgArgs a)
     asm volatile("cp.async.wait_group 0;\n" ::);
 }
 
+constexpr int ROWSUM_BLOCKS = 16;            // per SM
+constexpr int ROWSUM_LONG = 64;              // mean number of slots of a reached row from which sixteen loads at a time pay
+
 // Second pass of MTTKRP: one warp per row of A adds the partial slots of that row in increasing
-// order (units, then k-splits) and writes the row; rows the fibres do not reach are zero.
-__global__ void __launch_bounds__(256)
-mttkrp_rowsum_kernel(const float *part, float *A, int64_t I_full, int64_t i_off, MttkrpRows m,
-                     int R, int unit_rows, int ksplit)
+// order (units, then k-splits); rows that no fibre reaches become zero.  The warps walk the rows, since a block for every eight
+// of them costs more to place than its stores take (slice i of [200000,1000,64], R = 32, one row that is not zero: 35 us the
+// call, now 17).  BATCH: loads at a time.  The one row of a slice i has thousands of slots and its sum is a chain of round
+// trips ([3000,50000,64], R = 32: eight 92 us, sixteen 41); where rows have few, the registers of sixteen keep blocks from
+// starting beside the running kernel ([900,900,48], R = 64, split: eight 76.5 us, sixteen 80).
+template <int BATCH>
+__global__ void __launch_bounds__(256, BATCH > 8 ? 1 : 8)
+mttkrp_rowsum_kernel(const float *part, float *A, int64_t I_full, int64_t i_off, MttkrpRows m, int R, int unit_shift, int ksplit)
 {
-    // where this warp's slots are takes two 64-bit divisions and does not have to wait
     const int lane = threadIdx.x & 31;
-    const int64_t ii = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t i = ii - i_off;
-    float *dst = A + ii * R;
-    int64_t first = 0, n = 0;
-    if (ii < I_full && i >= 0 && i < m.I) {
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    int64_t ii = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    int64_t first, n;
+    // the slots of row ii; n = 0: a row of zeros
+    auto slots_of = [&](int64_t row) {
+        const int64_t i = row - i_off;
+        first = n = 0;
+        if (i < 0 || i >= m.I) return;
         int64_t s, e;
         if (m.mode == MK_PACKED) { s = tri_row_start(m.I, i); e = s + (m.I - i); }
         else { s = i * m.div; e = s + m.div; }
         if (e > m.rows) e = m.rows;
-        if (e > s) {
-            const int64_t u0 = s / unit_rows, u1 = (e - 1) / unit_rows;
-            first = (u0 + i) * ksplit;
-            n = (u1 - u0 + 1) * ksplit;
-            if (!ST_BOUNDS_OK(first + n - 1, mttkrp_slots(m.rows, unit_rows, m.I, ksplit), 6)) n = -1;
-        }
-    }
+        if (e <= s) return;
+        const int64_t u0 = s >> unit_shift, u1 = (e - 1) >> unit_shift;
+        first = (u0 + i) * ksplit;
+        n = (u1 - u0 + 1) * ksplit;
+        if (!ST_BOUNDS_OK(first + n - 1, mttkrp_slots(m.rows, 1 << unit_shift, m.I, ksplit), 6)) n = -1;
+    };
+    if (ii < I_full) slots_of(ii);                             // the first row's do not have to wait
     pdl_wait();
     pdl_trigger();
-    if (ii >= I_full || n < 0) return;
-    for (int r = lane; r < R; r += 32) {
-        float sum = 0.f;
-        const float *p = part + first * R + r;
-        for (int64_t k = 0; k < n; k += 8) {               // eight independent loads in flight
-            float t[8];
+    while (ii < I_full) {
+        for (int r = lane; r < R && n >= 0; r += 32) {
+            float sum = 0.f;
+            const float *p = part + first * R + r;
+            int64_t k = 0;
+            for (; k + BATCH <= n; k += BATCH) {
+                float t[BATCH];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) t[u] = k + u < n ? __ldcg(p + (k + u) * R) : 0.f;
+                for (int u = 0; u < BATCH; ++u) t[u] = __ldcg(p + (k + u) * R);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) sum += t[u];
+                for (int u = 0; u < BATCH; ++u) sum += t[u];
+            }
+            if (BATCH > 8 && k + 8 <= n) {
+                float t[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) t[u] = __ldcg(p + (k + u) * R);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) sum += t[u];
+                k += 8;
+            }
+            if (k < n) {
+                float t[7];
+#pragma unroll
+                for (int u = 0; u < 7; ++u) t[u] = k + u < n ? __ldcg(p + (k + u) * R) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 7; ++u) sum += t[u];
+            }
+            A[ii * R + r] = sum;
         }
-        dst[r] = sum;
+        ii += warps;
+        if (ii < I_full) slots_of(ii);
     }
 }
 
 st_status mttkrp_rowsum_launch(const float *part, float *A_full, int64_t I_full, int64_t i_off, const MttkrpRows &m,
                                int R, int unit_rows, int ksplit, cudaStream_t stream)
 {
-    return launch(mttkrp_rowsum_kernel, dim3((unsigned)((I_full + 7) / 8)), 256, 0, stream, part, A_full, I_full, i_off, m, R, unit_rows, ksplit);
+    int shift = 0;                                             // units are powers of two
+    while ((1 << shift) < unit_rows) ++shift;
+    const int64_t want = (I_full + 7) / 8, cap = (int64_t)sm_count_or_default() * ROWSUM_BLOCKS;
+    const bool many = m.rows / unit_rows / m.I * ksplit >= ROWSUM_LONG;
+    return launch(many ? mttkrp_rowsum_kernel<16> : mttkrp_rowsum_kernel<8>, (unsigned)(want < cap ? want : cap), 256, 0, stream, part, A_full, I_full, i_off, m, R, shift, ksplit);
 }
 
 // tile shape by R: {TM, stages}; a warp owns TM * 32 / (R/8) consecutive fibres, a tile is the block's 16 warps

@@ -1301,3 +1301,24 @@ def test_a_buffer_that_a_call_would_write_past_is_refused_before_anything_runs(s
                     torch.zeros(1, dtype=torch.uint8, device="cuda").expand(1 << 20)):
             with pytest.raises(ValueError):
                 call(ws=bad)
+
+
+# row sums: a row of more slots than are loaded at a time (sixteen, eight, a remainder) and rows of none, more rows than the
+# warps of the grid; slices whose rows of A have one fibre each, several to a unit and a ragged last unit
+@pytest.mark.parametrize("flag_name,R,tol", [("f32", 64, TOL_F32), ("tf32", 32, 5e-3), ("split", 32, TOL_F32)])
+def test_mttkrp_slices_with_long_rows_and_with_many_rows(st, flag_name, R, tol):
+    flags = {"f32": 0, "tf32": st.ST_FLAG_TC_TF32, "split": st.ST_FLAG_TC_SPLIT}[flag_name]
+    for I, J, fi, fj in ((9, 4099, 5, -1), (3, 700, 0, -1), (30011, 7, -1, 3), (2, 3, 1, 2), (25000, 40, 24999, -1)):
+        K = 16
+        rows = (1 if fj >= 0 else J) if fi >= 0 else I
+        B, C, D = (workloads.draw(s, "normal", 7 + I) for s in ((rows, K), (J, R), (K, R)))
+        got = st.st_mttkrp_slice(dev(B), dev(C), dev(D), I, fi, fj, flags=flags).cpu().numpy()
+        Y, S = B.astype(np.float64) @ D, np.abs(B).astype(np.float64) @ np.abs(D)
+        Cr = C[fj:fj + 1] if fj >= 0 else C
+        want, size = np.zeros((I, R)), np.full((I, R), 1e-30)
+        if fi >= 0:
+            want[fi], size[fi] = (Y * Cr).sum(0), (S * np.abs(Cr)).sum(0)
+        else:
+            want, size = Y * Cr, S * np.abs(Cr)
+        assert np.max(np.abs(got - want) / size) <= tol, (I, J, fi, fj)
+        assert np.count_nonzero(got[size[:, 0] == 1e-30]) == 0
