@@ -75,11 +75,18 @@ __device__ __forceinline__ UnitFibres unit_fibres(int64_t row0, int64_t rows, bo
     }
     f.i0 = (int)i;
     const int end = dense ? (div > (int64_t(1) << 30) ? 1 << 30 : (int)div) : I;
-    // m fibres on from (i0, j0): row i ends at j = end - 1, the next one starts at 0 (dense) or on the diagonal
+    // m fibres on from (i0, j0): row i ends at j = end - 1, the next one starts at 0 (dense; with rows of one fibre, a slice
+    // j, the loop would go round m times) or on the diagonal
     auto at = [&](int m, int &ii, int &jj) {
         ii = (int)i;
         jj = (int)j + m;
-        while (jj >= end) { ++ii; jj = jj - end + (dense ? 0 : ii); }
+        if (dense) {
+            const int rows_on = jj >= end ? jj / end : 0;
+            ii += rows_on;
+            jj -= rows_on * end;
+        } else {
+            while (jj >= end) { ++ii; jj = jj - end + ii; }
+        }
     };
     int last;
     if (f.n > 0) at(f.n - 1, f.i1, last);
