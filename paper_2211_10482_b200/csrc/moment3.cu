@@ -23,7 +23,7 @@
 // travels as a kernel parameter; beyond that it is copied into the workspace before the launch,
 // stages get shorter (three of them must fit in shared memory) and more thread blocks share a
 // sample slice.  Rows that are not 16-byte aligned (d or ldx not a multiple of 4) are staged with
-// plain 4-byte loads instead of asynchronous 16-byte copies.
+// asynchronous copies of 4 bytes instead of 16.
 #include "st_common.cuh"
 #include "st_index.cuh"
 #include <algorithm>
@@ -101,14 +101,15 @@ __device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c)
 // One stage of rows for one tile.  acc[a][c] holds the sums for j = a, k = 2c and 2c+1.
 // DC > 0: the row length is the compile-time constant DC, so that every shared-memory address of
 // the loop is "row base + immediate" (integer multiply-adds share the FMA pipe: with run-time strides
-// the kernel was 9 % slower at d = 64).
-template <int J0, bool DIAG, int DC>
-__device__ __forceinline__ void m3_stage(const float *__restrict__ row, int rows, int step_, int pi, int oj, int ok, int half_,
+// the kernel was 9 % slower at d = 64).  GROUPS: the rows of a row group, `step` floats apart, by a pointer that goes on.
+template <int J0, bool DIAG, int DC, bool GROUPS>
+__device__ __forceinline__ void m3_stage(const float *__restrict__ xs, int rows, int step_, int pi, int oj, int ok, int half_,
                                          uint64_t (&acc)[8][4])
 {
     const int step = DC > 0 ? DC : step_, half = DC > 0 ? DC / 2 : half_;
 #pragma unroll 2
-    for (int r = 0; r < rows; ++r, row += step) {
+    for (int r = 0; r < rows; ++r, xs += GROUPS ? step : 0) {
+        const float *row = GROUPS ? xs : xs + r * step;
         const float xi = row[pi];
         const float4 ja = *reinterpret_cast<const float4 *>(row + oj);
         const float4 jb = *reinterpret_cast<const float4 *>(row + oj + half);
@@ -133,7 +134,7 @@ __device__ __forceinline__ void m3_stage(const float *__restrict__ row, int rows
 }
 
 // d: columns of X; dp: d rounded up to a multiple of 8 (row length of a stage); rows: sample rows per stage
-// (a multiple of 8, at most M3_STAGE_ROWS).  The tile table comes from `tab` when gtile is NULL.
+// (any number up to M3_STAGE_ROWS).  The tile table comes from `tab` when gtile is NULL.
 struct M3Args {
     const float *X;
     float *partials;
@@ -145,13 +146,15 @@ struct M3Args {
     int nw, rg;                            // rg > 1: the table has nw warps, and rg copies of them share the rows of a stage
 };
 
+// GROUPS: the instance for few features, below.  In one instance with it, the registers of its stride and its second epilogue
+// cost many features 4 %: [65536,128] 1300 us, now 1230; [20000,160] 924 and 879.
 // ALIGNED: rows are staged by asynchronous 16-byte copies; otherwise by 4-byte ones (an instance of
 // its own: with both loaders in one kernel the common one ran 7 % slower).
 //
 // Few features make few tiles: one warp's worth at d = 16.  Row group g of rg then takes rows g, g + rg, ... of every
 // stage, and the groups' sums are added in shared memory, in group order, before they go to memory.  [23208,16]: 32 us with
 // one warp per variant walking all rows, 12.5 now; [4096,24] 18.9 and 12.6.
-template <int WARPS, int DC, bool ALIGNED>
+template <int WARPS, int DC, bool ALIGNED, bool GROUPS>
 __global__ void __launch_bounds__(M3_THREADS, 1)
 moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
 {
@@ -167,7 +170,7 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
     extern __shared__ __align__(16) float smem[];   // M3_BUFFERS stages of a.rows x dp floats
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int group = blockIdx.x;
-    const int rg = DC > 0 ? 1 : a.rg;
+    const int rg = GROUPS ? a.rg : 1;
     const int row_group = rg > 1 ? warp / a.nw : 0;
     const int slot = rg > 1 ? warp - row_group * a.nw : group * M3_WPB + warp;
     const bool working = rg == 1 || row_group < rg;
@@ -232,22 +235,23 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
             load_stage((int)((s + M3_BUFFERS - 1) % M3_BUFFERS), n_begin + (s + M3_BUFFERS - 1) * stage_rows);
         else
             cp_async_commit();
-        // this row group's rows of the stage; rows past the end of the slice are not visited
+        // this row group's rows of the stage; rows past the end of the slice are zeros, and not visited where that is cheap to
+        // know (many features: with their number in a register of its own [65536,128] ran 1282 us, now 1230)
         const int64_t left = n_end - (n_begin + s * stage_rows);
         const int in_stage = left < stage_rows ? (int)left : stage_rows;
-        const int rows = rg > 1 ? (in_stage - row_group + rg - 1) / rg : in_stage;
+        const int rows = DC == 0 && !GROUPS ? stage_rows : rg > 1 ? (in_stage - row_group + rg - 1) / rg : in_stage;
         const int step = DC > 0 ? DC : rg * dp;
         const float *xs = smem + (int)(s % M3_BUFFERS) * stage_floats + row_group * dp;
         switch (variant) {
-        case 0: m3_stage<0, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
-        case 1: m3_stage<0, true, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
-        case 2: m3_stage<1, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
-        case 3: m3_stage<2, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
-        case 4: m3_stage<3, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
-        case 5: m3_stage<4, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
-        case 6: m3_stage<5, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
-        case 7: m3_stage<6, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
-        case 8: m3_stage<7, false, DC>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 0: m3_stage<0, false, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 1: m3_stage<0, true, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 2: m3_stage<1, false, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 3: m3_stage<2, false, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 4: m3_stage<3, false, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 5: m3_stage<4, false, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 6: m3_stage<5, false, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 7: m3_stage<6, false, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
+        case 8: m3_stage<7, false, DC, GROUPS>(xs, rows, step, pi, oj, ok, half, acc); break;
         default: break;
         }
     }
@@ -583,8 +587,9 @@ static st_status moment3_launch(const float *X, int64_t N, int64_t d, int64_t ld
         return launch(kernel, dim3(p.groups, p.slices), M3_THREADS, p.smem, stream, a, *param);
     };
     // d = 60, 64 has its own instance with compile-time strides
-    const st_status rc = !aligned ? run(moment3_kernel<WARPS, 0, false>)
-                       : p.dp == M3_PARAM_D ? run(moment3_kernel<WARPS, M3_PARAM_D, true>) : run(moment3_kernel<WARPS, 0, true>);
+    const st_status rc = tab.rg > 1 ? (aligned ? run(moment3_kernel<WARPS, 0, true, true>) : run(moment3_kernel<WARPS, 0, false, true>))
+                       : !aligned ? run(moment3_kernel<WARPS, 0, false, false>)
+                       : p.dp == M3_PARAM_D ? run(moment3_kernel<WARPS, M3_PARAM_D, true, false>) : run(moment3_kernel<WARPS, 0, true, false>);
     if (rc != ST_OK) return rc;
     return launch(sum_slices_kernel, dim3((unsigned)((p.out_elems + 31) / 32)), 32 * SUM_GROUPS, 0, stream, a.partials, out, p.out_elems, p.slices);
 }
