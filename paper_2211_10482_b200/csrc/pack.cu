@@ -48,13 +48,10 @@ template <> struct Elem<4> { typedef uint32_t T; };
 template <> struct Elem<8> { typedef uint2 T; };
 template <> struct Elem<16> { typedef uint4 T; };
 
-// 16 bytes at byte `off` (a multiple of ES) of the two aligned units at p.
+// 16 bytes at byte `off` (a multiple of ES, not 0) of the two aligned units a and b.
 template <int ES>
-__device__ __forceinline__ uint4 load_unit(const uint4 *p, unsigned off)
+__device__ __forceinline__ uint4 shift_unit(const uint4 &a, const uint4 &b, unsigned off)
 {
-    const uint4 a = p[0];
-    if (off == 0) return a;
-    const uint4 b = p[1];
     uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x;
     if (off & 8) { w0 = a.z; w1 = a.w; w2 = b.x; w3 = b.y; w4 = b.z; }
     if (ES < 8) {
@@ -96,20 +93,39 @@ __device__ __forceinline__ void copy_flat(unsigned char *dst, const unsigned cha
     const uint4 *in = reinterpret_cast<const uint4 *>(src + head - off);
     uint4 *out = reinterpret_cast<uint4 *>(dst + head);
     const uint4 *m = MUL ? reinterpret_cast<const uint4 *>(mul + head) : nullptr;
-    for (int u0 = lane; u0 < units; u0 += U * g) {
-        uint4 v[U], w[U];
+    // The loads of a batch come before its first store in the source: coherent loads are not moved over a store by the compiler.
+    auto store = [&](int u, uint4 v, const uint4 &w) {
+        if (MUL) v = make_uint4(mul_word(v.x, w.x), mul_word(v.y, w.y), mul_word(v.z, w.z), mul_word(v.w, w.w));
+        out[u] = v;
+    };
+    if (ES == 16 || off == 0) {
+        for (int u0 = lane; u0 < units; u0 += U * g) {
+            uint4 v[U], w[U];
 #pragma unroll
-        for (int k = 0; k < U; ++k)
-            if (u0 + k * g < units) {
-                v[k] = load_unit<ES>(in + u0 + k * g, off);
-                if (MUL) w[k] = m[u0 + k * g];
-            }
+            for (int k = 0; k < U; ++k)
+                if (u0 + k * g < units) {
+                    v[k] = in[u0 + k * g];
+                    if (MUL) w[k] = m[u0 + k * g];
+                }
 #pragma unroll
-        for (int k = 0; k < U; ++k)
-            if (u0 + k * g < units) {
-                if (MUL) v[k] = make_uint4(mul_word(v[k].x, w[k].x), mul_word(v[k].y, w[k].y), mul_word(v[k].z, w[k].z), mul_word(v[k].w, w[k].w));
-                out[u0 + k * g] = v[k];
-            }
+            for (int k = 0; k < U; ++k)
+                if (u0 + k * g < units) store(u0 + k * g, v[k], w[k]);
+        }
+    } else {
+        constexpr int H = U > 1 ? U / 2 : U;                // two loads a unit: batches of half as many
+        for (int u0 = lane; u0 < units; u0 += H * g) {
+            uint4 v[H], y[H], w[H];
+#pragma unroll
+            for (int k = 0; k < H; ++k)
+                if (u0 + k * g < units) {
+                    v[k] = in[u0 + k * g];
+                    y[k] = in[u0 + k * g + 1];
+                    if (MUL) w[k] = m[u0 + k * g];
+                }
+#pragma unroll
+            for (int k = 0; k < H; ++k)
+                if (u0 + k * g < units) store(u0 + k * g, shift_unit<ES>(v[k], y[k], off), w[k]);
+        }
     }
     if (e0 < ends) *reinterpret_cast<E *>(dst + end_at(e0)) = ev;
     for (int e = e0 + g * ES; e < ends; e += g * ES) *reinterpret_cast<E *>(dst + end_at(e)) = end_load(e);   // small groups only
@@ -203,8 +219,11 @@ __device__ __forceinline__ void slice_run(const LayoutArgs &a, I &s, I &lo, I &h
     }
 }
 
+// Four blocks per SM: with the registers that the compiler would take (up to 96) fewer fit, and the zeros of a sparse slice are
+// bound by the number of blocks ([8000,8000] band 39.5 us, 37.7 with 64 registers; st_thp of a tet d = 120, rows of 64 floats
+// 52, now 39).
 template <int KIND, int ES, bool PACK, bool MUL, typename I>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I nitems, int group_shift, int parts,
                   int part_bytes, const unsigned char *mul)
 {
@@ -234,7 +253,7 @@ slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I 
         const int64_t x0 = u0 > c0 ? u0 : c0, x1 = u1 < c1 ? u1 : c1;   // run clipped to this part
         const int64_t p0 = (int64_t)prow * a.row_bytes - c0;           // packed byte of dense byte 0 of the slice, were it in the run
         if (PACK) {
-            if (x1 > x0) copy_flat<ES, MUL, COPY_UNITS>(dst + p0 + x0, src + (int64_t)s * sb + x0, mul + p0 + x0, (int)(x1 - x0), lane, g);
+            if (x1 > x0) copy_flat<ES, MUL, MUL ? COPY_UNITS / 2 : COPY_UNITS>(dst + p0 + x0, src + (int64_t)s * sb + x0, mul + p0 + x0, (int)(x1 - x0), lane, g);
             if (KIND == ST_BAND && part == 0) {
                 // slots of the fixed-width packed row that fall outside the matrix
                 unsigned char *row = dst + (int64_t)s * a.width * a.row_bytes;
@@ -301,7 +320,7 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
         if (xr < x1) {
             const I p = KIND == ST_TRI_UPPER ? tri_at<I>(d, a, xr) : KIND == ST_TET ? tet_at<I>(d, a, b, xr) : simp4_at<I>(d, a, b, c, xr);
             if (ST_BOUNDS_OK(p, packed_rows, 1) && ST_BOUNDS_OK((int64_t)p + (x1 - xr) - 1, packed_rows, 1))
-                copy_flat<ES, false, WIDE ? 2 : 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32);
+                copy_flat<ES, false, ES >= 8 ? 2 : 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32);
         }
         const I xe = x1 < top ? x1 : top;
         const int words = row_bytes / ES;
