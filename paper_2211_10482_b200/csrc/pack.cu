@@ -177,8 +177,8 @@ template <typename I> __device__ __forceinline__ void tet_dec(I d, I q, I &i, I 
 }
 
 // Run of unique columns of slice s: dense columns [lo,hi) of the slice map to packed rows prow.. (contiguous).
-// PACK of an order-3 or order-4 tensor visits the slices with a run only: item s is then the s-th of those, and s becomes
-// the number of its slice.
+// PACK of an order-3 or order-4 tensor or of one row visits the slices with a run only: item s is then the s-th of those, and
+// s becomes the number of its slice.
 template <int KIND, bool PACK, typename I>
 __device__ __forceinline__ void slice_run(const LayoutArgs &a, I &s, I &lo, I &hi, I &prow)
 {
@@ -197,6 +197,7 @@ __device__ __forceinline__ void slice_run(const LayoutArgs &a, I &s, I &lo, I &h
         if (hi < lo) hi = lo;
         prow = s * (I)a.width + (lo + kl - s);
     } else if (KIND == ST_FIXED_ROW) {
+        if (PACK) s = kl;
         if (s == kl) { lo = 0; hi = d; } else { lo = hi = 0; }
         prow = 0;
     } else if (KIND == ST_FIXED_COL) {
@@ -522,21 +523,24 @@ template <int KIND, int ES, bool PACK>
 static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cudaStream_t s, const void *mul)
 {
     const int64_t cap = MAX_GRID;
-    // slices: about four 16-byte units per thread, at most PART_BYTES per (slice, part).  Pack splits the
-    // longest run of unique columns, unpack the whole dense slice.
+    // slices: about four 16-byte units per thread, at most PART_BYTES per (slice, part), less where the slices are too few to
+    // fill the chip (one row of [1000,1000,128] in 16 parts 17 us the call with its empty slices, now 1.8).  Pack splits the
+    // longest run of unique columns (a band: its packed row), unpack the whole dense slice.
     int64_t run_rows = a.d;
     if (KIND == ST_BAND) run_rows = a.width < a.d ? a.width : a.d;
     if (KIND == ST_BLOCKDIAG) run_rows = a.bs;
     if (KIND == ST_FIXED_COL) run_rows = 1;
     const int64_t sb = (PACK ? run_rows : a.d) * a.row_bytes;
-    int64_t parts = (sb + PART_BYTES - 1) / PART_BYTES;
+    // pack of a tensor of order 3 or 4, or of one row: only the slices that have a run
+    const int64_t nslices = PACK && KIND == ST_FIXED_ROW ? 1 : KIND == ST_TET ? (PACK ? tri_rows(a.d) : a.d * a.d) : KIND == ST_SIMPLEX4 ? (PACK ? tet_rows(a.d) : a.d * a.d * a.d) : a.d;
+    int64_t part_bytes = PART_BYTES;
+    while (part_bytes > 4096 && nslices * ((sb + part_bytes - 1) / part_bytes) < 2 * (int64_t)sm_count_or_default()) part_bytes /= 2;
+    int64_t parts = (sb + part_bytes - 1) / part_bytes;
     const int64_t pb = ((sb + parts - 1) / parts + 15) / 16 * 16;
     parts = (sb + pb - 1) / pb;
     if (parts > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
     int shift = 0;
     while ((1 << shift) < 256 && (int64_t(16 * COPY_UNITS) << shift) < pb) ++shift;
-    // pack of a tensor of order 3 or 4: only the slices that have a run
-    const int64_t nslices = KIND == ST_TET ? (PACK ? tri_rows(a.d) : a.d * a.d) : KIND == ST_SIMPLEX4 ? (PACK ? tet_rows(a.d) : a.d * a.d * a.d) : a.d;
     const int64_t nitems = nslices * parts, threads = nitems << shift;
     const int64_t want = (threads + 255) / 256;
     const unsigned grid = (unsigned)(want < cap ? (want < 1 ? 1 : want) : cap);
