@@ -245,23 +245,22 @@ slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I 
                          ST_BOUNDS_OK((int64_t)prow + (hi - lo) - 1, a.packed_rows, 1)))
             continue;
         const int64_t c0 = (int64_t)lo * a.row_bytes, c1 = (int64_t)hi * a.row_bytes;   // the run inside the slice
-        // pack splits the run itself into parts, unpack the whole dense slice (it writes all of it)
-        const int64_t r0 = PACK ? c0 : 0, r1 = PACK ? c1 : sb;
-        int64_t u0 = r0 + part * part_bytes;                  // this part covers dense bytes [u0, u1) of the slice
+        // pack splits the run itself into parts (a band's fixed-width packed row, whose slots outside the matrix are zeros),
+        // unpack the whole dense slice (it writes all of it)
+        constexpr bool BAND_ROW = PACK && KIND == ST_BAND;
+        const int64_t shift = BAND_ROW ? ((int64_t)prow - (int64_t)s * a.width) * a.row_bytes - c0 : 0;
+        const int64_t d0 = c0 + shift, d1 = c1 + shift;       // the run inside what is split
+        const int64_t r0 = PACK && !BAND_ROW ? c0 : 0, r1 = BAND_ROW ? a.width * a.row_bytes : PACK ? c1 : sb;
+        int64_t u0 = r0 + part * part_bytes;                  // this part covers bytes [u0, u1) of it
         int64_t u1 = u0 + part_bytes;
         if (u0 > r1) u0 = r1;
         if (u1 > r1) u1 = r1;
-        const int64_t x0 = u0 > c0 ? u0 : c0, x1 = u1 < c1 ? u1 : c1;   // run clipped to this part
-        const int64_t p0 = (int64_t)prow * a.row_bytes - c0;           // packed byte of dense byte 0 of the slice, were it in the run
+        const int64_t x0 = u0 > d0 ? u0 : d0, x1 = u1 < d1 ? u1 : d1;   // run clipped to this part
+        const int64_t p0 = (int64_t)prow * a.row_bytes - d0;           // packed byte of its byte 0, were it in the run
         if (PACK) {
-            if (x1 > x0) copy_flat<ES, MUL, MUL ? COPY_UNITS / 2 : COPY_UNITS>(dst + p0 + x0, src + (int64_t)s * sb + x0, mul + p0 + x0, (int)(x1 - x0), lane, g);
-            if (KIND == ST_BAND && part == 0) {
-                // slots of the fixed-width packed row that fall outside the matrix
-                unsigned char *row = dst + (int64_t)s * a.width * a.row_bytes;
-                const int64_t first = ((int64_t)prow - (int64_t)s * a.width) * a.row_bytes, last = first + (c1 - c0), wb = a.width * a.row_bytes;
-                for (int64_t z = 0; z < first; z += part_bytes) zero_flat<ES>(row + z, (int)(first - z < part_bytes ? first - z : part_bytes), lane, g);
-                for (int64_t z = last; z < wb; z += part_bytes) zero_flat<ES>(row + z, (int)(wb - z < part_bytes ? wb - z : part_bytes), lane, g);
-            }
+            if (BAND_ROW && d0 > u0) zero_flat<ES>(dst + p0 + u0, (int)((u1 < d0 ? u1 : d0) - u0), lane, g);
+            if (x1 > x0) copy_flat<ES, MUL, MUL ? COPY_UNITS / 2 : COPY_UNITS>(dst + p0 + x0, src + (int64_t)s * sb + x0 - shift, mul + p0 + x0, (int)(x1 - x0), lane, g);
+            if (BAND_ROW && u1 > d1) zero_flat<ES>(dst + p0 + (u0 > d1 ? u0 : d1), (int)(u1 - (u0 > d1 ? u0 : d1)), lane, g);
         } else {
             unsigned char *out = dst + (int64_t)s * sb;
             const int64_t z1 = u1 < c0 ? u1 : c0;               // zeros before the run
@@ -527,7 +526,7 @@ static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cu
     // fill the chip (one row of [1000,1000,128] in 16 parts 17 us the call with its empty slices, now 1.8).  Pack splits the
     // longest run of unique columns (a band: its packed row), unpack the whole dense slice.
     int64_t run_rows = a.d;
-    if (KIND == ST_BAND) run_rows = a.width < a.d ? a.width : a.d;
+    if (KIND == ST_BAND) run_rows = a.width;
     if (KIND == ST_BLOCKDIAG) run_rows = a.bs;
     if (KIND == ST_FIXED_COL) run_rows = 1;
     const int64_t sb = (PACK ? run_rows : a.d) * a.row_bytes;
