@@ -11,6 +11,7 @@
 //   split into parts over several thread groups.
 //   sym_slice_kernel (st_unpack with symmetric fill): the positions of a slice from its largest fixed index on
 //   are such a run too; in front of it every position is mapped through the redundancy map by itself.
+//   sym_row_kernel: the same for wide positions, each by itself.
 //   sym_tile_kernel: the same for a matrix of single elements, through 32 x 32 tiles.
 //
 // A run starts wherever the closed form says, so source and destination usually differ in their offset from a
@@ -29,6 +30,7 @@ constexpr int COPY_UNITS = 4;              // 16-byte units that a thread of the
 // strides, of which only some fit at a time, it was written in several sweeps with holes ([4096,4096,64] zero fill 755 us,
 // now 624; [2000,2000,64] 253, now 229).
 constexpr int64_t MAX_GRID = int64_t(1) << 30;
+constexpr int ROW_SEG = 2048, ROW_WIDE = 512;   // symmetric fill of wide positions
 constexpr int SYM_WORDS = 4;               // words that a lane of the symmetric fill has in flight
 constexpr int64_t PART_BYTES = 32768;      // most of a slice that one thread group copies ([384,384,75]: 128 KiB starve the chip)
 
@@ -281,6 +283,33 @@ __device__ __forceinline__ I sym_row(I d, I a, I b, I c, I x)
     return x < a ? simp4_at<I>(d, x, a, b, c) : x < b ? simp4_at<I>(d, a, x, b, c) : simp4_at<I>(d, a, b, x, c);
 }
 
+// Fixed indices of slice s in increasing order (as many as KIND has); returns the largest.
+template <int KIND, typename I>
+__device__ __forceinline__ I sym_fixed(I d, I s, I &a, I &b, I &c)
+{
+    I t;
+    b = c = 0;
+    if (KIND == ST_TRI_UPPER) return a = s;
+    if (KIND == ST_TET) {
+        a = s / d; b = s - a * d;
+        if (a > b) { t = a; a = b; b = t; }
+        return b;
+    }
+    const I ij = s / d;
+    c = s - ij * d; a = ij / d; b = ij - a * d;
+    if (a > b) { t = a; a = b; b = t; }
+    if (b > c) { t = b; b = c; c = t; }
+    if (a > b) { t = a; a = b; b = t; }
+    return c;
+}
+
+// Packed row of position x of the slice whose fixed indices are a <= b <= c, from the largest on.
+template <int KIND, typename I>
+__device__ __forceinline__ I sym_run_row(I d, I a, I b, I c, I x)
+{
+    return KIND == ST_TRI_UPPER ? tri_at<I>(d, a, x) : KIND == ST_TET ? tet_at<I>(d, a, b, x) : simp4_at<I>(d, a, b, c, x);
+}
+
 // One warp per part of a slice.  Positions from the largest fixed index on: one flat copy.  In front of it lanes run along
 // the words of the positions (up to 32 words each), or a lane group copies a position (`inner` elements) at a time.
 template <int KIND, int ES, typename I>
@@ -289,9 +318,6 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
                  int row_bytes, unsigned inv, int group_shift, int64_t packed_rows)
 {
     typedef typename Elem<ES>::T E;
-    // rows of whole 16-byte units of a matrix: two units of a lane in flight ([1000,1000,40] 56 us, now 49; the shorter runs
-    // of a tet got slower)
-    constexpr bool WIDE = ES == 16 && KIND == ST_TRI_UPPER;
     pdl_wait();
     pdl_trigger();
     const int lane = (int)(threadIdx.x & 31);
@@ -300,25 +326,12 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
         const I s = parts == 1 ? item : item / (I)parts;
         const I x0 = (item - s * (I)parts) * (I)part_rows;
         const I x1 = x0 + (I)part_rows < d ? x0 + (I)part_rows : d;
-        I a, b = 0, c = 0, top, t;                                       // fixed indices in increasing order
-        if (KIND == ST_TRI_UPPER) {
-            a = top = s;
-        } else if (KIND == ST_TET) {
-            a = s / d; b = s - a * d;
-            if (a > b) { t = a; a = b; b = t; }
-            top = b;
-        } else {
-            const I ij = s / d;
-            c = s - ij * d; a = ij / d; b = ij - a * d;
-            if (a > b) { t = a; a = b; b = t; }
-            if (b > c) { t = b; b = c; c = t; }
-            if (a > b) { t = a; a = b; b = t; }
-            top = c;
-        }
+        I a, b, c;
+        const I top = sym_fixed<KIND, I>(d, s, a, b, c);
         unsigned char *out = dst + (int64_t)s * d * row_bytes;
         const I xr = x0 > top ? x0 : top;                                // first position of the run in this part
         if (xr < x1) {
-            const I p = KIND == ST_TRI_UPPER ? tri_at<I>(d, a, xr) : KIND == ST_TET ? tet_at<I>(d, a, b, xr) : simp4_at<I>(d, a, b, c, xr);
+            const I p = sym_run_row<KIND, I>(d, a, b, c, xr);
             if (ST_BOUNDS_OK(p, packed_rows, 1) && ST_BOUNDS_OK((int64_t)p + (x1 - xr) - 1, packed_rows, 1))
                 copy_flat<ES, false, ES >= 8 ? 2 : 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32);
         }
@@ -350,11 +363,34 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
                 if (!ST_BOUNDS_OK(p, packed_rows, 1)) continue;
                 unsigned char *o = out + (int64_t)x * row_bytes;
                 const unsigned char *from = src + (int64_t)p * row_bytes;
-                // more than one unit per lane: two in flight (aligned rows: rows of 800 bytes 172 us at d = 700, now 141)
-                if (WIDE && row_bytes > 512) copy_flat<ES, false, 2>(o, from, nullptr, row_bytes, lane & (g - 1), g);
-                else copy_flat<ES, false, 1>(o, from, nullptr, row_bytes, lane & (g - 1), g);
+                copy_flat<ES, false, 1>(o, from, nullptr, row_bytes, lane & (g - 1), g);
             }
         }
+    }
+}
+
+// Positions of more than ROW_WIDE bytes: a warp copies up to ROW_SEG bytes of one, U units of a lane in flight, in the order of
+// the dense array.  sym_slice_kernel, which served them before, has one unit in flight, one warp for a position however wide,
+// and blocks that walk the array: [384,384,300] 63 us, now 50; simplex4 d = 10, 5000 floats, 79 and 36; tri d = 12, 20000
+// floats, 26 and 4.4.
+template <int KIND, int ES, int U, typename I>
+__global__ void __launch_bounds__(256)
+sym_row_kernel(const unsigned char *src, unsigned char *dst, I d, I nitems, I segs, int64_t row_bytes, int64_t packed_rows)
+{
+    pdl_wait();
+    pdl_trigger();
+    const int lane = (int)(threadIdx.x & 31);
+    const I nwarps = (I)gridDim.x * (I)(blockDim.x / 32);
+    for (I item = (I)blockIdx.x * (I)(blockDim.x / 32) + (I)(threadIdx.x / 32); item < nitems; item += nwarps) {
+        const I row = segs == 1 ? item : item / segs;
+        const int64_t off = (int64_t)(item - row * segs) * ROW_SEG;
+        const I s = row / d, x = row - s * d;
+        I a, b, c;
+        const I top = sym_fixed<KIND, I>(d, s, a, b, c);
+        const I p = x < top ? sym_row<KIND, I>(d, a, b, c, x) : sym_run_row<KIND, I>(d, a, b, c, x);
+        if (!ST_BOUNDS_OK(p, packed_rows, 1)) continue;
+        const int n = row_bytes - off < ROW_SEG ? (int)(row_bytes - off) : ROW_SEG;
+        copy_flat<ES, false, U>(dst + (int64_t)row * row_bytes + off, src + (int64_t)p * row_bytes + off, nullptr, n, lane, 32);
     }
 }
 
@@ -498,19 +534,29 @@ static st_status launch_sym(const void *src, void *dst, const LayoutArgs &a, cud
         const dim3 grid(nt * (nt + 1) / 2, KIND == ST_TRI_UPPER ? 1u : (unsigned)a.d, KIND == ST_SIMPLEX4 ? (unsigned)a.d : 1u);
         return launch(sym_tile_kernel<KIND, ES>, grid, 256, 0, s, (const E *)src, (E *)dst, (unsigned)a.d, nt, a.packed_rows);
     }
-    if (a.row_bytes > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
-    // parts of about 2 KiB (4 KiB of 16-byte words)
-    const int64_t words = a.row_bytes / ES;
-    const int64_t part_rows = words <= 32 ? 256 / words < 8 ? 8 : 256 / words : (2048 + a.row_bytes - 1) / a.row_bytes;
+    const unsigned char *in = (const unsigned char *)src;
+    unsigned char *out = (unsigned char *)dst;
+    if (a.row_bytes > ROW_WIDE) {
+        const int64_t segs = (a.row_bytes + ROW_SEG - 1) / ROW_SEG, items = a.dense_rows * segs, want = (items + 7) / 8;
+        const unsigned grid = (unsigned)(want < MAX_GRID ? want : MAX_GRID);
+        const bool two = a.row_bytes <= 1024;              // units per lane
+        if (small && items < (int64_t(1) << 30))
+            return launch(two ? sym_row_kernel<KIND, ES, 2, unsigned> : sym_row_kernel<KIND, ES, 4, unsigned>, grid, 256, 0, s, in, out, (unsigned)a.d,
+                          (unsigned)items, (unsigned)segs, a.row_bytes, a.packed_rows);
+        return launch(two ? sym_row_kernel<KIND, ES, 2, int64_t> : sym_row_kernel<KIND, ES, 4, int64_t>, grid, 256, 0, s, in, out, a.d, items, segs,
+                      a.row_bytes, a.packed_rows);
+    }
+    // parts of about 2 KiB (4 KiB of 16-byte words), less where there are too few to fill the chip
+    const int64_t words = a.row_bytes / ES, nslices = a.dense_rows / a.d;
+    int64_t part_rows = words <= 32 ? 256 / words < 8 ? 8 : 256 / words : (2048 + a.row_bytes - 1) / a.row_bytes;
+    while (part_rows > 2 && nslices * ((a.d + part_rows - 1) / part_rows) < 16 * (int64_t)sm_count_or_default()) part_rows = (part_rows + 1) / 2;
     const unsigned inv = words <= 32 ? (unsigned)((65536 + words - 1) / words) : 0u;
     const int64_t parts = (a.d + part_rows - 1) / part_rows;
     int shift = 0;
     while (shift < 5 && (int64_t(16) << shift) < a.row_bytes) ++shift;
-    const int64_t nslices = a.dense_rows / a.d, items = nslices * parts;
+    const int64_t items = nslices * parts;
     const int64_t want = (items + 7) / 8, cap = (int64_t)sm_count_or_default() * 16;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
-    const unsigned char *in = (const unsigned char *)src;
-    unsigned char *out = (unsigned char *)dst;
     if (small && items < (int64_t(1) << 31))
         return launch(sym_slice_kernel<KIND, ES, unsigned>, grid, 256, 0, s, in, out, (unsigned)a.d, (unsigned)nslices, (int)parts, (int)part_rows,
                       (int)a.row_bytes, inv, shift, a.packed_rows);

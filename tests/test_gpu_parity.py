@@ -1322,3 +1322,28 @@ def test_mttkrp_slices_with_long_rows_and_with_many_rows(st, flag_name, R, tol):
             want, size = Y * Cr, S * np.abs(Cr)
         assert np.max(np.abs(got - want) / size) <= tol, (I, J, fi, fj)
         assert np.count_nonzero(got[size[:, 0] == 1e-30]) == 0
+
+
+# a band wider than the matrix, whose packed rows have several parts of zeros; one row in many parts; symmetric fills of wide
+# positions: two and four units per lane, several segments, of whole words of every size and of none
+@pytest.mark.parametrize("kind,d,inner,dtype,k", [
+    ("ST_BAND", 7, 3, np.uint32, dict(kl=4000, ku=3000)), ("ST_BAND", 40, 1, np.uint16, dict(kl=900, ku=33)), ("ST_BAND", 19, 5, np.uint64, dict(kl=0, ku=700)),
+    ("ST_FIXED_ROW", 300, 333, np.uint16, dict(kl=17)), ("ST_FIXED_ROW", 61, 64, np.uint32, dict(kl=60)),
+    ("ST_TRI_UPPER", 33, 132, np.uint32, {}), ("ST_TRI_UPPER", 20, 200, np.uint32, {}), ("ST_TRI_UPPER", 21, 66, np.uint64, {}), ("ST_TRI_UPPER", 9, 257, np.uint16, {}),
+    ("ST_TRI_UPPER", 5, 1537, np.uint32, {}), ("ST_TET", 9, 132, np.uint32, {}), ("ST_TET", 7, 1031, np.uint16, {}), ("ST_SIMPLEX4", 5, 515, np.uint32, {}),
+    ("ST_SIMPLEX4", 4, 130, np.uint64, {}), ("ST_TET", 12, 40, np.uint32, {})])
+def test_copies_of_wide_bands_rows_and_positions(st, kind, d, inner, dtype, k):
+    lay = st.Layout(getattr(st, kind), d, inner, **k)
+    nd = st.st_dense_elems(lay)
+    dense = np.random.default_rng(nd).integers(1, np.iinfo(dtype).max, size=nd, dtype=dtype)
+    signed = {2: np.int16, 4: np.int32, 8: np.int64}[dense.itemsize]
+    packed = oracle.pack(dense, lay.kind, d, inner=inner, **okw(lay))
+    got = st.st_pack(torch.from_numpy(dense.view(signed)).cuda(), lay)
+    assert np.array_equal(got.cpu().numpy().view(dtype), packed)
+    for fill in [st.ST_FILL_ZERO] + ([st.ST_FILL_SYMMETRIC] if not k else []):
+        want = oracle.unpack(packed, lay.kind, d, inner=inner, fill=fill, **okw(lay)).reshape(-1)
+        assert np.array_equal(st.st_unpack(got, lay, fill=fill).cpu().numpy().view(dtype), want), fill
+    if dtype == np.uint32:
+        B, C = (workloads.draw((n,), "normal", 5) for n in (packed.size, nd))
+        want = B * oracle.pack(C.view(np.uint32), lay.kind, d, inner=inner, **okw(lay)).view(np.float32)
+        assert np.array_equal(st.st_thp(dev(B), dev(C), lay).cpu().numpy(), want)
