@@ -31,6 +31,9 @@ constexpr int MG_KC = 8;        // sample rows per stage; the loop over them is 
 constexpr int MG_STAGES = 4;
 constexpr int MG_THREADS = 128;
 constexpr size_t MG_SMEM = (size_t)MG_STAGES * 2 * MG_KC * MG_T * sizeof(float);   // 32 KiB
+// One block per SM, where all blocks find one: behind another kernel they were placed two to an SM and left others idle
+// ([500,640] 18.8 us, now 13.3; [2000,256] 17.4 and 12.7).
+constexpr size_t MG_SMEM_ALONE = 120 * 1024;
 
 // What a tile computes of its four 64x64 quadrants.
 enum { MG_FULL = 0,             // all four
@@ -71,6 +74,17 @@ __device__ __forceinline__ void mg_tile(const MgGrid &g, int kind, int t, int &b
     }
 }
 
+// Tiles of each kind; returns the edge of the triangle of full and diagonal ones.
+static int mg_kinds(int64_t nt, int64_t d, bool dense, int n[4])
+{
+    const int full = (int)(d - (nt - 1) * MG_T <= 64 ? nt - 1 : nt);
+    n[MG_FULL] = dense ? (int)(nt * nt) : full * (full - 1) / 2;
+    n[MG_DIAG] = dense ? 0 : full;
+    n[MG_LEFT] = !dense && full < nt ? (int)nt - 1 : 0;
+    n[MG_QUAD] = !dense && full < nt ? 1 : 0;
+    return full;
+}
+
 // 64x64 quadrants computed per sample row.
 static int64_t moment2_gemm_quads(int64_t d, bool dense)
 {
@@ -86,16 +100,7 @@ static MgGrid moment2_gemm_plan(int64_t N, int64_t d, unsigned flags)
 {
     MgGrid g;
     g.nt = (int)((d + MG_T - 1) / MG_T);
-    g.full = (d - (int64_t)(g.nt - 1) * MG_T <= 64) ? g.nt - 1 : g.nt;
-    if (flags & ST_FLAG_DENSE_CONTROL) {
-        g.n[0] = g.nt * g.nt;
-        g.n[1] = g.n[2] = g.n[3] = 0;
-    } else {
-        g.n[MG_FULL] = g.full * (g.full - 1) / 2;
-        g.n[MG_DIAG] = g.full;
-        g.n[MG_LEFT] = g.full < g.nt ? g.nt - 1 : 0;
-        g.n[MG_QUAD] = g.full < g.nt ? 1 : 0;
-    }
+    g.full = mg_kinds(g.nt, d, (flags & ST_FLAG_DENSE_CONTROL) != 0, g.n);
     // Two thread blocks fit on an SM.  The splits of a full tile (w) are the number whose blocks fill whole waves of
     // 2 x SMs best, the smallest such number within 3 %; cheaper tiles get fewer splits in proportion, so that all
     // blocks take about as long.
@@ -128,6 +133,10 @@ static MgGrid moment2_gemm_plan(int64_t N, int64_t d, unsigned flags)
     return g;
 }
 
+// Blocks of the sum per SM together: with 128 for every tile, half of which had nothing to do, [64,4096] took 163 us, now 70.
+constexpr int MG_SUM_BLOCKS = 16;
+__host__ __device__ inline int mg_sum_warps(int nsplit) { return nsplit <= 8 ? 1 : nsplit <= 16 ? 2 : nsplit <= 32 ? 4 : 8; }   // about eight loads per thread
+
 // out[p(i,j)] = sum over the sample splits of a tile of 128 x 128 partial sums; i <= j only.  `wps` warps share 32
 // columns of a row: the first adds the splits 0, wps, 2 wps, ... with its loads in flight, and so on, then the sums are
 // added in order (a fixed order).  After the other kernels of a pipeline have streamed gigabytes, every dependent round
@@ -146,7 +155,7 @@ moment2_gemm_reduce_kernel(const float *partials, float *out, int d, const MgGri
     const int nsplit = g.split[kind];
     const float *base = partials + (size_t)(g.first[kind] + t) * (T * T);
     const size_t stride = (size_t)g.n[kind] * (T * T);
-    const int wps = nsplit <= 8 ? 1 : nsplit <= 16 ? 2 : nsplit <= 32 ? 4 : 8;      // about eight loads per thread
+    const int wps = mg_sum_warps(nsplit);
     pdl_wait();
     pdl_trigger();
     if (bi > bj) return;                                 // dense control: lower tiles are discarded
@@ -314,15 +323,27 @@ static st_status moment2_gemm(const float *X, int64_t N, int64_t d, int64_t ldx,
     if (!aligned256(ws)) return ST_ERR_ALIGN;
     float *partials = (float *)((unsigned char *)ws + kWsHeaderBytes);
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0, vec = d % 4 == 0 && ldx % 4 == 0;
-    auto run = [&](auto kernel) { return launch(kernel, g.first[4], MG_THREADS, MG_SMEM, stream, X, N, (int)d, ldx, partials, g, (unsigned *)ws); };
+    const size_t smem = g.first[4] <= sm_count_or_default() ? MG_SMEM_ALONE : MG_SMEM;
+    auto run = [&](auto kernel) {
+        if (!ensure_dynamic_smem(kernel, smem)) return ST_ERR_CUDA;
+        return launch(kernel, g.first[4], MG_THREADS, smem, stream, X, N, (int)d, ldx, partials, g, (unsigned *)ws);
+    };
     const st_status rc = dense ? (vec ? run(moment2_gemm_kernel<true, true>) : run(moment2_gemm_kernel<true, false>))
                                : (vec ? run(moment2_gemm_kernel<false, true>) : run(moment2_gemm_kernel<false, false>));
     if (rc != ST_OK) return rc;
-    return launch(dense ? moment2_gemm_reduce_kernel<true> : moment2_gemm_reduce_kernel<false>, dim3(g.n[0] + g.n[1] + g.n[2] + g.n[3], 128), 256, 0,
-                  stream, partials, out, (int)d, g);
+    // blocks for all rows of a tile, but not more than MG_SUM_BLOCKS per SM together
+    const int tiles = g.n[0] + g.n[1] + g.n[2] + g.n[3];
+    int most = 0;
+    for (int k = 0; k < 4; ++k)
+        if (g.n[k] > 0 && g.split[k] > most) most = g.split[k];
+    int blocks = MG_T * MG_T / 32 / 8 * mg_sum_warps(most);
+    const int cap = MG_SUM_BLOCKS * sm_count_or_default() / tiles;
+    if (blocks > cap) blocks = cap < 8 ? 8 : cap;
+    return launch(dense ? moment2_gemm_reduce_kernel<true> : moment2_gemm_reduce_kernel<false>, dim3(tiles, blocks), 256, 0, stream, partials, out,
+                  (int)d, g);
 }
 
-// Which of the two kernels: the one with fewer FMA slots per sample row, each divided by the fraction of the FMA
+// Which of the two kernels.  Many samples: the one with fewer FMA slots per sample row, each divided by the fraction of the FMA
 // peak that it reaches with those slots (register tiles 0.60: [1048576,64] 107 us; 128 x 128 tiles 0.75).
 static bool moment2_use_small(int64_t d, unsigned flags)
 {
