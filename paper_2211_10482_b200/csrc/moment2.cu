@@ -21,6 +21,7 @@ st_status moment2_split_tc(const float *X, int64_t N, int64_t d, int64_t ldx, fl
                            unsigned flags, cudaStream_t stream);
 size_t moment2_split_tc_workspace(int64_t N, int64_t d, unsigned flags);
 int64_t moment2_small_slots(int64_t d, unsigned flags);
+int64_t moment2_small_items(int64_t d, unsigned flags);
 size_t moment2_small_workspace(int64_t N, int64_t d, unsigned flags);
 st_status moment2_small(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
                         unsigned flags, cudaStream_t stream);
@@ -345,11 +346,23 @@ static st_status moment2_gemm(const float *X, int64_t N, int64_t d, int64_t ldx,
 
 // Which of the two kernels.  Many samples: the one with fewer FMA slots per sample row, each divided by the fraction of the FMA
 // peak that it reaches with those slots (register tiles 0.60: [1048576,64] 107 us; 128 x 128 tiles 0.75).
-static bool moment2_use_small(int64_t d, unsigned flags)
+// Few samples of more than 128 features: the register tiles write and add a partial result per SM, which takes as long as about
+// 70 samples of a full 128 x 128 tile per work item; the samples have to make up for that by what they save (15400 slots take as
+// long as a full tile).  Register tiles / 128 x 128 tiles, us: [4096,129] 17.0 / 14.9, [6000,129] 18.2 / 21.0,
+// [2000,160] 18.2 / 10.8, [16384,160] 28.3 / 26.6, [30000,160] 36.1 / 41.4, [64,248] 24.5 / 10, [4096,248] 33.0 / 20.1,
+// [30000,248] 65.7 / 56.4, [200000,248] 284 / 318.
+static bool moment2_use_small(int64_t N, int64_t d, unsigned flags)
 {
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
     const int64_t slots = moment2_small_slots(d, flags);
     if (slots == 0) return false;
+    if (d > 128) {
+        int n[4];
+        mg_kinds((d + MG_T - 1) / MG_T, d, dense, n);
+        double tiles = 0;
+        for (int k = 0; k < 4; ++k) tiles += MG_COST[k] * n[k];
+        if ((double)N * (tiles - (double)slots / 15400) < 70.0 * (double)moment2_small_items(d, flags)) return false;
+    }
     return (double)slots / 0.60 <= (double)(moment2_gemm_quads(d, dense) * 4096) / 0.75;
 }
 
@@ -357,7 +370,7 @@ static st_status moment2_f32(const float *X, int64_t N, int64_t d, int64_t ldx, 
                              size_t ws_bytes, unsigned flags, cudaStream_t stream)
 {
     if (d > 32768) return ST_ERR_UNSUPPORTED;
-    return moment2_use_small(d, flags) ? moment2_small(X, N, d, ldx, out, ws, ws_bytes, flags, stream)
+    return moment2_use_small(N, d, flags) ? moment2_small(X, N, d, ldx, out, ws, ws_bytes, flags, stream)
                                        : moment2_gemm(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
 }
 
@@ -370,7 +383,7 @@ size_t moment2_workspace(int64_t N, int64_t d, int xdt, unsigned flags)
     if (xdt == ST_F32 && (flags & ST_FLAG_TC_TF32)) return moment2_tf32_tc_workspace(N, d, flags & ~ST_FLAG_TC_TF32);
     if (xdt == ST_F32 && (flags & ST_FLAG_TC_SPLIT)) return moment2_split_tc_workspace(N, d, flags & ~ST_FLAG_TC_SPLIT);
     if (xdt != ST_F32 || d > 32768) return 0;
-    return moment2_use_small(d, flags) ? moment2_small_workspace(N, d, flags)
+    return moment2_use_small(N, d, flags) ? moment2_small_workspace(N, d, flags)
                                        : kWsHeaderBytes + mg_partial_bytes(moment2_gemm_plan(N, d, flags));
 }
 

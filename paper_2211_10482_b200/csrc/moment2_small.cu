@@ -370,6 +370,9 @@ int64_t moment2_small_slots(int64_t d, unsigned flags)
     return 128 * M2S_MAX_THREADS / (M2S_MAX_THREADS / n);
 }
 
+// Work items.
+int64_t moment2_small_items(int64_t d, unsigned flags) { return m2s_nitems((int)((d + 7) / 8), (flags & ST_FLAG_DENSE_CONTROL) != 0); }
+
 static M2SmallPlan moment2_small_plan(int64_t N, int64_t d, unsigned flags)
 {
     M2SmallPlan p;

@@ -1347,3 +1347,15 @@ def test_copies_of_wide_bands_rows_and_positions(st, kind, d, inner, dtype, k):
         B, C = (workloads.draw((n,), "normal", 5) for n in (packed.size, nd))
         want = B * oracle.pack(C.view(np.uint32), lay.kind, d, inner=inner, **okw(lay)).view(np.float32)
         assert np.array_equal(st.st_thp(dev(B), dev(C), lay).cpu().numpy(), want)
+
+
+# fp32 second moment of more than 128 features on both sides of the line between its two kernels, and of many tiles with few
+# samples, whose sums go round with fewer blocks than rows
+@pytest.mark.parametrize("N,d", [(4900, 129), (5000, 129), (1, 130), (9900, 160), (10100, 160), (33, 193), (1000, 248), (37000, 248), (5, 1300), (70, 2100),
+                                 (600, 640)])
+def test_moment2_f32_few_samples_of_many_features(st, N, d):
+    X = workloads.draw((N, d), "normal", 11 + N + d)
+    got = st.st_sym_moment2(dev(X)).cpu().numpy().astype(np.float64)
+    i, j = np.triu_indices(d)
+    X64 = X.astype(np.float64)
+    assert np.max(np.abs(got - (X64.T @ X64)[i, j]) / (np.abs(X64).T @ np.abs(X64))[i, j]) <= TOL_F32
