@@ -22,13 +22,14 @@
 #include "st_common.cuh"
 #include "st_index.cuh"
 #include "tc_common.cuh"
+#include "moment2_rule.cuh"
+#include <tuple>
 
 namespace st {
 
 constexpr int M2S_MAX_THREADS = 256;
 constexpr int M2S_MAX_BLOCKS = 31;         // column blocks: one item per thread at most (d <= 248; dense control: 22 blocks)
 constexpr int M2S_BUFFERS = 3;
-constexpr int M2S_CLUSTER = 16;            // one-launch form: blocks of a cluster
 constexpr int M2S_CLUSTER_THREADS = 128;   // half the threads: half the sums to add ([4096,64] 7.1 us, with 256 threads 7.9)
 constexpr int M2S_CLUSTER_ITEMS = 5;       // at most, per cluster ([4096,100]: five 9.3 us, three 15.2; [4096,64]: 7.1, nine 8.1)
 constexpr int M2S_STAGE_BYTES = 57344;     // upper bound of one stage (3 stages + slack fit in 227 KB)
@@ -429,27 +430,19 @@ static M2SmallPlan moment2_cluster_plan(int64_t N, int64_t d, unsigned flags, in
     return p;
 }
 
-// Few samples: one launch instead of two, about 2 us of the host's time per call.  On the GPU (us, one launch / two):
-// [256,64] 5.0 / 7.5, [4096,8] 4.0 / 5.8, [4096,64] 7.1 / 7.7, [4096,100] 9.3 / 12.3, but [16384,24] 8.3 / 6.3 and
-// [16384,64] 12.0 / 10.1: its blocks are fewer, and every cluster reads all of X.  Copies word by word: [256,75] 5.6 / 8.4,
-// [4096,75] 12.2 / 9.9.
-static bool m2s_use_cluster(int64_t N, int64_t d, bool bulk) { return N * d <= (bulk ? 300000 : 100000); }
-
 size_t moment2_small_workspace(int64_t N, int64_t d, unsigned flags)
 {
     return kWsHeaderBytes + moment2_small_plan(N, d, flags).partial_bytes;
 }
 
 template <class Kernel>
-static st_status m2s_launch_cluster(Kernel kernel, int clusters, const M2SmallPlan &p, const M2SmallArgs &a, cudaStream_t stream)
+static cudaLaunchConfig_t m2s_cluster_config(const M2SmallPlan &p, int clusters, cudaStream_t stream, cudaLaunchAttribute (&attr)[2])
 {
-    if (!ensure_dynamic_smem(kernel, p.smem) || (M2S_CLUSTER > 8 && !allow_large_clusters(kernel))) return ST_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(M2S_CLUSTER, (unsigned)clusters);
     cfg.blockDim = dim3((unsigned)p.threads);
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = M2S_CLUSTER;
     attr[0].val.clusterDim.y = 1;
@@ -458,36 +451,75 @@ static st_status m2s_launch_cluster(Kernel kernel, int clusters, const M2SmallPl
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, kernel, a) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return ST_ERR_CUDA;
+    return cfg;
+}
+
+// Clusters of a plan that can be active at once on the current device, asked once per shape of the launch.
+template <class Kernel>
+static int m2s_fitting_clusters(Kernel kernel, const M2SmallPlan &p, int clusters)
+{
+    static std::mutex lock;
+    static std::map<std::tuple<const void *, int, int, size_t>, int> known;
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const auto key = std::make_tuple((const void *)kernel, dev, p.threads, p.smem);
+    {
+        std::lock_guard<std::mutex> guard(lock);
+        const auto it = known.find(key);
+        if (it != known.end()) return it->second;
     }
-    return ST_OK;
+    if (ensure_dynamic_smem(kernel, p.smem) && allow_large_clusters(kernel)) {
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = m2s_cluster_config<Kernel>(p, clusters, nullptr, attr);
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+    }
+    std::lock_guard<std::mutex> guard(lock);
+    return known[key] = n;
 }
 
 st_status moment2_small(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
                         unsigned flags, cudaStream_t stream)
 {
     const bool bulk = d % 4 == 0 && ldx % 4 == 0;
-    int clusters = 0;
-    const M2SmallPlan p = m2s_use_cluster(N, d, bulk) ? moment2_cluster_plan(N, d, flags, clusters) : moment2_small_plan(N, d, flags);
-    if (!ws || ws_bytes < kWsHeaderBytes + p.partial_bytes) return ST_ERR_WORKSPACE;
+    if (!ws || ws_bytes < kWsHeaderBytes) return ST_ERR_WORKSPACE;
     if (!aligned256(ws)) return ST_ERR_ALIGN;
     M2SmallArgs a;
-    a.X = X;
-    a.partials = (float *)((unsigned char *)ws + kWsHeaderBytes);
-    a.N = N; a.ldx = ldx; a.rows_per_slice = p.rows_per_slice;
-    a.d = (int)d; a.pitch = p.pitch; a.nbk = p.nbk; a.rg = p.rg; a.rpg = p.rpg;
-    a.nitems = p.nitems;
-    a.status = (unsigned *)ws;
-    a.bar_floats = (int)(p.data_bytes / sizeof(float));
-    a.dense = (flags & ST_FLAG_DENSE_CONTROL) ? 1 : 0;
-    if (clusters > 0) {
-        a.out = out;
-        a.items_all = m2s_nitems(p.nbk, a.dense != 0);
-        return bulk ? m2s_launch_cluster(moment2_small_kernel<true, true>, clusters, p, a, stream)
-                    : m2s_launch_cluster(moment2_small_kernel<false, true>, clusters, p, a, stream);
+    auto fill = [&](const M2SmallPlan &p) {
+        a.X = X;
+        a.partials = (float *)((unsigned char *)ws + kWsHeaderBytes);
+        a.N = N; a.ldx = ldx; a.rows_per_slice = p.rows_per_slice;
+        a.d = (int)d; a.pitch = p.pitch; a.nbk = p.nbk; a.rg = p.rg; a.rpg = p.rpg;
+        a.nitems = p.nitems;
+        a.status = (unsigned *)ws;
+        a.bar_floats = (int)(p.data_bytes / sizeof(float));
+        a.dense = (flags & ST_FLAG_DENSE_CONTROL) ? 1 : 0;
+    };
+    {
+        int clusters = 0;
+        const M2SmallPlan p = moment2_cluster_plan(N, d, flags, clusters);
+        const int items = (int)moment2_small_items(d, flags);
+        auto run = [&](auto kernel) {
+            // (a first look without the device, so that calls that are far from it do not ask)
+            if (!m2s_use_cluster(N, items, clusters, p.rg, bulk, clusters) ||
+                !m2s_use_cluster(N, items, clusters, p.rg, bulk, m2s_fitting_clusters(kernel, p, clusters)))
+                return false;
+            fill(p);
+            a.out = out;
+            a.items_all = items;
+            cudaLaunchAttribute attr[2];
+            cudaLaunchConfig_t cfg = m2s_cluster_config<decltype(kernel)>(p, clusters, stream, attr);
+            if (cudaLaunchKernelEx(&cfg, kernel, a) == cudaSuccess) return true;
+            (void)cudaGetLastError();                  // a context with fewer SMs than the one that was asked: two launches
+            return false;
+        };
+        if (bulk ? run(moment2_small_kernel<true, true>) : run(moment2_small_kernel<false, true>)) return ST_OK;
     }
+    const M2SmallPlan p = moment2_small_plan(N, d, flags);
+    if (ws_bytes < kWsHeaderBytes + p.partial_bytes) return ST_ERR_WORKSPACE;
+    fill(p);
     auto run = [&](auto kernel) {
         if (!ensure_dynamic_smem(kernel, p.smem)) return ST_ERR_CUDA;
         return launch(kernel, p.slices, p.threads, p.smem, stream, a);

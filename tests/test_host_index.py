@@ -213,3 +213,26 @@ def test_arrivals_at_another_block_name_the_scope_of_the_cluster():
             if ".relaxed.cluster" not in m.group() or "fence.release.sync_restrict::shared::cta.cluster" not in text[max(0, m.start() - 200):m.start()]:
                 found.append((name, m.group()))
     assert not found, found
+
+
+def test_the_one_launch_second_moment_is_taken_where_clusters_fit_and_it_was_measured_to_be_faster():
+    src = os.path.join(tempfile.mkdtemp(prefix="st_rule_"), "rule.cpp")
+    with open(src, "w") as f:
+        f.write('#include "moment2_rule.cuh"\nextern "C" int rule(long long N, int items, int clusters, int rg, int bulk, int fit)\n'
+                "{ return st::m2s_use_cluster(N, items, clusters, rg, bulk != 0, fit); }\n")
+    subprocess.check_call(["g++", "-shared", "-fPIC", "-std=c++17", "-I", CSRC, src, "-o", src + ".so"])
+    rule = ctypes.CDLL(src + ".so").rule
+    rule.argtypes = [ctypes.c_longlong] + [ctypes.c_int] * 5
+
+    def use(N, d, fit=8):                                        # items, clusters and row groups as the plan makes them
+        nbk = (d + 7) // 8
+        items = (nbk * (nbk + 1) // 2 + 1) // 2
+        clusters = (items + 4) // 5
+        per = (items + clusters - 1) // clusters
+        rg = min(128 // per, 57344 // (4 * ((d + 3) // 4 * 4)) // 8)
+        return rule(N, items, (items + per - 1) // per, rg, d % 4 == 0, fit)
+
+    for N, d in ((32, 8), (16384, 8), (8192, 16), (4096, 24), (4096, 64), (8192, 64), (1, 100), (4096, 100), (3000, 120), (2000, 33), (1000, 75)):
+        assert use(N, d) and not use(N, d, fit=0), (N, d)        # no cluster fits: the two launches
+    for N, d in ((30000, 8), (16384, 16), (6000, 24), (16384, 64), (6000, 100), (4096, 120), (3000, 33), (2000, 75)):
+        assert not use(N, d), (N, d)
