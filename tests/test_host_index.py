@@ -232,7 +232,7 @@ def test_the_one_launch_second_moment_is_taken_where_clusters_fit_and_it_was_mea
         rg = min(128 // per, 57344 // (4 * ((d + 3) // 4 * 4)) // 8)
         return rule(N, items, (items + per - 1) // per, rg, d % 4 == 0, fit)
 
-    for N, d in ((32, 8), (16384, 8), (8192, 16), (4096, 24), (4096, 64), (8192, 64), (1, 100), (4096, 100), (3000, 120), (2000, 33), (1000, 75)):
+    for N, d in ((32, 8), (16384, 8), (8192, 16), (4096, 24), (8000, 64), (1, 100), (4096, 100), (3000, 120), (2000, 33), (1000, 75)):
         assert use(N, d) and not use(N, d, fit=0), (N, d)        # no cluster fits: the two launches
     for N, d in ((30000, 8), (16384, 16), (6000, 24), (16384, 64), (6000, 100), (4096, 120), (3000, 33), (2000, 75)):
         assert not use(N, d), (N, d)
