@@ -16,6 +16,7 @@ OBJDIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libstructtensor.so")
 BINDING_SRC = os.path.join(CSRC, "binding.cpp")
 BINDING = os.path.join(HERE, "_binding.so")
+BINDING_KEY = os.path.join(OBJDIR, "binding.key")      # what _binding.so was built for
 # debug build with device-side range checks (-DST_BOUNDS_CHECK; relocatable device code for its one device-wide word)
 OBJDIR_CHECK = os.path.join(HERE, "_build_check")
 LIB_CHECK = os.path.join(HERE, "libstructtensor_check.so")
@@ -56,9 +57,17 @@ def _compile(src: str, verbose: bool, check: bool = False) -> str:
     return obj
 
 
+def _binding_key() -> str:
+    """The Python and the torch that a binding is compiled against: it holds for no other."""
+    import torch
+    return "python %s, torch %s" % (sys.version.split()[0], torch.__version__)
+
+
 def _build_binding(force: bool) -> None:
     deps = (BINDING_SRC, os.path.join(INCLUDE, "structtensor.h"))
-    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(map(os.path.getmtime, deps)):
+    key = _binding_key()
+    built_for = open(BINDING_KEY).read() if os.path.exists(BINDING_KEY) else ""
+    if not force and built_for == key and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(map(os.path.getmtime, deps)):
         return
     import sysconfig
 
@@ -76,10 +85,14 @@ def _build_binding(force: bool) -> None:
     if res.returncode != 0:
         raise RuntimeError("g++ failed for binding.cpp:\n%s\n%s" % (res.stdout, res.stderr))
     os.replace(tmp, BINDING)
+    os.makedirs(OBJDIR, exist_ok=True)
+    with open(BINDING_KEY, "w") as f:
+        f.write(key)
 
 
 def build(force: bool = False, verbose: bool = False, check: bool = False) -> str:
-    """Compiles every .cu under csrc/ and links the shared library (check=True: the range-checking debug build)."""
+    """Compiles every .cu under csrc/ and links the shared library (check=True: the range-checking debug build), and the
+    binding, which both builds are called through."""
     objdir, lib = (OBJDIR_CHECK, LIB_CHECK) if check else (OBJDIR, LIB)
     os.makedirs(objdir, exist_ok=True)
     if force:
@@ -88,10 +101,9 @@ def build(force: bool = False, verbose: bool = False, check: bool = False) -> st
                 os.remove(os.path.join(objdir, f))
     srcs = _sources()
     with concurrent.futures.ThreadPoolExecutor(max_workers=min(8, len(srcs) + 1)) as ex:
-        binding = None if check else ex.submit(_build_binding, force)
+        binding = ex.submit(_build_binding, force)
         objs = list(ex.map(lambda s: _compile(s, verbose, check), srcs))
-    if binding is not None:
-        binding.result()
+    binding.result()
     if force or not os.path.exists(lib) or any(os.path.getmtime(o) > os.path.getmtime(lib) for o in objs):
         tmp = lib + ".%d.tmp" % os.getpid()
         cmd = ["nvcc", "-shared", "-gencode", "arch=compute_100a,code=sm_100a", *(["-rdc=true"] if check else []), "-o", tmp, *objs]

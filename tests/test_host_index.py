@@ -236,3 +236,27 @@ def test_the_one_launch_second_moment_is_taken_where_clusters_fit_and_it_was_mea
         assert use(N, d) and not use(N, d, fit=0), (N, d)        # no cluster fits: the two launches
     for N, d in ((30000, 8), (16384, 16), (6000, 24), (16384, 64), (6000, 100), (4096, 120), (3000, 33), (2000, 75)):
         assert not use(N, d), (N, d)
+
+
+def test_the_binding_belongs_to_either_build_and_to_one_python_and_torch(tmp_path, monkeypatch):
+    from paper_2211_10482_b200 import _build
+    for name in ("OBJDIR", "OBJDIR_CHECK", "LIB", "LIB_CHECK", "BINDING"):
+        monkeypatch.setattr(_build, name, str(tmp_path / name))
+    monkeypatch.setattr(_build, "BINDING_KEY", str(tmp_path / "key"))
+    monkeypatch.setattr(_build, "_sources", lambda: [])
+    made = []
+
+    def run(cmd, **kw):
+        made.append(cmd[0])
+        open(cmd[cmd.index("-o") + 1], "w").close()
+        return subprocess.CompletedProcess(cmd, 0, "", "")
+
+    monkeypatch.setattr(_build.subprocess, "run", run)
+    _build.build(check=True)
+    assert made == ["g++", "nvcc"] or made == ["nvcc", "g++"]
+    _build.build(check=True)
+    _build._build_binding(False)
+    assert len(made) == 2                                        # up to date
+    monkeypatch.setattr(_build, "_binding_key", lambda: "another torch")
+    _build._build_binding(False)
+    assert made[2:] == ["g++"]
