@@ -770,7 +770,8 @@ int64_t moment2_split_part_rows(int64_t N) { return (N + 63) / 64 * 64; }
 
 size_t moment2_pairs_partial_bytes(int64_t N, const PairLayout &L, bool split)
 {
-    if (N <= 0 || N > (int64_t(1) << 29)) return 0;
+    // the copies' row coordinate has 31 bits, and split features have two rows for a sample
+    if (N <= 0 || N > (split ? int64_t(1) << 29 : (int64_t(1) << 31) - 64)) return 0;
     const M2TcPlan &q = split ? m2tc_plan_pairs<M2_SPLIT>(N, L) : m2tc_plan_pairs<M2_BF16>(N, L);
     return q.ok ? q.partial_bytes : 0;
 }

@@ -260,3 +260,11 @@ def test_the_binding_belongs_to_either_build_and_to_one_python_and_torch(tmp_pat
     monkeypatch.setattr(_build, "_binding_key", lambda: "another torch")
     _build._build_binding(False)
     assert made[2:] == ["g++"]
+
+
+def test_fourth_moment_in_bf16_takes_as_many_samples_as_its_copies_can_name():
+    import paper_2211_10482_b200 as st
+    size = lambda N: st.st_workspace_bytes(st.ST_OP_SYM_MOMENT4, N, 4, 0, 0, st.ST_FLAG_TC_BF16)
+    for N in (1 << 29, (1 << 29) + 1, (1 << 31) - 64):
+        assert size(N) > N * 10 * 2, N                           # ten pair features a sample
+    assert size((1 << 31) - 63) == 0
