@@ -16,11 +16,12 @@
 //
 // A run starts wherever the closed form says, so source and destination usually differ in their offset from a
 // 16-byte boundary.  copy_flat stores whole 16-byte units all the same and takes each from the two aligned units
-// that hold it (the second one is an L1 hit), shifted in registers.  Measured against copies in the widest unit that
+// that hold it (the second one is an L1 hit), shifted in registers, never past the end of the source array.  Measured against copies in the widest unit that
 // divides a row, each position of a symmetric fill by itself (pack + unpack): tet d = 60, rows of 33 floats, 72 -> 24 us;
 // tri d = 900, rows of 17 bf16, 125 -> 21 us; simplex4 d = 64 floats, 220 -> 32 us; tet d = 200 bf16, 27 -> 9 us.
 #include "st_common.cuh"
 #include "st_index.cuh"
+#include "copy_span.cuh"
 #include <type_traits>
 
 namespace st {
@@ -75,13 +76,13 @@ __device__ __forceinline__ uint32_t mul_word(uint32_t a, uint32_t b) { return __
 // times mul[0..n), fp32, which is offset from a 16-byte boundary as dst is.  The elements in front of the first whole
 // unit of dst and behind the last one are loaded ahead of the units, so that they cost no round trip of their own.
 template <int ES, bool MUL, int U>
-__device__ __forceinline__ void copy_flat(unsigned char *dst, const unsigned char *src, const unsigned char *mul, int n, int lane, int g)
+__device__ __forceinline__ void copy_flat(unsigned char *dst, const unsigned char *src, const unsigned char *mul, int n, int lane, int g,
+                                          const unsigned char *src_end)
 {
     typedef typename Elem<ES>::T E;
-    int head = (int)((0u - (unsigned)(uintptr_t)dst) & 15u);
-    if (head > n) head = n;
-    const int units = (n - head) >> 4;
-    const int ends = n - (units << 4);
+    const CopySpan span = copy_span((uintptr_t)dst, (uintptr_t)src, n, (uintptr_t)src_end);
+    const int head = span.head, units = span.units, ends = span.ends;
+    const unsigned off = span.off;
     auto end_at = [&](int e) { return e < head ? e : e + (units << 4); };
     auto end_load = [&](int e) {
         E v = *reinterpret_cast<const E *>(src + end_at(e));
@@ -91,7 +92,6 @@ __device__ __forceinline__ void copy_flat(unsigned char *dst, const unsigned cha
     const int e0 = lane * ES;
     E ev = E{};
     if (e0 < ends) ev = end_load(e0);
-    const unsigned off = (unsigned)(uintptr_t)(src + head) & 15u;
     const uint4 *in = reinterpret_cast<const uint4 *>(src + head - off);
     uint4 *out = reinterpret_cast<uint4 *>(dst + head);
     const uint4 *m = MUL ? reinterpret_cast<const uint4 *>(mul + head) : nullptr;
@@ -238,6 +238,7 @@ slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I 
     const I gid = (I)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> group_shift);
     const I ngroups = (I)(((int64_t)gridDim.x * blockDim.x) >> group_shift);
     const int64_t sb = a.d * a.row_bytes;                     // bytes per dense slice
+    const unsigned char *src_end = src + (PACK ? a.dense_rows : a.packed_rows) * a.row_bytes;
     for (I item = gid; item < nitems; item += ngroups) {
         I s = parts == 1 ? item : item / (I)parts, lo, hi, prow;
         const int64_t part = item - s * (I)parts;
@@ -261,13 +262,13 @@ slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I 
         const int64_t p0 = (int64_t)prow * a.row_bytes - d0;           // packed byte of its byte 0, were it in the run
         if (PACK) {
             if (BAND_ROW && d0 > u0) zero_flat<ES>(dst + p0 + u0, (int)((u1 < d0 ? u1 : d0) - u0), lane, g);
-            if (x1 > x0) copy_flat<ES, MUL, MUL ? COPY_UNITS / 2 : COPY_UNITS>(dst + p0 + x0, src + (int64_t)s * sb + x0 - shift, mul + p0 + x0, (int)(x1 - x0), lane, g);
+            if (x1 > x0) copy_flat<ES, MUL, MUL ? COPY_UNITS / 2 : COPY_UNITS>(dst + p0 + x0, src + (int64_t)s * sb + x0 - shift, mul + p0 + x0, (int)(x1 - x0), lane, g, src_end);
             if (BAND_ROW && u1 > d1) zero_flat<ES>(dst + p0 + (u0 > d1 ? u0 : d1), (int)(u1 - (u0 > d1 ? u0 : d1)), lane, g);
         } else {
             unsigned char *out = dst + (int64_t)s * sb;
             const int64_t z1 = u1 < c0 ? u1 : c0;               // zeros before the run
             if (z1 > u0) zero_flat<ES>(out + u0, (int)(z1 - u0), lane, g);
-            if (x1 > x0) copy_flat<ES, false, COPY_UNITS>(out + x0, src + p0 + x0, nullptr, (int)(x1 - x0), lane, g);
+            if (x1 > x0) copy_flat<ES, false, COPY_UNITS>(out + x0, src + p0 + x0, nullptr, (int)(x1 - x0), lane, g, src_end);
             const int64_t z2 = u0 > c1 ? u0 : c1;               // zeros after the run
             if (u1 > z2) zero_flat<ES>(out + z2, (int)(u1 - z2), lane, g);
         }
@@ -321,6 +322,7 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
     pdl_wait();
     pdl_trigger();
     const int lane = (int)(threadIdx.x & 31);
+    const unsigned char *src_end = src + packed_rows * row_bytes;
     const I nitems = nslices * (I)parts, nwarps = (I)gridDim.x * (I)(blockDim.x / 32);
     for (I item = (I)blockIdx.x * (I)(blockDim.x / 32) + (I)(threadIdx.x / 32); item < nitems; item += nwarps) {
         const I s = parts == 1 ? item : item / (I)parts;
@@ -333,7 +335,7 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
         if (xr < x1) {
             const I p = sym_run_row<KIND, I>(d, a, b, c, xr);
             if (ST_BOUNDS_OK(p, packed_rows, 1) && ST_BOUNDS_OK((int64_t)p + (x1 - xr) - 1, packed_rows, 1))
-                copy_flat<ES, false, ES >= 8 ? 2 : 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32);
+                copy_flat<ES, false, ES >= 8 ? 2 : 1>(out + (int64_t)xr * row_bytes, src + (int64_t)p * row_bytes, nullptr, (int)(x1 - xr) * row_bytes, lane, 32, src_end);
         }
         const I xe = x1 < top ? x1 : top;
         const int words = row_bytes / ES;
@@ -363,7 +365,7 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
                 if (!ST_BOUNDS_OK(p, packed_rows, 1)) continue;
                 unsigned char *o = out + (int64_t)x * row_bytes;
                 const unsigned char *from = src + (int64_t)p * row_bytes;
-                copy_flat<ES, false, 1>(o, from, nullptr, row_bytes, lane & (g - 1), g);
+                copy_flat<ES, false, 1>(o, from, nullptr, row_bytes, lane & (g - 1), g, src_end);
             }
         }
     }
@@ -380,6 +382,7 @@ sym_row_kernel(const unsigned char *src, unsigned char *dst, I d, I nitems, I se
     pdl_wait();
     pdl_trigger();
     const int lane = (int)(threadIdx.x & 31);
+    const unsigned char *src_end = src + packed_rows * row_bytes;
     const I nwarps = (I)gridDim.x * (I)(blockDim.x / 32);
     for (I item = (I)blockIdx.x * (I)(blockDim.x / 32) + (I)(threadIdx.x / 32); item < nitems; item += nwarps) {
         const I row = segs == 1 ? item : item / segs;
@@ -390,7 +393,7 @@ sym_row_kernel(const unsigned char *src, unsigned char *dst, I d, I nitems, I se
         const I p = x < top ? sym_row<KIND, I>(d, a, b, c, x) : sym_run_row<KIND, I>(d, a, b, c, x);
         if (!ST_BOUNDS_OK(p, packed_rows, 1)) continue;
         const int n = row_bytes - off < ROW_SEG ? (int)(row_bytes - off) : ROW_SEG;
-        copy_flat<ES, false, U>(dst + (int64_t)row * row_bytes + off, src + (int64_t)p * row_bytes + off, nullptr, n, lane, 32);
+        copy_flat<ES, false, U>(dst + (int64_t)row * row_bytes + off, src + (int64_t)p * row_bytes + off, nullptr, n, lane, 32, src_end);
     }
 }
 

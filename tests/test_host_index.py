@@ -268,3 +268,34 @@ def test_fourth_moment_in_bf16_takes_as_many_samples_as_its_copies_can_name():
     for N in (1 << 29, (1 << 29) + 1, (1 << 31) - 64):
         assert size(N) > N * 10 * 2, N                           # ten pair features a sample
     assert size((1 << 31) - 63) == 0
+
+
+def test_copies_read_no_byte_behind_the_source_array():
+    src = os.path.join(tempfile.mkdtemp(prefix="st_span_"), "span.cpp")
+    with open(src, "w") as f:
+        f.write("""#include "copy_span.cuh"
+// runs [x, x + n) of an array of `size` bytes on a 16-byte boundary, to every offset: what is read stays inside, every byte is
+// copied once, and at most the last unit goes singly
+extern "C" long long bad(int size, int es)
+{
+    long long bad = 0;
+    const uintptr_t base = 4096, end = base + size;
+    for (int to = 0; to < 16; to += es)
+        for (int x = 0; x < size; x += es)
+            for (int n = es; x + n <= size; n += es) {
+                const st::CopySpan c = st::copy_span(8192 + to, base + x, n, end);
+                const uintptr_t first = base + x + c.head, last = first - c.off + 16 * (uintptr_t)(c.units + (c.off ? 1 : 0));
+                bad += c.units > 0 && (last > (end + (c.off ? 0 : 15)) || first - c.off < base);
+                bad += c.units > 0 && !c.off && first + 16 * (uintptr_t)c.units > end;
+                bad += c.units > 0 && (8192 + to + c.head) % 16 != 0;
+                bad += c.units < 0 || c.head + 16 * c.units > n || c.ends != n - 16 * c.units || c.ends % es || c.ends >= 48;
+            }
+    return bad;
+}
+""")
+    subprocess.check_call(["g++", "-O2", "-shared", "-fPIC", "-std=c++17", "-I", CSRC, src, "-o", src + ".so"])
+    L = ctypes.CDLL(src + ".so")
+    L.bad.restype = ctypes.c_longlong
+    for es in (2, 4, 8):
+        for size in range(es, 160, es):
+            assert L.bad(size, es) == 0, (size, es)
