@@ -1359,3 +1359,28 @@ def test_moment2_f32_few_samples_of_many_features(st, N, d):
     i, j = np.triu_indices(d)
     X64 = X.astype(np.float64)
     assert np.max(np.abs(got - (X64.T @ X64)[i, j]) / (np.abs(X64).T @ np.abs(X64))[i, j]) <= TOL_F32
+
+
+# copies whose indices leave 32 bits: slices of more than 20000 positions, symmetric fill past 32768, small otherwise
+def test_copies_with_64_bit_indices(st):
+    lay = st.Layout(st.ST_BAND, 20011, 1, kl=1, ku=2)
+    P = torch.arange(st.st_packed_elems(lay), device="cuda").to(torch.int16)
+    D = st.st_unpack(P, lay).view(20011, 20011)
+    for o in range(-1, 3):
+        i = torch.arange(max(0, -o), 20011 - max(0, o), device="cuda")
+        assert torch.equal(D[i, i + o], P[4 * i + o + 1])
+    assert int(torch.count_nonzero(D)) <= P.numel()
+    again = st.st_pack(D, lay)
+    inside = torch.ones_like(P, dtype=torch.bool)
+    inside[0] = inside[-1] = inside[-2] = inside[-5] = False                 # slots outside the matrix: zeros
+    assert torch.equal(again[inside], P[inside]) and int(torch.count_nonzero(again[~inside])) == 0
+    del D, again
+    d = 32771
+    lay = st.Layout(st.ST_TRI_UPPER, d)
+    P = torch.arange(st.st_packed_elems(lay), device="cuda").to(torch.int16)
+    D = st.st_unpack(P, lay, st.ST_FILL_SYMMETRIC).view(d, d)
+    i = torch.tensor([0, 1, 16000, 32000, d - 1], device="cuda")
+    j = torch.arange(d, device="cuda")
+    lo, hi = torch.minimum(i[:, None], j), torch.maximum(i[:, None], j)
+    want = P[lo * (2 * d - lo + 1) // 2 + hi - lo]
+    assert torch.equal(D[i], want) and torch.equal(D[:, i].T, want)
