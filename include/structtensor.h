@@ -183,7 +183,8 @@ st_status st_sym_moment3(const float *X, int64_t N, int64_t d, int64_t ldx,
  * the fp32 paths -- for d <= 90 every fp32 pair product is stored as hi + lo bf16 parts and the tensor-core
  * triangular tile GEMM adds three partial products (hi hi + hi lo + lo hi) with fp32 accumulation; for larger d
  * an fp32 P and fp32 FMA arithmetic.  ST_FLAG_TC_BF16 stores P rounded to bf16 and runs one pass of the same
- * GEMM (5e-3 tolerance for N >= 1000). */
+ * GEMM (5e-3 tolerance for N >= 1000).  Which pairs of a 4-tuple are multiplied is the library's choice: the product of any two
+ * features of a sample should lie in fp32's range. */
 st_status st_sym_moment4(const float *X, int64_t N, int64_t d, int64_t ldx,
                          float *out_packed, void *ws, size_t ws_bytes, unsigned flags,
                          void *stream);

@@ -83,12 +83,6 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *m)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
 }
 
-// Brings a box of a tensor map into L2.
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *m, int x, int y)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y) : "memory");
-}
-
 // 2-D tiled load global -> shared, completion counted in bytes on `bar`.  x is the innermost
 // coordinate (in elements; x * element size must be a multiple of 16 bytes).
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *m, uint64_t *bar, int x, int y)

@@ -8,7 +8,8 @@
 // 13 mantissa bits are ignored).  U is rounded to TF32, transposed once per block into the
 // same swizzled K-major form and stays in shared memory.  The 128 x R fp32 accumulator lives
 // in tensor memory, double buffered so that the epilogue of one tile overlaps the MMAs of the
-// next.  Warp roles: warp 0 TMA producer, warp 1 MMA issuer / TMEM owner, warps 2..5 epilogue.
+// next.  Warp roles: warp 0 TMA producer, warp 1 MMA issuer / TMEM owner, warps 2..9 epilogue, two groups
+// of four on alternate tiles.
 #include "tc_common.cuh"
 #include "st_index.cuh"
 #include "fibre_epilogue.cuh"
@@ -244,10 +245,9 @@ static TtmTcPlan ttm_tc_plan(int64_t K, int64_t R)
     p.ok = false;
     if (K <= 0 || R <= 0 || K % 4 != 0 || R % 16 != 0 || R > 256 || K > (1 << 20)) return p;
     p.kchunks = (int)((K + KC - 1) / KC);
-    // two accumulators of R columns; the epilogue reads them with 32-column loads, so the second one
-    // (which starts at column R) needs R rounded up to 32 columns behind it: 64 columns for R = 16
+    // two accumulators of R columns, which the epilogue reads 16 columns at a time; an allocation is a power of two, at least 32
     uint32_t cols = 32;
-    while (cols < (uint32_t)R + ((uint32_t)R + 31u) / 32u * 32u) cols *= 2;
+    while (cols < 2 * (uint32_t)R) cols *= 2;
     p.tmem_cols = cols;
     const size_t u_bytes = (size_t)p.kchunks * R * 128;
     const size_t fixed = 1024 + u_bytes + 512;
