@@ -116,7 +116,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     constexpr int KROWS = S::KROWS, BOXC = S::BOXC, BOX_BYTES = S::BOX_BYTES, NBOX = S::NBOX;
     constexpr int PARTS = S::PARTS;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char *smem = align_smem(smem_raw);
     const uint32_t part_bytes = (uint32_t)((a.nb + a.na) * BOX_BYTES), stage_bytes = PARTS * part_bytes;
     // M2_CONV: a box of fp32 becomes its hi and its lo box in place; else all hi boxes, then all lo boxes
     constexpr int BOX_PITCH = MODE == M2_CONV ? 2 * BOX_BYTES : BOX_BYTES;

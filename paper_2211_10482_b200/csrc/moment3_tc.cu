@@ -97,7 +97,7 @@ moment3_tc_kernel(const __grid_constant__ Args a)
     constexpr int KS = BF16 ? 64 : 32;           // samples per slice
     constexpr int NA = BF16 ? 8 : 10;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char *smem = align_smem(smem_raw);
     unsigned char *a_stage0 = smem;
     const int NB = a.nb, x_pitch = a.dcols + 1;
     const uint32_t B_STAGE_BYTES = (uint32_t)a.dcols * ROW_BYTES, X_STAGE_FLOATS = (uint32_t)(KS * x_pitch);
