@@ -4,7 +4,8 @@
 // Two main kernels, each followed by a sum of its partial results in a fixed order (deterministic result):
 // the register-tile kernel of moment2_small.cu for few features, and moment2_gemm_kernel below, which cuts the
 // upper triangle into 128x128 tiles and skips the 64x64 quadrants that lie below the diagonal or past d.
-// Either takes any d and any row pitch.
+// Either takes any d and any row pitch.  Many samples of more features, in rows that start on 16-byte boundaries, go to
+// the tensor cores instead, without loss of accuracy (moment2_exact.cuh).
 #include "st_common.cuh"
 #include "st_index.cuh"
 #include <type_traits>
@@ -20,6 +21,9 @@ size_t moment2_tf32_tc_workspace(int64_t N, int64_t d, unsigned flags);
 st_status moment2_split_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
                            unsigned flags, cudaStream_t stream);
 size_t moment2_split_tc_workspace(int64_t N, int64_t d, unsigned flags);
+st_status moment2_exact_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
+                           unsigned flags, cudaStream_t stream);
+size_t moment2_exact_tc_workspace(int64_t N, int64_t d, unsigned flags);
 int64_t moment2_small_slots(int64_t d, unsigned flags);
 int64_t moment2_small_items(int64_t d, unsigned flags);
 size_t moment2_small_workspace(int64_t N, int64_t d, unsigned flags);
@@ -366,10 +370,23 @@ static bool moment2_use_small(int64_t N, int64_t d, unsigned flags)
     return (double)slots / 0.60 <= (double)(moment2_gemm_quads(d, dense) * 4096) / 0.75;
 }
 
+// Tensor cores with the exact parts of x (moment2_exact.cuh), no less accurate: from where they are faster than the FMA kernels.
+// FMA / tensor cores, us: [12000,128] 17.1 / 17.3, [16384,128] 20.4 / 19.1, [200000,128] 106 / 92, [4096,192] 12.6 / 15.8,
+// [6000,192] 18.0 / 16.5, [4096,200] 20.6 / 15.9, [2000,260] 14.6 / 14.7, [3000,260] 22.1 / 15.5, [1000,512] 15.0 / 16.8,
+// [1500,512] 23.3 / 17.0, [65536,512] 370 / 122, [300,768] 14.6 / 16.5, [600,768] 22.6 / 17.3, [4096,2048] 374 / 104.  Up to 120
+// features the register tiles are the better ones ([200000,120] 78 / 92), and those of 129 to 136 are no worse ([65536,136] 43 / 43).
+static bool moment2_use_exact(int64_t N, int64_t d)
+{
+    if (d <= 120 || (d > 128 && d <= 136) || d > 4096 || N > (int64_t(1) << 31) - 64) return false;
+    const double values = (double)N * (double)d;
+    return values * (double)d >= 2.7e8 || (d > 136 && values >= 8e5);
+}
+
 static st_status moment2_f32(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws,
                              size_t ws_bytes, unsigned flags, cudaStream_t stream)
 {
     if (d > 32768) return ST_ERR_UNSUPPORTED;
+    if (ldx % 4 == 0 && moment2_use_exact(N, d)) return moment2_exact_tc(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
     return moment2_use_small(N, d, flags) ? moment2_small(X, N, d, ldx, out, ws, ws_bytes, flags, stream)
                                        : moment2_gemm(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
 }
@@ -383,8 +400,10 @@ size_t moment2_workspace(int64_t N, int64_t d, int xdt, unsigned flags)
     if (xdt == ST_F32 && (flags & ST_FLAG_TC_TF32)) return moment2_tf32_tc_workspace(N, d, flags & ~ST_FLAG_TC_TF32);
     if (xdt == ST_F32 && (flags & ST_FLAG_TC_SPLIT)) return moment2_split_tc_workspace(N, d, flags & ~ST_FLAG_TC_SPLIT);
     if (xdt != ST_F32 || d > 32768) return 0;
-    return moment2_use_small(N, d, flags) ? moment2_small_workspace(N, d, flags)
-                                       : kWsHeaderBytes + mg_partial_bytes(moment2_gemm_plan(N, d, flags));
+    const size_t fma = moment2_use_small(N, d, flags) ? moment2_small_workspace(N, d, flags)
+                                                      : kWsHeaderBytes + mg_partial_bytes(moment2_gemm_plan(N, d, flags));
+    const size_t exact = moment2_use_exact(N, d) ? moment2_exact_tc_workspace(N, d, flags) : 0;
+    return exact > fma ? exact : fma;
 }
 
 }  // namespace st

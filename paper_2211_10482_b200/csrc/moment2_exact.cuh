@@ -1,0 +1,494 @@
+// Second moment of fp32 samples on the tensor cores, no less accurate than a chain of fp32 FMAs (M2_EXACT of moment2_tc.cu,
+// which includes this file; tiles, clusters and the sum of the partial tiles are those of that file).
+//
+// x = hi + mid + lo in bfloat16, exactly: 24 bits are three times eight.  Of the nine products of the parts the three that lie
+// 2^-27 and more below the result are left out, the other six go through the tensor core.  It truncates what it adds to the
+// grid of the larger operand, so
+//   - the products of 32 samples, the small ones first, are added in tensor memory, and every further addition is an fp32 one
+//     in registers: an epilogue thread holds the sums of half a row of the tile, 128 of them;
+//   - the sums of squares, whose terms all have one sign, are added by the converting warps with fp32 FMAs; truncation would
+//     leave them half a unit in the last place too small (measured -5.8e-8 relative; other sums of both signs have no such drift).
+// Against 64 bits the 2-norm of the error is 4.5e-8 to 9e-8 of the result's where fp32 FMAs are 5.5e-8 to 5e-7 off.
+// What bounds it: per 32 samples of a full tile 1536 cycles of MMA, 1660 of shared memory (copies 256, loads 256 and stores 384 of
+// the converting warps, operands 768), and in the converting warps, which take the 2500 cycles that are measured, about 1400
+// of the issue slots of a scheduler, whose loads wait behind the tensor core's.  [65536,512] 370 us with fp32 FMAs, here 122;
+// [65536,256] 112 and 44; [4096,2048] 374 and 104.  Tried: four converting warps (139 at [65536,512]), two groups of four on
+// alternate stages (152), polls by one lane (148), the mixed-precision subtraction (134 instead of 131).
+// Values whose parts are not all bfloat16 numbers (infinities, NaN, |x| > 2^127.99, columns of |x| < 2^-100) give the samples of
+// the cluster that meets them to plain fp32 FMAs.
+#pragma once
+#include <type_traits>
+
+namespace st {
+
+namespace m2tc {
+// Warps 0 .. EX_CONV_WARPS - 1 convert, then copies, MMA, two idle ones, eight of the epilogue.
+constexpr int EX_CONV_WARPS = 8, EX_COPY_WARP = EX_CONV_WARPS, EX_MMA_WARP = EX_CONV_WARPS + 1, EX_EPI_WARP = EX_CONV_WARPS + 4;
+constexpr int EX_EPI_THREADS = 256;
+constexpr int EX_THREADS = 32 * EX_EPI_WARP + EX_EPI_THREADS;
+// Registers of a thread at launch, and of the warpgroups afterwards: an epilogue thread needs 128 for its sums alone.
+constexpr int EX_REGS = 65536 / EX_THREADS / 8 * 8, EX_REGS_MAIN = 32, EX_REGS_EPI = 168, EX_REGS_CONV = 56;
+static_assert(EX_CONV_WARPS / 4 * EX_REGS_CONV + EX_REGS_MAIN + 2 * EX_REGS_EPI <= EX_THREADS / 128 * EX_REGS,
+              "the warpgroups share what the block was launched with");
+static_assert(EX_REGS_CONV <= EX_REGS && EX_REGS_MAIN <= EX_REGS && EX_REGS_EPI >= EX_REGS, "setmaxnreg.dec must not add, .inc not take");
+// Stages of operands (3 boxes a unit) and of fp32 (2) in flight for tiles of 1 .. 4 boxes a part
+constexpr int EX_MAX_STAGES = 8, EX_BOXES = 52;
+__device__ constexpr int EX_STAGES[5] = {0, 8, 5, 3, 3}, EX_RAW_STAGES[5] = {0, 8, 5, 4, 2};
+constexpr int EX_LEVEL = 256;                          // phases that are added before the sum goes to the partial tile
+constexpr int EX_SQUARES = 2 * EX_CONV_WARPS;          // parts of a column's sum of squares
+constexpr uint32_t EX_TINY = 0x0D80;                   // 2^-100 in bfloat16
+constexpr int EX_AGAIN = 64;                           // samples at a time of the FMA path
+constexpr size_t EX_SMEM = 1024 + (size_t)EX_BOXES * 4096 + 512 + (size_t)EX_SQUARES * HALF * sizeof(float);
+static_assert((size_t)EX_AGAIN * (HALF + BN) * sizeof(float) <= (size_t)EX_BOXES * 4096, "the FMA path reuses the stages");
+}  // namespace m2tc
+
+template <int REGS> __device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS)); }
+template <int REGS> __device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS)); }
+
+// The halves' minimum, as signed numbers.
+__device__ __forceinline__ uint32_t ex_min_s16x2(uint32_t a, uint32_t b)
+{
+    asm("min.s16x2 %0, %0, %1;" : "+r"(a) : "r"(b));
+    return a;
+}
+// x += y and x -= y for two fp32 numbers at a time (y: their bits).
+__device__ __forceinline__ uint64_t ex_pack2(uint32_t lo, uint32_t hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ __forceinline__ void ex_add2(float &x0, float &x1, uint32_t y0, uint32_t y1)
+{
+    uint64_t x = ex_pack2(__float_as_uint(x0), __float_as_uint(x1));
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(ex_pack2(y0, y1)));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
+}
+__device__ __forceinline__ void ex_sub2(float &x0, float &x1, uint32_t y0, uint32_t y1)
+{
+    uint64_t x = ex_pack2(__float_as_uint(x0), __float_as_uint(x1));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(x) : "l"(ex_pack2(y0, y1)), "l"(0xBF800000BF800000ull));      // x + y (-1)
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
+}
+
+// Barrier of the epilogue warps of a block; true if any of them says so.
+__device__ __forceinline__ bool ex_any(bool x)
+{
+    uint32_t r = x ? 1u : 0u;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %0, 0;\n\tbar.red.or.pred q, 1, %1, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "+r"(r) : "n"(m2tc::EX_EPI_THREADS) : "memory");
+    return r != 0;
+}
+
+__global__ void __launch_bounds__(m2tc::EX_THREADS, 1)
+moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ m2tc::Args a)
+{
+    using namespace m2tc;
+    using namespace tc;
+    using S = Shape<M2_EXACT>;
+    constexpr int KROWS = S::KROWS, BOX_BYTES = S::BOX_BYTES;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = align_smem(smem_raw);
+    uint64_t *bars = (uint64_t *)(smem + EX_BOXES * BOX_BYTES);
+    uint64_t *full = bars, *empty = full + EX_MAX_STAGES, *raw_full = empty + EX_MAX_STAGES, *raw_empty = raw_full + EX_MAX_STAGES,
+             *acc_full = raw_empty + EX_MAX_STAGES, *acc_empty = acc_full + 2;
+    uint32_t *tmem_slot = (uint32_t *)(acc_empty + 2);
+    volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
+    unsigned *tiny_seen = (unsigned *)(tmem_slot + 2);
+    float *squares = reinterpret_cast<float *>(smem + EX_BOXES * BOX_BYTES + 512);       // [EX_SQUARES][HALF]: of this block's rows
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();            // 0 = leader
+    const int cluster = blockIdx.x >> 1;
+    const int tile = m2tc_tile_of(a.tab, cluster), split = cluster - a.tab.first[tile];
+    const int nsplit = a.tab.first[tile + 1] - a.tab.first[tile];
+    const int row = 8 * a.tab.row[tile], rows = a.tab.rows[tile], col = 8 * a.tab.col[tile], width = 32 * a.tab.width[tile];
+    const bool diag = a.tab.diag[tile] != 0;
+    const bool alias = diag && width == BN;             // A columns == B columns in both blocks: one copy serves both
+    const bool lead = diag && rows <= HALF;             // all rows in the first block, whose A holds its half of B as well
+    // A stage of operands: all hi boxes (64 columns x 32 samples), all mid boxes, all lo boxes; a stage as it was copied: boxes of
+    // 32 columns x 32 samples of fp32, two for each of those.  Boxes of B and of A, the most that either block has:
+    const int tb = ((lead && rows > width / 2 ? rows : width / 2) + 63) / 64, ta = alias || lead ? 0 : rows >= HALF ? 2 : (rows + 63) / 64;
+    const uint32_t part_bytes = (uint32_t)((tb + ta) * BOX_BYTES), stage_bytes = 3 * part_bytes, raw_bytes = 2 * part_bytes;
+    const int stages = EX_STAGES[tb + ta], raw_stages = EX_RAW_STAGES[tb + ta];
+    // an MMA reads 128 columns of A per block, of which fewer may have been written: behind the operands it meets the fp32 boxes
+    unsigned char *raw0 = smem + (size_t)stages * stage_bytes;
+    const int chunks_per_split = (a.chunks_total + nsplit - 1) / nsplit;
+    const int c_begin = split * chunks_per_split;
+    int c_end = c_begin + chunks_per_split;
+    if (c_end > a.chunks_total) c_end = a.chunks_total;
+    const int nchunks = c_end > c_begin ? c_end - c_begin : 0;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < stages; ++s) {
+            mbar_init(&full[s], 2 * EX_CONV_WARPS);     // the converting warps of both blocks (leader's copy is used)
+            mbar_init(&empty[s], 1);                    // one commit per use, delivered to both blocks
+        }
+        for (int s = 0; s < raw_stages; ++s) {
+            mbar_init(&raw_full[s], 1);
+            mbar_init(&raw_empty[s], EX_CONV_WARPS);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], 16);               // eight epilogue warps in each of the two blocks (leader's copy is used)
+        }
+        *abort_flag = 0;
+        *tiny_seen = 0;
+        fence_barrier_init();
+    }
+    if (warp == EX_MMA_WARP) {
+        tmem_alloc_pair(tmem_slot, TMEM_COLS);
+        tmem_relinquish_pair();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                      // both blocks' barriers exist before anything is signalled across
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
+    pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.status[kWsStatusWord] = 0;
+        a.status[kWsDetailWord] = 0;
+    }
+
+    // boxes of 32 columns that block r copies: of B, and of A the ones that hold rows of the result
+    auto boxes_b = [&](int r) {
+        int n = lead && r == 0 && rows > width / 2 ? rows : width / 2;
+        if (n > a.d - col - r * (width / 2)) n = a.d - col - r * (width / 2);
+        return n <= 0 ? 0 : (n + 31) / 32;
+    };
+    auto boxes_a = [&](int r) {
+        const int n = rows - r * HALF;
+        return alias || lead || n <= 0 ? 0 : n >= HALF ? HALF / 32 : (n + 31) / 32;
+    };
+    const int col_a = row + (int)rank * HALF, col_b = col + (int)rank * (width / 2);
+    const int nb = boxes_b((int)rank), na = boxes_a((int)rank);
+
+    if (warp < EX_CONV_WARPS) {
+        // ---------------- converting warps (both blocks): the parts of x, each in the form that a copy of boxes of 64 columns x 32
+        // rows with the 128-byte swizzle leaves.  A warp takes RPW rows of all boxes of a stage.
+        regs_down<EX_REGS_CONV>();
+        constexpr int RPW = KROWS / EX_CONV_WARPS, H = RPW / 2;
+        const int c4 = (lane & 15) * 4, r0 = ((warp * RPW) & 7) + (lane >> 4);    // columns c4 .. c4+3 of 64, rows r0 + 2h of eight
+        const uint32_t bar0 = map_to_cta(smem_u32(full), 0);
+        // of row r0; row r0 + 2h: 256 h further, and bits 5 and 6, where the swizzle puts bits 1 and 2 of the row, exclusive-or h
+        const uint32_t from0 = (uint32_t)(warp * RPW / 8 * 1024 + (c4 >> 5) * BOX_BYTES + r0 * 128 + ((((c4 >> 2) & 7) ^ r0) << 4));
+        const uint32_t to0 = (uint32_t)(warp * RPW / 8 * 1024 + r0 * 128 + (((c4 >> 3) ^ r0) << 4) + (c4 & 4) * 2);
+        uint32_t least[2] = {0x7FFF7FFFu, 0x7FFF7FFFu};           // two smallest |hi| - 2^15 - 1 each; zeros come out as the largest
+        auto convert = [&](auto diag_tag) {
+            constexpr bool DIAG = decltype(diag_tag)::value;
+            const int own = na > 0 ? 1 : 0;                       // the side that holds the columns of this block's rows
+            float square[8] = {};
+            // Items of a stage: 64 columns of B, the other 64 of B, of A, of A, whichever this block has.  The loads of an item are
+            // issued before the one ahead of it is converted.
+            const int qb = (nb + 1) / 2, items = qb + (na + 1) / 2 > 0 ? qb + (na + 1) / 2 : 1;
+            int s = 0, rs = 0;
+            uint32_t parity = 1, rparity = 0;
+            float rest[H][4], next[H][4];
+            auto there = [&](int item) { return 2 * (item < qb ? item : item - qb) + (c4 >> 5) < (item < qb ? nb : na); };
+            auto load = [&](int item) {
+                const unsigned char *p = raw0 + rs * raw_bytes + 2 * (item < qb ? item : tb + item - qb) * BOX_BYTES;
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const float4 v = there(item) ? *reinterpret_cast<const float4 *>(p + (from0 ^ (h << 5)) + 256 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    next[h][0] = v.x; next[h][1] = v.y; next[h][2] = v.z; next[h][3] = v.w;
+                }
+            };
+            bool ok = nchunks > 0 && mbar_wait(&raw_full[0], 0, abort_flag, a.status, 5);
+            if (ok) load(0);
+            for (int c = 0; c < nchunks && ok; ++c) {
+                if (c >= stages && !mbar_wait(&empty[s], parity, abort_flag, a.status, 6)) break;
+                bool loaded = false;
+                for (int item = 0; item < items; ++item) {
+#pragma unroll
+                    for (int h = 0; h < H; ++h)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) rest[h][e] = next[h][e];
+                    if (item + 1 < items) {
+                        load(item + 1);
+                    } else {
+                        __syncwarp();                             // all lanes have the last values of the stage
+                        if (lane == 0) mbar_arrive(&raw_empty[rs]);
+                        if (++rs == raw_stages) { rs = 0; rparity ^= 1u; }
+                        if (c + 1 < nchunks && __all_sync(0xFFFFFFFFu, mbar_try_wait(&raw_full[rs], rparity))) {
+                            load(0);
+                            loaded = true;
+                        }
+                    }
+                    const bool store = there(item);
+                    unsigned char *w = smem + s * stage_bytes + (item < qb ? item : tb + item - qb) * BOX_BYTES;
+                    if (DIAG && (item < qb) == (own == 0)) {
+                        const bool upper = (item < qb ? item : item - qb) != 0;
+#pragma unroll
+                        for (int h = 0; h < H; ++h)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                if (upper) square[4 + e] = fmaf(rest[h][e], rest[h][e], square[4 + e]);
+                                else square[e] = fmaf(rest[h][e], rest[h][e], square[e]);
+                            }
+                    }
+                    // all values of the item step by step: one after the other they would be a chain of seven results each
+#pragma unroll
+                    for (int part = 0; part < 3; ++part) {
+                        uint32_t b[H][2];
+#pragma unroll
+                        for (int h = 0; h < H; ++h)
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const __nv_bfloat162 r = __floats2bfloat162_rn(rest[h][2 * e], rest[h][2 * e + 1]);
+                                b[h][e] = *reinterpret_cast<const uint32_t *>(&r);
+                            }
+                        if (part == 0) {
+#pragma unroll
+                            for (int h = 0; h < H; ++h)
+#pragma unroll
+                                for (int e = 0; e < 2; ++e) least[e] = ex_min_s16x2(least[e], (b[h][e] & 0x7FFF7FFFu) + 0x7FFF7FFFu);
+                        }
+                        if (store) {
+#pragma unroll
+                            for (int h = 0; h < H; ++h)
+                                *reinterpret_cast<uint2 *>(w + part * part_bytes + (to0 ^ (h << 5)) + 256 * h) = make_uint2(b[h][0], b[h][1]);
+                        }
+                        if (part < 2) {
+#pragma unroll
+                            for (int h = 0; h < H; ++h)
+#pragma unroll
+                                for (int e = 0; e < 2; ++e) {
+                                    ex_sub2(rest[h][2 * e], rest[h][2 * e + 1], b[h][e] << 16, b[h][e] & 0xFFFF0000u);
+                                }
+                        }
+                    }
+                }
+                fence_proxy_async();          // generic writes, read by the tensor core
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster_smem(bar0 + (uint32_t)(s * sizeof(uint64_t)));
+                if (++s == stages) { s = 0; parity ^= 1u; }
+                if (c + 1 < nchunks && !loaded) {
+                    ok = mbar_wait(&raw_full[rs], rparity, abort_flag, a.status, 5);
+                    if (ok) load(0);
+                }
+            }
+            if (DIAG) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) squares[(warp * 2 + (lane >> 4)) * HALF + q * 64 + c4 + e] = square[4 * q + e];
+            }
+        };
+        if (diag) convert(std::integral_constant<bool, true>{});
+        else convert(std::integral_constant<bool, false>{});
+        least[0] = ex_min_s16x2(least[0], least[1]) ^ 0x80008000u;
+        if ((least[0] & 0xFFFFu) < EX_TINY - 1u || least[0] >> 16 < EX_TINY - 1u) atomicOr(tiny_seen, 1u);
+    } else if (warp < EX_EPI_WARP) {
+        regs_down<EX_REGS_MAIN>();
+        if (warp == EX_COPY_WARP && elect_one()) {
+            // ---------------- copies (both blocks): own boxes, fp32
+            prefetch_tmap(&tmap);
+            int s = 0;
+            uint32_t parity = 1;
+            for (int c = 0; c < nchunks; ++c) {
+                if (c >= raw_stages && !mbar_wait(&raw_empty[s], parity, abort_flag, a.status, 1)) break;
+                mbar_expect_tx(&raw_full[s], (uint32_t)((nb + na) * BOX_BYTES));
+                unsigned char *base = raw0 + s * raw_bytes;
+                const int y = (c_begin + c) * KROWS;
+                for (int b = 0; b < nb; ++b) tma_load_2d(base + b * BOX_BYTES, &tmap, &raw_full[s], col_b + b * 32, y);
+                for (int b = 0; b < na; ++b) tma_load_2d(base + (2 * tb + b) * BOX_BYTES, &tmap, &raw_full[s], col_a + b * 32, y);
+                if (++s == raw_stages) { s = 0; parity ^= 1u; }
+            }
+        } else if (warp == EX_MMA_WARP && rank == 0 && elect_one()) {
+            // ---------------- MMA issuer (leader only).  The small products first: only what follows the first hi^T hi is cut at the
+            // grid of the result.
+            const uint32_t idesc = make_idesc(1, 1, 1, BM, (uint32_t)width);
+            const uint32_t a_off = alias || lead ? 0u : (uint32_t)(tb * BOX_BYTES);
+            const uint32_t sb0 = smem_u32(smem);
+            const uint64_t adesc_base = make_smem_desc(sb0 + a_off, BOX_BYTES, 1024), bdesc_base = make_smem_desc(sb0, BOX_BYTES, 1024);
+            const uint64_t part = (uint64_t)(part_bytes >> 4);
+            int s = 0;
+            uint32_t parity = 0;
+            for (int c = 0; c < nchunks; ++c) {
+                const int buf = c & 1;
+                if (!mbar_wait<true>(&full[s], parity, abort_flag, a.status, 2)) break;
+                if (c >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((c >> 1) - 1) & 1), abort_flag, a.status, 4)) break;
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+                const uint64_t ad = adesc_base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
+                const uint64_t bd = bdesc_base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
+                constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};
+#pragma unroll
+                for (int p = 0; p < 6; ++p)
+#pragma unroll
+                    for (int k = 0; k < KROWS / S::KMMA; ++k) {
+                        constexpr int STEP = S::KMMA * 128 / 16;
+                        mma_bf16_pair(d_tmem, ad + PA[p] * part + (uint64_t)(k * STEP), bd + PB[p] * part + (uint64_t)(k * STEP), idesc,
+                                      p > 0 || k > 0 ? 1u : 0u);
+                    }
+                tc_commit_pair(&empty[s]);
+                tc_commit_pair(&acc_full[buf]);
+                if (++s == stages) { s = 0; parity ^= 1u; }
+            }
+        }
+        __syncwarp();
+    }
+    if (warp >= EX_EPI_WARP) {
+        // ---------------- epilogue (both blocks): a thread owns row row0 + lane of the tile and half of its columns, c_half ..
+        regs_up<EX_REGS_EPI>();
+        const int row0 = (int)rank * HALF + (warp & 3) * 32, half = width / 2, c_half = warp >= EX_EPI_WARP + 4 ? half : 0;
+        float *dst = a.partials + (size_t)blockIdx.x * HALF * BN + ((warp & 3) * 32 + lane) * 4;      // columns c .. c+3: + c HALF
+        // sixteen columns of the half: in the tile, and not wholly below the diagonal?
+        auto wanted = [&](int t) { return row0 < rows && 16 * t < half && !(diag && c_half + 16 * t + 15 < row0); };
+        float sum[128];
+#pragma unroll
+        for (int e = 0; e < 128; ++e) sum[e] = 0.f;
+        const uint32_t leader_acc_empty0 = map_to_cta(smem_u32(&acc_empty[0]), 0);
+        const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c_half;
+        auto store = [&](bool add) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                if (wanted(t)) {
+#pragma unroll
+                    for (int e = 16 * t; e < 16 * t + 16; e += 4) {
+                        float4 v = make_float4(sum[e], sum[e + 1], sum[e + 2], sum[e + 3]);
+                        float4 *p = reinterpret_cast<float4 *>(dst + (c_half + e) * HALF);
+                        if (add) {
+                            const float4 o = *p;
+                            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+                        }
+                        *p = v;
+                    }
+                }
+        };
+        int held = 0;
+        bool stored = false;
+        for (int c = 0; c < nchunks; ++c) {
+            const int buf = c & 1;
+            if (!mbar_wait(&acc_full[buf], (uint32_t)((c >> 1) & 1), abort_flag, a.status, 3)) break;
+            tc_fence_after();
+#pragma unroll
+            for (int t = 0; t < 8; t += 2)
+                if (wanted(t) || wanted(t + 1)) {
+                    uint32_t r[32];
+                    tmem_ld_32x32(taddr + (uint32_t)(buf * BN + 16 * t), r);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2) ex_add2(sum[16 * t + e], sum[16 * t + e + 1], r[e], r[e + 1]);
+                }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster_smem(leader_acc_empty0 + (uint32_t)(buf * sizeof(uint64_t)));
+            if (++held == EX_LEVEL) {
+                store(stored);
+                stored = true;
+                held = 0;
+#pragma unroll
+                for (int e = 0; e < 128; ++e) sum[e] = 0.f;
+            }
+        }
+        // every value of the pair's samples has been looked at when the converting warps have arrived here
+        __syncthreads();
+        cluster_sync_all();
+        uint32_t tiny[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+            asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(tiny[r]) : "r"(map_to_cta(smem_u32(tiny_seen), (uint32_t)r)));
+        const int i = row + row0 + lane, t = (int)threadIdx.x - 32 * EX_EPI_WARP;
+        const int64_t n0 = (int64_t)c_begin * KROWS, n1 = (int64_t)c_end * KROWS < a.N ? (int64_t)c_end * KROWS : a.N;
+        // infinities, NaN and what rounds to infinity in bfloat16 show in the sums: 0 times a number that is none
+        float zero = 0.f;
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+            if (wanted(g) && col + c_half + 16 * g < a.d) {       // columns from d on are zeros there
+#pragma unroll
+                for (int e = 16 * g; e < 16 * g + 16; ++e) zero = fmaf(sum[e], 0.f, zero);
+            }
+        bool again = zero != 0.f && row0 < rows && i < a.d;
+        if ((tiny[0] | tiny[1]) != 0) {
+            // tiny values matter in a column that has no others
+            float most_a = 0.f, most_b = 0.f;
+            const int ca = col_a + (t & (HALF - 1)), cb = col + t;
+#pragma unroll 8
+            for (int64_t n = n0; n < n1; ++n) {
+                if (ca < a.d && ca < row + rows) most_a = fmaxf(most_a, fabsf(a.X[n * a.ldx + ca]));
+                if (cb < a.d && t < width) most_b = fmaxf(most_b, fabsf(a.X[n * a.ldx + cb]));
+            }
+            again = again || (most_a > 0.f && most_a < 0x1p-100f) || (most_b > 0.f && most_b < 0x1p-100f);
+        }
+        again = ex_any(again);
+        if (again) {
+            // these samples once more, with fp32 FMAs
+#pragma unroll
+            for (int e = 0; e < 128; ++e) sum[e] = 0.f;
+            stored = false;
+            float *xa = reinterpret_cast<float *>(smem), *xb = xa + EX_AGAIN * HALF;
+            for (int64_t n = n0; n < n1; n += EX_AGAIN) {
+                const int count = n1 - n < EX_AGAIN ? (int)(n1 - n) : EX_AGAIN;
+                ex_any(false);                                    // the samples before these have been read
+                for (int k0 = 0; k0 < count; k0 += 8) {           // the loads of eight samples in front of their stores
+                    float va[8], vb[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float *x = a.X + (n + k0 + k) * a.ldx;
+                        const bool in = k0 + k < count;
+                        va[k] = in && t < HALF && col_a + t < a.d ? x[col_a + t] : 0.f;
+                        vb[k] = in && t < width && col + t < a.d ? x[col + t] : 0.f;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        if (t < HALF) xa[(k0 + k) * HALF + t] = va[k];
+                        xb[(k0 + k) * BN + t] = vb[k];
+                    }
+                }
+                ex_any(false);
+#pragma unroll 2
+                for (int k = 0; k < count; ++k) {
+                    const float xi = xa[k * HALF + (warp & 3) * 32 + lane];
+                    const float4 *xj = reinterpret_cast<const float4 *>(xb + k * BN + c_half);
+#pragma unroll
+                    for (int e = 0; e < 128; e += 4)
+                        if (e < half) {
+                            const float4 v = xj[e / 4];
+                            sum[e] = fmaf(xi, v.x, sum[e]);
+                            sum[e + 1] = fmaf(xi, v.y, sum[e + 1]);
+                            sum[e + 2] = fmaf(xi, v.z, sum[e + 2]);
+                            sum[e + 3] = fmaf(xi, v.w, sum[e + 3]);
+                        }
+                }
+            }
+        }
+        store(stored);
+        // the sums of squares take their places on the diagonal
+        const int o = i - row;
+        if (!again && diag && row0 < rows && i < a.d && o >= c_half && o < c_half + half) {
+            float total = 0.f;
+#pragma unroll
+            for (int p = 0; p < EX_SQUARES; ++p) total += squares[p * HALF + (warp & 3) * 32 + lane];
+            dst[(o & ~3) * HALF + (o & 3)] = total;
+        }
+    } else {
+        __syncwarp();
+        __syncthreads();
+        cluster_sync_all();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                      // no block leaves while its peer may still read its flag
+    if (warp == EX_MMA_WARP) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, TMEM_COLS);
+    }
+}
+
+// The warpgroups of moment2_exact_kernel pass registers among them: what they end with is what the block must start with, or
+// one of them would wait for good.
+inline bool m2tc_exact_fits()
+{
+    static const int regs = [] {
+        cudaFuncAttributes f;
+        if (cudaFuncGetAttributes(&f, moment2_exact_kernel) == cudaSuccess) return f.numRegs;
+        (void)cudaGetLastError();
+        return -1;
+    }();
+    return regs >= 0 && (regs + 7) / 8 * 8 >= m2tc::EX_REGS;
+}
+
+}  // namespace st

@@ -1,9 +1,10 @@
 // st_sym_moment2, tensor-core paths: out[p(i,j)] = sum_n X[n,i] X[n,j], fp32 accumulation (Section 3, M1; the outer
-// product summed over samples is a symmetric rank-N update, i.e. a triangular tile GEMM X^T X).  Four forms of X:
+// product summed over samples is a symmetric rank-N update, i.e. a triangular tile GEMM X^T X).  Five forms of X:
 //   M2_BF16   bfloat16
 //   M2_TF32   fp32, of which the tensor core reads the upper 19 bits
 //   M2_CONV   fp32, in the kernel x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi
 //   M2_SPLIT  the same products of hi and lo that lie in memory (the pair features of moment4.cu)
+//   M2_EXACT  fp32, in the kernel of moment2_exact.cuh x = hi + mid + lo, no less accurate than fp32 FMAs
 //
 // A cluster of two blocks owns an output tile of 256 rows (i) x up to 256 columns (j) for a range of the samples.
 // Only tiles that contain an entry with i <= j are launched, and a tile of the last column is as wide as the columns
@@ -50,7 +51,7 @@
 
 namespace st {
 
-enum { M2_BF16 = 0, M2_TF32 = 1, M2_SPLIT = 2, M2_CONV = 3 };
+enum { M2_BF16 = 0, M2_TF32 = 1, M2_SPLIT = 2, M2_CONV = 3, M2_EXACT = 4 };
 
 namespace m2tc {
 constexpr int BM = 256, BN = 256;               // tile of the pair
@@ -66,7 +67,7 @@ constexpr int MAX_TILES = 160;
 constexpr uint32_t TMEM_COLS = 512;
 template <int MODE> struct Shape {
     static constexpr int ELEM = MODE == M2_TF32 ? 4 : 2;
-    static constexpr int PARTS = MODE >= M2_SPLIT ? 2 : 1;  // hi and lo
+    static constexpr int PARTS = MODE == M2_EXACT ? 3 : MODE >= M2_SPLIT ? 2 : 1;   // hi (, mid) and lo
     static constexpr int KROWS = MODE == M2_BF16 ? 64 : 32; // sample rows per stage
     static constexpr int KMMA = MODE == M2_TF32 ? 8 : 16;   // sample rows per MMA
     static constexpr int BOXC = 128 / ELEM;                 // columns per TMA box (128 bytes)
@@ -90,6 +91,8 @@ struct Args {
     int d;                                             // columns of X
     int chunks_total, stages, nb, na;                  // nb, na: boxes of B and A per part in a stage
     int lo_row0;                                       // M2_SPLIT: first row of the lo part
+    const float *X;                                    // M2_EXACT: what the copies read
+    int64_t N, ldx;
     TileTable tab;
 };
 }  // namespace m2tc
@@ -105,6 +108,10 @@ __device__ __forceinline__ int m2tc_tile_of(const m2tc::TileTable &t, int cluste
     }
     return lo;
 }
+
+}  // namespace st
+#include "moment2_exact.cuh"
+namespace st {
 
 template <int MODE>
 __global__ void __launch_bounds__(MODE == M2_CONV ? m2tc::THREADS + m2tc::CONV_THREADS : m2tc::THREADS, 1)
@@ -471,6 +478,13 @@ struct M2TcPlan {
 // Time per stage, a full tile = 1: the 256 columns of A are loaded whatever the width (the MMA alone would be 43 cycles
 // at 64 columns against 128; with 0.35 in place of 0.7 [400000,304] bf16 ran 127 us instead of 111).
 static double m2tc_cost(int width) { return 0.7 + 0.3 * width / m2tc::BN; }
+// M2_EXACT, where a stage takes as long as its values are converted: us per 32 samples 1.36, on the diagonal 1.2, 1.27 at 32
+// columns off it, 1.0, 0.73 and 0.65 where all columns are 128, 64 or four.
+static double m2tc_exact_cost(int rows, int width, bool diag)
+{
+    if (!diag) return 0.92 + 0.08 * width / m2tc::BN;
+    return rows > m2tc::HALF ? 0.88 : 0.47 + 0.26 * rows / m2tc::HALF;
+}
 
 // Tiles of a plan while it is made.
 struct M2TcTiles {
@@ -488,7 +502,7 @@ struct M2TcTiles {
         p->tab.col[n] = (unsigned short)(col / 8);
         p->tab.width[n] = (unsigned char)(width / 32);
         p->tab.diag[n] = diag ? 1 : 0;
-        cost[n] = m2tc_cost(width);
+        cost[n] = MODE == M2_EXACT ? m2tc_exact_cost(rows, width, diag) : m2tc_cost(width);
         const bool lead = diag && rows <= HALF;
         const int cols_b = lead && rows > width / 2 ? rows : width / 2, nb = (cols_b + S::BOXC - 1) / S::BOXC;
         if (nb > p->nb) p->nb = nb;
@@ -520,7 +534,7 @@ static void m2tc_finish(M2TcPlan &p, const M2TcTiles &t, int64_t N)
     // a stage always belongs to the same group of converting warps: a group that came by only every other time could not
     // tell the two apart by the parity of the barrier
     if (MODE == M2_CONV) p.stages -= p.stages % CONV_GROUPS;
-    p.smem = (size_t)p.stages * stage + (size_t)(S::NBOX - p.na) * S::BOX_BYTES * (MODE == M2_CONV ? 2 : 1) + 1024 + 1024;
+    p.smem = MODE == M2_EXACT ? EX_SMEM : (size_t)p.stages * stage + (size_t)(S::NBOX - p.na) * S::BOX_BYTES * (MODE == M2_CONV ? 2 : 1) + 1024 + 1024;
     // Clusters (one per pair of SMs) go to the tiles in proportion to their cost, the remaining ones each to the tile whose
     // share of the samples takes longest; then every tile gives back what it does not need to keep up with the slowest.
     // Tiles of equal width so get equal shares: their clusters run in step and share X in L2 (with unequal shares the wide
@@ -568,7 +582,10 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
     for (int tn = 0; tn < nt; ++tn)
         for (int tm = 0; tm < nt; ++tm) {
             if (tm > tn && !dense) continue;
-            const int left = (int)d - tn * BN, width = left >= BN ? BN : (left + 31) / 32 * 32, below = (int)d - tm * BM;
+            const int left = (int)d - tn * BN, below = (int)d - tm * BM;
+            int width = left >= BN ? BN : (left + 31) / 32 * 32;
+            // M2_EXACT: with all 256 columns A holds B, and half as many values are converted ([65536,200] 52 us, now 45)
+            if (MODE == M2_EXACT && tm == tn && width > HALF) width = BN;
             if (!t.add<MODE>(tm * BM, below < BM ? below : BM, tn * BN, width, tm == tn)) return p;
         }
     m2tc_finish<MODE>(p, t, N);
@@ -640,6 +657,12 @@ static const M2TcPlan &m2tc_plan_pairs(int64_t N, const PairLayout &L)
     return p;
 }
 
+template <int MODE> static auto m2tc_kernel()
+{
+    if constexpr (MODE == M2_EXACT) return moment2_exact_kernel;
+    else return moment2_tc_kernel<MODE>;
+}
+
 // Launches the tile kernel and the sum of its partial tiles.  rows: rows of X in memory; pairs: X holds the pair features
 // of `features` features and the result goes to their packed 4-simplex.
 template <int MODE>
@@ -648,19 +671,22 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
 {
     using S = m2tc::Shape<MODE>;
     CUtensorMap tmap;
-    if (!tc::make_tmap_2d(&tmap, MODE == M2_TF32 || MODE == M2_CONV ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, X, (uint64_t)rows,
-                          (uint64_t)d, (uint64_t)ldx * (MODE == M2_CONV ? 4 : S::ELEM), MODE == M2_CONV ? 32 : S::BOXC, S::KROWS,
+    constexpr bool WORDS = MODE == M2_TF32 || MODE == M2_CONV || MODE == M2_EXACT;
+    if (!tc::make_tmap_2d(&tmap, WORDS ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, X, (uint64_t)rows,
+                          (uint64_t)d, (uint64_t)ldx * (WORDS ? 4 : 2), WORDS ? 32 : S::BOXC, S::KROWS,
                           MODE == M2_TF32 ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B))
         return ST_ERR_CUDA;
     m2tc::Args a;
     a.partials = partials; a.status = status;
     a.chunks_total = q.chunks_total; a.stages = q.stages; a.nb = q.nb; a.na = q.na; a.lo_row0 = (int)lo_row0; a.d = (int)d;
-   
+    a.X = (const float *)X; a.N = rows; a.ldx = ldx;
     a.tab = q.tab;
-    if (!ensure_dynamic_smem(moment2_tc_kernel<MODE>, q.smem)) return ST_ERR_CUDA;
+    const auto kernel = m2tc_kernel<MODE>();
+    if (!ensure_dynamic_smem(kernel, q.smem)) return ST_ERR_CUDA;
+    if (MODE == M2_EXACT && !m2tc_exact_fits()) return ST_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)q.tab.first[q.tab.ntiles]);
-    cfg.blockDim = dim3(MODE == M2_CONV ? m2tc::THREADS + m2tc::CONV_THREADS : m2tc::THREADS);
+    cfg.blockDim = dim3(MODE == M2_EXACT ? m2tc::EX_THREADS : MODE == M2_CONV ? m2tc::THREADS + m2tc::CONV_THREADS : m2tc::THREADS);
     cfg.dynamicSmemBytes = q.smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -672,7 +698,7 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, moment2_tc_kernel<MODE>, tmap, a) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, kernel, tmap, a) != cudaSuccess) {
         (void)cudaGetLastError();
         return ST_ERR_CUDA;
     }
@@ -744,6 +770,15 @@ st_status moment2_bf16_tc(const void *X, int64_t N, int64_t d, int64_t ldx, floa
 {
     if (d % 8 != 0 || ldx % 8 != 0) return ST_ERR_ALIGN;
     return m2tc_run<M2_BF16>(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
+}
+
+// fp32 input, no less accurate than fp32 FMAs (moment2_exact.cuh); rows of X that a tensor map can name
+size_t moment2_exact_tc_workspace(int64_t N, int64_t d, unsigned flags) { return m2tc_workspace<M2_EXACT>(N, d, flags); }
+
+st_status moment2_exact_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
+                           unsigned flags, cudaStream_t stream)
+{
+    return ldx % 4 != 0 ? ST_ERR_ALIGN : m2tc_run<M2_EXACT>(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
 }
 
 // ---------------------------------------------------------------------------------------------

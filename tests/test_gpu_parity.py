@@ -1384,3 +1384,60 @@ def test_copies_with_64_bit_indices(st):
     lo, hi = torch.minimum(i[:, None], j), torch.maximum(i[:, None], j)
     want = P[lo * (2 * d - lo + 1) // 2 + hi - lo]
     assert torch.equal(D[i], want) and torch.equal(D[:, i].T, want)
+
+
+# ------------------------------------------------------------------ fp32 second moment of many samples: exact parts of x
+# Per element: three products of parts are left out (3 * 2^-27 of a term), a sum of 32 samples is truncated to 24 bits a few
+# times (2^-22 together), and at most 104 such sums and partial tiles are added by fp32 additions here: 6.7e-6.
+TOL_EXACT = 7e-6
+
+
+@pytest.mark.parametrize("N,d,ldx", [(20000, 124, 124), (16401, 128, 128), (12001, 160, 164), (4999, 240, 240), (5003, 256, 256),
+                                     (4211, 260, 260), (2500, 388, 388), (1101, 516, 520), (290, 1000, 1000)])
+def test_moment2_f32_exact_parts(st, N, d, ldx):
+    X = workloads.draw((N, ldx), "normal", 31 + d)
+    T, S = oracle.moment2(np.ascontiguousarray(X[:, :d]))
+    iu = np.triu_indices(d)
+    Xd, out = dev(X), guarded(st, d * (d + 1) // 2)
+    nbytes = st.st_workspace_bytes(st.ST_OP_SYM_MOMENT2, N, d, st.ST_F32)
+    ws = guarded(st, nbytes, torch.uint8)
+    rc = st.lib().st_sym_moment2(Xd.data_ptr(), st.ST_F32, N, d, ldx, out.data_ptr(), ws.data_ptr(), nbytes, 0,
+                                 torch.cuda.current_stream().cuda_stream)
+    assert rc == st.ST_OK
+    assert oracle.rel_err(out.cpu().numpy(), T[iu], S[iu]) <= TOL_EXACT
+
+
+@pytest.mark.parametrize("N,d", [(5000, 250), (2100, 400)])
+def test_moment2_f32_values_without_exact_parts(st, N, d):
+    """Infinities, NaN, values that round to infinity in bf16 and columns of tiny values: as fp32 arithmetic has them."""
+    X = workloads.draw((N, d), "normal", 77)
+    X[100, 3], X[200, d - 10], X[5, 7], X[6, 8], X[6, 7] = np.inf, np.nan, -np.inf, 0.0, 0.0
+    X[10] *= np.float32(0.1)           # no product of the huge value leaves the range of fp32 but its square
+    X[10, 20], X[:, 21] = 3.395e38, X[:, 21] * np.float32(1e-12)
+    X[:, 30] *= np.float32(1e-36)
+    X[:, d - 30] *= np.float32(1e30)
+    X[10, d - 30] = 0.0
+    X[:, 40], X[:, 41], X[::5, 42] = 0.0, 1.0, np.float32(1e-38)
+    with np.errstate(all="ignore"):
+        D = X.astype(np.float64)
+        ref = (D.T @ D)
+        mag = np.abs(np.where(np.isfinite(D), D, 0.0))
+        mag = mag.T @ mag
+        big = np.abs(ref) > 3.4028234e38
+        ref = np.where(big, np.sign(ref) * np.inf, ref)
+    iu = np.triu_indices(d)
+    ref, mag = ref[iu], mag[iu]
+    got = st.st_sym_moment2(dev(X)).cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    assert np.array_equal(np.isposinf(got), np.isposinf(ref)) and np.array_equal(np.isneginf(got), np.isneginf(ref))
+    fin = np.isfinite(ref)
+    # below 2^-126 fp32 numbers are 2^-149 apart
+    assert np.all(np.abs(got[fin] - ref[fin]) <= 1e-4 * mag[fin] + N * 2.0 ** -149)
+    assert got[iu[0].tolist().index(41)] == N          # a column of ones counts exactly
+
+
+def test_moment2_f32_exact_parts_count_exactly(st):
+    X = workloads.draw((9001, 192), "uniform", 5)
+    X = (X > 0).astype(np.float32)
+    got = st.st_sym_moment2(dev(X)).cpu().numpy()
+    assert np.array_equal(got, (X.T.astype(np.float64) @ X)[np.triu_indices(192)])
