@@ -13,12 +13,13 @@
 // columns k >= 16*JB only: its MMA has N = d - 16*JB, so the part k < j of the iteration space
 // is (up to that granularity) never issued, and tiles with i > j everywhere do not exist.
 // Accumulators of all tiles of a block stay in tensor memory for the block's whole sample
-// range; at d = 64 they need 640 columns, so two blocks ("groups") share one sample range.
+// range; two to eight blocks ("groups") share one sample range and its tiles, for fewer partial sums.
 //
-// What bounds it: the latency of a stage, no unit is saturated ([40009,50] bf16: tensor pipe 10 %, FMA pipe 14 %, shared memory about
-// 31 %).  Per tile and slice the producers store 16 KB of products and the tensor core reads
-// them back with the columns of X^T (an MMA of M = 128, N <= 64 takes 39 to 48 cycles, bound by its operand reads); the
-// stages of eight producer warps come every 320 cycles.  Two issuer warps take alternate stages: polls and commits
+// What bounds it: issue slots and the latency of a stage, no unit is saturated.  Per tile and slice the producers store 16 KB of
+// products and the tensor core reads them back with the columns of X^T (an MMA of M = 128, N <= 64 takes 39 to 48 cycles, bound
+// by its operand reads).  A warp took 2700 cycles for a whole stage, 1300 of them for 128 products a lane, and eight warps made
+// one every 340; sixteen, two to a stage, and copies without a selected address for whole slices: [40009,50] bf16 36.0 us,
+// now 35.2, [200000,50] 140 (before generic loads went) and 117, TF32 246 and 183.  Two issuer warps take alternate stages: polls and commits
 // between the MMAs cost one alone about 100 cycles per stage.  bf16 halves the number of stages (64 samples per slice
 // instead of 32).  Products and x_k rounded to TF32 / bf16, fp32 accumulation: 5e-3 tolerance (bf16: for N >= 1000).
 #include "tc_common.cuh"
@@ -35,13 +36,13 @@ constexpr int ROW_BYTES = 128;               // one swizzled row: 32 TF32 or 64 
 constexpr int A_STAGE_BYTES = BM * ROW_BYTES; // 16 KiB
 constexpr int NA_MAX = 10;                   // A stages in flight (TF32: 10, bf16: 8; even: see the issuers)
 constexpr int NB_MAX = 16;                   // slices in flight: as many as fit beside the A stages (4 at d = 64), see ring()
-constexpr int PRODUCERS = 8;                 // producer warps (also the epilogue warps)
+constexpr int PRODUCERS = 16;                // producer warps (also the epilogue warps): two to a stage, half of its rows each
 constexpr int MMA_WARPS = 2;                 // issuer w takes the stages q = w (mod 2): while one polls, the other's MMAs run
 constexpr int MMA_WARP = PRODUCERS, LOAD_WARP = PRODUCERS + MMA_WARPS;
 constexpr int LOAD_WARPS = 4;                // fetch slices of X and turn them into the right operand
 constexpr int THREADS = 32 * (PRODUCERS + MMA_WARPS + LOAD_WARPS);
 constexpr uint32_t TMEM_COLS = 512;
-constexpr int MAX_GROUP_TILES = 12;
+constexpr int MAX_GROUP_TILES = 12, MAX_TILES = 20, MAX_GROUPS = 8;
 // A slice in flight: dcols rows of X^T as the right operand, and the samples as they are in memory, rows of dcols + 1
 // floats (an odd pitch: lanes that read one column of consecutive samples touch every bank once).
 constexpr size_t FIXED_SMEM = 1024 + 1024;    // alignment of the first stage; barriers
@@ -74,8 +75,8 @@ struct Args {
     int64_t N, ldx, rows_per_slice;
     int nb;                                  // slices in flight
     int d, dcols, part_elems;                // part_elems: partial sums per slice; dcols = d rounded up to a multiple of 16
-    int ntiles[2];
-    Tile tiles[2][MAX_GROUP_TILES];
+    int first[MAX_GROUPS + 1];               // tiles of group g: first[g] ..
+    Tile tiles[MAX_TILES];
 };
 
 // byte offset of the 4-byte word `lane` (one TF32 sample, or two bf16 samples) inside a 128-byte row whose
@@ -112,12 +113,12 @@ moment3_tc_kernel(const __grid_constant__ Args a)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int group = blockIdx.x;
-    const int tg = a.ntiles[group];                          // tiles of this block
-    const Tile *tiles = a.tiles[group];
+    const int tg = a.first[group + 1] - a.first[group];      // tiles of this block
+    const Tile *tiles = a.tiles + a.first[group];
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < NA; ++s) {
-            mbar_init(&a_full[s], 1);
+            mbar_init(&a_full[s], 2);
             mbar_init(&a_empty[s], 1);
         }
         for (int s = 0; s < NB; ++s) {
@@ -155,33 +156,34 @@ moment3_tc_kernel(const __grid_constant__ Args a)
     for (int m = 0; m < 8; ++m) sw[m] = swz(lane, m);
 
     if (warp < PRODUCERS) {
-        // ---- producers: A stage q = slice * tg + tile is made by warp q % PRODUCERS -------------
+        // ---- producers: A stage q = slice * tg + tile is made by the pair of warps q % (PRODUCERS / 2) -------------
         // A wait names a phase by its parity only, so a waiter must never be two phases ahead of its
-        // barrier: with stages dealt round-robin to `nprod` warps that holds when nprod <= NA (slots of
+        // barrier: with stages dealt round-robin to `nprod` pairs that holds when nprod <= NA (slots of
         // the A ring) and nprod <= NB * tg (stages covered by the slices of the X^T ring).
-        const int nprod = min(min(PRODUCERS, NA), NB * tg);
+        const int nprod = min(min(PRODUCERS / 2, NA), NB * tg), pair = warp >> 1;
+        const int e0 = (warp & 1) * (TI / 2);                 // values of i of this warp: e0 .. e0 + TI / 2 - 1 of the tile's
         bool ok = true;
-        int bs = warp / tg, ti = warp - bs * tg, as = warp, use = 0;           // of stage q; bs: ring position of its slice
+        int bs = pair / tg, ti = pair - bs * tg, as = pair, use = 0;           // of stage q; bs: ring position of its slice
         uint32_t b_parity = 0;
         while (bs >= NB) { bs -= NB; b_parity ^= 1u; }
         const int dslice = nprod / tg, dti = nprod - dslice * tg;
-        for (int64_t q = warp; q < nstages && ok && warp < nprod; q += nprod) {
+        for (int64_t q = pair; q < nstages && ok && pair < nprod; q += nprod) {
             if (!mbar_wait(&b_full[bs], b_parity, abort_flag, a.status, 11)) break;
             // this lane's sample: x_i for the tile's 8 values of i, x_j for its 16 values of j
             const unsigned char *bst = b_stage0 + (size_t)bs * B_STAGE_BYTES;
             const Tile t = tiles[ti];
             // TF32: the rounded values of the MMA's own slice; bf16: the slice of X itself, samples `lane` and
             // `lane` + 32, so that every product is rounded once
-            uint64_t xi[TI], xj[TJ];                       // TF32: the low word only
+            uint64_t xi[TI / 2], xj[TJ];                   // TF32: the low word only
             if (BF16) {
                 const float *xst = x_stage0 + (size_t)bs * X_STAGE_FLOATS + lane * x_pitch;
 #pragma unroll
-                for (int e = 0; e < TI; ++e) xi[e] = m3tc_pack2(xst[TI * t.ib + e], xst[(BF16 ? 32 : 0) * x_pitch + TI * t.ib + e]);
+                for (int e = 0; e < TI / 2; ++e) xi[e] = m3tc_pack2(xst[TI * t.ib + e0 + e], xst[(BF16 ? 32 : 0) * x_pitch + TI * t.ib + e0 + e]);
 #pragma unroll
                 for (int e = 0; e < TJ; ++e) xj[e] = m3tc_pack2(xst[TJ * t.jb + e], xst[(BF16 ? 32 : 0) * x_pitch + TJ * t.jb + e]);
             } else {
 #pragma unroll
-                for (int e = 0; e < TI; ++e) xi[e] = *reinterpret_cast<const uint32_t *>(bst + (TI * t.ib + e) * 128 + sw[e & 7]);
+                for (int e = 0; e < TI / 2; ++e) xi[e] = *reinterpret_cast<const uint32_t *>(bst + (TI * t.ib + e0 + e) * 128 + swz(lane, e0 + e));
 #pragma unroll
                 for (int e = 0; e < TJ; ++e) xj[e] = *reinterpret_cast<const uint32_t *>(bst + (TJ * t.jb + e) * 128 + sw[e & 7]);
             }
@@ -189,12 +191,12 @@ moment3_tc_kernel(const __grid_constant__ Args a)
                 ok = false;
                 break;
             }
-            unsigned char *ast = a_stage0 + (size_t)as * A_STAGE_BYTES;
+            unsigned char *ast = a_stage0 + (size_t)as * A_STAGE_BYTES + e0 * TJ * 128;
 #pragma unroll
-            for (int e = 0; e < TI; ++e)
+            for (int e = 0; e < TI / 2; ++e)
 #pragma unroll
                 for (int f = 0; f < TJ; ++f) {
-                    // row e*16+f of the tile
+                    // row (e0 + e) * 16 + f of the tile
                     uint32_t v;
                     if (BF16) {
                         // two samples per word, each product rounded once to bf16 (first sample in the low half)
@@ -324,6 +326,16 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             const int64_t src_step = STEP * a.ldx;
             const bool c0 = c < a.d, c1 = W == 32 && c + 32 < a.d, wide = W == 32 && a.dcols > 32;
             dst += (uint32_t)(r0 * x_pitch + c) * 4u;
+            if (W == 32 && rows == KS) {
+                // a whole slice: lanes of columns past d copy nothing (their words are zeros from the start)
+                const uint32_t dst_step = (uint32_t)(STEP * x_pitch) * 4u;
+#pragma unroll 8
+                for (int u = 0; u < KS / STEP; ++u, dst += dst_step, src += src_step) {
+                    if (c0) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src));
+                    if (c1) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 128u), "l"(src + 32));
+                }
+                return;
+            }
 #pragma unroll 8
             for (int r = r0; r < KS; r += STEP, dst += (uint32_t)(STEP * x_pitch) * 4u, src += src_step) {
                 const bool p0 = c0 && r < rows, p1 = c1 && r < rows;
@@ -334,6 +346,9 @@ moment3_tc_kernel(const __grid_constant__ Args a)
                     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 128u), "l"(s1), "r"(p1 ? 4 : 0));
             }
         };
+        // columns past d: zeros in every buffer before the first copy
+        for (int r = a.dcols > 16 ? lt : NB * KS; r < NB * KS; r += 32 * LOAD_WARPS)
+            for (int c = a.d; c < a.dcols; ++c) x_stage0[(size_t)(r / KS) * X_STAGE_FLOATS + (r % KS) * x_pitch + c] = 0.f;
         int fetch_slot = 0;
         auto fetch = [&](int slice) {                                     // called with slice = 0, 1, 2, ...
             const int64_t n0 = n_begin + (int64_t)slice * KS;
@@ -404,7 +419,7 @@ struct SumArgs {
     const float *partials;
     float *out;
     int slices, part_elems, d, ntiles;
-    Tile tiles[2 * MAX_GROUP_TILES];
+    Tile tiles[MAX_TILES];
 };
 
 // out[q(i,j,k)] = sum over the slices of the partial sum of row (i, j), column k of a tile: a block owns 32 rows of one
@@ -445,9 +460,9 @@ moment3_tc_sum_kernel(const __grid_constant__ SumArgs a)
 }
 
 struct Plan {
-    int groups, slices, dcols;
-    int ntiles[2];
-    Tile tiles[2][MAX_GROUP_TILES];
+    int groups, slices, dcols, ntiles;
+    int first[MAX_GROUPS + 1];
+    Tile tiles[MAX_TILES];
     int64_t rows_per_slice;
     int part_elems;
     bool ok;
@@ -461,41 +476,49 @@ static Plan plan(int64_t N, int64_t d, bool bf16)
     if (N <= 0 || d < 1 || d > DP) return p;
     p.dcols = (int)((d + 15) / 16 * 16);
     // tiles in the order (JB, IB); a tile exists when it holds some i <= j < d
-    Tile all[2 * MAX_GROUP_TILES];
-    int cols[2 * MAX_GROUP_TILES], n = 0, total_cols = 0;
+    int cols[MAX_TILES], n = 0;
     for (int jb = 0; jb * TJ < d; ++jb)
         for (int ib = 0; ib * TI < d && ib * TI <= jb * TJ + TJ - 1; ++ib) {
-            if (n >= 2 * MAX_GROUP_TILES) return p;
-            all[n].ib = (unsigned char)ib;
-            all[n].jb = (unsigned char)jb;
+            if (n >= MAX_TILES) return p;
+            p.tiles[n].ib = (unsigned char)ib;
+            p.tiles[n].jb = (unsigned char)jb;
             cols[n] = p.dcols - jb * TJ;
-            all[n].part = p.part_elems;
+            p.tiles[n].part = p.part_elems;
             p.part_elems += cols[n] * BM;
-            total_cols += cols[n];
             ++n;
         }
-    p.groups = total_cols > (int)TMEM_COLS ? 2 : 1;
-    const int first = p.groups == 1 ? n : (n + 1) / 2;      // equal numbers of tiles: the stores of P are the bound
-    if (first > MAX_GROUP_TILES || n - first > MAX_GROUP_TILES) return p;
-    for (int g = 0; g < p.groups; ++g) {
-        const int lo = g == 0 ? 0 : first, hi = g == 0 ? first : n;
-        int col = 0;
-        for (int t = lo; t < hi; ++t) {
-            p.tiles[g][t - lo] = all[t];
-            p.tiles[g][t - lo].col = (unsigned short)col;
-            col += cols[t];
-        }
-        if (col > (int)TMEM_COLS) return p;
-        p.ntiles[g] = hi - lo;
-    }
+    p.ntiles = n;
+    // Groups: the number for which the longest block and the sum after it take least, in cycles: 230 a stage, but 2000 a slice at
+    // least (what fetching and turning it takes), 650 a tile for its partial sums, 60 a slice in the sum.  With 1, 2, 4 and 8
+    // groups, bf16, us: [256,33] 11.2, 9.3, 8.2, 7.6; [4096,33] 11.9, 10.2, 10.0, 10.8; [40009,33] 23.6, 22.5, 26.1, 40.6;
+    // [200000,33] 66, 77, 101, 175.  Before, with as few groups as tensor memory allows: [256,50] 15.1, now 11.2; [256,64] 16.1, 12.1.
     const int sms = sm_count_or_default();
-    int64_t slices = sms / p.groups;
-    if (slices < 1) slices = 1;
-    int64_t rps = (N + slices - 1) / slices;
-    rps = (rps + KS - 1) / KS * KS;                        // whole MMA slices
-    p.rows_per_slice = rps;
-    p.slices = (int)((N + rps - 1) / rps);
-    p.ok = true;
+    double best = 0;
+    for (int groups = 1; groups <= MAX_GROUPS && groups <= n && groups <= sms; ++groups) {
+        // equal numbers of tiles: the stores of P are the bound
+        int first[MAX_GROUPS + 1], longest = 0;
+        bool fits = true;
+        for (int g = 0; g <= groups; ++g) first[g] = (int)((int64_t)n * g / groups);
+        for (int g = 0; g < groups; ++g) {
+            int col = 0;
+            for (int t = first[g]; t < first[g + 1]; ++t) col += cols[t];
+            if (first[g + 1] - first[g] > longest) longest = first[g + 1] - first[g];
+            fits = fits && col <= (int)TMEM_COLS;
+        }
+        if (!fits || longest > MAX_GROUP_TILES) continue;
+        int64_t slices = sms / groups, rps = ((N + slices - 1) / slices + KS - 1) / KS * KS;      // whole MMA slices
+        slices = (N + rps - 1) / rps;
+        const double cost = (double)(rps / KS) * (longest * 230 > 2000 ? longest * 230 : 2000) + longest * 650 + (double)slices * 60;
+        if (p.ok && cost >= best) continue;
+        best = cost;
+        p.groups = groups;
+        p.slices = (int)slices;
+        p.rows_per_slice = rps;
+        for (int g = 0; g <= groups; ++g) p.first[g] = first[g];
+        p.ok = true;
+    }
+    for (int g = 0; g < p.groups; ++g)
+        for (int t = p.first[g], col = 0; t < p.first[g + 1]; col += cols[t++]) p.tiles[t].col = (unsigned short)col;
     return p;
 }
 
@@ -527,10 +550,8 @@ st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *o
     a.N = N; a.ldx = ldx; a.rows_per_slice = p.rows_per_slice;
     a.nb = ring(p.dcols, bf16);
     a.d = (int)d; a.dcols = p.dcols; a.part_elems = p.part_elems;
-    for (int g = 0; g < 2; ++g) {
-        a.ntiles[g] = p.ntiles[g];
-        for (int t = 0; t < MAX_GROUP_TILES; ++t) a.tiles[g][t] = p.tiles[g][t];
-    }
+    for (int g = 0; g <= MAX_GROUPS; ++g) a.first[g] = p.first[g <= p.groups ? g : p.groups];
+    for (int t = 0; t < MAX_TILES; ++t) a.tiles[t] = p.tiles[t];
     auto run = [&](auto kernel) {
         if (!ensure_dynamic_smem(kernel, smem_bytes(p.dcols, bf16))) return ST_ERR_CUDA;
         return launch(kernel, dim3(p.groups, p.slices), THREADS, smem_bytes(p.dcols, bf16), stream, a);
@@ -543,8 +564,8 @@ st_status moment3_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *o
     m.slices = p.slices;
     m.part_elems = p.part_elems;
     m.d = (int)d;
-    m.ntiles = p.ntiles[0] + p.ntiles[1];
-    for (int t = 0; t < m.ntiles; ++t) m.tiles[t] = t < p.ntiles[0] ? p.tiles[0][t] : p.tiles[1][t - p.ntiles[0]];
+    m.ntiles = p.ntiles;
+    for (int t = 0; t < MAX_TILES; ++t) m.tiles[t] = p.tiles[t];
     return launch(moment3_tc_sum_kernel, (unsigned)(p.part_elems / 32), 32 * SUM_WARPS, 0, stream, m);
 }
 
