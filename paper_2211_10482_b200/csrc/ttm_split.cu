@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(split::THREADS, 1) ttm_split_kernel(const Spli
     using namespace split;
     using namespace tc;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *smem = align_smem(smem_raw);
+    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int w_region = 2 * a.R * 128;                               // [Wh; Wl] of one chunk of 64 k-values
     unsigned char *w_smem = smem;
     unsigned char *stage0 = smem + (size_t)a.kchunks * w_region;

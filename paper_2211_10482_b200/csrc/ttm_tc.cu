@@ -51,7 +51,7 @@ ttm_tc_kernel(const __grid_constant__ CUtensorMap tmap, const TtmTcArgs a)
     using namespace ttmtc;
     using namespace tc;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *smem = align_smem(smem_raw);
+    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int u_region = a.R * 128;                                  // bytes of one k-slice of U^T (multiple of 2048)
     unsigned char *u_smem = smem;                                    // kchunks regions
     unsigned char *stage0 = smem + (size_t)a.kchunks * u_region;
