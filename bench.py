@@ -130,7 +130,9 @@ def call_table(cfg):
     m2l = dict(flops=2 * c5["N"] * tri(c5["d"]))
     t["sym_moment2_large"] = dict(m2l, bytes=2 * c5["N"] * c5["d"] + 4 * tri(c5["d"]), bound="tensor", launches=2,
                                   tensor_scale=1.0)
-    t["sym_moment2_large_f32"] = dict(m2l, bytes=4 * c5["N"] * c5["d"] + 4 * tri(c5["d"]), bound="alu", launches=2)
+    # six bf16 products of the exact parts per term
+    t["sym_moment2_large_f32"] = dict(m2l, bytes=4 * c5["N"] * c5["d"] + 4 * tri(c5["d"]), bound="tensor", launches=2,
+                                      tensor_scale=1.0 / 6.0)
     t["sym_moment2_large_f32_tf32"] = dict(m2l, bytes=4 * c5["N"] * c5["d"] + 4 * tri(c5["d"]), bound="tensor", launches=2,
                                            tensor_scale=TF32_OVER_BF16)
     # three bf16 partial products per term; the split pass reads X and writes as many bytes, the GEMM passes read them again
