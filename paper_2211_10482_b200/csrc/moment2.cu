@@ -377,7 +377,7 @@ static bool moment2_use_small(int64_t N, int64_t d, unsigned flags)
 // features the register tiles are the better ones ([200000,120] 78 / 92), and those of 129 to 136 are no worse ([65536,136] 43 / 43).
 static bool moment2_use_exact(int64_t N, int64_t d)
 {
-    if (d <= 120 || (d > 128 && d <= 136) || d > 4096 || N > (int64_t(1) << 31) - 64) return false;
+    if (d % 4 != 0 || d <= 120 || (d > 128 && d <= 136) || d > 4096 || N > (int64_t(1) << 31) - 64) return false;
     const double values = (double)N * (double)d;
     return values * (double)d >= 2.7e8 || (d > 136 && values >= 8e5);
 }

@@ -1393,7 +1393,7 @@ TOL_EXACT = 7e-6
 
 
 @pytest.mark.parametrize("N,d,ldx", [(20000, 124, 124), (16401, 128, 128), (12001, 160, 164), (4999, 240, 240), (5003, 256, 256),
-                                     (4211, 260, 260), (3301, 255, 256), (2700, 389, 392), (1101, 516, 520), (290, 1000, 1000)])
+                                     (4211, 260, 260), (2500, 388, 388), (1101, 516, 520), (290, 1000, 1000)])
 def test_moment2_f32_exact_parts(st, N, d, ldx):
     X = workloads.draw((N, ldx), "normal", 31 + d)
     T, S = oracle.moment2(np.ascontiguousarray(X[:, :d]))
