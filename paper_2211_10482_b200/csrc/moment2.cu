@@ -386,7 +386,11 @@ static st_status moment2_f32(const float *X, int64_t N, int64_t d, int64_t ldx, 
                              size_t ws_bytes, unsigned flags, cudaStream_t stream)
 {
     if (d > 32768) return ST_ERR_UNSUPPORTED;
-    if (ldx % 4 == 0 && moment2_use_exact(N, d)) return moment2_exact_tc(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
+    if (ldx % 4 == 0 && moment2_use_exact(N, d)) {
+        // more tiles than the plan holds (dense control of more than 3072 features): the FMA kernels take it
+        const st_status rc = moment2_exact_tc(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
+        if (rc != ST_ERR_UNSUPPORTED) return rc;
+    }
     return moment2_use_small(N, d, flags) ? moment2_small(X, N, d, ldx, out, ws, ws_bytes, flags, stream)
                                        : moment2_gemm(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
 }

@@ -1441,3 +1441,12 @@ def test_moment2_f32_exact_parts_count_exactly(st):
     X = (X > 0).astype(np.float32)
     got = st.st_sym_moment2(dev(X)).cpu().numpy()
     assert np.array_equal(got, (X.T.astype(np.float64) @ X)[np.triu_indices(192)])
+
+
+def test_moment2_f32_dense_control_of_more_tiles_than_a_plan_holds(st):
+    N, d = 260, 3076
+    X = workloads.draw((N, d), "normal", 6)
+    T, S = oracle.moment2(X)
+    got = st.st_sym_moment2(dev(X), flags=st.ST_FLAG_DENSE_CONTROL).cpu().numpy()
+    iu = np.triu_indices(d)
+    assert oracle.rel_err(got, T[iu], S[iu]) <= TOL_F32

@@ -144,6 +144,10 @@ def test_layout_sizes_and_host_side_validation():
     assert L.st_sym_moment2(256, st.ST_F32, 4, 4, 4, 512, None, 0, 0, None) == st.ST_ERR_WORKSPACE
     assert L.st_sym_moment3(256, 4, 257, 257, 512, None, 0, 0, None) == st.ST_ERR_UNSUPPORTED
     assert L.st_sym_moment3(264, 4, 16, 16, 512, None, 0, 0, None) == st.ST_ERR_ALIGN
+    # fp32 takes any feature count, dense control too, also where one of its routes has no plan
+    for d in (3068, 3072, 3076, 4096, 4100):
+        for flags in (0, st.ST_FLAG_DENSE_CONTROL):
+            assert L.st_sym_moment2(256, st.ST_F32, 260, d, d, 512, None, 0, flags, None) == st.ST_ERR_WORKSPACE, (d, flags)
     assert L.st_sym_moment3(256, 4, 16, 16, 512, None, 0, 0, None) == st.ST_ERR_WORKSPACE
     assert L.st_sym_moment3(256, 4, 12, 18, 512, None, 0, 0, None) == st.ST_ERR_WORKSPACE     # any d, any pitch
     assert L.st_sym_moment3(256, 4, 72, 72, 512, None, 0, st.ST_FLAG_TC_TF32, None) == st.ST_ERR_UNSUPPORTED
