@@ -17,6 +17,7 @@
 // Values whose parts are not all bfloat16 numbers (infinities, NaN, |x| > 2^127.99, columns of |x| < 2^-100) give the samples of
 // the cluster that meets them to plain fp32 FMAs.
 #pragma once
+#include <atomic>
 #include <type_traits>
 
 namespace st {
@@ -479,16 +480,20 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
 }
 
 // The warpgroups of moment2_exact_kernel pass registers among them: what they end with is what the block must start with, or
-// one of them would wait for good.
+// one of them would wait for good.  A kernel that was built with fewer is not launched.
 inline bool m2tc_exact_fits()
 {
-    static const int regs = [] {
+    static std::atomic<int> known{0};
+    int regs = known.load(std::memory_order_relaxed);
+    if (regs == 0) {
         cudaFuncAttributes f;
-        if (cudaFuncGetAttributes(&f, moment2_exact_kernel) == cudaSuccess) return f.numRegs;
-        (void)cudaGetLastError();
-        return -1;
-    }();
-    return regs >= 0 && (regs + 7) / 8 * 8 >= m2tc::EX_REGS;
+        if (cudaFuncGetAttributes(&f, moment2_exact_kernel) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        known.store(regs = f.numRegs, std::memory_order_relaxed);
+    }
+    return (regs + 7) / 8 * 8 >= m2tc::EX_REGS;
 }
 
 }  // namespace st

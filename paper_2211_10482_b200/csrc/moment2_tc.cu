@@ -683,7 +683,6 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     a.tab = q.tab;
     const auto kernel = m2tc_kernel<MODE>();
     if (!ensure_dynamic_smem(kernel, q.smem)) return ST_ERR_CUDA;
-    if (MODE == M2_EXACT && !m2tc_exact_fits()) return ST_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)q.tab.first[q.tab.ntiles]);
     cfg.blockDim = dim3(MODE == M2_EXACT ? m2tc::EX_THREADS : MODE == M2_CONV ? m2tc::THREADS + m2tc::CONV_THREADS : m2tc::THREADS);
@@ -778,7 +777,9 @@ size_t moment2_exact_tc_workspace(int64_t N, int64_t d, unsigned flags) { return
 st_status moment2_exact_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
                            unsigned flags, cudaStream_t stream)
 {
-    return ldx % 4 != 0 ? ST_ERR_ALIGN : m2tc_run<M2_EXACT>(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
+    if (ldx % 4 != 0) return ST_ERR_ALIGN;
+    if (!m2tc_exact_fits()) return ST_ERR_UNSUPPORTED;
+    return m2tc_run<M2_EXACT>(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
 }
 
 // ---------------------------------------------------------------------------------------------
