@@ -388,9 +388,9 @@ static st_status moment2_f32(const float *X, int64_t N, int64_t d, int64_t ldx, 
     if (d > 32768) return ST_ERR_UNSUPPORTED;
     if (ldx % 4 == 0 && moment2_use_exact(N, d)) {
         // the FMA kernels take what this route does not: more tiles than its plan holds (dense control of more than 3072
-        // features), a build of its kernel with too few registers
+        // features), a build of its kernel with too few registers, a workspace that is large enough for them alone
         const st_status rc = moment2_exact_tc(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
-        if (rc != ST_ERR_UNSUPPORTED) return rc;
+        if (rc != ST_ERR_UNSUPPORTED && rc != ST_ERR_WORKSPACE) return rc;
     }
     return moment2_use_small(N, d, flags) ? moment2_small(X, N, d, ldx, out, ws, ws_bytes, flags, stream)
                                        : moment2_gemm(X, N, d, ldx, out, ws, ws_bytes, flags, stream);

@@ -1450,3 +1450,20 @@ def test_moment2_f32_dense_control_of_more_tiles_than_a_plan_holds(st):
     got = st.st_sym_moment2(dev(X), flags=st.ST_FLAG_DENSE_CONTROL).cpu().numpy()
     iu = np.triu_indices(d)
     assert oracle.rel_err(got, T[iu], S[iu]) <= TOL_F32
+
+
+def test_moment2_f32_workspace_for_the_fma_kernels_alone(st):
+    # 17.8 MB are enough for the FMA kernels; the tensor-core route has more partial tiles
+    N, d = 4096, 2048
+    X = workloads.draw((N, d), "normal", 8)
+    nbytes = st.st_workspace_bytes(st.ST_OP_SYM_MOMENT2, N, d, st.ST_F32) - 1
+    Xd, out, ws = dev(X), guarded(st, d * (d + 1) // 2), guarded(st, nbytes, torch.uint8)
+    rc = st.lib().st_sym_moment2(Xd.data_ptr(), st.ST_F32, N, d, d, out.data_ptr(), ws.data_ptr(), nbytes, 0,
+                                 torch.cuda.current_stream().cuda_stream)
+    assert rc == st.ST_OK
+    T, S = oracle.moment2(X)
+    iu = np.triu_indices(d)
+    assert oracle.rel_err(out.cpu().numpy(), T[iu], S[iu]) <= TOL_F32
+    rc = st.lib().st_sym_moment2(Xd.data_ptr(), st.ST_F32, N, d, d, out.data_ptr(), ws.data_ptr(), 1 << 20, 0,
+                                 torch.cuda.current_stream().cuda_stream)
+    assert rc == st.ST_ERR_WORKSPACE
