@@ -359,6 +359,17 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
                     }
                 }
         };
+        // infinities, NaN and what rounds to infinity in bfloat16 show in the sums, 0 times a number that is none; looked at
+        // whenever the sums leave the registers (columns from d on are zeros there)
+        float zero = 0.f;
+        auto look = [&]() {
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                if (wanted(t) && col + c_half + 16 * t < a.d) {
+#pragma unroll
+                    for (int e = 16 * t; e < 16 * t + 16; ++e) zero = fmaf(sum[e], 0.f, zero);
+                }
+        };
         int held = 0;
         bool stored = false;
         for (int c = 0; c < nchunks; ++c) {
@@ -378,6 +389,7 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster_smem(leader_acc_empty0 + (uint32_t)(buf * sizeof(uint64_t)));
             if (++held == EX_LEVEL) {
+                look();
                 store(stored);
                 stored = true;
                 held = 0;
@@ -394,14 +406,7 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
             asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(tiny[r]) : "r"(map_to_cta(smem_u32(tiny_seen), (uint32_t)r)));
         const int i = row + row0 + lane, t = (int)threadIdx.x - 32 * EX_EPI_WARP;
         const int64_t n0 = (int64_t)c_begin * KROWS, n1 = (int64_t)c_end * KROWS < a.N ? (int64_t)c_end * KROWS : a.N;
-        // infinities, NaN and what rounds to infinity in bfloat16 show in the sums: 0 times a number that is none
-        float zero = 0.f;
-#pragma unroll
-        for (int g = 0; g < 8; ++g)
-            if (wanted(g) && col + c_half + 16 * g < a.d) {       // columns from d on are zeros there
-#pragma unroll
-                for (int e = 16 * g; e < 16 * g + 16; ++e) zero = fmaf(sum[e], 0.f, zero);
-            }
+        look();
         bool again = zero != 0.f && row0 < rows && i < a.d;
         if ((tiny[0] | tiny[1]) != 0) {
             // tiny values matter in a column that has no others

@@ -1467,3 +1467,39 @@ def test_moment2_f32_workspace_for_the_fma_kernels_alone(st):
     rc = st.lib().st_sym_moment2(Xd.data_ptr(), st.ST_F32, N, d, d, out.data_ptr(), ws.data_ptr(), 1 << 20, 0,
                                  torch.cuda.current_stream().cuda_stream)
     assert rc == st.ST_ERR_WORKSPACE
+
+
+def moment2_in_64_bits(X):
+    """Packed second moment and sums of |terms| on the GPU in fp64; infinities and NaN as the arithmetic has them."""
+    D = X.double()
+    iu = torch.triu_indices(X.shape[1], X.shape[1], device="cuda")
+    T = (D.T @ D)[iu[0], iu[1]]
+    D = torch.where(D.isfinite(), D.abs(), 0.0)
+    return T, (D.T @ D)[iu[0], iu[1]]
+
+
+def assert_moment2_as_fp32_arithmetic_has_it(got, X, tol):
+    """NaN and infinities where they belong, every other sum within tol of its |terms| (below 2^-126 numbers are 2^-149 apart)."""
+    got = got.double()
+    T, S = moment2_in_64_bits(X)
+    T = torch.where((T.abs() > 3.4028235e38) & ~T.isnan(), torch.sign(T) * math.inf, T)
+    assert torch.equal(got.isnan(), T.isnan())
+    assert torch.equal(got == math.inf, T == math.inf) and torch.equal(got == -math.inf, T == -math.inf)
+    fin = T.isfinite()
+    excess = (got[fin] - T[fin]).abs() - tol * S[fin] - X.shape[0] * 2.0 ** -149
+    assert excess.max() <= 0, float(excess.max())
+
+
+# More than 8192 samples to a cluster, whose sums leave the registers every 8192.  Per element: as TOL_EXACT, with up to 360 sums of
+# 32 samples and partial tiles: 360 * 2^-24 and the 2^-22 and 3 * 2^-27 of the parts.
+@pytest.mark.parametrize("N,d", [(8192, 4096), (9000, 4096), (262144, 512)])
+def test_moment2_f32_exact_parts_of_long_sample_ranges(st, N, d):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N + d)
+    X = torch.randn((N, d), generator=g, device="cuda")
+    assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(X), X, 2.2e-5)
+    # early in the range: infinities, NaN and a number that rounds to infinity in bf16, in a sample that keeps its products finite
+    X[10] *= 0.1
+    X[10, 20] = 3.395e38
+    X[40, 3], X[50, d - 10], X[60, 300] = math.inf, math.nan, -math.inf
+    assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(X), X, TOL_F32)
