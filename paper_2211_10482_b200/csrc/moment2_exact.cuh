@@ -14,8 +14,9 @@
 // of the issue slots of a scheduler, whose loads wait behind the tensor core's.  [65536,512] 370 us with fp32 FMAs, here 122;
 // [65536,256] 112 and 44; [4096,2048] 374 and 104.  Tried: four converting warps (139 at [65536,512]), two groups of four on
 // alternate stages (152), polls by one lane (148), the mixed-precision subtraction (134 instead of 131).
-// Values whose parts are not all bfloat16 numbers (infinities, NaN, |x| > 2^127.99, columns of |x| < 2^-100) give the samples of
-// the cluster that meets them to plain fp32 FMAs.
+// Infinities, NaN and |x| > 2^127.99 have no parts and make a sum that is no number; of |x| < 2^-102 parts may be lost or subnormal.
+// A cluster that meets either looks its samples through, and gives them to plain fp32 FMAs if a sum is no number though neither of
+// its columns has a NaN, or if tiny values may have lost more than 2^-25 of it.
 #pragma once
 #include <atomic>
 #include <type_traits>
@@ -37,7 +38,8 @@ constexpr int EX_MAX_STAGES = 8, EX_BOXES = 52;
 __device__ constexpr int EX_STAGES[5] = {0, 8, 5, 3, 3}, EX_RAW_STAGES[5] = {0, 8, 5, 4, 2};
 constexpr int EX_LEVEL = 256;                          // phases that are added before the sum goes to the partial tile
 constexpr int EX_SQUARES = 2 * EX_CONV_WARPS;          // parts of a column's sum of squares
-constexpr uint32_t EX_TINY = 0x0D80;                   // 2^-100 in bfloat16
+constexpr uint32_t EX_TINY = 2 * (25u << 23) - 1;      // 2 |x| - 1 of 2^-102, in bits; of zero it is the largest
+constexpr float EX_LOST = 0x1p-125f;                   // most that the parts of a number below it can lack
 constexpr int EX_AGAIN = 64;                           // samples at a time of the FMA path
 constexpr size_t EX_SMEM = 1024 + (size_t)EX_BOXES * 4096 + 512 + (size_t)EX_SQUARES * HALF * sizeof(float);
 static_assert((size_t)EX_AGAIN * (HALF + BN) * sizeof(float) <= (size_t)EX_BOXES * 4096, "the FMA path reuses the stages");
@@ -46,12 +48,6 @@ static_assert((size_t)EX_AGAIN * (HALF + BN) * sizeof(float) <= (size_t)EX_BOXES
 template <int REGS> __device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS)); }
 template <int REGS> __device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS)); }
 
-// The halves' minimum, as signed numbers.
-__device__ __forceinline__ uint32_t ex_min_s16x2(uint32_t a, uint32_t b)
-{
-    asm("min.s16x2 %0, %0, %1;" : "+r"(a) : "r"(b));
-    return a;
-}
 // x += y and x -= y for two fp32 numbers at a time (y: their bits).
 __device__ __forceinline__ uint64_t ex_pack2(uint32_t lo, uint32_t hi)
 {
@@ -176,10 +172,9 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
         // of row r0; row r0 + 2h: 256 h further, and bits 5 and 6, where the swizzle puts bits 1 and 2 of the row, exclusive-or h
         const uint32_t from0 = (uint32_t)(warp * RPW / 8 * 1024 + (c4 >> 5) * BOX_BYTES + r0 * 128 + ((((c4 >> 2) & 7) ^ r0) << 4));
         const uint32_t to0 = (uint32_t)(warp * RPW / 8 * 1024 + r0 * 128 + (((c4 >> 3) ^ r0) << 4) + (c4 & 4) * 2);
-        uint32_t least[2] = {0x7FFF7FFFu, 0x7FFF7FFFu};           // two smallest |hi| - 2^15 - 1 each; zeros come out as the largest
+        uint32_t least[2] = {~0u, ~0u};                                     // smallest 2 |x| - 1, as bits: zeros come out as the largest
         auto convert = [&](auto diag_tag) {
             constexpr bool DIAG = decltype(diag_tag)::value;
-            const int own = na > 0 ? 1 : 0;                       // the side that holds the columns of this block's rows
             float square[8] = {};
             // Items of a stage: 64 columns of B, the other 64 of B, of A, of A, whichever this block has.  The loads of an item are
             // issued before the one ahead of it is converted.
@@ -219,8 +214,8 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
                     }
                     const bool store = there(item);
                     unsigned char *w = smem + s * stage_bytes + (item < qb ? item : tb + item - qb) * BOX_BYTES;
-                    if (DIAG && (item < qb) == (own == 0)) {
-                        const bool upper = (item < qb ? item : item - qb) != 0;
+                    if (DIAG && item < qb) {                          // B holds the columns of a diagonal block's rows
+                        const bool upper = item != 0;
 #pragma unroll
                         for (int h = 0; h < H; ++h)
 #pragma unroll
@@ -244,7 +239,8 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
 #pragma unroll
                             for (int h = 0; h < H; ++h)
 #pragma unroll
-                                for (int e = 0; e < 2; ++e) least[e] = ex_min_s16x2(least[e], (b[h][e] & 0x7FFF7FFFu) + 0x7FFF7FFFu);
+                                for (int e = 0; e < 2; ++e)
+                                    least[e] = __vimin3_u32(least[e], 2 * __float_as_uint(rest[h][2 * e]) - 1, 2 * __float_as_uint(rest[h][2 * e + 1]) - 1);
                         }
                         if (store) {
 #pragma unroll
@@ -279,8 +275,7 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
         };
         if (diag) convert(std::integral_constant<bool, true>{});
         else convert(std::integral_constant<bool, false>{});
-        least[0] = ex_min_s16x2(least[0], least[1]) ^ 0x80008000u;
-        if ((least[0] & 0xFFFFu) < EX_TINY - 1u || least[0] >> 16 < EX_TINY - 1u) atomicOr(tiny_seen, 1u);
+        if (min(least[0], least[1]) < EX_TINY) atomicOr(tiny_seen, 1u);
     } else if (warp < EX_EPI_WARP) {
         regs_down<EX_REGS_MAIN>();
         if (warp == EX_COPY_WARP && elect_one()) {
@@ -397,6 +392,8 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
                 for (int e = 0; e < 128; ++e) sum[e] = 0.f;
             }
         }
+        look();
+        store(stored);
         // every value of the pair's samples has been looked at when the converting warps have arrived here
         __syncthreads();
         cluster_sync_all();
@@ -406,65 +403,121 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
             asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(tiny[r]) : "r"(map_to_cta(smem_u32(tiny_seen), (uint32_t)r)));
         const int i = row + row0 + lane, t = (int)threadIdx.x - 32 * EX_EPI_WARP;
         const int64_t n0 = (int64_t)c_begin * KROWS, n1 = (int64_t)c_end * KROWS < a.N ? (int64_t)c_end * KROWS : a.N;
-        look();
-        bool again = zero != 0.f && row0 < rows && i < a.d;
-        if ((tiny[0] | tiny[1]) != 0) {
-            // tiny values matter in a column that has no others
-            float most_a = 0.f, most_b = 0.f;
-            const int ca = col_a + (t & (HALF - 1)), cb = col + t;
-#pragma unroll 8
-            for (int64_t n = n0; n < n1; ++n) {
-                if (ca < a.d && ca < row + rows) most_a = fmaxf(most_a, fabsf(a.X[n * a.ldx + ca]));
-                if (cb < a.d && t < width) most_b = fmaxf(most_b, fabsf(a.X[n * a.ldx + cb]));
+        if ((tiny[0] | tiny[1]) != 0 || ex_any(zero != 0.f && row0 < rows && i < a.d)) {
+            // of the rows' columns and the tile's the largest |x| and the smallest 2 |x| - 1, as bits
+            uint32_t *most = reinterpret_cast<uint32_t *>(smem), *least = most + HALF + BN;
+            for (int k = t; k < HALF + BN; k += EX_EPI_THREADS) {
+                most[k] = 0;
+                least[k] = ~0u;
             }
-            again = again || (most_a > 0.f && most_a < 0x1p-100f) || (most_b > 0.f && most_b < 0x1p-100f);
-        }
-        again = ex_any(again);
-        if (again) {
-            // these samples once more, with fp32 FMAs
+            ex_any(false);
+            // Columns of a side (of the tile: 0, of the block's rows: 1, unless the tile's hold them), four to a thread; all samples,
+            // `step` at a time.
+            auto side_first = [&](int side) { return side ? col_a : col; };
+            auto side_quads = [&](int side) {
+                const int n = side ? min(HALF, rows - (int)rank * HALF) : width;
+                return (min(n, a.d - side_first(side)) + 3) / 4;
+            };
+            for (int side = 0; side < (diag ? 1 : 2); ++side) {
+                const int quads = side_quads(side);
+                if (quads <= 0) continue;
+                const int step = EX_EPI_THREADS / quads, r = t / quads, q = t % quads;
+                uint32_t m[4] = {0, 0, 0, 0}, l[4] = {~0u, ~0u, ~0u, ~0u};
+                constexpr int U = 16;
+                for (int64_t n = n0 + r; r < step && n < n1; n += U * step) {
+                    uint4 v[U];
 #pragma unroll
-            for (int e = 0; e < 128; ++e) sum[e] = 0.f;
-            stored = false;
-            float *xa = reinterpret_cast<float *>(smem), *xb = xa + EX_AGAIN * HALF;
-            for (int64_t n = n0; n < n1; n += EX_AGAIN) {
-                const int count = n1 - n < EX_AGAIN ? (int)(n1 - n) : EX_AGAIN;
-                ex_any(false);                                    // the samples before these have been read
-                for (int k0 = 0; k0 < count; k0 += 8) {           // the loads of eight samples in front of their stores
-                    float va[8], vb[8];
+                    for (int k = 0; k < U; ++k)
+                        v[k] = n + k * step < n1 ? *reinterpret_cast<const uint4 *>(a.X + (n + k * step) * a.ldx + side_first(side) + 4 * q) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const float *x = a.X + (n + k0 + k) * a.ldx;
-                        const bool in = k0 + k < count;
-                        va[k] = in && t < HALF && col_a + t < a.d ? x[col_a + t] : 0.f;
-                        vb[k] = in && t < width && col + t < a.d ? x[col + t] : 0.f;
-                    }
+                    for (int k = 0; k < U; ++k) {
+                        const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        if (t < HALF) xa[(k0 + k) * HALF + t] = va[k];
-                        xb[(k0 + k) * BN + t] = vb[k];
-                    }
-                }
-                ex_any(false);
-#pragma unroll 2
-                for (int k = 0; k < count; ++k) {
-                    const float xi = xa[k * HALF + (warp & 3) * 32 + lane];
-                    const float4 *xj = reinterpret_cast<const float4 *>(xb + k * BN + c_half);
-#pragma unroll
-                    for (int e = 0; e < 128; e += 4)
-                        if (e < half) {
-                            const float4 v = xj[e / 4];
-                            sum[e] = fmaf(xi, v.x, sum[e]);
-                            sum[e + 1] = fmaf(xi, v.y, sum[e + 1]);
-                            sum[e + 2] = fmaf(xi, v.z, sum[e + 2]);
-                            sum[e + 3] = fmaf(xi, v.w, sum[e + 3]);
+                        for (int e = 0; e < 4; ++e) {
+                            m[e] = max(m[e], w[e] & 0x7FFFFFFFu);
+                            l[e] = min(l[e], 2 * w[e] - 1);
                         }
+                    }
+                }
+                const int at = (side ? 0 : HALF) + 4 * q;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    atomicMax(most + at + e, m[e]);
+                    atomicMin(least + at + e, l[e]);
                 }
             }
+            ex_any(false);
+            // Which sums: no number, though neither column has a NaN; or what the parts of a column lack, times the largest value of
+            // the other in every sample, is more than 2^-25 of the sum.
+            const float lost = (float)(n1 - n0) * (EX_LOST * 0x1p25f);
+            const int own = (diag ? HALF + (int)rank * HALF : 0) + (warp & 3) * 32 + lane;
+            const uint32_t most_row = most[own];
+            const bool tiny_row = least[own] < EX_TINY, nan_row = most_row > 0x7F800000u;
+            bool again = false;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                float4 v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    v[q] = wanted(2 * w + q / 4) ? *reinterpret_cast<const float4 *>(dst + (c_half + 32 * w + 4 * q) * HALF) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                    const int c = 32 * w + e;
+                    if (!wanted(c >> 4) || i >= a.d || col + c_half + c >= a.d || i == col + c_half + c) continue;    // squares: below
+                    const float4 f = v[e / 4];
+                    const float s = fabsf(e % 4 == 0 ? f.x : e % 4 == 1 ? f.y : e % 4 == 2 ? f.z : f.w);
+                    const uint32_t most_col = most[HALF + c_half + c];
+                    const bool tiny_col = least[HALF + c_half + c] < EX_TINY;
+                    const float may_lack = (tiny_row ? lost : 0.f) * __uint_as_float(most_col) + (tiny_col ? lost : 0.f) * __uint_as_float(most_row);
+                    const bool poor = (tiny_row || tiny_col) && !(s >= may_lack);
+                    again = again || (!nan_row && most_col <= 0x7F800000u && (poor || !(s <= 0x1.fffffep127f)));
+                }
+            }
+            if (ex_any(again)) {
+                // these samples once more, with fp32 FMAs
+#pragma unroll
+                for (int e = 0; e < 128; ++e) sum[e] = 0.f;
+                float *xa = reinterpret_cast<float *>(smem), *xb = xa + EX_AGAIN * HALF;
+                for (int64_t n = n0; n < n1; n += EX_AGAIN) {
+                    const int count = n1 - n < EX_AGAIN ? (int)(n1 - n) : EX_AGAIN;
+                    ex_any(false);                                    // the samples before these have been read
+                    for (int k0 = 0; k0 < count; k0 += 8) {           // the loads of eight samples in front of their stores
+                        float va[8], vb[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const float *x = a.X + (n + k0 + k) * a.ldx;
+                            const bool in = k0 + k < count;
+                            va[k] = in && t < HALF && col_a + t < a.d ? x[col_a + t] : 0.f;
+                            vb[k] = in && t < width && col + t < a.d ? x[col + t] : 0.f;
+                        }
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            if (t < HALF) xa[(k0 + k) * HALF + t] = va[k];
+                            xb[(k0 + k) * BN + t] = vb[k];
+                        }
+                    }
+                    ex_any(false);
+#pragma unroll 2
+                    for (int k = 0; k < count; ++k) {
+                        const float xi = xa[k * HALF + (warp & 3) * 32 + lane];
+                        const float4 *xj = reinterpret_cast<const float4 *>(xb + k * BN + c_half);
+#pragma unroll
+                        for (int e = 0; e < 128; e += 4)
+                            if (e < half) {
+                                const float4 v = xj[e / 4];
+                                sum[e] = fmaf(xi, v.x, sum[e]);
+                                sum[e + 1] = fmaf(xi, v.y, sum[e + 1]);
+                                sum[e + 2] = fmaf(xi, v.z, sum[e + 2]);
+                                sum[e + 3] = fmaf(xi, v.w, sum[e + 3]);
+                            }
+                    }
+                }
+                store(false);
+            }
         }
-        store(stored);
         // the sums of squares take their places on the diagonal
         const int o = i - row;
-        if (!again && diag && row0 < rows && i < a.d && o >= c_half && o < c_half + half) {
+        if (diag && row0 < rows && i < a.d && o >= c_half && o < c_half + half) {
             float total = 0.f;
 #pragma unroll
             for (int p = 0; p < EX_SQUARES; ++p) total += squares[p * HALF + (warp & 3) * 32 + lane];

@@ -1503,3 +1503,26 @@ def test_moment2_f32_exact_parts_of_long_sample_ranges(st, N, d):
     X[10, 20] = 3.395e38
     X[40, 3], X[50, d - 10], X[60, 300] = math.inf, math.nan, -math.inf
     assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(X), X, TOL_F32)
+
+
+# Numbers without exact parts (below 2^-109 they have bits below 2^-133) beside a column that is zero or small in the other samples:
+# these terms are the whole sum.  Per element as above.
+@pytest.mark.parametrize("whole", [False, True])
+@pytest.mark.parametrize("N,d", [(4100, 260), (2100, 400), (12000, 128)])
+def test_moment2_f32_tiny_values_beside_sparse_columns(st, N, d, whole):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    X = torch.randn((N, d), generator=g, device="cuda")
+    signs = torch.sign(torch.randn((N, d), generator=g, device="cuda"))
+    rows = torch.arange(N, device="cuda") % 5 == 0
+    for k, v in enumerate((1e-33, 1.3e-36, 1.1e-38, 2.1e-40, 4.3e-41, 1.4e-45)):
+        X[:, 3 * k] = torch.where(rows, v * signs[:, k], X[:, 3 * k])             # tiny in every fifth sample
+        X[:, 3 * k + 1] = torch.where(rows, (1e12 if k else 1e17) * signs[:, k + 60], 0.0)        # large there, zero in the others
+        X[:, d - 2 - 3 * k] = torch.where(rows, 1e9 * signs[:, k + 90], 1e-12)
+        if whole:
+            X[:, d - 1 - 3 * k] = torch.where(rows, v * signs[:, k + 30], 0.0)    # nothing but tiny
+    X[:, 40:43] *= 1e-20                                                          # sums below 2^-126
+    if whole:
+        X[:, 43] *= 1e-36
+    X[7::100, 44] = 0.0
+    assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(X), X, 2.2e-5)
