@@ -15,8 +15,11 @@
 // [65536,256] 112 and 44; [4096,2048] 374 and 104.  Tried: four converting warps (139 at [65536,512]), two groups of four on
 // alternate stages (152), polls by one lane (148), the mixed-precision subtraction (134 instead of 131).
 // Infinities, NaN and |x| > 2^127.99 have no parts and make a sum that is no number; of |x| < 2^-102 parts may be lost or subnormal.
-// A cluster that meets either looks its samples through, and gives them to plain fp32 FMAs if a sum is no number though neither of
-// its columns has a NaN, or if tiny values may have lost more than 2^-25 of it.
+// A cluster that meets either looks its samples through, and adds once more, with fp32 FMAs, the sums that are no number though
+// neither of their columns has a NaN, and those of which tiny values may have lost more than 2^-25: lines (rows or columns of the
+// tile) that hold such sums, or where there are many of them the whole tile.  [65536,512], us, 371 with FMA kernels whatever the
+// values: 121 with ordinary ones, 230 with a |x| of 1e-38 or a NaN among them, 364 with infinities in one to four columns, 526 in
+// sixteen, 935 where one value in a hundred is one (all samples to 256 threads with a row each: 3640 with any of these).
 #pragma once
 #include <atomic>
 #include <type_traits>
@@ -40,9 +43,13 @@ constexpr int EX_LEVEL = 256;                          // phases that are added 
 constexpr int EX_SQUARES = 2 * EX_CONV_WARPS;          // parts of a column's sum of squares
 constexpr uint32_t EX_TINY = 2 * (25u << 23) - 1;      // 2 |x| - 1 of 2^-102, in bits; of zero it is the largest
 constexpr float EX_LOST = 0x1p-125f;                   // most that the parts of a number below it can lack
-constexpr int EX_AGAIN = 64;                           // samples at a time of the FMA path
+constexpr int EX_LINES = 8, EX_MOST_LINES = 64;        // lines of a pass over the samples; from where the whole tile takes less
+constexpr int EX_FEW = 32;                             // sums of half a row that are left to their columns, if no more than half of them
+constexpr int EX_AGAIN = 64;                           // samples at a time of the whole tile, two of them in shared memory
+constexpr int EX_AGAIN_FLOATS = EX_AGAIN * (HALF + BN);
 constexpr size_t EX_SMEM = 1024 + (size_t)EX_BOXES * 4096 + 512 + (size_t)EX_SQUARES * HALF * sizeof(float);
-static_assert((size_t)EX_AGAIN * (HALF + BN) * sizeof(float) <= (size_t)EX_BOXES * 4096, "the FMA path reuses the stages");
+static_assert((2 * (size_t)EX_AGAIN_FLOATS + 2 * (HALF + BN) + 12) * sizeof(float) <= (size_t)EX_BOXES * 4096, "the FMA path reuses the stages");
+static_assert(EX_LINES * EX_EPI_THREADS * 4 <= 2 * EX_AGAIN_FLOATS, "the sums of a pass take the place of the samples");
 }  // namespace m2tc
 
 template <int REGS> __device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS)); }
@@ -404,12 +411,15 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
         const int i = row + row0 + lane, t = (int)threadIdx.x - 32 * EX_EPI_WARP;
         const int64_t n0 = (int64_t)c_begin * KROWS, n1 = (int64_t)c_end * KROWS < a.N ? (int64_t)c_end * KROWS : a.N;
         if ((tiny[0] | tiny[1]) != 0 || ex_any(zero != 0.f && row0 < rows && i < a.d)) {
-            // of the rows' columns and the tile's the largest |x| and the smallest 2 |x| - 1, as bits
-            uint32_t *most = reinterpret_cast<uint32_t *>(smem), *least = most + HALF + BN;
+            // two buffers of samples (64 x 128 values of the rows' columns, 64 x 256 of the tile's); of the rows' columns and the
+            // tile's the largest |x| and the smallest 2 |x| - 1, as bits; lines
+            float *panels = reinterpret_cast<float *>(smem), *block = a.partials + (size_t)blockIdx.x * HALF * BN;
+            uint32_t *most = reinterpret_cast<uint32_t *>(panels + 2 * EX_AGAIN_FLOATS), *least = most + HALF + BN, *lines = least + HALF + BN;
             for (int k = t; k < HALF + BN; k += EX_EPI_THREADS) {
                 most[k] = 0;
                 least[k] = ~0u;
             }
+            if (t < 12) lines[t] = 0;
             ex_any(false);
             // Columns of a side (of the tile: 0, of the block's rows: 1, unless the tile's hold them), four to a thread; all samples,
             // `step` at a time.
@@ -453,7 +463,8 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
             const int own = (diag ? HALF + (int)rank * HALF : 0) + (warp & 3) * 32 + lane;
             const uint32_t most_row = most[own];
             const bool tiny_row = least[own] < EX_TINY, nan_row = most_row > 0x7F800000u;
-            bool again = false;
+            uint32_t which[4] = {0, 0, 0, 0};
+            int count = 0, all = 0;
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
                 float4 v[8];
@@ -464,55 +475,146 @@ moment2_exact_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_cons
                 for (int e = 0; e < 32; ++e) {
                     const int c = 32 * w + e;
                     if (!wanted(c >> 4) || i >= a.d || col + c_half + c >= a.d || i == col + c_half + c) continue;    // squares: below
+                    ++all;
                     const float4 f = v[e / 4];
                     const float s = fabsf(e % 4 == 0 ? f.x : e % 4 == 1 ? f.y : e % 4 == 2 ? f.z : f.w);
                     const uint32_t most_col = most[HALF + c_half + c];
                     const bool tiny_col = least[HALF + c_half + c] < EX_TINY;
                     const float may_lack = (tiny_row ? lost : 0.f) * __uint_as_float(most_col) + (tiny_col ? lost : 0.f) * __uint_as_float(most_row);
                     const bool poor = (tiny_row || tiny_col) && !(s >= may_lack);
-                    again = again || (!nan_row && most_col <= 0x7F800000u && (poor || !(s <= 0x1.fffffep127f)));
+                    if (!nan_row && most_col <= 0x7F800000u && (poor || !(s <= 0x1.fffffep127f))) {
+                        which[w] |= 1u << e;
+                        ++count;
+                    }
                 }
             }
-            if (ex_any(again)) {
-                // these samples once more, with fp32 FMAs
+            // Their lines: rows of the block (four words; on the diagonal the columns that they are too), columns of the tile (eight)
+            if (count > EX_FEW || 2 * count > all) {
+                atomicOr(lines + (diag ? 4 + 4 * (int)rank : 0) + (warp & 3), 1u << lane);
+            } else if (count > 0) {
 #pragma unroll
-                for (int e = 0; e < 128; ++e) sum[e] = 0.f;
-                float *xa = reinterpret_cast<float *>(smem), *xb = xa + EX_AGAIN * HALF;
-                for (int64_t n = n0; n < n1; n += EX_AGAIN) {
-                    const int count = n1 - n < EX_AGAIN ? (int)(n1 - n) : EX_AGAIN;
-                    ex_any(false);                                    // the samples before these have been read
-                    for (int k0 = 0; k0 < count; k0 += 8) {           // the loads of eight samples in front of their stores
-                        float va[8], vb[8];
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const float *x = a.X + (n + k0 + k) * a.ldx;
-                            const bool in = k0 + k < count;
-                            va[k] = in && t < HALF && col_a + t < a.d ? x[col_a + t] : 0.f;
-                            vb[k] = in && t < width && col + t < a.d ? x[col + t] : 0.f;
-                        }
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            if (t < HALF) xa[(k0 + k) * HALF + t] = va[k];
-                            xb[(k0 + k) * BN + t] = vb[k];
-                        }
+                for (int w = 0; w < 4; ++w)
+                    if (which[w] != 0) {
+                        // columns c_half + 32 w ..: they straddle two words where a half is no multiple of 32
+                        const int c = c_half + 32 * w;
+                        atomicOr(lines + 4 + c / 32, which[w] << (c & 31));
+                        if ((c & 31) != 0) atomicOr(lines + 4 + c / 32 + 1, which[w] >> (32 - (c & 31)));
                     }
-                    ex_any(false);
-#pragma unroll 2
-                    for (int k = 0; k < count; ++k) {
-                        const float xi = xa[k * HALF + (warp & 3) * 32 + lane];
-                        const float4 *xj = reinterpret_cast<const float4 *>(xb + k * BN + c_half);
+            }
+            ex_any(false);
+            int line_rows = 0, line_cols = 0;
 #pragma unroll
-                        for (int e = 0; e < 128; e += 4)
-                            if (e < half) {
-                                const float4 v = xj[e / 4];
-                                sum[e] = fmaf(xi, v.x, sum[e]);
-                                sum[e + 1] = fmaf(xi, v.y, sum[e + 1]);
-                                sum[e + 2] = fmaf(xi, v.z, sum[e + 2]);
-                                sum[e + 3] = fmaf(xi, v.w, sum[e + 3]);
+            for (int w = 0; w < 12; ++w) (w < 4 ? line_rows : line_cols) += __popc(lines[w]);
+            if (line_rows + line_cols <= EX_MOST_LINES) {
+                // x of EX_LINES lines times x of the columns across them; on the diagonal across all of the tile's
+                for (int side = 0; side < 2; ++side) {
+                    const int total = side ? line_cols : line_rows, words = side ? 8 : 4, across = diag ? 0 : side, quads = side_quads(across);
+                    if (total == 0 || quads <= 0) continue;
+                    const uint32_t *set = side ? lines + 4 : lines;
+                    auto line = [&](int k) {                      // the k-th one
+                        int w = 0, n = __popc(set[0]);
+                        while (k >= n && w + 1 < words) { k -= n; n = __popc(set[++w]); }
+                        return k < n ? 32 * w + (int)__fns(set[w], 0, k + 1) : 0;
+                    };
+                    const int step = EX_EPI_THREADS / quads, r = t / quads, q = t % quads;
+                    for (int first = 0; first < total; first += EX_LINES) {
+                        int from[EX_LINES];                       // column of a line less the ones across it
+                        float acc[EX_LINES][4] = {};
+#pragma unroll
+                        for (int l = 0; l < EX_LINES; ++l)
+                            from[l] = side_first(1 - side) + line(first + l < total ? first + l : first) - side_first(across) - 4 * q;
+                        if (r < step) {
+                            const float *x = a.X + (n0 + r) * a.ldx + side_first(across) + 4 * q;
+#pragma unroll 4
+                            for (int64_t n = n0 + r; n < n1; n += step, x += step * a.ldx) {
+                                const float4 v = *reinterpret_cast<const float4 *>(x);
+#pragma unroll
+                                for (int l = 0; l < EX_LINES; ++l) {
+                                    const float y = x[from[l]];
+                                    acc[l][0] = fmaf(y, v.x, acc[l][0]);
+                                    acc[l][1] = fmaf(y, v.y, acc[l][1]);
+                                    acc[l][2] = fmaf(y, v.z, acc[l][2]);
+                                    acc[l][3] = fmaf(y, v.w, acc[l][3]);
+                                }
                             }
+#pragma unroll
+                            for (int l = 0; l < EX_LINES; ++l)
+                                *reinterpret_cast<float4 *>(panels + ((l * step + r) * quads + q) * 4) = make_float4(acc[l][0], acc[l][1], acc[l][2], acc[l][3]);
+                        }
+                        ex_any(false);
+                        for (int k = t; k < EX_LINES * 4 * quads; k += EX_EPI_THREADS) {
+                            const int l = k / (4 * quads), o = k % (4 * quads);
+                            if (first + l >= total) break;
+                            float total_sum = 0.f;
+                            for (int p = 0; p < step; ++p) total_sum += panels[(l * step + p) * quads * 4 + o];
+                            const int at = line(first + l);
+                            auto put = [&](int r, int c) {
+                                if (r >= 0 && r < HALF) block[(c & ~3) * HALF + r * 4 + (c & 3)] = total_sum;
+                            };
+                            if (!diag) {
+                                put(side ? o : at, side ? at : o);
+                            } else {
+                                put(o - (int)rank * HALF, at);
+                                put(at - (int)rank * HALF, o);
+                            }
+                        }
+                        ex_any(false);
                     }
                 }
-                store(false);
+            } else {
+                // the whole tile: a thread has eight rows and, of each 32 columns of its half of 128, four
+                // EX_AGAIN samples at a time (zeros past the end): body(rows' columns, tile's columns)
+                auto samples = [&](auto body) {
+                    auto fetch = [&](int64_t n, int buf) {
+                        const uint32_t xa = smem_u32(panels + buf * EX_AGAIN_FLOATS), xb = xa + EX_AGAIN * HALF * 4;
+                        for (int k = t; k < EX_AGAIN * (HALF + BN) / 4; k += EX_EPI_THREADS) {
+                            const bool is_a = k < EX_AGAIN * HALF / 4;
+                            const int u = is_a ? k : k - EX_AGAIN * HALF / 4, r = is_a ? u / (HALF / 4) : u / (BN / 4), c = 4 * (is_a ? u % (HALF / 4) : u % (BN / 4));
+                            const int gc = (is_a ? col_a : col) + c;
+                            const bool in = n + r < n1 && gc < a.d && (is_a || c < width);
+                            const float *src = in ? a.X + (n + r) * a.ldx + gc : a.X;
+                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((is_a ? xa : xb) + 16u * (uint32_t)u), "l"(src), "r"(in ? 16 : 0) : "memory");
+                        }
+                        asm volatile("cp.async.commit_group;" ::: "memory");
+                    };
+                    int buf = 0;
+                    fetch(n0, 0);
+                    for (int64_t n = n0; n < n1; n += EX_AGAIN, buf ^= 1) {
+                        fetch(n + EX_AGAIN, buf ^ 1);
+                        asm volatile("cp.async.wait_group 1;" ::: "memory");
+                        ex_any(false);
+                        body(panels + buf * EX_AGAIN_FLOATS, panels + buf * EX_AGAIN_FLOATS + EX_AGAIN * HALF);
+                        ex_any(false);
+                    }
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                };
+                const int ra = (warp & 3) * 32 + (lane >> 3) * 8, cb = (warp >= EX_EPI_WARP + 4 ? HALF : 0) + (lane & 7) * 4;
+                uint64_t acc[8][8] = {};
+                samples([&](const float *xa, const float *xb) {
+#pragma unroll 1
+                    for (int k = 0; k < EX_AGAIN; ++k) {
+                        const float4 a0 = *reinterpret_cast<const float4 *>(xa + k * HALF + ra), a1 = *reinterpret_cast<const float4 *>(xa + k * HALF + ra + 4);
+                        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+                        ulonglong2 b[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) b[q] = *reinterpret_cast<const ulonglong2 *>(xb + k * BN + cb + 32 * q);
+#pragma unroll
+                        for (int r = 0; r < 8; ++r) {
+                            const uint64_t aa = ex_pack2(__float_as_uint(av[r]), __float_as_uint(av[r]));
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[r][2 * q]) : "l"(aa), "l"(b[q].x));
+                                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[r][2 * q + 1]) : "l"(aa), "l"(b[q].y));
+                            }
+                        }
+                    }
+                });
+#pragma unroll
+                for (int r = 0; r < 8; ++r)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        *reinterpret_cast<ulonglong2 *>(block + (cb + 32 * q) * HALF + (ra + r) * 4) = make_ulonglong2(acc[r][2 * q], acc[r][2 * q + 1]);
+                ex_any(false);
             }
         }
         // the sums of squares take their places on the diagonal

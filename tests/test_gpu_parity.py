@@ -1526,3 +1526,26 @@ def test_moment2_f32_tiny_values_beside_sparse_columns(st, N, d, whole):
         X[:, 43] *= 1e-36
     X[7::100, 44] = 0.0
     assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(X), X, 2.2e-5)
+
+
+# Sums that are added once more: a few rows and columns of a tile, more than a pass takes, more than are taken one by one; in
+# tiles of all 256 columns, of four, and of an odd number of steps.
+@pytest.mark.parametrize("N,d", [(4100, 260), (3300, 396), (2300, 512), (12000, 128), (9000, 140)])
+@pytest.mark.parametrize("columns", [1, 3, 20, 100])
+def test_moment2_f32_sums_added_once_more(st, N, d, columns):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + columns)
+    X = torch.randn((N, d), generator=g, device="cuda")
+    which = torch.randperm(d, generator=g, device="cuda")[:columns]
+    Y = X.clone()
+    Y[:, which] *= 1e-36
+    assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(Y), Y, 2.2e-5)
+    Y = X.abs() + 0.5
+    Y[N // 2] *= 0.1                   # no product of the huge value leaves the range of fp32 but its square
+    Y[:, which] = -math.inf
+    Y[N // 2, (which[0] + 5) % d] = 3.395e38
+    assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(Y), Y, TOL_F32)
+    Y = X.clone()
+    Y[torch.randint(N, (columns,), generator=g, device="cuda"), which] = math.inf
+    Y[torch.randint(N, (columns,), generator=g, device="cuda"), which] = math.nan
+    assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(Y), Y, 2.2e-5)
