@@ -254,8 +254,9 @@ moment3_tc_kernel(const __grid_constant__ Args a)
         // ---- MMA issuers: two warps.  A barrier poll issued behind tcgen05.mma instructions of the same thread
         // returns only as they drain, so one issuer alone leaves the tensor pipe idle while it polls.
         // A ring slot q % NA has the parity of q (NA is even), so every slot has one issuer and its uses are polled in
-        // order.  The MMAs of slice 0 overwrite the accumulators: both issuers wait until all of them are complete
-        // before either adds slice 1, after which the order of the additions into a tile is free.
+        // order.  An even number of tiles has one issuer each.  Of an odd number every tile changes issuers from slice to
+        // slice, and MMAs of two threads into one accumulator are in no order by themselves: both issuers have then issued
+        // all of a slice before either goes on to the next.
         const int iw = warp - MMA_WARP;
         if (elect_one()) {
             bool ok = true;
@@ -293,9 +294,10 @@ moment3_tc_kernel(const __grid_constant__ Args a)
                 }
                 if (!ok) break;
                 tc_commit(&b_empty[bs]);
-                if (slice == 0 && nslices > 1) {
-                    tc_commit(iss_sync);
-                    if (!mbar_wait(iss_sync, 0u, abort_flag, a.status, 17)) break;
+                if (tg % 2 != 0 && slice + 1 < nslices) {
+                    tc_fence_before();
+                    mbar_arrive(iss_sync);
+                    if (!mbar_wait(iss_sync, (uint32_t)(slice & 1), abort_flag, a.status, 17)) break;
                     tc_fence_after();
                 }
                 if (slice == nslices - 1) tc_commit(acc_full);

@@ -1549,3 +1549,16 @@ def test_moment2_f32_sums_added_once_more(st, N, d, columns):
     Y[torch.randint(N, (columns,), generator=g, device="cuda"), which] = math.inf
     Y[torch.randint(N, (columns,), generator=g, device="cuda"), which] = math.nan
     assert_moment2_as_fp32_arithmetic_has_it(st.st_sym_moment2(Y), Y, 2.2e-5)
+
+
+def test_tensor_core_moments_give_the_same_bits_twenty_times(st):
+    """Blocks of one tile and of an odd number of tiles, whose stages two warps issue, for several slices a block."""
+    X2 = dev(workloads.draw((30000, 260), "normal", 41))
+    calls = [lambda: st.st_sym_moment2(X2)]
+    for N, d in ((40000, 8), (8000, 12), (16000, 16), (40000, 24), (20000, 33), (20000, 50)):
+        X = dev(workloads.draw((N, d), "normal", d))
+        for flags in (st.ST_FLAG_TC_TF32, st.ST_FLAG_TC_BF16):
+            calls.append(lambda X=X, flags=flags: st.st_sym_moment3(X, flags=flags))
+    for fn in calls:
+        first = fn()
+        assert all(torch.equal(first, fn()) for _ in range(20))
