@@ -491,9 +491,11 @@ static Plan plan(int64_t N, int64_t d, bool bf16)
         }
     p.ntiles = n;
     // Groups: the number for which the longest block and the sum after it take least, in cycles: 230 a stage, but 2000 a slice at
-    // least (what fetching and turning it takes), 650 a tile for its partial sums, 60 a slice in the sum.  With 1, 2, 4 and 8
-    // groups, bf16, us: [256,33] 11.2, 9.3, 8.2, 7.6; [4096,33] 11.9, 10.2, 10.0, 10.8; [40009,33] 23.6, 22.5, 26.1, 40.6;
-    // [200000,33] 66, 77, 101, 175.  Before, with as few groups as tensor memory allows: [256,50] 15.1, now 11.2; [256,64] 16.1, 12.1.
+    // least (what fetching and turning it takes), 650 a tile for its partial sums (two at least: one is no faster), 60 a slice in the
+    // sum.  With 1, 2, 4 and 8 groups, bf16, us: [256,33] 11.2, 9.3, 8.2, 7.6; [4096,33] 11.9, 10.2, 10.0, 10.8; [40009,33] 23.6,
+    // 22.5, 26.1, 40.6; [200000,33] 66, 77, 101, 175.  With 1, 2 and 4: [4096,32] 9.5, 8.5, 8.4, TF32 10.6, 9.5, 9.7; [16384,32]
+    // 12.4, 12.4, 12.6, TF32 14.9, 14.8, 16.6; with 1 and 2: [4096,16] 7.4, 7.6, TF32 8.6, 8.3; [40009,16] 11.8, 14.2, TF32 15.7, 19.1.
+    // Before, with as few groups as tensor memory allows: [256,50] 15.1, now 11.2; [256,64] 16.1, 12.1.
     const int sms = sm_count_or_default();
     double best = 0;
     for (int groups = 1; groups <= MAX_GROUPS && groups <= n && groups <= sms; ++groups) {
@@ -510,7 +512,7 @@ static Plan plan(int64_t N, int64_t d, bool bf16)
         if (!fits || longest > MAX_GROUP_TILES) continue;
         int64_t slices = sms / groups, rps = ((N + slices - 1) / slices + KS - 1) / KS * KS;      // whole MMA slices
         slices = (N + rps - 1) / rps;
-        const double cost = (double)(rps / KS) * (longest * 230 > 2000 ? longest * 230 : 2000) + longest * 650 + (double)slices * 60;
+        const double cost = (double)(rps / KS) * (longest * 230 > 2000 ? longest * 230 : 2000) + (longest > 2 ? longest : 2) * 650 + (double)slices * 60;
         if (p.ok && cost >= best) continue;
         best = cost;
         p.groups = groups;
