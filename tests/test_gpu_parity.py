@@ -1562,3 +1562,33 @@ def test_tensor_core_moments_give_the_same_bits_twenty_times(st):
     for fn in calls:
         first = fn()
         assert all(torch.equal(first, fn()) for _ in range(20))
+
+
+# What the exact parts are for: each product of parts counts.  Every pair of columns shares one sample, so that a sum is one product:
+# 2^-23 for each of the two additions that are cut at the grid of the result, 2^-24 for its rounding and 2^-26 for the products
+# that are left out (without lo hi, or mid mid, it would be 2^-18).
+@pytest.mark.parametrize("d", [160, 260, 388])
+def test_moment2_f32_exact_parts_product_by_product(st, d):
+    iu = torch.triu_indices(d, d, 1, device="cuda")
+    N = iu.shape[1]
+    order = torch.randperm(N, generator=torch.Generator().manual_seed(d)).cuda()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    v = torch.randn((2, N), generator=g, device="cuda")
+    X = torch.zeros((N, d), device="cuda")
+    X[order, iu[0]], X[order, iu[1]] = v[0], v[1]
+    got = st.st_unpack(st.st_sym_moment2(X), st.Layout(st.ST_TRI_UPPER, d), fill=st.ST_FILL_SYMMETRIC).view(d, d)[iu[0], iu[1]].double()
+    want = v[0].double() * v[1].double()
+    assert ((got - want).abs() / want.abs()).max() <= 2.6 * 2.0 ** -23
+
+
+# The 2-norm of the error, where fp32 arithmetic alone would have at best 2.5e-8 from the rounding of the results.
+@pytest.mark.parametrize("N,d", [(8192, 256), (65536, 140), (5000, 520)])
+@pytest.mark.parametrize("positive", [False, True])
+def test_moment2_f32_exact_parts_norm_of_the_error(st, N, d, positive):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+    X = torch.rand((N, d), generator=g, device="cuda") if positive else torch.randn((N, d), generator=g, device="cuda")
+    T, _ = moment2_in_64_bits(X)
+    # samples that are all positive: cut at the grid of 32 samples and of 16, by half of 2^-23 and of 2^-24 of the sum on average
+    assert (st.st_sym_moment2(X).double() - T).norm() / T.norm() <= 9e-8

@@ -53,7 +53,7 @@ def test_parity_suite_under_the_range_checks():
         from paper_2211_10482_b200 import _build
         _build.build(check=True)
     select = ("pack_unpack or small or closed_form or mttkrp_config or ttm_config or moment3_config or moment4 or "
-              "slice or structure or thp or chain or fixed_order or split or tf32")
+              "slice or structure or thp or chain or fixed_order or split or tf32 or exact_parts or once_more or twenty_times")
     res = run(["-m", "pytest", "tests/test_gpu_parity.py", "-q", "-x", "-m", "gpu", "-k", select])
     tail = (res.stdout + res.stderr)[-3000:]
     assert res.returncode == 0, tail
