@@ -135,17 +135,20 @@ size_t st_workspace_bytes(st_op op, int64_t a, int64_t b, int64_t c, int64_t e, 
 /* Second moment over the unique set of the symmetric output (Section 3, M1 = f (x) f
  * summed over samples; Section 5.5, "Vector Self-Outer-Product": y_U = 0<=i<=j<n):
  *     out[p(i,j)] = sum_n X[n,i] * X[n,j]      for 0 <= i <= j < d
- * X: [N, ldx] with ldx >= d, dtype ST_F32 (fp32 FMA path, any d) or ST_BF16 (tensor-core
+ * X: [N, ldx] with ldx >= d, dtype ST_F32 (any d <= 32768) or ST_BF16 (tensor-core
  * path: bf16 products, fp32 accumulation; needs d % 8 == 0, ldx % 8 == 0).
+ * ST_F32 without a flag: the error of fp32 arithmetic, 1e-4 of sum |terms| at most.  FMA kernels, or for many samples of more
+ * than 120 and up to 4096 features, d % 4 == 0 and ldx % 4 == 0, tensor cores with every x as the sum of three bf16 numbers
+ * (infinities, NaN and subnormal numbers as in fp32 arithmetic; typical error 5e-8 of the result, sums of positive terms
+ * low by 5e-8 on average).  A workspace that is large enough for the FMA kernels alone selects these.
  * out_packed: d(d+1)/2 floats in ST_TRI_UPPER order.
  * ST_FLAG_TC_TF32 (ST_F32 input only): the tensor cores read the fp32 words of X as TF32 (the 13 low
  * mantissa bits are ignored: both factors of every product are truncated, so sums of positive products come out
  * low by about 1e-3 relative), fp32 accumulation; 5e-3 tolerance; needs d % 4 == 0, ldx % 4 == 0, d <= 4096;
- * about 15 times faster than the fp32 FMA path at d = 1024.
- * ST_FLAG_TC_SPLIT (ST_F32 input only): every x is split into hi = bf16(x) and lo = bf16(x - hi) by a first pass
- * (the workspace holds both parts: 4 bytes per element of X), then hi^T hi + hi^T lo + lo^T hi on the tensor
- * cores with fp32 accumulation: the tolerance of the fp32 path (1e-4) about five times faster; d % 8 == 0,
- * ldx % 4 == 0, d <= 4096, N <= 2^29.
+ * [1048576,1024] in 1.75 ms where the default takes 6.0.
+ * ST_FLAG_TC_SPLIT (ST_F32 input only): the kernel splits every x into hi = bf16(x) and lo = bf16(x - hi) and adds
+ * hi^T hi + hi^T lo + lo^T hi on the tensor cores with fp32 accumulation: the 1e-4 tolerance of the default in
+ * 3.3 ms at [1048576,1024]; d % 8 == 0, ldx % 4 == 0, d <= 4096, N <= 2^29.
  * ST_FLAG_DENSE_CONTROL: all d*d products are computed (lower-triangle tiles too) and
  * the lower results discarded; the output is the same. */
 st_status st_sym_moment2(const void *X, st_dtype xdt, int64_t N, int64_t d, int64_t ldx,

@@ -5,7 +5,7 @@
 // the register-tile kernel of moment2_small.cu for few features, and moment2_gemm_kernel below, which cuts the
 // upper triangle into 128x128 tiles and skips the 64x64 quadrants that lie below the diagonal or past d.
 // Either takes any d and any row pitch.  Many samples of more features, in rows that start on 16-byte boundaries, go to
-// the tensor cores instead, without loss of accuracy (moment2_exact.cuh).
+// the tensor cores instead, at the error of fp32 arithmetic (moment2_exact.cuh).
 #include "st_common.cuh"
 #include "st_index.cuh"
 #include <type_traits>
@@ -370,11 +370,13 @@ static bool moment2_use_small(int64_t N, int64_t d, unsigned flags)
     return (double)slots / 0.60 <= (double)(moment2_gemm_quads(d, dense) * 4096) / 0.75;
 }
 
-// Tensor cores with the exact parts of x (moment2_exact.cuh), no less accurate: from where they are faster than the FMA kernels.
-// FMA / tensor cores, us: [12000,128] 17.1 / 17.3, [16384,128] 20.4 / 19.1, [200000,128] 106 / 92, [4096,192] 12.6 / 15.8,
+// Tensor cores with the exact parts of x (moment2_exact.cuh): from where they are faster than the FMA kernels.  Other feature
+// counts than multiples of four have rows that a tensor map can name in a padded table only, and stay with the FMA kernels.
+// FMA / tensor cores, us (the main kernel and the sums after it): [12000,128] 17.1 / 17.3, [16384,128] 20.4 / 19.1, [200000,128] 106 / 92, [4096,192] 12.6 / 15.8,
 // [6000,192] 18.0 / 16.5, [4096,200] 20.6 / 15.9, [2000,260] 14.6 / 14.7, [3000,260] 22.1 / 15.5, [1000,512] 15.0 / 16.8,
 // [1500,512] 23.3 / 17.0, [65536,512] 370 / 122, [300,768] 14.6 / 16.5, [600,768] 22.6 / 17.3, [4096,2048] 374 / 104.  Up to 120
 // features the register tiles are the better ones ([200000,120] 78 / 92), and those of 129 to 136 are no worse ([65536,136] 43 / 43).
+// [4096,192] and [3000,260] are as many values on different sides of the line: it lies above both.
 static bool moment2_use_exact(int64_t N, int64_t d)
 {
     if (d % 4 != 0 || d <= 120 || (d > 128 && d <= 136) || d > 4096 || N > (int64_t(1) << 31) - 64) return false;

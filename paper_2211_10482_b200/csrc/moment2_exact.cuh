@@ -1,5 +1,5 @@
-// Second moment of fp32 samples on the tensor cores, no less accurate than a chain of fp32 FMAs (M2_EXACT of moment2_tc.cu,
-// which includes this file; tiles, clusters and the sum of the partial tiles are those of that file).
+// Second moment of fp32 samples on the tensor cores, at the error of fp32 arithmetic (M2_EXACT of moment2_tc.cu, which includes
+// this file; tiles, clusters and the sum of the partial tiles are those of that file).
 //
 // x = hi + mid + lo in bfloat16, exactly: 24 bits are three times eight.  Of the nine products of the parts the three that lie
 // 2^-27 and more below the result are left out, the other six go through the tensor core.  It truncates what it adds to the
@@ -8,11 +8,16 @@
 //     in registers: an epilogue thread holds the sums of half a row of the tile, 128 of them;
 //   - the sums of squares, whose terms all have one sign, are added by the converting warps with fp32 FMAs; truncation would
 //     leave them half a unit in the last place too small (measured -5.8e-8 relative; other sums of both signs have no such drift).
-// Against 64 bits the 2-norm of the error is 4.5e-8 to 9e-8 of the result's where fp32 FMAs are 5.5e-8 to 5e-7 off.
+// 2-norm of the error against 64 bits, of the result's, FMA kernels / here: N(0,1) [4096,256] 6.2e-8 / 4.8e-8, [65536,140]
+// 5.4e-8 / 5.5e-8, [65536,512] 1.8e-7 / 5.5e-8, [1500,2048] 3.9e-7 / 8.3e-8.  Where all x are positive sums come out 5e-8 (long
+// tails 7e-8) too small, which short chains of FMAs do not: uniform [4096,256] 5.3e-8 / 7.1e-8, [5000,520] 5.8e-8 / 6.9e-8,
+// [262144,256] 9.2e-8 / 7.3e-8, [65536,512] 1.3e-7 / 7.7e-8, [1500,2048] 2.9e-7 / 7.9e-8.  With the small products in an accumulator
+// of their own the first would be 5.9e-8, but lognormal 7.9e-8 where it is 8.1e-8, and the kernel takes 7 to 10 % longer.
 // What bounds it: per 32 samples of a full tile 1536 cycles of MMA, 1660 of shared memory (copies 256, loads 256 and stores 384 of
 // the converting warps, operands 768), and in the converting warps, which take the 2500 cycles that are measured, about 1400
-// of the issue slots of a scheduler, whose loads wait behind the tensor core's.  [65536,512] 370 us with fp32 FMAs, here 122;
-// [65536,256] 112 and 44; [4096,2048] 374 and 104.  Tried: four converting warps (139 at [65536,512]), two groups of four on
+// of the issue slots of a scheduler, whose loads wait behind the tensor core's; 12 bytes of their registers are spilled.  Calls in a
+// row on one table, us: [65536,512] 371 with fp32 FMAs, here 121; [65536,256] 112 and 47; [4096,2048] 376 and 113.  Tried (the kernel
+// alone, when it took 122): four converting warps (139 at [65536,512]), two groups of four on
 // alternate stages (152), polls by one lane (148), the mixed-precision subtraction (134 instead of 131).
 // Infinities, NaN and |x| > 2^127.99 have no parts and make a sum that is no number; of |x| < 2^-102 parts may be lost or subnormal.
 // A cluster that meets either looks its samples through, and adds once more, with fp32 FMAs, the sums that are no number though

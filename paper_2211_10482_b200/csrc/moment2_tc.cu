@@ -4,7 +4,7 @@
 //   M2_TF32   fp32, of which the tensor core reads the upper 19 bits
 //   M2_CONV   fp32, in the kernel x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi
 //   M2_SPLIT  the same products of hi and lo that lie in memory (the pair features of moment4.cu)
-//   M2_EXACT  fp32, in the kernel of moment2_exact.cuh x = hi + mid + lo, no less accurate than fp32 FMAs
+//   M2_EXACT  fp32, in the kernel of moment2_exact.cuh x = hi + mid + lo, at the error of fp32 arithmetic
 //
 // A cluster of two blocks owns an output tile of 256 rows (i) x up to 256 columns (j) for a range of the samples.
 // Only tiles that contain an entry with i <= j are launched, and a tile of the last column is as wide as the columns
@@ -771,7 +771,7 @@ st_status moment2_bf16_tc(const void *X, int64_t N, int64_t d, int64_t ldx, floa
     return m2tc_run<M2_BF16>(X, N, d, ldx, out, ws, ws_bytes, flags, stream);
 }
 
-// fp32 input, no less accurate than fp32 FMAs (moment2_exact.cuh); rows of X that a tensor map can name
+// fp32 input at the error of fp32 arithmetic (moment2_exact.cuh); rows of X that a tensor map can name
 size_t moment2_exact_tc_workspace(int64_t N, int64_t d, unsigned flags) { return m2tc_workspace<M2_EXACT>(N, d, flags); }
 
 st_status moment2_exact_tc(const float *X, int64_t N, int64_t d, int64_t ldx, float *out, void *ws, size_t ws_bytes,
