@@ -15,6 +15,14 @@
 // and adds it into an fp32 partial tile; a second kernel adds the partial tiles of all sample ranges in a fixed order
 // and writes the packed upper triangle.
 //
+// Up to 128 columns that are left over after whole tiles of 256 (`ext`) have no tiles of their own, which would load 256 columns
+// of A for a few of B: the tiles on the diagonal, whose A is B, load them in the place of A and make a second product of
+// their rows with them, and the last of these tiles also the product of the left-over columns with themselves.  Such a tile
+// needs the tensor memory of both accumulators, so that its MMAs wait while the epilogue empties them (a tenth of a phase
+// with one load from tensor memory at a time and sums that come back from L2; hardly anything with m2tc_add_in_l2).
+// us, with tiles of their own / carried along: [262144,520] split 389 / 308, TF32 287 / 204, bf16 153 / 117; [131072,776] 346 / 286,
+// 229 / 187, 129 / 110; [262144,264] 161 / 109, 137 / 76, 71 / 43; [131072,896] (128 columns) 399 / 327, 250 / 217, 131 / 117.
+//
 // The tensor core adds into its fp32 accumulator without round-to-nearest, so a chain of
 // many thousands of accumulating MMAs drifts low (measured: -7.7e-4 relative on all-positive
 // sums of 150k terms).  The chain is therefore cut every FLUSH_CHUNKS stages: the MMAs switch
@@ -35,7 +43,7 @@
 // 96 bytes per sample and column pair).  Few features: the latency of a stage, hence more and smaller stages.
 //
 // M2_CONV: a pass that wrote hi and lo before moved 8 bytes a value through HBM on top of the 4 read here, and took
-// 176 of the 590 us of [262144,520], now 410; [1048576,256] 700, now 285; [1048576,64] 245, now 143.  Copies bring the
+// 176 of the 590 us of [262144,520], now 308; [1048576,256] 700, now 285; [1048576,64] 245, now 143.  Copies bring the
 // fp32 boxes, converting warps rewrite them in place and arrive at the leader's barrier.  Bound by shared memory: per
 // 32 samples of a full tile off the diagonal 256 cycles each for the copy, the reads and the writes and 384 for the
 // operands of 768 cycles of MMA.  Loads through registers instead of the copies avoid two of these, but every arrival
@@ -64,6 +72,7 @@ constexpr int CONV_GROUPS = 3;                  // M2_CONV: groups of four conve
 constexpr int CONV_THREADS = 128 * CONV_GROUPS;
 constexpr size_t STAGES_BYTES_CONV = 196608;    // with 131072 [262144,520] ran 552 us instead of 510, [30000,520] 78 instead of 68
 constexpr int MAX_TILES = 160;
+constexpr int MAX_EXT = 16;                     // 4096 columns in tiles of 256
 constexpr uint32_t TMEM_COLS = 512;
 template <int MODE> struct Shape {
     static constexpr int ELEM = MODE == M2_TF32 ? 4 : 2;
@@ -84,12 +93,20 @@ struct TileTable {
     unsigned short row[MAX_TILES], col[MAX_TILES];     // first row and column of the result, units of 8
     unsigned short rows[MAX_TILES];                    // at most 256
     unsigned short first[MAX_TILES + 1];               // first cluster: the clusters of a tile share its samples
+    unsigned char ext[MAX_TILES];                      // columns that are left over after the whole tiles, units of 16: 0 or, on
+                                                       // tiles that carry them, all of them
+    unsigned char next, carrier[MAX_EXT];              // those tiles
+    unsigned char corner;                              // the last of them also has the left-over columns among themselves
+    unsigned short ext_col;                            // first left-over column, units of 8
 };
+// A partial tile holds four columns of a row side by side: [BN / 4][HALF][4] for each block, and after the BN columns of the
+// tile the left-over ones, and after these the corner.
 struct Args {
-    float *partials;                                   // [2 * cluster + block][BN / 4][HALF][4]: four columns of a row side by side
+    float *partials;                                   // [2 * cluster + block][pitch]
     unsigned *status;
     int d;                                             // columns of X
     int chunks_total, stages, nb, na;                  // nb, na: boxes of B and A per part in a stage
+    int pitch;                                         // floats of a block's partial tile
     int lo_row0;                                       // M2_SPLIT: first row of the lo part
     const float *X;                                    // M2_EXACT: what the copies read
     int64_t N, ldx;
@@ -107,6 +124,32 @@ __device__ __forceinline__ int m2tc_tile_of(const m2tc::TileTable &t, int cluste
         else hi = mid - 1;
     }
     return lo;
+}
+
+// Adds 32 columns of a thread's row, those of `mask`, to the partial tile, in L2 and without an answer;
+// the additions of one thread to one place take effect in their order.  L2 takes subnormal numbers for zero.  Where |v| is
+// at least 2^-100 no sum is one, and what it lacks is below 2^-25 of v; other columns are added here.
+__device__ __forceinline__ void m2tc_add_in_l2(float *p, const uint32_t (&r)[32], uint32_t mask)
+{
+    constexpr int QUAD = 4 * m2tc::HALF;                   // floats from one group of four columns to the next
+    float least = INFINITY;
+#pragma unroll
+    for (int e = 0; e < 32; ++e)
+        if (mask >> e & 1u) least = fminf(least, fabsf(__uint_as_float(r[e])));
+    const bool fast = least >= 0x1p-100f;
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+        if (!(mask >> e & 15u)) continue;
+        const float x = __uint_as_float(r[e]), y = __uint_as_float(r[e + 1]), z = __uint_as_float(r[e + 2]), w = __uint_as_float(r[e + 3]);
+        float *q = p + e / 4 * QUAD;
+        if (fast) {
+            asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+        } else {
+            float4 o;
+            asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w) : "l"(q) : "memory");
+            asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(o.x + x), "f"(o.y + y), "f"(o.z + z), "f"(o.w + w) : "memory");
+        }
+    }
 }
 
 }  // namespace st
@@ -147,6 +190,9 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     const int FLUSH_CHUNKS = MODE == M2_BF16 && width <= HALF ? S::FLUSH_CHUNKS / 2 : S::FLUSH_CHUNKS;
     const bool alias = diag && width == BN;             // A columns == B columns in both blocks: one load serves both
     const bool lead = diag && rows <= HALF;             // all rows in the first block, whose A holds its half of B as well
+    // (a tile that carries left-over columns is on the diagonal, and full; products of pairs have none)
+    const int ext = MODE == M2_SPLIT ? 0 : 16 * a.tab.ext[tile], ecol = 8 * a.tab.ext_col;
+    const bool corner = ext > 0 && a.tab.corner && tile == a.tab.carrier[a.tab.next - 1];
     const int chunks_per_split = (a.chunks_total + nsplit - 1) / nsplit;
     const int c_begin = split * chunks_per_split;
     int c_end = c_begin + chunks_per_split;
@@ -195,10 +241,12 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         return n <= 0 ? 0 : (n + BU - 1) / BU;
     };
     auto boxes_a = [&](int r) {
-        const int n = rows - r * HALF;
-        return alias || lead || n <= 0 ? 0 : n >= HALF ? HALF / BU : (n + BU - 1) / BU;
+        int n = rows - r * HALF;
+        if (ext > 0) n = min(ext / 2, a.d - ecol - r * (ext / 2));      // in the place of A, which B holds there
+        else if (alias || lead) n = 0;
+        return n <= 0 ? 0 : n >= HALF ? HALF / BU : (n + BU - 1) / BU;
     };
-    const int col_a = row + (int)rank * HALF, col_b = col + (int)rank * (width / 2);
+    const int col_a = ext > 0 ? ecol + (int)rank * (ext / 2) : row + (int)rank * HALF, col_b = col + (int)rank * (width / 2);
     if (MODE == M2_CONV && warp == 0) {
         // ---------------- TMA producer (both blocks): own boxes, fp32
         if (elect_one()) {
@@ -251,13 +299,18 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             // bf16: groups of 8 sample rows, 16-byte swizzle units; fp32 read as TF32: groups of 4, 32-byte units
             const uint64_t adesc_base = make_smem_desc(sb0 + a_off, BOX_PITCH, MODE == M2_TF32 ? 512 : 1024, MODE == M2_TF32 ? 1 : 2);
             const uint64_t bdesc_base = make_smem_desc(sb0, BOX_PITCH, MODE == M2_TF32 ? 512 : 1024, MODE == M2_TF32 ? 1 : 2);
-            const uint64_t lo = (uint64_t)(lo_off >> 4);
+            const uint64_t lo = (uint64_t)(lo_off >> 4), ext_off = (uint64_t)((a.nb * BOX_PITCH) >> 4);
+            const uint32_t idesc_ext = make_idesc(MODE == M2_TF32 ? 2 : 1, 1, 1, BM, (uint32_t)ext);
             bool ok = true;
             int c = 0, s = 0;
             uint32_t parity = 0;
             for (int ph = 0; ph < nphases && ok; ++ph) {
-                const int buf = ph & 1;
-                if (ph >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((ph >> 1) - 1) & 1), abort_flag, a.status, 4)) break;
+                const int buf = ext > 0 ? 0 : ph & 1;
+                if (ext > 0) {
+                    if (ph >= 1 && !mbar_wait(&acc_empty[0], (uint32_t)((ph - 1) & 1), abort_flag, a.status, 4)) break;
+                } else if (ph >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((ph >> 1) - 1) & 1), abort_flag, a.status, 4)) {
+                    break;
+                }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
                 const int ce = (c + FLUSH_CHUNKS < nchunks) ? c + FLUSH_CHUNKS : nchunks;
@@ -270,19 +323,28 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                     tc_fence_after();
                     const uint64_t ad = adesc_base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
                     const uint64_t bd = bdesc_base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
+                    auto products = [&](uint32_t acc, uint64_t a0, uint64_t b0, uint32_t shape) {
+                        uint32_t on = accumulate;
 #pragma unroll
-                    for (int k = 0; k < KROWS / S::KMMA; ++k) {
-                        // one MMA spans KMMA sample rows of 128 bytes: 2048 bytes (bf16) or 1024 bytes (TF32) further on
-                        constexpr int STEP = S::KMMA * 128 / 16;
-                        const uint64_t ak = ad + (uint64_t)(k * STEP), bk = bd + (uint64_t)(k * STEP);
-                        if (MODE == M2_TF32) mma_tf32_pair(d_tmem, ak, bk, idesc, accumulate);
-                        else mma_bf16_pair(d_tmem, ak, bk, idesc, accumulate);
-                        accumulate = 1;
-                        if (PARTS == 2) {
-                            mma_bf16_pair(d_tmem, ak, bk + lo, idesc, 1u);
-                            mma_bf16_pair(d_tmem, ak + lo, bk, idesc, 1u);
+                        for (int k = 0; k < KROWS / S::KMMA; ++k) {
+                            // one MMA spans KMMA sample rows of 128 bytes: 2048 bytes (bf16) or 1024 bytes (TF32) further on
+                            constexpr int STEP = S::KMMA * 128 / 16;
+                            const uint64_t ak = a0 + (uint64_t)(k * STEP), bk = b0 + (uint64_t)(k * STEP);
+                            if (MODE == M2_TF32) mma_tf32_pair(acc, ak, bk, shape, on);
+                            else mma_bf16_pair(acc, ak, bk, shape, on);
+                            on = 1;
+                            if (PARTS == 2) {
+                                mma_bf16_pair(acc, ak, bk + lo, shape, 1u);
+                                mma_bf16_pair(acc, ak + lo, bk, shape, 1u);
+                            }
                         }
+                    };
+                    products(d_tmem, ad, bd, idesc);
+                    if (ext > 0) {
+                        products(tmem_base + BN, ad, bd + ext_off, idesc_ext);
+                        if (corner) products(tmem_base + (uint32_t)(BN + ext), bd + ext_off, bd + ext_off, idesc_ext);
                     }
+                    accumulate = 1;
                     tc_commit_pair(&empty[s]);
                     if (++s == stages) { s = 0; parity ^= 1u; }
                 }
@@ -353,16 +415,52 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         const int row0 = (int)rank * HALF + q * 32;
         const bool used = row0 < rows;
         const int c_first = diag ? row0 : 0;         // row0 is a multiple of 32
-        float *dst = a.partials + (size_t)blockIdx.x * HALF * BN + (q * 32 + lane) * 4;       // columns c .. c+3: + c HALF
+        float *dst = a.partials + (size_t)blockIdx.x * (MODE == M2_SPLIT ? HALF * BN : a.pitch) + (q * 32 + lane) * 4;         // columns c .. c+3: + c HALF
+        // columns in use: c_first .. width, and where the tile carries left-over columns all in between and after them
+        const int c_end = ext > 0 ? BN + (ext * (corner && q * 32 < ext / 2 ? 2 : 1) + 31) / 32 * 32 : width;
         const uint32_t leader_acc_empty0 = map_to_cta(smem_u32(&acc_empty[0]), 0);
         if (nphases == 0 && used) {
-            for (int c0 = c_first; c0 < width; c0 += 4) *reinterpret_cast<float4 *>(dst + c0 * HALF) = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int c0 = c_first; c0 < c_end; c0 += 4) *reinterpret_cast<float4 *>(dst + c0 * HALF) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         for (int ph = 0; ph < nphases; ++ph) {
-            const int buf = ph & 1;
-            if (!mbar_wait(&acc_full[buf], (uint32_t)((ph >> 1) & 1), abort_flag, a.status, 3)) break;
+            const int buf = ext > 0 ? 0 : ph & 1;
+            if (!mbar_wait(&acc_full[buf], (uint32_t)((ext > 0 ? ph : ph >> 1) & 1), abort_flag, a.status, 3)) break;
             tc_fence_after();
-            if (used) {
+            if (used && ext > 0) {
+                // The MMAs wait until the accumulators have been read: 32 columns are on their way from tensor memory while the
+                // 32 before them are added to the partial tile, in L2, so that nothing has to come back for it.
+                const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16);
+                auto add = [&](int c0, const uint32_t (&r)[32]) {
+                    if (ph > 0) {
+                        if (c0 < BN) {
+                            m2tc_add_in_l2(dst + c0 * HALF, r, ~0u);
+                        } else {
+                            // the left-over columns and those of the corner, without what fills them up
+                            const int c = c0 - BN, left = a.d - ecol;
+                            auto low = [](int n) { return n <= 0 ? 0u : n >= 32 ? ~0u : (1u << n) - 1; };
+                            m2tc_add_in_l2(dst + c0 * HALF, r, low(left - c) | (low(ext - c + left) & ~low(ext - c)));
+                        }
+                        return;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 32; e += 4)
+                        *reinterpret_cast<float4 *>(dst + (c0 + e) * HALF) = make_float4(
+                            __uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
+                };
+                uint32_t r0[32], r1[32];
+                tmem_ld_32x32(t0 + (uint32_t)c_first, r0);
+#pragma unroll 1
+                for (int c0 = c_first; c0 < c_end; c0 += 64) {
+                    tmem_ld_wait();
+                    if (c0 + 32 < c_end) tmem_ld_32x32(t0 + (uint32_t)(c0 + 32), r1);
+                    add(c0, r0);
+                    if (c0 + 32 < c_end) {
+                        tmem_ld_wait();
+                        if (c0 + 64 < c_end) tmem_ld_32x32(t0 + (uint32_t)(c0 + 64), r0);
+                        add(c0 + 32, r1);
+                    }
+                }
+            } else if (used) {
 #pragma unroll 1
                 for (int c0 = c_first; c0 < width; c0 += 32) {
                     uint32_t r[32];
@@ -407,17 +505,24 @@ __host__ __device__ inline int m2tc_sum_warps(int nsplit) { return nsplit <= 4 ?
 template <bool PAIRS>
 __global__ void __launch_bounds__(256)
 moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features, int within, int64_t out_elems,
-                         const unsigned *pairs, const __grid_constant__ m2tc::TileTable tab)
+                         const unsigned *pairs, int pitch, const __grid_constant__ m2tc::TileTable tab)
 {
     using namespace m2tc;
     __shared__ float4 part[2][8][32];
-    const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int row = 8 * tab.row[tile], col = 8 * tab.col[tile], rows = tab.rows[tile];
-    const int quads = (min(32 * (int)tab.width[tile], d - col) + 3) / 4, units = (rows + 31) / 32 * quads;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the tiles, then the left-over columns of each tile that carries them, then the corner
+    const int e = PAIRS ? -1 : (int)blockIdx.x - tab.ntiles;
+    const bool corner = !PAIRS && e >= (int)tab.next;
+    const int tile = e < 0 ? (int)blockIdx.x : tab.carrier[corner ? (int)tab.next - 1 : e], ext = 16 * tab.ext[tile];
+    const int row = 8 * (corner ? tab.ext_col : tab.row[tile]), col = 8 * (e < 0 ? tab.col[tile] : tab.ext_col);
+    const int rows = corner ? min(ext, d - row) : tab.rows[tile], block_rows = corner ? ext / 2 : HALF;
+    const int at_col = e < 0 ? 0 : corner ? BN + ext : BN;                                    // in the partial tile
+    const int quads = (min(e < 0 ? 32 * (int)tab.width[tile] : ext, d - col) + 3) / 4, units = (rows + 31) / 32 * quads;
     const int first = tab.first[tile], nsplit = tab.first[tile + 1] - first;
     const int wps = m2tc_sum_warps(nsplit);
     const int per = 8 / wps, w0 = warp % wps;
-    const size_t stride = (size_t)2 * HALF * BN;
+    const int block = PAIRS ? HALF * BN : pitch;           // floats of a block's partial tile
+    const size_t stride = (size_t)2 * block;
     constexpr int BATCH = 4;
     pdl_wait();
     pdl_trigger();
@@ -428,7 +533,8 @@ moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features,
         // what is loaded does not wait for what has to be looked up
         const bool use = u < units && r < rows && gj + 4 > (PAIRS && gi >= within ? 0 : gi);
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float *base = partials + (size_t)(2 * first + (r >> 7)) * HALF * BN + c * HALF + (r & 127) * 4;
+        const int second = PAIRS ? r >> 7 : r >= block_rows ? 1 : 0, in_block = PAIRS ? r & 127 : r - second * block_rows;
+        const float *base = partials + (size_t)(2 * first + second) * block + (at_col + c) * HALF + in_block * 4;
         for (int k0 = w0; k0 < nsplit; k0 += BATCH * wps) {
             float4 v[BATCH];
 #pragma unroll
@@ -470,14 +576,19 @@ moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features,
 
 struct M2TcPlan {
     m2tc::TileTable tab;
-    int chunks_total, stages, nb, na;
+    int chunks_total, stages, nb, na, pitch;
     size_t partial_bytes, smem;
     bool ok;
 };
 
 // Time per stage, a full tile = 1: the 256 columns of A are loaded whatever the width (the MMA alone would be 43 cycles
-// at 64 columns against 128; with 0.35 in place of 0.7 [400000,304] bf16 ran 127 us instead of 111).
-static double m2tc_cost(int width) { return 0.7 + 0.3 * width / m2tc::BN; }
+// at 64 columns against 128; with 0.35 in place of 0.7 [400000,304] bf16 ran 127 us instead of 111).  ext: left-over columns
+// that the tile carries along, times the products that it makes of them (with those for nothing [262144,520] split ran 325 us
+// instead of 311, [131072,776] 320 and 288, [131072,896] 412 and 340).
+static double m2tc_cost(int width, int ext, int products)
+{
+    return 0.7 + 0.3 * width / m2tc::BN + (ext > 0 ? products * (0.08 + (double)ext / m2tc::BN) : 0);
+}
 // M2_EXACT, where a stage takes as long as its values are converted: us per 32 samples 1.36, on the diagonal 1.2, 1.27 at 32
 // columns off it, 1.0, 0.73 and 0.65 where all columns are 128, 64 or four.
 static double m2tc_exact_cost(int rows, int width, bool diag)
@@ -486,13 +597,16 @@ static double m2tc_exact_cost(int rows, int width, bool diag)
     return rows > m2tc::HALF ? 0.88 : 0.47 + 0.26 * rows / m2tc::HALF;
 }
 
+// Columns that are left over after `full` tiles of 256: carried along by the tiles on the diagonal, or tiles of their own.
+static bool m2tc_carry(int full, int left_over) { return full > 0 && left_over > 0 && left_over <= m2tc::HALF; }
+
 // Tiles of a plan while it is made.
 struct M2TcTiles {
     M2TcPlan *p;
     int n;
     double cost[m2tc::MAX_TILES];
     template <int MODE>
-    bool add(int row, int rows, int col, int width, bool diag)
+    bool add(int row, int rows, int col, int width, bool diag, int ext_col = 0, int ext = 0, bool corner = false)
     {
         using namespace m2tc;
         using S = Shape<MODE>;
@@ -502,14 +616,24 @@ struct M2TcTiles {
         p->tab.col[n] = (unsigned short)(col / 8);
         p->tab.width[n] = (unsigned char)(width / 32);
         p->tab.diag[n] = diag ? 1 : 0;
-        cost[n] = MODE == M2_EXACT ? m2tc_exact_cost(rows, width, diag) : m2tc_cost(width);
+        cost[n] = MODE == M2_EXACT ? m2tc_exact_cost(rows, width, diag) : m2tc_cost(width, ext, corner ? 2 : 1);
         const bool lead = diag && rows <= HALF;
         const int cols_b = lead && rows > width / 2 ? rows : width / 2, nb = (cols_b + S::BOXC - 1) / S::BOXC;
         if (nb > p->nb) p->nb = nb;
-        if (!(diag && width == BN) && !lead) {
-            const int na = rows >= HALF ? S::NBOX : (rows + S::BOXC - 1) / S::BOXC;
+        if (ext > 0 || (!(diag && width == BN) && !lead)) {
+            const int n_a = ext > 0 ? ext / 2 : rows;
+            const int na = n_a >= HALF ? S::NBOX : (n_a + S::BOXC - 1) / S::BOXC;
             if (na > p->na) p->na = na;
         }
+        p->tab.ext[n] = (unsigned char)(ext / 16);
+        if (ext > 0) {
+            if (p->tab.next >= MAX_EXT) return false;
+            p->tab.carrier[p->tab.next++] = (unsigned char)n;
+            p->tab.ext_col = (unsigned short)(ext_col / 8);
+            if (corner) p->tab.corner = 1;
+        }
+        const int columns = BN + (ext * (corner ? 2 : 1) + 31) / 32 * 32;             // written 32 at a time
+        if (columns * HALF > p->pitch) p->pitch = columns * HALF;
         ++n;
         return true;
     }
@@ -567,7 +691,7 @@ static void m2tc_finish(M2TcPlan &p, const M2TcTiles &t, int64_t N)
         first += split[i];
     }
     for (int i = n; i <= MAX_TILES; ++i) p.tab.first[i] = (unsigned short)first;
-    p.partial_bytes = (size_t)2 * first * HALF * BN * sizeof(float);
+    p.partial_bytes = (size_t)2 * first * p.pitch * sizeof(float);
     p.ok = true;
 }
 
@@ -578,7 +702,10 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
     M2TcPlan p{};
     M2TcTiles t{&p, 0, {}};
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
-    const int nt = (int)((d + BM - 1) / BM);
+    const int full = (int)(d / BM), left_over = (int)(d % BM);
+    const bool carry = MODE != M2_EXACT && !dense && m2tc_carry(full, left_over);
+    const int ext = carry ? (left_over + 15) / 16 * 16 : 0;
+    const int nt = carry ? full : (int)((d + BM - 1) / BM);
     for (int tn = 0; tn < nt; ++tn)
         for (int tm = 0; tm < nt; ++tm) {
             if (tm > tn && !dense) continue;
@@ -586,13 +713,15 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
             int width = left >= BN ? BN : (left + 31) / 32 * 32;
             // M2_EXACT: with all 256 columns A holds B, and half as many values are converted ([65536,200] 52 us, now 45)
             if (MODE == M2_EXACT && tm == tn && width > HALF) width = BN;
-            if (!t.add<MODE>(tm * BM, below < BM ? below : BM, tn * BN, width, tm == tn)) return p;
+            const int e = tm == tn ? ext : 0;
+            if (!t.add<MODE>(tm * BM, below < BM ? below : BM, tn * BN, width, tm == tn, full * BM, e, tm == nt - 1)) return p;
         }
     m2tc_finish<MODE>(p, t, N);
     return p;
 }
 
 // Tiles of the products of pair features that pair_layout.cuh names, in turn to f(row, rows, col, width, on the diagonal).
+// (Left-over columns carried by the tile on the diagonal: [30011,45] 92 us without, 96 with them.)
 template <class F>
 static void pair_tiles(const PairLayout &L, F f)
 {
@@ -632,7 +761,7 @@ PairLayout pair_layout(int features, bool one)
         L.prod = (L.rows + L.rows_n + 7) / 8 * 8;
         L.cols = L.prod + (int)tri_rows(features) - within - L.rows_n;
         double cost = 0;
-        pair_tiles(L, [&](int, int, int, int width, bool) { cost += m2tc_cost(width); });
+        pair_tiles(L, [&](int, int, int, int width, bool) { cost += m2tc_cost(width, 0, 0); });
         if (option == 0 || cost < least) {
             best = L;
             least = cost;
@@ -678,7 +807,7 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
         return ST_ERR_CUDA;
     m2tc::Args a;
     a.partials = partials; a.status = status;
-    a.chunks_total = q.chunks_total; a.stages = q.stages; a.nb = q.nb; a.na = q.na; a.lo_row0 = (int)lo_row0; a.d = (int)d;
+    a.chunks_total = q.chunks_total; a.stages = q.stages; a.nb = q.nb; a.na = q.na; a.pitch = q.pitch; a.lo_row0 = (int)lo_row0; a.d = (int)d;
     a.X = (const float *)X; a.N = rows; a.ldx = ldx;
     a.tab = q.tab;
     const auto kernel = m2tc_kernel<MODE>();
@@ -710,9 +839,9 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     }
     const unsigned most = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
     if (blocks > most) blocks = most < 64 ? 64 : most;
-    const dim3 rgrid((unsigned)q.tab.ntiles, blocks);
+    const dim3 rgrid((unsigned)(q.tab.ntiles + q.tab.next + q.tab.corner), blocks);
     return launch(pairs ? moment2_tc_reduce_kernel<true> : moment2_tc_reduce_kernel<false>, rgrid, 256, 0, stream, partials, out, (int)d,
-                  features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.tab);
+                  features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.pitch, q.tab);
 }
 
 // Room for the partial tiles of the structured call and of its dense control: one workspace serves both.

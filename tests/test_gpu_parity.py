@@ -853,6 +853,46 @@ def test_moment2_tensor_core_tile_widths(st, N, d):
     assert oracle.rel_err(expand2(st, st.st_sym_moment2(dev(X), flags=st.ST_FLAG_TC_TF32), d), Tt, St) <= TOL_F32
 
 
+# columns left over after whole tiles of 256, carried along by the tiles on the diagonal: 16 to 128 of them in steps of 16, one
+# tile and several, the first length that has tiles of its own
+@pytest.mark.parametrize("N,d", [(1, 264), (33, 272), (700, 280), (65, 304), (1300, 320), (900, 384), (400, 392), (5000, 520), (257, 600),
+                                 (300, 896), (100, 1048)])
+def test_moment2_tensor_core_left_over_columns(st, N, d):
+    X = workloads.draw((N, d), "normal", 41 + N + d)
+    bits = workloads.f32_to_bf16_bits(X)
+    Tb, Sb = oracle.moment2(workloads.bf16_bits_to_f32(bits))
+    assert oracle.rel_err(expand2(st, st.st_sym_moment2(bf16_dev(bits)), d), Tb, Sb) <= TOL_F32
+    T, S = oracle.moment2(X)
+    assert oracle.rel_err(expand2(st, st.st_sym_moment2(dev(X), flags=st.ST_FLAG_TC_SPLIT), d), T, S) <= TOL_F32
+    Tt, St = oracle.moment2((X.view(np.uint32) & np.uint32(0xFFFFE000)).view(np.float32))
+    assert oracle.rel_err(expand2(st, st.st_sym_moment2(dev(X), flags=st.ST_FLAG_TC_TF32), d), Tt, St) <= TOL_F32
+    # 4 columns fewer: the last group of four columns of TF32
+    Tt, St = oracle.moment2(np.ascontiguousarray((X.view(np.uint32) & np.uint32(0xFFFFE000)).view(np.float32)[:, :d - 4]))
+    assert oracle.rel_err(expand2(st, st.st_sym_moment2(dev(X[:, :d - 4].copy()), flags=st.ST_FLAG_TC_TF32), d - 4), Tt, St) <= TOL_F32
+
+
+@pytest.mark.parametrize("mode,N,d", [("split", 210000, 264), ("split", 230000, 304), ("tf32", 640000, 260), ("bf16", 640000, 384)])
+def test_moment2_left_over_columns_of_long_sample_ranges(st, mode, N, d):
+    """Accumulators that are added to the partial tile several times, in L2 and, where sums are tiny, outside: columns scaled by a
+    power of two (no sum becomes subnormal) give the same bits but for the scale."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    X = torch.randn(N, d, generator=g, device="cuda")
+    flags = {"split": st.ST_FLAG_TC_SPLIT, "tf32": st.ST_FLAG_TC_TF32, "bf16": 0}[mode]
+    scale = torch.ones(d, device="cuda")
+    scale[::3] = 2.0 ** -54                            # times 2^-54 is 2^-108, where sums are added outside L2
+    scale[1::3] = 2.0 ** -47                           # some above 2^-100 and some below
+    if mode == "bf16":
+        X = X.bfloat16()
+    iu = torch.triu_indices(d, d, device="cuda")
+    plain = st.st_sym_moment2(X, flags=flags)
+    scaled = st.st_sym_moment2(X * scale.to(X.dtype), flags=flags)
+    assert torch.equal(scaled, plain * scale[iu[0]] * scale[iu[1]])
+    X64 = X.double()
+    T, S = X64.T @ X64, X64.abs().T @ X64.abs()
+    assert ((plain.double() - T[iu[0], iu[1]]).abs() / S[iu[0], iu[1]]).max().item() <= (TOL_TC if mode == "tf32" else TOL_F32)
+
+
 def test_moment2_split_sums_of_squares_do_not_drift(st):
     """All-positive sums over many samples: the accumulation chain is cut often enough that the diagonal stays
     inside the fp32 tolerance (a tensor-core accumulator rounds towards zero)."""
