@@ -34,6 +34,7 @@ constexpr int64_t MAX_GRID = int64_t(1) << 30;
 constexpr int ROW_SEG = 2048, ROW_WIDE = 512;   // symmetric fill of wide positions
 constexpr int SYM_WORDS = 4;               // words that a lane of the symmetric fill has in flight
 constexpr int64_t PART_BYTES = 32768;      // most of a slice that one thread group copies ([384,384,75]: 128 KiB starve the chip)
+constexpr int64_t ONCE_BYTES = 256 * 16 * COPY_UNITS;     // the same in one pass (copy_once)
 
 struct LayoutArgs {
     int kind;
@@ -133,6 +134,53 @@ __device__ __forceinline__ void copy_flat(unsigned char *dst, const unsigned cha
     for (int e = e0 + g * ES; e < ends; e += g * ES) *reinterpret_cast<E *>(dst + end_at(e)) = end_load(e);   // small groups only
 }
 
+// The same by whole warps, for at most 16 U bytes a thread: warp l / 32 of the group takes the 32 U units from there on.  Where the
+// source is off a boundary a unit is put together from the aligned unit that its lane loaded and the one of the next lane,
+// which is half the loads of copy_flat and leaves room for U units in flight.
+template <int ES, bool MUL, int U>
+__device__ __forceinline__ void copy_once(unsigned char *dst, const unsigned char *src, const unsigned char *mul, int n, int lane,
+                                          const unsigned char *src_end)
+{
+    typedef typename Elem<ES>::T E;
+    const CopySpan span = copy_span((uintptr_t)dst, (uintptr_t)src, n, (uintptr_t)src_end);
+    const int units = span.units;
+    const unsigned off = span.off;
+    const int l = lane & 31, e = lane * ES, b = (lane & ~31) * U + l;
+    const int end_at = e < span.head ? e : e + (units << 4);             // less than 32 elements
+    E ev = E{};
+    if (e < span.ends) ev = *reinterpret_cast<const E *>(src + end_at);
+    const uint4 *in = reinterpret_cast<const uint4 *>(src + span.head - off) + b;
+    const int loads = (off != 0 && units > 0 ? units + 1 : units) - b, stores = units - b;
+    uint4 v[U + 1], w[MUL ? U : 1];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+        if (32 * k < loads) v[k] = in[32 * k];
+        if (MUL && 32 * k < stores) w[k] = reinterpret_cast<const uint4 *>(mul + span.head)[b + 32 * k];
+    }
+    if (off != 0 && l == 0 && 32 * U < loads) v[U] = in[32 * U];
+    if constexpr (MUL)
+        if (e < span.ends) ev = mul_word(ev, *reinterpret_cast<const uint32_t *>(mul + end_at));
+    uint4 *out = reinterpret_cast<uint4 *>(dst + span.head) + b;
+    const int next = (l + 1) & 31;                                       // lane 0 has the unit behind those of all lanes
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+        uint4 r = v[k];
+        if (ES < 16 && off != 0) {
+            uint4 y = make_uint4(0, 0, 0, 0);                            // as far as it is needed
+            y.x = __shfl_sync(0xFFFFFFFFu, l == 0 ? v[k + 1].x : r.x, next);
+            if (off > 4) y.y = __shfl_sync(0xFFFFFFFFu, l == 0 ? v[k + 1].y : r.y, next);
+            if (ES < 8 && off > 8) y.z = __shfl_sync(0xFFFFFFFFu, l == 0 ? v[k + 1].z : r.z, next);
+            if (ES < 4 && off > 12) y.w = __shfl_sync(0xFFFFFFFFu, l == 0 ? v[k + 1].w : r.w, next);
+            r = shift_unit<ES>(r, y, off);
+        }
+        if (32 * k < stores) {
+            if (MUL) r = make_uint4(mul_word(r.x, w[k].x), mul_word(r.y, w[k].y), mul_word(r.z, w[k].z), mul_word(r.w, w[k].w));
+            out[32 * k] = r;
+        }
+    }
+    if (e < span.ends) *reinterpret_cast<E *>(dst + end_at) = ev;
+}
+
 template <int ES>
 __device__ __forceinline__ void zero_flat(unsigned char *dst, int n, int lane, int g)
 {
@@ -225,7 +273,8 @@ __device__ __forceinline__ void slice_run(const LayoutArgs &a, I &s, I &lo, I &h
 // Four blocks per SM: with the registers that the compiler would take (up to 96) fewer fit, and the zeros of a sparse slice are
 // bound by the number of blocks ([8000,8000] band 39.5 us, 37.7 with 64 registers; st_thp of a tet d = 120, rows of 64 floats
 // 52, now 39).
-template <int KIND, int ES, bool PACK, bool MUL, typename I>
+// ONCE: blocks that go through their part of a slice in one pass (copy_once).
+template <int KIND, int ES, bool PACK, bool MUL, bool ONCE, typename I>
 __global__ void __launch_bounds__(256, 4)
 slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I nitems, int group_shift, int parts,
                   int part_bytes, const unsigned char *mul)
@@ -239,6 +288,10 @@ slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I 
     const I ngroups = (I)(((int64_t)gridDim.x * blockDim.x) >> group_shift);
     const int64_t sb = a.d * a.row_bytes;                     // bytes per dense slice
     const unsigned char *src_end = src + (PACK ? a.dense_rows : a.packed_rows) * a.row_bytes;
+    auto copy = [&](unsigned char *to, const unsigned char *from, const unsigned char *times, int n) {
+        if constexpr (ONCE) copy_once<ES, MUL, COPY_UNITS>(to, from, times, n, lane, src_end);
+        else copy_flat<ES, MUL, MUL ? COPY_UNITS / 2 : COPY_UNITS>(to, from, times, n, lane, g, src_end);
+    };
     for (I item = gid; item < nitems; item += ngroups) {
         I s = parts == 1 ? item : item / (I)parts, lo, hi, prow;
         const int64_t part = item - s * (I)parts;
@@ -262,13 +315,13 @@ slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I 
         const int64_t p0 = (int64_t)prow * a.row_bytes - d0;           // packed byte of its byte 0, were it in the run
         if (PACK) {
             if (BAND_ROW && d0 > u0) zero_flat<ES>(dst + p0 + u0, (int)((u1 < d0 ? u1 : d0) - u0), lane, g);
-            if (x1 > x0) copy_flat<ES, MUL, MUL ? COPY_UNITS / 2 : COPY_UNITS>(dst + p0 + x0, src + (int64_t)s * sb + x0 - shift, mul + p0 + x0, (int)(x1 - x0), lane, g, src_end);
+            if (x1 > x0) copy(dst + p0 + x0, src + (int64_t)s * sb + x0 - shift, mul + p0 + x0, (int)(x1 - x0));
             if (BAND_ROW && u1 > d1) zero_flat<ES>(dst + p0 + (u0 > d1 ? u0 : d1), (int)(u1 - (u0 > d1 ? u0 : d1)), lane, g);
         } else {
             unsigned char *out = dst + (int64_t)s * sb;
             const int64_t z1 = u1 < c0 ? u1 : c0;               // zeros before the run
             if (z1 > u0) zero_flat<ES>(out + u0, (int)(z1 - u0), lane, g);
-            if (x1 > x0) copy_flat<ES, false, COPY_UNITS>(out + x0, src + p0 + x0, nullptr, (int)(x1 - x0), lane, g, src_end);
+            if (x1 > x0) copy(out + x0, src + p0 + x0, nullptr, (int)(x1 - x0));
             const int64_t z2 = u0 > c1 ? u0 : c1;               // zeros after the run
             if (u1 > z2) zero_flat<ES>(out + z2, (int)(u1 - z2), lane, g);
         }
@@ -571,6 +624,12 @@ template <int KIND, int ES, bool PACK>
 static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cudaStream_t s, const void *mul)
 {
     const int64_t cap = MAX_GRID;
+    // A block per 16 KB, in one pass: long runs off 16-byte boundaries, that is slices of a matrix; bound by HBM and L2.  us, blocks that
+    // walk 32 KB / one pass: times a packed operand [384,384,75] 13.6 / 11.2, [4000,4000,3] 52.1 / 45.4, [2000,2000,10] 41.4 / 37.3;
+    // zero fill 11.4 / 11.0, 50.1 / 45.9, 40.5 / 37.6; pack 8.7 / 9.0, 38.5 / 35.7, 29.4 / 28.6; pack, product, sum and fill of
+    // [384,384,75] out of HBM 54.2 / 48.2 together.  Not where runs are short or most parts of a slice empty (pack of a tet d = 160,
+    // 33 floats, 52 / 74; 2-byte words [900,900,17] 5.3 / 6.8), nor where all is aligned ([1024,1024,64] doubles 81 / 84).
+    constexpr bool ONCE = KIND == ST_TRI_UPPER && (ES == 4 || ES == 8);
     // slices: about four 16-byte units per thread, at most PART_BYTES per (slice, part), less where the slices are too few to
     // fill the chip (one row of [1000,1000,128] in 16 parts 17 us the call with its empty slices, now 1.8).  Pack splits the
     // longest run of unique columns (a band: its packed row), unpack the whole dense slice.
@@ -581,14 +640,16 @@ static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cu
     const int64_t sb = (PACK ? run_rows : a.d) * a.row_bytes;
     // pack of a tensor of order 3 or 4, or of one row: only the slices that have a run
     const int64_t nslices = PACK && KIND == ST_FIXED_ROW ? 1 : KIND == ST_TET ? (PACK ? tri_rows(a.d) : a.d * a.d) : KIND == ST_SIMPLEX4 ? (PACK ? tet_rows(a.d) : a.d * a.d * a.d) : a.d;
-    int64_t part_bytes = PART_BYTES;
-    while (part_bytes > 4096 && nslices * ((sb + part_bytes - 1) / part_bytes) < 2 * (int64_t)sm_count_or_default()) part_bytes /= 2;
+    bool once = false;
+    if constexpr (ONCE) once = a.row_bytes % 16 != 0 && sb >= ONCE_BYTES;
+    int64_t part_bytes = once ? ONCE_BYTES : PART_BYTES;
+    while (!once && part_bytes > 4096 && nslices * ((sb + part_bytes - 1) / part_bytes) < 2 * (int64_t)sm_count_or_default()) part_bytes /= 2;
     int64_t parts = (sb + part_bytes - 1) / part_bytes;
     const int64_t pb = ((sb + parts - 1) / parts + 15) / 16 * 16;
     parts = (sb + pb - 1) / pb;
     if (parts > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
     int shift = 0;
-    while ((1 << shift) < 256 && (int64_t(16 * COPY_UNITS) << shift) < pb) ++shift;
+    while ((1 << shift) < 256 && (once || (int64_t(16 * COPY_UNITS) << shift) < pb)) ++shift;
     const int64_t nitems = nslices * parts, threads = nitems << shift;
     const int64_t want = (threads + 255) / 256;
     const unsigned grid = (unsigned)(want < cap ? (want < 1 ? 1 : want) : cap);
@@ -599,8 +660,11 @@ static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cu
                        a.d <= (KIND == ST_TET ? 1024 : KIND == ST_SIMPLEX4 ? 200 : 20000);
     auto run = [&](auto mul_tag, auto index) {
         typedef decltype(index) I;
-        return launch(slice_copy_kernel<KIND, ES, PACK, decltype(mul_tag)::value, I>, grid, 256, 0, s, in, out, a, (I)nitems, shift, (int)parts,
-                      (int)pb, m);
+        constexpr bool MUL = decltype(mul_tag)::value;
+        if constexpr (ONCE)
+            if (once)
+                return launch(slice_copy_kernel<KIND, ES, PACK, MUL, true, I>, grid, 256, 0, s, in, out, a, (I)nitems, 8, (int)parts, (int)pb, m);
+        return launch(slice_copy_kernel<KIND, ES, PACK, MUL, false, I>, grid, 256, 0, s, in, out, a, (I)nitems, shift, (int)parts, (int)pb, m);
     };
     if constexpr (PACK && ES == 4)
         if (mul) return small ? run(std::true_type{}, 0u) : run(std::true_type{}, int64_t(0));

@@ -1389,6 +1389,30 @@ def test_copies_of_wide_bands_rows_and_positions(st, kind, d, inner, dtype, k):
         assert np.array_equal(st.st_thp(dev(B), dev(C), lay).cpu().numpy(), want)
 
 
+# slices of 16 KB and more whose rows are off 16-byte boundaries (every offset of words), on both sides of that line; symmetric
+# fill word by word: the first and last widths of it, rows found by one lane for all and by each for itself, parts that end early
+@pytest.mark.parametrize("kind,d,inner,dtype", [
+    ("ST_TRI_UPPER", 70, 59, np.uint32), ("ST_TRI_UPPER", 69, 59, np.uint32), ("ST_TRI_UPPER", 131, 127, np.uint32), ("ST_TRI_UPPER", 37, 111, np.uint64),
+    ("ST_TRI_UPPER", 4100, 1, np.uint32), ("ST_TRI_UPPER", 67, 129, np.uint32), ("ST_TRI_UPPER", 300, 33, np.uint32), ("ST_TET", 21, 33, np.uint32),
+    ("ST_TET", 19, 127, np.uint32), ("ST_TET", 35, 8, np.uint32), ("ST_TET", 35, 9, np.uint32), ("ST_TET", 40, 21, np.uint64), ("ST_TET", 33, 29, np.uint16),
+    ("ST_SIMPLEX4", 9, 7, np.uint32), ("ST_SIMPLEX4", 9, 65, np.uint32), ("ST_SIMPLEX4", 10, 31, np.uint64), ("ST_SIMPLEX4", 10, 40, np.uint16)])
+def test_copies_of_rows_off_boundaries(st, kind, d, inner, dtype):
+    lay = st.Layout(getattr(st, kind), d, inner)
+    nd = st.st_dense_elems(lay)
+    dense = np.random.default_rng(nd).integers(1, np.iinfo(dtype).max, size=nd, dtype=dtype)
+    signed = {2: np.int16, 4: np.int32, 8: np.int64}[dense.itemsize]
+    packed = oracle.pack(dense, lay.kind, d, inner=inner)
+    got = st.st_pack(torch.from_numpy(dense.view(signed)).cuda(), lay)
+    assert np.array_equal(got.cpu().numpy().view(dtype), packed)
+    for fill in (st.ST_FILL_ZERO, st.ST_FILL_SYMMETRIC):
+        want = oracle.unpack(packed, lay.kind, d, inner=inner, fill=fill).reshape(-1)
+        assert np.array_equal(st.st_unpack(got, lay, fill=fill).cpu().numpy().view(dtype), want), fill
+    if dtype == np.uint32:
+        B, C = (workloads.draw((n,), "normal", 5) for n in (packed.size, nd))
+        want = B * oracle.pack(C.view(np.uint32), lay.kind, d, inner=inner).view(np.float32)
+        assert np.array_equal(st.st_thp(dev(B), dev(C), lay).cpu().numpy(), want)
+
+
 # fp32 second moment of more than 128 features on both sides of the line between its two kernels, and of many tiles with few
 # samples, whose sums go round with fewer blocks than rows
 @pytest.mark.parametrize("N,d", [(4900, 129), (5000, 129), (1, 130), (9900, 160), (10100, 160), (33, 193), (1000, 248), (37000, 248), (5, 1300), (70, 2100),
