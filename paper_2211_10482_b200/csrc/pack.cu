@@ -365,8 +365,12 @@ __device__ __forceinline__ I sym_run_row(I d, I a, I b, I c, I x)
 }
 
 // One warp per part of a slice.  Positions from the largest fixed index on: one flat copy.  In front of it lanes run along
-// the words of the positions (up to 32 words each), or a lane group copies a position (`inner` elements) at a time.
-template <int KIND, int ES, typename I>
+// the words of the positions (inv != 0), or a lane group copies a position (`inner` elements) at a time.
+// FORM: 2 both; for tensors of order 3 and 4 with words of 4 bytes and more, whose rows take longer to find, an instance for the
+// words (1) and one for the positions (0).  In the first a lane finds the row of one position of the part for all lanes, but not for
+// the words of 8 bytes of order 3 (tet d = 160, 33 floats, 208 us with a row found for every word, now 196; simplex4 d = 24, 41
+// floats, 31 and 22; tet d = 100, 21 doubles, 50 with rows for every word, 56 from lanes).
+template <int KIND, int ES, int FORM, typename I>
 __global__ void __launch_bounds__(256)
 sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, int parts, int part_rows,
                  int row_bytes, unsigned inv, int group_shift, int64_t packed_rows)
@@ -392,18 +396,37 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
         }
         const I xe = x1 < top ? x1 : top;
         const int words = row_bytes / ES;
-        if (words <= 32) {
-            // lanes along the words of consecutive positions: word e belongs to position e / words (inv: 2^16 / words rounded
-            // up; e < 2^12)
+        if (FORM == 1 || (FORM == 2 && inv != 0)) {
+            // lanes along the words of consecutive positions: word e belongs to position e / words (inv: 2^32 / words rounded up,
+            // exact for e < 2^17 and up to 128 words)
             const unsigned n = xe > x0 ? (unsigned)(xe - x0) * (unsigned)words : 0u;
             E *o = reinterpret_cast<E *>(out + (int64_t)x0 * row_bytes);
+            if (FORM == 1 && (KIND == ST_SIMPLEX4 || ES == 4) && words >= 8) {
+                // a part has at most 32 positions, and each lane finds the row of one for all lanes
+                const I mine = x0 + (I)lane < xe ? sym_row<KIND, I>(d, a, b, c, x0 + (I)lane) : (I)0;
+                for (unsigned e0 = 0; e0 < n; e0 += 32 * SYM_WORDS) {
+                    E v[SYM_WORDS];
+#pragma unroll
+                    for (int u = 0; u < SYM_WORDS; ++u) {
+                        const unsigned e = e0 + 32 * u + (unsigned)lane;
+                        const unsigned dx = __umulhi(e, inv);
+                        const I p = __shfl_sync(0xFFFFFFFFu, mine, (int)dx & 31);
+                        if (e < n) v[u] = ST_BOUNDS_OK(p, packed_rows, 1) ? reinterpret_cast<const E *>(src)[(int64_t)p * words + (e - dx * (unsigned)words)] : E{};
+                    }
+#pragma unroll
+                    for (int u = 0; u < SYM_WORDS; ++u)
+                        if (e0 + 32 * u + (unsigned)lane < n) o[e0 + 32 * u + (unsigned)lane] = v[u];
+                }
+                continue;
+            }
             for (unsigned e0 = (unsigned)lane; e0 < n; e0 += 32 * SYM_WORDS) {
                 E v[SYM_WORDS];
 #pragma unroll
                 for (int u = 0; u < SYM_WORDS; ++u) {
                     const unsigned e = e0 + 32 * u;
                     if (e >= n) continue;
-                    const unsigned dx = (e * inv) >> 16;
+                    // (order 3: the high half of a product costs 7 % there, and below 2^12 that by 2^16 / words does)
+                    const unsigned dx = words == 1 ? e : FORM == 1 && KIND == ST_TET && words <= 32 ? (e * ((inv + 0xFFFF) >> 16)) >> 16 : __umulhi(e, inv);
                     const I p = sym_row<KIND, I>(d, a, b, c, x0 + (I)dx);
                     v[u] = ST_BOUNDS_OK(p, packed_rows, 1) ? reinterpret_cast<const E *>(src)[(int64_t)p * words + (e - dx * (unsigned)words)] : E{};
                 }
@@ -604,20 +627,29 @@ static st_status launch_sym(const void *src, void *dst, const LayoutArgs &a, cud
     }
     // parts of about 2 KiB (4 KiB of 16-byte words), less where there are too few to fill the chip
     const int64_t words = a.row_bytes / ES, nslices = a.dense_rows / a.d;
+    // word by word up to 32 words, and where rows are off 16-byte boundaries up to 128 (positions one by one, in units of 16 bytes
+    // put together from two: [384,384,75] 19.3 us, now 15.4; tet d = 160, 33 floats, 284 and 197; d = 60, 33, 18.8 and 11.4); 2-byte
+    // words gain nothing ([500,500,99] 23.0 and 24.7)
+    const bool flat = words <= (ES >= 4 && ES < 16 && a.row_bytes % 16 != 0 ? 128 : 32);
     int64_t part_rows = words <= 32 ? 256 / words < 8 ? 8 : 256 / words : (2048 + a.row_bytes - 1) / a.row_bytes;
     while (part_rows > 2 && nslices * ((a.d + part_rows - 1) / part_rows) < 16 * (int64_t)sm_count_or_default()) part_rows = (part_rows + 1) / 2;
-    const unsigned inv = words <= 32 ? (unsigned)((65536 + words - 1) / words) : 0u;
+    const unsigned inv = !flat ? 0u : words == 1 ? 1u : (unsigned)(0xFFFFFFFFu / words + 1);
     const int64_t parts = (a.d + part_rows - 1) / part_rows;
     int shift = 0;
     while (shift < 5 && (int64_t(16) << shift) < a.row_bytes) ++shift;
     const int64_t items = nslices * parts;
     const int64_t want = (items + 7) / 8, cap = (int64_t)sm_count_or_default() * 16;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
-    if (small && items < (int64_t(1) << 31))
-        return launch(sym_slice_kernel<KIND, ES, unsigned>, grid, 256, 0, s, in, out, (unsigned)a.d, (unsigned)nslices, (int)parts, (int)part_rows,
+    auto run = [&](auto form) {
+        constexpr int FORM = decltype(form)::value;
+        if (small && items < (int64_t(1) << 31))
+            return launch(sym_slice_kernel<KIND, ES, FORM, unsigned>, grid, 256, 0, s, in, out, (unsigned)a.d, (unsigned)nslices, (int)parts,
+                          (int)part_rows, (int)a.row_bytes, inv, shift, a.packed_rows);
+        return launch(sym_slice_kernel<KIND, ES, FORM, int64_t>, grid, 256, 0, s, in, out, a.d, nslices, (int)parts, (int)part_rows,
                       (int)a.row_bytes, inv, shift, a.packed_rows);
-    return launch(sym_slice_kernel<KIND, ES, int64_t>, grid, 256, 0, s, in, out, a.d, nslices, (int)parts, (int)part_rows, (int)a.row_bytes, inv, shift,
-                  a.packed_rows);
+    };
+    if constexpr (KIND == ST_TRI_UPPER || ES == 2) return run(std::integral_constant<int, 2>{});
+    else return flat ? run(std::integral_constant<int, 1>{}) : run(std::integral_constant<int, 0>{});
 }
 
 template <int KIND, int ES, bool PACK>
