@@ -113,7 +113,10 @@ __device__ __forceinline__ bool m2s_output(int k, int item, int nbk, bool dense,
 // BULK: rows start on 16-byte boundaries and arrive by bulk copies, in shared memory at their own pitch; otherwise
 // they are copied word by word to a pitch rounded up to 16 bytes (one copy instruction per 32 words, against more
 // than 64 FMA instructions).  Either way a tile that reaches past column d reads whatever follows the row: only
-// sums that are dropped contain it.  [50021,75]: 23 us the call, 71 with the plain 64 x 64 tiles that served it before.
+// sums that are dropped contain it.  [50021,75]: 18 us the call, 71 with the plain 64 x 64 tiles that served it before.
+// What bounds it: two warps to a scheduler issue in 68 % of the cycles ([300000,64]; FMA pipe 59 %), the rest waits for operands.
+// Packed FMAs (two to an instruction) are slower here, [1000000,64] 109 us instead of 102, and so is the next row's operands loaded
+// ahead of this one's FMAs, 107: both take registers from what the compiler overlaps by itself.
 // CLUSTER: few samples, one launch.  A cluster of M2S_CLUSTER blocks (gridDim.x) owns nitems work items (gridDim.y clusters),
 // its blocks own slices of the samples, and the sums of the blocks are added through distributed shared memory instead of
 // partials and a second launch.
@@ -162,8 +165,10 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
 
     const int nstages = (n_end > n_begin) ? (int)((n_end - n_begin + stage_rows - 1) / stage_rows) : 0;
     const bool contiguous = (a.ldx == a.d);
-    const int copy_r = tid / a.d, copy_c = tid - copy_r * a.d;                   // word copies: first element of this thread,
-    const int copy_dr = nthreads / a.d, copy_dc = nthreads - copy_dr * a.d;      // and the way to its next one
+    // Word copies: whole rows at a time by as many threads as make whole rows, so that a thread stays in its column and a copy takes
+    // three instructions instead of fourteen ([50021,75] 21.4 us the call, now 19.2; [1000000,13] 38.2 and 30.3).
+    const int copy_dr = nthreads >= a.d ? nthreads / a.d : 1;
+    const int copy_r = tid / a.d, copy_c = tid - copy_r * a.d;
     // the rows of a stage arrive by bulk copies issued from warp 0: one copy when the rows are
     // contiguous in memory, one per row otherwise; rows past the end of the slice are not copied
     // and not read
@@ -173,13 +178,15 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
         const int rows = (n_end - n0 < stage_rows) ? (int)(n_end - n0) : stage_rows;
         float *dst = smem + buf * stage_floats;
         if (!BULK) {
-            const float *src = a.X + n0 * a.ldx;
-            int r = copy_r, c = copy_c;
-            while (r < rows) {
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(tc::smem_u32(dst + r * a.pitch + c)), "l"(src + r * a.ldx + c));
-                r += copy_dr;
-                c += copy_dc;
-                if (c >= a.d) { c -= a.d; ++r; }
+            if (copy_r >= copy_dr) return;
+            for (int c = copy_c; c < a.d; c += nthreads) {                       // once, but for rows of more words than threads
+                const float *src = a.X + (n0 + copy_r) * a.ldx + c;
+                uint32_t to = tc::smem_u32(dst + copy_r * a.pitch + c);
+                const int64_t src_step = copy_dr * a.ldx;
+                const uint32_t to_step = (uint32_t)(copy_dr * a.pitch) * 4u;
+#pragma unroll 4
+                for (int r = copy_r; r < rows; r += copy_dr, src += src_step, to += to_step)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(src));
             }
             return;
         }
@@ -274,13 +281,17 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
     if (parts > a.rg) parts = a.rg;
     float *mine = CLUSTER ? red + 128 * cells + M2S_MAX_THREADS : a.partials + (size_t)blockIdx.x * nout;
     if (parts == 1) {
+        const int dk = nthreads / nitems, dt = nthreads - dk * nitems;     // (a division for each: [50021,75] 19.2 us, now 18.2)
+        int k = tid / nitems, t = tid - k * nitems;
         for (int o = tid; o < nout; o += nthreads) {
-            const int k = o / nitems, t = o - k * nitems;
             const float *p = red + k * cells + t;
             float sum = 0.f;
 #pragma unroll 8
             for (int g = 0; g < a.rg; ++g) sum += p[g * nitems];
             mine[o] = sum;
+            k += dk;
+            t += dt;
+            if (t >= nitems) { t -= nitems; ++k; }
         }
     } else {
         float *scratch = red + 128 * cells;            // [parts][nout]
