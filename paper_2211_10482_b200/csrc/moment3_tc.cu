@@ -229,7 +229,7 @@ moment3_tc_kernel(const __grid_constant__ Args a)
             const int q4 = warp & 3;                                // lanes 32*q4 .. 32*q4+31 of tensor memory
             for (int ti = warp >> 2; ti < tg; ti += PRODUCERS / 4) {
                 const Tile t = tiles[ti];
-                const int ncols = a.dcols - TJ * t.jb;
+                const int ncols = a.d - TJ * t.jb;                  // (with the columns that fill up to dcols [40009,50] bf16 35.7 us, without 33.4)
                 uint32_t v[DP];
 #pragma unroll
                 for (int c0 = 0; c0 < DP; c0 += 16)                 // all loads of the tile in flight, one wait
@@ -245,7 +245,7 @@ moment3_tc_kernel(const __grid_constant__ Args a)
                         if (c0 < ncols) {
 #pragma unroll
                             for (int e = 0; e < 16; ++e)
-                                if (ST_BOUNDS_OK(t.part + r + (c0 + e) * BM, a.part_elems, 4)) dst[(c0 + e) * BM] = __uint_as_float(v[c0 + e]);
+                                if (c0 + e < ncols && ST_BOUNDS_OK(t.part + r + (c0 + e) * BM, a.part_elems, 4)) dst[(c0 + e) * BM] = __uint_as_float(v[c0 + e]);
                         }
                 }
             }
@@ -486,7 +486,7 @@ static Plan plan(int64_t N, int64_t d, bool bf16)
             p.tiles[n].jb = (unsigned char)jb;
             cols[n] = p.dcols - jb * TJ;
             p.tiles[n].part = p.part_elems;
-            p.part_elems += cols[n] * BM;
+            p.part_elems += ((int)d - jb * TJ) * BM;      // columns past d are not stored
             ++n;
         }
     p.ntiles = n;
