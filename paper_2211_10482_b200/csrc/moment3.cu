@@ -27,6 +27,7 @@
 #include "st_common.cuh"
 #include "st_index.cuh"
 #include <algorithm>
+#include <type_traits>
 #include <mutex>
 #include <vector>
 
@@ -316,40 +317,53 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
     }
 }
 
-// out[e] = sum over slices of partials[slice][e], in a fixed order.  A block covers 32 consecutive
-// elements; warp w adds the slices w, w+8, w+16, ..., five loads at a time, then the eight partial sums are added
-// through shared memory.  Latency and placement bound it: with twelve loads at a time the blocks take more registers
-// than the running kernel leaves, and start later ([4096,24] 12.2 us the call, now 11.2; twenty 14.7).
-constexpr int SUM_GROUPS = 8;
-__global__ void __launch_bounds__(32 * SUM_GROUPS)
+// out[e] = sum over slices of partials[slice][e], in a fixed order.  A block covers 32 V consecutive elements, V of them a lane (four
+// where that is aligned and leaves blocks for the chip); warp w of W adds the slices w, w + W, ..., five loads at a time, then
+// the sums of the warps are added through shared memory.  Latency and placement bound it: with twelve loads at a time the blocks
+// take more registers than the running kernel leaves, and start later ([4096,24] 12.2 us the call, with five 11.2, twenty 14.7);
+// with V = 1 and eight warps whatever the slices [4096,24] 11.9 us the call, now 10.2, [6000,128] 147 and 139, [50000,21] 25.1 and 23.4.
+constexpr int SUM_BATCH = 5;
+constexpr int64_t SUM_V4 = 128 * 64;       // elements from where V = 4 ([4096,24], 2600 of them, 11.1 us with it and 10.2 without)
+template <int V, int W>
+__global__ void __launch_bounds__(32 * W)
 sum_slices_kernel(const float *partials, float *out, int64_t elems, int slices)
 {
-    __shared__ float part[SUM_GROUPS][32];
+    __shared__ float part[W][32 * V];
     pdl_wait();
     pdl_trigger();
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int64_t e = (int64_t)blockIdx.x * 32 + lane;
-    float s = 0.f;
+    const int64_t e0 = (int64_t)blockIdx.x * (32 * V), e = e0 + lane * V;
+    float s[V] = {};
     if (e < elems) {
-        constexpr int BATCH = 5;
-        for (int k0 = g; k0 < slices; k0 += BATCH * SUM_GROUPS) {
-            float v[BATCH];
+        for (int k0 = g; k0 < slices; k0 += SUM_BATCH * W) {
+            float v[SUM_BATCH][V] = {};
 #pragma unroll
-            for (int u = 0; u < BATCH; ++u) {
-                const int k = k0 + u * SUM_GROUPS;
-                v[u] = k < slices ? __ldcg(&partials[(size_t)k * elems + e]) : 0.f;
+            for (int u = 0; u < SUM_BATCH; ++u) {
+                const int k = k0 + u * W;
+                if (k >= slices) continue;
+                const float *p = &partials[(size_t)k * elems + e];
+                if constexpr (V == 4) {
+                    const float4 x = __ldcg(reinterpret_cast<const float4 *>(p));
+                    v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
+                } else {
+                    v[u][0] = __ldcg(p);
+                }
             }
 #pragma unroll
-            for (int u = 0; u < BATCH; ++u) s += v[u];
+            for (int u = 0; u < SUM_BATCH; ++u)
+#pragma unroll
+                for (int x = 0; x < V; ++x) s[x] += v[u][x];
         }
     }
-    part[g][lane] = s;
-    __syncthreads();
-    if (g == 0 && e < elems) {
-        float t = part[0][lane];
 #pragma unroll
-        for (int w = 1; w < SUM_GROUPS; ++w) t += part[w][lane];
-        out[e] = t;
+    for (int x = 0; x < V; ++x) part[g][lane * V + x] = s[x];
+    __syncthreads();
+    const int o = threadIdx.x;
+    if (o < 32 * V && e0 + o < elems) {
+        float t = part[0][o];
+#pragma unroll
+        for (int w = 1; w < W; ++w) t += part[w][o];
+        out[e0 + o] = t;
     }
 }
 
@@ -601,7 +615,17 @@ static st_status moment3_launch(const float *X, int64_t N, int64_t d, int64_t ld
                        : !aligned ? run(moment3_kernel<WARPS, 0, false, false>)
                        : p.dp == M3_PARAM_D ? run(moment3_kernel<WARPS, M3_PARAM_D, true, false>) : run(moment3_kernel<WARPS, 0, true, false>);
     if (rc != ST_OK) return rc;
-    return launch(sum_slices_kernel, dim3((unsigned)((p.out_elems + 31) / 32)), 32 * SUM_GROUPS, 0, stream, a.partials, out, p.out_elems, p.slices);
+    auto sum = [&](auto v, auto w) {
+        constexpr int V = decltype(v)::value, W = decltype(w)::value;
+        return launch(sum_slices_kernel<V, W>, dim3((unsigned)((p.out_elems + 32 * V - 1) / (32 * V))), 32u * W, 0, stream, a.partials, out, p.out_elems,
+                      p.slices);
+    };
+    auto with_warps = [&](auto v) {
+        return p.slices <= 8 * SUM_BATCH ? sum(v, std::integral_constant<int, 8>{})
+             : p.slices <= 16 * SUM_BATCH ? sum(v, std::integral_constant<int, 16>{}) : sum(v, std::integral_constant<int, 32>{});
+    };
+    if (p.out_elems % 4 == 0 && p.out_elems >= SUM_V4 && aligned16(a.partials)) return with_warps(std::integral_constant<int, 4>{});
+    return with_warps(std::integral_constant<int, 1>{});
 }
 
 size_t moment3_tc_workspace(int64_t N, int64_t d, bool bf16);
