@@ -24,6 +24,7 @@
 #include "tc_common.cuh"
 #include "moment2_rule.cuh"
 #include <tuple>
+#include <type_traits>
 
 namespace st {
 
@@ -333,37 +334,57 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
     }
 }
 
-// out[p(ci,cj)] = sum over the slices of element (k, item) of the partials: a block owns 32 elements, warp w adds the
-// slices w, w + 8, ..., seven loads at a time, then the eight sums are added in order (a fixed order).  Twenty at a time
-// (all that there are) take registers that the running kernel does not leave: [20000,64] 10.8 us the call, now 9.9.
-__global__ void __launch_bounds__(256)
+// out[p(ci,cj)] = sum over the slices of element (k, item) of the partials: a block owns 32 V elements, V of them a lane, warp w of W
+// adds the slices w, w + W, ..., five loads at a time, then the W sums are added in order (a fixed order).  Latency and
+// placement bound it: twenty loads at a time take registers that the running kernel does not leave ([20000,64] 10.8 us the call,
+// with seven 9.9); with eight warps whatever the slices, seven loads at a time, [50021,75] 18.2 us, now 17.6, [30000,120] 22.5 and
+// 20.6, [50000,150] 62 and 49.
+constexpr int M2S_SUM_BATCH = 5, M2S_SUM_V4 = 24;      // work items from where V = 4 ([50021,75], 28 items, 17.7 us with V = 1, 17.6)
+template <int V, int W>
+__global__ void __launch_bounds__(32 * W)
 moment2_small_reduce_kernel(const float *partials, float *out, int d, int nbk, int slices,
                             int dense, int nitems)
 {
-    __shared__ float part[8][32];
+    __shared__ float part[W][32 * V];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int o = blockIdx.x * 32 + lane;              // < nitems * 128, a multiple of 32
-    const int k = o / nitems, item = o - k * nitems;
-    int64_t at;
-    const bool use = m2s_output(k, item, nbk, dense != 0, d, at);
+    const int o0 = blockIdx.x * 32 * V;                // < nitems * 128, a multiple of 32 V
+    int64_t at = -1;
+    bool use = false;
+    if (threadIdx.x < 32 * V) {
+        const int o = o0 + (int)threadIdx.x, k = o / nitems, item = o - k * nitems;
+        use = m2s_output(k, item, nbk, dense != 0, d, at);
+    }
     pdl_wait();
     pdl_trigger();
     const size_t stride = (size_t)nitems * 128;
-    float s = 0.f;
-    for (int k0 = warp; k0 < slices; k0 += 8 * 7) {
-        float v[7];
+    float s[V] = {};
+    const float *p = partials + o0 + lane * V;
+    for (int k0 = warp; k0 < slices; k0 += W * M2S_SUM_BATCH) {
+        float v[M2S_SUM_BATCH][V] = {};
 #pragma unroll
-        for (int u = 0; u < 7; ++u) v[u] = (use && k0 + 8 * u < slices) ? __ldcg(partials + (size_t)(k0 + 8 * u) * stride + o) : 0.f;
+        for (int u = 0; u < M2S_SUM_BATCH; ++u) {
+            if (k0 + W * u >= slices) continue;
+            const float *q = p + (size_t)(k0 + W * u) * stride;
+            if constexpr (V == 4) {
+                const float4 x = __ldcg(reinterpret_cast<const float4 *>(q));
+                v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
+            } else {
+                v[u][0] = __ldcg(q);
+            }
+        }
 #pragma unroll
-        for (int u = 0; u < 7; ++u) s += v[u];
+        for (int u = 0; u < M2S_SUM_BATCH; ++u)
+#pragma unroll
+            for (int x = 0; x < V; ++x) s[x] += v[u][x];
     }
-    part[warp][lane] = s;
-    __syncthreads();
-    if (warp != 0 || !use) return;
-    s = part[0][lane];
 #pragma unroll
-    for (int w = 1; w < 8; ++w) s += part[w][lane];
-    if (ST_BOUNDS_OK(at, tri_rows(d), 2)) out[at] = s;
+    for (int x = 0; x < V; ++x) part[warp][lane * V + x] = s[x];
+    __syncthreads();
+    if (!use) return;
+    float sum = part[0][threadIdx.x];
+#pragma unroll
+    for (int w = 1; w < W; ++w) sum += part[w][threadIdx.x];
+    if (ST_BOUNDS_OK(at, tri_rows(d), 2)) out[at] = sum;
 }
 
 struct M2SmallPlan {
@@ -537,7 +558,16 @@ st_status moment2_small(const float *X, int64_t N, int64_t d, int64_t ldx, float
     };
     const st_status rc = bulk ? run(moment2_small_kernel<true, false>) : run(moment2_small_kernel<false, false>);
     if (rc != ST_OK) return rc;
-    return launch(moment2_small_reduce_kernel, (unsigned)(p.nitems * 128 / 32), 256, 0, stream, a.partials, out, (int)d, p.nbk, p.slices, a.dense, p.nitems);
+    auto sum = [&](auto v, auto w) {
+        constexpr int V = decltype(v)::value, W = decltype(w)::value;
+        return launch(moment2_small_reduce_kernel<V, W>, (unsigned)(p.nitems * 4 / V), 32u * W, 0, stream, a.partials, out, (int)d, p.nbk, p.slices, a.dense,
+                      p.nitems);
+    };
+    auto with_warps = [&](auto v) {
+        return p.slices <= 8 * M2S_SUM_BATCH ? sum(v, std::integral_constant<int, 8>{})
+             : p.slices <= 16 * M2S_SUM_BATCH ? sum(v, std::integral_constant<int, 16>{}) : sum(v, std::integral_constant<int, 32>{});
+    };
+    return p.nitems >= M2S_SUM_V4 ? with_warps(std::integral_constant<int, 4>{}) : with_warps(std::integral_constant<int, 1>{});
 }
 
 }  // namespace st
