@@ -156,7 +156,8 @@ __device__ __forceinline__ void m2tc_add_in_l2(float *p, const uint32_t (&r)[32]
 #include "moment2_exact.cuh"
 namespace st {
 
-template <int MODE>
+// EXT: some tiles carry left-over columns (an instance of its own: the registers of their epilogue cost small calls without any 2 to 6 %).
+template <int MODE, bool EXT>
 __global__ void __launch_bounds__(MODE == M2_CONV ? m2tc::THREADS + m2tc::CONV_THREADS : m2tc::THREADS, 1)
 moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ m2tc::Args a)
 {
@@ -190,8 +191,8 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     const int FLUSH_CHUNKS = MODE == M2_BF16 && width <= HALF ? S::FLUSH_CHUNKS / 2 : S::FLUSH_CHUNKS;
     const bool alias = diag && width == BN;             // A columns == B columns in both blocks: one load serves both
     const bool lead = diag && rows <= HALF;             // all rows in the first block, whose A holds its half of B as well
-    // (a tile that carries left-over columns is on the diagonal, and full; products of pairs have none)
-    const int ext = MODE == M2_SPLIT ? 0 : 16 * a.tab.ext[tile], ecol = 8 * a.tab.ext_col;
+    // (a tile that carries left-over columns is on the diagonal, and full)
+    const int ext = EXT ? 16 * a.tab.ext[tile] : 0, ecol = 8 * a.tab.ext_col;
     const bool corner = ext > 0 && a.tab.corner && tile == a.tab.carrier[a.tab.next - 1];
     const int chunks_per_split = (a.chunks_total + nsplit - 1) / nsplit;
     const int c_begin = split * chunks_per_split;
@@ -415,7 +416,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         const int row0 = (int)rank * HALF + q * 32;
         const bool used = row0 < rows;
         const int c_first = diag ? row0 : 0;         // row0 is a multiple of 32
-        float *dst = a.partials + (size_t)blockIdx.x * (MODE == M2_SPLIT ? HALF * BN : a.pitch) + (q * 32 + lane) * 4;         // columns c .. c+3: + c HALF
+        float *dst = a.partials + (size_t)blockIdx.x * (EXT ? a.pitch : HALF * BN) + (q * 32 + lane) * 4;         // columns c .. c+3: + c HALF
         // columns in use: c_first .. width, and where the tile carries left-over columns all in between and after them
         const int c_end = ext > 0 ? BN + (ext * (corner && q * 32 < ext / 2 ? 2 : 1) + 31) / 32 * 32 : width;
         const uint32_t leader_acc_empty0 = map_to_cta(smem_u32(&acc_empty[0]), 0);
@@ -502,7 +503,8 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 // PAIRS: X holds pair features in the order of pair_layout.cuh; pairs[column] is the pair of a column, and an entry goes
 // to the place of its 4-tuple in the packed 4-simplex, if this is the product that was chosen for that tuple.
 __host__ __device__ inline int m2tc_sum_warps(int nsplit) { return nsplit <= 4 ? 1 : nsplit <= 8 ? 2 : nsplit <= 16 ? 4 : 8; }
-template <bool PAIRS>
+// EXT: some tiles carry left-over columns (an instance of its own: with them in it the others took 1 to 2 us longer).
+template <bool PAIRS, bool EXT>
 __global__ void __launch_bounds__(256)
 moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features, int within, int64_t out_elems,
                          const unsigned *pairs, int pitch, const __grid_constant__ m2tc::TileTable tab)
@@ -511,8 +513,8 @@ moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features,
     __shared__ float4 part[2][8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the tiles, then the left-over columns of each tile that carries them, then the corner
-    const int e = PAIRS ? -1 : (int)blockIdx.x - tab.ntiles;
-    const bool corner = !PAIRS && e >= (int)tab.next;
+    const int e = EXT ? (int)blockIdx.x - tab.ntiles : -1;
+    const bool corner = EXT && e >= (int)tab.next;
     const int tile = e < 0 ? (int)blockIdx.x : tab.carrier[corner ? (int)tab.next - 1 : e], ext = 16 * tab.ext[tile];
     const int row = 8 * (corner ? tab.ext_col : tab.row[tile]), col = 8 * (e < 0 ? tab.col[tile] : tab.ext_col);
     const int rows = corner ? min(ext, d - row) : tab.rows[tile], block_rows = corner ? ext / 2 : HALF;
@@ -521,7 +523,7 @@ moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features,
     const int first = tab.first[tile], nsplit = tab.first[tile + 1] - first;
     const int wps = m2tc_sum_warps(nsplit);
     const int per = 8 / wps, w0 = warp % wps;
-    const int block = PAIRS ? HALF * BN : pitch;           // floats of a block's partial tile
+    const int block = EXT ? pitch : HALF * BN;           // floats of a block's partial tile
     const size_t stride = (size_t)2 * block;
     constexpr int BATCH = 4;
     pdl_wait();
@@ -533,7 +535,7 @@ moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features,
         // what is loaded does not wait for what has to be looked up
         const bool use = u < units && r < rows && gj + 4 > (PAIRS && gi >= within ? 0 : gi);
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int second = PAIRS ? r >> 7 : r >= block_rows ? 1 : 0, in_block = PAIRS ? r & 127 : r - second * block_rows;
+        const int second = EXT ? r >= block_rows ? 1 : 0 : r >> 7, in_block = EXT ? r - second * block_rows : r & 127;
         const float *base = partials + (size_t)(2 * first + second) * block + (at_col + c) * HALF + in_block * 4;
         for (int k0 = w0; k0 < nsplit; k0 += BATCH * wps) {
             float4 v[BATCH];
@@ -597,8 +599,21 @@ static double m2tc_exact_cost(int rows, int width, bool diag)
     return rows > m2tc::HALF ? 0.88 : 0.47 + 0.26 * rows / m2tc::HALF;
 }
 
-// Columns that are left over after `full` tiles of 256: carried along by the tiles on the diagonal, or tiles of their own.
-static bool m2tc_carry(int full, int left_over) { return full > 0 && left_over > 0 && left_over <= m2tc::HALF; }
+// Columns that are left over after `full` tiles of 256: carried along by the tiles on the diagonal, or tiles of their own.  The
+// epilogue of a tile that carries them has up to twice the columns, and the sum more parts: a fixed time that the samples of a
+// cluster, in cycles of their stages, have to outweigh.  us, tiles of their own / carried: TF32 [20000,300] 17.9 / 19.1, [60000,300]
+// 35.8 / 29.0, [20000,380] 19.7 / 24.1, [60000,380] 39.6 / 36.9; bf16 [20000,264] 13.3 / 15.2, [60000,264] 22.7 / 20.8, [20000,800] 26.3 /
+// 27.7, [60000,800] 59 / 53; split [6000,520] 19.5 / 21.7, [20000,520] 39.4 / 36.0, [20000,384] 24.4 / 27.4, [60000,384] 51.5 / 43.8.
+template <int MODE>
+static bool m2tc_carry(int64_t N, int full, int left_over)
+{
+    using S = m2tc::Shape<MODE>;
+    if (MODE == M2_EXACT || full == 0 || left_over == 0 || left_over > m2tc::HALF) return false;
+    const int tiles = full * (full + 1) / 2, ext = (left_over + 15) / 16 * 16;
+    const double sum = tiles + (full + 1) * (m2tc_cost(m2tc::BN, ext, 1) - 1);
+    const double cycles = (double)((N + S::KROWS - 1) / S::KROWS) * sum * (MODE == M2_CONV ? 1226 : 512) / (sm_count_or_default() / 2);
+    return cycles >= (MODE == M2_CONV ? 1.6 : 1.0) * (6000 + 130 * ext + 3500 * (tiles - 1));
+}
 
 // Tiles of a plan while it is made.
 struct M2TcTiles {
@@ -703,7 +718,7 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
     M2TcTiles t{&p, 0, {}};
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
     const int full = (int)(d / BM), left_over = (int)(d % BM);
-    const bool carry = MODE != M2_EXACT && !dense && m2tc_carry(full, left_over);
+    const bool carry = !dense && m2tc_carry<MODE>(N, full, left_over);
     const int ext = carry ? (left_over + 15) / 16 * 16 : 0;
     const int nt = carry ? full : (int)((d + BM - 1) / BM);
     for (int tn = 0; tn < nt; ++tn)
@@ -786,10 +801,11 @@ static const M2TcPlan &m2tc_plan_pairs(int64_t N, const PairLayout &L)
     return p;
 }
 
-template <int MODE> static auto m2tc_kernel()
+template <int MODE> static auto m2tc_kernel(bool ext)
 {
     if constexpr (MODE == M2_EXACT) return moment2_exact_kernel;
-    else return moment2_tc_kernel<MODE>;
+    else if constexpr (MODE == M2_SPLIT) return moment2_tc_kernel<MODE, false>;        // products of pairs carry none
+    else return ext ? moment2_tc_kernel<MODE, true> : moment2_tc_kernel<MODE, false>;
 }
 
 // Launches the tile kernel and the sum of its partial tiles.  rows: rows of X in memory; pairs: X holds the pair features
@@ -810,7 +826,7 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     a.chunks_total = q.chunks_total; a.stages = q.stages; a.nb = q.nb; a.na = q.na; a.pitch = q.pitch; a.lo_row0 = (int)lo_row0; a.d = (int)d;
     a.X = (const float *)X; a.N = rows; a.ldx = ldx;
     a.tab = q.tab;
-    const auto kernel = m2tc_kernel<MODE>();
+    const auto kernel = m2tc_kernel<MODE>(q.tab.next > 0);
     if (!ensure_dynamic_smem(kernel, q.smem)) return ST_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)q.tab.first[q.tab.ntiles]);
@@ -840,7 +856,8 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     const unsigned most = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
     if (blocks > most) blocks = most < 64 ? 64 : most;
     const dim3 rgrid((unsigned)(q.tab.ntiles + q.tab.next + q.tab.corner), blocks);
-    return launch(pairs ? moment2_tc_reduce_kernel<true> : moment2_tc_reduce_kernel<false>, rgrid, 256, 0, stream, partials, out, (int)d,
+    return launch(pairs ? moment2_tc_reduce_kernel<true, false> : q.tab.next > 0 ? moment2_tc_reduce_kernel<false, true> : moment2_tc_reduce_kernel<false, false>,
+                  rgrid, 256, 0, stream, partials, out, (int)d,
                   features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.pitch, q.tab);
 }
 
