@@ -256,6 +256,23 @@ constexpr int ROWSUM_LONG = 64;              // mean number of slots of a reache
 // call, now 17).  BATCH: loads at a time.  The one row of a slice i has thousands of slots and its sum is a chain of round
 // trips ([3000,50000,64], R = 32: eight 92 us, sixteen 41); where rows have few, the registers of sixteen keep blocks from
 // starting beside the running kernel ([900,900,48], R = 64, split: eight 76.5 us, sixteen 80).
+// The slots of row `row` of A; n = 0: a row of zeros, -1: out of range.
+__device__ __forceinline__ void mttkrp_row_slots(const MttkrpRows &m, int64_t row, int64_t i_off, int unit_shift, int ksplit, int64_t &first, int64_t &n)
+{
+    const int64_t i = row - i_off;
+    first = n = 0;
+    if (i < 0 || i >= m.I) return;
+    int64_t s, e;
+    if (m.mode == MK_PACKED) { s = tri_row_start(m.I, i); e = s + (m.I - i); }
+    else { s = i * m.div; e = s + m.div; }
+    if (e > m.rows) e = m.rows;
+    if (e <= s) return;
+    const int64_t u0 = s >> unit_shift, u1 = (e - 1) >> unit_shift;
+    first = (u0 + i) * ksplit;
+    n = (u1 - u0 + 1) * ksplit;
+    if (!ST_BOUNDS_OK(first + n - 1, mttkrp_slots(m.rows, 1 << unit_shift, m.I, ksplit), 6)) n = -1;
+}
+
 template <int BATCH>
 __global__ void __launch_bounds__(256, BATCH > 8 ? 1 : 8)
 mttkrp_rowsum_kernel(const float *part, float *A, int64_t I_full, int64_t i_off, MttkrpRows m, int R, int unit_shift, int ksplit)
@@ -264,21 +281,7 @@ mttkrp_rowsum_kernel(const float *part, float *A, int64_t I_full, int64_t i_off,
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     int64_t ii = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     int64_t first, n;
-    // the slots of row ii; n = 0: a row of zeros
-    auto slots_of = [&](int64_t row) {
-        const int64_t i = row - i_off;
-        first = n = 0;
-        if (i < 0 || i >= m.I) return;
-        int64_t s, e;
-        if (m.mode == MK_PACKED) { s = tri_row_start(m.I, i); e = s + (m.I - i); }
-        else { s = i * m.div; e = s + m.div; }
-        if (e > m.rows) e = m.rows;
-        if (e <= s) return;
-        const int64_t u0 = s >> unit_shift, u1 = (e - 1) >> unit_shift;
-        first = (u0 + i) * ksplit;
-        n = (u1 - u0 + 1) * ksplit;
-        if (!ST_BOUNDS_OK(first + n - 1, mttkrp_slots(m.rows, 1 << unit_shift, m.I, ksplit), 6)) n = -1;
-    };
+    auto slots_of = [&](int64_t row) { mttkrp_row_slots(m, row, i_off, unit_shift, ksplit, first, n); };
     if (ii < I_full) slots_of(ii);                             // the first row's do not have to wait
     pdl_wait();
     pdl_trigger();
@@ -316,12 +319,54 @@ mttkrp_rowsum_kernel(const float *part, float *A, int64_t I_full, int64_t i_off,
     }
 }
 
+// The same with four warps to a row, two rows to a block: warp w adds slots w, w + 4, ..., eight loads at a time, and the four sums are
+// added in order.  For rows few enough that a block for every two of them starts at once: one batch of loads where one warp took
+// several after each other.  us the call, a warp to a row / four: [300,300,128], R = 64, split 23.5 / 21.8; [1000,1000,40], R = 32, fp32
+// 69.8 / 67.4; [700,700,200], R = 32, split 54.5 / 53.0; slice i of [100,50000,64] 41.3 / 26.6; but with three slots a row
+// [200,200,300], R = 64, fp32 49.2 / 50.2, with fewer [16,16,16], R = 16 7.0 / 7.3.
+constexpr int ROWSUM_WARPS = 4, ROWSUM_FEW = 4;            // ROWSUM_FEW: mean number of slots of a reached row from which it pays
+__global__ void __launch_bounds__(256)
+mttkrp_rowsum_few_kernel(const float *part, float *A, int64_t I_full, int64_t i_off, MttkrpRows m, int R, int unit_shift, int ksplit)
+{
+    constexpr int ROWS = 8 / ROWSUM_WARPS, BATCH = 8;
+    __shared__ float sums[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = warp % ROWSUM_WARPS;
+    const int64_t ii = (int64_t)blockIdx.x * ROWS + warp / ROWSUM_WARPS;
+    int64_t first = 0, n = -1;
+    if (ii < I_full) mttkrp_row_slots(m, ii, i_off, unit_shift, ksplit, first, n);
+    pdl_wait();
+    pdl_trigger();
+    for (int r0 = 0; r0 < R; r0 += 32) {
+        const int r = r0 + lane;
+        float sum = 0.f;
+        const float *p = part + first * R + r;
+        for (int64_t k0 = w; k0 < n; k0 += ROWSUM_WARPS * BATCH) {
+            float t[BATCH];
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) t[u] = k0 + ROWSUM_WARPS * u < n && r < R ? __ldcg(p + (k0 + ROWSUM_WARPS * u) * R) : 0.f;
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) sum += t[u];
+        }
+        sums[warp][lane] = sum;
+        __syncthreads();
+        if (w == 0 && n >= 0 && r < R) {
+#pragma unroll
+            for (int v = 1; v < ROWSUM_WARPS; ++v) sum += sums[warp + v][lane];
+            A[ii * R + r] = sum;
+        }
+        __syncthreads();
+    }
+}
+
 st_status mttkrp_rowsum_launch(const float *part, float *A_full, int64_t I_full, int64_t i_off, const MttkrpRows &m,
                                int R, int unit_rows, int ksplit, cudaStream_t stream)
 {
     int shift = 0;                                             // units are powers of two
     while ((1 << shift) < unit_rows) ++shift;
     const int64_t want = (I_full + 7) / 8, cap = (int64_t)sm_count_or_default() * ROWSUM_BLOCKS;
+    const int64_t blocks = (I_full * ROWSUM_WARPS + 7) / 8;
+    if (blocks <= (int64_t)sm_count_or_default() * 8 && m.rows / unit_rows * ksplit >= ROWSUM_FEW * m.I)
+        return launch(mttkrp_rowsum_few_kernel, (unsigned)blocks, 256, 0, stream, part, A_full, I_full, i_off, m, R, shift, ksplit);
     const bool many = m.rows / unit_rows / m.I * ksplit >= ROWSUM_LONG;
     return launch(many ? mttkrp_rowsum_kernel<16> : mttkrp_rowsum_kernel<8>, (unsigned)(want < cap ? want : cap), 256, 0, stream, part, A_full, I_full, i_off, m, R, shift, ksplit);
 }

@@ -1345,6 +1345,18 @@ def test_a_buffer_that_a_call_would_write_past_is_refused_before_anything_runs(s
                 call(ws=bad)
 
 
+# row sums with four warps to a row: more slots than one batch of all warps, fewer than one, rows of none, a last block of one row,
+# a last group of columns that is not full
+@pytest.mark.parametrize("I,J,R", [(9, 9001, 8), (31, 2000, 48), (2, 33, 96), (5, 5000, 64)])
+def test_mttkrp_slice_of_few_rows(st, I, J, R):
+    K = 8
+    B, C, D = (workloads.draw(s, "normal", 60 + i) for i, s in enumerate(((J, K), (J, R), (K, R))))
+    A = st.st_mttkrp_slice(dev(B), dev(C), dev(D), I, fixed_i=I - 1).cpu().numpy()
+    Y, S = (np.einsum("jk,jr,kr->r", *(f(v.astype(np.float64)) for v in (B, C, D))) for f in (lambda v: v, np.abs))
+    assert np.max(np.abs(A[I - 1] - Y) / S) <= TOL_F32
+    assert not A[:I - 1].any()
+
+
 # row sums: a row of more slots than are loaded at a time (sixteen, eight, a remainder) and rows of none, more rows than the
 # warps of the grid; slices whose rows of A have one fibre each, several to a unit and a ragged last unit
 @pytest.mark.parametrize("flag_name,R,tol", [("f32", 64, TOL_F32), ("tf32", 32, 5e-3), ("split", 32, TOL_F32)])
