@@ -15,9 +15,11 @@
 // Accumulators of all tiles of a block stay in tensor memory for the block's whole sample
 // range; two to eight blocks ("groups") share one sample range and its tiles, for fewer partial sums.
 //
-// What bounds it: issue slots and the latency of a stage, no unit is saturated.  Per tile and slice the producers store 16 KB of
-// products and the tensor core reads them back with the columns of X^T (an MMA of M = 128, N <= 64 takes 39 to 48 cycles, bound
-// by its operand reads).  A warp took 2700 cycles for a whole stage, 1300 of them for 128 products a lane, and eight warps made
+// What bounds it: shared memory.  A stage takes 465 cycles at [40009,50] in bf16; per tile and slice the producers store 16 KB of
+// products (128 cycles) and the tensor core reads them back with the columns of X^T (128 and 33 to 64; an MMA of M = 128, N <= 64 takes
+// 39 to 48 cycles), the producers' own operands take 80.  Products straight into tensor memory, a row to a thread, load an x_i
+// for each of them: 51 us where this takes 33.
+// A warp took 2700 cycles for a whole stage, 1300 of them for 128 products a lane, and eight warps made
 // one every 340; sixteen, two to a stage, and copies without a selected address for whole slices: [40009,50] bf16 36.0 us,
 // now 35.2, [200000,50] 140 (before generic loads went) and 117, TF32 246 and 183.  Two issuer warps take alternate stages: polls and commits
 // between the MMAs cost one alone about 100 cycles per stage.  bf16 halves the number of stages (64 samples per slice
