@@ -2,7 +2,7 @@
 // product summed over samples is a symmetric rank-N update, i.e. a triangular tile GEMM X^T X).  Five forms of X:
 //   M2_BF16   bfloat16
 //   M2_TF32   fp32, of which the tensor core reads the upper 19 bits
-//   M2_CONV   fp32, in the kernel x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi
+//   M2_CONV   fp32, in the kernel x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi (M2TC_SYM_CYCLES: two of the three)
 //   M2_SPLIT  the same products of hi and lo that lie in memory (the pair features of moment4.cu)
 //   M2_EXACT  fp32, in the kernel of moment2_exact.cuh x = hi + mid + lo, at the error of fp32 arithmetic
 //
@@ -98,6 +98,7 @@ struct TileTable {
     unsigned char next, carrier[MAX_EXT];              // those tiles
     unsigned char corner;                              // the last of them also has the left-over columns among themselves
     unsigned short ext_col;                            // first left-over column, units of 8
+    unsigned char sym;                                 // M2_CONV: full diagonal tiles hold S, of which (S + S^T) / 2 is the result
 };
 // A partial tile holds four columns of a row side by side: [BN / 4][HALF][4] for each block, and after the BN columns of the
 // tile the left-over ones, and after these the corner.
@@ -191,6 +192,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     const int FLUSH_CHUNKS = MODE == M2_BF16 && width <= HALF ? S::FLUSH_CHUNKS / 2 : S::FLUSH_CHUNKS;
     const bool alias = diag && width == BN;             // A columns == B columns in both blocks: one load serves both
     const bool lead = diag && rows <= HALF;             // all rows in the first block, whose A holds its half of B as well
+    const bool sym = MODE == M2_CONV && alias && a.tab.sym;
     // (a tile that carries left-over columns is on the diagonal, and full)
     const int ext = EXT ? 16 * a.tab.ext[tile] : 0, ecol = 8 * a.tab.ext_col;
     const bool corner = ext > 0 && a.tab.corner && tile == a.tab.carrier[a.tab.next - 1];
@@ -324,7 +326,9 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                     tc_fence_after();
                     const uint64_t ad = adesc_base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
                     const uint64_t bd = bdesc_base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
-                    auto products = [&](uint32_t acc, uint64_t a0, uint64_t b0, uint32_t shape) {
+                    // sym: lo holds 2 lo, S = hi^T hi + hi^T 2 lo, and the sum of the partial tiles makes (S + S^T) / 2 of it; with 2 lo
+                    // the left-over columns take hi / 2, which lies `half` behind hi
+                    auto products = [&](uint32_t acc, uint64_t a0, uint64_t b0, uint32_t shape, bool two, uint64_t half) {
                         uint32_t on = accumulate;
 #pragma unroll
                         for (int k = 0; k < KROWS / S::KMMA; ++k) {
@@ -336,14 +340,14 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                             on = 1;
                             if (PARTS == 2) {
                                 mma_bf16_pair(acc, ak, bk + lo, shape, 1u);
-                                mma_bf16_pair(acc, ak + lo, bk, shape, 1u);
+                                if (!two) mma_bf16_pair(acc, ak + lo, bk + half, shape, 1u);
                             }
                         }
                     };
-                    products(d_tmem, ad, bd, idesc);
+                    products(d_tmem, ad, bd, idesc, sym, 0);
                     if (ext > 0) {
-                        products(tmem_base + BN, ad, bd + ext_off, idesc_ext);
-                        if (corner) products(tmem_base + (uint32_t)(BN + ext), bd + ext_off, bd + ext_off, idesc_ext);
+                        products(tmem_base + BN, ad, bd + ext_off, idesc_ext, false, sym ? (uint64_t)(BOX_PITCH >> 4) : 0);
+                        if (corner) products(tmem_base + (uint32_t)(BN + ext), bd + ext_off, bd + ext_off, idesc_ext, false, 0);
                     }
                     accumulate = 1;
                     tc_commit_pair(&empty[s]);
@@ -378,6 +382,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             for (int side = 0; side < 2; ++side) {
                 const int n = side ? na : nb;
                 unsigned char *p = stage + (side ? a.nb * BOX_PITCH : 0);
+                const float twice = sym && side == 0 ? 2.f : 1.f;
                 float4 v[PAIRS_B][H];
 #pragma unroll
                 for (int q = 0; q < PAIRS_B; ++q)
@@ -394,12 +399,18 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                             const float4 x = v[q][h];
                             const __nv_bfloat162 h0 = __floats2bfloat162_rn(x.x, x.y), h1 = __floats2bfloat162_rn(x.z, x.w);
                             const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
-                            const __nv_bfloat162 l0 = __floats2bfloat162_rn(x.x - f0.x, x.y - f0.y), l1 = __floats2bfloat162_rn(x.z - f1.x, x.w - f1.y);
+                            const __nv_bfloat162 l0 = __floats2bfloat162_rn(twice * (x.x - f0.x), twice * (x.y - f0.y)),
+                                                 l1 = __floats2bfloat162_rn(twice * (x.z - f1.x), twice * (x.w - f1.y));
                             unsigned char *w = p + q * BOX_PITCH + to[h];
                             *reinterpret_cast<uint2 *>(w) =
                                 make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
                             *reinterpret_cast<uint2 *>(w + BOX_BYTES) =
                                 make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
+                            if (EXT && side == 1 && sym) {
+                                const __nv_bfloat162 g0 = __floats2bfloat162_rn(0.5f * f0.x, 0.5f * f0.y), g1 = __floats2bfloat162_rn(0.5f * f1.x, 0.5f * f1.y);
+                                *reinterpret_cast<uint2 *>(w + BOX_PITCH) =
+                                    make_uint2(*reinterpret_cast<const uint32_t *>(&g0), *reinterpret_cast<const uint32_t *>(&g1));
+                            }
                         }
                     }
             }
@@ -415,7 +426,7 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         const int q = warp & 3;
         const int row0 = (int)rank * HALF + q * 32;
         const bool used = row0 < rows;
-        const int c_first = diag ? row0 : 0;         // row0 is a multiple of 32
+        const int c_first = diag && !sym ? row0 : 0;         // row0 is a multiple of 32
         float *dst = a.partials + (size_t)blockIdx.x * (EXT ? a.pitch : HALF * BN) + (q * 32 + lane) * 4;         // columns c .. c+3: + c HALF
         // columns in use: c_first .. width, and where the tile carries left-over columns all in between and after them
         const int c_end = ext > 0 ? BN + (ext * (corner && q * 32 < ext / 2 ? 2 : 1) + 31) / 32 * 32 : width;
@@ -504,7 +515,8 @@ moment2_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 // to the place of its 4-tuple in the packed 4-simplex, if this is the product that was chosen for that tuple.
 __host__ __device__ inline int m2tc_sum_warps(int nsplit) { return nsplit <= 4 ? 1 : nsplit <= 8 ? 2 : nsplit <= 16 ? 4 : 8; }
 // EXT: some tiles carry left-over columns (an instance of its own: with them in it the others took 1 to 2 us longer).
-template <bool PAIRS, bool EXT>
+// SYM: full diagonal tiles hold S, of which (S + S^T) / 2 is the result.
+template <bool PAIRS, bool EXT, bool SYM>
 __global__ void __launch_bounds__(256)
 moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features, int within, int64_t out_elems,
                          const unsigned *pairs, int pitch, const __grid_constant__ m2tc::TileTable tab)
@@ -545,6 +557,27 @@ moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features,
                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int e = 0; e < BATCH; ++e) { s.x += v[e].x; s.y += v[e].y; s.z += v[e].z; s.w += v[e].w; }
+        }
+        if (SYM && e < 0 && tab.diag[tile] && 32 * (int)tab.width[tile] == BN) {
+            // S^T of the four columns: rows c .. c+3, column r.  Halved before they are added: their sum may be no fp32 number.
+            s.x *= 0.5f; s.y *= 0.5f; s.z *= 0.5f; s.w *= 0.5f;
+            const bool in = use && gj < d;
+            const float *t = partials + (size_t)2 * first * block + (r & ~3) * HALF + (r & 3);
+            for (int k0 = w0; k0 < nsplit; k0 += BATCH * wps) {
+                float v[BATCH][4];
+#pragma unroll
+                for (int b = 0; b < BATCH; ++b)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        const int k = k0 + wps * b;
+                        v[b][x] = in && k < nsplit ? __ldcg(t + (size_t)k * stride + (size_t)((c + x) >> 7) * block + ((c + x) & 127) * 4) : 0.f;
+                    }
+#pragma unroll
+                for (int b = 0; b < BATCH; ++b) {
+                    s.x = fmaf(0.5f, v[b][0], s.x); s.y = fmaf(0.5f, v[b][1], s.y);
+                    s.z = fmaf(0.5f, v[b][2], s.z); s.w = fmaf(0.5f, v[b][3], s.w);
+                }
+            }
         }
         int at[4];                                         // where the columns go to, -1: not an output
         const int at0 = PAIRS ? 0 : (int)tri_encode(d, gi, gj);
@@ -605,15 +638,25 @@ static double m2tc_exact_cost(int rows, int width, bool diag)
 // 35.8 / 29.0, [20000,380] 19.7 / 24.1, [60000,380] 39.6 / 36.9; bf16 [20000,264] 13.3 / 15.2, [60000,264] 22.7 / 20.8, [20000,800] 26.3 /
 // 27.7, [60000,800] 59 / 53; split [6000,520] 19.5 / 21.7, [20000,520] 39.4 / 36.0, [20000,384] 24.4 / 27.4, [60000,384] 51.5 / 43.8.
 template <int MODE>
+static double m2tc_cycles(int64_t N, double cost)          // of a cluster, where tiles of this cost together share the chip
+{
+    return (double)((N + m2tc::Shape<MODE>::KROWS - 1) / m2tc::Shape<MODE>::KROWS) * cost * (MODE == M2_CONV ? 1226 : 512) / (sm_count_or_default() / 2);
+}
+template <int MODE>
 static bool m2tc_carry(int64_t N, int full, int left_over)
 {
-    using S = m2tc::Shape<MODE>;
     if (MODE == M2_EXACT || full == 0 || left_over == 0 || left_over > m2tc::HALF) return false;
     const int tiles = full * (full + 1) / 2, ext = (left_over + 15) / 16 * 16;
-    const double sum = tiles + (full + 1) * (m2tc_cost(m2tc::BN, ext, 1) - 1);
-    const double cycles = (double)((N + S::KROWS - 1) / S::KROWS) * sum * (MODE == M2_CONV ? 1226 : 512) / (sm_count_or_default() / 2);
+    const double cycles = m2tc_cycles<MODE>(N, tiles + (full + 1) * (m2tc_cost(m2tc::BN, ext, 1) - 1));
     return cycles >= (MODE == M2_CONV ? 1.6 : 1.0) * (6000 + 130 * ext + 3500 * (tiles - 1));
 }
+
+// Whether the full diagonal tiles of M2_CONV make two products instead of three, S = hi^T hi + hi^T 2 lo: C = (S + S^T) / 2.  Wide
+// tiles run at the power cap, where fewer products are more clock; their error is smaller too, as fewer sums are truncated (2-norm
+// against 64 bits [262144,520] 8.9e-6 with three, 7.5e-6).  The sum takes up to 9 us more, as it reads S^T across its rows, so that
+// it takes samples enough.  us in long rows of calls, three / two products: [262144,520] 361 / 328, [131072,776] 338 / 317,
+// [262144,264] 125 / 115, [100000,264] 70 / 57; alone [60000,384] 50 / 55, [8000,256] 18 / 27.
+constexpr double M2TC_SYM_CYCLES = 50000;
 
 // Tiles of a plan while it is made.
 struct M2TcTiles {
@@ -632,12 +675,13 @@ struct M2TcTiles {
         p->tab.width[n] = (unsigned char)(width / 32);
         p->tab.diag[n] = diag ? 1 : 0;
         cost[n] = MODE == M2_EXACT ? m2tc_exact_cost(rows, width, diag) : m2tc_cost(width, ext, corner ? 2 : 1);
+        if (p->tab.sym && diag && width == BN) cost[n] -= 0.1;      // two products for three (0 to 0.3 tried)
         const bool lead = diag && rows <= HALF;
         const int cols_b = lead && rows > width / 2 ? rows : width / 2, nb = (cols_b + S::BOXC - 1) / S::BOXC;
         if (nb > p->nb) p->nb = nb;
         if (ext > 0 || (!(diag && width == BN) && !lead)) {
             const int n_a = ext > 0 ? ext / 2 : rows;
-            const int na = n_a >= HALF ? S::NBOX : (n_a + S::BOXC - 1) / S::BOXC;
+            const int na = n_a >= HALF || (MODE == M2_CONV && ext > 0) ? S::NBOX : (n_a + S::BOXC - 1) / S::BOXC;     // (with room for hi / 2)
             if (na > p->na) p->na = na;
         }
         p->tab.ext[n] = (unsigned char)(ext / 16);
@@ -721,6 +765,7 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
     const bool carry = !dense && m2tc_carry<MODE>(N, full, left_over);
     const int ext = carry ? (left_over + 15) / 16 * 16 : 0;
     const int nt = carry ? full : (int)((d + BM - 1) / BM);
+    p.tab.sym = MODE == M2_CONV && !dense && d >= BN && m2tc_cycles<MODE>(N, 0.5 * nt * (nt + 1)) >= M2TC_SYM_CYCLES;
     for (int tn = 0; tn < nt; ++tn)
         for (int tm = 0; tm < nt; ++tm) {
             if (tm > tn && !dense) continue;
@@ -856,7 +901,11 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
     const unsigned most = 16u * (unsigned)sm_count_or_default() / (unsigned)q.tab.ntiles;
     if (blocks > most) blocks = most < 64 ? 64 : most;
     const dim3 rgrid((unsigned)(q.tab.ntiles + q.tab.next + q.tab.corner), blocks);
-    return launch(pairs ? moment2_tc_reduce_kernel<true, false> : q.tab.next > 0 ? moment2_tc_reduce_kernel<false, true> : moment2_tc_reduce_kernel<false, false>,
+    constexpr bool CONV = MODE == M2_CONV;
+    const auto sum = pairs ? moment2_tc_reduce_kernel<true, false, false>
+                   : q.tab.next > 0 ? (q.tab.sym ? moment2_tc_reduce_kernel<false, true, CONV> : moment2_tc_reduce_kernel<false, true, false>)
+                                    : (q.tab.sym ? moment2_tc_reduce_kernel<false, false, CONV> : moment2_tc_reduce_kernel<false, false, false>);
+    return launch(sum,
                   rgrid, 256, 0, stream, partials, out, (int)d,
                   features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.pitch, q.tab);
 }
