@@ -755,17 +755,17 @@ static void m2tc_finish(M2TcPlan &p, const M2TcTiles &t, int64_t N)
 }
 
 template <int MODE>
-static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
+static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags, bool may_carry = true, bool may_sym = true)
 {
     using namespace m2tc;
     M2TcPlan p{};
     M2TcTiles t{&p, 0, {}};
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
     const int full = (int)(d / BM), left_over = (int)(d % BM);
-    const bool carry = !dense && m2tc_carry<MODE>(N, full, left_over);
+    const bool carry = may_carry && !dense && m2tc_carry<MODE>(N, full, left_over);
     const int ext = carry ? (left_over + 15) / 16 * 16 : 0;
     const int nt = carry ? full : (int)((d + BM - 1) / BM);
-    p.tab.sym = MODE == M2_CONV && !dense && d >= BN && m2tc_cycles<MODE>(N, 0.5 * nt * (nt + 1)) >= M2TC_SYM_CYCLES;
+    p.tab.sym = may_sym && MODE == M2_CONV && !dense && d >= BN && m2tc_cycles<MODE>(N, 0.5 * nt * (nt + 1)) >= M2TC_SYM_CYCLES;
     for (int tn = 0; tn < nt; ++tn)
         for (int tm = 0; tm < nt; ++tm) {
             if (tm > tn && !dense) continue;
@@ -910,23 +910,25 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
                   features, within, pairs ? simp4_rows(features) : tri_rows(d), pairs, q.pitch, q.tab);
 }
 
-// Room for the partial tiles of the structured call and of its dense control: one workspace serves both.
-template <int MODE>
-static size_t m2tc_partial_room(int64_t N, int64_t d, size_t bytes)
-{
-    for (unsigned f : {0u, ST_FLAG_DENSE_CONTROL}) {
-        const M2TcPlan q = m2tc_plan<MODE>(N, d, f);
-        if (q.ok && q.partial_bytes > bytes) bytes = q.partial_bytes;
-    }
-    return bytes;
-}
-
+// One workspace serves the structured call and its dense control, and the same calls of fewer samples too: their plan may be one that
+// is not taken for these samples, with tiles of their own for the left-over columns or with three products, and may need more room.
 template <int MODE>
 static size_t m2tc_workspace(int64_t N, int64_t d, unsigned flags)
 {
     if (N <= 0 || d <= 0 || d > 4096 || N > (int64_t(1) << 31) - 64) return 0;
-    const M2TcPlan q = m2tc_plan<MODE>(N, d, flags);
-    return q.ok ? kWsHeaderBytes + m2tc_partial_room<MODE>(N, d, q.partial_bytes) : 0;
+    const M2TcPlan plain = m2tc_plan<MODE>(N, d, 0u), dense = m2tc_plan<MODE>(N, d, ST_FLAG_DENSE_CONTROL);
+    if (!(flags & ST_FLAG_DENSE_CONTROL ? dense : plain).ok) return 0;
+    size_t bytes = 0;
+    auto fit = [&](const M2TcPlan &q) {
+        if (q.ok && q.partial_bytes > bytes) bytes = q.partial_bytes;
+    };
+    fit(plain);
+    fit(dense);
+    const bool carries = plain.tab.next > 0, sym = plain.tab.sym != 0;
+    if (carries) fit(m2tc_plan<MODE>(N, d, 0u, false, true));
+    if (sym) fit(m2tc_plan<MODE>(N, d, 0u, true, false));
+    if (carries && sym) fit(m2tc_plan<MODE>(N, d, 0u, false, false));
+    return kWsHeaderBytes + bytes;
 }
 
 template <int MODE>

@@ -274,6 +274,17 @@ def test_fourth_moment_in_bf16_takes_as_many_samples_as_its_copies_can_name():
     assert size((1 << 31) - 63) == 0
 
 
+def test_a_workspace_for_more_samples_serves_fewer_on_the_tensor_cores():
+    """Second moment in bf16, TF32 and split: columns that many samples carry along have tiles of their own with few."""
+    import paper_2211_10482_b200 as st
+    modes = ((st.ST_BF16, 0, 8), (st.ST_F32, st.ST_FLAG_TC_TF32, 4), (st.ST_F32, st.ST_FLAG_TC_SPLIT, 8))
+    samples = sorted({1, 33, 66, 128} | {500 * i for i in range(1, 200)} | {1 << k for k in range(10, 29)})
+    for dtype, flags, step in modes:
+        for d in sorted({256 * k + step * c for k in range(1, 16) for c in (1, 2, 5, 9, 128 // step)} | {824, 1800, 4096}):
+            sizes = [st.st_workspace_bytes(st.ST_OP_SYM_MOMENT2, N, d, dtype, 0, flags) for N in samples]
+            assert sizes == sorted(sizes), (flags, d)
+
+
 def test_copies_read_no_byte_behind_the_source_array():
     src = os.path.join(tempfile.mkdtemp(prefix="st_span_"), "span.cpp")
     with open(src, "w") as f:
