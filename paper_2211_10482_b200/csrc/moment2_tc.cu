@@ -127,29 +127,37 @@ __device__ __forceinline__ int m2tc_tile_of(const m2tc::TileTable &t, int cluste
     return lo;
 }
 
-// Adds 32 columns of a thread's row, those of `mask`, to the partial tile, in L2 and without an answer;
+// Adds 32 columns of a thread's row, those of `mask` (four by four), to the partial tile, in L2 and without an answer;
 // the additions of one thread to one place take effect in their order.  L2 takes subnormal numbers for zero.  Where |v| is
-// at least 2^-100 no sum is one, and what it lacks is below 2^-25 of v; other columns are added here.
+// at least 2^-100 no sum is one, and what it lacks is below 2^-25 of v; four columns with a smaller value among them are added here.  But
+// a zero changes no sum, and where the others are large they go one by one: padding, and categories that a sample range lacks.
+// [262144,520] in rows of calls, us: N(0,1) split 283, bf16 119, TF32 207; with zeros added here, and 32 columns for one of them, / now:
+// split, a zero column 447 / 303, 128 categories in sorted order 436 / 287; bf16, 300 of these 159 / 112; TF32, 300 unsorted 241 / 191.
+// Sums below 2^-100 wait for L2: split with a third of the columns times 2^-54 500 (tiles of their own 392), bf16 with all 163 (150).
 __device__ __forceinline__ void m2tc_add_in_l2(float *p, const uint32_t (&r)[32], uint32_t mask)
 {
     constexpr int QUAD = 4 * m2tc::HALF;                   // floats from one group of four columns to the next
-    float least = INFINITY;
-#pragma unroll
-    for (int e = 0; e < 32; ++e)
-        if (mask >> e & 1u) least = fminf(least, fabsf(__uint_as_float(r[e])));
-    const bool fast = least >= 0x1p-100f;
 #pragma unroll
     for (int e = 0; e < 32; e += 4) {
         if (!(mask >> e & 15u)) continue;
-        const float x = __uint_as_float(r[e]), y = __uint_as_float(r[e + 1]), z = __uint_as_float(r[e + 2]), w = __uint_as_float(r[e + 3]);
+        const float v[4] = {__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])};
         float *q = p + e / 4 * QUAD;
-        if (fast) {
-            asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
-        } else {
-            float4 o;
-            asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w) : "l"(q) : "memory");
-            asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(o.x + x), "f"(o.y + y), "f"(o.z + z), "f"(o.w + w) : "memory");
+        if (fminf(fminf(fabsf(v[0]), fabsf(v[1])), fminf(fabsf(v[2]), fabsf(v[3]))) >= 0x1p-100f) {
+            asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+            continue;
         }
+        bool tiny = false;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tiny |= fabsf(v[i]) < 0x1p-100f && v[i] != 0.f;
+        if (!tiny) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (v[i] != 0.f) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(q + i), "f"(v[i]) : "memory");
+            continue;
+        }
+        float4 o;
+        asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w) : "l"(q) : "memory");
+        asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(o.x + v[0]), "f"(o.y + v[1]), "f"(o.z + v[2]), "f"(o.w + v[3]) : "memory");
     }
 }
 

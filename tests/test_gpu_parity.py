@@ -896,6 +896,57 @@ def test_moment2_left_over_columns_of_long_sample_ranges(st, mode, N, d):
     assert ((plain.double() - T[iu[0], iu[1]]).abs() / S[iu[0], iu[1]]).max().item() <= (TOL_TC if mode == "tf32" else TOL_F32)
 
 
+# the same of tables with zeros, other row strides, infinities and NaN: columns that are zero, that are zero but for one range of the
+# samples (a category of a sorted table), and tiny ones beside them, in whole tiles, among the left-over columns and in the corner
+@pytest.mark.parametrize("mode,N,d", [("bf16", 90001, 264), ("bf16", 130003, 520), ("tf32", 100003, 380), ("split", 120011, 304), ("split", 250007, 520),
+                                      ("split", 160009, 512)])
+def test_moment2_left_over_columns_of_tables_with_zeros_and_without_numbers(st, mode, N, d):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+    ldx = d + 24
+    wide = torch.randn(N, ldx, generator=g, device="cuda")
+    n = torch.arange(N, device="cuda")
+    for k in range(3, d, 8):
+        wide[:, k] *= (n * d // N // 8 == k // 8)
+    for k in (10, 200, d - 1):
+        wide[:, k] = 0
+    wide[:, [4, d - 3]] *= 2.0 ** -60                  # squares: sums of about 2^-104
+    flags = {"split": st.ST_FLAG_TC_SPLIT, "tf32": st.ST_FLAG_TC_TF32, "bf16": 0}[mode]
+    wide = wide.bfloat16() if mode == "bf16" else wide
+    X = wide[:, :d].contiguous()
+    got = st.st_sym_moment2(X, flags=flags)
+    iu = torch.triu_indices(d, d, device="cuda")
+    X64 = X.double()
+    T, S = X64.T @ X64, X64.abs().T @ X64.abs()
+    assert bool(((got.double() - T[iu[0], iu[1]]).abs() <= (TOL_TC if mode == "tf32" else TOL_F32) * S[iu[0], iu[1]]).all())
+    del X64
+    dtype = st.ST_BF16 if mode == "bf16" else st.ST_F32
+    out, ws = guarded(st, got.numel()), guarded(st, st.st_workspace_bytes(st.ST_OP_SYM_MOMENT2, N, d, dtype, 0, flags), torch.uint8)
+    assert st.lib().st_sym_moment2(wide.data_ptr(), dtype, N, d, ldx, out.data_ptr(), ws.data_ptr(), ws.numel(), flags,
+                                   torch.cuda.current_stream().cuda_stream) == st.ST_OK
+    assert torch.equal(out, got)
+    X[N // 2, 5] = math.inf
+    X[N - 1, d - 2] = math.nan
+    there = ((iu == 5) | (iu == d - 2)).any(0)
+    odd = st.st_sym_moment2(X, flags=flags)
+    assert not bool(torch.isfinite(odd[there]).any())
+    assert torch.equal(odd[~there], got[~there])
+
+
+# all-positive sums, where an accumulator that rounds towards zero drifts: with columns carried along and with two products
+@pytest.mark.parametrize("mode,N,d", [("split", 262147, 520), ("split", 320009, 256), ("bf16", 262147, 264)])
+def test_moment2_left_over_columns_of_positive_tables_do_not_drift(st, mode, N, d):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    X = torch.rand(N, d, generator=g, device="cuda") + 0.5
+    X = X.bfloat16() if mode == "bf16" else X
+    got = st.st_sym_moment2(X, flags=st.ST_FLAG_TC_SPLIT if mode == "split" else 0)
+    iu = torch.triu_indices(d, d, device="cuda")
+    X64 = X.double()
+    T = (X64.T @ X64)[iu[0], iu[1]]
+    assert ((got.double() - T).abs() / T).max().item() <= TOL_F32
+
+
 def test_moment2_split_sums_of_squares_do_not_drift(st):
     """All-positive sums over many samples: the accumulation chain is cut often enough that the diagonal stays
     inside the fp32 tolerance (a tensor-core accumulator rounds towards zero)."""
