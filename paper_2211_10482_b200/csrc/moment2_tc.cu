@@ -2,7 +2,7 @@
 // product summed over samples is a symmetric rank-N update, i.e. a triangular tile GEMM X^T X).  Five forms of X:
 //   M2_BF16   bfloat16
 //   M2_TF32   fp32, of which the tensor core reads the upper 19 bits
-//   M2_CONV   fp32, in the kernel x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi (M2TC_SYM_CYCLES: two of the three)
+//   M2_CONV   fp32, in the kernel x = hi + lo in bfloat16: hi^T hi + hi^T lo + lo^T hi (M2TC_SYM_SUM: two of the three)
 //   M2_SPLIT  the same products of hi and lo that lie in memory (the pair features of moment4.cu)
 //   M2_EXACT  fp32, in the kernel of moment2_exact.cuh x = hi + mid + lo, at the error of fp32 arithmetic
 //
@@ -20,8 +20,8 @@
 // their rows with them, and the last of these tiles also the product of the left-over columns with themselves.  Such a tile
 // needs the tensor memory of both accumulators, so that its MMAs wait while the epilogue empties them (a tenth of a phase
 // with one load from tensor memory at a time and sums that come back from L2; hardly anything with m2tc_add_in_l2).
-// us, with tiles of their own / carried along: [262144,520] split 389 / 308, TF32 287 / 204, bf16 153 / 117; [131072,776] 346 / 286,
-// 229 / 187, 129 / 110; [262144,264] 161 / 109, 137 / 76, 71 / 43; [131072,896] (128 columns) 399 / 327, 250 / 217, 131 / 117.
+// us, with tiles of their own / carried along: [262144,520] split 384 / 314 (with M2TC_SYM_SUM 283), TF32 287 / 206, bf16 161 / 119;
+// [131072,776] 346 / 286, 229 / 187, 129 / 110; [262144,264] 161 / 109, 137 / 76, 71 / 43; [131072,896] (128 columns) 399 / 327, 250 / 217, 131 / 117.
 //
 // The tensor core adds into its fp32 accumulator without round-to-nearest, so a chain of
 // many thousands of accumulating MMAs drifts low (measured: -7.7e-4 relative on all-positive
@@ -43,7 +43,7 @@
 // 96 bytes per sample and column pair).  Few features: the latency of a stage, hence more and smaller stages.
 //
 // M2_CONV: a pass that wrote hi and lo before moved 8 bytes a value through HBM on top of the 4 read here, and took
-// 176 of the 590 us of [262144,520], now 308; [1048576,256] 700, now 285; [1048576,64] 245, now 143.  Copies bring the
+// 176 of the 590 us of [262144,520], now 283; [1048576,256] 700, now 285; [1048576,64] 245, now 143.  Copies bring the
 // fp32 boxes, converting warps rewrite them in place and arrive at the leader's barrier.  Bound by shared memory: per
 // 32 samples of a full tile off the diagonal 256 cycles each for the copy, the reads and the writes and 384 for the
 // operands of 768 cycles of MMA.  Loads through registers instead of the copies avoid two of these, but every arrival
@@ -567,25 +567,29 @@ moment2_tc_reduce_kernel(const float *partials, float *out, int d, int features,
             for (int e = 0; e < BATCH; ++e) { s.x += v[e].x; s.y += v[e].y; s.z += v[e].z; s.w += v[e].w; }
         }
         if (SYM && e < 0 && tab.diag[tile] && 32 * (int)tab.width[tile] == BN) {
-            // S^T of the four columns: rows c .. c+3, column r.  Halved before they are added: their sum may be no fp32 number.
-            s.x *= 0.5f; s.y *= 0.5f; s.z *= 0.5f; s.w *= 0.5f;
-            const bool in = use && gj < d;
-            const float *t = partials + (size_t)2 * first * block + (r & ~3) * HALF + (r & 3);
+            // S^T of the four columns: rows c .. c+3, column r.  Four lanes read four columns of these rows, 64 bytes in a row, and
+            // exchange their sums.  Halved before they are added: their sum may be no fp32 number.
+            const int j = lane & 3;
+            const bool in = u < units && (r & ~3) < rows && gj + 4 > (gi & ~3);
+            const float *t = partials + (size_t)(2 * first + ((c + j) >> 7)) * block + (r & ~3) * HALF + ((c + j) & 127) * 4;
+            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
             for (int k0 = w0; k0 < nsplit; k0 += BATCH * wps) {
-                float v[BATCH][4];
+                float4 v[BATCH];
 #pragma unroll
                 for (int b = 0; b < BATCH; ++b)
+                    v[b] = in && k0 + wps * b < nsplit ? __ldcg(reinterpret_cast<const float4 *>(t + (size_t)(k0 + wps * b) * stride))
+                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const int k = k0 + wps * b;
-                        v[b][x] = in && k < nsplit ? __ldcg(t + (size_t)k * stride + (size_t)((c + x) >> 7) * block + ((c + x) & 127) * 4) : 0.f;
-                    }
-#pragma unroll
-                for (int b = 0; b < BATCH; ++b) {
-                    s.x = fmaf(0.5f, v[b][0], s.x); s.y = fmaf(0.5f, v[b][1], s.y);
-                    s.z = fmaf(0.5f, v[b][2], s.z); s.w = fmaf(0.5f, v[b][3], s.w);
-                }
+                for (int b = 0; b < BATCH; ++b) { y.x += v[b].x; y.y += v[b].y; y.z += v[b].z; y.w += v[b].w; }
             }
+            auto exchange = [&](float &lo, float &hi, int bit) {           // of lanes that differ in `bit`
+                const float got = __shfl_xor_sync(0xFFFFFFFFu, lane & bit ? lo : hi, bit);
+                (lane & bit ? lo : hi) = got;
+            };
+            exchange(y.x, y.y, 1); exchange(y.z, y.w, 1);
+            exchange(y.x, y.z, 2); exchange(y.y, y.w, 2);
+            s.x = fmaf(0.5f, y.x, 0.5f * s.x); s.y = fmaf(0.5f, y.y, 0.5f * s.y);
+            s.z = fmaf(0.5f, y.z, 0.5f * s.z); s.w = fmaf(0.5f, y.w, 0.5f * s.w);
         }
         int at[4];                                         // where the columns go to, -1: not an output
         const int at0 = PAIRS ? 0 : (int)tri_encode(d, gi, gj);
@@ -621,6 +625,7 @@ struct M2TcPlan {
     m2tc::TileTable tab;
     int chunks_total, stages, nb, na, pitch;
     size_t partial_bytes, smem;
+    double time;                                       // stages of a full tile that the call takes
     bool ok;
 };
 
@@ -645,10 +650,11 @@ static double m2tc_exact_cost(int rows, int width, bool diag)
 // cluster, in cycles of their stages, have to outweigh.  us, tiles of their own / carried: TF32 [20000,300] 17.9 / 19.1, [60000,300]
 // 35.8 / 29.0, [20000,380] 19.7 / 24.1, [60000,380] 39.6 / 36.9; bf16 [20000,264] 13.3 / 15.2, [60000,264] 22.7 / 20.8, [20000,800] 26.3 /
 // 27.7, [60000,800] 59 / 53; split [6000,520] 19.5 / 21.7, [20000,520] 39.4 / 36.0, [20000,384] 24.4 / 27.4, [60000,384] 51.5 / 43.8.
+constexpr double m2tc_stage_cycles(int mode) { return mode == M2_CONV ? 1226 : 512; }      // a full tile's
 template <int MODE>
 static double m2tc_cycles(int64_t N, double cost)          // of a cluster, where tiles of this cost together share the chip
 {
-    return (double)((N + m2tc::Shape<MODE>::KROWS - 1) / m2tc::Shape<MODE>::KROWS) * cost * (MODE == M2_CONV ? 1226 : 512) / (sm_count_or_default() / 2);
+    return (double)((N + m2tc::Shape<MODE>::KROWS - 1) / m2tc::Shape<MODE>::KROWS) * cost * m2tc_stage_cycles(MODE) / (sm_count_or_default() / 2);
 }
 template <int MODE>
 static bool m2tc_carry(int64_t N, int full, int left_over)
@@ -659,17 +665,23 @@ static bool m2tc_carry(int64_t N, int full, int left_over)
     return cycles >= (MODE == M2_CONV ? 1.6 : 1.0) * (6000 + 130 * ext + 3500 * (tiles - 1));
 }
 
-// Whether the full diagonal tiles of M2_CONV make two products instead of three, S = hi^T hi + hi^T 2 lo: C = (S + S^T) / 2.  Wide
-// tiles run at the power cap, where fewer products are more clock; their error is smaller too, as fewer sums are truncated (2-norm
-// against 64 bits [262144,520] 8.9e-6 with three, 7.5e-6).  The sum takes up to 9 us more, as it reads S^T across its rows, so that
-// it takes samples enough.  us in long rows of calls, three / two products: [262144,520] 361 / 328, [131072,776] 338 / 317,
-// [262144,264] 125 / 115, [100000,264] 70 / 57; alone [60000,384] 50 / 55, [8000,256] 18 / 27.
-constexpr double M2TC_SYM_CYCLES = 50000;
+// Full diagonal tiles of M2_CONV may make two products instead of three, S = hi^T hi + hi^T 2 lo: C = (S + S^T) / 2 (their error is
+// smaller too, as fewer sums are truncated: 2-norm against 64 bits [262144,520] 8.9e-6 with three, 7.5e-6).  M2TC_SYM_*: what a stage of
+// such a tile takes less, a full tile = 1, as rows of calls show it (wide tiles run at the power cap, where fewer products are more
+// clock): with left-over columns, for a table of one tile, others.  Their clusters have twice the sums to add and the sum has S^T to read,
+// M2TC_SYM_SUM cycles for each: the two products are taken where the call is shortened by more, that is where the clusters that
+// they free shorten the longest one.  us in rows of calls / alone, three products -> two: taken [50000,512] 53 / 60 -> 49 / 59,
+// [160000,512] 159 / 167 -> 149 / 157, [60000,520] 79 / 89 -> 76 / 85, [120000,520] 146 / 153 -> 132 / 142, [60000,776] 137 / 145 -> 129 / 136,
+// [10000,1024] 42 / 48 -> 37 / 44, [262144,1024] 990 / 1028 -> 861 / 896, [60000,1280] 358 / 363 -> 290 / 304, [10000,3072] 369 / 378 -> 350 / 359,
+// [300000,256] 89 / 93 -> 82 / 94; not taken [120000,256] 41 / 48 -> 44 / 52, [60000,280] 34 / 42 -> 37 / 45, [15000,896] 53 / 60 -> 54 / 62,
+// [120000,1536] 949 / 980 -> 966 / 984, [30000,1800] 330 / 339 -> 347 / 356, [60000,2048] 762 / 793 -> 769 / 797.
+constexpr double M2TC_SYM_EXT = 0.1, M2TC_SYM_ONE = 0.06, M2TC_SYM_FULL = 0.2, M2TC_SYM_SUM = 110;
 
 // Tiles of a plan while it is made.
 struct M2TcTiles {
     M2TcPlan *p;
     int n;
+    bool one;                                          // the only tile of its plan
     double cost[m2tc::MAX_TILES];
     template <int MODE>
     bool add(int row, int rows, int col, int width, bool diag, int ext_col = 0, int ext = 0, bool corner = false)
@@ -683,7 +695,7 @@ struct M2TcTiles {
         p->tab.width[n] = (unsigned char)(width / 32);
         p->tab.diag[n] = diag ? 1 : 0;
         cost[n] = MODE == M2_EXACT ? m2tc_exact_cost(rows, width, diag) : m2tc_cost(width, ext, corner ? 2 : 1);
-        if (p->tab.sym && diag && width == BN) cost[n] -= 0.1;      // two products for three (0 to 0.3 tried)
+        if (p->tab.sym && diag && width == BN) cost[n] -= ext > 0 ? M2TC_SYM_EXT : one ? M2TC_SYM_ONE : M2TC_SYM_FULL;
         const bool lead = diag && rows <= HALF;
         const int cols_b = lead && rows > width / 2 ? rows : width / 2, nb = (cols_b + S::BOXC - 1) / S::BOXC;
         if (nb > p->nb) p->nb = nb;
@@ -759,21 +771,19 @@ static void m2tc_finish(M2TcPlan &p, const M2TcTiles &t, int64_t N)
     }
     for (int i = n; i <= MAX_TILES; ++i) p.tab.first[i] = (unsigned short)first;
     p.partial_bytes = (size_t)2 * first * p.pitch * sizeof(float);
+    p.time = (double)chunks * (longest > sum / clusters ? longest : sum / clusters);        // (more tiles than pairs of SMs: several waves)
     p.ok = true;
 }
 
 template <int MODE>
-static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags, bool may_carry = true, bool may_sym = true)
+static M2TcPlan m2tc_plan_of(int64_t N, int64_t d, bool dense, bool carry, bool sym)
 {
     using namespace m2tc;
     M2TcPlan p{};
-    M2TcTiles t{&p, 0, {}};
-    const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
-    const int full = (int)(d / BM), left_over = (int)(d % BM);
-    const bool carry = may_carry && !dense && m2tc_carry<MODE>(N, full, left_over);
-    const int ext = carry ? (left_over + 15) / 16 * 16 : 0;
+    const int full = (int)(d / BM), ext = carry ? (int)(d % BM + 15) / 16 * 16 : 0;
     const int nt = carry ? full : (int)((d + BM - 1) / BM);
-    p.tab.sym = may_sym && MODE == M2_CONV && !dense && d >= BN && m2tc_cycles<MODE>(N, 0.5 * nt * (nt + 1)) >= M2TC_SYM_CYCLES;
+    M2TcTiles t{&p, 0, nt == 1, {}};
+    p.tab.sym = sym;
     for (int tn = 0; tn < nt; ++tn)
         for (int tm = 0; tm < nt; ++tm) {
             if (tm > tn && !dense) continue;
@@ -786,6 +796,25 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags, bool may_carry =
         }
     m2tc_finish<MODE>(p, t, N);
     return p;
+}
+
+template <int MODE>
+static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
+{
+    using namespace m2tc;
+    const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
+    const bool carry = !dense && m2tc_carry<MODE>(N, (int)(d / BM), (int)(d % BM));
+    const M2TcPlan three = m2tc_plan_of<MODE>(N, d, dense, carry, false);
+    if constexpr (MODE == M2_CONV) {
+        const double most = M2TC_SYM_FULL * m2tc_stage_cycles(MODE) * three.time;            // that two products can save
+        if (dense || d < BN || !three.ok || most < M2TC_SYM_SUM) return three;
+        const M2TcPlan two = m2tc_plan_of<MODE>(N, d, dense, carry, true);
+        int clusters = 0;
+        for (int i = 0; i < two.tab.ntiles; ++i)
+            if (two.tab.diag[i] && 32 * (int)two.tab.width[i] == BN) clusters += two.tab.first[i + 1] - two.tab.first[i];
+        if (two.ok && (three.time - two.time) * m2tc_stage_cycles(MODE) >= M2TC_SYM_SUM * clusters) return two;
+    }
+    return three;
 }
 
 // Tiles of the products of pair features that pair_layout.cuh names, in turn to f(row, rows, col, width, on the diagonal).
@@ -847,7 +876,7 @@ static const M2TcPlan &m2tc_plan_pairs(int64_t N, const PairLayout &L)
     if (of[0] == now[0] && of[1] == now[1] && of[2] == now[2]) return p;
     for (int i = 0; i < 3; ++i) of[i] = now[i];
     p = M2TcPlan{};
-    M2TcTiles t{&p, 0, {}};
+    M2TcTiles t{&p, 0, false, {}};
     bool ok = true;
     pair_tiles(L, [&](int row, int rows, int col, int width, bool diag) { ok = ok && t.add<MODE>(row, rows, col, width, diag); });
     if (ok) m2tc_finish<MODE>(p, t, N);
@@ -919,7 +948,8 @@ static st_status m2tc_launch(const M2TcPlan &q, const void *X, int64_t rows, int
 }
 
 // One workspace serves the structured call and its dense control, and the same calls of fewer samples too: their plan may be one that
-// is not taken for these samples, with tiles of their own for the left-over columns or with three products, and may need more room.
+// is not taken for these samples, with tiles of their own for the left-over columns or with another number of products, and may need
+// more room.
 template <int MODE>
 static size_t m2tc_workspace(int64_t N, int64_t d, unsigned flags)
 {
@@ -932,10 +962,8 @@ static size_t m2tc_workspace(int64_t N, int64_t d, unsigned flags)
     };
     fit(plain);
     fit(dense);
-    const bool carries = plain.tab.next > 0, sym = plain.tab.sym != 0;
-    if (carries) fit(m2tc_plan<MODE>(N, d, 0u, false, true));
-    if (sym) fit(m2tc_plan<MODE>(N, d, 0u, true, false));
-    if (carries && sym) fit(m2tc_plan<MODE>(N, d, 0u, false, false));
+    for (int carry = 0; carry <= (plain.tab.next > 0); ++carry)
+        for (int sym = 0; sym <= (MODE == M2_CONV && d >= m2tc::BN); ++sym) fit(m2tc_plan_of<MODE>(N, d, false, carry != 0, sym != 0));
     return kWsHeaderBytes + bytes;
 }
 
@@ -989,8 +1017,8 @@ st_status moment2_exact_tc(const float *X, int64_t N, int64_t d, int64_t ldx, fl
 
 // ---------------------------------------------------------------------------------------------
 // fp32 input at the fp32 tolerance on the tensor cores (ST_FLAG_TC_SPLIT): x = hi + lo with hi = bf16(x) and
-// lo = bf16(x - hi) (what is left is below 2^-16 |x|), and the pair kernel adds hi^T hi + hi^T lo + lo^T hi (lo^T lo is
-// below 2^-16 of the result).
+// lo = bf16(x - hi) (what is left is below 2^-16 |x|), and the pair kernel adds hi^T hi + hi^T lo + lo^T hi, or on full diagonal tiles
+// hi^T hi + hi^T 2 lo, whose symmetric part that is (M2TC_SYM_SUM); either way lo^T lo, below 2^-16 of the result, is left out.
 size_t moment2_split_tc_workspace(int64_t N, int64_t d, unsigned flags)
 {
     return d % 8 != 0 || N > (int64_t(1) << 29) ? 0 : m2tc_workspace<M2_CONV>(N, d, flags);

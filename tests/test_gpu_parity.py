@@ -947,6 +947,20 @@ def test_moment2_left_over_columns_of_positive_tables_do_not_drift(st, mode, N, 
     assert ((got.double() - T).abs() / T).max().item() <= TOL_F32
 
 
+# two products on full diagonal tiles: their sums over one to eight ranges per warp, a last tile that is not quite full, carried columns
+@pytest.mark.parametrize("N,d", [(290011, 256), (90001, 304), (60011, 504), (30011, 512), (15013, 776), (12007, 768), (9001, 1024), (15001, 1280), (6007, 3072),
+                                 (4001, 4096)])
+def test_moment2_split_with_two_products_on_the_diagonal(st, N, d):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+    X = torch.randn(N, d, generator=g, device="cuda")
+    got = st.st_sym_moment2(X, flags=st.ST_FLAG_TC_SPLIT)
+    X64 = X.double()
+    T, S = X64.T @ X64, X64.abs().T @ X64.abs()
+    iu = torch.triu_indices(d, d, device="cuda")
+    assert ((got.double() - T[iu[0], iu[1]]).abs() / S[iu[0], iu[1]]).max().item() <= TOL_F32
+
+
 def test_moment2_split_sums_of_squares_do_not_drift(st):
     """All-positive sums over many samples: the accumulation chain is cut often enough that the diagonal stays
     inside the fp32 tolerance (a tensor-core accumulator rounds towards zero)."""
