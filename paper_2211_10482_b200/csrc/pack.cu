@@ -273,7 +273,7 @@ __device__ __forceinline__ void slice_run(const LayoutArgs &a, I &s, I &lo, I &h
 // Four blocks per SM: with the registers that the compiler would take (up to 96) fewer fit, and the zeros of a sparse slice are
 // bound by the number of blocks ([8000,8000] band 39.5 us, 37.7 with 64 registers; st_thp of a tet d = 120, rows of 64 floats
 // 52, now 39).
-// ONCE: blocks that go through their part of a slice in one pass (copy_once).
+// ONCE: blocks, of as many warps as it takes, that go through their part of a slice in one pass (copy_once).
 template <int KIND, int ES, bool PACK, bool MUL, bool ONCE, typename I>
 __global__ void __launch_bounds__(256, 4)
 slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I nitems, int group_shift, int parts,
@@ -282,10 +282,10 @@ slice_copy_kernel(const unsigned char *src, unsigned char *dst, LayoutArgs a, I 
     // MUL (pack only, fp32 elements): a second packed operand; the gathered values are multiplied by it
     pdl_wait();
     pdl_trigger();
-    const int g = 1 << group_shift;
-    const int lane = (int)(threadIdx.x & (g - 1));
-    const I gid = (I)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> group_shift);
-    const I ngroups = (I)(((int64_t)gridDim.x * blockDim.x) >> group_shift);
+    const int g = ONCE ? (int)blockDim.x : 1 << group_shift;
+    const int lane = ONCE ? (int)threadIdx.x : (int)(threadIdx.x & (g - 1));
+    const I gid = ONCE ? (I)blockIdx.x : (I)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> group_shift);
+    const I ngroups = ONCE ? (I)gridDim.x : (I)(((int64_t)gridDim.x * blockDim.x) >> group_shift);
     const int64_t sb = a.d * a.row_bytes;                     // bytes per dense slice
     const unsigned char *src_end = src + (PACK ? a.dense_rows : a.packed_rows) * a.row_bytes;
     auto copy = [&](unsigned char *to, const unsigned char *from, const unsigned char *times, int n) {
@@ -425,7 +425,7 @@ sym_slice_kernel(const unsigned char *src, unsigned char *dst, I d, I nslices, i
                 for (int u = 0; u < SYM_WORDS; ++u) {
                     const unsigned e = e0 + 32 * u;
                     if (e >= n) continue;
-                    // (order 3: the high half of a product costs 7 % there, and below 2^12 that by 2^16 / words does)
+                    // (order 3: the high half of a product costs 7 % there, and for the at most 256 words of a part that by 2^16 / words does)
                     const unsigned dx = words == 1 ? e : FORM == 1 && KIND == ST_TET && words <= 32 ? (e * ((inv + 0xFFFF) >> 16)) >> 16 : __umulhi(e, inv);
                     const I p = sym_row<KIND, I>(d, a, b, c, x0 + (I)dx);
                     v[u] = ST_BOUNDS_OK(p, packed_rows, 1) ? reinterpret_cast<const E *>(src)[(int64_t)p * words + (e - dx * (unsigned)words)] : E{};
@@ -656,10 +656,12 @@ template <int KIND, int ES, bool PACK>
 static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cudaStream_t s, const void *mul)
 {
     const int64_t cap = MAX_GRID;
-    // A block per 16 KB, in one pass: long runs off 16-byte boundaries, that is slices of a matrix; bound by HBM and L2.  us, blocks that
-    // walk 32 KB / one pass: times a packed operand [384,384,75] 13.6 / 11.2, [4000,4000,3] 52.1 / 45.4, [2000,2000,10] 41.4 / 37.3;
-    // zero fill 11.4 / 11.0, 50.1 / 45.9, 40.5 / 37.6; pack 8.7 / 9.0, 38.5 / 35.7, 29.4 / 28.6; pack, product, sum and fill of
-    // [384,384,75] out of HBM 54.2 / 48.2 together.  Not where runs are short or most parts of a slice empty (pack of a tet d = 160,
+    // A block per 16 KB, in one pass: long runs off 16-byte boundaries, that is slices of a matrix; bound by HBM and L2.  A block has the
+    // warps that its part needs, as parts of a slice are even: with 256 threads the half-empty blocks of a slice a little longer than
+    // 16 KB cost more than the pass saves.  us in rows of calls, blocks that walk 32 KB / one pass with 256 threads / now: pack
+    // [384,384,75] 8.2 / 8.6 / 8.0, [2000,2000,3] 8.4 / 11.2 / 8.6, [4100,4100] 13.5 / 20.3 / 12.8, [4000,4000,3] 38.4 / 35.4 / 33.9; times
+    // a packed operand 10.9 / 9.7 / 8.9, 10.6 / 13.0 / 9.5, 20.4 / 24.6 / 16.4, 52.2 / 45.2 / 44.0; zero fill 11.7 / 10.9 / 10.6, 12.5 / 14.0 /
+    // 11.7, 20.9 / 25.8 / 18.5, 49.9 / 45.7 / 45.1.  Not where runs are short or most parts of a slice empty (pack of a tet d = 160,
     // 33 floats, 52 / 74; 2-byte words [900,900,17] 5.3 / 6.8), nor where all is aligned ([1024,1024,64] doubles 81 / 84).
     constexpr bool ONCE = KIND == ST_TRI_UPPER && (ES == 4 || ES == 8);
     // slices: about four 16-byte units per thread, at most PART_BYTES per (slice, part), less where the slices are too few to
@@ -681,9 +683,10 @@ static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cu
     parts = (sb + pb - 1) / pb;
     if (parts > (int64_t(1) << 30)) return ST_ERR_UNSUPPORTED;
     int shift = 0;
-    while ((1 << shift) < 256 && (once || (int64_t(16 * COPY_UNITS) << shift) < pb)) ++shift;
-    const int64_t nitems = nslices * parts, threads = nitems << shift;
-    const int64_t want = (threads + 255) / 256;
+    while ((1 << shift) < 256 && (int64_t(16 * COPY_UNITS) << shift) < pb) ++shift;
+    const int64_t nitems = nslices * parts, want = once ? nitems : ((nitems << shift) + 255) / 256;
+    constexpr int64_t WARP_BYTES = 32 * 16 * COPY_UNITS;      // of a warp in one pass
+    const unsigned threads = once ? (unsigned)((pb + WARP_BYTES - 1) / WARP_BYTES) * 32u : 256u;
     const unsigned grid = (unsigned)(want < cap ? (want < 1 ? 1 : want) : cap);
     const unsigned char *in = (const unsigned char *)src, *m = (const unsigned char *)mul;
     unsigned char *out = (unsigned char *)dst;
@@ -695,7 +698,7 @@ static st_status launch_copy(const void *src, void *dst, const LayoutArgs &a, cu
         constexpr bool MUL = decltype(mul_tag)::value;
         if constexpr (ONCE)
             if (once)
-                return launch(slice_copy_kernel<KIND, ES, PACK, MUL, true, I>, grid, 256, 0, s, in, out, a, (I)nitems, 8, (int)parts, (int)pb, m);
+                return launch(slice_copy_kernel<KIND, ES, PACK, MUL, true, I>, grid, threads, 0, s, in, out, a, (I)nitems, 0, (int)parts, (int)pb, m);
         return launch(slice_copy_kernel<KIND, ES, PACK, MUL, false, I>, grid, 256, 0, s, in, out, a, (I)nitems, shift, (int)parts, (int)pb, m);
     };
     if constexpr (PACK && ES == 4)

@@ -1493,6 +1493,24 @@ def test_copies_of_rows_off_boundaries(st, kind, d, inner, dtype):
         assert np.array_equal(st.st_thp(dev(B), dev(C), lay).cpu().numpy(), want)
 
 
+# the same in parts of every length: one to eight warps for the last of a slice, of one part and of several, a first part of a slice
+# that is short, runs that end in front of it
+@pytest.mark.parametrize("d,inner,dtype", [(d, 1, np.uint32) for d in (4097, 4609, 5121, 6143)] + [(1366, 3, np.uint32), (1537, 3, np.uint32), (1879, 3, np.uint32),
+                                           (2050, 1, np.uint64), (2305, 1, np.uint64), (701, 6, np.uint32), (97, 45, np.uint32), (91, 91, np.uint32)])
+def test_copies_of_parts_of_every_length(st, d, inner, dtype):
+    lay = st.Layout(st.ST_TRI_UPPER, d, inner)
+    nd = st.st_dense_elems(lay)
+    dense = np.random.default_rng(nd).integers(1, np.iinfo(dtype).max, size=nd, dtype=dtype)
+    signed = {4: np.int32, 8: np.int64}[dense.itemsize]
+    packed = oracle.pack(dense, lay.kind, d, inner=inner)
+    got = st.st_pack(torch.from_numpy(dense.view(signed)).cuda(), lay)
+    assert np.array_equal(got.cpu().numpy().view(dtype), packed)
+    assert np.array_equal(st.st_unpack(got, lay).cpu().numpy().view(dtype), oracle.unpack(packed, lay.kind, d, inner=inner, fill=st.ST_FILL_ZERO).reshape(-1))
+    if dtype == np.uint32:
+        B, C = (workloads.draw((n,), "normal", 5) for n in (packed.size, nd))
+        assert np.array_equal(st.st_thp(dev(B), dev(C), lay).cpu().numpy(), B * oracle.pack(C.view(np.uint32), lay.kind, d, inner=inner).view(np.float32))
+
+
 # fp32 second moment of more than 128 features on both sides of the line between its two kernels, and of many tiles with few
 # samples, whose sums go round with fewer blocks than rows
 @pytest.mark.parametrize("N,d", [(4900, 129), (5000, 129), (1, 130), (9900, 160), (10100, 160), (33, 193), (1000, 248), (37000, 248), (5, 1300), (70, 2100),
@@ -1528,6 +1546,48 @@ def test_copies_with_64_bit_indices(st):
     lo, hi = torch.minimum(i[:, None], j), torch.maximum(i[:, None], j)
     want = P[lo * (2 * d - lo + 1) // 2 + hi - lo]
     assert torch.equal(D[i], want) and torch.equal(D[:, i].T, want)
+
+
+# the same of words of 4 and 8 bytes, slices off 16-byte boundaries in one pass
+@pytest.mark.parametrize("dtype", [torch.int32, torch.int64])
+def test_copies_with_64_bit_indices_off_boundaries(st, dtype):
+    d = 20003
+    lay = st.Layout(st.ST_TRI_UPPER, d)
+    P = torch.arange(st.st_packed_elems(lay), device="cuda").to(dtype)
+    D = st.st_unpack(P, lay).view(d, d)
+    assert torch.equal(D, torch.triu(D))
+    i = torch.tensor([0, 1, 2, 3, 9999, 19990, d - 2, d - 1], device="cuda")
+    j = torch.arange(d, device="cuda")
+    at = i[:, None] * (2 * d - i[:, None] + 1) // 2 + j - i[:, None]
+    assert torch.equal(D[i], torch.where(j >= i[:, None], at, 0).to(dtype))
+    assert torch.equal(st.st_pack(D, lay), P)
+    if dtype == torch.int32:
+        C, F = torch.rand(d * d, device="cuda"), torch.rand(P.numel(), device="cuda")
+        assert torch.equal(st.st_thp(F, C, lay), F * st.st_pack(C, lay))
+
+
+# the same of symmetric fills word by word: a row found for every word and one for all lanes
+@pytest.mark.parametrize("kind,d,inner,dtype", [("ST_TRI_UPPER", 32771, 3, torch.int16), ("ST_TET", 1027, 3, torch.int32), ("ST_TET", 1027, 9, torch.int32),
+                                                ("ST_SIMPLEX4", 202, 3, torch.int32)])
+def test_symmetric_fill_with_64_bit_indices(st, kind, d, inner, dtype):
+    lay = st.Layout(getattr(st, kind), d, inner)
+    P = torch.arange(st.st_packed_elems(lay), device="cuda").to(dtype)
+    order = {"ST_TRI_UPPER": 2, "ST_TET": 3, "ST_SIMPLEX4": 4}[kind]
+    D = st.st_unpack(P, lay, st.ST_FILL_SYMMETRIC).view((d,) * order + (inner,))
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    # positions at random and with the largest indices; their packed place by counting from the end: the sorted index's successors
+    idx = torch.randint(0, d, (200000, order), generator=g, device="cuda")
+    idx[:1000] = d - 1 - torch.randint(0, 3, (1000, order), generator=g, device="cuda")
+    s = torch.sort(idx, dim=1).values
+    place = torch.full((idx.shape[0],), P.numel() // inner - 1, device="cuda")
+    for o in range(order):
+        r, k = d - 1 - s[:, o], order - o                 # C(r + k - 1, k) later tuples start with a larger index in this place
+        c = torch.ones_like(r)
+        for m in range(k):
+            c = c * (r + m) // (m + 1)
+        place -= c
+    assert torch.equal(D[tuple(idx.T)], P.view(-1, inner)[place])
 
 
 # ------------------------------------------------------------------ fp32 second moment of many samples: exact parts of x
