@@ -339,7 +339,10 @@ __global__ void __launch_bounds__(M2S_MAX_THREADS, 1) moment2_small_kernel(const
 // placement bound it: twenty loads at a time take registers that the running kernel does not leave ([20000,64] 10.8 us the call,
 // with seven 9.9); with eight warps whatever the slices, seven loads at a time, [50021,75] 18.2 us, now 17.6, [30000,120] 22.5 and
 // 20.6, [50000,150] 62 and 49.
-constexpr int M2S_SUM_BATCH = 5, M2S_SUM_V4 = 24;      // work items from where V = 4 ([50021,75], 28 items, 17.7 us with V = 1, 17.6)
+// M2S_SUM_V4: work items from where V = 4.  us in rows of calls, V = 1 / 4: 5 items [50021,32] 7.8 / 8.1, [20000,32] 6.7 / 6.9; 8 items
+// [20000,40] 6.8 / 7.0, [50021,40] 8.2 / 8.2; 11 items [20000,48] 8.2 / 8.0, [300000,48] 26.2 / 26.0; 18 items [50021,64] 12.5 / 12.3, [300000,64]
+// 35.1 / 34.8; 28 items [300000,80] 50.5 / 50.2.
+constexpr int M2S_SUM_BATCH = 5, M2S_SUM_V4 = 10;
 template <int V, int W>
 __global__ void __launch_bounds__(32 * W)
 moment2_small_reduce_kernel(const float *partials, float *out, int d, int nbk, int slices,

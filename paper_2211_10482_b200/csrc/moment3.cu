@@ -323,7 +323,10 @@ moment3_kernel(const M3Args a, const __grid_constant__ M3Table<WARPS> tab)
 // take more registers than the running kernel leaves, and start later ([4096,24] 12.2 us the call, with five 11.2, twenty 14.7);
 // with V = 1 and eight warps whatever the slices [4096,24] 11.9 us the call, now 10.2, [6000,128] 147 and 139, [50000,21] 25.1 and 23.4.
 constexpr int SUM_BATCH = 5;
-constexpr int64_t SUM_V4 = 128 * 64;       // elements from where V = 4 ([4096,24], 2600 of them, 11.1 us with it and 10.2 without)
+// SUM_V4: elements from where V = 4.  us in rows of calls, V = 1 / 4: 2600 elements [4096,24] 10.1 / 10.6, 5984 [4096,32] 12.4 / 12.8, 8436
+// [1000,36] 11.3 / 11.6, [4096,36] 13.6 / 14.1, [40000,36] 39.5 / 39.8; 9880 [700,38] 12.1 / 12.3, [20000,38] 25.9 / 25.5; 10660 [4096,39] 16.1 /
+// 15.7, 11480 [4096,40] 16.8 / 16.4, [40000,40] 41.8 / 41.2; 45760 [4096,64] 30.3 / 28.3.
+constexpr int64_t SUM_V4 = 9500;
 template <int V, int W>
 __global__ void __launch_bounds__(32 * W)
 sum_slices_kernel(const float *partials, float *out, int64_t elems, int slices)

@@ -1511,6 +1511,22 @@ def test_copies_of_parts_of_every_length(st, d, inner, dtype):
         assert np.array_equal(st.st_thp(dev(B), dev(C), lay).cpu().numpy(), B * oracle.pack(C.view(np.uint32), lay.kind, d, inner=inner).view(np.float32))
 
 
+# sums over the slices on both sides of the lines from where a lane has four elements, over 8, 16 and 32 warps
+@pytest.mark.parametrize("N", [2011, 9001, 50021])
+@pytest.mark.parametrize("d", [36, 38, 39, 40, 41, 48, 55, 64])
+def test_moments_sums_of_four_elements_to_a_lane(st, N, d):
+    X = workloads.draw((N, d), "normal", 13 + N + d)
+    X64 = torch.from_numpy(X).cuda().double()
+    i, j = (torch.from_numpy(v).cuda() for v in np.triu_indices(d))
+    T, S = (V.T @ V for V in (X64, X64.abs()))
+    got = st.st_sym_moment2(dev(X)).double()
+    assert ((got - T[i, j]).abs() / S[i, j]).max().item() <= TOL_F32
+    i, j, k = (torch.tensor(v, device="cuda") for v in zip(*itertools.combinations_with_replacement(range(d), 3)))
+    got = st.st_sym_moment3(dev(X)).double()
+    T, S = (torch.einsum("na,nb,nc->abc", V, V, V)[i, j, k] for V in (X64, X64.abs()))
+    assert ((got - T).abs() / S).max().item() <= TOL_F32
+
+
 # fp32 second moment of more than 128 features on both sides of the line between its two kernels, and of many tiles with few
 # samples, whose sums go round with fewer blocks than rows
 @pytest.mark.parametrize("N,d", [(4900, 129), (5000, 129), (1, 130), (9900, 160), (10100, 160), (33, 193), (1000, 248), (37000, 248), (5, 1300), (70, 2100),
