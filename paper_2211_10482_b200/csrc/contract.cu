@@ -250,12 +250,6 @@ __global__ void __launch_bounds__(RG_THREADS, 1) rowgemm_kernel(const RgArgs a)
 constexpr int ROWSUM_BLOCKS = 16;            // per SM
 constexpr int ROWSUM_LONG = 64;              // mean number of slots of a reached row from which sixteen loads at a time pay
 
-// Second pass of MTTKRP: one warp per row of A adds the partial slots of that row in increasing
-// order (units, then k-splits); rows that no fibre reaches become zero.  The warps walk the rows, since a block for every eight
-// of them costs more to place than its stores take (slice i of [200000,1000,64], R = 32, one row that is not zero: 35 us the
-// call, now 17).  BATCH: loads at a time.  The one row of a slice i has thousands of slots and its sum is a chain of round
-// trips ([3000,50000,64], R = 32: eight 92 us, sixteen 41); where rows have few, the registers of sixteen keep blocks from
-// starting beside the running kernel ([900,900,48], R = 64, split: eight 76.5 us, sixteen 80).
 // The slots of row `row` of A; n = 0: a row of zeros, -1: out of range.
 __device__ __forceinline__ void mttkrp_row_slots(const MttkrpRows &m, int64_t row, int64_t i_off, int unit_shift, int ksplit, int64_t &first, int64_t &n)
 {
@@ -273,6 +267,12 @@ __device__ __forceinline__ void mttkrp_row_slots(const MttkrpRows &m, int64_t ro
     if (!ST_BOUNDS_OK(first + n - 1, mttkrp_slots(m.rows, 1 << unit_shift, m.I, ksplit), 6)) n = -1;
 }
 
+// Second pass of MTTKRP, for many rows of A and for rows of few slots (others: mttkrp_rowsum_few_kernel): one warp per row adds the
+// partial slots of that row in increasing order (units, then k-splits); rows that no fibre reaches become zero.  The warps walk the
+// rows, since a block for every eight of them costs more to place than its stores take (slice i of [200000,1000,64], R = 32, one row
+// that is not zero: 35 us the call, now 17).  BATCH: loads at a time.  The one row of a slice i has thousands of slots and its sum is
+// a chain of round trips ([3000,50000,64], R = 32: eight 92 us, sixteen 41); where rows have few, the registers of sixteen keep
+// blocks from starting beside the running kernel ([900,900,48], R = 64, split: eight 76.5 us, sixteen 80).
 template <int BATCH>
 __global__ void __launch_bounds__(256, BATCH > 8 ? 1 : 8)
 mttkrp_rowsum_kernel(const float *part, float *A, int64_t I_full, int64_t i_off, MttkrpRows m, int R, int unit_shift, int ksplit)

@@ -1423,8 +1423,8 @@ def test_mttkrp_slice_of_few_rows(st, I, J, R):
     assert not A[:I - 1].any()
 
 
-# row sums: a row of more slots than are loaded at a time (sixteen, eight, a remainder) and rows of none, more rows than the
-# warps of the grid; slices whose rows of A have one fibre each, several to a unit and a ragged last unit
+# row sums: a long row and rows of none, by four warps to a row; rows of one slot at most, of which there are more than warps in the
+# grid; slices whose rows of A have one fibre each, several to a unit and a ragged last unit
 @pytest.mark.parametrize("flag_name,R,tol", [("f32", 64, TOL_F32), ("tf32", 32, 5e-3), ("split", 32, TOL_F32)])
 def test_mttkrp_slices_with_long_rows_and_with_many_rows(st, flag_name, R, tol):
     flags = {"f32": 0, "tf32": st.ST_FLAG_TC_TF32, "split": st.ST_FLAG_TC_SPLIT}[flag_name]
@@ -1442,6 +1442,22 @@ def test_mttkrp_slices_with_long_rows_and_with_many_rows(st, flag_name, R, tol):
             want, size = Y * Cr, S * np.abs(Cr)
         assert np.max(np.abs(got - want) / size) <= tol, (I, J, fi, fj)
         assert np.count_nonzero(got[size[:, 0] == 1e-30]) == 0
+
+
+# row sums by one warp with sixteen loads at a time: more rows of A than four warps to a row are for, and one of them with 64 slots
+# and more; sixteens alone, with an eight and a remainder, with a remainder
+@pytest.mark.parametrize("flag_name,R,tol", [("f32", 64, TOL_F32), ("tf32", 32, 5e-3), ("split", 32, TOL_F32)])
+@pytest.mark.parametrize("I,J", [(3000, 4099), (2500, 9500), (2400, 16384), (30000, 20011)])
+def test_mttkrp_slice_of_one_long_row_among_many(st, flag_name, R, tol, I, J):
+    flags = {"f32": 0, "tf32": st.ST_FLAG_TC_TF32, "split": st.ST_FLAG_TC_SPLIT}[flag_name]
+    K, fi = 16, 5
+    B, C, D = (workloads.draw(s, "normal", 9 + i) for i, s in enumerate(((J, K), (J, R), (K, R))))
+    got = st.st_mttkrp_slice(dev(B), dev(C), dev(D), I, fi, -1, flags=flags).cpu().numpy()
+    B, C, D = (v.astype(np.float64) for v in (B, C, D))
+    want, size = ((B @ D) * C).sum(0), ((np.abs(B) @ np.abs(D)) * np.abs(C)).sum(0)
+    assert np.max(np.abs(got[fi] - want) / size) <= tol
+    got[fi] = 0
+    assert not got.any()
 
 
 # a band wider than the matrix, whose packed rows have several parts of zeros; one row in many parts; symmetric fills of wide
