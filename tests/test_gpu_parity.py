@@ -870,8 +870,8 @@ def test_moment2_tensor_core_left_over_columns(st, N, d):
     assert oracle.rel_err(expand2(st, st.st_sym_moment2(dev(X[:, :d - 4].copy()), flags=st.ST_FLAG_TC_TF32), d - 4), Tt, St) <= TOL_F32
 
 
-# the same carried along by the tiles on the diagonal: 16 to 128 of them, one tile and several, one phase and many; split also with
-# two products on the diagonal, with and without such columns
+# the same carried along by the tiles on the diagonal: 16 to 128 of them, one tile and several, one phase and many (bf16 [50021,264]: tiles of
+# their own); split also with two products on the diagonal, with and without such columns
 @pytest.mark.parametrize("mode,N,d", [("split", 210000, 264), ("split", 230000, 304), ("tf32", 640000, 260), ("bf16", 640000, 384), ("split", 20011, 520),
                                       ("split", 64000, 384), ("split", 70013, 1032), ("split", 60011, 512), ("split", 130001, 256), ("tf32", 50007, 300), ("tf32", 70001, 380), ("tf32", 100003, 516),
                                       ("bf16", 50021, 264), ("bf16", 90001, 600), ("bf16", 60017, 800)])
