@@ -56,6 +56,8 @@
 #include "st_index.cuh"
 #include "pair_layout.cuh"
 #include <cuda_bf16.h>
+#include <algorithm>
+#include <functional>
 
 namespace st {
 
@@ -645,17 +647,24 @@ static double m2tc_exact_cost(int rows, int width, bool diag)
     return rows > m2tc::HALF ? 0.88 : 0.47 + 0.26 * rows / m2tc::HALF;
 }
 
-// Columns that are left over after `full` tiles of 256: carried along by the tiles on the diagonal, or tiles of their own.  The
-// epilogue of a tile that carries them has up to twice the columns, and the sum more parts: a fixed time that the samples of a
-// cluster, in cycles of their stages, have to outweigh.  us, tiles of their own / carried: TF32 [20000,300] 17.9 / 19.1, [60000,300]
-// 35.8 / 29.0, [20000,380] 19.7 / 24.1, [60000,380] 39.6 / 36.9; bf16 [20000,264] 13.3 / 15.2, [60000,264] 22.7 / 20.8, [20000,800] 26.3 /
-// 27.7, [60000,800] 59 / 53; split [6000,520] 19.5 / 21.7, [20000,520] 39.4 / 36.0, [20000,384] 24.4 / 27.4, [60000,384] 51.5 / 43.8.
 constexpr double m2tc_stage_cycles(int mode) { return mode == M2_CONV ? 1226 : 512; }      // a full tile's
 template <int MODE>
 static double m2tc_cycles(int64_t N, double cost)          // of a cluster, where tiles of this cost together share the chip
 {
     return (double)((N + m2tc::Shape<MODE>::KROWS - 1) / m2tc::Shape<MODE>::KROWS) * cost * m2tc_stage_cycles(MODE) / (sm_count_or_default() / 2);
 }
+// Columns that are left over after `full` tiles of 256: carried along by the tiles on the diagonal, or tiles of their own.  The
+// epilogue of a tile that carries them has up to twice the columns, and the sum more parts: a fixed time that the samples of a
+// cluster, in cycles of their stages, have to outweigh.  us, tiles of their own / carried: TF32 [20000,300] 17.9 / 19.1, [60000,300]
+// 35.8 / 29.0, [20000,380] 19.7 / 24.1, [60000,380] 39.6 / 36.9; bf16 [20000,264] 13.3 / 15.2, [60000,264] 22.7 / 20.8, [20000,800] 26.3 /
+// 27.7, [60000,800] 59 / 53; split [6000,520] 19.5 / 21.7, [20000,520] 39.4 / 36.0, [20000,384] 24.4 / 27.4, [60000,384] 51.5 / 43.8.
+// The tiles that carry them are longer, too, which costs more than it saves where a tile has a cluster or two.  M2TC_CARRY_GAIN: the
+// longest cluster has to become that much shorter.  1800 features are 36 tiles of two clusters each, or 28 of which those off the
+// diagonal have two as well; 3200 are 91, or 78 on 74 pairs of SMs of which the last takes twice as long.  us in rows of calls: TF32
+// [81405,1800] 524 / 566, [80567,2568] 1033 / 1098, [80386,3080] 1836 / 2296, [78977,3200] 1702 / 2514, bf16 [63182,3200] 712 / 1087, split
+// [52771,3200] 1916 / 2701; a gain where the longest becomes 6 % shorter, TF32 [97053,1152] 292 / 266, 21 %, [81425,2176] 890 / 799, and
+// 43 %, bf16 [64795,2056] 463 / 278.
+constexpr double M2TC_CARRY_GAIN = 0.97;
 template <int MODE>
 static bool m2tc_carry(int64_t N, int full, int left_over)
 {
@@ -771,7 +780,19 @@ static void m2tc_finish(M2TcPlan &p, const M2TcTiles &t, int64_t N)
     }
     for (int i = n; i <= MAX_TILES; ++i) p.tab.first[i] = (unsigned short)first;
     p.partial_bytes = (size_t)2 * first * p.pitch * sizeof(float);
-    p.time = (double)chunks * (longest > sum / clusters ? longest : sum / clusters);        // (more tiles than pairs of SMs: several waves)
+    if (first > clusters) {                            // several waves: each cluster in turn on the pair of SMs that is free first
+        double busy[MAX_TILES] = {};                   // a heap, that pair in front
+        const int pairs = clusters < MAX_TILES ? clusters : MAX_TILES;
+        longest = 0;
+        for (int i = 0; i < n; ++i)
+            for (int k = 0; k < split[i]; ++k) {
+                std::pop_heap(busy, busy + pairs, std::greater<double>());
+                busy[pairs - 1] += cost[i] / split[i];
+                if (busy[pairs - 1] > longest) longest = busy[pairs - 1];
+                std::push_heap(busy, busy + pairs, std::greater<double>());
+            }
+    }
+    p.time = (double)chunks * longest;
     p.ok = true;
 }
 
@@ -803,8 +824,13 @@ static M2TcPlan m2tc_plan(int64_t N, int64_t d, unsigned flags)
 {
     using namespace m2tc;
     const bool dense = (flags & ST_FLAG_DENSE_CONTROL) != 0;
-    const bool carry = !dense && m2tc_carry<MODE>(N, (int)(d / BM), (int)(d % BM));
-    const M2TcPlan three = m2tc_plan_of<MODE>(N, d, dense, carry, false);
+    M2TcPlan three = m2tc_plan_of<MODE>(N, d, dense, false, false);
+    bool carry = !dense && m2tc_carry<MODE>(N, (int)(d / BM), (int)(d % BM));
+    if (carry) {
+        const M2TcPlan with = m2tc_plan_of<MODE>(N, d, false, true, false);
+        carry = with.ok && (!three.ok || with.time < M2TC_CARRY_GAIN * three.time);
+        if (carry) three = with;
+    }
     if constexpr (MODE == M2_CONV) {
         const double most = M2TC_SYM_FULL * m2tc_stage_cycles(MODE) * three.time;            // that two products can save
         if (dense || d < BN || !three.ok || most < M2TC_SYM_SUM) return three;

@@ -949,7 +949,7 @@ def test_moment2_left_over_columns_of_positive_tables_do_not_drift(st, mode, N, 
 
 # two products on full diagonal tiles: their sums over one to eight ranges per warp, a last tile that is not quite full, carried columns
 @pytest.mark.parametrize("N,d", [(290011, 256), (90001, 304), (60011, 504), (30011, 512), (15013, 776), (12007, 768), (9001, 1024), (15001, 1280), (6007, 3072),
-                                 (4001, 4096)])
+                                 (4001, 4096), (12007, 2056), (6001, 3080)])
 def test_moment2_split_with_two_products_on_the_diagonal(st, N, d):
     g = torch.Generator(device="cuda")
     g.manual_seed(N)
